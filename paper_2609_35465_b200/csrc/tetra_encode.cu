@@ -2,23 +2,37 @@
 // direction is closest to the block, and the gain bit.
 //
 // The paper's own search is not exhaustive and runs on a CPU; this kernel computes the exact optimum of the
-// same objective,  max <w, y> / (|w| |y|)  over all 2^47 indices, by using what the format's structure gives:
-//   * a section's coordinates depend on (parity p, pattern byte c, rank row) only, the pattern bytes of all
-//     three sections are the 128 even-weight bytes, and for fixed (p, c, class) the section's squared norm is
-//     16 k + r with r fixed by (p, weight of c, class) and k = 0..9: per section, byte and class only ten best
-//     correlations matter (one per k);
-//   * the sections are tied by the trellis path, by the parity and by Eq. (3) (r3 = p ^ r ^ delta): they are
-//     joined state by state with the summed norm and the class parity as extra state.
-// One CTA of 384 threads works on one block at a time: three groups of 128 threads, one per section, thread =
-// pattern byte.  For every batch of 32 rank rows a group tabulates, per row, the partial correlations and
-// norms of the 16 patterns of each half of the byte (so a (row, byte) candidate costs two shared loads and two
-// additions) while every thread scans the batch before for its own byte and keeps the best correlation per
-// (class, k) in a private column of shared memory (no atomics; two columns, for even and odd rows, so that
-// two updates are in flight).  The join runs on the same CTA, every thread gathering a few entries of the
-// second cut; the rows that attain the winning entries are found by a second scan of three lists.
+// same objective,  max <w, y> / (|w| |y|)  over all 2^47 indices, without visiting the rows of the lists one by
+// one.  Facts of the format that it uses:
+//   * Rank rows.  With weights 0, 1, 3, 6, 10 for ranks 0..4 a row's cost is 8 + 8 W, W the sum of its eight
+//     ranks' weights, and its class is the parity of W.  A list is therefore every row of class cls up to some
+//     W plus, of the next shell, the rows up to a limit in the order of the packed row value (the tie rule of
+//     the sort):  sections 0 and 2 hold W <= 8 and W = 10 up to 0x11030011 (class 0), W <= 9 and W = 11 up to
+//     0x00222011 (class 1); the middle list holds W <= 6 and W = 8 up to 0x30001010 (class 0), W <= 7 (class 1).
+//     tetra_build_table checks these limits.
+//   * Halves.  Rank vectors of coordinates 0..3 and 4..7 combine freely except for those limits, so the best
+//     correlation of a section for (pattern byte, class, squared norm) is a maximum of sums of two half-table
+//     entries (best correlation of a half for its pattern nibble, weight, norm); "row <= limit" is "high half
+//     below the limit's" (a table of its own) or "equal, and low half up to the limit's" (a few entries).
+//   * Norms.  A section's squared norm is 16 k + r, r in {0, 8} fixed by (parity, byte, class).  At odd parity
+//     it is the row's cost, so W gives it; at even parity a coordinate adds kappa(pattern bit, rank) =
+//     0,1,1,4,4 or 0,0,2,2,6 to k, and the byte floor(ones / 4).
+//   * Trellis.  An even-weight byte up to complement is h(alpha) + h'(xi), alpha and xi of three bits each; the
+//     codewords are exactly the triples (alpha, xi), (beta, xi), (alpha + beta, xi) with any complements.  So the
+//     sections' tables hold 64 rows, and joining sections 1 and 2 is, for every xi, an XOR convolution over eight
+//     alphas.  At even parity r = 8 exactly where |h(alpha) & h'(xi)| is odd, a bilinear form.
+// One CTA of 192 threads works on one block at a time: half tables (a thread per section, half and nibble; both
+// parities at once), section tables (a thread per section and byte pair), join and objective (a thread per end
+// state and class parity), and, when a parity improves on the other, the winner traced back through the same
+// tables by one warp per section.  Every sum is formed in the same order wherever it is needed, so the trace
+// matches floats exactly.
+//
+// Bound by instruction issue (adds and maxima of the section tables and the join; all tables sit in shared
+// memory).  On 24,576 Gaussian blocks: see the figures at launch_encode.
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "../../include/tetra.h"
 #include "tetra_device.cuh"
@@ -28,460 +42,1019 @@
 namespace tetra {
 namespace {
 
-constexpr int kEncThreads = 384;
-constexpr int kEncBatch = 32;       // rank rows per batch
-constexpr int kEncStride = 33;      // row-table entries are 33 rows apart (bank spread)
+constexpr int kEncThreads = 192;
+constexpr int kEncCtasPerSm = 3;
 constexpr float kNeg = -1.0e30f;
-constexpr float kNegTest = -1.0e29f;
 
-struct EncShared {
-    uint32_t rows[4096];
-    uint16_t branches[1024];
-    uint8_t prefixes[128];
-    uint8_t suffixes[128];
-    uint16_t incoming[64][16];                 // per state after the branch: s8 | b2 << 6
-    int incoming_count[64];
-    float A[3][8][4][8];                       // w_j * value(o, rank)
-    int V2[4][8];                              // value(o, rank)^2
-    uint2 rowtab[2][3][32 * kEncStride];       // two buffers of (partial correlation, partial norm): entry (half * 16 + pattern), row
-    float T[3][2][20][128];                    // best correlation per (class * 10 + k), byte; one copy for even, one for odd rows
-    float F1[64][2][20];                       // after section 1: state, class, norm / 8
-    float H[39][128];                          // after section 2: norm / 8, (state after the branch) * 2 + class parity
-    float red_val[kEncThreads / 32];
-    uint32_t red_arg[kEncThreads / 32];
-    float w[24];
-    // best so far
-    float best_val, best_corr;
-    int best_norm;
-    uint32_t best_path;                        // s8 | b1 << 6 | b2 << 7 | b3 << 11 | p << 12 | r << 13
-    int best_field[3];
-    int found_field[3];
+// ---------------------------------------------------------------------------
+// compile-time shapes of the tables
+// ---------------------------------------------------------------------------
+constexpr int kMaxW = 11;   // largest weight of a half
+constexpr int kMaxK = 9;    // largest k of a section (even parity)
+
+__host__ __device__ constexpr int rank_weight(int r) { return r * (r + 1) / 2; }
+__host__ __device__ constexpr int kappa(int c, int r) {
+    const int t = (r + 1) / 2;                       // y = +-4 t (c = 0) or 2 -+ 4 t (c = 1)
+    return c == 0 ? t * t : ((r & 1) ? t * t - t : t * t + t);
+}
+
+// Which (weight, kappa) cells can occur after j coordinates of a half, whatever the pattern bits.
+struct Cells {
+    bool v[5][kMaxW + 1][kMaxK + 1];
 };
-
-__device__ __forceinline__ int even_byte(int ci) {  // the 128 even-weight bytes, by index
-    const int h = ci >> 3, li = ci & 7;
-    return (h << 4) | (li << 1) | ((__popc(li) ^ __popc(h)) & 1);
+constexpr Cells free_cells() {
+    Cells C{};
+    C.v[0][0][0] = true;
+    for (int j = 0; j < 4; ++j)
+        for (int w = 0; w <= kMaxW; ++w)
+            for (int k = 0; k <= kMaxK; ++k)
+                if (C.v[j][w][k])
+                    for (int r = 0; r < 5; ++r)
+                        for (int c = 0; c < 2; ++c) {
+                            const int w2 = w + rank_weight(r), k2 = k + kappa(c, r);
+                            if (w2 <= kMaxW && k2 <= kMaxK) C.v[j + 1][w2][k2] = true;
+                        }
+    return C;
 }
-__device__ __forceinline__ int even_index(int byte) { return ((byte >> 4) << 3) | ((byte & 15) >> 1); }
-// squared norm of a section = 16 k + residue
-__device__ __forceinline__ int norm_residue(int p, int cls, int byte) { return p ? (cls ? 0 : 8) : ((4 * __popc(byte)) & 15); }
+constexpr Cells kFree = free_cells();
+// The same for vectors whose packed value is below (or, with `equal`, up to) that of the digits d0 (lowest) .. d3.
+constexpr Cells prefix_cells(int d0, int d1, int d2, int d3, bool equal) {
+    Cells C{};
+    const int d[4] = {d0, d1, d2, d3};
+    C.v[0][0][0] = equal;
+    for (int j = 0; j < 4; ++j)
+        for (int w = 0; w <= kMaxW; ++w)
+            for (int k = 0; k <= kMaxK; ++k)
+                for (int r = 0; r <= d[j]; ++r)
+                    for (int c = 0; c < 2; ++c) {
+                        const bool from = r < d[j] ? kFree.v[j][w][k] : C.v[j][w][k];
+                        const int w2 = w + rank_weight(r), k2 = k + kappa(c, r);
+                        if (from && w2 <= kMaxW && k2 <= kMaxK) C.v[j + 1][w2][k2] = true;
+                    }
+    return C;
+}
+// The limits of the partial shells, as (high half digits, low half digits), lowest coordinate first.
+struct Limit {
+    int hi[4], lo[4];
+};
+constexpr Limit kLimit0{{3, 0, 1, 1}, {1, 1, 0, 0}};    // class 0, sections 0 and 2: 0x11030011, W = 10
+constexpr Limit kLimit1{{2, 2, 0, 0}, {1, 1, 0, 2}};    // class 1, sections 0 and 2: 0x00222011, W = 11
+constexpr Limit kLimitM{{0, 0, 0, 3}, {0, 1, 0, 1}};    // class 0, middle section:   0x30001010, W = 8
+constexpr int half_value(const int (&d)[4]) { return d[0] | (d[1] << 4) | (d[2] << 8) | (d[3] << 12); }
+constexpr int half_weight(const int (&d)[4]) {
+    return rank_weight(d[0]) + rank_weight(d[1]) + rank_weight(d[2]) + rank_weight(d[3]);
+}
+static_assert(((uint32_t(half_value(kLimit0.hi)) << 16) | uint32_t(half_value(kLimit0.lo))) == kLastRowClass0, "limit");
+static_assert(((uint32_t(half_value(kLimit1.hi)) << 16) | uint32_t(half_value(kLimit1.lo))) == kLastRowClass1, "limit");
+static_assert(((uint32_t(half_value(kLimitM.hi)) << 16) | uint32_t(half_value(kLimitM.lo))) == kLastRowMiddle0, "limit");
+static_assert(half_weight(kLimit0.hi) == 8 && half_weight(kLimit0.lo) == 2, "limit shell");
+static_assert(half_weight(kLimit1.hi) == 6 && half_weight(kLimit1.lo) == 5, "limit shell");
+static_assert(half_weight(kLimitM.hi) == 6 && half_weight(kLimitM.lo) == 2, "limit shell");
+constexpr Cells cells_of(const int (&d)[4], bool equal) { return prefix_cells(d[0], d[1], d[2], d[3], equal); }
+constexpr Cells kLess0 = cells_of(kLimit0.hi, false), kLess1 = cells_of(kLimit1.hi, false), kLessM = cells_of(kLimitM.hi, false);
+constexpr Cells kUpTo0 = cells_of(kLimit0.lo, true), kUpTo1 = cells_of(kLimit1.lo, true), kUpToM = cells_of(kLimitM.lo, true);
 
-__device__ __forceinline__ void group_barrier(int group) {
-    asm volatile("bar.sync %0, 128;" ::"r"(1 + group) : "memory");
+// Tables of a nibble at even parity.  High half: one entry per possible cell, weights 0..9 without restriction
+// (H), 0..10 below limit 0 or limit M (A), 0..11 below limit 1 (B), then the limits' own correlations.  Low
+// half: for every W the best over weights W, W - 2, ... (C: only the parity of the weight and an upper bound
+// matter), then the entries of the limits' low halves.
+constexpr int cells_before(const Cells& C, int max_w, int w, int k) {
+    int n = 0;
+    for (int a = 0; a <= max_w; ++a)
+        for (int b = 0; b <= kMaxK; ++b) {
+            if (a == w && b == k) return n;
+            if (C.v[4][a][b]) ++n;
+        }
+    return n;
+}
+constexpr int cells_total(const Cells& C, int max_w) { return cells_before(C, max_w, kMaxW + 1, 0); }
+constexpr int c_last(int W) {  // largest kappa over the weights W, W - 2, ...
+    int m = 0;
+    for (int a = W; a >= 0; a -= 2)
+        for (int b = 0; b <= kMaxK; ++b)
+            if (kFree.v[4][a][b] && b > m) m = b;
+    return m;
+}
+constexpr int c_offset(int W) {
+    int n = 0;
+    for (int a = 0; a < W; ++a) n += c_last(a) + 1;
+    return n;
+}
+constexpr Cells kLess0orM = [] {
+    Cells C = kLess0;
+    for (int w = 0; w <= kMaxW; ++w)
+        for (int k = 0; k <= kMaxK; ++k) C.v[4][w][k] = C.v[4][w][k] || (kLessM.v[4][w][k] && w <= 8);
+    return C;
+}();
+constexpr int kOffA = cells_total(kFree, 9), kOffB = kOffA + cells_total(kLess0orM, 10);
+constexpr int kOffHs = kOffB + cells_total(kLess1, 11);   // correlations of the limits' high halves: 0 (or M), 1
+constexpr int kHiStride = (kOffHs + 2) | 1;               // odd: a warp's nibbles fall into different banks
+constexpr int kOffRes0 = c_offset(kMaxW + 1);             // low halves up to limit 0 (or M), by kappa 0..2
+constexpr int kOffRes1 = kOffRes0 + 3;                    // low halves up to limit 1, by kappa 0..4
+constexpr int kLoStride = (kOffRes1 + 5) | 1;
+template <int W, int K> constexpr int kAtH = cells_before(kFree, 9, W, K);
+template <int W, int K> constexpr int kAtA = kOffA + cells_before(kLess0orM, 10, W, K);
+template <int W, int K> constexpr int kAtB = kOffB + cells_before(kLess1, 11, W, K);
+template <int W> constexpr int kAtC = c_offset(W);
+template <int W> constexpr int kLastC = c_last(W);
+constexpr int kCells = c_offset(kMaxW + 1);
+
+// Tables of a nibble at odd parity (the weight is the norm): low L[0..11], limits 0 or M, 1; high H[0..9],
+// A[0..10], B[0..11], limits.
+constexpr int kOddLoStride = 15;                          // 12 + 2, odd
+constexpr int kOddOffA = 10, kOddOffB = 21, kOddOffHs = 33, kOddHiStride = 35;
+
+// Half vectors for the trace, weight <= 11: value | weight << 16.
+struct HalfList {
+    uint32_t v[176];
+    int n;
+};
+constexpr HalfList half_list() {
+    HalfList L{};
+    for (int code = 0; code < 625; ++code) {
+        const int d[4] = {code % 5, (code / 5) % 5, (code / 25) % 5, code / 125};
+        const int w = half_weight(d);
+        if (w <= kMaxW) L.v[L.n++] = uint32_t(half_value(d)) | (uint32_t(w) << 16);
+    }
+    return L;
+}
+constexpr HalfList kHalfListHost = half_list();
+constexpr int kHalfVectors = kHalfListHost.n;
+__device__ const HalfList kHalfList = half_list();
+
+template <int I, int N, typename F>
+__device__ __forceinline__ void static_for(F&& f) {
+    if constexpr (I < N) {
+        f(std::integral_constant<int, I>{});
+        static_for<I + 1, N>(f);
+    }
+}
+template <int I, typename F>
+__device__ __forceinline__ void static_down(F&& f) {
+    if constexpr (I >= 0) {
+        f(std::integral_constant<int, I>{});
+        static_down<I - 1>(f);
+    }
 }
 
-// Rows of a section's list for a class: sections 0 and 2 read all 2048 rows of the class, the middle section
-// the first 1240 (class 0) or 808 (class 1) of them (Sec. 3.3).
-__device__ __forceinline__ int list_length(int section, int cls) {
-    return section == 1 ? (cls ? 2048 - kMiddleClass0 : kMiddleClass0) : 2048;
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
 }
 
-// Largest value over the CTA with its argument; ties go to the smaller argument.  Everyone gets the result.
-__device__ void cta_argmax(EncShared& S, float& val, uint32_t& arg) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// ---------------------------------------------------------------------------
+// shared memory of a CTA
+// ---------------------------------------------------------------------------
+constexpr int kRow = 12;     // floats per section-table row at even parity (k, or k + 1, from 0; the rest absent)
+constexpr int kOddRow = 8;   // at odd parity: index W / 2, 0..5
+struct EncShared {
+    float lo[3][16 * kLoStride];
+    float hi[3][16 * kHiStride];
+    float lo_odd[3][16 * kOddLoStride];
+    float hi_odd[3][16 * kOddHiStride];
+    // section tables: [class][pair = alpha + 8 xi][row].  F1 exists twice at even parity: plain and one entry up.
+    alignas(16) float F1[2][2][64 * kRow];
+    alignas(16) float F2[2][64 * kRow];
+    alignas(16) float F3[2][64 * kRow];
+    float rs[32];             // 1 / sqrt(16 m)
+    float w[24];
+    uint32_t halves[kHalfVectors];
+    uint8_t bytes[64];        // h(alpha) + h'(xi)
+    float red_val[4];
+    uint32_t red_arg[4];
+    float win_H[20];
+    float win_G;
+    int win_arg;
+    uint32_t found_row[3];    // index inside the section's list
+    uint32_t found_byte[3];
+    uint32_t found_cls[3];
+};
+static_assert(sizeof(EncShared) <= 74 * 1024, "three CTAs per SM");
+
+// h(a), a < 8, and h'(x), x < 8: representatives of the bytes of the two [8,4] codes up to complement.
+__device__ __forceinline__ uint32_t hamming_byte(uint32_t v, uint32_t b0, uint32_t b1, uint32_t b2) {
+    return ((v & 1) ? b0 : 0u) ^ ((v & 2) ? b1 : 0u) ^ ((v & 4) ? b2 : 0u);
+}
+__device__ __forceinline__ uint32_t pair_byte(int pair) {
+    return hamming_byte(uint32_t(pair) & 7u, 0x8Bu, 0x96u, 0xACu) ^ hamming_byte(uint32_t(pair) >> 3, 0x8Du, 0x9Au, 0xB4u);
+}
+// 1 where the squared norm of a section with this byte is 8 modulo 16 at even parity (byte and complement alike)
+__device__ __forceinline__ int odd_overlap(uint32_t byte) { return (__popc(byte) >> 1) & 1; }
+
+// At even parity a coordinate with a pattern bit adds 4 to the squared norm besides 16 kappa: k = kappa + this.
+__device__ __forceinline__ int ones_offset(uint32_t byte) { return __popc(byte) >> 2; }
+
+// ---------------------------------------------------------------------------
+// half tables
+// ---------------------------------------------------------------------------
+// The five products of a coordinate, w y(rank): the trace forms them the same way.
+__device__ __forceinline__ void products_even(float w, int c, float (&a)[5]) {
+    a[0] = __fmul_rn(w, c ? 2.f : 0.f);
+    a[1] = __fmul_rn(w, c ? -2.f : 4.f);
+    a[2] = __fmul_rn(w, c ? 6.f : -4.f);
+    a[3] = __fmul_rn(w, c ? -6.f : 8.f);
+    a[4] = __fmul_rn(w, c ? 10.f : -8.f);
+}
+__device__ __forceinline__ void products_odd(float w, int c, float (&a)[5]) {
+    const float s = c ? -w : w;
+    a[0] = s;
+    a[1] = __fmul_rn(s, -3.f);
+    a[2] = __fmul_rn(s, 5.f);
+    a[3] = __fmul_rn(s, -7.f);
+    a[4] = __fmul_rn(s, 9.f);
+}
+
+// One step of the prefix-limited table (before the free table takes the same step): vectors below the digits so
+// far = a smaller digit after anything, or the same digit after a smaller prefix.
+template <int J, int D, const Cells& PC>
+__device__ __forceinline__ void prefix_step(const float (&F)[kMaxW + 1][kMaxK + 1], float (&P)[kMaxW + 1][kMaxK + 1],
+                                            const float (&a)[5], int c) {
+    static_down<kMaxW>([&](auto wi) {
+        constexpr int W = decltype(wi)::value;
+        static_down<kMaxK>([&](auto ki) {
+            constexpr int K = decltype(ki)::value;
+            if constexpr (PC.v[J + 1][W][K]) {
+                float v = kNeg;
+                static_for<0, D + 1>([&](auto ri) {
+                    constexpr int R = decltype(ri)::value;
+                    if constexpr (W >= rank_weight(R)) {
+                        constexpr int W0 = W - rank_weight(R), K0 = K - kappa(0, R), K1 = K - kappa(1, R);
+                        constexpr bool f0 = K0 >= 0 && (R < D ? kFree.v[J][W0][K0 < 0 ? 0 : K0] : PC.v[J][W0][K0 < 0 ? 0 : K0]);
+                        constexpr bool f1 = K1 >= 0 && (R < D ? kFree.v[J][W0][K1 < 0 ? 0 : K1] : PC.v[J][W0][K1 < 0 ? 0 : K1]);
+                        if constexpr (f0 || f1) {
+                            float s0 = kNeg, s1 = kNeg;
+                            if constexpr (f0) s0 = R < D ? F[W0][K0] : P[W0][K0];
+                            if constexpr (f1) s1 = R < D ? F[W0][K1] : P[W0][K1];
+                            v = fmaxf(v, __fadd_rn(K0 == K1 ? s0 : (c ? s1 : s0), a[R]));
+                        }
+                    }
+                });
+                P[W][K] = v;
+            }
+        });
+    });
+}
+template <int J>
+__device__ __forceinline__ void free_step(float (&F)[kMaxW + 1][kMaxK + 1], const float (&a)[5], int c) {
+    static_down<kMaxW>([&](auto wi) {
+        constexpr int W = decltype(wi)::value;
+        static_down<kMaxK>([&](auto ki) {
+            constexpr int K = decltype(ki)::value;
+            if constexpr (kFree.v[J + 1][W][K]) {
+                float v = kNeg;
+                static_for<0, 5>([&](auto ri) {
+                    constexpr int R = decltype(ri)::value;
+                    if constexpr (W >= rank_weight(R)) {
+                        constexpr int W0 = W - rank_weight(R), K0 = K - kappa(0, R), K1 = K - kappa(1, R);
+                        constexpr bool f0 = K0 >= 0 && kFree.v[J][W0][K0 < 0 ? 0 : K0];
+                        constexpr bool f1 = K1 >= 0 && kFree.v[J][W0][K1 < 0 ? 0 : K1];
+                        if constexpr (f0 || f1) {
+                            float s0 = kNeg, s1 = kNeg;
+                            if constexpr (f0) s0 = F[W0][K0];
+                            if constexpr (f1) s1 = F[W0][K1];
+                            v = fmaxf(v, __fadd_rn(K0 == K1 ? s0 : (c ? s1 : s0), a[R]));
+                        }
+                    }
+                });
+                F[W][K] = v;
+            }
+        });
+    });
+}
+
+// Even parity: the tables of (section, half, nibble).  w4: the half's four weights.
+template <bool HIGH, bool MID>
+__device__ __forceinline__ void half_even(const float* w4, int nibble, float* out) {
+    float F[kMaxW + 1][kMaxK + 1], A[kMaxW + 1][kMaxK + 1], B[kMaxW + 1][kMaxK + 1];
+    F[0][0] = 0.f;
+    A[0][0] = 0.f;   // only the "up to" tables read it
+    B[0][0] = 0.f;
+    float hs0 = 0.f, hs1 = 0.f;  // correlations of the limits' high halves
+    static_for<0, 4>([&](auto ji) {
+        constexpr int J = decltype(ji)::value;
+        constexpr int D0 = kLimit0.hi[J], D1 = kLimit1.hi[J], DM = kLimitM.hi[J];  // digits of the limits' high halves
+        const int c = (nibble >> J) & 1;
+        float a[5];
+        products_even(w4[J], c, a);
+        if constexpr (HIGH) {
+            if constexpr (MID) {
+                prefix_step<J, kLimitM.hi[J], kLessM>(F, A, a, c);
+                hs0 = __fadd_rn(hs0, a[DM]);
+            } else {
+                prefix_step<J, kLimit0.hi[J], kLess0>(F, A, a, c);
+                prefix_step<J, kLimit1.hi[J], kLess1>(F, B, a, c);
+                hs0 = __fadd_rn(hs0, a[D0]);
+                hs1 = __fadd_rn(hs1, a[D1]);
+            }
+        } else {
+            if constexpr (MID) {
+                prefix_step<J, kLimitM.lo[J], kUpToM>(F, A, a, c);
+            } else {
+                prefix_step<J, kLimit0.lo[J], kUpTo0>(F, A, a, c);
+                prefix_step<J, kLimit1.lo[J], kUpTo1>(F, B, a, c);
+            }
+        }
+        free_step<J>(F, a, c);
+    });
+    if constexpr (HIGH) {
+        static_for<0, kMaxW + 1>([&](auto wi) {
+            constexpr int W = decltype(wi)::value;
+            static_for<0, kMaxK + 1>([&](auto ki) {
+                constexpr int K = decltype(ki)::value;
+                if constexpr (W <= 9 && kFree.v[4][W][K]) out[kAtH<W, K>] = F[W][K];
+                if constexpr (W <= 10 && kLess0orM.v[4][W][K]) {
+                    constexpr bool have = MID ? kLessM.v[4][W][K] : kLess0.v[4][W][K];
+                    float v = kNeg;
+                    if constexpr (have) v = A[W][K];
+                    out[kAtA<W, K>] = v;
+                }
+                if constexpr (!MID && kLess1.v[4][W][K]) out[kAtB<W, K>] = B[W][K];
+            });
+        });
+        out[kOffHs] = hs0;
+        out[kOffHs + 1] = hs1;
+    } else {
+        static_for<0, 2>([&](auto pi) {
+            float best[kMaxK + 1];
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-        const float v2 = __shfl_xor_sync(0xFFFFFFFFu, val, o);
-        const uint32_t a2 = __shfl_xor_sync(0xFFFFFFFFu, arg, o);
-        if (v2 > val || (v2 == val && a2 < arg)) {
-            val = v2;
-            arg = a2;
+            for (int k = 0; k <= kMaxK; ++k) best[k] = kNeg;
+            static_for<0, (kMaxW + 1) / 2>([&](auto ii) {
+                constexpr int W = 2 * decltype(ii)::value + decltype(pi)::value;
+                static_for<0, kLastC<W> + 1>([&](auto ki) {
+                    constexpr int K = decltype(ki)::value;
+                    if constexpr (kFree.v[4][W][K]) best[K] = fmaxf(best[K], F[W][K]);
+                    out[kAtC<W> + K] = best[K];
+                });
+            });
+        });
+        static_for<0, 5>([&](auto ki) {
+            constexpr int K = decltype(ki)::value;
+            if constexpr (K < 3) {
+                float v = kNeg;
+                if constexpr (MID ? kUpToM.v[4][2][K] : kUpTo0.v[4][2][K]) v = A[2][K];
+                out[kOffRes0 + K] = v;
+            }
+            if constexpr (!MID) {
+                float v = kNeg;
+                if constexpr (kUpTo1.v[4][5][K]) v = B[5][K];
+                out[kOffRes1 + K] = v;
+            }
+        });
+    }
+}
+
+// Odd parity: the same with the weight as the only index.
+constexpr bool odd_cell_at(const Cells& C, int j, int w) {
+    for (int k = 0; k <= kMaxK; ++k)
+        if (C.v[j][w][k]) return true;
+    return false;
+}
+template <const Cells& C, int J, int W> constexpr bool kOddCell = odd_cell_at(C, J, W);
+template <int J, int D, const Cells& PC>
+__device__ __forceinline__ void odd_prefix_step(const float (&F)[kMaxW + 1], float (&P)[kMaxW + 1], const float (&a)[5]) {
+    static_down<kMaxW>([&](auto wi) {
+        constexpr int W = decltype(wi)::value;
+        if constexpr (kOddCell<PC, J + 1, W>) {
+            float v = kNeg;
+            static_for<0, D + 1>([&](auto ri) {
+                constexpr int R = decltype(ri)::value;
+                if constexpr (W >= rank_weight(R)) {
+                    constexpr int W0 = W - rank_weight(R);
+                    if constexpr (R < D) {
+                        if constexpr (kOddCell<kFree, J, W0>) v = fmaxf(v, __fadd_rn(F[W0], a[R]));
+                    } else {
+                        if constexpr (kOddCell<PC, J, W0>) v = fmaxf(v, __fadd_rn(P[W0], a[R]));
+                    }
+                }
+            });
+            P[W] = v;
         }
+    });
+}
+template <bool HIGH, bool MID>
+__device__ __forceinline__ void half_odd(const float* w4, int nibble, float* out) {
+    float F[kMaxW + 1], A[kMaxW + 1], B[kMaxW + 1];
+#pragma unroll
+    for (int w = 0; w <= kMaxW; ++w) F[w] = A[w] = B[w] = kNeg;
+    F[0] = A[0] = B[0] = 0.f;
+    float hs0 = 0.f, hs1 = 0.f;
+    static_for<0, 4>([&](auto ji) {
+        constexpr int J = decltype(ji)::value;
+        constexpr int D0 = kLimit0.hi[J], D1 = kLimit1.hi[J], DM = kLimitM.hi[J];  // digits of the limits' high halves
+        float a[5];
+        products_odd(w4[J], (nibble >> J) & 1, a);
+        if constexpr (HIGH) {
+            if constexpr (MID) {
+                odd_prefix_step<J, kLimitM.hi[J], kLessM>(F, A, a);
+                hs0 = __fadd_rn(hs0, a[DM]);
+            } else {
+                odd_prefix_step<J, kLimit0.hi[J], kLess0>(F, A, a);
+                odd_prefix_step<J, kLimit1.hi[J], kLess1>(F, B, a);
+                hs0 = __fadd_rn(hs0, a[D0]);
+                hs1 = __fadd_rn(hs1, a[D1]);
+            }
+        } else {
+            if constexpr (MID) {
+                odd_prefix_step<J, kLimitM.lo[J], kUpToM>(F, A, a);
+            } else {
+                odd_prefix_step<J, kLimit0.lo[J], kUpTo0>(F, A, a);
+                odd_prefix_step<J, kLimit1.lo[J], kUpTo1>(F, B, a);
+            }
+        }
+        static_down<kMaxW>([&](auto wi) {
+            constexpr int W = decltype(wi)::value;
+            if constexpr (kOddCell<kFree, J + 1, W>) {
+                float v = kNeg;
+                static_for<0, 5>([&](auto ri) {
+                    constexpr int R = decltype(ri)::value;
+                    if constexpr (W >= rank_weight(R)) {
+                        constexpr int W0 = W - rank_weight(R);
+                        if constexpr (kOddCell<kFree, J, W0>) v = fmaxf(v, __fadd_rn(F[W0], a[R]));
+                    }
+                });
+                F[W] = v;
+            }
+        });
+    });
+    if constexpr (HIGH) {
+        static_for<0, kMaxW + 1>([&](auto wi) {
+            constexpr int W = decltype(wi)::value;
+            if constexpr (W <= 9) out[W] = F[W];
+            if constexpr (W <= 10) {
+                float v = kNeg;
+                if constexpr (MID ? kOddCell<kLessM, 4, W> : kOddCell<kLess0, 4, W>) v = A[W];
+                out[kOddOffA + W] = v;
+            }
+            float v = kNeg;
+            if constexpr (!MID && kOddCell<kLess1, 4, W>) v = B[W];
+            out[kOddOffB + W] = v;
+        });
+        out[kOddOffHs] = hs0;
+        out[kOddOffHs + 1] = hs1;
+    } else {
+#pragma unroll
+        for (int w = 0; w <= kMaxW; ++w) out[w] = F[w];
+        out[12] = A[2];
+        if constexpr (!MID) out[13] = B[5];
     }
-    __syncthreads();
-    if (lane == 0) {
-        S.red_val[warp] = val;
-        S.red_arg[warp] = arg;
+}
+
+// ---------------------------------------------------------------------------
+// section tables
+// ---------------------------------------------------------------------------
+// T[k] = max(T[k], h + C[W][k - k']) for a high-half entry h of weight and kappa (., k'): two norms per addition.
+template <int KH, int W, int KMAX>
+__device__ __forceinline__ void combine_even(float h, const float (&C)[kCells], float (&T)[kMaxK + 1]) {
+    static_for<0, kLastC<W> + 1>([&](auto ki) {
+        constexpr int KL = decltype(ki)::value;
+        if constexpr (KH + KL <= KMAX) T[KH + KL] = fmaxf(T[KH + KL], __fadd_rn(h, C[kAtC<W> + KL]));
+    });
+}
+
+template <bool MID>
+__device__ __forceinline__ void section_even(const float* lo, const float* hi, float (&T0)[kMaxK + 1], float (&T1)[kMaxK + 1]) {
+    float C[kCells];
+#pragma unroll
+    for (int i = 0; i < kCells; ++i) C[i] = lo[i];
+    static_for<0, kMaxW + 1>([&](auto wi) {
+        constexpr int W = decltype(wi)::value;
+        static_for<0, kMaxK + 1>([&](auto ki) {
+            constexpr int K = decltype(ki)::value;
+            if constexpr (MID) {
+                if constexpr (W <= 7 && kFree.v[4][W][K]) combine_even<K, 7 - W, 7>(hi[kAtH<W, K>], C, T1);
+                if constexpr (W <= 8 && kLessM.v[4][W][K])
+                    combine_even<K, 8 - W, kMaxK - 1>(hi[kAtA<W, K>], C, T0);
+            } else {
+                if constexpr (W <= 9 && kFree.v[4][W][K]) {
+                    const float h = hi[kAtH<W, K>];
+                    combine_even<K, 9 - W, kMaxK>(h, C, T1);
+                    if constexpr (W <= 8) combine_even<K, 8 - W, kMaxK - 1>(h, C, T0);
+                }
+                if constexpr (W <= 10 && kLess0.v[4][W][K])
+                    combine_even<K, 10 - W, kMaxK - 1>(hi[kAtA<W, K>], C, T0);
+                if constexpr (kLess1.v[4][W][K]) combine_even<K, 11 - W, kMaxK>(hi[kAtB<W, K>], C, T1);
+            }
+        });
+    });
+}
+
+// kappa of the limits' high halves for a pattern nibble
+__device__ __forceinline__ int kappa_hs(int which, int nibble) {  // which: 0, 1 or 2 = M
+    const int c0 = nibble & 1, c1 = (nibble >> 1) & 1, c2 = (nibble >> 2) & 1, c3 = (nibble >> 3) & 1;
+    if (which == 0) return (c0 ? 2 : 4) + (c2 ? 0 : 1) + (c3 ? 0 : 1);
+    if (which == 1) return (c0 ? 2 : 1) + (c1 ? 2 : 1);
+    return c3 ? 2 : 4;
+}
+
+template <bool MID>
+__device__ __forceinline__ void section_odd(const float* lo, const float* hi, float (&T)[kMaxW + 1]) {
+    float L[kMaxW + 1];
+#pragma unroll
+    for (int w = 0; w <= kMaxW; ++w) L[w] = lo[w];
+    constexpr int FULL = MID ? 7 : 9;
+#pragma unroll
+    for (int wh = 0; wh <= FULL; ++wh) {
+        const float h = hi[wh];
+#pragma unroll
+        for (int wl = 0; wl <= FULL - wh; ++wl) T[wh + wl] = fmaxf(T[wh + wl], __fadd_rn(h, L[wl]));
     }
-    __syncthreads();
-    val = S.red_val[0];
-    arg = S.red_arg[0];
-    for (int k = 1; k < kEncThreads / 32; ++k) {
-        const float v2 = S.red_val[k];
-        const uint32_t a2 = S.red_arg[k];
-        if (v2 > val || (v2 == val && a2 < arg)) {
-            val = v2;
-            arg = a2;
+    if constexpr (MID) {
+#pragma unroll
+        for (int wh = 0; wh <= 8; ++wh) T[8] = fmaxf(T[8], __fadd_rn(hi[kOddOffA + wh], L[8 - wh]));
+        T[8] = fmaxf(T[8], __fadd_rn(hi[kOddOffHs], lo[12]));
+    } else {
+#pragma unroll
+        for (int wh = 0; wh <= 10; ++wh) T[10] = fmaxf(T[10], __fadd_rn(hi[kOddOffA + wh], L[10 - wh]));
+        T[10] = fmaxf(T[10], __fadd_rn(hi[kOddOffHs], lo[12]));
+        static_for<0, kMaxW + 1>([&](auto wi) {
+            constexpr int WH = decltype(wi)::value;
+            if constexpr (kOddCell<kLess1, 4, WH>) T[11] = fmaxf(T[11], __fadd_rn(hi[kOddOffB + WH], L[11 - WH]));
+        });
+        T[11] = fmaxf(T[11], __fadd_rn(hi[kOddOffHs + 1], lo[13]));
+    }
+}
+
+// The section tables of one section, thread = byte pair.  EVEN: rows of k; else rows of W / 2.
+template <bool EVEN, bool MID>
+__device__ __forceinline__ void section_rows(EncShared& S, int s, int pair) {
+    float* rows0 = s == 0 ? S.F1[0][0] : (s == 1 ? S.F2[0] : S.F3[0]);
+    float* rows1 = s == 0 ? S.F1[0][1] : (s == 1 ? S.F2[1] : S.F3[1]);
+    const uint32_t byte = S.bytes[pair];
+    if constexpr (EVEN) {
+        float* r0 = rows0 + pair * kRow;
+        float* r1 = rows1 + pair * kRow;
+#pragma unroll
+        for (int k = 0; k < kRow; ++k) r0[k] = r1[k] = kNeg;
+#pragma unroll 1
+        for (int e = 0; e < 2; ++e) {
+            const uint32_t b = e ? byte ^ 0xFFu : byte;
+            float T0[kMaxK + 1], T1[kMaxK + 1];
+#pragma unroll
+            for (int k = 0; k <= kMaxK; ++k) T0[k] = T1[k] = kNeg;
+            section_even<MID>(S.lo[s] + (b & 15u) * kLoStride, S.hi[s] + (b >> 4) * kHiStride, T0, T1);
+            const int up = ones_offset(b);
+#pragma unroll
+            for (int k = 0; k <= kMaxK; ++k) {
+                if (k < kMaxK) r0[up + k] = fmaxf(r0[up + k], T0[k]);
+                r1[up + k] = fmaxf(r1[up + k], T1[k]);
+            }
+        }
+        // the rows whose high half IS a limit's: their norms depend on the nibble, so they are added in place
+#pragma unroll 1
+        for (int e = 0; e < 2; ++e) {
+            const uint32_t b = e ? byte ^ 0xFFu : byte;
+            const float* lo = S.lo[s] + (b & 15u) * kLoStride;
+            const float* hi = S.hi[s] + (b >> 4) * kHiStride;
+            const float h0 = hi[kOffHs];
+            const int k0 = kappa_hs(MID ? 2 : 0, int(b >> 4)) + ones_offset(b);
+            if constexpr (MID) r0[k0] = fmaxf(r0[k0], __fadd_rn(h0, lo[kAtC<0>]));  // 0x30000000, W = 6
+#pragma unroll
+            for (int k = 0; k < 3; ++k) r0[k0 + k] = fmaxf(r0[k0 + k], __fadd_rn(h0, lo[kOffRes0 + k]));
+            if constexpr (!MID) {
+                const float h1 = hi[kOffHs + 1];
+                const int k1 = kappa_hs(1, int(b >> 4)) + ones_offset(b);
+#pragma unroll
+                for (int k = 0; k < 5; ++k) r1[k1 + k] = fmaxf(r1[k1 + k], __fadd_rn(h1, lo[kOffRes1 + k]));
+            }
+        }
+        if (s == 0) {  // the second copy, one entry up
+            float* u0 = S.F1[1][0] + pair * kRow;
+            float* u1 = S.F1[1][1] + pair * kRow;
+            u0[0] = u1[0] = kNeg;
+#pragma unroll
+            for (int k = 0; k < kRow - 1; ++k) {
+                u0[k + 1] = r0[k];
+                u1[k + 1] = r1[k];
+            }
+        }
+    } else {
+        float T[kMaxW + 1];
+#pragma unroll
+        for (int w = 0; w <= kMaxW; ++w) T[w] = kNeg;
+#pragma unroll 1
+        for (int e = 0; e < 2; ++e) {
+            const uint32_t b = e ? byte ^ 0xFFu : byte;
+            section_odd<MID>(S.lo_odd[s] + (b & 15u) * kOddLoStride, S.hi_odd[s] + (b >> 4) * kOddHiStride, T);
+        }
+        float* r0 = rows0 + pair * kOddRow;
+        float* r1 = rows1 + pair * kOddRow;
+#pragma unroll
+        for (int k = 0; k < kOddRow; ++k) {
+            r0[k] = k < 6 ? T[k < 6 ? 2 * k : 0] : kNeg;
+            r1[k] = k < 6 ? T[k < 6 ? 2 * k + 1 : 0] : kNeg;
         }
     }
 }
 
-__global__ void __launch_bounds__(kEncThreads, 1)
+// ---------------------------------------------------------------------------
+// join and objective: thread = (end state gamma + 8 xi, parity `par` of the classes of sections 1 and 2)
+// ---------------------------------------------------------------------------
+template <int N>
+__device__ __forceinline__ void load_row(const float* row, float (&v)[N]) {
+    static_assert(N % 4 == 0, "whole quads");
+#pragma unroll
+    for (int i = 0; i < N; i += 4) {
+        const float4 q = *reinterpret_cast<const float4*>(row + i);
+        v[i] = q.x;
+        v[i + 1] = q.y;
+        v[i + 2] = q.z;
+        v[i + 3] = q.w;
+    }
+}
+
+// H[i + j + SHIFT] = max(., a[i] + b[j]) for i < NA, j < NB, two candidates per maximum.
+template <int NA, int NB, int SHIFT, int LA, int LB, int LH>
+__device__ __forceinline__ void max_plus(const float (&a)[LA], const float (&b)[LB], float (&H)[LH]) {
+    static_for<0, NA + NB - 1>([&](auto ni) {
+        constexpr int n = decltype(ni)::value;
+        constexpr int first = n < NB ? 0 : n - NB + 1, last = n < NA ? n : NA - 1, count = last - first + 1;
+        float v = H[n + SHIFT];
+        static_for<0, count / 2>([&](auto ti) {
+            constexpr int i = first + 2 * decltype(ti)::value;
+            v = max3(v, __fadd_rn(a[i], b[n - i]), __fadd_rn(a[i + 1], b[n - i - 1]));
+        });
+        if constexpr (count & 1) v = fmaxf(v, __fadd_rn(a[last], b[n - last]));
+        H[n + SHIFT] = v;
+    });
+}
+
+constexpr int kH = 20;  // entries after two sections: norms 16 i (+ 8), i < 20
+
+// Row lengths in use: even parity k <= 9 (one more in the raised copy of F1), the middle list k <= 8 (class 0)
+// and k <= 7.  Odd parity: W / 2 <= 5, the middle list 4 and 3.
+template <bool EVEN, int PAR>
+__device__ __forceinline__ void join_two(const EncShared& S, int gamma, int xi, bool odd_end, float (&H)[kH]) {
+#pragma unroll
+    for (int i = 0; i < kH; ++i) H[i] = kNeg;
+#pragma unroll 1
+    for (int alpha = 0; alpha < 8; ++alpha) {
+        const int i = alpha + 8 * xi, j = (alpha ^ gamma) + 8 * xi;
+        static_for<0, 2>([&](auto ci) {
+            constexpr int c1 = decltype(ci)::value, c2 = c1 ^ PAR;
+            if constexpr (EVEN) {
+                // norms 16 k1 + r1 and 16 k2 + r2: index k1 + k2, plus one when both residues are 8
+                const int raised = !odd_end && odd_overlap(S.bytes[i]) ? 1 : 0;
+                float a[12], b[12];
+                load_row(S.F1[raised][c1] + i * kRow, a);
+                load_row(S.F2[c2] + j * kRow, b);
+                max_plus<11, c2 ? 8 : 9, 0>(a, b, H);
+            } else {
+                float a[8], b[8];
+                load_row(S.F1[0][c1] + i * kOddRow, a);
+                load_row(S.F2[c2] + j * kOddRow, b);
+                max_plus<6, c2 ? 4 : 5, c1 & c2>(a, b, H);  // W1 + W2 = 2 (index) + (classes' parity)
+            }
+        });
+    }
+}
+
+// G[n] = best correlation of all three sections at squared norm 16 (n + m0): returns the best of G / norm.
+template <bool EVEN, int CLS3>
+__device__ __forceinline__ void objective(const EncShared& S, int m0, int end_pair, const float (&H)[kH], float& val, float& corr, int& arg) {
+    constexpr int NA = EVEN ? 19 : 10, NB = EVEN ? 10 : 6, NG = NA + NB - 1;
+    float G[NG];
+#pragma unroll
+    for (int n = 0; n < NG; ++n) G[n] = kNeg;
+    float b[EVEN ? 12 : 8];
+    load_row(S.F3[CLS3] + end_pair * (EVEN ? kRow : kOddRow), b);
+    max_plus<NA, NB, 0>(H, b, G);
+    val = kNeg;
+    corr = kNeg;
+    arg = 0;
+#pragma unroll
+    for (int n = 0; n < NG; ++n) {
+        const float v = G[n] * S.rs[n + m0];
+        if (v > val) {
+            val = v;
+            corr = G[n];
+            arg = n;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// trace of the winner: one warp per section
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ bool row_in_list(int section, int cls, int w, uint32_t row) {
+    if (section == 1) return cls ? w <= 7 : (w <= 6 || (w == 8 && row <= kLastRowMiddle0));
+    return cls ? (w <= 9 || (w == 11 && row <= kLastRowClass1)) : (w <= 8 || (w == 10 && row <= kLastRowClass0));
+}
+// correlation and kappa of a half vector, the sums in the tables' order
+__device__ __forceinline__ float half_corr(bool even, const float* w4, int nibble, uint32_t value, int& kap) {
+    float sum = 0.f;
+    kap = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int c = (nibble >> j) & 1, r = int((value >> (4 * j)) & 7u), t = (r + 1) >> 1;
+        const int v0 = (r & 1) ? 4 * t : -4 * t;
+        int y;
+        if (even) {
+            y = c ? 2 - v0 : v0;
+            kap += c ? ((r & 1) ? t * t - t : t * t + t) : t * t;
+        } else {
+            y = c ? v0 - 1 : 1 - v0;
+        }
+        sum = __fadd_rn(sum, __fmul_rn(w4[j], float(y)));
+    }
+    return sum;
+}
+
+// Finds the row (and which byte of the pair) whose correlation is `target` at index k of the section's table.
+__device__ __noinline__ void trace_section(EncShared& S, const DeviceTables* __restrict__ tab, bool even, int s, int pair, int cls, int k,
+                                           float target) {
+    const int lane = threadIdx.x & 31;
+    const int w_total = 2 * k + cls;  // odd parity: the row's weight
+    const float* w = S.w + 8 * s;
+    uint32_t row = 0;
+    uint32_t byte = S.bytes[pair];
+    bool found = false;
+    for (int e = 0; e < 2 && !found; ++e, byte ^= 0xFFu) {
+        const int nlo = int(byte & 15u), nhi = int(byte >> 4);
+        const int kap = k - ones_offset(byte);
+        const float* lo = even ? S.lo[s] + nlo * kLoStride : S.lo_odd[s] + nlo * kOddLoStride;
+        // 1. a high half with a partner in the low tables
+        uint32_t high = 0;
+        float high_corr = 0.f;
+        int high_kap = 0;
+        bool have = false;
+        for (int i0 = 0; i0 < kHalfVectors && !have; i0 += 32) {
+            const int i = i0 + lane;
+            bool hit = false;
+            uint32_t hv = 0;
+            float hc = 0.f;
+            int hk = 0;
+            if (i < kHalfVectors) {
+                hv = S.halves[i];
+                const int wh = int(hv >> 16);
+                const uint32_t v = hv & 0xFFFFu;
+                hc = half_corr(even, w + 4, nhi, v, hk);
+                const uint32_t lim = s == 1 ? kLastRowMiddle0 >> 16 : (cls ? kLastRowClass1 >> 16 : kLastRowClass0 >> 16);
+                const bool limited = !(s == 1 && cls);            // the list has a partial shell
+                const int full = s == 1 ? (cls ? 7 : 6) : (cls ? 9 : 8);
+                if (even) {
+                    auto partner = [&](int W) {  // best low half of weights W, W - 2, ...
+                        if (W < 0) return;
+                        int off = 0, last = 0;
+                        static_for<0, kMaxW + 1>([&](auto ai) {
+                            constexpr int a = decltype(ai)::value;
+                            if (W == a) { off = kAtC<a>; last = kLastC<a>; }
+                        });
+                        const int kl = kap - hk;
+                        if (kl >= 0 && kl <= last) hit = hit || __fadd_rn(hc, lo[off + kl]) == target;
+                    };
+                    partner(full - wh);
+                    if (limited && v < lim) partner(full + 2 - wh);
+                    if (limited && v == lim) {
+                        const int kl = kap - hk;
+                        const int n = cls ? 5 : 3, off = cls ? kOffRes1 : kOffRes0;
+                        if (kl >= 0 && kl < n) hit = hit || __fadd_rn(hc, lo[off + kl]) == target;
+                    }
+                } else {
+                    const int wl = w_total - wh;
+                    if (wl >= 0) {
+                        const bool whole = w_total <= full || (limited && v < lim);
+                        if (whole) hit = __fadd_rn(hc, lo[wl]) == target;
+                        else if (limited && v == lim) hit = __fadd_rn(hc, lo[cls ? 13 : 12]) == target;
+                    }
+                }
+            }
+            const uint32_t any = __ballot_sync(0xFFFFFFFFu, hit);
+            if (any) {
+                const int src = __ffs(int(any)) - 1;
+                high = __shfl_sync(0xFFFFFFFFu, hv, src);
+                high_corr = __shfl_sync(0xFFFFFFFFu, hc, src);
+                high_kap = __shfl_sync(0xFFFFFFFFu, hk, src);
+                have = true;
+            }
+        }
+        if (!have) continue;
+        // 2. the low half: sum, norm and membership decide
+        for (int i0 = 0; i0 < kHalfVectors && !found; i0 += 32) {
+            const int i = i0 + lane;
+            bool hit = false;
+            uint32_t cand = 0;
+            if (i < kHalfVectors) {
+                const uint32_t lv = S.halves[i];
+                int lk;
+                const float lc = half_corr(even, w, nlo, lv & 0xFFFFu, lk);
+                const int wt = int(high >> 16) + int(lv >> 16);
+                cand = ((high & 0xFFFFu) << 16) | (lv & 0xFFFFu);
+                hit = __fadd_rn(high_corr, lc) == target && (wt & 1) == cls && (even ? high_kap + lk == kap : wt == w_total) &&
+                      row_in_list(s, cls, wt, cand);
+            }
+            const uint32_t any = __ballot_sync(0xFFFFFFFFu, hit);
+            if (any) {
+                row = __shfl_sync(0xFFFFFFFFu, cand, __ffs(int(any)) - 1);
+                found = true;
+            }
+        }
+        if (found) break;
+    }
+    // 3. its index: the shells of a class follow one another, rows of a shell ascend
+    int wt = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) wt += rank_weight(int((row >> (4 * j)) & 7u));
+    int begin = 0, end = 0;
+    {
+        constexpr int start[2][7] = {{0, 1, 29, 155, 499, 1256, 2048}, {0, 8, 72, 296, 808, 1816, 2048}};
+        const int shell = wt >> 1;
+#pragma unroll
+        for (int q = 0; q < 6; ++q)
+            if (shell == q) {
+                begin = cls ? start[1][q] : start[0][q];
+                end = cls ? start[1][q + 1] : start[0][q + 1];
+            }
+    }
+    const uint32_t* rows = tab->paper.rows + 2048 * cls;
+    const int stride = (end - begin + 31) >> 5;
+    const int probe = begin + lane * stride;
+    const uint32_t below = __ballot_sync(0xFFFFFFFFu, probe < end && __ldg(rows + (probe < end ? probe : 0)) <= row);
+    const int block0 = begin + max(__popc(below) - 1, 0) * stride;
+    const int at = block0 + lane;
+    const uint32_t eq = __ballot_sync(0xFFFFFFFFu, lane < stride && at < end && __ldg(rows + (at < end ? at : 0)) == row);
+    if (lane == 0) {
+        S.found_row[s] = uint32_t(eq ? block0 + __ffs(int(eq)) - 1 : 0);
+        S.found_byte[s] = byte;
+        S.found_cls[s] = uint32_t(cls);
+    }
+}
+
+// Warp s < 3: the winning entry of the objective, back through the join, then the row of section s.
+__device__ __noinline__ void trace(EncShared& S, const DeviceTables* __restrict__ tab, bool even, int s, int end_pair, int par, int n) {
+    const int lane = threadIdx.x & 31;
+    const int cls3 = (even ? 0 : 1) ^ par;
+    const int row_len = even ? kRow : kOddRow;
+    const int gamma = end_pair & 7, xi = end_pair >> 3;
+    // index after two sections and of the third
+    int q = 0, k3 = 0;
+    {
+        const int j = lane, i = n - j;
+        const int nb = even ? 10 : 6, na = even ? 19 : 10;
+        const bool hit = j < nb && i >= 0 && i < na && __fadd_rn(S.win_H[i >= 0 && i < na ? i : 0], S.F3[cls3][end_pair * row_len + (j < nb ? j : 0)]) == S.win_G;
+        const uint32_t any = __ballot_sync(0xFFFFFFFFu, hit);
+        if (any) {
+            k3 = __ffs(int(any)) - 1;
+            q = n - k3;
+        }
+    }
+    // section 1's pair, class and index: lane = alpha + 8 c1 + 16 (half of the indices)
+    const float h = S.win_H[q];
+    const int alpha = lane & 7, c1 = (lane >> 3) & 1, c2 = c1 ^ par;
+    const int p1 = alpha + 8 * xi, p2 = (alpha ^ gamma) + 8 * xi;
+    const bool odd_end = odd_overlap(S.bytes[end_pair]) != 0;
+    const int raised = even && !odd_end && odd_overlap(S.bytes[p1]) ? 1 : 0;
+    const int shift = even ? 0 : (c1 & c2);
+    int hit_i = -1;
+    for (int i = lane >> 4; i < (even ? 11 : 6); i += 2) {
+        const int j = q - shift - i;
+        const int nb = even ? (c2 ? 8 : 9) : (c2 ? 4 : 5);
+        if (hit_i < 0 && j >= 0 && j < nb && __fadd_rn(S.F1[raised][c1][p1 * row_len + i], S.F2[c2][p2 * row_len + j]) == h) hit_i = i;
+    }
+    const uint32_t any = __ballot_sync(0xFFFFFFFFu, hit_i >= 0);
+    const int src = any ? __ffs(int(any)) - 1 : 0;
+    const int i1 = max(__shfl_sync(0xFFFFFFFFu, hit_i, src), 0);
+    const int w_p1 = __shfl_sync(0xFFFFFFFFu, p1, src), w_p2 = __shfl_sync(0xFFFFFFFFu, p2, src);
+    const int w_c1 = __shfl_sync(0xFFFFFFFFu, c1, src), w_c2 = w_c1 ^ par;
+    const int w_raised = __shfl_sync(0xFFFFFFFFu, raised, src), w_shift = __shfl_sync(0xFFFFFFFFu, shift, src);
+    const int j2 = max(q - w_shift - i1, 0);
+    if (s == 0) trace_section(S, tab, even, 0, w_p1, w_c1, max(i1 - w_raised, 0), S.F1[w_raised][w_c1][w_p1 * row_len + i1]);
+    else if (s == 1) trace_section(S, tab, even, 1, w_p2, w_c2, j2, S.F2[w_c2][w_p2 * row_len + j2]);
+    else trace_section(S, tab, even, 2, end_pair, cls3, k3, S.F3[cls3][end_pair * row_len + k3]);
+}
+
+template <bool EVEN>
+__device__ __forceinline__ void search_parity(EncShared& S, const DeviceTables* __restrict__ tab, float& best_val, uint64_t& best_word) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    {   // section tables: warps 0, 1 = section 0, warps 2, 3 = section 1, warps 4, 5 = section 2
+        const int s = tid >> 6, pair = tid & 63;
+        if (s == 1) section_rows<EVEN, true>(S, 1, pair);
+        else section_rows<EVEN, false>(S, s, pair);
+    }
+    __syncthreads();
+    float H[kH];
+    float val = kNeg, corr = kNeg;
+    int arg = 0;
+    if (tid < 128) {
+        const int end_pair = tid & 63, par = tid >> 6;
+        const int gamma = end_pair & 7, xi = end_pair >> 3;
+        const bool odd_end = odd_overlap(S.bytes[end_pair]) != 0;
+        // squared norm = 16 (index + m0)
+        const int m0 = EVEN ? (odd_end ? 1 : 0) : 2;
+        if (par == 0) {
+            join_two<EVEN, 0>(S, gamma, xi, odd_end, H);
+            objective<EVEN, EVEN ? 0 : 1>(S, m0, end_pair, H, val, corr, arg);
+        } else {
+            join_two<EVEN, 1>(S, gamma, xi, odd_end, H);
+            objective<EVEN, EVEN ? 1 : 0>(S, m0, end_pair, H, val, corr, arg);
+        }
+        // the warp's best; the objective of a non-zero block is positive at its best, so bit patterns compare like values
+        const uint32_t bits = val > 0.f ? __float_as_uint(val) : 0u;
+        const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, bits);
+        const uint32_t who = __ballot_sync(0xFFFFFFFFu, bits == top);
+        if (lane == __ffs(int(who)) - 1) {
+            S.red_val[warp] = top ? val : kNeg;
+            S.red_arg[warp] = uint32_t(tid);
+        }
+    }
+    __syncthreads();
+    float top = S.red_val[0];
+    uint32_t winner = S.red_arg[0];
+#pragma unroll
+    for (int k = 1; k < 4; ++k)
+        if (S.red_val[k] > top) {
+            top = S.red_val[k];
+            winner = S.red_arg[k];
+        }
+    if (top > best_val) {  // uniform
+        best_val = top;
+        if (uint32_t(tid) == winner) {
+#pragma unroll
+            for (int i = 0; i < kH; ++i) S.win_H[i] = H[i];
+            S.win_G = corr;
+            S.win_arg = arg;
+        }
+        __syncthreads();
+        if (warp < 3) trace(S, tab, EVEN, warp, int(winner) & 63, int(winner) >> 6, S.win_arg);
+        __syncthreads();
+        if (warp == 0) {
+            const uint32_t c1 = S.found_byte[0], c2 = S.found_byte[1], c3 = S.found_byte[2];
+            const uint32_t b1 = c1 >> 7, b3 = c3 >> 7, s8 = (b1 ? ~c1 : c1) & 63u;
+            const uint32_t leaves = tab->paper.branches[16 * s8 + (lane & 15)] & 0xFFu;
+            const uint32_t eq = __ballot_sync(0xFFFFFFFFu, leaves == c2);
+            const uint32_t b2 = eq ? uint32_t(__ffs(int(eq)) - 1) & 15u : 0u;
+            const uint32_t i2 = S.found_row[1] + (S.found_cls[1] ? uint32_t(kMiddleClass0) : 0u);
+            best_word = uint64_t(S.found_row[0]) | (uint64_t(i2) << 11) | (uint64_t(S.found_row[2]) << 22) | (uint64_t(s8) << 33) |
+                        (uint64_t(b1) << 39) | (uint64_t(b2) << 40) | (uint64_t(b3) << 44) | (uint64_t(EVEN ? 0 : 1) << 45) |
+                        (uint64_t(S.found_cls[0]) << 46);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kEncThreads, kEncCtasPerSm)
 k_encode(const float* __restrict__ w, const float* __restrict__ sigma, const DeviceTables* __restrict__ tab,
          unsigned char* __restrict__ codes, float* __restrict__ cosine, size_t nblocks) {
     extern __shared__ __align__(16) unsigned char enc_smem[];
     EncShared& S = *reinterpret_cast<EncShared*>(enc_smem);
     const int tid = threadIdx.x;
-    const int sg = tid >> 7, ct = tid & 127;  // section group, pattern-byte index
-    // --- tables, once per CTA ---
-    for (int i = tid; i < 4096; i += kEncThreads) S.rows[i] = tab->paper.rows[i];
-    for (int i = tid; i < 1024; i += kEncThreads) S.branches[i] = tab->paper.branches[i];
-    if (tid < 128) {
-        S.prefixes[tid] = tab->paper.prefixes[tid];
-        S.suffixes[tid] = tab->paper.suffixes[tid];
-    }
-    if (tid < 64) S.incoming_count[tid] = 0;
-    if (tid < 32) S.V2[tid >> 3][tid & 7] = rank_value(tid >> 3, tid & 7) * rank_value(tid >> 3, tid & 7);
-    __syncthreads();
-    for (int i = tid; i < 1024; i += kEncThreads) {  // order within a state's list does not matter for the maximum,
-        const int s16 = S.branches[i] >> 8;          // but it decides ties: sort below
-        const int slot = atomicAdd(&S.incoming_count[s16], 1);
-        if (slot < 16) S.incoming[s16][slot] = uint16_t(i);  // i = 16 s8 + b2
-    }
-    __syncthreads();
-    if (tid < 64) {  // insertion sort of 16 entries: the same order in every CTA and run
-        for (int a = 1; a < 16; ++a) {
-            const uint16_t v = S.incoming[tid][a];
-            int b = a - 1;
-            while (b >= 0 && S.incoming[tid][b] > v) {
-                S.incoming[tid][b + 1] = S.incoming[tid][b];
-                --b;
-            }
-            S.incoming[tid][b + 1] = v;
-        }
-    }
+    if (tid < 64) S.bytes[tid] = uint8_t(pair_byte(tid));
+    if (tid < 32) S.rs[tid] = tab->paper.rsqrt16m[tid];
+    for (int i = tid; i < kHalfVectors; i += kEncThreads) S.halves[i] = kHalfList.v[i];
     const float gain0 = tab->gain[0], gain1 = tab->gain[1];
-    const int my_byte = even_byte(ct);
-    const int my_lo = my_byte & 15, my_hi = my_byte >> 4;
-    __syncthreads();
 
     for (size_t block = blockIdx.x; block < nblocks; block += gridDim.x) {
         if (tid < 24) S.w[tid] = w[block * 24 + tid];
-        if (tid == 0) {
-            S.best_val = kNeg;
-            S.best_corr = 0.f;
-            S.best_norm = 0;
-            S.best_path = 0;
-            S.best_field[0] = S.best_field[1] = S.best_field[2] = 0;
-        }
         __syncthreads();
-        for (int i = tid; i < 3 * 8 * 4 * 8; i += kEncThreads) {
-            const int rho = i & 7, o = (i >> 3) & 3, j = (i >> 5) & 7, s = i >> 8;
-            S.A[s][j][o][rho] = S.w[8 * s + j] * float(rank_value(o, rho));
-        }
         float wn2 = 0.f;
 #pragma unroll
         for (int j = 0; j < 24; ++j) wn2 = fmaf(S.w[j], S.w[j], wn2);
-        __syncthreads();
         if (wn2 == 0.f) {  // a zero block encodes as the all-zero word
             if (tid < 6) codes[block * 6 + tid] = 0;
             if (tid == 0 && cosine) cosine[block] = 0.f;
+            __syncthreads();
             continue;
         }
-
-        for (int p = 0; p < 2; ++p) {
-            // ---------------- section tables ----------------
-            for (int i = ct; i < 2 * 20 * 128; i += 128) (&S.T[sg][0][0][0])[i] = kNeg;
-            // thread (row of the batch = ct / 2, half of the byte = ct & 1) tabulates 16 patterns while the whole
-            // group scans the batch before: one barrier per batch
-            auto produce = [&](int buf, int cls, int b0) {
-                const int len = list_length(sg, cls);
-                const int r = ct >> 1, half = ct & 1;
-                if (ct < 2 * kEncBatch && b0 + r < len) {
-                    const uint32_t rw = S.rows[2048 * cls + b0 + r];
-                    float P[16];
-                    int Nn[16];
-                    P[0] = 0.f;
-                    Nn[0] = 0;
-                    float d[4];
-                    int dn[4];
-#pragma unroll
-                    for (int jj = 0; jj < 4; ++jj) {
-                        const int j = 4 * half + jj, rho = (rw >> (4 * j)) & 7;
-                        const float a0 = S.A[sg][j][p][rho], a1 = S.A[sg][j][p + 2][rho];
-                        const int n0 = S.V2[p][rho], n1 = S.V2[p + 2][rho];
-                        P[0] += a0;
-                        Nn[0] += n0;
-                        d[jj] = a1 - a0;
-                        dn[jj] = n1 - n0;
-                    }
-#pragma unroll
-                    for (int jj = 0; jj < 4; ++jj)
-#pragma unroll
-                        for (int m = 0; m < (1 << jj); ++m) {
-                            P[m | (1 << jj)] = P[m] + d[jj];
-                            Nn[m | (1 << jj)] = Nn[m] + dn[jj];
-                        }
-#pragma unroll
-                    for (int m = 0; m < 16; ++m)
-                        S.rowtab[buf][sg][(half * 16 + m) * kEncStride + r] = make_uint2(__float_as_uint(P[m]), uint32_t(Nn[m]) * 32u);
-                }
-            };
-            // the batches of both classes as one sequence
-            const int nb0 = (list_length(sg, 0) + kEncBatch - 1) / kEncBatch, nb1 = (list_length(sg, 1) + kEncBatch - 1) / kEncBatch;
-            produce(0, 0, 0);
-            group_barrier(sg);
-            for (int bi = 0; bi < nb0 + nb1; ++bi) {
-                const int buf = bi & 1;
-                const int cls = bi < nb0 ? 0 : 1, b0 = (bi < nb0 ? bi : bi - nb0) * kEncBatch;
-                if (bi + 1 < nb0 + nb1) {
-                    const int nbi = bi + 1;
-                    produce(buf ^ 1, nbi < nb0 ? 0 : 1, (nbi < nb0 ? nbi : nbi - nb0) * kEncBatch);
-                }
-                const int nb = min(kEncBatch, list_length(sg, cls) - b0);
-                const uint2* lo_tab = &S.rowtab[buf][sg][my_lo * kEncStride];
-                const uint2* hi_tab = &S.rowtab[buf][sg][(16 + my_hi) * kEncStride];
-                // a candidate's cell: the tables hold 32 x norm, a column's cells are 512 bytes apart and the norm is
-                // 16 k + residue, so  cell = column + 32 norm - 32 residue  (one three-input addition)
-                const uint32_t res32 = uint32_t(norm_residue(p, cls, my_byte)) * 32u;
-                const uint32_t t_even = smem_u32(&S.T[sg][0][cls * 10][ct]) - res32;
-                const uint32_t t_odd = smem_u32(&S.T[sg][1][cls * 10][ct]) - res32;
-                auto update = [&](uint32_t column, uint2 lo, uint2 hi) {
-                    const uint32_t cell = column + lo.y + hi.y;
-                    float v;
-                    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(cell));
-                    v = fmaxf(v, __uint_as_float(lo.x) + __uint_as_float(hi.x));
-                    asm volatile("st.shared.f32 [%0], %1;" ::"r"(cell), "f"(v) : "memory");
-                };
-                // At odd parity every coordinate is +-(2 rank + 1) whatever the pattern byte, so a row's norm is its
-                // cost and the rows of a class come sorted by cost: nearly every batch has ONE norm, the same for
-                // all bytes, and its best correlation is a running maximum in a register.
-                const uint32_t n_first = lo_tab[0].y + hi_tab[0].y, n_last = lo_tab[nb - 1].y + hi_tab[nb - 1].y;
-                if (p == 1 && nb == kEncBatch && n_first == n_last) {
-                    float m0 = kNeg, m1 = kNeg;
-#pragma unroll
-                    for (int r = 0; r < kEncBatch; r += 2) {
-                        m0 = fmaxf(m0, __uint_as_float(lo_tab[r].x) + __uint_as_float(hi_tab[r].x));
-                        m1 = fmaxf(m1, __uint_as_float(lo_tab[r + 1].x) + __uint_as_float(hi_tab[r + 1].x));
-                    }
-                    const uint32_t cell = t_even + n_first;
-                    float v;
-                    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(cell));
-                    v = fmaxf(v, fmaxf(m0, m1));
-                    asm volatile("st.shared.f32 [%0], %1;" ::"r"(cell), "f"(v) : "memory");
-                } else if (nb == kEncBatch) {
-#pragma unroll
-                    for (int r = 0; r < kEncBatch; r += 2) {  // two independent read-modify-write chains, loads first
-                        const uint2 lo0 = lo_tab[r], hi0 = hi_tab[r], lo1 = lo_tab[r + 1], hi1 = hi_tab[r + 1];
-                        const uint32_t cell0 = t_even + lo0.y + hi0.y, cell1 = t_odd + lo1.y + hi1.y;
-                        float v0, v1;
-                        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v0) : "r"(cell0));
-                        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v1) : "r"(cell1));
-                        v0 = fmaxf(v0, __uint_as_float(lo0.x) + __uint_as_float(hi0.x));
-                        v1 = fmaxf(v1, __uint_as_float(lo1.x) + __uint_as_float(hi1.x));
-                        asm volatile("st.shared.f32 [%0], %1;" ::"r"(cell0), "f"(v0) : "memory");
-                        asm volatile("st.shared.f32 [%0], %1;" ::"r"(cell1), "f"(v1) : "memory");
-                    }
+        {   // half tables: warps 0..2 the even parity of section 0..2, warps 3..5 the odd one; lanes 0..15 the low half
+            const int s = (tid >> 5) % 3, nibble = tid & 15;
+            const bool high = (tid & 16) != 0, odd = tid >= 96;
+            if (!odd) {
+                float* lo = S.lo[s] + nibble * kLoStride;
+                float* hi = S.hi[s] + nibble * kHiStride;
+                if (s == 1) {
+                    if (high) half_even<true, true>(S.w + 12, nibble, hi);
+                    else half_even<false, true>(S.w + 8, nibble, lo);
                 } else {
-                    for (int r = 0; r < nb; ++r) update(t_even, lo_tab[r], hi_tab[r]);
+                    if (high) half_even<true, false>(S.w + 8 * s + 4, nibble, hi);
+                    else half_even<false, false>(S.w + 8 * s, nibble, lo);
                 }
-                group_barrier(sg);
-            }
-            for (int i = ct; i < 20 * 128; i += 128)  // fold the odd rows' copy into the even rows'
-                (&S.T[sg][0][0][0])[i] = fmaxf((&S.T[sg][0][0][0])[i], (&S.T[sg][1][0][0])[i]);
-            __syncthreads();
-
-            // ---------------- join: first cut ----------------
-            for (int e = tid; e < 64 * 2 * 20; e += kEncThreads) {
-                const int n8 = e % 20, cls = (e / 20) & 1, s8 = e / 40;
-                float best = kNeg;
-#pragma unroll
-                for (int b1 = 0; b1 < 2; ++b1) {
-                    const int byte = S.prefixes[2 * s8 + b1];
-                    const int rem = 8 * n8 - norm_residue(p, cls, byte);
-                    if (rem >= 0 && (rem & 15) == 0 && (rem >> 4) < 10) best = fmaxf(best, S.T[0][0][cls * 10 + (rem >> 4)][even_index(byte)]);
-                }
-                S.F1[s8][cls][n8] = best;
-            }
-            __syncthreads();
-            // ---------------- second cut ----------------
-            // thread = (state after the branch, class parity): all 39 entries of its column are accumulated in
-            // registers (two sets, for the two possible norm residues of section 2's byte) over the 16 branches
-            // into the state, the class of section 1, the 20 norms after section 1 and the 10 of section 2
-            if (tid < 128) {
-                const int s16 = tid >> 1, par = tid & 1;
-                float h0[38], h1[38];  // index n8 + 2 k2, residue 0 / 8 of section 2
-#pragma unroll
-                for (int i = 0; i < 38; ++i) h0[i] = h1[i] = kNeg;
-                for (int in = 0; in < 16; ++in) {
-                    const int sb = S.incoming[s16][in], s8 = sb >> 4;
-                    const int byte2 = S.branches[sb] & 0xFF, ci2 = even_index(byte2);
-                    for (int cls1 = 0; cls1 < 2; ++cls1) {
-                        const int cls2 = par ^ cls1;
-                        float a[20], b[10];
-#pragma unroll
-                        for (int n8 = 0; n8 < 20; ++n8) a[n8] = S.F1[s8][cls1][n8];
-#pragma unroll
-                        for (int k2 = 0; k2 < 10; ++k2) b[k2] = S.T[1][0][cls2 * 10 + k2][ci2];
-                        if (norm_residue(p, cls2, byte2)) {
-#pragma unroll
-                            for (int n8 = 0; n8 < 20; ++n8)
-#pragma unroll
-                                for (int k2 = 0; k2 < 10; ++k2) h1[n8 + 2 * k2] = fmaxf(h1[n8 + 2 * k2], a[n8] + b[k2]);
-                        } else {
-#pragma unroll
-                            for (int n8 = 0; n8 < 20; ++n8)
-#pragma unroll
-                                for (int k2 = 0; k2 < 10; ++k2) h0[n8 + 2 * k2] = fmaxf(h0[n8 + 2 * k2], a[n8] + b[k2]);
-                        }
-                    }
-                }
-                // an absent entry stays far below every real one (sums of two absent entries are more negative still)
-#pragma unroll
-                for (int q = 0; q < 39; ++q) {
-                    float v = q < 38 ? h0[q] : kNeg;
-                    if (q >= 1) v = fmaxf(v, h1[q - 1]);
-                    S.H[q][tid] = v > kNegTest ? v : kNeg;
+            } else {
+                float* lo = S.lo_odd[s] + nibble * kOddLoStride;
+                float* hi = S.hi_odd[s] + nibble * kOddHiStride;
+                if (s == 1) {
+                    if (high) half_odd<true, true>(S.w + 12, nibble, hi);
+                    else half_odd<false, true>(S.w + 8, nibble, lo);
+                } else {
+                    if (high) half_odd<true, false>(S.w + 8 * s + 4, nibble, hi);
+                    else half_odd<false, false>(S.w + 8 * s, nibble, lo);
                 }
             }
-            __syncthreads();
-            // ---------------- last section and the objective ----------------
-            float val = kNeg;
-            uint32_t arg = 0xFFFFFFFFu;
-            if (tid < 256) {
-                const int s16 = tid >> 2, b3 = (tid >> 1) & 1, par = tid & 1;
-                const int byte3 = S.suffixes[2 * s16 + b3], ci3 = even_index(byte3);
-                const int cls3 = p ^ par, res3 = norm_residue(p, cls3, byte3);
-                for (int q = 0; q < 39; ++q) {
-                    const float a = S.H[q][s16 * 2 + par];
-                    if (a < kNegTest) continue;
-#pragma unroll
-                    for (int k3 = 0; k3 < 10; ++k3) {
-                        const float b = S.T[2][0][cls3 * 10 + k3][ci3];
-                        const int n = 8 * q + 16 * k3 + res3;
-                        if (b > kNegTest && n > 0) {
-                            const float v = (a + b) / sqrtf(float(n));
-                            const uint32_t code = (uint32_t(tid) << 16) | (uint32_t(q) << 8) | uint32_t(k3);
-                            if (v > val || (v == val && code < arg)) {
-                                val = v;
-                                arg = code;
-                            }
-                        }
-                    }
-                }
-            }
-            cta_argmax(S, val, arg);
-            if (val > S.best_val) {  // uniform: resolve the path and the rows while this parity's tables are alive
-                const int wt = int(arg >> 16), q = int(arg >> 8) & 0xFF, k3 = int(arg & 0xFF);
-                const int s16 = wt >> 2, b3 = (wt >> 1) & 1, par = wt & 1;
-                // which branch, class and norms attain the winning entry of the second cut: the first, in (branch,
-                // class, norm) order, whose sum is the entry (the same additions as above, so the match is exact)
-                uint32_t back = 0;
-                {
-                    const float target = S.H[q][s16 * 2 + par];
-                    bool found = false;
-                    for (int in = 0; in < 16 && !found; ++in) {
-                        const int sb = S.incoming[s16][in], s8c = sb >> 4, b2c = sb & 15;
-                        const int byte2 = S.branches[sb] & 0xFF, ci2 = even_index(byte2);
-                        for (int c1 = 0; c1 < 2 && !found; ++c1) {
-                            const int c2 = par ^ c1, res2 = norm_residue(p, c2, byte2) >> 3;
-                            for (int kk = 0; kk < 10 && !found; ++kk) {
-                                const int n8c = q - 2 * kk - res2;
-                                if (n8c < 0 || n8c >= 20) continue;
-                                if (S.F1[s8c][c1][n8c] + S.T[1][0][c2 * 10 + kk][ci2] == target) {
-                                    back = uint32_t(s8c) | (uint32_t(b2c) << 6) | (uint32_t(c1) << 10) |
-                                           (uint32_t(n8c) << 11) | (uint32_t(kk) << 16);
-                                    found = true;
-                                }
-                            }
-                        }
-                    }
-                }
-                const int s8 = back & 63, b2 = (back >> 6) & 15, cls1 = (back >> 10) & 1, n8 = (back >> 11) & 31,
-                          k2 = (back >> 16) & 15;
-                const int cls2 = par ^ cls1, cls3 = p ^ par;
-                // the prefix that attains F1
-                int b1 = 0, k1 = 0;
-                {
-                    float bestv = kNeg;
-                    for (int bb = 0; bb < 2; ++bb) {
-                        const int byte = S.prefixes[2 * s8 + bb];
-                        const int rem = 8 * n8 - norm_residue(p, cls1, byte);
-                        if (rem >= 0 && (rem & 15) == 0 && (rem >> 4) < 10) {
-                            const float v = S.T[0][0][cls1 * 10 + (rem >> 4)][even_index(byte)];
-                            if (v > bestv) {
-                                bestv = v;
-                                b1 = bb;
-                                k1 = rem >> 4;
-                            }
-                        }
-                    }
-                }
-                const int bytes[3] = {S.prefixes[2 * s8 + b1], S.branches[16 * s8 + b2] & 0xFF, S.suffixes[2 * s16 + b3]};
-                const int clss[3] = {cls1, cls2, cls3};
-                const int ks[3] = {k1, k2, k3};
-                // second scan: group sg looks for the row of section sg (largest correlation at that byte, class, k)
-                {
-                    const int byte = bytes[sg], cls = clss[sg], kk = ks[sg];
-                    const int len = list_length(sg, cls), base = 2048 * cls;
-                    float rv = kNeg;
-                    uint32_t ra = 0xFFFFFFFFu;
-                    for (int i = ct; i < len; i += 128) {
-                        const uint32_t rw = S.rows[base + i];
-                        float corr = 0.f;
-                        int nn = 0;
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const int rho = (rw >> (4 * j)) & 7, o = p + 2 * ((byte >> j) & 1);
-                            corr += S.A[sg][j][o][rho];
-                            const int v = rank_value(o, rho);
-                            nn += v * v;
-                        }
-                        if ((nn >> 4) == kk && (corr > rv || (corr == rv && uint32_t(i) < ra))) {
-                            rv = corr;
-                            ra = uint32_t(i);
-                        }
-                    }
-                    // reduce within the group of 128 threads (four warps)
-#pragma unroll
-                    for (int o = 16; o >= 1; o >>= 1) {
-                        const float v2 = __shfl_xor_sync(0xFFFFFFFFu, rv, o);
-                        const uint32_t a2 = __shfl_xor_sync(0xFFFFFFFFu, ra, o);
-                        if (v2 > rv || (v2 == rv && a2 < ra)) {
-                            rv = v2;
-                            ra = a2;
-                        }
-                    }
-                    __syncthreads();
-                    if ((tid & 31) == 0) {
-                        S.red_val[tid >> 5] = rv;
-                        S.red_arg[tid >> 5] = ra;
-                    }
-                    __syncthreads();
-                    if (ct == 0) {
-                        float bv = S.red_val[4 * sg];
-                        uint32_t ba = S.red_arg[4 * sg];
-                        for (int k = 1; k < 4; ++k) {
-                            const float v2 = S.red_val[4 * sg + k];
-                            const uint32_t a2 = S.red_arg[4 * sg + k];
-                            if (v2 > bv || (v2 == bv && a2 < ba)) {
-                                bv = v2;
-                                ba = a2;
-                            }
-                        }
-                        S.found_field[sg] = ba == 0xFFFFFFFFu ? 0 : int(ba);
-                    }
-                    __syncthreads();
-                }
-                if (tid == 0) {
-                    const int n_total = 8 * q + 16 * k3 + norm_residue(p, cls3, bytes[2]);
-                    S.best_val = val;
-                    S.best_norm = n_total;
-                    S.best_corr = val * sqrtf(float(n_total));
-                    S.best_path = uint32_t(s8) | (uint32_t(b1) << 6) | (uint32_t(b2) << 7) | (uint32_t(b3) << 11) |
-                                  (uint32_t(p) << 12) | (uint32_t(cls1) << 13);
-                    S.best_field[0] = S.found_field[0];
-                    S.best_field[1] = cls2 ? kMiddleClass0 + S.found_field[1] : S.found_field[1];
-                    S.best_field[2] = S.found_field[2];
-                }
-            }
-            __syncthreads();
         }
+        __syncthreads();
+        float best_val = kNeg;
+        uint64_t best_word = 0;
+        search_parity<false>(S, tab, best_val, best_word);
+        __syncthreads();
+        search_parity<true>(S, tab, best_val, best_word);
 
         if (tid == 0) {
-            const uint32_t path = S.best_path;
             const float sg_ = sigma ? sigma[block] : 1.f;
             // gain bit: argmin_g (gain sigma)^2 - 2 gain sigma <w, y> / |y|
-            const float c = S.best_val;
+            const float c = best_val;
             const float e0 = gain0 * sg_ * (gain0 * sg_ - 2.f * c), e1 = gain1 * sg_ * (gain1 * sg_ - 2.f * c);
-            const uint64_t gbit = e1 < e0 ? 1u : 0u;
-            const uint64_t word = uint64_t(S.best_field[0]) | (uint64_t(S.best_field[1]) << 11) |
-                                  (uint64_t(S.best_field[2]) << 22) | (uint64_t(path & 63u) << 33) |
-                                  (uint64_t((path >> 6) & 1u) << 39) | (uint64_t((path >> 7) & 15u) << 40) |
-                                  (uint64_t((path >> 11) & 1u) << 44) | (uint64_t((path >> 12) & 1u) << 45) |
-                                  (uint64_t((path >> 13) & 1u) << 46) | (gbit << 47);
+            const uint64_t word = best_word | (uint64_t(e1 < e0 ? 1u : 0u) << 47);
+#pragma unroll
             for (int k = 0; k < 6; ++k) codes[block * 6 + k] = uint8_t(word >> (8 * k));
-            if (cosine) cosine[block] = S.best_val / sqrtf(wn2);
+            if (cosine) cosine[block] = best_val / sqrtf(wn2);
         }
         __syncthreads();
     }
@@ -498,7 +1071,8 @@ cudaError_t launch_encode(const float* w, const float* sigma, const void* table,
     static PerDeviceOnce once;
     e = once.run([smem] { return cudaFuncSetAttribute(k_encode, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
     if (e != cudaSuccess) return e;
-    const unsigned grid = unsigned(nblocks < size_t(sms) ? nblocks : size_t(sms));
+    const size_t resident = size_t(sms) * kEncCtasPerSm;
+    const unsigned grid = unsigned(nblocks < resident ? nblocks : resident);
     k_encode<<<grid, kEncThreads, smem, s>>>(w, sigma, static_cast<const DeviceTables*>(table), codes, cosine, nblocks);
     return cudaGetLastError();
 }

@@ -163,6 +163,11 @@ int build_device_tables(DeviceTables* out, const float* gain2) {
     rc = build_rows(&out->paper, &n0);
     if (rc) return rc;
     if (n0 != kMiddleClass0) return -20;
+    if (out->paper.rows[2047] != kLastRowClass0 || out->paper.rows[4095] != kLastRowClass1 ||
+        out->paper.rows[kMiddleClass0 - 1] != kLastRowMiddle0 || row_cost(out->paper.rows[2047]) != 88 ||
+        row_cost(out->paper.rows[4095]) != 96 || row_cost(out->paper.rows[kMiddleClass0 - 1]) != 72 ||
+        row_cost(out->paper.rows[2048 + 807]) != 64 || row_cost(out->paper.rows[2048 + 808]) != 80)
+        return -29;
     out->paper.rsqrt16m[0] = 0.0f;
     for (int m = 1; m < 32; ++m) out->paper.rsqrt16m[m] = static_cast<float>(1.0 / std::sqrt(16.0 * m));
     out->gain[0] = gain2 ? gain2[0] : 4.3156f;

@@ -20,6 +20,9 @@ constexpr uint32_t kTableMagic = 0x54455442u;  // "TETB"
 constexpr uint32_t kTableVersion = 7;
 constexpr int kRank4Slots = 32;                // slots at the start of each class whose pool is patched
 constexpr int kMiddleClass0 = 1240;            // N0 of Sec. 3.3 (checked at build)
+// The last row of a class's 2048 and of the middle list's class 0 (checked at build): each cuts a shell of equal
+// cost at this packed value; the middle list's class 1 ends with a whole shell.
+constexpr uint32_t kLastRowClass0 = 0x11030011u, kLastRowClass1 = 0x00222011u, kLastRowMiddle0 = 0x30001010u;
 
 // Everything tetra_build_table copies to the device, in one blob.
 struct DeviceTables {
