@@ -42,8 +42,8 @@
 namespace tetra {
 namespace {
 
-constexpr int kEncThreads = 192;
-constexpr int kEncCtasPerSm = 3;
+constexpr int kEncThreads = 192;   // per block of weights
+constexpr int kEncGroups = 3;      // blocks of weights a CTA works on, in step
 constexpr float kNeg = -1.0e30f;
 
 // ---------------------------------------------------------------------------
@@ -230,7 +230,7 @@ struct EncShared {
     uint32_t found_byte[3];
     uint32_t found_cls[3];
 };
-static_assert(sizeof(EncShared) <= 74 * 1024, "three CTAs per SM");
+static_assert(sizeof(EncShared) * kEncGroups <= 226 * 1024, "one CTA per SM");
 
 // h(a), a < 8, and h'(x), x < 8: representatives of the bytes of the two [8,4] codes up to complement.
 __device__ __forceinline__ uint32_t hamming_byte(uint32_t v, uint32_t b0, uint32_t b1, uint32_t b2) {
@@ -924,9 +924,10 @@ __device__ __noinline__ void trace(EncShared& S, const DeviceTables* __restrict_
 }
 
 template <bool EVEN>
-__device__ __forceinline__ void search_parity(EncShared& S, const DeviceTables* __restrict__ tab, float& best_val, uint64_t& best_word) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    {   // section tables: warps 0, 1 = section 0, warps 2, 3 = section 1, warps 4, 5 = section 2
+__device__ __forceinline__ void search_parity(EncShared& S, const DeviceTables* __restrict__ tab, int tid, bool live, float& best_val,
+                                              uint64_t& best_word) {
+    const int warp = tid >> 5, lane = tid & 31;
+    if (live) {  // section tables: warps 0, 1 = section 0, warps 2, 3 = section 1, warps 4, 5 = section 2
         const int s = tid >> 6, pair = tid & 63;
         if (s == 1) section_rows<EVEN, true>(S, 1, pair);
         else section_rows<EVEN, false>(S, s, pair);
@@ -935,7 +936,7 @@ __device__ __forceinline__ void search_parity(EncShared& S, const DeviceTables* 
     float H[kH];
     float val = kNeg, corr = kNeg;
     int arg = 0;
-    if (tid < 128) {
+    if (live && tid < 128) {
         const int end_pair = tid & 63, par = tid >> 6;
         const int gamma = end_pair & 7, xi = end_pair >> 3;
         const bool odd_end = odd_overlap(S.bytes[end_pair]) != 0;
@@ -958,63 +959,68 @@ __device__ __forceinline__ void search_parity(EncShared& S, const DeviceTables* 
         }
     }
     __syncthreads();
-    float top = S.red_val[0];
-    uint32_t winner = S.red_arg[0];
+    bool better = false;
+    uint32_t winner = 0;
+    if (live) {
+        float top = S.red_val[0];
+        winner = S.red_arg[0];
 #pragma unroll
-    for (int k = 1; k < 4; ++k)
-        if (S.red_val[k] > top) {
-            top = S.red_val[k];
-            winner = S.red_arg[k];
-        }
-    if (top > best_val) {  // uniform
-        best_val = top;
-        if (uint32_t(tid) == winner) {
+        for (int k = 1; k < 4; ++k)
+            if (S.red_val[k] > top) {
+                top = S.red_val[k];
+                winner = S.red_arg[k];
+            }
+        better = top > best_val;  // the same for all threads of the group
+        if (better) {
+            best_val = top;
+            if (uint32_t(tid) == winner) {
 #pragma unroll
-            for (int i = 0; i < kH; ++i) S.win_H[i] = H[i];
-            S.win_G = corr;
-            S.win_arg = arg;
+                for (int i = 0; i < kH; ++i) S.win_H[i] = H[i];
+                S.win_G = corr;
+                S.win_arg = arg;
+            }
         }
-        __syncthreads();
-        if (warp < 3) trace(S, tab, EVEN, warp, int(winner) & 63, int(winner) >> 6, S.win_arg);
-        __syncthreads();
-        if (warp == 0) {
-            const uint32_t c1 = S.found_byte[0], c2 = S.found_byte[1], c3 = S.found_byte[2];
-            const uint32_t b1 = c1 >> 7, b3 = c3 >> 7, s8 = (b1 ? ~c1 : c1) & 63u;
-            const uint32_t leaves = tab->paper.branches[16 * s8 + (lane & 15)] & 0xFFu;
-            const uint32_t eq = __ballot_sync(0xFFFFFFFFu, leaves == c2);
-            const uint32_t b2 = eq ? uint32_t(__ffs(int(eq)) - 1) & 15u : 0u;
-            const uint32_t i2 = S.found_row[1] + (S.found_cls[1] ? uint32_t(kMiddleClass0) : 0u);
-            best_word = uint64_t(S.found_row[0]) | (uint64_t(i2) << 11) | (uint64_t(S.found_row[2]) << 22) | (uint64_t(s8) << 33) |
-                        (uint64_t(b1) << 39) | (uint64_t(b2) << 40) | (uint64_t(b3) << 44) | (uint64_t(EVEN ? 0 : 1) << 45) |
-                        (uint64_t(S.found_cls[0]) << 46);
-        }
+    }
+    if (!__syncthreads_or(better)) return;
+    if (better && warp < 3) trace(S, tab, EVEN, warp, int(winner) & 63, int(winner) >> 6, S.win_arg);
+    __syncthreads();
+    if (better && warp == 0) {
+        const uint32_t c1 = S.found_byte[0], c2 = S.found_byte[1], c3 = S.found_byte[2];
+        const uint32_t b1 = c1 >> 7, b3 = c3 >> 7, s8 = (b1 ? ~c1 : c1) & 63u;
+        const uint32_t leaves = tab->paper.branches[16 * s8 + (lane & 15)] & 0xFFu;
+        const uint32_t eq = __ballot_sync(0xFFFFFFFFu, leaves == c2);
+        const uint32_t b2 = eq ? uint32_t(__ffs(int(eq)) - 1) & 15u : 0u;
+        const uint32_t i2 = S.found_row[1] + (S.found_cls[1] ? uint32_t(kMiddleClass0) : 0u);
+        best_word = uint64_t(S.found_row[0]) | (uint64_t(i2) << 11) | (uint64_t(S.found_row[2]) << 22) | (uint64_t(s8) << 33) |
+                    (uint64_t(b1) << 39) | (uint64_t(b2) << 40) | (uint64_t(b3) << 44) | (uint64_t(EVEN ? 0 : 1) << 45) |
+                    (uint64_t(S.found_cls[0]) << 46);
     }
 }
 
-__global__ void __launch_bounds__(kEncThreads, kEncCtasPerSm)
+__global__ void __launch_bounds__(kEncThreads * kEncGroups, 1)
 k_encode(const float* __restrict__ w, const float* __restrict__ sigma, const DeviceTables* __restrict__ tab,
          unsigned char* __restrict__ codes, float* __restrict__ cosine, size_t nblocks) {
     extern __shared__ __align__(16) unsigned char enc_smem[];
-    EncShared& S = *reinterpret_cast<EncShared*>(enc_smem);
-    const int tid = threadIdx.x;
+    const int group = threadIdx.x / kEncThreads, tid = threadIdx.x - group * kEncThreads;
+    EncShared& S = reinterpret_cast<EncShared*>(enc_smem)[group];
     if (tid < 64) S.bytes[tid] = uint8_t(pair_byte(tid));
     if (tid < 32) S.rs[tid] = tab->paper.rsqrt16m[tid];
     for (int i = tid; i < kHalfVectors; i += kEncThreads) S.halves[i] = kHalfList.v[i];
     const float gain0 = tab->gain[0], gain1 = tab->gain[1];
 
-    for (size_t block = blockIdx.x; block < nblocks; block += gridDim.x) {
-        if (tid < 24) S.w[tid] = w[block * 24 + tid];
+    // every group of every CTA takes the same number of turns; the first groups of all CTAs come first, so that few
+    // blocks spread over all SMs
+    const size_t per_turn = size_t(gridDim.x) * kEncGroups;
+    for (size_t first = 0; first < nblocks; first += per_turn) {
+        const size_t block = first + size_t(group) * gridDim.x + blockIdx.x;
+        const bool mine = block < nblocks;
+        if (tid < 24) S.w[tid] = mine ? w[block * 24 + tid] : 0.f;
         __syncthreads();
         float wn2 = 0.f;
 #pragma unroll
         for (int j = 0; j < 24; ++j) wn2 = fmaf(S.w[j], S.w[j], wn2);
-        if (wn2 == 0.f) {  // a zero block encodes as the all-zero word
-            if (tid < 6) codes[block * 6 + tid] = 0;
-            if (tid == 0 && cosine) cosine[block] = 0.f;
-            __syncthreads();
-            continue;
-        }
-        {   // half tables: warps 0..2 the even parity of section 0..2, warps 3..5 the odd one; lanes 0..15 the low half
+        const bool live = wn2 != 0.f;  // a zero block encodes as the all-zero word
+        if (live) {  // half tables: warps 0..2 the even parity of section 0..2, warps 3..5 the odd one; lanes 0..15 the low half
             const int s = (tid >> 5) % 3, nibble = tid & 15;
             const bool high = (tid & 16) != 0, odd = tid >= 96;
             if (!odd) {
@@ -1042,19 +1048,19 @@ k_encode(const float* __restrict__ w, const float* __restrict__ sigma, const Dev
         __syncthreads();
         float best_val = kNeg;
         uint64_t best_word = 0;
-        search_parity<false>(S, tab, best_val, best_word);
+        search_parity<false>(S, tab, tid, live, best_val, best_word);
         __syncthreads();
-        search_parity<true>(S, tab, best_val, best_word);
+        search_parity<true>(S, tab, tid, live, best_val, best_word);
 
-        if (tid == 0) {
+        if (mine && tid == 0) {
             const float sg_ = sigma ? sigma[block] : 1.f;
             // gain bit: argmin_g (gain sigma)^2 - 2 gain sigma <w, y> / |y|
             const float c = best_val;
             const float e0 = gain0 * sg_ * (gain0 * sg_ - 2.f * c), e1 = gain1 * sg_ * (gain1 * sg_ - 2.f * c);
-            const uint64_t word = best_word | (uint64_t(e1 < e0 ? 1u : 0u) << 47);
+            const uint64_t word = live ? best_word | (uint64_t(e1 < e0 ? 1u : 0u) << 47) : 0u;
 #pragma unroll
             for (int k = 0; k < 6; ++k) codes[block * 6 + k] = uint8_t(word >> (8 * k));
-            if (cosine) cosine[block] = best_val / sqrtf(wn2);
+            if (cosine) cosine[block] = live ? best_val / sqrtf(wn2) : 0.f;
         }
         __syncthreads();
     }
@@ -1067,13 +1073,12 @@ cudaError_t launch_encode(const float* w, const float* sigma, const void* table,
     int sms = 0;
     cudaError_t e = device_sms(&sms);
     if (e != cudaSuccess) return e;
-    const int smem = int(sizeof(EncShared));
+    const int smem = int(sizeof(EncShared)) * kEncGroups;
     static PerDeviceOnce once;
     e = once.run([smem] { return cudaFuncSetAttribute(k_encode, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
     if (e != cudaSuccess) return e;
-    const size_t resident = size_t(sms) * kEncCtasPerSm;
-    const unsigned grid = unsigned(nblocks < resident ? nblocks : resident);
-    k_encode<<<grid, kEncThreads, smem, s>>>(w, sigma, static_cast<const DeviceTables*>(table), codes, cosine, nblocks);
+    const unsigned grid = unsigned(nblocks < size_t(sms) ? nblocks : size_t(sms));
+    k_encode<<<grid, kEncThreads * kEncGroups, smem, s>>>(w, sigma, static_cast<const DeviceTables*>(table), codes, cosine, nblocks);
     return cudaGetLastError();
 }
 
