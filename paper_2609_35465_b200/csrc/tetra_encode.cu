@@ -333,7 +333,7 @@ __device__ __forceinline__ void half_even(const float* w4, int nibble, float* ou
     float hs0 = 0.f, hs1 = 0.f;  // correlations of the limits' high halves
     static_for<0, 4>([&](auto ji) {
         constexpr int J = decltype(ji)::value;
-        constexpr int D0 = kLimit0.hi[J], D1 = kLimit1.hi[J], DM = kLimitM.hi[J];  // digits of the limits' high halves
+        [[maybe_unused]] constexpr int D0 = kLimit0.hi[J], D1 = kLimit1.hi[J], DM = kLimitM.hi[J];  // digits of the limits' high halves
         const int c = (nibble >> J) & 1;
         float a[5];
         products_even(w4[J], c, a);
@@ -441,7 +441,7 @@ __device__ __forceinline__ void half_odd(const float* w4, int nibble, float* out
     float hs0 = 0.f, hs1 = 0.f;
     static_for<0, 4>([&](auto ji) {
         constexpr int J = decltype(ji)::value;
-        constexpr int D0 = kLimit0.hi[J], D1 = kLimit1.hi[J], DM = kLimitM.hi[J];  // digits of the limits' high halves
+        [[maybe_unused]] constexpr int D0 = kLimit0.hi[J], D1 = kLimit1.hi[J], DM = kLimitM.hi[J];  // digits of the limits' high halves
         float a[5];
         products_odd(w4[J], (nibble >> J) & 1, a);
         if constexpr (HIGH) {

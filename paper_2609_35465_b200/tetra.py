@@ -4,6 +4,10 @@ Argument marshalling only: every step of the decode-and-multiply path runs in
 the CUDA kernels of libtetra_b200.so.  PyTorch supplies device memory and
 streams.  There is no CPU fallback: if the library is missing or a call fails,
 an exception is raised.
+
+The calls of a decode step, of the encoder and of loading go through _binding.so
+(csrc/binding.cpp), which checks the tensors and calls the library in well under
+a microsecond; plans, tables and the comparison arms go through ctypes.
 """
 import ctypes as C
 import os
@@ -36,6 +40,22 @@ class Problem(C.Structure):
 
 
 _lib = None
+_nat = None
+
+
+def _native():
+    """The native half of this binding; raises if it has not been built."""
+    global _nat
+    if _nat is None:
+        if not os.path.exists(LIB_PATH):
+            lib()                       # raises: not built
+        try:
+            from . import _binding
+        except ImportError as e:
+            raise TetraError("binding not built (run python -m paper_2609_35465_b200.build): %s" % e)
+        _binding.setup(LIB_PATH, TetraError)
+        _nat = _binding
+    return _nat
 
 
 def lib():
@@ -172,39 +192,21 @@ def tetra_codes_bytes(N: int, nblocks: int) -> int:
 
 def tetra_pack_codes(codes: torch.Tensor, table: torch.Tensor, N: int, nblocks: int, out=None, stream=None):
     """codes: uint8 [N, nblocks, 6] file order on the device -> packed uint8 tensor."""
-    assert codes.dtype == torch.uint8 and codes.is_cuda and codes.is_contiguous()
-    assert codes.numel() == N * nblocks * WORD_BYTES
-    nbytes = tetra_codes_bytes(N, nblocks)
-    if out is None:
-        out = torch.empty(nbytes, dtype=torch.uint8, device=codes.device)
-    assert out.numel() >= nbytes
-    _check(lib().tetra_pack_codes(_ptr(codes), _ptr(table), _ptr(out), N, nblocks, _stream(stream)),
-           "tetra_pack_codes")
-    return out
+    return (_nat or _native()).pack_codes(codes, table, N, nblocks, out, stream)
 
 
 def tetra_decode_packed(packed: torch.Tensor, table: torch.Tensor, N: int, nblocks: int, want_mg=True, stream=None):
-    y = torch.empty((N, nblocks, BLOCK), dtype=torch.int8, device=packed.device)
-    mg = torch.empty((N, nblocks, 2), dtype=torch.uint8, device=packed.device) if want_mg else None
-    _check(lib().tetra_decode_packed(_ptr(packed), _ptr(table), _ptr(y), _ptr(mg), N, nblocks, _stream(stream)),
-           "tetra_decode_packed")
-    return y, mg
+    return (_nat or _native()).decode_packed(packed, table, N, nblocks, want_mg, stream)
 
 
 def tetra_gemv(codes, row_scales, table, x, y, N: int, K: int, batch: int = 1, stream=None):
     """Zero-pad rule: ceil(K/24) words per row."""
-    _need_gemv("tetra_gemv", codes, row_scales, x, y, N, K, batch, None, False)
-    _check(lib().tetra_gemv(_ptr(codes), _ptr(row_scales), _ptr(table), _ptr(x), _ptr(y), N, K, batch,
-                            _stream(stream)), "tetra_gemv")
-    return y
+    return (_nat or _native()).gemv(codes, row_scales, table, x, y, N, K, batch, stream)
 
 
 def tetra_gemv_tail(codes, row_scales, table, x, y, N: int, K: int, batch: int = 1, tail=None, stream=None):
     """The paper's rule: floor(K/24) words per row plus a float16 tail."""
-    _need_gemv("tetra_gemv_tail", codes, row_scales, x, y, N, K, batch, tail, tail is not None)
-    _check(lib().tetra_gemv_tail(_ptr(codes), _ptr(row_scales), _ptr(table), _ptr(x), _ptr(y), N, K, batch,
-                                 _ptr(tail), _stream(stream)), "tetra_gemv_tail")
-    return y
+    return (_nat or _native()).gemv_tail(codes, row_scales, table, x, y, N, K, batch, tail, stream)
 
 
 def make_problems(items):
@@ -222,7 +224,7 @@ def make_problems(items):
 
 def tetra_gemv_list(problems, table, stream=None):
     """Batch-1 products of a short list (ctypes array from make_problems, at most LIST_MAX) in one launch."""
-    _check(lib().tetra_gemv_list(problems, len(problems), _ptr(table), _stream(stream)), "tetra_gemv_list")
+    (_nat or _native()).gemv_list(problems, table, stream)
 
 
 def tetra_grouped_workspace_bytes(problems) -> int:
@@ -237,7 +239,7 @@ def tetra_gemv_grouped_plan(problems, workspace: torch.Tensor, stream=None):
 
 def tetra_gemv_grouped_run(workspace: torch.Tensor, table, stream=None):
     """One step of a planned list: activation pre-pass + persistent GEMV kernel."""
-    _check(lib().tetra_gemv_grouped_run(_ptr(workspace), _ptr(table), _stream(stream)), "tetra_gemv_grouped_run")
+    (_nat or _native()).grouped_run(workspace, table, stream)
 
 
 def tetra_gemv_grouped(problems, table, workspace: torch.Tensor, stream=None):
@@ -278,10 +280,7 @@ def tetra_gemv_noalloc(codes, row_scales, table, x, y, N: int, K: int, tail=None
     """Batch-1 product for callers that may not allocate device memory: the
     scratch buffer lives inside the library (a fixed array, K <= NOALLOC_MAX_K).
     Calls on one device share that array, so they must not overlap on the GPU."""
-    _need_gemv("tetra_gemv_noalloc", codes, row_scales, x, y, N, K, 1, tail, tail is not None)
-    _check(lib().tetra_gemv_noalloc(_ptr(codes), _ptr(row_scales), _ptr(table), _ptr(x), _ptr(y), N, K,
-                                    _ptr(tail), _stream(stream)), "tetra_gemv_noalloc")
-    return y
+    return (_nat or _native()).gemv_noalloc(codes, row_scales, table, x, y, N, K, tail, stream)
 
 
 def tetra_batched_workspace_bytes(N: int, K: int) -> int:
@@ -291,13 +290,9 @@ def tetra_batched_workspace_bytes(N: int, K: int) -> int:
 def tetra_gemv_batched(codes, row_scales, table, x, y, N: int, K: int, batch: int, tail=None, workspace=None,
                        stream=None):
     """1..16 activation vectors at once: decode once per block, tensor-core contraction per block."""
-    _need_gemv("tetra_gemv_batched", codes, row_scales, x, y, N, K, batch, tail, tail is not None)
     if workspace is None:
         workspace = torch.empty(tetra_batched_workspace_bytes(N, K), dtype=torch.uint8, device=y.device)
-    _check(lib().tetra_gemv_batched(_ptr(codes), _ptr(row_scales), _ptr(table), _ptr(x), _ptr(y), N, K, batch,
-                                    _ptr(tail), _ptr(workspace), workspace.numel(), _stream(stream)),
-           "tetra_gemv_batched")
-    return y
+    return (_nat or _native()).gemv_batched(codes, row_scales, table, x, y, N, K, batch, tail, workspace, stream)
 
 
 # ---------------------------------------------------------------------------
@@ -312,49 +307,20 @@ def tetra_q4_packed_bytes(N: int, K: int, G: int) -> int:
 
 def tetra_q4_pack(q, scale, offset, N: int, K: int, G: int, stream=None):
     """File-order matrix (uint8 [N, K/2], float16 [N, K/G] x 2, all on the device) -> packed device buffer."""
-    packed = torch.empty(tetra_q4_packed_bytes(N, K, G), dtype=torch.uint8, device=q.device)
-    _need(q, N * (K // 2), "tetra_q4_pack q")
-    _need(scale, 2 * N * (K // G), "tetra_q4_pack scale")
-    _need(offset, 2 * N * (K // G), "tetra_q4_pack offset")
-    _check(lib().tetra_q4_pack(_ptr(q), _ptr(scale), _ptr(offset), _ptr(packed), packed.numel(), N, K, G,
-                               _stream(stream)), "tetra_q4_pack")
-    return packed
-
-
-def _need_q4(what, packed, x, y, N, K, G, batch):
-    n = lib().tetra_q4_packed_bytes(N, K, G)
-    if n == 0 or batch <= 0:
-        return  # the library rejects the shape
-    _need(packed, n, what + " packed")
-    _need(x, 2 * batch * K, what + " x")
-    _need(y, 4 * batch * N, what + " y")
+    return (_nat or _native()).q4_pack(q, scale, offset, N, K, G, stream)
 
 
 def tetra_q4_gemv(packed, x, y, N: int, K: int, G: int, batch: int = 1, stream=None):
-    _need_q4("tetra_q4_gemv", packed, x, y, N, K, G, batch)
-    _check(lib().tetra_q4_gemv(_ptr(packed), _ptr(x), _ptr(y), N, K, G, batch, _stream(stream)), "tetra_q4_gemv")
-    return y
+    return (_nat or _native()).q4_gemv(packed, x, y, N, K, G, batch, stream)
 
 
 def tetra_q4_rows(packed, ids, out, N: int, K: int, G: int, stream=None):
-    _need_q4("tetra_q4_rows", packed, None, None, N, K, G, 1)
-    _need(ids, 4 * int(ids.numel()), "tetra_q4_rows ids")
-    _need(out, 2 * int(ids.numel()) * K, "tetra_q4_rows out")
-    _check(lib().tetra_q4_rows(_ptr(packed), _ptr(ids), int(ids.numel()), _ptr(out), N, K, G, _stream(stream)),
-           "tetra_q4_rows")
-    return out
+    return (_nat or _native()).q4_rows(packed, ids, out, N, K, G, stream)
 
 
 def tetra_encode_blocks(w, table, sigma=None, want_cosine=True, stream=None):
     """w: float32 [n, 24] on the device -> (codes uint8 [n, 6] in file order, cosines float32 [n] or None)."""
-    n = w.numel() // 24
-    _need(w, 4 * 24 * n, "tetra_encode_blocks w")
-    _need(sigma, 4 * n, "tetra_encode_blocks sigma")
-    codes = torch.empty((n, 6), dtype=torch.uint8, device=w.device)
-    cos = torch.empty(n, dtype=torch.float32, device=w.device) if want_cosine else None
-    _check(lib().tetra_encode_blocks(_ptr(w), _ptr(sigma), _ptr(table), _ptr(codes), _ptr(cos), n, _stream(stream)),
-           "tetra_encode_blocks")
-    return codes, cos
+    return (_nat or _native()).encode_blocks(w, table, sigma, want_cosine, stream)
 
 
 def make_q4_problems(items):
@@ -378,4 +344,4 @@ def tetra_q4_list_plan(problems, G: int, stream=None) -> torch.Tensor:
 
 
 def tetra_q4_list_run(workspace: torch.Tensor, G: int, stream=None):
-    _check(lib().tetra_q4_list_run(_ptr(workspace), G, _stream(stream)), "tetra_q4_list_run")
+    (_nat or _native()).q4_list_run(workspace, G, stream)
