@@ -318,10 +318,11 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
 
 // Float16 weights of the rows of some tokens (Sec. 4.4).  A thread takes the 16 columns 16 t .. of one 64-column
 // tile: one 16-byte load (a quarter of the 64 bytes in which the tile holds the row and its neighbour eight rows
-// away), the row's scale record, 32 bytes out.  PER tokens at a time, their loads all in flight together: the chain
-// token number -> weights -> store is what a short call consists of.  WIDE: `out` allows 16-byte stores.
+// away), the row's scale record, 32 bytes out.  WIDE: `out` allows 16-byte stores.  A short call is the chain token
+// number -> weights -> store, and only resident warps hide it: one token per CTA row (two or four tokens a thread,
+// their loads together, take 5.8 and 8.4 us where one takes 4.6).
 // 1024 tokens x 4096: 7.9 us with a thread per four columns, now 4.6 us.
-template <int G, int PER, bool WIDE>
+template <int G, bool WIDE>
 __global__ void __launch_bounds__(256) k_q4_rows(const unsigned char* __restrict__ packed, const int32_t* __restrict__ ids,
                                                  int count, __half* __restrict__ out, int N, int K) {
     constexpr int CH = q4_chunk_bytes(G);
@@ -331,50 +332,37 @@ __global__ void __launch_bounds__(256) k_q4_rows(const unsigned char* __restrict
     if (at >= per_row) return;
     const int c = 16 * at, group = c / G, j = (c % G) >> 6, t = at & 3;
     pdl_wait();  // the ids may come from the preceding kernel
-    for (int tok0 = blockIdx.y * PER; tok0 < count; tok0 += gridDim.y * PER) {
-        int row[PER];
-        uint4 w[PER];
-        uint32_t rec[PER];
-#pragma unroll
-        for (int i = 0; i < PER; ++i) row[i] = tok0 + i < count ? __ldg(ids + tok0 + i) : -1;
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            if (row[i] < 0 || row[i] >= N) {
-                row[i] = -1;
-                w[i] = make_uint4(0u, 0u, 0u, 0u);
-                rec[i] = 0u;
-                continue;
-            }
-            const int strip = row[i] >> 5, rr = row[i] & 31, h = rr >> 4, g = rr & 7;
+    for (int tok = blockIdx.y; tok < count; tok += gridDim.y) {
+        const int row = __ldg(ids + tok);
+        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+        uint32_t rec = 0u;
+        if (row >= 0 && row < N) {  // otherwise the record stays zero, and with it the row
+            const int strip = row >> 5, rr = row & 31, h = rr >> 4, g = rr & 7;
             const unsigned char* chunk = packed + (size_t(strip) * groups + group) * CH;
-            w[i] = __ldg(reinterpret_cast<const uint4*>(chunk + j * 1024 + h * 512 + (g * 4 + t) * 16));
-            rec[i] = __ldg(reinterpret_cast<const uint32_t*>(chunk + (G / 64) * 1024 + rr * 4));
+            w = __ldg(reinterpret_cast<const uint4*>(chunk + j * 1024 + h * 512 + (g * 4 + t) * 16));
+            rec = __ldg(reinterpret_cast<const uint32_t*>(chunk + (G / 64) * 1024 + rr * 4));
         }
+        const int half = (row >> 3) & 1;
+        const float2 sc = __half22float2(*reinterpret_cast<const __half2*>(&rec));
+        const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+        uint32_t r[8];
 #pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            if (tok0 + i >= count) break;
-            const int half = (row[i] >> 3) & 1;  // a row number outside the matrix: the record is zero, so the row is
-            const float2 sc = __half22float2(*reinterpret_cast<const __half2*>(&rec[i]));
-            const uint32_t ww[4] = {w[i].x, w[i].y, w[i].z, w[i].w};
-            uint32_t r[8];
+        for (int m = 0; m < 4; ++m) {
+            const uint32_t v = ww[m] >> (8 * half);
+            const float n0 = float(v & 15u), n1 = float((v >> 16) & 15u);        // columns 4 m, 4 m + 1
+            const float n2 = float((v >> 4) & 15u), n3 = float((v >> 20) & 15u);  // columns 4 m + 2, 4 m + 3
+            const __half2 lo = __floats2half2_rn(__fmaf_rn(sc.x, n0, sc.y), __fmaf_rn(sc.x, n1, sc.y));
+            const __half2 hi = __floats2half2_rn(__fmaf_rn(sc.x, n2, sc.y), __fmaf_rn(sc.x, n3, sc.y));
+            r[2 * m] = *reinterpret_cast<const uint32_t*>(&lo);
+            r[2 * m + 1] = *reinterpret_cast<const uint32_t*>(&hi);
+        }
+        __half* dst = out + size_t(tok) * K + c;
+        if (WIDE) {
+            reinterpret_cast<uint4*>(dst)[0] = make_uint4(r[0], r[1], r[2], r[3]);
+            reinterpret_cast<uint4*>(dst)[1] = make_uint4(r[4], r[5], r[6], r[7]);
+        } else {
 #pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                const uint32_t v = ww[m] >> (8 * half);
-                const float n0 = float(v & 15u), n1 = float((v >> 16) & 15u);        // columns 4 m, 4 m + 1
-                const float n2 = float((v >> 4) & 15u), n3 = float((v >> 20) & 15u);  // columns 4 m + 2, 4 m + 3
-                const __half2 lo = __floats2half2_rn(__fmaf_rn(sc.x, n0, sc.y), __fmaf_rn(sc.x, n1, sc.y));
-                const __half2 hi = __floats2half2_rn(__fmaf_rn(sc.x, n2, sc.y), __fmaf_rn(sc.x, n3, sc.y));
-                r[2 * m] = *reinterpret_cast<const uint32_t*>(&lo);
-                r[2 * m + 1] = *reinterpret_cast<const uint32_t*>(&hi);
-            }
-            __half* dst = out + size_t(tok0 + i) * K + c;
-            if (WIDE) {
-                reinterpret_cast<uint4*>(dst)[0] = make_uint4(r[0], r[1], r[2], r[3]);
-                reinterpret_cast<uint4*>(dst)[1] = make_uint4(r[4], r[5], r[6], r[7]);
-            } else {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) reinterpret_cast<uint2*>(dst)[k] = make_uint2(r[2 * k], r[2 * k + 1]);
-            }
+            for (int k = 0; k < 4; ++k) reinterpret_cast<uint2*>(dst)[k] = make_uint2(r[2 * k], r[2 * k + 1]);
         }
     }
 }
@@ -489,12 +477,9 @@ int tetra_q4_rows(const void* packed_dev, const int32_t* ids_dev, int count, voi
     if (rc != TETRA_OK) return rc;
     if (count < 0) return TETRA_ERR_SHAPE;
     if (!aligned(packed_dev, 16) || !aligned(ids_dev, 4) || !aligned(out_dev, 8)) return TETRA_ERR_ALIGN;
-    // A thread per 16 columns; one token at a time until two thousand CTAs are out (a few per SM hide the latency of
-    // the loads), then four.
+    // a thread per 16 columns, a CTA row per token
     const int threads = K / 16 < 256 ? K / 16 : 256, gx = (K / 16 + threads - 1) / threads;
-    const int per = (long long)count * gx <= 2048 ? 1 : 4;
-    const long long turns = (count + per - 1) / per;
-    const int gy = int(turns < 65535 ? turns : 65535);
+    const int gy = count < 65535 ? count : 65535;
     const bool wide = aligned(out_dev, 16);
     auto launch = [&](auto kernel) {
         cudaLaunchAttribute attr[1];
@@ -509,12 +494,8 @@ int tetra_q4_rows(const void* packed_dev, const int32_t* ids_dev, int count, voi
         return cuda_status(cudaLaunchKernelEx(&cfg, kernel, static_cast<const unsigned char*>(packed_dev), ids_dev, count,
                                               static_cast<__half*>(out_dev), N, K));
     };
-    if (G == 128) {
-        if (per == 1) return wide ? launch(k_q4_rows<128, 1, true>) : launch(k_q4_rows<128, 1, false>);
-        return wide ? launch(k_q4_rows<128, 4, true>) : launch(k_q4_rows<128, 4, false>);
-    }
-    if (per == 1) return wide ? launch(k_q4_rows<64, 1, true>) : launch(k_q4_rows<64, 1, false>);
-    return wide ? launch(k_q4_rows<64, 4, true>) : launch(k_q4_rows<64, 4, false>);
+    if (G == 128) return wide ? launch(k_q4_rows<128, true>) : launch(k_q4_rows<128, false>);
+    return wide ? launch(k_q4_rows<64, true>) : launch(k_q4_rows<64, false>);
 }
 
 }  // extern "C"
