@@ -45,7 +45,7 @@ constexpr int kPassTiles = 8;  // 16-row x 1-column tiles per warp and pass (fou
 //   chunk 2 n     = B-fragment registers (plane 0, h 0), (0, 1), (1, 0), (1, 1)
 //   chunk 2 n + 1 = (2, 0), (2, 1), step of vector 8 n + 2 t, step of vector 8 n + 2 t + 1
 // where the lane multiplies with vector 8 n + lane / 4, t = lane % 4, register h = 0 holds coordinates
-// 4 t .. 4 t + 3 and h = 1 coordinates 16 + 4 t .. 16 + 4 t + 3 (24..31 and unused vectors are zero), and
+// of the decoder's word t and h = 1 those of word 4 + t (words 6, 7 and unused vectors are zero), and
 // the steps are those of the lane's two result columns.  A column takes ng x 1 KiB (ng = 1 or 2 groups).
 // The image lives in shared memory only: the CTA builds it for a chunk of its passes at a time.
 constexpr int kBatGroupWords = 2 * 32 * 4;
@@ -56,17 +56,18 @@ constexpr int kBatGroupWords = 2 * 32 * 4;
 // into the three int8 planes.  A float16 x_j is held exactly when |x_j| >= 2^(E-12), E the exponent of the
 // column's largest magnitude; smaller ones are rounded to a multiple of the step 2^(E-22).
 struct ImageTask {
-    float v[8];  // coordinates 4 t .. 4 t + 3 and (t < 2) 16 + 4 t .. 19 + 4 t of the column
+    float v[8];  // the coordinates of the decoder's words t and (t < 2) 4 + t of the column
 };
 __device__ __forceinline__ void image_load(const __half* __restrict__ x, int K, int batch, int col, int vec, int t,
                                            ImageTask& T) {
     const __half* xv = x + size_t(vec) * K;
-    const int k0 = 24 * col + 4 * t;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        T.v[i] = (vec < batch && k0 + i < K) ? __half2float(__ldg(xv + k0 + i)) : 0.f;
-        T.v[4 + i] = (vec < batch && t < 2 && k0 + 16 + i < K) ? __half2float(__ldg(xv + k0 + 16 + i)) : 0.f;
-    }
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int k = 24 * col + word_coordinate(4 * h + t, i);
+            T.v[4 * h + i] = (vec < batch && (h == 0 || t < 2) && k < K) ? __half2float(__ldg(xv + k)) : 0.f;
+        }
 }
 // group_base: shared-memory address of the column's 1 KiB group for the vector's group of eight.
 __device__ __forceinline__ void image_store(const ImageTask& T, uint32_t group_base, int vec, int t) {
@@ -254,10 +255,7 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const unsigned char* __rest
                 asm volatile("ld.shared.u16 %0, [%1];" : "=r"(w1) : "r"(src + lane_w1 + (j % RB) * 2 * kBatRingGroup + (j / RB) * 32));
                 FastBlock fb;
                 fast_decode<false>(sm_tab, w0, w1, fb);
-                int n2 = int(fb.goff);  // the squared norm on top of the gain's column of the scale table: the scale's address
-#pragma unroll
-                for (int k = 0; k < 6; ++k) n2 = dp4a_ss(fb.y[k], fb.y[k], n2);
-                const float scale = lds32f(uint32_t(n2));  // -gain[g] / sqrt(16 m), with -y in the tile
+                const float scale = lds32f(scale_address(fb));  // -gain[g] / sqrt(16 m), with -8 y in the tile
                 const int tile_id = (j % RB) * PC + 2 * (j / RB);  // + colsel
                 unsigned char* dst = tiles + (tile_id + colsel) * kTileBytes + row16 * kTileRow;
                 // coordinates 24..31 of a tile row meet zeros in the activation image, so those eight bytes
@@ -301,9 +299,7 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const unsigned char* __rest
                         // this lane's results: rows g (i = 0, 1) and g + 8 (i = 2, 3), vectors 8 n + 2 t4 + (i & 1)
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            int dot;  // dh * 65536 + dm * 256 + dl, exact (|dot| < 2^31), on the multiply-add pipe
-                            asm("mad.lo.s32 %0, %1, 256, %2;" : "=r"(dot) : "r"(dm[i]), "r"(dl[i]));
-                            asm("mad.lo.s32 %0, %1, 65536, %0;" : "+r"(dot) : "r"(dh[i]));
+                            const int dot = combine_planes(dh[i], dm[i], dl[i]);
                             acc[rb][n][i] = fmaf(float(dot), (i < 2 ? s_lo : s_hi) * ((i & 1) ? step_odd : step_even),
                                                  acc[rb][n][i]);
                         }
@@ -479,10 +475,7 @@ k_gemv_few(const DeviceTables* __restrict__ tab, const unsigned char* __restrict
                 fast_decode<true>(sm_tab, w0.y, w1pair, f[rb][1]);
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    int n2 = int(f[rb][j].goff);
-#pragma unroll
-                    for (int k = 0; k < 6; ++k) n2 = dp4a_ss(f[rb][j].y[k], f[rb][j].y[k], n2);
-                    scale[rb][j] = lds32f(uint32_t(n2));
+                    scale[rb][j] = lds32f(scale_address(f[rb][j]));
                 }
             }
             const uint32_t img = image + in_chunk * (V * kQuadBytes);
@@ -513,8 +506,8 @@ k_gemv_few(const DeviceTables* __restrict__ tab, const unsigned char* __restrict
                     }
 #pragma unroll
                 for (int rb = 0; rb < RB; ++rb) {
-                    const int dot0 = dh[rb][0] * 65536 + (dm[rb][0] * 256 + dm[rb][1]);
-                    const int dot1 = dh[rb][2] * 65536 + (dm[rb][2] * 256 + dm[rb][3]);
+                    const int dot0 = combine_planes(dh[rb][0], dm[rb][0], dm[rb][1]);
+                    const int dot1 = combine_planes(dh[rb][2], dm[rb][2], dm[rb][3]);
                     acc[rb][0][v] = fmaf(float(dot0), scale[rb][0] * step, acc[rb][0][v]);
                     acc[rb][1][v] = fmaf(float(dot1), scale[rb][1] * step, acc[rb][1][v]);
                 }
@@ -530,8 +523,8 @@ k_gemv_few(const DeviceTables* __restrict__ tab, const unsigned char* __restrict
                                bh[pr].x, bh[pr].y, dh, true);
                     }
                     // exact int32 dot products of -y with the 24-bit activations (the scale carries the other minus sign)
-                    const int dot0 = dh[0] * 65536 + (dm[0] * 256 + dm[1]);
-                    const int dot1 = dh[2] * 65536 + (dm[2] * 256 + dm[3]);
+                    const int dot0 = combine_planes(dh[0], dm[0], dm[1]);
+                    const int dot1 = combine_planes(dh[2], dm[2], dm[3]);
                     acc[rb][0][v] = fmaf(float(dot0), scale[rb][0] * step, acc[rb][0][v]);
                     acc[rb][1][v] = fmaf(float(dot1), scale[rb][1] * step, acc[rb][1][v]);
                 }

@@ -5,13 +5,9 @@
 //     word in file order, reading the paper-format tables.  Used by
 //     tetra_decode_blocks and by the paper-design GEMV.
 //   * the fast decoder: works on the re-ordered 48-bit device word written by
-//     tetra_pack_codes and on tables staged in shared memory.  It produces the
-//     lattice point (negated) as packed int8, four coordinates per register and
-//     one PRMT per four: a selector nibble is c | rank << 1 and the 8-byte PRMT
-//     pool holds the rank lists of Sec. 3.3 for the block's parity p.
-//     Branch-free: rows with a coordinate of rank 4 sit in the first 32 slots of
-//     their class, and for those slots one select swaps in a pool word whose
-//     rank-2 entries are the rank-4 values.
+//     tetra_pack_codes and on tables staged in shared memory.  It produces MINUS
+//     EIGHT TIMES the lattice point as packed int8, four coordinates per
+//     register, with two logic operations per four (see fast_decode).
 #pragma once
 #include <cstdint>
 #include <cuda_fp16.h>
@@ -115,37 +111,35 @@ __device__ __forceinline__ void decode_file_word(const PaperTables* T, uint64_t 
 
 // ---------------------------------------------------------------------------
 // Device word (written by the pack kernel).  48 bits = w0 (32) + w1 (16):
-//   w0: [0..10] i1'  [11] r  [12..22] i3'  [23] q = p^r  [24..27] a  [28..31] b
-//   w1: [0..10] i2  [11..14] x  [15] g
-// i1', i3' are the row indices after the per-class permutation row_perm (class r
-// for section 1, class r3 = p^r^delta for section 3).  (a, b, x) are the Turyn
-// coordinates of the trellis path: the three pattern bytes are h(a)+h'(x),
-// h(b)+h'(x), h(a)+h(b)+h'(x).
+//   w0: [2..12] i1  [13] r  [14..24] i3  [25] g  [26..29] a  [30, 31, 0, 1] b
+//   w1: [0..10] i2  [11] p  [12..15] x
+// (a, b, x) are the Turyn coordinates of the trellis path: the three pattern
+// bytes are h(a)+h'(x), h(b)+h'(x), h(a)+h(b)+h'(x).  i1 with r above it is a
+// byte offset into the row table as it stands; b is one rotation away from its
+// place in a table offset; p sits where i2's byte offset ends and below x, so
+// that (x, p) is one five-bit index.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void file_to_device_word(uint64_t w, const DeviceTables* tab, uint32_t* w0, uint32_t* w1) {
-    uint32_t i1 = uint32_t(w & 0x7FF), i3 = uint32_t((w >> 22) & 0x7FF);
-    const uint32_t i2 = uint32_t((w >> 11) & 0x7FF);
-    const uint32_t path = uint32_t((w >> 33) & 0xFFF);
+__device__ __forceinline__ void file_to_device_word(uint64_t w, uint32_t abx, uint32_t* w0, uint32_t* w1) {
+    const uint32_t i1 = uint32_t(w & 0x7FF), i2 = uint32_t((w >> 11) & 0x7FF), i3 = uint32_t((w >> 22) & 0x7FF);
     const uint32_t p = uint32_t((w >> 45) & 1), r = uint32_t((w >> 46) & 1), g = uint32_t((w >> 47) & 1);
-    const uint32_t r3 = p ^ r ^ uint32_t(i2 >= uint32_t(kMiddleClass0));  // Eq. (3)
-    i1 = tab->row_perm[r][i1];
-    i3 = tab->row_perm[r3][i3];
-    const uint32_t abx = tab->trellis_to_abx[path];
-    *w0 = i1 | (r << 11) | (i3 << 12) | ((p ^ r) << 23) | ((abx & 0xFFu) << 24);
-    *w1 = i2 | ((abx >> 8) << 11) | (g << 15);
+    const uint32_t a = abx & 15u, b = (abx >> 4) & 15u, x = abx >> 8;
+    *w0 = (i1 << 2) | (r << 13) | (i3 << 14) | (g << 25) | (a << 26) | (b << 30) | (b >> 2);
+    *w1 = i2 | (p << 11) | (x << 12);
 }
+// The twelve trellis bits of a file-order word: index of DeviceTables::trellis_to_abx.
+__device__ __forceinline__ uint32_t trellis_path(uint64_t w) { return uint32_t((w >> 33) & 0xFFF); }
 
 // Byte offsets of the staged tables inside the shared-memory copy of the fast part.
 constexpr uint32_t kSmRows = 0;
 constexpr uint32_t kSmMid = 16384;
 constexpr uint32_t kSmScale = 24576;
 constexpr uint32_t kSmMaskH = 25600;
-constexpr uint32_t kSmMaskHr = 25664;
+constexpr uint32_t kSmMaskXp = 25728;
 constexpr uint32_t kSmAlign = 16384;  // the staged copy starts on a 16 KiB boundary of shared memory
 static_assert(kSmMid == offsetof(DeviceTables, mid_fast) - kFastOffset, "staged layout");
 static_assert(kSmScale == offsetof(DeviceTables, scale) - kFastOffset, "staged layout");
 static_assert(kSmMaskH == offsetof(DeviceTables, mask_h) - kFastOffset, "staged layout");
-static_assert(kSmMaskHr == offsetof(DeviceTables, mask_hr) - kFastOffset, "staged layout");
+static_assert(kSmMaskXp == offsetof(DeviceTables, mask_xp) - kFastOffset && kSmMaskXp % 128 == 0, "staged layout");
 
 // Copies the staged part of the tables to the first 16 KiB boundary of the
 // CTA's dynamic shared memory (all threads; the caller synchronises) and returns
@@ -170,72 +164,67 @@ __device__ __forceinline__ unsigned char* stage_fast_tables_async(const DeviceTa
 }
 constexpr uint32_t kTableSmemBytes = uint32_t(kFastBytes) + kSmAlign;
 
-// PRMT pools.  A selector nibble is c | rank << 1 (c: the coordinate's pattern bit, ranks 0..3 of the
-// lists of Sec. 3.3), so the low pool word serves ranks 0 and 1 and the high word ranks 2 and 3:
-//   lo = { r0c0, r0c1, r1c0, r1c1 }    hi = { r2c0, r2c1, r3c0, r3c1 }
-// The pools hold MINUS the coordinate (the scale table holds minus the block scale, so products come
-// out with the right sign):
-//   p = 0:  y = 0, 2 | 4, -2 | -4, 6 | 8, -6        p = 1:  y = 1, -1 | -3, 3 | 5, -5 | -7, 7
-// A row with a coordinate of rank 4 (y = -8, 10 for p = 0; 9, -9 for p = 1) stores it as rank 2 and
-// sits in the first kRank4Slots slots of its class; for those slots the two rank-2 bytes of the high
-// word become the rank-4 values, which in this sign convention is the same XOR for both parities.
-constexpr uint32_t kPool0Lo = 0x02FCFE00u, kPool0Hi = 0x06F8FA04u;
-constexpr uint32_t kPool1Lo = 0xFD0301FFu, kPool1Hi = 0xF90705FBu;
-constexpr uint32_t kRank4Patch = 0x00000C0Cu;
-constexpr uint32_t kSpecialAddrMask = uint32_t(2048 - kRank4Slots) * 4u;  // zero <=> slot < kRank4Slots
-static_assert(kRank4Slots == 32 && kSpecialAddrMask == 0x1F80u, "special slots are the first 32 of a class");
-
 struct FastBlock {
-    uint32_t y[6];  // MINUS the lattice point, int8 x 4, coordinate 4k+i in byte i of y[k]
+    // MINUS EIGHT TIMES the lattice point, int8 x 4: y[2 s] holds coordinates 8 s + 1, 3, 5, 7 of section s in
+    // its bytes 0..3, y[2 s + 1] coordinates 8 s + 0, 2, 4, 6.  The activations' planes use the same order.
+    uint32_t y[6];
     uint32_t goff;  // shared-memory address of the scale table plus 8 g (the gain's column of the table)
 };
+// Coordinate of a block held by byte i of word k.
+__host__ __device__ constexpr int word_coordinate(int k, int i) { return 8 * (k >> 1) + 2 * i + ((k & 1) ? 0 : 1); }
 
+// A row table entry holds, per coordinate, the nibble -2 k, where 4 k = 0, 4, -4, 8, -8 is the rank's element of
+// the o = 0 list (Sec. 3.3).  The lists of o = p + 2 c are 4 k, 1 - 4 k, 2 - 4 k, 4 k - 1, so with the nibble z
+// complemented where the pattern bit c is set and once more everywhere if p = 1,
+//     -y = 2 z + p     for all four lists and all five ranks
+// (two's complement, -5 <= z <= 4).  The pattern masks and the complement for p are XORs; z moves to the upper
+// half of its byte and p below it: a byte 16 z + 8 p = -8 y costs half a logic operation.
 // HI = false: w1 sits in bits 0..15 of `w1pair`; HI = true: in bits 16..31.
 // sm_tab: shared-memory address of the staged tables, a multiple of 16 KiB, so
 // that every index is merged with its table's address by the same LOP3 that
 // masks it.
 template <bool HI>
 __device__ __forceinline__ void fast_decode(uint32_t sm_tab, uint32_t w0, uint32_t w1pair, FastBlock& out) {
-    const uint32_t addr1 = ((w0 << 2) & 0x3FFCu) | (sm_tab + kSmRows);    // (i1' | r << 11) * 4
-    const uint32_t addr3p = ((w0 >> 10) & 0x3FFCu) | (sm_tab + kSmRows);  // (i3' | q << 11) * 4
-    const uint32_t a4 = ((w0 >> 22) & 0x3Cu) | (sm_tab + kSmMaskH);
-    const uint32_t b4 = ((w0 >> 26) & 0x3Cu) | (sm_tab + kSmMaskH);
-    uint32_t addr2, x4;
-    if (HI) {
-        addr2 = ((w1pair >> 14) & 0x1FFCu) | (sm_tab + kSmMid);
-        x4 = ((w1pair >> 25) & 0x3Cu) | (sm_tab + kSmMaskHr);
-        out.goff = ((w1pair >> 28) & 8u) | (sm_tab + kSmScale);
-    } else {
-        addr2 = ((w1pair << 2) & 0x1FFCu) | (sm_tab + kSmMid);
-        x4 = ((w1pair >> 9) & 0x3Cu) | (sm_tab + kSmMaskHr);
-        out.goff = ((w1pair >> 12) & 8u) | (sm_tab + kSmScale);
-    }
+    const uint32_t sh = HI ? w1pair >> 14 : w1pair << 2;                 // [2..12] i2, [13] p, [14..17] x
+    const uint32_t addr1 = (w0 & 0x3FFCu) | (sm_tab + kSmRows);          // (i1 | r << 11) * 4
+    const uint32_t addr2 = (sh & 0x1FFCu) | (sm_tab + kSmMid);
+    const uint32_t addr3i = ((w0 >> 12) & 0x1FFCu) | (sm_tab + kSmRows);
+    const uint32_t a4 = ((w0 >> 24) & 0x3Cu) | (sm_tab + kSmMaskH);
+    const uint32_t b4 = (__funnelshift_l(w0, w0, 4) & 0x3Cu) | (sm_tab + kSmMaskH);
+    const uint32_t x4 = ((sh >> 11) & 0x7Cu) | (sm_tab + kSmMaskXp);     // (p | x << 1) * 4
+    out.goff = ((w0 >> 22) & 8u) | (sm_tab + kSmScale);
     const uint32_t row1 = lds32(addr1);
     const uint32_t row2 = lds32(addr2);
-    // delta = [i2 >= 1240]: bit 11 of i2 + 808, i.e. bit 13 of the byte offset; Eq. (3).
-    // (the table bases are multiples of 8 KiB, so they do not disturb bits 0..12 of the sum)
-    const uint32_t addr3 = addr3p ^ ((addr2 + 808u * 4u) & 0x2000u);
-    const uint32_t row3 = lds32(addr3);
+    // class of row 3 (Eq. (3)): p ^ r ^ delta, delta = [i2 >= 1240] = bit 11 of i2 + 808; all three at bit 13
+    // (the table bases are multiples of 16 KiB, so they do not disturb bits 0..13)
+    const uint32_t row3 = lds32(addr3i ^ ((addr1 ^ (addr2 + 808u * 4u) ^ sh) & 0x2000u));
     const uint32_t ma = lds32(a4);
     const uint32_t mb = lds32(b4);
     const uint32_t mx = lds32(x4);
-    const uint32_t sel1 = row1 ^ ma ^ mx;
-    const uint32_t sel2 = row2 ^ mb ^ mx;
-    const uint32_t sel3 = row3 ^ (ma ^ mb) ^ mx;
-    // p = r ^ q sits at bit 13 of both row addresses: one test, two selects for the pools
-    const bool p = ((addr1 ^ addr3p) & 0x2000u) != 0;
-    const uint32_t lo = p ? kPool1Lo : kPool0Lo;
-    const uint32_t hi = p ? kPool1Hi : kPool0Hi;
-    const uint32_t hix = hi ^ kRank4Patch;
-    const uint32_t hi1 = (addr1 & kSpecialAddrMask) ? hi : hix;
-    const uint32_t hi3 = (addr3p & kSpecialAddrMask) ? hi : hix;
-    out.y[0] = prmt(lo, hi1, sel1);
-    out.y[1] = prmt(lo, hi1, sel1 >> 16);
-    out.y[2] = prmt(lo, hi, sel2);
-    out.y[3] = prmt(lo, hi, sel2 >> 16);
-    out.y[4] = prmt(lo, hi3, sel3);
-    out.y[5] = prmt(lo, hi3, sel3 >> 16);
+    const uint32_t z1 = row1 ^ ma ^ mx;
+    const uint32_t z2 = row2 ^ mb ^ mx;
+    const uint32_t z3 = row3 ^ (ma ^ mb) ^ mx;
+    const uint32_t p8 = (x4 & 4u) * 0x02020202u;                         // 8 p in every byte
+    out.y[0] = (z1 & 0xF0F0F0F0u) | p8;
+    out.y[1] = ((z1 << 4) & 0xF0F0F0F0u) | p8;
+    out.y[2] = (z2 & 0xF0F0F0F0u) | p8;
+    out.y[3] = ((z2 << 4) & 0xF0F0F0F0u) | p8;
+    out.y[4] = (z3 & 0xF0F0F0F0u) | p8;
+    out.y[5] = ((z3 << 4) & 0xF0F0F0F0u) | p8;
 }
+
+// Shared-memory address of -gain[g] / sqrt(16 m): the squared norm of the packed point is 64 * 16 m, the table has
+// 16 bytes per m (16 m <= 416 for every word, Sec. 3.4, so the address stays inside it).
+__device__ __forceinline__ uint32_t scale_address(const FastBlock& fb) {
+    int n2 = 0;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) n2 = dp4a_ss(fb.y[k], fb.y[k], n2);
+    return (uint32_t(n2) >> 6) + fb.goff;
+}
+
+// sum of -y q from the sums of -8 y over the planes of q (high signed, middle, low): every term is a multiple of
+// 8 and |sum y q| <= sqrt(24 * 416) * 2^23 < 2^30, so the int32 is exact.
+__device__ __forceinline__ int combine_planes(int dh, int dm, int dl) { return dh * 8192 + ((dm * 256 + dl) >> 3); }
 
 // ---------------------------------------------------------------------------
 // Activations
@@ -243,7 +232,7 @@ __device__ __forceinline__ void fast_decode(uint32_t sm_tab, uint32_t w0, uint32
 // Fixed-point image of one block column of activations (20 words).
 // step = 2^(E-22) with 2^E <= max|x| < 2^(E+1); q_j = rint(x_j / step), |q_j| < 2^23,
 // stored as three byte planes (bits 23..16 signed, 15..8 and 7..0 unsigned), four
-// coordinates per 32-bit word: words 0..5 high, 6..11 middle, 12..17 low plane;
+// coordinates per 32-bit word in the decoder's order (word_coordinate): words 0..5 high, 6..11 middle, 12..17 low plane;
 // word 18 = step (float), word 19 = sum(q_j).  A float16 x_j is held exactly when
 // |x_j| >= 2^(E-12); smaller ones are rounded to a multiple of the step.  If a value
 // is NaN or infinite the step is NaN (and the planes zero).
@@ -284,7 +273,7 @@ __device__ __forceinline__ void quantise_column(const __half* __restrict__ x, in
         uint32_t hi = 0, mid = 0, lo = 0;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int q = __float2int_rn(v[4 * k + i] * inv);
+            const int q = __float2int_rn(v[word_coordinate(k, i)] * inv);
             sum += q;
             hi |= (uint32_t(q >> 16) & 0xFFu) << (8 * i);
             mid |= (uint32_t(q >> 8) & 0xFFu) << (8 * i);

@@ -38,22 +38,16 @@ __device__ __forceinline__ float block_value(uint32_t sm_tab, uint32_t w0, uint3
                                              float addend = 0.f) {
     FastBlock fb;
     fast_decode<HI>(sm_tab, w0, w1pair, fb);
-    // The squared norm 16 m is accumulated on top of the address of the gain's half of the scale table:
-    // that table holds -gain[g] / sqrt(16 m) at 512 g + 16 m, so the sum IS the address of the scale
-    // (16 m <= 416 for every word, Sec. 3.4, so it stays inside the table's half).
-    int dh = 0, dm = 0, dl = 0, n2 = int(fb.goff);
+    int dh = 0, dm = 0, dl = 0;
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
         dh = dp4a_ss(fb.y[k], X.hi[k], dh);
         dm = dp4a_su(fb.y[k], X.mid[k], dm);
         dl = dp4a_su(fb.y[k], X.lo[k], dl);
-        n2 = dp4a_ss(fb.y[k], fb.y[k], n2);
     }
-    // |sum_j y_j q_j| <= sqrt(24 * 416) * 2^23 < 2^31: the block's dot product is an exact int32
-    // (of -y: the scale carries the other minus sign)
-    int dot = dh * 65536 + (dm * 256 + dl);
-    const float scale = lds32f(uint32_t(n2));
-    return fmaf(float(dot), scale * X.step, addend);  // addend: the caller's running sum (one FFMA)
+    const float scale = lds32f(scale_address(fb));
+    // addend: the caller's running sum (one FFMA)
+    return fmaf(float(combine_planes(dh, dm, dl)), scale * X.step, addend);
 }
 
 // The eight blocks of one 48-byte record (rows 8G..8G+7 of one column).

@@ -175,79 +175,33 @@ int build_device_tables(DeviceTables* out, const float* gain2) {
     out->magic = kTableMagic;
     out->version = kTableVersion;
 
-    // Fast-path rows.  Per class: rows holding a rank-4 coordinate go to the first
-    // kRank4Slots slots, topped up with rows that use ranks 0 and 1 only (a patched
-    // pool serves ranks 0, 1 and 4); everything else keeps its order behind them.
-    for (int cls = 0; cls < 2; ++cls) {
-        std::vector<int> tail_rows, fillers, front;
-        for (int i = 0; i < 2048; ++i) {
-            const uint32_t row = out->paper.rows[2048 * cls + i];
-            int max_rank = 0, n4 = 0;
-            for (int j = 0; j < 8; ++j) {
-                const int r = (row >> (4 * j)) & 15;
-                if (r > 4) return -21;
-                if (r == 4) ++n4;
-                if (r > max_rank) max_rank = r;
-            }
-            if (n4 > 1) return -22;
-            if (n4 == 1) {
-                for (int j = 0; j < 8; ++j) {  // the other coordinates of such a row are of rank 0 or 1
-                    const int r = (row >> (4 * j)) & 15;
-                    if (r == 2 || r == 3) return -24;
-                }
-                tail_rows.push_back(i);
-            } else if (max_rank <= 1) {
-                fillers.push_back(i);
-            } else {
-                front.push_back(i);
-            }
-        }
-        if (int(tail_rows.size()) > kRank4Slots) return -25;
-        // Fillers are taken cheapest first and go in front of the rank-4 rows, so slot 0 of class 0 is
-        // the all-zero row: the all-zero device word then decodes to the origin, which the kernels rely
-        // on when they pad.
-        const int nfill = kRank4Slots - int(tail_rows.size());
-        if (int(fillers.size()) < nfill) return -26;
-        std::vector<int> special(fillers.begin(), fillers.begin() + nfill);
-        special.insert(special.end(), tail_rows.begin(), tail_rows.end());
-        front.insert(front.end(), fillers.begin() + nfill, fillers.end());
-        std::sort(front.begin(), front.end());
-        if (int(front.size()) != 2048 - kRank4Slots) return -27;
-        if (cls == 0 && out->paper.rows[special[0]] != 0u) return -28;
-        for (int slot = 0; slot < 2048; ++slot) {
-            const int i = slot < kRank4Slots ? special[slot] : front[slot - kRank4Slots];
-            const uint32_t row = out->paper.rows[2048 * cls + i];
-            uint32_t fast = 0;
-            for (int j = 0; j < 8; ++j) {
-                unsigned r = (row >> (4 * j)) & 15u;
-                if (r == 4) r = 2;
-                fast |= (r << 1) << (4 * j);
-            }
-            out->rows_fast[2048 * cls + slot] = fast;
-            out->row_perm[cls][i] = static_cast<uint16_t>(slot);
-        }
-    }
-    // The middle list keeps its own copy in i2 order; its rows never reach rank 4.
-    for (int i2 = 0; i2 < 2048; ++i2) {
-        const int idx = i2 < n0 ? i2 : 2048 + (i2 - n0);
-        const uint32_t row = out->paper.rows[idx];
-        uint32_t fast = 0;
+    // Fast-path rows: the rank's nibble -2 k.  The all-zero row comes first in class 0, so the all-zero device
+    // word decodes to the origin, which the kernels rely on when they pad.
+    auto fast_row = [](uint32_t row, uint32_t* fast) {
+        static const unsigned nibble[5] = {0u, 14u, 2u, 12u, 4u};
+        *fast = 0;
         for (int j = 0; j < 8; ++j) {
             const unsigned r = (row >> (4 * j)) & 15u;
-            if (r > 3) return -23;
-            fast |= (r << 1) << (4 * j);
+            if (r > 4) return false;
+            *fast |= nibble[r] << (4 * j);
         }
-        out->mid_fast[i2] = fast;
-    }
+        return true;
+    };
+    if (out->paper.rows[0] != 0u) return -28;
+    for (int i = 0; i < 4096; ++i)
+        if (!fast_row(out->paper.rows[i], &out->rows_fast[i])) return -21;
+    // The middle list keeps its own copy in i2 order.
+    for (int i2 = 0; i2 < 2048; ++i2) out->mid_fast[i2] = out->rows_fast[i2 < n0 ? i2 : 2048 + (i2 - n0)];
     for (unsigned v = 0; v < 16; ++v) {
         const uint8_t h = span4(turyn.h, v), hr = span4(turyn.hr, v);
         uint32_t mh = 0, mhr = 0;
         for (int j = 0; j < 8; ++j) {
-            mh |= uint32_t((h >> j) & 1) << (4 * j);
-            mhr |= uint32_t((hr >> j) & 1) << (4 * j);
+            mh |= ((h >> j) & 1) ? 15u << (4 * j) : 0u;
+            mhr |= ((hr >> j) & 1) ? 15u << (4 * j) : 0u;
         }
         out->mask_h[v] = mh;
-        out->mask_hr[v] = mhr;
+        out->mask_xp[2 * v] = mhr;
+        out->mask_xp[2 * v + 1] = ~mhr;
     }
     for (int g = 0; g < 2; ++g)
         for (int m = 0; m < 32; ++m)

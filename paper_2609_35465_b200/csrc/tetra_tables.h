@@ -17,8 +17,7 @@ struct PaperTables {
 static_assert(sizeof(PaperTables) == 18816, "paper table blob is 18,816 bytes");
 
 constexpr uint32_t kTableMagic = 0x54455442u;  // "TETB"
-constexpr uint32_t kTableVersion = 7;
-constexpr int kRank4Slots = 32;                // slots at the start of each class whose pool is patched
+constexpr uint32_t kTableVersion = 8;
 constexpr int kMiddleClass0 = 1240;            // N0 of Sec. 3.3 (checked at build)
 // The last row of a class's 2048 and of the middle list's class 0 (checked at build): each cuts a shell of equal
 // cost at this packed value; the middle list's class 1 ends with a whole shell.
@@ -31,31 +30,24 @@ struct DeviceTables {
     uint32_t magic;             // 18824
     uint32_t version;           // 18828
     // ---- fast path: everything below is staged in shared memory ------------
-    // Rank rows for PRMT lookup, class by class in the permuted order of
-    // row_perm: nibble j = rank << 1 (ranks 0..3; bit 0 is where the pattern bit
-    // goes).  The first 32 slots of each class hold the rows with a coordinate of
-    // rank 4 (stored there as rank 2) and, as fillers, rows that use ranks 0 and
-    // 1 only: for those slots the kernels swap in a PRMT pool word whose rank-2
-    // entries are the rank-4 values.
+    // Rank rows, class by class: nibble j = -2 k (two's complement) of coordinate j's rank, k = 0, 1, -1, 2, -2.
     // (the kernels place this part on a 16 KiB boundary of shared memory, so each
     //  sub-table's offset can be OR-ed into an index instead of added)
     uint32_t rows_fast[4096];   // +0
     uint32_t mid_fast[2048];    // +16384: rows_fast[mix(i2)], indexed by i2 directly
     float scale[2][32][4];      // +24576: -gain[g] / sqrt(16 m) in entry [0][m][2 g] (the second half is spare):
-                                //         16 bytes per m, so that the block's squared norm 16 m is the byte
-                                //         offset itself, and the two gains 8 bytes apart, so that lanes with
-                                //         nearby m or different g read different banks.  Minus: the fast
-                                //         decoder emits -y.
-    // Pattern-byte masks of the Turyn coordinates: bit 4j set where the
-    // Hamming word has coordinate j set; H for a and b, H' for x.
+                                //         16 bytes per m, the two gains 8 bytes apart, so that lanes with nearby
+                                //         m or different g read different banks.  Minus: the fast decoder emits
+                                //         minus (eight times) the point.
+    // Pattern-byte masks of the Turyn coordinates: nibble j all ones where the Hamming word has coordinate j
+    // set; H for a and b, H' for x.  mask_xp has x and the parity in one index, x << 1 | p, and is complemented
+    // where p = 1.
     uint32_t mask_h[16];        // +25600
-    uint32_t mask_hr[16];       // +25664
-    uint32_t pad_[16];          // +25728 (spare)
+    uint32_t spare_[16];        // +25664
+    uint32_t mask_xp[32];       // +25728
     // ---- pack-time only (global memory) ------------------------------------
     // 12 trellis bits (s8 | b1<<6 | b2<<7 | b3<<11) -> Turyn coordinates a | b<<4 | x<<8.
     uint16_t trellis_to_abx[4096];
-    // row_perm[cls][i]: slot of file-order row 2048 cls + i inside its class of rows_fast.
-    uint16_t row_perm[2][2048];
 };
 
 constexpr size_t kFastOffset = offsetof(DeviceTables, rows_fast);
