@@ -233,59 +233,90 @@ __device__ __forceinline__ int combine_planes(int dh, int dm, int dl) { return d
 // step = 2^(E-22) with 2^E <= max|x| < 2^(E+1); q_j = rint(x_j / step), |q_j| < 2^23,
 // stored as three byte planes (bits 23..16 signed, 15..8 and 7..0 unsigned), four
 // coordinates per 32-bit word in the decoder's order (word_coordinate): words 0..5 high, 6..11 middle, 12..17 low plane;
-// word 18 = step (float), word 19 = sum(q_j).  A float16 x_j is held exactly when
+// word 18 = step (float), word 19 is spare.  A float16 x_j is held exactly when
 // |x_j| >= 2^(E-12); smaller ones are rounded to a multiple of the step.  If a value
 // is NaN or infinite the step is NaN (and the planes zero).
-__device__ __forceinline__ void quantise_column(const __half* __restrict__ x, int K, int c, uint32_t out[20]) {
-    float v[24];
+// The 24 activations of block column c, as twelve pairs of float16 (zeros beyond K).
+__device__ __forceinline__ void load_column(const __half* __restrict__ x, int K, int c, uint32_t (&w)[12]) {
     const int k0 = 24 * c;
     if (k0 + 24 <= K && ((reinterpret_cast<uintptr_t>(x) & 15) == 0)) {  // 48-byte column, 16-byte aligned
         const uint4* src = reinterpret_cast<const uint4*>(x + k0);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             const uint4 u = __ldg(src + i);
-            const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const __half2 h = *reinterpret_cast<const __half2*>(&w[j]);
-                v[8 * i + 2 * j] = __low2float(h);
-                v[8 * i + 2 * j + 1] = __high2float(h);
-            }
+            w[4 * i] = u.x;
+            w[4 * i + 1] = u.y;
+            w[4 * i + 2] = u.z;
+            w[4 * i + 3] = u.w;
         }
     } else {
+        const unsigned short* src = reinterpret_cast<const unsigned short*>(x + k0);
 #pragma unroll
-        for (int j = 0; j < 24; ++j) v[j] = k0 + j < K ? __half2float(x[k0 + j]) : 0.f;
-    }
-    // largest magnitude, compared as bit patterns (same order as the values for non-negative floats):
-    // a NaN or an infinity, whose exponent field is all ones, then counts as the largest
-    uint32_t mxb = 0u;
-#pragma unroll
-    for (int j = 0; j < 24; ++j) mxb = max(mxb, __float_as_uint(v[j]) & 0x7FFFFFFFu);
-    const bool finite = mxb < 0x7F800000u;
-    const uint32_t e = mxb >> 23;  // biased exponent of the largest
-    // A NaN or an infinity among the 24 values makes the step NaN, so every product with this column, and
-    // with it every output row that reads the column, comes out NaN instead of a finite, wrong number.
-    const float step = !finite ? __uint_as_float(0x7FC00000u) : (mxb ? __uint_as_float((e - 22u) << 23) : 0.f);
-    const float inv = (finite && mxb) ? __uint_as_float((276u - e) << 23) : 0.f;
-    int sum = 0;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        uint32_t hi = 0, mid = 0, lo = 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int q = __float2int_rn(v[word_coordinate(k, i)] * inv);
-            sum += q;
-            hi |= (uint32_t(q >> 16) & 0xFFu) << (8 * i);
-            mid |= (uint32_t(q >> 8) & 0xFFu) << (8 * i);
-            lo |= (uint32_t(q) & 0xFFu) << (8 * i);
+        for (int j = 0; j < 12; ++j) {
+            const uint32_t lo = k0 + 2 * j < K ? __ldg(src + 2 * j) : 0u, hi = k0 + 2 * j + 1 < K ? __ldg(src + 2 * j + 1) : 0u;
+            w[j] = lo | (hi << 16);
         }
-        out[k] = hi;
-        out[6 + k] = mid;
-        out[12 + k] = lo;
+    }
+}
+// Step of a column and its inverse.  Magnitudes are compared as bit patterns (same order as the values): a NaN or an
+// infinity, whose exponent field is all ones, counts as the largest and makes the step NaN, so every product with
+// the column, and with it every output row that reads the column, comes out NaN instead of a finite, wrong number.
+__device__ __forceinline__ float column_step(const uint32_t (&w)[12], float& inv) {
+    uint32_t m = w[0] & 0x7FFF7FFFu;
+#pragma unroll
+    for (int j = 1; j < 12; ++j) m = __vmaxu2(m, w[j] & 0x7FFF7FFFu);
+    const uint32_t top = max(m & 0xFFFFu, m >> 16);
+    const uint32_t bits = __float_as_uint(__half2float(__ushort_as_half(static_cast<unsigned short>(top))));
+    const bool finite = top < 0x7C00u, some = finite && top != 0u;
+    const uint32_t e = bits >> 23;  // biased float exponent of the largest
+    inv = some ? __uint_as_float((276u - e) << 23) : 0.f;
+    return !finite ? __uint_as_float(0x7FC00000u) : (some ? __uint_as_float((e - 22u) << 23) : 0.f);
+}
+// rint(x inv) of the low (HIGH = false) or high half of a pair: |x| inv + 2^23 rounds to the integer |q| in the
+// mantissa (|q| < 2^23), then the sign.  If the column is not finite, inv is 0 and the result arbitrary (the step is NaN).
+template <bool HIGH>
+__device__ __forceinline__ uint32_t quantise_value(uint32_t w, float inv) {
+    const uint32_t h = HIGH ? w >> 16 : w & 0xFFFFu;
+    const float a = __half2float(__ushort_as_half(static_cast<unsigned short>(h & 0x7FFFu)));
+    const uint32_t q = __float_as_uint(fmaf(a, inv, 8388608.f)) - 0x4B000000u;
+    const uint32_t s = uint32_t(int32_t(HIGH ? w : w << 16) >> 31);
+    return (q ^ s) - s;
+}
+// The three plane words of four values.
+__device__ __forceinline__ void split_planes(uint32_t q0, uint32_t q1, uint32_t q2, uint32_t q3, uint32_t& hi, uint32_t& mid,
+                                             uint32_t& lo) {
+    const uint32_t a = prmt(q0, q1, 0x5140u), b = prmt(q2, q3, 0x5140u);
+    lo = prmt(a, b, 0x5410u);
+    mid = prmt(a, b, 0x7632u);
+    hi = prmt(prmt(q0, q1, 0x0062u), prmt(q2, q3, 0x0062u), 0x5410u);
+}
+// Plane words 2 s and 2 s + 1 of section s, from its four pairs: odd coordinates first, the decoder's order.
+__device__ __forceinline__ void quantise_section(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, float inv, uint32_t (&hi)[2],
+                                                 uint32_t (&mid)[2], uint32_t (&lo)[2]) {
+    static_assert(word_coordinate(0, 1) == 3 && word_coordinate(1, 1) == 2 && word_coordinate(5, 3) == 22, "odd coordinates first");
+    split_planes(quantise_value<true>(w0, inv), quantise_value<true>(w1, inv), quantise_value<true>(w2, inv),
+                 quantise_value<true>(w3, inv), hi[0], mid[0], lo[0]);
+    split_planes(quantise_value<false>(w0, inv), quantise_value<false>(w1, inv), quantise_value<false>(w2, inv),
+                 quantise_value<false>(w3, inv), hi[1], mid[1], lo[1]);
+}
+__device__ __forceinline__ void quantise_column(const __half* __restrict__ x, int K, int c, uint32_t out[20]) {
+    uint32_t w[12];
+    load_column(x, K, c, w);
+    float inv;
+    const float step = column_step(w, inv);
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        uint32_t hi[2], mid[2], lo[2];
+        quantise_section(w[4 * s], w[4 * s + 1], w[4 * s + 2], w[4 * s + 3], inv, hi, mid, lo);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            out[2 * s + k] = hi[k];
+            out[6 + 2 * s + k] = mid[k];
+            out[12 + 2 * s + k] = lo[k];
+        }
     }
     out[18] = __float_as_uint(step);
-    out[19] = uint32_t(sum);
+    out[19] = 0u;
 }
-
 
 }  // namespace tetra

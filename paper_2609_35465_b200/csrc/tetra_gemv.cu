@@ -249,7 +249,6 @@ __device__ __forceinline__ void load_lane_x(const unsigned char* xq_rec, bool ac
     X.mid[0] = t1.z; X.mid[1] = t1.w; X.mid[2] = t2.x; X.mid[3] = t2.y; X.mid[4] = t2.z; X.mid[5] = t2.w;
     X.lo[0] = t3.x; X.lo[1] = t3.y; X.lo[2] = t3.z; X.lo[3] = t3.w; X.lo[4] = t4.x; X.lo[5] = t4.y;
     X.step = active ? __uint_as_float(t4.z) : 0.f;  // an inactive lane contributes exact zeros
-    X.sum = int(t4.w);
 }
 
 #ifndef TETRA_UNIT_THREADS

@@ -10,14 +10,13 @@ namespace tetra {
 
 constexpr int kRedStride = 36;                 // floats per row of the transpose buffer (32 + pad)
 constexpr int kRedFloats = 8 * kRedStride;     // per warp
-constexpr int kXqBytesPerCol = 80;             // 3 planes x 24 bytes, step, sum
+constexpr int kXqBytesPerCol = 80;             // 3 planes x 24 bytes, step, spare
 
 struct LaneX {
     uint32_t hi[6];   // bits 23..16 of q (signed), int8 x 4
     uint32_t mid[6];  // bits 15..8 (unsigned)
     uint32_t lo[6];   // bits 7..0 (unsigned)
     float step;       // 2^(E-22)
-    int sum;          // sum of q over the 24 coordinates (kept in the record; unused by the kernels)
 };
 
 __device__ __forceinline__ void lane_x_from_words(const uint32_t q[20], bool active, LaneX& X) {
@@ -28,7 +27,6 @@ __device__ __forceinline__ void lane_x_from_words(const uint32_t q[20], bool act
         X.lo[k] = active ? q[12 + k] : 0u;
     }
     X.step = active ? __uint_as_float(q[18]) : 0.f;
-    X.sum = active ? int(q[19]) : 0;
 }
 
 // One block: device word -> contribution scale_b * sum_j y_j x_j (Eq. (2) without
@@ -50,30 +48,29 @@ __device__ __forceinline__ float block_value(uint32_t sm_tab, uint32_t w0, uint3
     return fmaf(float(combine_planes(dh, dm, dl)), scale * X.step, addend);
 }
 
-// The eight blocks of one 48-byte record (rows 8G..8G+7 of one column).
-__device__ __forceinline__ void record_values(uint32_t sm_tab, const uint4& a, const uint4& b, const uint4& h,
-                                              const LaneX& X, float v[8]) {
-    v[0] = block_value<false>(sm_tab, a.x, h.x, X);
-    v[1] = block_value<true>(sm_tab, a.y, h.x, X);
-    v[2] = block_value<false>(sm_tab, a.z, h.y, X);
-    v[3] = block_value<true>(sm_tab, a.w, h.y, X);
-    v[4] = block_value<false>(sm_tab, b.x, h.z, X);
-    v[5] = block_value<true>(sm_tab, b.y, h.z, X);
-    v[6] = block_value<false>(sm_tab, b.z, h.w, X);
-    v[7] = block_value<true>(sm_tab, b.w, h.w, X);
-}
-
-// The same, added to the caller's eight running sums.
+// The blocks of one 48-byte record (rows 8G..8G+7 of one column), added to the caller's running sums.  R = 4: half
+// a record, the four w0 words in `a` and the two w1 words in h.x, h.y.
+template <int R = 8>
 __device__ __forceinline__ void record_accumulate(uint32_t sm_tab, const uint4& a, const uint4& b, const uint4& h,
-                                                  const LaneX& X, float acc[8]) {
+                                                  const LaneX& X, float (&acc)[R]) {
     acc[0] = block_value<false>(sm_tab, a.x, h.x, X, acc[0]);
     acc[1] = block_value<true>(sm_tab, a.y, h.x, X, acc[1]);
     acc[2] = block_value<false>(sm_tab, a.z, h.y, X, acc[2]);
     acc[3] = block_value<true>(sm_tab, a.w, h.y, X, acc[3]);
-    acc[4] = block_value<false>(sm_tab, b.x, h.z, X, acc[4]);
-    acc[5] = block_value<true>(sm_tab, b.y, h.z, X, acc[5]);
-    acc[6] = block_value<false>(sm_tab, b.z, h.w, X, acc[6]);
-    acc[7] = block_value<true>(sm_tab, b.w, h.w, X, acc[7]);
+    if constexpr (R == 8) {
+        acc[4] = block_value<false>(sm_tab, b.x, h.z, X, acc[4]);
+        acc[5] = block_value<true>(sm_tab, b.y, h.z, X, acc[5]);
+        acc[6] = block_value<false>(sm_tab, b.z, h.w, X, acc[6]);
+        acc[7] = block_value<true>(sm_tab, b.w, h.w, X, acc[7]);
+    }
+}
+// The same, on their own.
+template <int R = 8>
+__device__ __forceinline__ void record_values(uint32_t sm_tab, const uint4& a, const uint4& b, const uint4& h,
+                                              const LaneX& X, float (&v)[R]) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = 0.f;
+    record_accumulate<R>(sm_tab, a, b, h, X, v);
 }
 
 // Sums v[r] over the 32 lanes for r = 0..7 through the warp's shared-memory

@@ -65,9 +65,6 @@ cudaError_t launch_gemv_paper(const void* codes, size_t row_stride, const float*
 constexpr int kListMax = 8;
 struct ListDesc {
     int32_t count;
-    int32_t total_groups;               // eight-row groups of all matrices
-    int32_t group_prefix[kListMax + 1]; // row groups before matrix i
-    int32_t max_blocks;                 // largest number of words per row in the list
     Problem problems[kListMax];
 };
 cudaError_t launch_gemv_list(const ListDesc& list, int batch, const void* table, cudaStream_t s);

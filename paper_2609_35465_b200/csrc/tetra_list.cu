@@ -3,19 +3,29 @@
 // tetra_gemv, tetra_gemv_tail and tetra_gemv_list.
 //
 // Sec. 5.2 of the paper times one launch per matrix; on B200 such a launch holds
-// a few microseconds of work, so what is left of it is a chain of latencies.  The
-// kernel is arranged to shorten that chain:
-//   * everything that does not depend on the activations is started before the
-//     kernel waits for its predecessor in the stream (programmatic dependent
-//     launch): the decode tables are staged, every warp's first code record is
-//     on its way into shared memory, the row scales and tails are pulled into L2;
-//   * a CTA of 256 threads takes at most half an SM, so the CTAs of the next
-//     launch become resident, and do all of the above, while this launch runs;
-//   * after the wait a CTA turns the activations of the matrix it works on into
-//     their fixed-point image in shared memory (once per CTA, one column per
-//     thread), and its warps split the (row group, column group) passes of the
-//     CTA's rows evenly and in memory order, with the decoder, the per-warp
-//     cp.async ring and the transpose reduction of the planned-list kernel;
+// a few microseconds of work, so what is left of it is a chain of latencies:
+// dependency wait, activations, their fixed-point image, the passes, the sums.
+// The kernel is arranged to shorten that chain (%globaltimer stamps on q, k, v of
+// an 8B layer, 8.5 us a launch before: 1.3 us of prologue instructions ahead of
+// the wait, 1.3 us of image, 3.1 us of passes, 0.7 us of epilogue, and CTAs that
+// straddled two matrices and finished 2.5 us after the others):
+//   * one CTA of sixteen warps per SM: the image and the tables are built and
+//     fetched once per SM (two CTAs of eight warps, which let the next launch start
+//     in the gaps of this one, spend more on doing both twice: q, k, v 7.8 against
+//     6.3 us);
+//   * a CTA works on ONE matrix; the host cuts every matrix's row groups into the
+//     CTAs' shares, and the kernel finds its share with a few comparisons of
+//     parameters: no division, no chain of loads;
+//   * everything that does not depend on the activations is requested before the
+//     wait for the predecessor in the stream (programmatic dependent launch) and
+//     waited for only after the image has been built: the decode tables, every
+//     warp's first code record, row scales, tails;
+//   * the image takes a thread per (column, section), eight activations each;
+//   * the warps split the CTA's passes evenly in memory order, a pass being 32
+//     consecutive (row group, column) cells: where a row ends inside a pass the
+//     next row group's first columns fill the lanes.  A row group is a record's
+//     eight rows or (R = 4) half of them, whichever leaves the last pass of the
+//     busiest warp earlier;
 //   * per-(row group, warp) partial sums meet in shared memory and are added in
 //     warp order (deterministic), then row scale and tail.
 // The only waits are CTA barriers, cp.async.wait_group and griddepcontrol.wait.
@@ -26,221 +36,271 @@ namespace tetra {
 
 static_assert(kListMax == TETRA_LIST_MAX, "list length limit must agree with the header");
 
-constexpr int kChunkGroups = 32;  // row groups whose partial sums share the shared-memory buffer
+constexpr int kListWarps = 16, kListThreads = 32 * kListWarps;
+constexpr int kChunkRows = 128;  // rows whose partial sums share the shared-memory buffer
+
+// Kernel parameters: the list and its split over the grid.  CTAs [cta_begin[i], cta_begin[i + 1]) work on matrix i
+// (entries beyond the list: never reached); the first `extra` of them take base + 1 row groups, the others base.
+// What a CTA needs of its matrix is one 64-byte line of constant memory: parameters are cold in every launch.
+struct alignas(64) ListMatrix {
+    const void* codes;
+    const __half* x;
+    const float* row_scales;
+    const __half* tail;
+    float* y;
+    int32_t N, K;
+    int32_t base, extra;
+    uint32_t inv_bs;  // ceil(2^32 / max(words per row, 32)): cell -> row group by one high multiply
+    int32_t begin;    // first CTA
+};
+static_assert(sizeof(ListMatrix) == 64, "one line");
+struct ListParams {
+    int32_t cta_begin[kListMax];
+    int32_t image_cols;         // largest number of words per row, if the image fits
+    int32_t batch;
+    ListMatrix m[kListMax];
+};
 
 struct ListSmem {
     // offsets from the 16 KiB-aligned table copy; total includes the alignment slack
-    uint32_t xq, xtail, ring, red, part, rs, tail, total;
+    uint32_t xq, xtail, ring, part, rs, tail, total;
 };
-__host__ __device__ inline ListSmem list_smem(int warps, int image_cols) {
+__host__ __device__ inline ListSmem list_smem(int image_cols) {
     ListSmem S;
     S.xq = uint32_t(kFastBytes);
     S.xtail = S.xq + uint32_t(image_cols) * kXqBytesPerCol;               // float [24]: x beyond the last word
     S.ring = S.xtail + 96u;
-    S.red = S.ring + uint32_t(warps) * 3072u;
-    S.part = S.red + uint32_t(warps) * kRedFloats * 4u;
-    S.rs = S.part + uint32_t(kChunkGroups * warps * 8 * 4);              // float [chunk rows]: row scales
-    S.tail = S.rs + uint32_t(kChunkGroups * 8 * 4);                       // half [chunk rows][24]: tails
-    S.total = S.tail + uint32_t(kChunkGroups * 8 * 24 * 2) + kSmAlign;
+    S.part = S.ring + kListWarps * 3072u;
+    S.rs = S.part + uint32_t(kChunkRows * kListWarps * 4);                // float [chunk rows]: row scales
+    S.tail = S.rs + uint32_t(kChunkRows * 4);                             // half [chunk rows][24]: tails
+    S.total = S.tail + uint32_t(kChunkRows * 24 * 2) + kSmAlign;
     return S;
 }
 
-__device__ __forceinline__ void ring_fetch(uint32_t dst, const uint4* src, uint32_t Bu) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst), "l"(src));
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 512), "l"(src + Bu));
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 1024), "l"(src + 2 * Bu));
+// Record of one lane in the ring: R = 8: the three 16-byte parts at +0, +512, +1024; R = 4: the half's four w0 words
+// at +0, its two w1 words at +1024.
+template <int R>
+__device__ __forceinline__ void ring_fetch(uint32_t dst, const uint4* codes, uint32_t Bu, int group, uint32_t col) {
+    if (R == 8) {
+        const uint4* rec = codes + size_t(group) * 3 * Bu + col;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst), "l"(rec));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 512), "l"(rec + Bu));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 1024), "l"(rec + 2 * Bu));
+    } else {
+        const uint4* rec = codes + size_t(group >> 1) * 3 * Bu + col;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst), "l"(rec + ((group & 1) ? Bu : 0u)));
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" :: "r"(dst + 1024), "l"(reinterpret_cast<const uint2*>(rec + 2 * Bu) + (group & 1)));
+    }
 }
 
-// Geometry of one chunk (row groups [ga, ga + ng) of a matrix with Bu words per row).  Its cells
-// (row group, column) are numbered row group by row group, Bs = max(Bu, 32) to a row group (cells
-// with column >= Bu are empty), and a pass is 32 consecutive cells: no lane idles at the end of a
-// row because the next row group's first columns fill the pass.  Warp w of W takes passes
-// [passes w / W, passes (w + 1) / W).
-struct Chunk {
-    uint32_t Bu, Bs;
-    int ga, ng, passes;
-};
-__device__ __forceinline__ Chunk make_chunk(const Problem& P, int ga, int ng) {
-    Chunk C;
-    C.Bu = uint32_t(P.tail ? P.K / 24 : (P.K + 23) / 24);
-    C.Bs = C.Bu < 32u ? 32u : C.Bu;
-    C.ga = ga;
-    C.ng = ng;
-    C.passes = int((uint32_t(ng) * C.Bs + 31u) >> 5);
-    return C;
+// Sums v[r] over the 32 lanes for r < R through a warp-private buffer (R x kRedStride floats); the result for row
+// lane / (32 / R) ends up in all 32 / R lanes of that row.
+template <int R>
+__device__ __forceinline__ float warp_row_sums(float* red, int lane, const float (&v)[R]) {
+    constexpr int L = 32 / R;  // lanes per row, R values each
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < R; ++r) red[r * kRedStride + lane] = v[r];
+    __syncwarp();
+    const float4* src = reinterpret_cast<const float4*>(red + (lane / L) * kRedStride + R * (lane % L));
+    float s = 0.f;
+#pragma unroll
+    for (int k = 0; k < R / 4; ++k) {
+        const float4 q = src[k];
+        s += (q.x + q.y) + (q.z + q.w);
+    }
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+    return s;
 }
 
-// IMAGE: the CTA keeps the fixed-point image of the matrix's activations in shared memory
-// (one 80-byte record per column); otherwise (more columns than fit) a lane builds its column's
-// record from x for every pass.
-template <int THREADS, bool IMAGE>
-__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 2 : 1)
-k_gemv_list(const DeviceTables* __restrict__ tab, const __grid_constant__ ListDesc L, int batch) {
-    constexpr int W = THREADS / 32;
+// R: rows of a row group (8: a record, 4: half of one);
+// IMAGE: the CTA keeps the fixed-point image of the matrix's activations in shared memory (one 80-byte record per
+// column); otherwise (more columns than fit) a lane builds its column's record from x for every pass.
+template <int R, bool IMAGE>
+__global__ void __launch_bounds__(kListThreads, 1)
+k_gemv_list(const DeviceTables* __restrict__ tab, const __grid_constant__ ListParams L) {
+    constexpr int THREADS = kListThreads, W = kListWarps, CHUNK = kChunkRows / R;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_release();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const ListSmem S = list_smem(W, IMAGE ? L.max_blocks : 0);
-    unsigned char* smem = stage_fast_tables_async(tab, smem_raw);
+    const ListSmem S = list_smem(IMAGE ? L.image_cols : 0);
+    const uint32_t sm_raw = smem_u32(smem_raw);
+    unsigned char* smem = smem_raw + (((sm_raw + kSmAlign - 1) & ~(kSmAlign - 1)) - sm_raw);
     const uint32_t sm_tab = smem_u32(smem);
-    float* red = reinterpret_cast<float*>(smem + S.red) + warp * kRedFloats;
     float* part = reinterpret_cast<float*>(smem + S.part);
     float* xtail = reinterpret_cast<float*>(smem + S.xtail);
     float* rs_sm = reinterpret_cast<float*>(smem + S.rs);
     __half* tail_sm = reinterpret_cast<__half*>(smem + S.tail);
-    const uint32_t ring = sm_tab + S.ring + uint32_t(warp) * 3072u + uint32_t(lane) * 16u;
+    const uint32_t ring_base = S.ring + uint32_t(warp) * 3072u;
+    const uint32_t ring = sm_tab + ring_base + uint32_t(lane) * 16u;
 
-    // This CTA's share of the row groups of the whole list, in list order.
-    const int g_lo = int((long long)blockIdx.x * L.total_groups / gridDim.x);
-    const int g_hi = int((long long)(blockIdx.x + 1) * L.total_groups / gridDim.x);
-    if (g_lo >= g_hi) return;
-    int p_first = 0;
-    while (L.group_prefix[p_first + 1] <= g_lo) ++p_first;
+    // this CTA's matrix and row groups
+    int p = 0;
+#pragma unroll
+    for (int i = 1; i < kListMax; ++i) p += int(blockIdx.x) >= L.cta_begin[i] ? 1 : 0;
+    const ListMatrix& P = L.m[p];
+    const int j = int(blockIdx.x) - P.begin;
+    const int g_lo = j * P.base + min(j, P.extra);
+    const int g_hi = g_lo + P.base + (j < P.extra ? 1 : 0);
+    const uint32_t inv_bs = P.inv_bs;
+    const int K = P.K, ntail = P.tail ? K % 24 : 0;
+    const uint32_t Bu = uint32_t(P.tail ? K / 24 : (K + 23) / 24), Bs = Bu < 32u ? 32u : Bu;
+    const uint4* codes = static_cast<const uint4*>(P.codes);
 
-    // Row scales and tails of a chunk's rows into shared memory (they are constants of the model, so
-    // this may run before the wait below).  cp.async where the addresses allow it, so that nothing
-    // here waits for memory; the caller waits for the group.
-    auto stage_rows = [&](const Problem& P, int ga, int ng) {
-        const int ntail = P.tail ? P.K % 24 : 0;
-        const int rows = min(ng * 8, P.N - ga * 8);
-        const float* rs = P.row_scales + size_t(ga) * 8;
+    // Geometry of a chunk (row groups [ga, ga + ng)): its cells (row group, column) are numbered row group by row
+    // group, Bs to a row group (cells with column >= Bu are empty), a pass is 32 consecutive cells.
+    auto fetch = [&](uint32_t dst, int ga, int ng, int rgl, uint32_t col) {
+        ring_fetch<R>(dst, codes, Bu, ga + min(rgl, ng - 1), min(col, Bu - 1));
+    };
+    auto cell_of = [&](int ps, int& rgl, uint32_t& col) {
+        const uint32_t cell = uint32_t(ps) * 32u + uint32_t(lane);
+        const uint32_t r = __umulhi(cell, inv_bs);
+        rgl = int(r);
+        col = cell - r * Bs;
+    };
+    // Row scales and tails of a chunk's rows into shared memory; cp.async where the addresses allow it, so that
+    // nothing here waits for memory.  Eight threads per row.
+    auto stage_rows = [&](int ga, int ng) {
+        const int rows = min(ng * R, P.N - ga * R);
+        const float* rs = P.row_scales + size_t(ga) * R;
         for (int t = threadIdx.x; t < rows; t += THREADS)
             asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(smem_u32(rs_sm + t)), "l"(rs + t));
-        const __half* tl = static_cast<const __half*>(P.tail) + size_t(ga) * 8 * ntail;
-        if (ntail && (ntail & 1) == 0 && (reinterpret_cast<uintptr_t>(tl) & 3) == 0) {
-            const int pairs = ntail >> 1;  // two tail values per 4-byte request
-            for (int i = threadIdx.x; i < rows * pairs; i += THREADS) {
-                const int t = i / pairs, k = i - t * pairs;
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;"
-                             :: "r"(smem_u32(tail_sm + t * 24 + 2 * k)), "l"(tl + size_t(t) * ntail + 2 * k));
-            }
-        } else {
-            for (int i = threadIdx.x; i < rows * ntail; i += THREADS) {
-                const int t = i / ntail, k = i - t * ntail;
-                tail_sm[t * 24 + k] = tl[size_t(t) * ntail + k];
+        if (ntail) {
+            const __half* tl = P.tail + size_t(ga) * R * ntail;
+            const bool pairs = (ntail & 1) == 0 && (reinterpret_cast<uintptr_t>(tl) & 3) == 0;
+            for (int t = threadIdx.x >> 3; t < rows; t += THREADS / 8) {
+                if (pairs) {
+                    for (int k = 2 * (threadIdx.x & 7); k < ntail; k += 16)
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;"
+                                     :: "r"(smem_u32(tail_sm + t * 24 + k)), "l"(tl + size_t(t) * ntail + k));
+                } else {
+                    for (int k = threadIdx.x & 7; k < ntail; k += 8) tail_sm[t * 24 + k] = tl[size_t(t) * ntail + k];
+                }
             }
         }
     };
-    // Lane's first cell of pass `ps`: row group (within the chunk) and column.
-    auto cell_of = [&](const Chunk& C, int ps, int* rgl, uint32_t* col) {
-        const uint32_t cell = uint32_t(ps) * 32u + uint32_t(lane);
-        const uint32_t r = cell / C.Bs;
-        *rgl = int(r);
-        *col = cell - r * C.Bs;
-    };
-    auto record_ptr = [&](const Problem& P, const Chunk& C, int rgl, uint32_t col) -> const uint4* {
-        const int rg = min(rgl, C.ng - 1);
-        return static_cast<const uint4*>(P.codes) + size_t(C.ga + rg) * 3 * C.Bu + min(col, C.Bu - 1);
-    };
 
-    // ---- before the wait: work that does not depend on the activations ----------------------
-    bool first_chunk = true;
+    // ---- before the wait: requests that do not depend on the activations ----------------------
     {
-        const Problem& P = L.problems[p_first];
-        const int ga = g_lo - L.group_prefix[p_first];
-        const int ng = min(min(g_hi, L.group_prefix[p_first + 1]) - g_lo, kChunkGroups);
-        const Chunk C = make_chunk(P, ga, ng);
-        const int ps0 = C.passes * warp / W, ps1 = C.passes * (warp + 1) / W;
+        const int ng = min(g_hi - g_lo, CHUNK);
+        const int passes = int((uint32_t(ng) * Bs + 31u) >> 5);
+        const int ps0 = passes * warp / W, ps1 = passes * (warp + 1) / W;
         if (ps0 < ps1) {
             int rgl;
             uint32_t col;
-            cell_of(C, ps0, &rgl, &col);
-            ring_fetch(ring, record_ptr(P, C, rgl, col), C.Bu);
+            cell_of(ps0, rgl, col);
+            fetch(ring, g_lo, ng, rgl, col);
         }
-        stage_rows(P, ga, ng);
+        stage_fast_tables_async(tab, smem_raw);
+        stage_rows(g_lo, ng);
         asm volatile("cp.async.commit_group;");
     }
     pdl_wait();  // the activations may come from the previous kernel of the stream
-    asm volatile("cp.async.wait_group 0;" ::: "memory");  // tables, first rows and first record (the barrier follows)
+
+    // Image task: (column, section) `id`, from the column's pairs w.
+    auto image_task = [&](uint32_t id, const uint32_t (&w)[12]) {
+        const uint32_t s = (id >= Bu ? 1u : 0u) + (id >= 2 * Bu ? 1u : 0u), c = id - s * Bu;
+        float inv;
+        const float step = column_step(w, inv);
+        const uint32_t w0 = s == 0 ? w[0] : (s == 1 ? w[4] : w[8]), w1 = s == 0 ? w[1] : (s == 1 ? w[5] : w[9]);
+        const uint32_t w2 = s == 0 ? w[2] : (s == 1 ? w[6] : w[10]), w3 = s == 0 ? w[3] : (s == 1 ? w[7] : w[11]);
+        uint32_t hi[2], mid[2], lo[2];
+        quantise_section(w0, w1, w2, w3, inv, hi, mid, lo);
+        unsigned char* rec = smem + S.xq + c * kXqBytesPerCol;
+        *reinterpret_cast<uint2*>(rec + 8 * s) = make_uint2(hi[0], hi[1]);
+        *reinterpret_cast<uint2*>(rec + 24 + 8 * s) = make_uint2(mid[0], mid[1]);
+        *reinterpret_cast<uint2*>(rec + 48 + 8 * s) = make_uint2(lo[0], lo[1]);
+        if (s == 0) *reinterpret_cast<float*>(rec + 72) = step;
+    };
+    auto image_column = [&](uint32_t id) { return int(id - (id >= 2 * Bu ? 2 * Bu : (id >= Bu ? Bu : 0u))); };
 
     int parity = 0;
-    for (int job = 0; job < batch; ++job) {  // activation vector `job` of every matrix
-        int p = p_first;
-        int p_staged = -1;  // matrix whose activations are in the shared-memory image
-        for (int g = g_lo; g < g_hi;) {
-            while (L.group_prefix[p + 1] <= g) ++p;
-            const Problem& P = L.problems[p];
-            const int seg_end = min(g_hi, L.group_prefix[p + 1]);
-            const int ntail = P.tail ? P.K % 24 : 0;
-            const __half* xj = static_cast<const __half*>(P.x) + size_t(job) * P.K;
-            float* yj = P.y + size_t(job) * P.N;
-            const int ga = g - L.group_prefix[p];
-            const int ng = min(seg_end - g, kChunkGroups);
-            const Chunk C = make_chunk(P, ga, ng);
-            const uint32_t Bu = C.Bu;
-
-            __syncthreads();  // the previous chunk's epilogue has read its buffers; its passes have read the image
-            for (int i = threadIdx.x; i < ng * W * 8; i += THREADS) part[i] = 0.f;
+    bool first_chunk = true;
+    for (int job = 0; job < L.batch; ++job) {  // activation vector `job`
+        const __half* xj = P.x + size_t(job) * K;
+        float* yj = P.y + size_t(job) * P.N;
+        // the first round's activations are requested, then the rest of what a chunk needs, then the image is built
+        uint32_t w[12];
+        if (IMAGE && threadIdx.x < 3 * Bu) load_column(xj, K, image_column(threadIdx.x), w);
+        const float xt = int(threadIdx.x) < ntail ? __half2float(xj[24 * Bu + threadIdx.x]) : 0.f;
+        if (job > 0) {
+            __syncthreads();  // the vector before is done with the image and the buffers
+        } else {
+            for (int i = threadIdx.x; i < min(g_hi - g_lo, CHUNK) * W * R; i += THREADS) part[i] = 0.f;
+        }
+        if (IMAGE) {
+            if (threadIdx.x < 3 * Bu) image_task(threadIdx.x, w);
+            for (uint32_t id = threadIdx.x + THREADS; id < 3 * Bu; id += THREADS) {
+                load_column(xj, K, image_column(id), w);
+                image_task(id, w);
+            }
+        }
+        if (threadIdx.x < 24) xtail[threadIdx.x] = xt;
+        for (int g = g_lo; g < g_hi; g += CHUNK) {
+            const int ng = min(g_hi - g, CHUNK);
+            const int passes = int((uint32_t(ng) * Bs + 31u) >> 5);
             if (!first_chunk) {
-                stage_rows(P, ga, ng);
+                __syncthreads();  // the epilogue before has read its buffers
+                for (int i = threadIdx.x; i < ng * W * R; i += THREADS) part[i] = 0.f;
+                stage_rows(g, ng);
                 asm volatile("cp.async.commit_group;");
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
             }
-            if (p_staged != p) {
-                const float xt = (threadIdx.x < 24 && int(threadIdx.x) < ntail) ? __half2float(xj[24 * Bu + threadIdx.x]) : 0.f;
-                if (IMAGE) {
-                    for (int c = threadIdx.x; c < int(Bu); c += THREADS) {
-                        uint32_t q[20];
-                        quantise_column(xj, P.K, c, q);
-                        uint4* dst = reinterpret_cast<uint4*>(smem + S.xq + c * kXqBytesPerCol);
-#pragma unroll
-                        for (int k = 0; k < 5; ++k) dst[k] = make_uint4(q[4 * k], q[4 * k + 1], q[4 * k + 2], q[4 * k + 3]);
-                    }
-                }
-                if (threadIdx.x < 24) xtail[threadIdx.x] = xt;
-                p_staged = p;
-            }
-            __syncthreads();
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();  // tables, rows and image are in place, the partial sums are zero
 
             // ---- this warp's passes --------------------------------------------------------
-            const int ps0 = C.passes * warp / W, ps1 = C.passes * (warp + 1) / W;
+            const int ps0 = passes * warp / W, ps1 = passes * (warp + 1) / W;
             if (ps0 < ps1) {
                 int rgl;
                 uint32_t col;
-                cell_of(C, ps0, &rgl, &col);
+                cell_of(ps0, rgl, col);
                 if (!first_chunk) {
-                    ring_fetch(ring + uint32_t(parity * 1536), record_ptr(P, C, rgl, col), Bu);
+                    fetch(ring + uint32_t(parity * 1536), g, ng, rgl, col);
                     asm volatile("cp.async.commit_group;");
                 }
                 int rg_acc = __shfl_sync(0xFFFFFFFFu, rgl, 0);  // row group the accumulators belong to
-                float acc[8];
+                float acc[R];
 #pragma unroll
-                for (int r = 0; r < 8; ++r) acc[r] = 0.f;
-                // folds the accumulators of row group rg_acc into this warp's slot of the partial sums
+                for (int r = 0; r < R; ++r) acc[r] = 0.f;
+                // folds the accumulators of row group rg_acc into this warp's slot of the partial sums, through the
+                // ring slot of the pass at hand, which every lane has read
                 auto flush = [&]() {
-                    float sum = transpose_partial(red, lane, acc);
-                    sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
-                    sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 2);
-                    if ((lane & 3) == 0) part[(rg_acc * W + warp) * 8 + (lane >> 2)] = sum;
+                    const float sum = warp_row_sums<R>(reinterpret_cast<float*>(smem + ring_base + parity * 1536), lane, acc);
+                    constexpr int PL = 32 / R;
+                    if (lane % PL == 0) part[(rg_acc * W + warp) * R + lane / PL] = sum;
+                    __syncwarp();  // the buffer has been read before the slot is filled again
                 };
                 for (int ps = ps0; ps < ps1; ++ps) {
-                    uint4 a, b, h;
                     asm volatile("cp.async.wait_group 0;" ::: "memory");
-                    {
-                        const uint32_t src = ring + uint32_t(parity * 1536);
-                        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w) : "r"(src));
+                    const uint32_t src = ring + uint32_t(parity * 1536);
+                    uint4 a, b, h;
+                    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w) : "r"(src));
+                    if (R == 8) {
                         asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "r"(src + 512));
                         asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(h.x), "=r"(h.y), "=r"(h.z), "=r"(h.w) : "r"(src + 1024));
+                    } else {
+                        asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(h.x), "=r"(h.y) : "r"(src + 1024));
                     }
                     // this lane's cell of the next pass: 32 cells on, at most one row group further
                     int nrgl = rgl;
                     uint32_t ncol = col + 32u;
-                    if (ncol >= C.Bs) { ncol -= C.Bs; ++nrgl; }
-                    if (ps + 1 < ps1) ring_fetch(ring + uint32_t((parity ^ 1) * 1536), record_ptr(P, C, nrgl, ncol), Bu);
+                    if (ncol >= Bs) { ncol -= Bs; ++nrgl; }
+                    if (ps + 1 < ps1) fetch(ring + uint32_t((parity ^ 1) * 1536), g, ng, nrgl, ncol);
                     asm volatile("cp.async.commit_group;");
-                    const bool active = rgl < C.ng && col < Bu;
+                    const bool active = rgl < ng && col < Bu;
                     LaneX X;
                     {
                         uint32_t q[20];
                         if (IMAGE) {
-                            const uint4* src = reinterpret_cast<const uint4*>(smem + S.xq + min(col, Bu - 1) * kXqBytesPerCol);
+                            const uint4* rec = reinterpret_cast<const uint4*>(smem + S.xq + min(col, Bu - 1) * kXqBytesPerCol);
 #pragma unroll
                             for (int k = 0; k < 5; ++k) {
-                                const uint4 u = src[k];
+                                const uint4 u = rec[k];
                                 q[4 * k] = u.x; q[4 * k + 1] = u.y; q[4 * k + 2] = u.z; q[4 * k + 3] = u.w;
                             }
                         } else {
-                            quantise_column(xj, P.K, int(min(col, Bu - 1)), q);
+                            quantise_column(xj, K, int(min(col, Bu - 1)), q);
                         }
                         lane_x_from_words(q, active, X);
                     }
@@ -249,47 +309,104 @@ k_gemv_list(const DeviceTables* __restrict__ tab, const __grid_constant__ ListDe
                     // folded and then start the next row group's.
                     const int rg_last = __shfl_sync(0xFFFFFFFFu, rgl, 31);
                     if (rg_last == rg_acc) {
-                        record_accumulate(sm_tab, a, b, h, X, acc);
+                        record_accumulate<R>(sm_tab, a, b, h, X, acc);
                     } else {
-                        float v[8];
-                        record_values(sm_tab, a, b, h, X, v);
+                        float v[R];
+                        record_values<R>(sm_tab, a, b, h, X, v);
                         const bool mine = rgl == rg_acc;
 #pragma unroll
-                        for (int r = 0; r < 8; ++r) acc[r] += mine ? v[r] : 0.f;
+                        for (int r = 0; r < R; ++r) acc[r] += mine ? v[r] : 0.f;
                         flush();
                         rg_acc = rg_last;
 #pragma unroll
-                        for (int r = 0; r < 8; ++r) acc[r] = mine ? 0.f : v[r];
+                        for (int r = 0; r < R; ++r) acc[r] = mine ? 0.f : v[r];
                     }
+                    if (ps + 1 == ps1 && rg_acc < ng) flush();
                     parity ^= 1;
                     rgl = nrgl;
                     col = ncol;
                 }
-                if (rg_acc < C.ng) flush();
             }
             first_chunk = false;
             __syncthreads();
-            // ---- epilogue: eight threads per row.  Thread j of a row takes warp j's partial sum (W = 8)
-            // or warps j and j + 8 (W = 16) and every eighth tail product; three shuffles add them in a
-            // fixed order; row scale, tail (Sec. 5.1), store.
-            for (int i = threadIdx.x; i < ng * 64; i += THREADS) {
-                const int t = i >> 3, j = i & 7;
-                const float* pr = part + (t >> 3) * W * 8 + (t & 7);
-                float v = pr[8 * j];
-                if (W == 16) v += pr[8 * (j + 8)];
+            // ---- epilogue: eight threads per row.  Thread k of a row takes the partial sums of slots k and k + 8
+            // and every eighth tail product; three shuffles add them in a fixed order; row scale, tail (Sec. 5.1).
+            for (int i = threadIdx.x; i < ng * R * 8; i += THREADS) {
+                const int t = i >> 3, k8 = i & 7;
+                const float* pr = part + (t / R) * W * R + t % R;
+                float v = pr[R * k8] + pr[R * (k8 + 8)];
                 v *= rs_sm[t];
-                for (int k = j; k < ntail; k += 8) v = fmaf(__half2float(tail_sm[t * 24 + k]), xtail[k], v);
+                for (int k = k8; k < ntail; k += 8) v = fmaf(__half2float(tail_sm[t * 24 + k]), xtail[k], v);
                 v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
                 v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
                 v += __shfl_xor_sync(0xFFFFFFFFu, v, 4);
-                const int row = ga * 8 + t;
-                if (j == 0 && row < P.N) yj[row] = v;
+                const int row = g * R + t;
+                if (k8 == 0 && row < P.N) yj[row] = v;
             }
-            g += ng;
         }
     }
 }
 
+namespace {
+
+struct ListShape {
+    int rows[kListMax], blocks[kListMax];
+    int count, max_blocks;
+};
+
+// Splits the list's row groups of R rows over at most `ctas` CTAs; fills P's shares and returns the CTAs used and
+// the passes of the busiest warp.
+int split_list(const ListShape& Q, int R, int ctas, ListParams& P, int* warp_passes) {
+    int n[kListMax] = {}, groups[kListMax] = {}, used = 0;
+    long long work = 0, total = 0;
+    for (int i = 0; i < Q.count; ++i) {
+        groups[i] = (Q.rows[i] + R - 1) / R;
+        work += (long long)groups[i] * Q.blocks[i];
+        total += groups[i];
+    }
+    if (total < ctas) ctas = int(total);
+    auto cost = [&](int i, int c) { return (long long)((groups[i] + c - 1) / c) * Q.blocks[i]; };  // of a share, with c CTAs
+    for (int i = 0; i < Q.count; ++i) {
+        const long long share = (long long)groups[i] * Q.blocks[i] * ctas / work;
+        n[i] = int(share < 1 ? 1 : (share > groups[i] ? groups[i] : share));
+        used += n[i];
+    }
+    while (used < ctas) {  // what rounding left goes to the matrix whose CTAs are loaded most
+        int at = -1;
+        for (int i = 0; i < Q.count; ++i)
+            if (n[i] < groups[i] && (at < 0 || cost(i, n[i]) > cost(at, n[at]))) at = i;
+        if (at < 0) break;
+        ++n[at];
+        ++used;
+    }
+    while (used > ctas) {  // the smallest matrices took a whole CTA each
+        int at = -1;
+        for (int i = 0; i < Q.count; ++i)
+            if (n[i] > 1 && (at < 0 || cost(i, n[i] - 1) < cost(at, n[at] - 1))) at = i;
+        if (at < 0) break;
+        --n[at];
+        --used;
+    }
+    *warp_passes = 0;
+    int begin = 0;
+    for (int i = 0; i < kListMax; ++i) {
+        P.cta_begin[i] = i < Q.count ? begin : 0x7FFFFFFF;
+        if (i >= Q.count) continue;
+        ListMatrix& M = P.m[i];
+        M.base = groups[i] / n[i];
+        M.extra = groups[i] % n[i];
+        M.begin = begin;
+        const int bs = Q.blocks[i] < 32 ? 32 : Q.blocks[i];
+        M.inv_bs = uint32_t(((1ull << 32) + bs - 1) / bs);
+        const long long cells = (long long)(M.base + (M.extra ? 1 : 0)) * bs;
+        const int passes = int(((cells + 31) / 32 + kListWarps - 1) / kListWarps);
+        if (passes > *warp_passes) *warp_passes = passes;
+        begin += n[i];
+    }
+    return begin;
+}
+
+}  // namespace
 
 cudaError_t launch_gemv_list(const ListDesc& list, int batch, const void* table, cudaStream_t s) {
     int sms = 0;
@@ -297,24 +414,46 @@ cudaError_t launch_gemv_list(const ListDesc& list, int batch, const void* table,
     if (e != cudaSuccess) return e;
     static PerDeviceOnce once;
     e = once.run([] {
-        cudaError_t r = cudaFuncSetAttribute(k_gemv_list<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-        if (r == cudaSuccess) r = cudaFuncSetAttribute(k_gemv_list<512, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-        if (r == cudaSuccess) r = cudaFuncSetAttribute(k_gemv_list<512, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        auto set = [](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); };
+        cudaError_t r = set(k_gemv_list<8, true>);
+        if (r == cudaSuccess) r = set(k_gemv_list<4, true>);
+        if (r == cudaSuccess) r = set(k_gemv_list<8, false>);
         return r;
     });
     if (e != cudaSuccess) return e;
-    // Two CTAs of eight warps per SM when their shared memory fits side by side (the next launch's
-    // CTAs can then start early); one CTA of sixteen warps otherwise; and without the shared-memory
-    // image of the activations when even that does not fit.
-    const ListSmem small = list_smem(8, list.max_blocks), large = list_smem(16, list.max_blocks);
-    const DeviceTables* tab = static_cast<const DeviceTables*>(table);
-    if (2u * (small.total + 1024u) <= 227u * 1024u) {
-        const int grid = list.total_groups < 2 * sms ? list.total_groups : 2 * sms;
-        return launch_pdl(k_gemv_list<256, true>, grid, 256, small.total, s, tab, list, batch);
+    ListShape Q;
+    Q.count = list.count;
+    Q.max_blocks = 0;
+    ListParams P;
+    for (int i = 0; i < list.count; ++i) {
+        const Problem& q = list.problems[i];
+        ListMatrix& M = P.m[i];
+        M.codes = q.codes;
+        M.x = static_cast<const __half*>(q.x);
+        M.row_scales = q.row_scales;
+        M.tail = static_cast<const __half*>(q.tail);
+        M.y = q.y;
+        M.N = q.N;
+        M.K = q.K;
+        Q.rows[i] = q.N;
+        Q.blocks[i] = (q.tail || q.K % 24 == 0) ? q.K / 24 : (q.K + 23) / 24;
+        if (Q.blocks[i] > Q.max_blocks) Q.max_blocks = Q.blocks[i];
     }
-    const int grid = list.total_groups < sms ? list.total_groups : sms;
-    if (large.total <= 227u * 1024u) return launch_pdl(k_gemv_list<512, true>, grid, 512, large.total, s, tab, list, batch);
-    return launch_pdl(k_gemv_list<512, false>, grid, 512, list_smem(16, 0).total, s, tab, list, batch);
+    P.batch = batch;
+    P.image_cols = Q.max_blocks;
+    const DeviceTables* tab = static_cast<const DeviceTables*>(table);
+    int passes = 0;
+    int grid = split_list(Q, 8, sms, P, &passes);
+    const uint32_t smem = list_smem(Q.max_blocks).total;
+    if (smem > 227u * 1024u)  // more columns than the shared-memory image can hold
+        return launch_pdl(k_gemv_list<8, false>, grid, kListThreads, list_smem(0).total, s, tab, P);
+    // A warp's pass over eight rows is a chain of eight blocks, and every warp runs a whole number of them: half
+    // records when their chain is shorter.  A block costs about 82 instructions, a pass another 60.
+    const long long chain8 = (long long)passes * (8 * 82 + 60);
+    grid = split_list(Q, 4, sms, P, &passes);
+    if ((long long)passes * (4 * 82 + 60) < chain8) return launch_pdl(k_gemv_list<4, true>, grid, kListThreads, smem, s, tab, P);
+    grid = split_list(Q, 8, sms, P, &passes);
+    return launch_pdl(k_gemv_list<8, true>, grid, kListThreads, smem, s, tab, P);
 }
 
 }  // namespace tetra
