@@ -19,12 +19,13 @@ struct LaneX {
     float step;       // 2^(E-22)
 };
 
+// An inactive lane keeps whatever planes it has read and contributes exact zeros through its step.
 __device__ __forceinline__ void lane_x_from_words(const uint32_t q[20], bool active, LaneX& X) {
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-        X.hi[k] = active ? q[k] : 0u;
-        X.mid[k] = active ? q[6 + k] : 0u;
-        X.lo[k] = active ? q[12 + k] : 0u;
+        X.hi[k] = q[k];
+        X.mid[k] = q[6 + k];
+        X.lo[k] = q[12 + k];
     }
     X.step = active ? __uint_as_float(q[18]) : 0.f;
 }

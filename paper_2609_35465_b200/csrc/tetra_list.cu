@@ -448,10 +448,12 @@ cudaError_t launch_gemv_list(const ListDesc& list, int batch, const void* table,
     if (smem > 227u * 1024u)  // more columns than the shared-memory image can hold
         return launch_pdl(k_gemv_list<8, false>, grid, kListThreads, list_smem(0).total, s, tab, P);
     // A warp's pass over eight rows is a chain of eight blocks, and every warp runs a whole number of them: half
-    // records when their chain is shorter.  A block costs about 82 instructions, a pass another 60.
-    const long long chain8 = (long long)passes * (8 * 82 + 60);
+    // records when their chain is shorter.  A block costs about 82 instructions, a pass about 150 more (record and
+    // activations in, row ends): measured on both sides of the line, 12288 x 4096: four passes of eight rows 9.4 us,
+    // seven of four 10.2 us; 6144 x 2560: two of eight 6.1 us, three of four 5.6 us.
+    const long long chain8 = (long long)passes * (8 * 82 + 150);
     grid = split_list(Q, 4, sms, P, &passes);
-    if ((long long)passes * (4 * 82 + 60) < chain8) return launch_pdl(k_gemv_list<4, true>, grid, kListThreads, smem, s, tab, P);
+    if ((long long)passes * (4 * 82 + 150) < chain8) return launch_pdl(k_gemv_list<4, true>, grid, kListThreads, smem, s, tab, P);
     grid = split_list(Q, 8, sms, P, &passes);
     return launch_pdl(k_gemv_list<8, true>, grid, kListThreads, smem, s, tab, P);
 }
