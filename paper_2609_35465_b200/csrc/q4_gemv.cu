@@ -22,8 +22,7 @@
 #include "../../include/tetra.h"
 #include "../../include/tetra_q4.h"
 #include "q4_common.cuh"
-#include "tetra_device.cuh"
-#include "tetra_launch.h"
+#include "tetra_gemv_common.cuh"
 
 namespace tetra {
 namespace {
@@ -58,6 +57,8 @@ __global__ void __launch_bounds__(256) k_q4_pack(const uint8_t* __restrict__ q, 
     constexpr int TPG = G / 64, CH = q4_chunk_bytes(G);
     const int strips = (N + 31) / 32, groups = K / G;
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    pdl_release();
+    pdl_wait();  // the matrix may come from, the packed one be read by, the kernel before
     const size_t chunks = size_t(strips) * groups;
     for (size_t chunk = (blockIdx.x * size_t(blockDim.x) + threadIdx.x) >> 5; chunk < chunks;
          chunk += (size_t(gridDim.x) * blockDim.x) >> 5) {
@@ -449,9 +450,7 @@ int tetra_q4_pack(const void* q_dev, const void* scale_dev, const void* offset_d
     const auto* q = static_cast<const uint8_t*>(q_dev);
     const auto *scale = static_cast<const __half*>(scale_dev), *offset = static_cast<const __half*>(offset_dev);
     auto* packed = static_cast<unsigned char*>(packed_dev);
-    if (G == 128) k_q4_pack<128><<<grid, 256, 0, s>>>(q, scale, offset, packed, N, K);
-    else k_q4_pack<64><<<grid, 256, 0, s>>>(q, scale, offset, packed, N, K);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_pdl(G == 128 ? k_q4_pack<128> : k_q4_pack<64>, int(grid), 256, 0, s, q, scale, offset, packed, N, K));
 }
 
 int tetra_q4_gemv(const void* packed_dev, const void* x_dev, float* y_dev, int N, int K, int G, int batch,
