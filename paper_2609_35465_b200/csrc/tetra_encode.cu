@@ -226,9 +226,12 @@ struct EncShared {
     float win_H[20];
     float win_G;
     int win_arg;
-    uint32_t found_row[3];    // index inside the section's list
-    uint32_t found_byte[3];
-    uint32_t found_cls[3];
+    // the winner so far, per section: byte pair, class, index and value of its table entry
+    int hit_pair[3], hit_cls[3], hit_k[3];
+    float hit_target[3];
+    // its row, looked for with the pair's byte and with its complement: index inside the section's list, or none
+    uint32_t found_row[3][2];
+    bool found[3][2];
 };
 static_assert(sizeof(EncShared) * kEncGroups <= 226 * 1024, "one CTA per SM");
 
@@ -503,12 +506,39 @@ __device__ __forceinline__ void half_odd(const float* w4, int nibble, float* out
 // ---------------------------------------------------------------------------
 // section tables
 // ---------------------------------------------------------------------------
-// T[k] = max(T[k], h + C[W][k - k']) for a high-half entry h of weight and kappa (., k'): two norms per addition.
-template <int KH, int W, int KMAX>
-__device__ __forceinline__ void combine_even(float h, const float (&C)[kCells], float (&T)[kMaxK + 1]) {
-    static_for<0, kLastC<W> + 1>([&](auto ki) {
-        constexpr int KL = decltype(ki)::value;
-        if constexpr (KH + KL <= KMAX) T[KH + KL] = fmaxf(T[KH + KL], __fadd_rn(h, C[kAtC<W> + KL]));
+// The possible kappas of a weight in a high-half table.
+constexpr int cell_count(const Cells& C, int w) {
+    int n = 0;
+    for (int k = 0; k <= kMaxK; ++k) n += C.v[4][w][k] ? 1 : 0;
+    return n;
+}
+constexpr int cell_nth(const Cells& C, int w, int i) {
+    for (int k = 0; k <= kMaxK; ++k)
+        if (C.v[4][w][k] && i-- == 0) return k;
+    return -1;
+}
+template <const Cells& C, int W> constexpr int kCellCount = cell_count(C, W);
+template <const Cells& C, int W, int I> constexpr int kCellNth = cell_nth(C, W, I);
+template <int TABLE, int W, int K> constexpr int kAtHigh = TABLE == 0 ? kAtH<W, K> : (TABLE == 1 ? kAtA<W, K> : kAtB<W, K>);
+
+// T[n] = max(T[n], h[W][k] + C[V][n - k]) over the cells k of weight W of a high-half table (TABLE 0: H, 1: A, 2: B;
+// CELLS: its possible cells); two cells at a time, so that most maxima take two candidates.
+template <int TABLE, const Cells& CELLS, int W, int V, int KMAX>
+__device__ __forceinline__ void combine_even(const float* hi, const float (&C)[kCells], float (&T)[kMaxK + 1]) {
+    constexpr int LAST = kLastC<V>;
+    static_for<0, (kCellCount<CELLS, W> + 1) / 2>([&](auto ti) {
+        constexpr int I = 2 * decltype(ti)::value;
+        constexpr int KA = kCellNth<CELLS, W, I>, KB = kCellNth<CELLS, W, I + 1>;  // KB = -1: no second cell
+        const float ha = hi[kAtHigh<TABLE, W, KA>];
+        float hb = kNeg;
+        if constexpr (KB >= 0) hb = hi[kAtHigh<TABLE, W, KB>];
+        static_for<0, KMAX + 1>([&](auto ni) {
+            constexpr int N = decltype(ni)::value;
+            constexpr bool a = N >= KA && N - KA <= LAST, b = KB >= 0 && N >= KB && N - KB <= LAST;
+            if constexpr (a && b) T[N] = max3(T[N], __fadd_rn(ha, C[kAtC<V> + N - KA]), __fadd_rn(hb, C[kAtC<V> + N - KB]));
+            else if constexpr (a) T[N] = fmaxf(T[N], __fadd_rn(ha, C[kAtC<V> + N - KA]));
+            else if constexpr (b) T[N] = fmaxf(T[N], __fadd_rn(hb, C[kAtC<V> + N - KB]));
+        });
     });
 }
 
@@ -519,23 +549,15 @@ __device__ __forceinline__ void section_even(const float* lo, const float* hi, f
     for (int i = 0; i < kCells; ++i) C[i] = lo[i];
     static_for<0, kMaxW + 1>([&](auto wi) {
         constexpr int W = decltype(wi)::value;
-        static_for<0, kMaxK + 1>([&](auto ki) {
-            constexpr int K = decltype(ki)::value;
-            if constexpr (MID) {
-                if constexpr (W <= 7 && kFree.v[4][W][K]) combine_even<K, 7 - W, 7>(hi[kAtH<W, K>], C, T1);
-                if constexpr (W <= 8 && kLessM.v[4][W][K])
-                    combine_even<K, 8 - W, kMaxK - 1>(hi[kAtA<W, K>], C, T0);
-            } else {
-                if constexpr (W <= 9 && kFree.v[4][W][K]) {
-                    const float h = hi[kAtH<W, K>];
-                    combine_even<K, 9 - W, kMaxK>(h, C, T1);
-                    if constexpr (W <= 8) combine_even<K, 8 - W, kMaxK - 1>(h, C, T0);
-                }
-                if constexpr (W <= 10 && kLess0.v[4][W][K])
-                    combine_even<K, 10 - W, kMaxK - 1>(hi[kAtA<W, K>], C, T0);
-                if constexpr (kLess1.v[4][W][K]) combine_even<K, 11 - W, kMaxK>(hi[kAtB<W, K>], C, T1);
-            }
-        });
+        if constexpr (MID) {
+            if constexpr (W <= 7) combine_even<0, kFree, W, 7 - W, 7>(hi, C, T1);
+            if constexpr (W <= 8) combine_even<1, kLessM, W, 8 - W, kMaxK - 1>(hi, C, T0);
+        } else {
+            if constexpr (W <= 9) combine_even<0, kFree, W, 9 - W, kMaxK>(hi, C, T1);
+            if constexpr (W <= 8) combine_even<0, kFree, W, 8 - W, kMaxK - 1>(hi, C, T0);
+            if constexpr (W <= 10) combine_even<1, kLess0, W, 10 - W, kMaxK - 1>(hi, C, T0);
+            combine_even<2, kLess1, W, 11 - W, kMaxK>(hi, C, T1);
+        }
     });
 }
 
@@ -760,16 +782,18 @@ __device__ __forceinline__ float half_corr(bool even, const float* w4, int nibbl
     return sum;
 }
 
-// Finds the row (and which byte of the pair) whose correlation is `target` at index k of the section's table.
-__device__ __noinline__ void trace_section(EncShared& S, const DeviceTables* __restrict__ tab, bool even, int s, int pair, int cls, int k,
-                                           float target) {
+// Looks for the row of section s whose correlation with the pair's byte (e = 0) or its complement (e = 1) is the
+// winner's at its index of the section's table.
+__device__ __noinline__ void trace_section(EncShared& S, const DeviceTables* __restrict__ tab, bool even, int s, int e) {
     const int lane = threadIdx.x & 31;
+    const int cls = S.hit_cls[s], k = S.hit_k[s];
+    const float target = S.hit_target[s];
     const int w_total = 2 * k + cls;  // odd parity: the row's weight
     const float* w = S.w + 8 * s;
     uint32_t row = 0;
-    uint32_t byte = S.bytes[pair];
+    const uint32_t byte = S.bytes[S.hit_pair[s]] ^ (e ? 0xFFu : 0u);
     bool found = false;
-    for (int e = 0; e < 2 && !found; ++e, byte ^= 0xFFu) {
+    {
         const int nlo = int(byte & 15u), nhi = int(byte >> 4);
         const int kap = k - ones_offset(byte);
         const float* lo = even ? S.lo[s] + nlo * kLoStride : S.lo_odd[s] + nlo * kOddLoStride;
@@ -828,9 +852,8 @@ __device__ __noinline__ void trace_section(EncShared& S, const DeviceTables* __r
                 have = true;
             }
         }
-        if (!have) continue;
         // 2. the low half: sum, norm and membership decide
-        for (int i0 = 0; i0 < kHalfVectors && !found; i0 += 32) {
+        for (int i0 = 0; i0 < kHalfVectors && have && !found; i0 += 32) {
             const int i = i0 + lane;
             bool hit = false;
             uint32_t cand = 0;
@@ -849,7 +872,6 @@ __device__ __noinline__ void trace_section(EncShared& S, const DeviceTables* __r
                 found = true;
             }
         }
-        if (found) break;
     }
     // 3. its index: the shells of a class follow one another, rows of a shell ascend
     int wt = 0;
@@ -874,14 +896,13 @@ __device__ __noinline__ void trace_section(EncShared& S, const DeviceTables* __r
     const int at = block0 + lane;
     const uint32_t eq = __ballot_sync(0xFFFFFFFFu, lane < stride && at < end && __ldg(rows + (at < end ? at : 0)) == row);
     if (lane == 0) {
-        S.found_row[s] = uint32_t(eq ? block0 + __ffs(int(eq)) - 1 : 0);
-        S.found_byte[s] = byte;
-        S.found_cls[s] = uint32_t(cls);
+        S.found_row[s][e] = uint32_t(eq ? block0 + __ffs(int(eq)) - 1 : 0);
+        S.found[s][e] = found && eq;
     }
 }
 
-// Warp s < 3: the winning entry of the objective, back through the join, then the row of section s.
-__device__ __noinline__ void trace(EncShared& S, const DeviceTables* __restrict__ tab, bool even, int s, int end_pair, int par, int n) {
+// One warp: the winning entry of the objective, back through the join to the entries of the section tables.
+__device__ __noinline__ void trace_join(EncShared& S, bool even, int end_pair, int par, int n) {
     const int lane = threadIdx.x & 31;
     const int cls3 = (even ? 0 : 1) ^ par;
     const int row_len = even ? kRow : kOddRow;
@@ -918,14 +939,19 @@ __device__ __noinline__ void trace(EncShared& S, const DeviceTables* __restrict_
     const int w_c1 = __shfl_sync(0xFFFFFFFFu, c1, src), w_c2 = w_c1 ^ par;
     const int w_raised = __shfl_sync(0xFFFFFFFFu, raised, src), w_shift = __shfl_sync(0xFFFFFFFFu, shift, src);
     const int j2 = max(q - w_shift - i1, 0);
-    if (s == 0) trace_section(S, tab, even, 0, w_p1, w_c1, max(i1 - w_raised, 0), S.F1[w_raised][w_c1][w_p1 * row_len + i1]);
-    else if (s == 1) trace_section(S, tab, even, 1, w_p2, w_c2, j2, S.F2[w_c2][w_p2 * row_len + j2]);
-    else trace_section(S, tab, even, 2, end_pair, cls3, k3, S.F3[cls3][end_pair * row_len + k3]);
+    if (lane < 3) {
+        const int pair = lane == 0 ? w_p1 : (lane == 1 ? w_p2 : end_pair), cls = lane == 0 ? w_c1 : (lane == 1 ? w_c2 : cls3);
+        const int at = lane == 0 ? i1 : (lane == 1 ? j2 : k3);
+        const float* rows = lane == 0 ? S.F1[w_raised][w_c1] : (lane == 1 ? S.F2[w_c2] : S.F3[cls3]);
+        S.hit_pair[lane] = pair;
+        S.hit_cls[lane] = cls;
+        S.hit_k[lane] = lane == 0 ? max(i1 - w_raised, 0) : at;
+        S.hit_target[lane] = rows[pair * row_len + at];
+    }
 }
 
 template <bool EVEN>
-__device__ __forceinline__ void search_parity(EncShared& S, const DeviceTables* __restrict__ tab, int tid, bool live, float& best_val,
-                                              uint64_t& best_word) {
+__device__ __forceinline__ void search_parity(EncShared& S, int tid, bool live, float& best_val, bool& best_even) {
     const int warp = tid >> 5, lane = tid & 31;
     if (live) {  // section tables: warps 0, 1 = section 0, warps 2, 3 = section 1, warps 4, 5 = section 2
         const int s = tid >> 6, pair = tid & 63;
@@ -973,6 +999,7 @@ __device__ __forceinline__ void search_parity(EncShared& S, const DeviceTables* 
         better = top > best_val;  // the same for all threads of the group
         if (better) {
             best_val = top;
+            best_even = EVEN;
             if (uint32_t(tid) == winner) {
 #pragma unroll
                 for (int i = 0; i < kH; ++i) S.win_H[i] = H[i];
@@ -981,20 +1008,28 @@ __device__ __forceinline__ void search_parity(EncShared& S, const DeviceTables* 
             }
         }
     }
-    if (!__syncthreads_or(better)) return;
-    if (better && warp < 3) trace(S, tab, EVEN, warp, int(winner) & 63, int(winner) >> 6, S.win_arg);
     __syncthreads();
-    if (better && warp == 0) {
-        const uint32_t c1 = S.found_byte[0], c2 = S.found_byte[1], c3 = S.found_byte[2];
-        const uint32_t b1 = c1 >> 7, b3 = c3 >> 7, s8 = (b1 ? ~c1 : c1) & 63u;
-        const uint32_t leaves = tab->paper.branches[16 * s8 + (lane & 15)] & 0xFFu;
-        const uint32_t eq = __ballot_sync(0xFFFFFFFFu, leaves == c2);
-        const uint32_t b2 = eq ? uint32_t(__ffs(int(eq)) - 1) & 15u : 0u;
-        const uint32_t i2 = S.found_row[1] + (S.found_cls[1] ? uint32_t(kMiddleClass0) : 0u);
-        best_word = uint64_t(S.found_row[0]) | (uint64_t(i2) << 11) | (uint64_t(S.found_row[2]) << 22) | (uint64_t(s8) << 33) |
-                    (uint64_t(b1) << 39) | (uint64_t(b2) << 40) | (uint64_t(b3) << 44) | (uint64_t(EVEN ? 0 : 1) << 45) |
-                    (uint64_t(S.found_cls[0]) << 46);
+    if (better && warp == 0) trace_join(S, EVEN, int(winner) & 63, int(winner) >> 6, S.win_arg);
+    __syncthreads();
+}
+
+// The file-order word (without the gain bit) of the traced winner; one warp.
+__device__ __forceinline__ uint64_t winner_word(const EncShared& S, const DeviceTables* __restrict__ tab, bool even) {
+    const int lane = threadIdx.x & 31;
+    uint32_t c[3], row[3];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        const int e = S.found[s][0] ? 0 : 1;
+        c[s] = S.bytes[S.hit_pair[s]] ^ (e ? 0xFFu : 0u);
+        row[s] = S.found_row[s][e];
     }
+    const uint32_t b1 = c[0] >> 7, b3 = c[2] >> 7, s8 = (b1 ? ~c[0] : c[0]) & 63u;
+    const uint32_t leaves = tab->paper.branches[16 * s8 + (lane & 15)] & 0xFFu;
+    const uint32_t eq = __ballot_sync(0xFFFFFFFFu, leaves == c[1]);
+    const uint32_t b2 = eq ? uint32_t(__ffs(int(eq)) - 1) & 15u : 0u;
+    const uint32_t i2 = row[1] + (S.hit_cls[1] ? uint32_t(kMiddleClass0) : 0u);
+    return uint64_t(row[0]) | (uint64_t(i2) << 11) | (uint64_t(row[2]) << 22) | (uint64_t(s8) << 33) | (uint64_t(b1) << 39) |
+           (uint64_t(b2) << 40) | (uint64_t(b3) << 44) | (uint64_t(even ? 0 : 1) << 45) | (uint64_t(uint32_t(S.hit_cls[0])) << 46);
 }
 
 __global__ void __launch_bounds__(kEncThreads * kEncGroups, 1)
@@ -1015,42 +1050,47 @@ k_encode(const float* __restrict__ w, const float* __restrict__ sigma, const Dev
         const size_t block = first + size_t(group) * gridDim.x + blockIdx.x;
         const bool mine = block < nblocks;
         if (tid < 24) S.w[tid] = mine ? w[block * 24 + tid] : 0.f;
+        if (tid < 3) S.hit_pair[tid] = S.hit_cls[tid] = S.hit_k[tid] = 0;  // what a block without a best point (NaN) is traced to
         __syncthreads();
         float wn2 = 0.f;
 #pragma unroll
         for (int j = 0; j < 24; ++j) wn2 = fmaf(S.w[j], S.w[j], wn2);
         const bool live = wn2 != 0.f;  // a zero block encodes as the all-zero word
-        if (live) {  // half tables: warps 0..2 the even parity of section 0..2, warps 3..5 the odd one; lanes 0..15 the low half
-            const int s = (tid >> 5) % 3, nibble = tid & 15;
-            const bool high = (tid & 16) != 0, odd = tid >= 96;
-            if (!odd) {
-                float* lo = S.lo[s] + nibble * kLoStride;
-                float* hi = S.hi[s] + nibble * kHiStride;
-                if (s == 1) {
-                    if (high) half_even<true, true>(S.w + 12, nibble, hi);
-                    else half_even<false, true>(S.w + 8, nibble, lo);
-                } else {
-                    if (high) half_even<true, false>(S.w + 8 * s + 4, nibble, hi);
-                    else half_even<false, false>(S.w + 8 * s, nibble, lo);
-                }
-            } else {
-                float* lo = S.lo_odd[s] + nibble * kOddLoStride;
-                float* hi = S.hi_odd[s] + nibble * kOddHiStride;
-                if (s == 1) {
-                    if (high) half_odd<true, true>(S.w + 12, nibble, hi);
-                    else half_odd<false, true>(S.w + 8, nibble, lo);
-                } else {
-                    if (high) half_odd<true, false>(S.w + 8 * s + 4, nibble, hi);
-                    else half_odd<false, false>(S.w + 8 * s, nibble, lo);
-                }
+        if (live) {
+            // half tables, lane = section (0 or 2) and nibble, or nibble of the middle section: warps 0 and 1 the high
+            // and low halves of the outer sections at even parity, warps 2 and 3 those of the middle one, warps 4 and
+            // 5 the odd parity
+            const int nibble = tid & 15, outer = (tid & 16) ? 2 : 0;
+            float *lo = S.lo[outer] + nibble * kLoStride, *hi = S.hi[outer] + nibble * kHiStride;
+            float *lo_odd = S.lo_odd[outer] + nibble * kOddLoStride, *hi_odd = S.hi_odd[outer] + nibble * kOddHiStride;
+            const float* wo = S.w + 8 * outer;
+            switch (tid >> 5) {
+                case 0: half_even<true, false>(wo + 4, nibble, hi); break;
+                case 1: half_even<false, false>(wo, nibble, lo); break;
+                case 2: if (outer == 0) half_even<true, true>(S.w + 12, nibble, S.hi[1] + nibble * kHiStride); break;
+                case 3: if (outer == 0) half_even<false, true>(S.w + 8, nibble, S.lo[1] + nibble * kLoStride); break;
+                case 4:
+                    half_odd<true, false>(wo + 4, nibble, hi_odd);
+                    half_odd<false, false>(wo, nibble, lo_odd);
+                    break;
+                default:
+                    if (outer == 0) {
+                        half_odd<true, true>(S.w + 12, nibble, S.hi_odd[1] + nibble * kOddHiStride);
+                        half_odd<false, true>(S.w + 8, nibble, S.lo_odd[1] + nibble * kOddLoStride);
+                    }
             }
         }
         __syncthreads();
         float best_val = kNeg;
-        uint64_t best_word = 0;
-        search_parity<false>(S, tab, tid, live, best_val, best_word);
+        bool best_even = false;
+        search_parity<false>(S, tid, live, best_val, best_even);
+        search_parity<true>(S, tid, live, best_val, best_even);
+        if (live) {  // a warp per section and byte of its pair
+            const int warp = tid >> 5;
+            trace_section(S, tab, best_even, warp >> 1, warp & 1);
+        }
         __syncthreads();
-        search_parity<true>(S, tab, tid, live, best_val, best_word);
+        const uint64_t best_word = live && tid < 32 && best_val > 0.f ? winner_word(S, tab, best_even) : 0ull;
 
         if (mine && tid == 0) {
             const float sg_ = sigma ? sigma[block] : 1.f;
