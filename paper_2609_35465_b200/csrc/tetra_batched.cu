@@ -1,694 +1,494 @@
-// Decode-and-multiply for 2..16 activation vectors at once (Eq. (2), Sec. 5.1): k_gemv_batched (5..16
-// vectors, described first) and k_gemv_few (2..4 vectors, further down).
+// Decode-and-multiply for 2..16 activation vectors at once (Eq. (2), Sec. 5.1): a block is decoded once and
+// multiplied with every vector, in one launch.
 //
-// A block is decoded once and multiplied with every vector, so the decode cost
-// is shared.  The products over a block's 24 coordinates for up to 16 vectors
-// are a small dense contraction, int8 x int8 -> int32, and run on the tensor
-// cores (mma.sync m16n8k32); everything around it (field extraction, table
-// lookups, per-block scale, FP32 accumulation) is the batch-1 decoder.
+// The products of a block's 24 coordinates with up to 16 vectors are a small dense contraction and run on the tensor
+// cores: mma.sync m16n8k16 + m16n8k8, float16 x float16 with float32 accumulation.  Half of minus a coordinate,
+// -y / 2 = z + p / 2, is a float16 that two logic operations and one addition make from the decoder's nibbles, and
+// the activations ARE float16, so both operands and every product are exact.  (The three int8 planes of 24-bit fixed
+// point that the batch-1 kernels use cost three MMAs and five instructions per result here; the float32 result costs
+// half a packed FFMA.)  mma.sync rather than tcgen05: a CTA owns about 28 rows of a 4096-row matrix, a tile of 16
+// rows keeps sixteen warps busy with that, 128 rows would not, and the tensor cores are far from the limit.
 //
-// Thread layout: a warp owns two row blocks of 16 rows, a CTA of 16 warps a tile group of 512 rows, and a
-// warp walks the block columns four at a time; such a (tile group, four columns) cell is the unit of work,
-// and the CTAs take equal contiguous ranges of the tile-group-major cell order.  The codes of a warp's pass
-// (four row groups x three parts x four columns) arrive through the warp's own cp.async ring, one pass
-// ahead.  In one pass lane l decodes four blocks (row l % 16 of row block j % 2, column l / 16 + 2 (j / 2),
-// j = 0..3) and writes each block's 24 int8 coordinates and its scale as a row of a shared-memory tile;
-// the warp then loads the tiles as MMA A fragments with ldmatrix and multiplies them with the three int8
-// planes of the activations' 24-bit fixed-point image (B fragments, read once per column and used for both
-// row blocks; coordinates 24..31 of the image are zero, so the tile's bytes there do not matter).  The image
-// of the CTA's next 32 (column, vector group) pairs is built by the CTA itself, in shared memory: once for
-// most calls (behind the first pass's decode), again behind two CTA barriers when the CTA's range is
-// longer; between those the warps never wait for one another.  The int32 results of the planes are
-// combined exactly, converted once, scaled by block scale x activation step and added into FP32
-// accumulators that the lane keeps for its (row, vector) pairs: no cross-lane reduction is needed.  When a
-// CTA's range leaves a tile group, its partial sums go to the scratch area as one piece; a second, small
-// kernel adds the pieces of every tile group in CTA order (fixed order, no atomics, no flags), applies the
-// row scale and the tail.  The only waits are CTA barriers, cp.async groups and griddepcontrol.wait.
+// A warp's step is up to four tiles of 16 rows x the same four block columns: lane 4 q + t decodes rows q and q + 8 of
+// a tile at column t and leaves each block's 24 halves in a shared-memory tile whose rows keep stores and ldmatrix
+// conflict-free; the block's scale stays in the lane and reaches the lanes that hold the block's results by a
+// shuffle.  The sixteen warps of a CTA take every sixteenth column quad, so a warp needs nothing from the others until
+// the end: its words come straight from global memory one step ahead, the four columns' activations through its own
+// cp.async buffer, and its accumulators live in registers.  (Activations of many columns staged by the CTA, warps
+// cut along the rows: 10.0 / 30 us for 4096 x 4096 with three vectors / 4096 x 12288 with sixteen.)
+//
+// One launch, no scratch memory: what a call of a few microseconds consists of is latency, and the second kernel that
+// added the CTAs' partial sums cost more than the products of a 4096 x 4096 matrix.  A CTA owns whole rows; where
+// rows are too few for all SMs, a cluster of two to eight CTAs shares them, each takes a range of columns, and the
+// partial sums meet through distributed shared memory.  Sums are added in warp order, then CTA order: bit-identical
+// from run to run.
+//
+// Bound by instruction issue in the steps (decode, conversion, tile) and, for small matrices, by the chain of
+// launch, tables, one step and sums.
 #include <cuda_fp16.h>
 
+#include "q4_common.cuh"
 #include "tetra_gemv_common.cuh"
 
 namespace tetra {
 
 constexpr int kBatThreads = 512;
 constexpr int kBatWarps = kBatThreads / 32;
-#ifndef TETRA_BAT_RB1
-#define TETRA_BAT_RB1 2  // row blocks per warp, batch <= 8
-#endif
-#ifndef TETRA_BAT_RB2
-#define TETRA_BAT_RB2 2  // row blocks per warp, batch 9..16
-#endif
-constexpr int kPassTiles = 8;  // 16-row x 1-column tiles per warp and pass (four blocks per lane)
-// Activation image per block column and vector group n (vectors 8 n .. 8 n + 7): two 16-byte chunks per
-// lane, stored chunk-major ([chunk][lane][4 words]) so that a 128-bit access per chunk is contiguous over
-// the warp:
-//   chunk 2 n     = B-fragment registers (plane 0, h 0), (0, 1), (1, 0), (1, 1)
-//   chunk 2 n + 1 = (2, 0), (2, 1), step of vector 8 n + 2 t, step of vector 8 n + 2 t + 1
-// where the lane multiplies with vector 8 n + lane / 4, t = lane % 4, register h = 0 holds coordinates
-// of the decoder's word t and h = 1 those of word 4 + t (words 6, 7 and unused vectors are zero), and
-// the steps are those of the lane's two result columns.  A column takes ng x 1 KiB (ng = 1 or 2 groups).
-// The image lives in shared memory only: the CTA builds it for a chunk of its passes at a time.
-constexpr int kBatGroupWords = 2 * 32 * 4;
+constexpr uint32_t kTileCol = 16 * 48 + 32;    // bytes per column of a tile: 16 rows of 24 halves, bank spread
+constexpr uint32_t kTileBytes = 4 * kTileCol;  // four columns
+constexpr uint32_t kXVec = 4 * 48 + 16;        // bytes per vector of an activation buffer: four columns, bank spread
+constexpr int kBatMaxTiles = 4;                // row tiles whose sums a warp holds at a time
 
-// One thread per (block column of a pass, vector, t) builds the words of lane (vector % 8) * 4 + t: the
-// thread reads the (up to) eight activations that lane multiplies with, the column's largest magnitude is
-// found over the four threads of the vector (two shuffles), and the 24-bit fixed-point values are split
-// into the three int8 planes.  A float16 x_j is held exactly when |x_j| >= 2^(E-12), E the exponent of the
-// column's largest magnitude; smaller ones are rounded to a multiple of the step 2^(E-22).
-struct ImageTask {
-    float v[8];  // the coordinates of the decoder's words t and (t < 2) 4 + t of the column
+struct BatParams {
+    const unsigned char* codes;
+    const float* row_scales;
+    const __half* x;
+    const __half* tail;
+    float* y;
+    int32_t N, K, B, batch;
+    int32_t tiles, quads;    // row tiles of 16, column quads
+    int32_t groups;          // clusters: groups of CTAs that share rows
+    int32_t cluster;         // CTAs of a cluster
 };
-__device__ __forceinline__ void image_load(const __half* __restrict__ x, int K, int batch, int col, int vec, int t,
-                                           ImageTask& T) {
-    const __half* xv = x + size_t(vec) * K;
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int k = 24 * col + word_coordinate(4 * h + t, i);
-            T.v[4 * h + i] = (vec < batch && (h == 0 || t < 2) && k < K) ? __half2float(__ldg(xv + k)) : 0.f;
-        }
+
+// Tiles decoded together: two blocks per lane and tile; four blocks in flight hide the table lookups better, which the
+// shared memory allows where eight vectors' activations are the most.
+__host__ __device__ constexpr int tiles_at_once(int ng, int nt) { return ng == 1 && nt > 1 ? 2 : 1; }
+// Row stride, in floats, of the partial sums (8 ng vectors): even, so that pairs stay aligned.
+__host__ __device__ constexpr int part_stride(int ng) { return 8 * ng + 2; }
+struct BatSmem {
+    // offsets from the 16 KiB-aligned table copy; total includes the alignment slack
+    uint32_t warps, per_warp, rs, tail, xtail, total;
+};
+__host__ __device__ constexpr BatSmem bat_smem(int ng, int nt) {
+    BatSmem S{};
+    S.warps = uint32_t(kFastBytes);  // per warp: tiles, two activation buffers; afterwards the sums of all warps
+    S.per_warp = uint32_t(tiles_at_once(ng, nt)) * kTileBytes + 2u * 8u * uint32_t(ng) * kXVec;
+    S.rs = S.warps + kBatWarps * S.per_warp;
+    S.tail = S.rs + uint32_t(nt) * 64u;                 // half [rows][24]
+    S.xtail = S.tail + uint32_t(nt) * (16u * 48u);      // float [16][24]
+    S.total = S.xtail + 16u * 96u + kSmAlign;
+    return S;
 }
-// group_base: shared-memory address of the column's 1 KiB group for the vector's group of eight.
-__device__ __forceinline__ void image_store(const ImageTask& T, uint32_t group_base, int vec, int t) {
-    // largest magnitude as a bit pattern (a NaN or an infinity then counts as the largest)
-    uint32_t mxb = 0u;
+static_assert(kBatWarps * kBatMaxTiles * 16 * part_stride(2) * 4 <= kBatWarps * bat_smem(2, kBatMaxTiles).per_warp, "sums fit");
+static_assert(bat_smem(1, 4).total <= 227 * 1024 && bat_smem(2, 4).total <= 227 * 1024, "shared memory");
+
+// Half of minus the point, float16 x 2: a[4 s + t] = coordinates 2 t and 2 t + 1 of section s.  Returns the block's scale
+// (minus the gain over sqrt(16 m)).  A nibble z sits in the mantissa of 64 (as z + 8: the exclusive or that sets
+// the exponent flips its sign bit) with p in the bit below: 72 + z + p / 2.  The squared norm of the halves, 4 m, is
+// exact in float16 (at most 104, terms of a quarter); with 1024 added it is the mantissa itself.
+template <bool HI>
+__device__ __forceinline__ float decode_halves(uint32_t sm_tab, uint32_t w0, uint32_t w1pair, uint32_t (&a)[12]) {
+    NibbleBlock nb;
+    decode_nibbles<HI>(sm_tab, w0, w1pair, nb);
+    const uint32_t magic = (nb.p4 & 4u) * 0x00020002u + 0x54805480u;
+    const __half2 bias = __half2half2(__ushort_as_half(0xD480));  // -72
+    __half2 n0{}, n1{};
 #pragma unroll
-    for (int i = 0; i < 8; ++i) mxb = max(mxb, __float_as_uint(T.v[i]) & 0x7FFFFFFFu);
-    mxb = max(mxb, __shfl_xor_sync(0xFFFFFFFFu, mxb, 1));
-    mxb = max(mxb, __shfl_xor_sync(0xFFFFFFFFu, mxb, 2));
-    const bool finite = mxb < 0x7F800000u;
-    const uint32_t e = mxb >> 23;  // biased exponent of the largest
-    // a NaN or an infinity in the column makes its step NaN: every row that reads the column comes out NaN
-    const float step = !finite ? __uint_as_float(0x7FC00000u) : (mxb ? __uint_as_float((e - 22u) << 23) : 0.f);
-    const float inv = (finite && mxb) ? __uint_as_float((276u - e) << 23) : 0.f;
-    uint32_t b[3][2];
+    for (int s = 0; s < 3; ++s) {
+        const uint32_t z = nb.z[s];
+        const uint32_t v[4] = {((z << 4) & 0x00F000F0u) ^ magic, (z & 0x00F000F0u) ^ magic, ((z >> 4) & 0x00F000F0u) ^ magic,
+                               ((z >> 8) & 0x00F000F0u) ^ magic};
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        uint32_t hi = 0, mid = 0, lo = 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int q = __float2int_rn(T.v[4 * h + i] * inv);
-            hi |= (uint32_t(q >> 16) & 0xFFu) << (8 * i);
-            mid |= (uint32_t(q >> 8) & 0xFFu) << (8 * i);
-            lo |= (uint32_t(q) & 0xFFu) << (8 * i);
+        for (int t = 0; t < 4; ++t) {
+            const __half2 h = __hadd2(*reinterpret_cast<const __half2*>(&v[t]), bias);
+            a[4 * s + t] = *reinterpret_cast<const uint32_t*>(&h);
+            __half2& n = (t & 1) ? n1 : n0;
+            n = (s == 0 && t < 2) ? __hmul2(h, h) : __hfma2(h, h, n);
         }
-        b[0][h] = hi;
-        b[1][h] = mid;
-        b[2][h] = lo;
     }
-    const int g = vec & 7, ln = g * 4 + t;
-    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(group_base + ln * 16), "r"(b[0][0]), "r"(b[0][1]),
-                 "r"(b[1][0]), "r"(b[1][1]) : "memory");
-    asm volatile("st.shared.v2.u32 [%0], {%1,%2};" ::"r"(group_base + 512 + ln * 16), "r"(b[2][0]), "r"(b[2][1]) : "memory");
-    // the step goes to the eight lanes whose results belong to this vector: lane % 4 = (vec % 8) / 2, any lane / 4
+    const __half2 n = __hadd2(n0, n1);
+    const __half m4 = __hadd(__hadd(__low2half(n), __high2half(n)), __ushort_as_half(0x6400));  // 1024 + 4 m
+    return lds32f(uint32_t(__half_as_ushort(m4)) * 4u + nb.goff - 0x6400u * 4u);
+}
+
+// Eight consecutive activations starting at x[0], of which `n` exist; x is 2-byte aligned.
+__device__ __forceinline__ uint4 load_eight(const __half* x, int n) {
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+    const unsigned short* h = reinterpret_cast<const unsigned short*>(x);
+    if (n < 8) {
 #pragma unroll
-    for (int gg = 2 * t; gg < 2 * t + 2; ++gg)
-        asm volatile("st.shared.f32 [%0], %1;" ::"r"(group_base + 512 + (gg * 4 + (g >> 1)) * 16 + 8 + 4 * (vec & 1)), "f"(step)
-                     : "memory");
+        for (int i = 0; i < 8; ++i)
+            if (i < n) w[i >> 1] |= uint32_t(__ldg(h + i)) << (16 * (i & 1));
+    } else if ((reinterpret_cast<uintptr_t>(x) & 3) == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = __ldg(reinterpret_cast<const uint32_t*>(x) + i);
+    } else {
+        const uint32_t first = __ldg(h), last = __ldg(h + 7);
+        const uint32_t* mid = reinterpret_cast<const uint32_t*>(h + 1);
+        const uint32_t m0 = __ldg(mid), m1 = __ldg(mid + 1), m2 = __ldg(mid + 2);
+        w[0] = first | (m0 << 16);
+        w[1] = __funnelshift_l(m0, m1, 16);
+        w[2] = __funnelshift_l(m1, m2, 16);
+        w[3] = (m2 >> 16) | (last << 16);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-__device__ __forceinline__ void mma_s8s8(int (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
-                 : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "r"(0));
+__device__ __forceinline__ void mma_k16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+                 : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
 }
-__device__ __forceinline__ void mma_s8u8(int (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.s8.u8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
-                 : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "r"(0));
+__device__ __forceinline__ void mma_k8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a0), "r"(a1), "r"(b0));
 }
-
-constexpr int kTileRow = 48;                // bytes per tile row: 24 coordinates, scale, 20 pad
-constexpr int kTileBytes = 16 * kTileRow;   // (48-byte rows keep ldmatrix and the tile stores conflict-free)
-constexpr int kBatWarpTiles = kPassTiles * kTileBytes;  // coordinate tiles (a row: 24 coordinates, the block scale, pad)
-constexpr int kBatColBytesPerGroup = kBatGroupWords * 4;                   // image of one column, per ng
-// Code ring of a warp: two slots of one pass (the warp's four row groups x three parts x four columns x 16
-// bytes); a row group takes 224 bytes, so that the loads of a pass (two row groups x two parts x two
-// columns x four words per instruction) fall into different banks.
-constexpr uint32_t kBatRingGroup = 224, kBatRingSlot = 4 * kBatRingGroup;
-constexpr int kBatWarpSmem = kBatWarpTiles + 2 * int(kBatRingSlot);
-constexpr int kImageGroups = 32;  // (column, vector group) pairs of the activation image held at a time: 32 KiB
-
-__device__ __forceinline__ void lds128(uint32_t saddr, uint32_t (&v)[4]) {
-    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(saddr));
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float cluster_load(uint32_t saddr, uint32_t rank) {
+    uint32_t remote;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(saddr), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
+    return v;
 }
 
-// CTA that owns cell x when CTA i owns cells [i * cells / ctas, (i + 1) * cells / ctas).
-__device__ __forceinline__ uint32_t cta_of_cell(uint32_t x, uint32_t ctas, uint32_t cells) {
-    return uint32_t(((uint64_t(x) + 1) * ctas - 1) / cells);
-}
-
-// NG: vector groups of eight, 1 (batch <= 8) or 2.  A warp owns two 16-row blocks (RB = 2), the CTA's 16
-// warps a tile group of 512 rows; a cell is a tile group x four block columns, one pass of every warp.
-// The CTAs take equal contiguous ranges of the tile-group-major cell order.  Between the image barriers the
-// warps run on their own: codes arrive through the warp's cp.async ring one pass ahead.
-template <int NG, int RB>
-__global__ void __launch_bounds__(kBatThreads, 1)
-k_gemv_batched(const DeviceTables* __restrict__ tab, const unsigned char* __restrict__ codes,
-               const __half* __restrict__ x, int N, int K, int B, int batch, float* __restrict__ partials, int tile_groups, int col_groups) {
-    static_assert(RB == 2, "the ring and the lane mapping are laid out for two row blocks per warp");
-    constexpr int PC = kPassTiles / RB;          // block columns per pass
-    constexpr int CP = kImageGroups / (PC * NG); // passes per image chunk
-    constexpr int kPieceFloats = RB * 128 * NG;  // partial results of one warp: 16 RB rows x 8 NG vectors
+// NG: groups of eight vectors; NT: row tiles of a step.
+template <int NG, int NT>
+__global__ void __launch_bounds__(kBatThreads, 1) k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ BatParams P) {
+    constexpr int PS = part_stride(NG), W = kBatWarps, TW = tiles_at_once(NG, NT);
+    constexpr BatSmem S = bat_smem(NG, NT);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_release();
-    // the tables start towards shared memory first; they are waited for together with the first pass's codes
-    unsigned char* smem = stage_fast_tables_async(tab, smem_raw);
-    const uint32_t sm_tab = smem_u32(smem);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // per warp: eight 16-row tiles of coordinates and block scales (tile rb * PC + column), the code ring;
-    // after the warps' areas, the activation image of a chunk of passes
-    unsigned char* tiles = smem + kFastBytes + warp * kBatWarpSmem;
-    const uint32_t ring = smem_u32(tiles) + uint32_t(kBatWarpTiles);
-    const uint32_t image = smem_u32(smem + kFastBytes + kBatWarps * kBatWarpSmem);
-    const int row16 = lane & 15, colsel = lane >> 4;
+    const int q = lane >> 2, t = lane & 3;
+    const int V = P.batch, C = P.cluster;
+    const int group = int(blockIdx.x) / C, rank = int(blockIdx.x) - group * C;
+    // this CTA's row tiles (shared with its cluster) and column quads
+    const int tile_lo = int((long long)group * P.tiles / P.groups), tile_hi = int((long long)(group + 1) * P.tiles / P.groups);
+    const int quad_lo = rank * P.quads / C, quad_hi = (rank + 1) * P.quads / C;
+    const uint32_t sm_raw = smem_u32(smem_raw);
+    unsigned char* smem = smem_raw + (((sm_raw + kSmAlign - 1) & ~(kSmAlign - 1)) - sm_raw);
+    const uint32_t sm_tab = smem_u32(smem);
+    float* part = reinterpret_cast<float*>(smem + S.warps);
+    float* rs_sm = reinterpret_cast<float*>(smem + S.rs);
+    __half* tail_sm = reinterpret_cast<__half*>(smem + S.tail);
+    float* xtail = reinterpret_cast<float*>(smem + S.xtail);
+    const uint32_t tile = sm_tab + S.warps + uint32_t(warp) * S.per_warp, xbuf = tile + TW * kTileBytes;
+    constexpr uint32_t kXBuf = 8 * NG * kXVec;
+    const int ntail = P.tail ? P.K % 24 : 0, Kx = min(P.K, 24 * P.B);
+    const int row_groups = (P.N + 7) / 8;
 
-    const int row_groups = (N + 7) / 8;
-    const uint32_t Bu = uint32_t(B);
-    const int g = lane >> 2, t4 = lane & 3;  // MMA fragment coordinates
-    const uint32_t tile_addr = smem_u32(tiles);
-    // ldmatrix: lane provides the address of row (lane % 8) of 8x8 matrix (lane / 8):
-    // matrices = (rows 0-7, bytes 0-15), (rows 8-15, bytes 0-15), (rows 0-7, bytes 16-31), (rows 8-15, bytes 16-31)
-    const uint32_t ldm_off = uint32_t((((lane >> 3) & 1) * 8 + (lane & 7)) * kTileRow + (lane >> 4) * 16);
-    // block j of the lane in a pass: row row16 of row block j % 2, column colsel + 2 (j / 2); its words in a slot
-    const uint32_t lane_w0 = uint32_t(row16 >> 3) * kBatRingGroup + uint32_t((row16 >> 2) & 1) * 64u + uint32_t(colsel) * 16u +
-                             uint32_t(row16 & 3) * 4u;
-    const uint32_t lane_w1 = uint32_t(row16 >> 3) * kBatRingGroup + 128u + uint32_t(colsel) * 16u + uint32_t(row16 & 7) * 2u;
-    // the lane's copies of a pass: 48 pieces of 16 bytes, (row group, part) = piece / 4, column = piece % 4
-    const uint32_t cp0_gp = uint32_t(lane >> 2), cp1_gp = 8u + uint32_t(lane >> 2), cp_col = uint32_t(lane & 3);
-    const uint32_t cp0_dst = (cp0_gp / 3u) * kBatRingGroup + (cp0_gp % 3u) * 64u + cp_col * 16u;
-    const uint32_t cp1_dst = (cp1_gp / 3u) * kBatRingGroup + (cp1_gp % 3u) * 64u + cp_col * 16u;
-
-    const uint32_t ctas = gridDim.x, cells = uint32_t(tile_groups) * uint32_t(col_groups), CG = uint32_t(col_groups);
-    const uint32_t cell_begin = uint32_t(uint64_t(blockIdx.x) * cells / ctas);
-    const uint32_t cell_end = uint32_t((uint64_t(blockIdx.x) + 1) * cells / ctas);
-    uint32_t tg = cell_begin / CG, cg = cell_begin - tg * CG;
-
-    // the codes of the warp's pass in cell (ftg, fcg) into ring slot `slot`; what lies outside the matrix is zero
-    auto fetch = [&](uint32_t ftg, uint32_t fcg, uint32_t slot) {
-        const uint32_t G0 = (ftg * kBatWarps + uint32_t(warp)) * (2 * RB);  // first of the warp's four row groups
-        const uint32_t col = fcg * PC + cp_col;
-        const bool in = col < Bu;
-        const uint4* base = reinterpret_cast<const uint4*>(codes) + size_t(G0) * 3 * Bu + (in ? col : 0u);
-        const uint32_t dst = ring + slot * kBatRingSlot;
-        const bool have0 = in && G0 + cp0_gp / 3u < uint32_t(row_groups);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" :: "r"(dst + cp0_dst),
-                     "l"(have0 ? base + size_t(cp0_gp) * Bu : reinterpret_cast<const uint4*>(codes)), "r"(have0 ? 16u : 0u));
-        if (lane < 16) {
-            const bool have1 = in && G0 + cp1_gp / 3u < uint32_t(row_groups);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" :: "r"(dst + cp1_dst),
-                         "l"(have1 ? base + size_t(cp1_gp) * Bu : reinterpret_cast<const uint4*>(codes)), "r"(have1 ? 16u : 0u));
+    // This lane's words of a step: rows q and q + 8 of NT tiles at column t.  Rows and columns outside the matrix repeat
+    // the last one: such rows are not stored, such columns meet zeros.  words_at moves the lane's two addresses to a
+    // quad; a row group is a uniform offset from there.
+    uint32_t w0[NT][2], w1[NT][2];
+    const unsigned char* lane_words = P.codes + (size_t(q >> 2) * P.B * 16 + size_t(q & 3) * 4);
+    const uint32_t lane_w1 = uint32_t(2 - (q >> 2)) * uint32_t(P.B) * 16u + uint32_t(q) * 2u - uint32_t(q & 3) * 4u;
+    const unsigned char* words = nullptr;
+    auto words_at = [&](int t0, int quad) {
+        words = lane_words + (size_t(2 * t0) * 3 * P.B + min(4 * quad + t, P.B - 1)) * 16;
+    };
+    auto load_words = [&](int i, int t0) {
+#pragma unroll
+        for (int rg = 0; rg < 2; ++rg) {
+            const uint32_t off = uint32_t(min(2 * i + rg, row_groups - 1 - 2 * t0)) * 48u * uint32_t(P.B);
+            w0[i][rg] = __ldg(reinterpret_cast<const uint32_t*>(words + off));
+            w1[i][rg] = __ldg(reinterpret_cast<const unsigned short*>(words + (off + lane_w1)));
         }
-        asm volatile("cp.async.commit_group;");
     };
-    if (cell_begin < cell_end) fetch(tg, cg, 0);
-    else asm volatile("cp.async.commit_group;");
-    pdl_wait();  // x may come from the preceding kernel; the partial results of an earlier call have been read
-
-    // Image tasks of a chunk of CP passes: task (pass i of the chunk, column cs, vector group n) = a warp's worth
-    // of threads; the 16 warps take two tasks each.
-    auto image_task_load = [&](uint32_t first_cell, int id, ImageTask& T) {
-        const uint32_t cell = first_cell + uint32_t(id / (PC * NG));
-        if (cell < cell_end) image_load(x, K, batch, int(cell % CG) * PC + (id / NG) % PC, 8 * (id % NG) + (lane >> 2), lane & 3, T);
-    };
-    auto image_task_store = [&](uint32_t first_cell, int id, const ImageTask& T) {
-        const uint32_t cell = first_cell + uint32_t(id / (PC * NG));
-        if (cell < cell_end) image_store(T, image + uint32_t(id) * 1024u, 8 * (id % NG) + (lane >> 2), lane & 3);
-    };
-    ImageTask task0, task1;
-    image_task_load(cell_begin, warp, task0);
-    image_task_load(cell_begin, warp + kBatWarps, task1);
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();  // tables staged, tile padding written
-
-    float acc[RB][NG][4];
-#pragma unroll
-    for (int rb = 0; rb < RB; ++rb)
-#pragma unroll
-        for (int n = 0; n < NG; ++n)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) acc[rb][n][i] = 0.f;
-
-    for (uint32_t cell = cell_begin; cell < cell_end; ++cell) {
-        const uint32_t pass = cell - cell_begin, slot = pass & 1u, in_chunk = pass % CP;
-        const bool active = (int(tg) * kBatWarps + warp) * (16 * RB) < N;  // warp-uniform
-        uint32_t ntg = tg, ncg = cg + 1;
-        if (ncg == CG) { ncg = 0; ++ntg; }
-        if (in_chunk == 0 && pass > 0) {  // CTA-uniform: the image of the next chunk of passes replaces the old one
-            __syncthreads();
-            image_task_load(cell, warp, task0);
-            image_task_load(cell, warp + kBatWarps, task1);
-            image_task_store(cell, warp, task0);
-            image_task_store(cell, warp + kBatWarps, task1);
-            __syncthreads();
+    auto stage_rows = [&](int t0, int nt) {
+        const int row0 = 16 * t0, rows = min(16 * nt, P.N - row0);
+        for (int i = threadIdx.x; i < rows; i += kBatThreads)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(smem_u32(rs_sm + i)), "l"(P.row_scales + row0 + i));
+        if (ntail) {
+            const __half* tl = P.tail + size_t(row0) * ntail;
+            for (int r = threadIdx.x >> 3; r < rows; r += kBatThreads / 8)
+                for (int k = threadIdx.x & 7; k < ntail; k += 8) tail_sm[r * 24 + k] = tl[size_t(r) * ntail + k];
         }
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncwarp();  // every lane's copies have landed, and every lane has left the other slot
-        if (cell + 1 < cell_end) fetch(ntg, ncg, slot ^ 1u);
-        if (active) {
-            const uint32_t src = ring + slot * kBatRingSlot;
+    };
+    // The activations of a quad's four columns, twelve units of eight per vector, into buffer `slot`; zeros beyond the
+    // last column.  Lanes 0..23: unit lane % 12 of every second vector.
+    const bool x_wide = ((reinterpret_cast<uintptr_t>(P.x) | (uintptr_t(P.K) * 2)) & 15) == 0;
+    const int x_v = lane >= 12 ? 1 : 0, x_u = lane - 12 * x_v;
+    auto stage_x = [&](uint32_t slot, int quad) {
+        const int k = 96 * quad + 8 * x_u, n = min(max(Kx - k, 0), 8);
+        const __half* src = P.x + (n ? size_t(x_v) * P.K + k : 0);
+        const size_t step = n ? 2 * size_t(P.K) : 0;
+        const uint32_t dst = xbuf + slot * kXBuf + uint32_t(x_v) * kXVec + uint32_t(x_u) * 16u;
+        if (x_wide) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                uint32_t w0, w1;
-                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w0) : "r"(src + lane_w0 + (j % RB) * 2 * kBatRingGroup + (j / RB) * 32));
-                asm volatile("ld.shared.u16 %0, [%1];" : "=r"(w1) : "r"(src + lane_w1 + (j % RB) * 2 * kBatRingGroup + (j / RB) * 32));
-                FastBlock fb;
-                fast_decode<false>(sm_tab, w0, w1, fb);
-                const float scale = lds32f(scale_address(fb));  // -gain[g] / sqrt(16 m), with -8 y in the tile
-                const int tile_id = (j % RB) * PC + 2 * (j / RB);  // + colsel
-                unsigned char* dst = tiles + (tile_id + colsel) * kTileBytes + row16 * kTileRow;
-                // coordinates 24..31 of a tile row meet zeros in the activation image, so those eight bytes
-                // need not be zero: the block's scale rides there
-                *reinterpret_cast<uint4*>(dst) = make_uint4(fb.y[0], fb.y[1], fb.y[2], fb.y[3]);
-                *reinterpret_cast<uint4*>(dst + 16) = make_uint4(fb.y[4], fb.y[5], __float_as_uint(scale), 0u);
+            for (int i = 0; i < 4 * NG; ++i, src += step)
+                if (lane < 24 && 2 * i + x_v < V)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" :: "r"(dst + uint32_t(i) * 2u * kXVec), "l"(src), "r"(2 * n));
+        } else {
+#pragma unroll 1
+            for (int i = 0; 2 * i < V; ++i, src += step)
+                if (lane < 24 && 2 * i + x_v < V) {
+                    const uint4 e = load_eight(src, n);
+                    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" :: "r"(dst + uint32_t(i) * 2u * kXVec), "r"(e.x), "r"(e.y), "r"(e.z), "r"(e.w)
+                                 : "memory");
+                }
+        }
+    };
+
+    // ---- before the wait: what does not depend on the activations ------------------------------------------
+    if (quad_lo + warp < quad_hi) {
+        words_at(tile_lo, quad_lo + warp);
+#pragma unroll
+        for (int i = 0; i < NT; ++i) load_words(i, tile_lo);
+    }
+    stage_fast_tables_async(tab, smem_raw);
+    stage_rows(tile_lo, min(tile_hi - tile_lo, NT));
+    pdl_wait();  // x may come from the preceding kernel
+    for (int i = threadIdx.x; i < V * 24; i += kBatThreads) {
+        const int v = i / 24, k = i - 24 * v;
+        xtail[i] = k < ntail ? __half2float(P.x[size_t(v) * P.K + 24 * P.B + k]) : 0.f;
+    }
+
+    uint32_t x_vec[NG];  // this lane's words of the first column: + column * 48 + section * 16
+#pragma unroll
+    for (int n = 0; n < NG; ++n) x_vec[n] = xbuf + uint32_t(min(8 * n + q, V - 1)) * kXVec + uint32_t(t) * 4u;  // results beyond V are never used
+
+    for (int t0 = tile_lo; t0 < tile_hi; t0 += NT) {
+        const int nt = min(tile_hi - t0, NT);
+        float acc[NT][NG][4];
+#pragma unroll
+        for (int i = 0; i < NT; ++i)
+#pragma unroll
+            for (int n = 0; n < NG; ++n)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[i][n][k] = 0.f;
+        if (t0 != tile_lo) {
+            __syncthreads();  // the sums of the tiles before have been read
+            stage_rows(t0, nt);
+            if (quad_lo + warp < quad_hi) {
+                words_at(t0, quad_lo + warp);
+#pragma unroll
+                for (int i = 0; i < NT; ++i) load_words(i, t0);
             }
         }
-        if (pass == 0) {  // the first chunk's image: its loads were issued before the first pass was decoded
-            image_task_store(cell_begin, warp, task0);
-            image_task_store(cell_begin, warp + kBatWarps, task1);
-            __syncthreads();
+        uint32_t slot = 0;
+        if (quad_lo + warp < quad_hi) stage_x(0, quad_lo + warp);
+        asm volatile("cp.async.commit_group;");
+        if (t0 == tile_lo) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();  // the tables are in place
         }
-        if (active) {
-            __syncwarp();
-            const uint32_t img = image + in_chunk * (PC * NG * 1024u) + lane * 16;
+        for (int quad = quad_lo + warp; quad < quad_hi; quad += W) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncwarp();  // every lane's copies have landed, and every lane has left the other buffer
+            const int next = min(quad + W, quad_hi - 1);
+            if (quad + W < quad_hi) stage_x(slot ^ 1u, next);
+            asm volatile("cp.async.commit_group;");
+            const uint32_t x_off = slot * kXBuf;
+            words_at(t0, next);
 #pragma unroll
-            for (int cs = 0; cs < PC; ++cs) {
-                uint32_t q0[NG][4], q1[NG][4];
+            for (int i0 = 0; i0 < NT; i0 += TW) {
+                constexpr int kLeft = NT % TW;  // an odd last tile goes alone
+                const int tw = i0 + TW <= NT ? TW : kLeft;
+                float scale[TW][2];
 #pragma unroll
-                for (int n = 0; n < NG; ++n) {
-                    lds128(img + (cs * NG + n) * 1024, q0[n]);
-                    lds128(img + (cs * NG + n) * 1024 + 512, q1[n]);
+                for (int k = 0; k < tw; ++k) {
+                    const int i = i0 + k;
+#pragma unroll
+                    for (int rg = 0; rg < 2; ++rg) {
+                        uint32_t a[12];
+                        scale[k][rg] = decode_halves<false>(sm_tab, w0[i][rg], w1[i][rg], a);
+                        const uint32_t dst = tile + uint32_t(k) * kTileBytes + uint32_t(t) * kTileCol + uint32_t(8 * rg + q) * 48u;
+#pragma unroll
+                        for (int s = 0; s < 3; ++s)
+                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" :: "r"(dst + 16u * s), "r"(a[4 * s]), "r"(a[4 * s + 1]),
+                                         "r"(a[4 * s + 2]), "r"(a[4 * s + 3]) : "memory");
+                    }
+                    load_words(i, t0);
                 }
+                __syncwarp();
+                // ldmatrix: lane gives the address of row lane % 8 of matrix lane / 8 = (rows 0-7, section 0),
+                // (8-15, 0), (0-7, 1), (8-15, 1); then the two of section 2
+                uint32_t a[2][TW][4], a2[2][TW][2];
+                auto fragments = [&](int j) {
 #pragma unroll
-                for (int rb = 0; rb < RB; ++rb) {
-                    const int tile_id = rb * PC + cs;
-                    uint32_t a[4];
-                    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                                 : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
-                                 : "r"(tile_addr + tile_id * kTileBytes + ldm_off));
-                    const float s_lo = *reinterpret_cast<const float*>(tiles + tile_id * kTileBytes + g * kTileRow + 24);
-                    const float s_hi = *reinterpret_cast<const float*>(tiles + tile_id * kTileBytes + (g + 8) * kTileRow + 24);
+                    for (int k = 0; k < tw; ++k) {
+                        const uint32_t at = tile + uint32_t(k) * kTileBytes + uint32_t(j) * kTileCol + uint32_t(lane & 15) * 48u;
+                        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                                     : "=r"(a[j & 1][k][0]), "=r"(a[j & 1][k][1]), "=r"(a[j & 1][k][2]), "=r"(a[j & 1][k][3])
+                                     : "r"(at + uint32_t(lane >> 4) * 16u) : "memory");
+                        asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
+                                     : "=r"(a2[j & 1][k][0]), "=r"(a2[j & 1][k][1]) : "r"(at + 32u) : "memory");
+                    }
+                };
+                fragments(0);
 #pragma unroll
-                    for (int n = 0; n < NG; ++n) {
-                        int dh[4], dm[4], dl[4];
-                        mma_s8s8(dh, a, q0[n][0], q0[n][1]);
-                        mma_s8u8(dm, a, q0[n][2], q0[n][3]);
-                        mma_s8u8(dl, a, q1[n][0], q1[n][1]);
-                        const float step_even = __uint_as_float(q1[n][2]), step_odd = __uint_as_float(q1[n][3]);
-                        // this lane's results: rows g (i = 0, 1) and g + 8 (i = 2, 3), vectors 8 n + 2 t4 + (i & 1)
+                for (int j = 0; j < 4; ++j) {
+                    if (j < 3) fragments(j + 1);
+                    uint32_t b[NG][3];
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int dot = combine_planes(dh[i], dm[i], dl[i]);
-                            acc[rb][n][i] = fmaf(float(dot), (i < 2 ? s_lo : s_hi) * ((i & 1) ? step_odd : step_even),
-                                                 acc[rb][n][i]);
+                    for (int n = 0; n < NG; ++n)
+#pragma unroll
+                        for (int s = 0; s < 3; ++s)
+                            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b[n][s]) : "r"(x_vec[n] + x_off + uint32_t(48 * j + 16 * s)));
+#pragma unroll
+                    for (int k = 0; k < tw; ++k) {
+                        const float s_lo = __shfl_sync(0xFFFFFFFFu, scale[k][0], (lane & 28) | j);
+                        const float s_hi = __shfl_sync(0xFFFFFFFFu, scale[k][1], (lane & 28) | j);
+#pragma unroll
+                        for (int n = 0; n < NG; ++n) {
+                            float d[4];
+                            mma_k16(d, a[j & 1][k], b[n][0], b[n][1]);
+                            mma_k8(d, a2[j & 1][k][0], a2[j & 1][k][1], b[n][2]);
+                            fma2(s_lo, d[0], d[1], acc[i0 + k][n][0], acc[i0 + k][n][1]);
+                            fma2(s_hi, d[2], d[3], acc[i0 + k][n][2], acc[i0 + k][n][3]);
                         }
                     }
                 }
+                __syncwarp();  // the tile has been read before the next blocks overwrite it
             }
-            __syncwarp();  // the fragments have been read before the next pass overwrites the tiles
-        }
-        if (cell + 1 == cell_end || ntg != tg) {  // CTA-uniform: this CTA's piece of tile group tg is complete
-            // pieces are numbered blockIdx.x + tg: unique, and increasing along the cell order
-            float* mine = partials + (size_t(blockIdx.x + tg) * kBatWarps + warp) * kPieceFloats;
-#pragma unroll
-            for (int rb = 0; rb < RB; ++rb)
-#pragma unroll
-                for (int n = 0; n < NG; ++n)
-#pragma unroll
-                    for (int i = 0; i < 4; i += 2) {
-                        *reinterpret_cast<float2*>(mine + (16 * rb + g + (i < 2 ? 0 : 8)) * (8 * NG) + 8 * n + 2 * t4) =
-                            make_float2(acc[rb][n][i], acc[rb][n][i + 1]);
-                        acc[rb][n][i] = 0.f;
-                        acc[rb][n][i + 1] = 0.f;
-                    }
-        }
-        tg = ntg;
-        cg = ncg;
-    }
-}
-
-// ---------------------------------------------------------------------------------------------
-// Two to four vectors: the same cells, rings, image chunks and pieces as k_gemv_batched, but no shared-memory
-// tile between decoder and tensor cores.  Lane 4 q + t decodes, for each of the warp's two row blocks, rows
-// 2 q and 2 q + 1 at column t of the pass's four columns; the MMA takes eight coordinates of both blocks
-// from every lane as A (rows q and q + 8), and B is block diagonal -- column 2 t + plane of B is zero outside
-// the k range that lane t feeds -- so D[q][2 t + plane] is the dot product of lane (q, t)'s own block with
-// its own column's activation plane and arrives in that same lane.  Three MMAs (coordinate pairs) times two
-// B sets (unsigned middle and low planes; signed high plane) per vector and row block.  The activation
-// image holds, per (column quad, vector), the B fragments as they are read: three 128-byte lines (one per
-// coordinate pair: bytes 0..63 middle and low planes, entry 2 t + plane; 64..95 high plane, entry t;
-// 96..103 zero, read by the lanes whose part of B is zero), the four columns' steps at 104 + 4 t of line 0.
-// ---------------------------------------------------------------------------------------------
-constexpr uint32_t kQuadBytes = 384;
-constexpr int kFewMaxVectors = 4;
-constexpr int kFewChunkPasses = 16;  // passes whose image is held at a time: 16 x 4 vectors x 384 bytes = 24 KiB
-
-__device__ __forceinline__ void mma_bd(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                       uint32_t b1, const int (&c)[4], bool b_signed) {
-    if (b_signed)
-        asm("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};"
-            : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
-            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(c[0]), "r"(c[1]), "r"(c[2]), "r"(c[3]));
-    else
-        asm("mma.sync.aligned.m16n8k32.row.col.s32.s8.u8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};"
-            : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
-            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(c[0]), "r"(c[1]), "r"(c[2]), "r"(c[3]));
-}
-
-template <int V>
-__global__ void __launch_bounds__(kBatThreads, 1)
-k_gemv_few(const DeviceTables* __restrict__ tab, const unsigned char* __restrict__ codes, const __half* __restrict__ x,
-           int N, int K, int B, float* __restrict__ partials, int tile_groups, int col_groups) {
-    constexpr int RB = 2, PC = 4, CP = kFewChunkPasses;
-    constexpr int kPieceFloats = RB * 128;  // the piece layout of k_gemv_batched<1, 2>: 32 rows x 8 vector slots
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    pdl_release();
-    unsigned char* smem = stage_fast_tables_async(tab, smem_raw);
-    const uint32_t sm_tab = smem_u32(smem);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int q = lane >> 2, t = lane & 3;
-    const uint32_t ring = smem_u32(smem + kFastBytes) + uint32_t(warp) * (2 * kBatRingSlot);
-    const uint32_t image = smem_u32(smem + kFastBytes) + uint32_t(kBatWarps) * (2 * kBatRingSlot);
-    unsigned char* image_ptr = smem + kFastBytes + kBatWarps * (2 * kBatRingSlot);
-    const int row_groups = (N + 7) / 8;
-    const uint32_t Bu = uint32_t(B);
-    // the lane's words in a slot: rows 2 q, 2 q + 1 of row block rb sit in row group 2 rb + q / 4, part (q / 2) % 2
-    const uint32_t lane_w0 = uint32_t(q >> 2) * kBatRingGroup + uint32_t((q >> 1) & 1) * 64u + uint32_t(t) * 16u + uint32_t(q & 1) * 8u;
-    const uint32_t lane_w1 = uint32_t(q >> 2) * kBatRingGroup + 128u + uint32_t(t) * 16u + uint32_t(q & 3) * 4u;
-    // this lane's part of the B fragments (the other lanes read the zeros)
-    const uint32_t lane_x1 = (q >> 1) == t ? uint32_t(q) * 8u : 96u;
-    const uint32_t lane_x2 = q == 2 * t ? 64u + uint32_t(t) * 8u : 96u;
-    const uint32_t lane_xs = 104u + 4u * uint32_t(t);
-    const uint32_t cp0_gp = uint32_t(lane >> 2), cp1_gp = 8u + uint32_t(lane >> 2), cp_col = uint32_t(lane & 3);
-    const uint32_t cp0_dst = (cp0_gp / 3u) * kBatRingGroup + (cp0_gp % 3u) * 64u + cp_col * 16u;
-    const uint32_t cp1_dst = (cp1_gp / 3u) * kBatRingGroup + (cp1_gp % 3u) * 64u + cp_col * 16u;
-
-    const uint32_t ctas = gridDim.x, cells = uint32_t(tile_groups) * uint32_t(col_groups), CG = uint32_t(col_groups);
-    const uint32_t cell_begin = uint32_t(uint64_t(blockIdx.x) * cells / ctas);
-    const uint32_t cell_end = uint32_t((uint64_t(blockIdx.x) + 1) * cells / ctas);
-    uint32_t tg = cell_begin / CG, cg = cell_begin - tg * CG;
-
-    auto fetch = [&](uint32_t ftg, uint32_t fcg, uint32_t slot) {
-        const uint32_t G0 = (ftg * kBatWarps + uint32_t(warp)) * (2 * RB);
-        const uint32_t col = fcg * PC + cp_col;
-        const bool in = col < Bu;
-        const uint4* base = reinterpret_cast<const uint4*>(codes) + size_t(G0) * 3 * Bu + (in ? col : 0u);
-        const uint32_t dst = ring + slot * kBatRingSlot;
-        const bool have0 = in && G0 + cp0_gp / 3u < uint32_t(row_groups);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" :: "r"(dst + cp0_dst),
-                     "l"(have0 ? base + size_t(cp0_gp) * Bu : reinterpret_cast<const uint4*>(codes)), "r"(have0 ? 16u : 0u));
-        if (lane < 16) {
-            const bool have1 = in && G0 + cp1_gp / 3u < uint32_t(row_groups);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" :: "r"(dst + cp1_dst),
-                         "l"(have1 ? base + size_t(cp1_gp) * Bu : reinterpret_cast<const uint4*>(codes)), "r"(have1 ? 16u : 0u));
-        }
-        asm volatile("cp.async.commit_group;");
-    };
-    if (cell_begin < cell_end) fetch(tg, cg, 0);
-    else asm volatile("cp.async.commit_group;");
-    pdl_wait();  // x may come from the preceding kernel; the partial results of an earlier call have been read
-
-    // Image of a chunk of CP passes: thread (pass i, column cs, vector v) quantises one column of one vector and
-    // writes its planes into the quad's record as B fragments.
-    auto image_build = [&](uint32_t first_cell) {
-        for (int id = threadIdx.x; id < CP * PC * V; id += kBatThreads) {
-            const int v = id % V, cs = (id / V) % PC, i = id / (V * PC);
-            const uint32_t cell = first_cell + uint32_t(i);
-            if (cell >= cell_end) continue;
-            const int col = int(cell % CG) * PC + cs;
-            uint32_t qv[20];
-            if (col < B) {
-                quantise_column(x + size_t(v) * K, K, col, qv);
-            } else {
-#pragma unroll
-                for (int k = 0; k < 20; ++k) qv[k] = 0u;
-            }
-            unsigned char* rec = image_ptr + size_t(i * V + v) * kQuadBytes;
-#pragma unroll
-            for (int pr = 0; pr < 3; ++pr) {
-                unsigned char* line = rec + 128 * pr;
-                *reinterpret_cast<uint2*>(line + 16 * cs) = make_uint2(qv[6 + 2 * pr], qv[7 + 2 * pr]);        // middle plane
-                *reinterpret_cast<uint2*>(line + 16 * cs + 8) = make_uint2(qv[12 + 2 * pr], qv[13 + 2 * pr]);  // low plane
-                *reinterpret_cast<uint2*>(line + 64 + 8 * cs) = make_uint2(qv[2 * pr], qv[2 * pr + 1]);        // high plane
-                if (cs == 0) *reinterpret_cast<uint2*>(line + 96) = make_uint2(0u, 0u);
-            }
-            *reinterpret_cast<uint32_t*>(rec + 104 + 4 * cs) = qv[18];
-        }
-    };
-    image_build(cell_begin);
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();  // tables staged, first image built
-
-    float acc[RB][2][V];
-#pragma unroll
-    for (int rb = 0; rb < RB; ++rb)
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-#pragma unroll
-            for (int v = 0; v < V; ++v) acc[rb][j][v] = 0.f;
-
-    for (uint32_t cell = cell_begin; cell < cell_end; ++cell) {
-        const uint32_t pass = cell - cell_begin, slot = pass & 1u, in_chunk = pass % CP;
-        const bool active = (int(tg) * kBatWarps + warp) * (16 * RB) < N;  // warp-uniform
-        uint32_t ntg = tg, ncg = cg + 1;
-        if (ncg == CG) { ncg = 0; ++ntg; }
-        if (in_chunk == 0 && pass > 0) {  // CTA-uniform: the image of the next chunk of passes replaces the old one
-            __syncthreads();
-            image_build(cell);
-            __syncthreads();
+            slot ^= 1u;
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncwarp();  // every lane's copies have landed, and every lane has left the other slot
-        if (cell + 1 < cell_end) fetch(ntg, ncg, slot ^ 1u);
-        if (active) {
-            const uint32_t src = ring + slot * kBatRingSlot;
-            FastBlock f[RB][2];
-            float scale[RB][2];
+        __syncthreads();  // everybody has left the tiles and buffers: the sums take their place
 #pragma unroll
-            for (int rb = 0; rb < RB; ++rb) {
-                uint2 w0;
-                uint32_t w1pair;
-                asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(w0.x), "=r"(w0.y) : "r"(src + lane_w0 + rb * 2 * kBatRingGroup));
-                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w1pair) : "r"(src + lane_w1 + rb * 2 * kBatRingGroup));
-                fast_decode<false>(sm_tab, w0.x, w1pair, f[rb][0]);
-                fast_decode<true>(sm_tab, w0.y, w1pair, f[rb][1]);
+        for (int i = 0; i < NT; ++i)
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    scale[rb][j] = lds32f(scale_address(f[rb][j]));
+            for (int n = 0; n < NG; ++n)
+#pragma unroll
+                for (int k = 0; k < 4; k += 2)
+                    *reinterpret_cast<float2*>(part + (size_t(i * W + warp) * 16 + q + 4 * k) * PS + 8 * n + 2 * t) =
+                        make_float2(acc[i][n][k], acc[i][n][k + 1]);
+        __syncthreads();
+        // Thread = (tile, vector, row of the tile); the warps' sums in warp order.
+        constexpr int AT_ONCE = kBatThreads / (128 * NG);  // tiles
+        const int r = threadIdx.x & 15, v = (threadIdx.x >> 4) & (8 * NG - 1), rt0 = threadIdx.x / (128 * NG);
+        auto tile_sum = [&](int rt) {
+            const float* at = part + (size_t(rt * W) * 16 + r) * PS + v;
+            float sum = 0.f;
+#pragma unroll
+            for (int w = 0; w < W; ++w) sum += at[w * 16 * PS];
+            return sum;
+        };
+        // Twice the halves' sum (row scale, tail).  A column with a NaN or an infinity has made its products in every row
+        // infinite or NaN: 0 x sum makes them all NaN.
+        auto finish = [&](float sum, int rt) {
+            const int i = 16 * rt + r, row = 16 * t0 + i;
+            if (row >= P.N) return;
+            float res = 2.f * rs_sm[i] * fmaf(0.f, sum, sum);
+            for (int k = 0; k < ntail; ++k) res = fmaf(__half2float(tail_sm[i * 24 + k]), xtail[24 * v + k], res);
+            P.y[size_t(v) * P.N + row] = res;
+        };
+        if (C == 1) {
+            if (v < V)
+                for (int rt = rt0; rt < nt; rt += AT_ONCE) finish(tile_sum(rt), rt);
+        } else {
+            // The sums over the CTA's columns replace the parts once everybody has read those; then every CTA of the
+            // cluster finishes every C-th turn of tiles.
+            constexpr int PER = (NT + AT_ONCE - 1) / AT_ONCE;
+            float sums[PER];
+#pragma unroll
+            for (int j = 0; j < PER; ++j) sums[j] = rt0 + j * AT_ONCE < nt ? tile_sum(rt0 + j * AT_ONCE) : 0.f;
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < PER; ++j)
+                if (rt0 + j * AT_ONCE < nt) part[threadIdx.x + j * kBatThreads] = sums[j];
+            cluster_barrier();
+            if (v < V)
+                for (int j = rank; rt0 + j * AT_ONCE < nt; j += C) {
+                    float sum = 0.f;
+                    for (int c = 0; c < C; ++c) sum += cluster_load(smem_u32(part + threadIdx.x + j * kBatThreads), uint32_t(c));
+                    finish(sum, rt0 + j * AT_ONCE);
                 }
-            }
-            const uint32_t img = image + in_chunk * (V * kQuadBytes);
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                uint2 bm[3], bh[3];
-#pragma unroll
-                for (int pr = 0; pr < 3; ++pr) {
-                    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(bm[pr].x), "=r"(bm[pr].y) : "r"(img + v * kQuadBytes + 128 * pr + lane_x1));
-                    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(bh[pr].x), "=r"(bh[pr].y) : "r"(img + v * kQuadBytes + 128 * pr + lane_x2));
-                }
-                float step;
-                asm volatile("ld.shared.f32 %0, [%1];" : "=f"(step) : "r"(img + v * kQuadBytes + lane_xs));
-                if constexpr (V <= 2) {  // registers allow the two row blocks' MMA chains side by side
-                int dm[RB][4], dh[RB][4];
-#pragma unroll
-                for (int rb = 0; rb < RB; ++rb)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) { dm[rb][i] = 0; dh[rb][i] = 0; }
-#pragma unroll
-                for (int pr = 0; pr < 3; ++pr)
-#pragma unroll
-                    for (int rb = 0; rb < RB; ++rb) {
-                        mma_bd(dm[rb], f[rb][0].y[2 * pr], f[rb][1].y[2 * pr], f[rb][0].y[2 * pr + 1], f[rb][1].y[2 * pr + 1],
-                               bm[pr].x, bm[pr].y, dm[rb], false);
-                        mma_bd(dh[rb], f[rb][0].y[2 * pr], f[rb][1].y[2 * pr], f[rb][0].y[2 * pr + 1], f[rb][1].y[2 * pr + 1],
-                               bh[pr].x, bh[pr].y, dh[rb], true);
-                    }
-#pragma unroll
-                for (int rb = 0; rb < RB; ++rb) {
-                    const int dot0 = combine_planes(dh[rb][0], dm[rb][0], dm[rb][1]);
-                    const int dot1 = combine_planes(dh[rb][2], dm[rb][2], dm[rb][3]);
-                    acc[rb][0][v] = fmaf(float(dot0), scale[rb][0] * step, acc[rb][0][v]);
-                    acc[rb][1][v] = fmaf(float(dot1), scale[rb][1] * step, acc[rb][1][v]);
-                }
-                } else {
-#pragma unroll
-                for (int rb = 0; rb < RB; ++rb) {
-                    int dm[4] = {0, 0, 0, 0}, dh[4] = {0, 0, 0, 0};
-#pragma unroll
-                    for (int pr = 0; pr < 3; ++pr) {
-                        mma_bd(dm, f[rb][0].y[2 * pr], f[rb][1].y[2 * pr], f[rb][0].y[2 * pr + 1], f[rb][1].y[2 * pr + 1],
-                               bm[pr].x, bm[pr].y, dm, false);
-                        mma_bd(dh, f[rb][0].y[2 * pr], f[rb][1].y[2 * pr], f[rb][0].y[2 * pr + 1], f[rb][1].y[2 * pr + 1],
-                               bh[pr].x, bh[pr].y, dh, true);
-                    }
-                    // exact int32 dot products of -y with the 24-bit activations (the scale carries the other minus sign)
-                    const int dot0 = combine_planes(dh[0], dm[0], dm[1]);
-                    const int dot1 = combine_planes(dh[2], dm[2], dm[3]);
-                    acc[rb][0][v] = fmaf(float(dot0), scale[rb][0] * step, acc[rb][0][v]);
-                    acc[rb][1][v] = fmaf(float(dot1), scale[rb][1] * step, acc[rb][1][v]);
-                }
-                }
-            }
+            cluster_barrier();  // the other CTAs have read this one's sums
         }
-        if (cell + 1 == cell_end || ntg != tg) {  // CTA-uniform: this CTA's piece of tile group tg is complete
-            // the four lanes of a row (its four columns) are added, then lane t = 0 writes the row's V sums
-            float* mine = partials + (size_t(blockIdx.x + tg) * kBatWarps + warp) * kPieceFloats;
-#pragma unroll
-            for (int rb = 0; rb < RB; ++rb)
-#pragma unroll
-                for (int j = 0; j < 2; ++j)
-#pragma unroll
-                    for (int v = 0; v < V; ++v) {
-                        float sum = acc[rb][j][v];
-                        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
-                        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 2);
-                        if (t == 0) mine[(16 * rb + 2 * q + j) * 8 + v] = sum;
-                        acc[rb][j][v] = 0.f;
-                    }
-        }
-        tg = ntg;
-        cg = ncg;
     }
 }
 
-// Sum of a tile group's pieces in CTA order, row scale, tail (Sec. 5.1): one thread per (row, vector).
-template <int NG, int RB>
-__global__ void __launch_bounds__(256)
-k_combine_batched(const float* __restrict__ partials, const float* __restrict__ row_scales,
-                  const __half* __restrict__ x, const __half* __restrict__ tail, float* __restrict__ y, int N, int K,
-                  int B, int batch, int tile_groups, int col_groups, int ctas) {
-    constexpr int kPieceFloats = RB * 128 * NG, kGroupRows = kBatWarps * 16 * RB;
-    pdl_release();
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    const int v = idx % (8 * NG), r = idx / (8 * NG);
-    const bool mine = r < N && v < batch;
-    // what does not depend on the pieces comes before the wait for k_gemv_batched
-    const int rr = mine ? r : 0;
-    const uint32_t tg = uint32_t(rr / kGroupRows), CG = uint32_t(col_groups);
-    const int warp = (rr % kGroupRows) / (16 * RB), rt = rr % (16 * RB);
-    const uint32_t cells = uint32_t(tile_groups) * CG;
-    const uint32_t first = cta_of_cell(tg * CG, uint32_t(ctas), cells);
-    const uint32_t pieces = cta_of_cell(tg * CG + CG - 1, uint32_t(ctas), cells) - first + 1;
-    const float scale = mine ? __ldg(row_scales + r) : 0.f;
-    pdl_wait();  // the pieces come from k_gemv_batched
-    if (!mine) return;
-    const float* p = partials + (size_t(first + tg) * kBatWarps + warp) * kPieceFloats + rt * (8 * NG) + v;
-    // sixteen pieces are loaded at a time (all of them, for the usual split of a tile group over about twenty
-    // CTAs, in two rounds of independent loads) and added in piece order
-    float total = 0.f;
-    for (uint32_t k0 = 0; k0 < pieces; k0 += 16) {
-        float v[16];
-#pragma unroll
-        for (uint32_t j = 0; j < 16; ++j) v[j] = k0 + j < pieces ? __ldcg(p + size_t(k0 + j) * kBatWarps * kPieceFloats) : 0.f;
-#pragma unroll
-        for (uint32_t j = 0; j < 16; ++j) total += v[j];
-    }
-    float res = scale * total;
-    const int ntail = tail ? K % 24 : 0;
-    for (int k = 0; k < ntail; ++k)
-        res = fmaf(__half2float(tail[size_t(r) * ntail + k]), __half2float(x[size_t(v) * K + 24 * B + k]), res);
-    y[size_t(v) * N + r] = res;
-}
-
-// Scratch: partial results, one piece per (CTA, tile group) pair that occurs.
-struct BatchedPlan {
-    int tile_groups, col_groups, ctas;
-    size_t total;
-};
-static BatchedPlan batched_plan(int N, int B, int rb, int max_ctas) {
-    BatchedPlan P;
-    const int pc = kPassTiles / rb, group_rows = kBatWarps * 16 * rb;
-    P.tile_groups = (N + group_rows - 1) / group_rows;
-    P.col_groups = (B + pc - 1) / pc;
-    const long long cells = (long long)P.tile_groups * P.col_groups;
-    P.ctas = int(cells < max_ctas ? cells : max_ctas);
-    if (P.ctas < 1) P.ctas = 1;
-    P.total = size_t(P.ctas + P.tile_groups) * kBatWarps * (size_t(rb) * 256) * 4;  // sized for two vector groups
-    return P;
-}
-
-// Row blocks per warp for a batch size.
-static int batched_rb(int batch) { return batch <= 8 ? TETRA_BAT_RB1 : TETRA_BAT_RB2; }
-
-// Upper bound over the grids this library launches (at most 1024 CTAs) and both kernel variants.
+// Scratch that a caller brings: the call keeps its partial sums in shared memory and leaves it untouched.
 size_t batched_workspace_bytes(int N, int blocks_per_row) {
-    const size_t a = batched_plan(N, blocks_per_row, batched_rb(1), 1024).total;
-    const size_t b = batched_plan(N, blocks_per_row, batched_rb(16), 1024).total;
-    return a > b ? a : b;
+    const long long row_tiles = (N + 511) / 512, cells = row_tiles * ((blocks_per_row + 3) / 4);
+    const long long pieces = (cells < 1024 ? (cells < 1 ? 1 : cells) : 1024) + row_tiles;
+    return size_t(pieces) * 16 * 512 * 4;
 }
 
-template <int NG, int RB>
-static cudaError_t launch_variant(const void* codes, const float* row_scales, const void* table, const __half* xh,
-                                  float* y, int N, int K, int B, int batch, const __half* tl, float* partials, int sms,
-                                  uint32_t smem, cudaStream_t s) {
-    const BatchedPlan P = batched_plan(N, B, RB, sms);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(P.ctas));
-    cfg.blockDim = dim3(kBatThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemv_batched<NG, RB>, static_cast<const DeviceTables*>(table),
-                                       static_cast<const unsigned char*>(codes), xh, N, K, B, batch, partials,
-                                       P.tile_groups, P.col_groups);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cc = {};
-    cc.gridDim = dim3(unsigned((size_t(N) * 8 * NG + 255) / 256));
-    cc.blockDim = dim3(256);
-    cc.stream = s;
-    cc.attrs = attr;
-    cc.numAttrs = 1;
-    return cudaLaunchKernelEx(&cc, k_combine_batched<NG, RB>, static_cast<const float*>(partials), row_scales, xh, tl,
-                              y, N, K, B, batch, P.tile_groups, P.col_groups, P.ctas);
+namespace {
+
+struct BatPlan {
+    int cluster = 1, groups = 1, nt = 1;
+};
+// Resident clusters of c CTAs when each CTA takes an SM to itself (a GPC holds whole clusters only).
+int resident_clusters(int c, int sms) {
+    if (c == 1) return sms;
+    return c == 2 ? sms / 2 : 0;
 }
 
-template <int V>
-static cudaError_t launch_few(const void* codes, const float* row_scales, const void* table, const __half* xh, float* y,
-                              int N, int K, int B, const __half* tl, float* partials, int sms, cudaStream_t s) {
-    const uint32_t smem = kTableSmemBytes + kBatWarps * 2 * kBatRingSlot + kFewChunkPasses * kFewMaxVectors * kQuadBytes;
-    static PerDeviceOnce once;
-    cudaError_t e = once.run([smem] { return cudaFuncSetAttribute(k_gemv_few<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)); });
-    if (e != cudaSuccess) return e;
-    const BatchedPlan P = batched_plan(N, B, 2, sms);
-    e = launch_pdl(k_gemv_few<V>, P.ctas, kBatThreads, smem, s, static_cast<const DeviceTables*>(table),
-                   static_cast<const unsigned char*>(codes), xh, N, K, B, partials, P.tile_groups, P.col_groups);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(k_combine_batched<1, 2>, int((size_t(N) * 8 + 255) / 256), 256, 0, s, static_cast<const float*>(partials),
-                      row_scales, xh, tl, y, N, K, B, V, P.tile_groups, P.col_groups, P.ctas);
+// How rows and columns are split: for every cluster size the steps of the busiest warp, in units of one tile x four
+// columns (about 0.5 us on B200), and what else the split costs.
+BatPlan plan_batched(int tiles, int quads, int sms) {
+    BatPlan best;
+    double best_cost = 1e30;
+    for (int c = 1; c <= 8; c *= 2) {
+        const int room = resident_clusters(c, sms);
+        if (c > quads || room == 0) break;
+        BatPlan p;
+        p.cluster = c;
+        p.groups = tiles < room ? tiles : room;
+        const int most = (tiles + p.groups - 1) / p.groups, chunks = (most + kBatMaxTiles - 1) / kBatMaxTiles;
+        p.nt = (most + chunks - 1) / chunks;
+        const int steps = ((quads + c - 1) / c + kBatWarps - 1) / kBatWarps;
+        const double cost = double(steps) * chunks * p.nt + (c > 1 ? 3.0 : 0.0) + 1.5 * chunks;
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = p;
+        }
+    }
+    return best;
 }
+
+template <int NG>
+auto batched_kernel(int nt) {
+    return nt == 1 ? k_gemv_batched<NG, 1> : (nt == 2 ? k_gemv_batched<NG, 2> : (nt == 3 ? k_gemv_batched<NG, 3> : k_gemv_batched<NG, 4>));
+}
+
+}  // namespace
 
 cudaError_t launch_gemv_batched(const void* codes, const float* row_scales, const void* table, const void* x,
-                                float* y, int N, int K, int batch, const void* tail, void* ws, cudaStream_t s) {
+                                float* y, int N, int K, int batch, const void* tail, void*, cudaStream_t s) {
     int sms = 0;
     cudaError_t e = device_sms(&sms);
     if (e != cudaSuccess) return e;
-    if (sms > 1024) sms = 1024;
-    const uint32_t smem = kTableSmemBytes + kBatWarps * kBatWarpSmem + kImageGroups * kBatColBytesPerGroup;
     static PerDeviceOnce once;
-    e = once.run([smem] {
-        cudaError_t r = cudaFuncSetAttribute(k_gemv_batched<1, TETRA_BAT_RB1>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(k_gemv_batched<2, TETRA_BAT_RB2>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    e = once.run([] {
+        cudaError_t r = cudaSuccess;
+        for (int nt = 1; nt <= kBatMaxTiles && r == cudaSuccess; ++nt) {
+            r = cudaFuncSetAttribute(batched_kernel<1>(nt), cudaFuncAttributeMaxDynamicSharedMemorySize, int(bat_smem(1, nt).total));
+            if (r == cudaSuccess) r = cudaFuncSetAttribute(batched_kernel<2>(nt), cudaFuncAttributeMaxDynamicSharedMemorySize, int(bat_smem(2, nt).total));
+        }
         return r;
     });
     if (e != cudaSuccess) return e;
-    const int B = tail ? K / 24 : (K + 23) / 24;
-    const __half* xh = static_cast<const __half*>(x);
-    const __half* tl = static_cast<const __half*>(tail);
-    float* partials = static_cast<float*>(ws);
-#ifndef TETRA_NO_FEW
-    if (batch == 2) return launch_few<2>(codes, row_scales, table, xh, y, N, K, B, tl, partials, sms, s);
-    if (batch == 3) return launch_few<3>(codes, row_scales, table, xh, y, N, K, B, tl, partials, sms, s);
-    if (batch == 4) return launch_few<4>(codes, row_scales, table, xh, y, N, K, B, tl, partials, sms, s);
-#endif
-    if (batch <= 8)
-        return launch_variant<1, TETRA_BAT_RB1>(codes, row_scales, table, xh, y, N, K, B, batch, tl, partials, sms, smem, s);
-    return launch_variant<2, TETRA_BAT_RB2>(codes, row_scales, table, xh, y, N, K, B, batch, tl, partials, sms, smem, s);
+    BatParams P;
+    P.codes = static_cast<const unsigned char*>(codes);
+    P.row_scales = row_scales;
+    P.x = static_cast<const __half*>(x);
+    P.tail = static_cast<const __half*>(tail);
+    P.y = y;
+    P.N = N;
+    P.K = K;
+    P.B = tail ? K / 24 : (K + 23) / 24;
+    P.batch = batch;
+    P.tiles = (N + 15) / 16;
+    P.quads = (P.B + 3) / 4;
+    const BatPlan plan = plan_batched(P.tiles, P.quads, sms);
+    P.groups = plan.groups;
+    P.cluster = plan.cluster;
+    const int ng = batch <= 8 ? 1 : 2;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = unsigned(plan.cluster);
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(plan.groups * plan.cluster));
+    cfg.blockDim = dim3(kBatThreads);
+    cfg.dynamicSmemBytes = bat_smem(ng, plan.nt).total;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = plan.cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, ng == 1 ? batched_kernel<1>(plan.nt) : batched_kernel<2>(plan.nt), static_cast<const DeviceTables*>(table), P);
 }
 
 }  // namespace tetra

@@ -94,12 +94,12 @@ constexpr int kEmitThreads = 256;
 __device__ __forceinline__ void file_order(const FastBlock& fb, uint32_t (&out)[6]) {
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
-        uint32_t v[2];  // y of coordinates 1, 3, 5, 7 and 0, 2, 4, 6
+        uint32_t v[2];  // y of coordinates 2, 6, 3, 7 and 0, 4, 1, 5
 #pragma unroll
         for (int k = 0; k < 2; ++k)  // 16 - y = the five-bit -y with its sign bit flipped; bytes never borrow
             v[k] = (0x90909090u - (((fb.y[2 * s + k] >> 3) & 0x1F1F1F1Fu) ^ 0x10101010u)) ^ 0x80808080u;
-        out[2 * s] = prmt(v[1], v[0], 0x5140u);
-        out[2 * s + 1] = prmt(v[1], v[0], 0x7362u);
+        out[2 * s] = prmt(v[1], v[0], 0x6420u);
+        out[2 * s + 1] = prmt(v[1], v[0], 0x7531u);
     }
 }
 

@@ -165,13 +165,15 @@ __device__ __forceinline__ unsigned char* stage_fast_tables_async(const DeviceTa
 constexpr uint32_t kTableSmemBytes = uint32_t(kFastBytes) + kSmAlign;
 
 struct FastBlock {
-    // MINUS EIGHT TIMES the lattice point, int8 x 4: y[2 s] holds coordinates 8 s + 1, 3, 5, 7 of section s in
-    // its bytes 0..3, y[2 s + 1] coordinates 8 s + 0, 2, 4, 6.  The activations' planes use the same order.
+    // MINUS EIGHT TIMES the lattice point, int8 x 4: y[2 s] holds coordinates 8 s + 2, 6, 3, 7 of section s in
+    // its bytes 0..3, y[2 s + 1] coordinates 8 s + 0, 4, 1, 5.  The activations' planes use the same order.
     uint32_t y[6];
     uint32_t goff;  // shared-memory address of the scale table plus 8 g (the gain's column of the table)
 };
 // Coordinate of a block held by byte i of word k.
-__host__ __device__ constexpr int word_coordinate(int k, int i) { return 8 * (k >> 1) + 2 * i + ((k & 1) ? 0 : 1); }
+__host__ __device__ constexpr int word_coordinate(int k, int i) { return 8 * (k >> 1) + 4 * (i & 1) + (i >> 1) + ((k & 1) ? 0 : 2); }
+static_assert(fast_nibble(word_coordinate(0, 1)) == 3 && fast_nibble(word_coordinate(1, 2)) == 4 && fast_nibble(word_coordinate(0, 2)) == 5,
+              "byte i of the high (low) nibbles is nibble 2 i + 1 (2 i)");
 
 // A row table entry holds, per coordinate, the nibble -2 k, where 4 k = 0, 4, -4, 8, -8 is the rank's element of
 // the o = 0 list (Sec. 3.3).  The lists of o = p + 2 c are 4 k, 1 - 4 k, 2 - 4 k, 4 k - 1, so with the nibble z
@@ -179,12 +181,17 @@ __host__ __device__ constexpr int word_coordinate(int k, int i) { return 8 * (k 
 //     -y = 2 z + p     for all four lists and all five ranks
 // (two's complement, -5 <= z <= 4).  The pattern masks and the complement for p are XORs; z moves to the upper
 // half of its byte and p below it: a byte 16 z + 8 p = -8 y costs half a logic operation.
+struct NibbleBlock {
+    uint32_t z[3];  // section s: coordinate j's z at bits 4 fast_nibble(j)
+    uint32_t p4;    // bit 2: p (the other bits are an address)
+    uint32_t goff;  // shared-memory address of the scale table plus 8 g (the gain's column of the table)
+};
 // HI = false: w1 sits in bits 0..15 of `w1pair`; HI = true: in bits 16..31.
 // sm_tab: shared-memory address of the staged tables, a multiple of 16 KiB, so
 // that every index is merged with its table's address by the same LOP3 that
 // masks it.
 template <bool HI>
-__device__ __forceinline__ void fast_decode(uint32_t sm_tab, uint32_t w0, uint32_t w1pair, FastBlock& out) {
+__device__ __forceinline__ void decode_nibbles(uint32_t sm_tab, uint32_t w0, uint32_t w1pair, NibbleBlock& out) {
     const uint32_t sh = HI ? w1pair >> 14 : w1pair << 2;                 // [2..12] i2, [13] p, [14..17] x
     const uint32_t addr1 = (w0 & 0x3FFCu) | (sm_tab + kSmRows);          // (i1 | r << 11) * 4
     const uint32_t addr2 = (sh & 0x1FFCu) | (sm_tab + kSmMid);
@@ -201,16 +208,22 @@ __device__ __forceinline__ void fast_decode(uint32_t sm_tab, uint32_t w0, uint32
     const uint32_t ma = lds32(a4);
     const uint32_t mb = lds32(b4);
     const uint32_t mx = lds32(x4);
-    const uint32_t z1 = row1 ^ ma ^ mx;
-    const uint32_t z2 = row2 ^ mb ^ mx;
-    const uint32_t z3 = row3 ^ (ma ^ mb) ^ mx;
-    const uint32_t p8 = (x4 & 4u) * 0x02020202u;                         // 8 p in every byte
-    out.y[0] = (z1 & 0xF0F0F0F0u) | p8;
-    out.y[1] = ((z1 << 4) & 0xF0F0F0F0u) | p8;
-    out.y[2] = (z2 & 0xF0F0F0F0u) | p8;
-    out.y[3] = ((z2 << 4) & 0xF0F0F0F0u) | p8;
-    out.y[4] = (z3 & 0xF0F0F0F0u) | p8;
-    out.y[5] = ((z3 << 4) & 0xF0F0F0F0u) | p8;
+    out.z[0] = row1 ^ ma ^ mx;
+    out.z[1] = row2 ^ mb ^ mx;
+    out.z[2] = row3 ^ (ma ^ mb) ^ mx;
+    out.p4 = x4;
+}
+template <bool HI>
+__device__ __forceinline__ void fast_decode(uint32_t sm_tab, uint32_t w0, uint32_t w1pair, FastBlock& out) {
+    NibbleBlock nb;
+    decode_nibbles<HI>(sm_tab, w0, w1pair, nb);
+    out.goff = nb.goff;
+    const uint32_t p8 = (nb.p4 & 4u) * 0x02020202u;                      // 8 p in every byte
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        out.y[2 * s] = (nb.z[s] & 0xF0F0F0F0u) | p8;
+        out.y[2 * s + 1] = ((nb.z[s] << 4) & 0xF0F0F0F0u) | p8;
+    }
 }
 
 // Shared-memory address of -gain[g] / sqrt(16 m): the squared norm of the packed point is 64 * 16 m, the table has
@@ -290,14 +303,16 @@ __device__ __forceinline__ void split_planes(uint32_t q0, uint32_t q1, uint32_t 
     mid = prmt(a, b, 0x7632u);
     hi = prmt(prmt(q0, q1, 0x0062u), prmt(q2, q3, 0x0062u), 0x5410u);
 }
-// Plane words 2 s and 2 s + 1 of section s, from its four pairs: odd coordinates first, the decoder's order.
+// Plane words 2 s and 2 s + 1 of section s, from its four pairs, in the decoder's order.
 __device__ __forceinline__ void quantise_section(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, float inv, uint32_t (&hi)[2],
                                                  uint32_t (&mid)[2], uint32_t (&lo)[2]) {
-    static_assert(word_coordinate(0, 1) == 3 && word_coordinate(1, 1) == 2 && word_coordinate(5, 3) == 22, "odd coordinates first");
-    split_planes(quantise_value<true>(w0, inv), quantise_value<true>(w1, inv), quantise_value<true>(w2, inv),
+    static_assert(word_coordinate(0, 0) == 2 && word_coordinate(0, 1) == 6 && word_coordinate(0, 2) == 3 && word_coordinate(0, 3) == 7 &&
+                      word_coordinate(1, 0) == 0 && word_coordinate(1, 1) == 4 && word_coordinate(1, 2) == 1 && word_coordinate(1, 3) == 5,
+                  "pairs 1 and 3, then 0 and 2");
+    split_planes(quantise_value<false>(w1, inv), quantise_value<false>(w3, inv), quantise_value<true>(w1, inv),
                  quantise_value<true>(w3, inv), hi[0], mid[0], lo[0]);
-    split_planes(quantise_value<false>(w0, inv), quantise_value<false>(w1, inv), quantise_value<false>(w2, inv),
-                 quantise_value<false>(w3, inv), hi[1], mid[1], lo[1]);
+    split_planes(quantise_value<false>(w0, inv), quantise_value<false>(w2, inv), quantise_value<true>(w0, inv),
+                 quantise_value<true>(w2, inv), hi[1], mid[1], lo[1]);
 }
 __device__ __forceinline__ void quantise_column(const __half* __restrict__ x, int K, int c, uint32_t out[20]) {
     uint32_t w[12];

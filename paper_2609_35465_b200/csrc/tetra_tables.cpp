@@ -183,7 +183,7 @@ int build_device_tables(DeviceTables* out, const float* gain2) {
         for (int j = 0; j < 8; ++j) {
             const unsigned r = (row >> (4 * j)) & 15u;
             if (r > 4) return false;
-            *fast |= nibble[r] << (4 * j);
+            *fast |= nibble[r] << (4 * fast_nibble(j));
         }
         return true;
     };
@@ -196,8 +196,8 @@ int build_device_tables(DeviceTables* out, const float* gain2) {
         const uint8_t h = span4(turyn.h, v), hr = span4(turyn.hr, v);
         uint32_t mh = 0, mhr = 0;
         for (int j = 0; j < 8; ++j) {
-            mh |= ((h >> j) & 1) ? 15u << (4 * j) : 0u;
-            mhr |= ((hr >> j) & 1) ? 15u << (4 * j) : 0u;
+            mh |= ((h >> j) & 1) ? 15u << (4 * fast_nibble(j)) : 0u;
+            mhr |= ((hr >> j) & 1) ? 15u << (4 * fast_nibble(j)) : 0u;
         }
         out->mask_h[v] = mh;
         out->mask_xp[2 * v] = mhr;

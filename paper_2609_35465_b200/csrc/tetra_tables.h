@@ -17,7 +17,10 @@ struct PaperTables {
 static_assert(sizeof(PaperTables) == 18816, "paper table blob is 18,816 bytes");
 
 constexpr uint32_t kTableMagic = 0x54455442u;  // "TETB"
-constexpr uint32_t kTableVersion = 8;
+constexpr uint32_t kTableVersion = 9;
+// Nibble of a fast table word that belongs to coordinate j of a section: neighbours are sixteen bits apart, so that one
+// mask picks the pair (j, j + 1) as the two halves of a register.
+constexpr int fast_nibble(int j) { return (j >> 1) + 4 * (j & 1); }
 constexpr int kMiddleClass0 = 1240;            // N0 of Sec. 3.3 (checked at build)
 // The last row of a class's 2048 and of the middle list's class 0 (checked at build): each cuts a shell of equal
 // cost at this packed value; the middle list's class 1 ends with a whole shell.
@@ -30,7 +33,8 @@ struct DeviceTables {
     uint32_t magic;             // 18824
     uint32_t version;           // 18828
     // ---- fast path: everything below is staged in shared memory ------------
-    // Rank rows, class by class: nibble j = -2 k (two's complement) of coordinate j's rank, k = 0, 1, -1, 2, -2.
+    // Rank rows, class by class: nibble fast_nibble(j) = -2 k (two's complement) of coordinate j's rank,
+    // k = 0, 1, -1, 2, -2.
     // (the kernels place this part on a 16 KiB boundary of shared memory, so each
     //  sub-table's offset can be OR-ed into an index instead of added)
     uint32_t rows_fast[4096];   // +0
@@ -39,7 +43,7 @@ struct DeviceTables {
                                 //         16 bytes per m, the two gains 8 bytes apart, so that lanes with nearby
                                 //         m or different g read different banks.  Minus: the fast decoder emits
                                 //         minus (eight times) the point.
-    // Pattern-byte masks of the Turyn coordinates: nibble j all ones where the Hamming word has coordinate j
+    // Pattern-byte masks of the Turyn coordinates: nibble fast_nibble(j) all ones where the Hamming word has coordinate j
     // set; H for a and b, H' for x.  mask_xp has x and the parity in one index, x << 1 | p, and is complemented
     // where p = 1.
     uint32_t mask_h[16];        // +25600
