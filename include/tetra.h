@@ -190,17 +190,15 @@ int tetra_gemv_grouped(const tetra_problem *problems_host, int count, const void
 
 /* Several activation vectors at once (1 <= batch <= 16): every block is decoded
  * once and multiplied with all vectors; the contraction over a block's 24
- * coordinates runs on the tensor cores (int8 x int8 -> int32, exact), the
- * per-block scale and the accumulation across blocks in float32.  Same result
- * definition as tetra_gemv_tail.  workspace_dev: 16-byte aligned scratch of at
- * least tetra_batched_workspace_bytes(N, K) bytes (partial results of column
- * ranges, which a second small kernel sums in a fixed order; its contents need
- * no initialisation), private to the call until it completes.  Two kernel
- * launches; the result is bit-identical from run to run.  With one vector
- * the call runs tetra_gemv_tail's kernel instead (one launch, the workspace
- * untouched), which is faster there; two to four vectors run a kernel that
- * feeds the tensor cores from the decoder's registers, five and more one
- * that goes through shared-memory tiles. */
+ * coordinates runs on the tensor cores (float16 x float16, both operands exact,
+ * products accumulated in float32), the per-block scale and the accumulation
+ * across blocks in float32.  Same result definition as tetra_gemv_tail, and the
+ * same rule for non-finite activations; every finite float16 activation is used
+ * as it is (no fixed point).  workspace_dev: 16-byte aligned memory of at least
+ * tetra_batched_workspace_bytes(N, K) bytes, private to the call until it
+ * completes; the present kernels keep their partial sums on chip and leave it
+ * untouched.  One kernel launch; the result is bit-identical from run to run.
+ * With one vector the call runs tetra_gemv_tail's kernel, which is faster there. */
 size_t tetra_batched_workspace_bytes(int N, int K);
 int tetra_gemv_batched(const void *codes, const float *row_scales, const void *table,
                        const void *x, float *y, int N, int K, int batch, const void *tail,

@@ -219,8 +219,8 @@ int tetra_gemv_batched(const void* codes, const float* row_scales, const void* t
     const int B = tail_mode ? K / 24 : (K + 23) / 24;
     if (B <= 0 || B > kMaxBlocksPerRow) return TETRA_ERR_SHAPE;
     if (workspace_bytes < batched_workspace_bytes(N, B)) return TETRA_ERR_SIZE;
-    // One vector: the single-launch kernel is faster than the tensor-core paths' fixed costs (measured on
-    // B200, 4096 x 12288: 11.6 us against 15.8 us for two vectors on the tensor cores).
+    // One vector: the integer products of the single-matrix kernel need fewer instructions per block than the
+    // conversion to float16 that several vectors share (4096 x 4096: 5.4 us against 6.8 us for two vectors).
     if (batch <= kBatchedMinVectors - 1)
         return tetra_gemv_tail(codes, row_scales, table, x, y, N, K, batch, tail, stream);
     return cuda_status(launch_gemv_batched(codes, row_scales, table, x, y, N, K, batch, (K % 24) ? tail : nullptr,

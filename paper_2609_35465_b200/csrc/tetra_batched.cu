@@ -2,29 +2,38 @@
 // multiplied with every vector, in one launch.
 //
 // The products of a block's 24 coordinates with up to 16 vectors are a small dense contraction and run on the tensor
-// cores: mma.sync m16n8k16 + m16n8k8, float16 x float16 with float32 accumulation.  Half of minus a coordinate,
-// -y / 2 = z + p / 2, is a float16 that two logic operations and one addition make from the decoder's nibbles, and
-// the activations ARE float16, so both operands and every product are exact.  (The three int8 planes of 24-bit fixed
-// point that the batch-1 kernels use cost three MMAs and five instructions per result here; the float32 result costs
-// half a packed FFMA.)  mma.sync rather than tcgen05: a CTA owns about 28 rows of a 4096-row matrix, a tile of 16
-// rows keeps sixteen warps busy with that, 128 rows would not, and the tensor cores are far from the limit.
+// cores: mma.sync m16n8k16, float16 x float16 with float32 accumulation.  Half of minus a coordinate, -y / 2 = z + p / 2,
+// is a float16 that two logic operations and one addition make from the decoder's nibbles, and the activations ARE
+// float16, so both operands and every product are exact.  (The three int8 planes of 24-bit fixed point that the batch-1
+// kernels use cost three times the MMAs and five instructions per result here; the float32 result costs half a packed
+// FFMA.)  mma.sync rather than tcgen05: a CTA owns about 28 rows of a 4096-row matrix, a tile of 16 rows keeps sixteen
+// warps busy with that, 128 rows would not.
 //
-// A warp's step is up to four tiles of 16 rows x the same four block columns: lane 4 q + t decodes rows q and q + 8 of
-// a tile at column t and leaves each block's 24 halves in a shared-memory tile whose rows keep stores and ldmatrix
-// conflict-free; the block's scale stays in the lane and reaches the lanes that hold the block's results by a
-// shuffle.  The sixteen warps of a CTA take every sixteenth column quad, so a warp needs nothing from the others until
-// the end: its words come straight from global memory one step ahead, the four columns' activations through its own
-// cp.async buffer, and its accumulators live in registers.  (Activations of many columns staged by the CTA, warps
-// cut along the rows: 10.0 / 30 us for 4096 x 4096 with three vectors / 4096 x 12288 with sixteen.)
+// Lane 4 q + t decodes rows 2 q and 2 q + 1 of a 16-row tile at column t of four.  Two ways from there:
+//   up to four vectors: straight from registers.  An MMA takes four coordinates of both blocks from every lane as A
+//   (rows q and q + 8), and B is block diagonal -- column 2 t + v of B is zero outside the k range that lane t feeds --
+//   so D[q][2 t + v] is the product of lane (q, t)'s own block with vector v of its own column and arrives in that same
+//   lane, next to the block's scale: six MMAs for two blocks per lane and two vectors, no shuffle, no shared-memory
+//   tile, and B is the activations as they lie in memory;
+//   five and more: dense B.  A block's 24 halves go through a shared-memory tile whose rows keep stores and ldmatrix
+//   conflict-free, an MMA pair (k16 + k8) multiplies sixteen blocks of ONE column with eight vectors, and the
+//   block's scale reaches the lanes that hold its results by a shuffle.
+// The line lies where the tensor pipe's time for the zeros overtakes the tile: 4096 x 4096 with 2 / 4 / 8 / 16 vectors
+// takes 6.7 / 7.5 / 9.3 / 13.3 us block diagonal and 8.5 / 8.7 / 9.0 / 11.1 us dense (11.9 us for three vectors and
+// 27.2 us for sixteen at 4096 x 12288 with int8 planes, activations staged by the CTA and a combining kernel;
+// now 7.4 and 24.6 us).
 //
-// One launch, no scratch memory: what a call of a few microseconds consists of is latency, and the second kernel that
-// added the CTAs' partial sums cost more than the products of a 4096 x 4096 matrix.  A CTA owns whole rows; where
-// rows are too few for all SMs, a cluster of two to eight CTAs shares them, each takes a range of columns, and the
-// partial sums meet through distributed shared memory.  Sums are added in warp order, then CTA order: bit-identical
-// from run to run.
+// A warp's step is NT row tiles x four block columns.  The sixteen warps of a CTA take every sixteenth column quad, so a
+// warp needs nothing from the others until the end: its words come straight from global memory one step ahead, the four
+// columns' activations through its own cp.async buffer, and its accumulators live in registers.
 //
-// Bound by instruction issue in the steps (decode, conversion, tile) and, for small matrices, by the chain of
-// launch, tables, one step and sums.
+// One launch, no scratch memory: what a call of a few microseconds consists of is latency, and a second kernel that
+// adds the CTAs' partial sums costs more than the products of a 4096 x 4096 matrix.  A CTA owns whole rows; where
+// rows are too few for all SMs, a cluster of two CTAs shares them, each takes a range of columns, and the partial sums
+// meet through distributed shared memory.  Sums are added in warp order, then CTA order: bit-identical from run to run.
+//
+// Bound by instruction issue in the steps (decode and conversion) and, for small matrices, by the chain of launch,
+// tables, one step and sums.
 #include <cuda_fp16.h>
 
 #include "q4_common.cuh"
@@ -32,12 +41,8 @@
 
 namespace tetra {
 
-constexpr int kBatThreads = 512;
-constexpr int kBatWarps = kBatThreads / 32;
-constexpr uint32_t kTileCol = 16 * 48 + 32;    // bytes per column of a tile: 16 rows of 24 halves, bank spread
-constexpr uint32_t kTileBytes = 4 * kTileCol;  // four columns
-constexpr uint32_t kXVec = 4 * 48 + 16;        // bytes per vector of an activation buffer: four columns, bank spread
-constexpr int kBatMaxTiles = 4;                // row tiles whose sums a warp holds at a time
+constexpr uint32_t kXVec = 4 * 48 + 16;        // bytes per vector of an activation buffer: four columns, a line of zeros
+constexpr int kBatMaxTiles = 4;                // row tiles of a step
 
 struct BatParams {
     const unsigned char* codes;
@@ -51,27 +56,40 @@ struct BatParams {
     int32_t cluster;         // CTAs of a cluster
 };
 
-// Tiles decoded together: two blocks per lane and tile; four blocks in flight hide the table lookups better, which the
-// shared memory allows where eight vectors' activations are the most.
-__host__ __device__ constexpr int tiles_at_once(int ng, int nt) { return ng == 1 && nt > 1 ? 2 : 1; }
-// Row stride, in floats, of the partial sums (8 ng vectors): even, so that pairs stay aligned.
-__host__ __device__ constexpr int part_stride(int ng) { return 8 * ng + 2; }
+constexpr int kBatWarps = 16, kBatThreads = 32 * kBatWarps;
+constexpr uint32_t kTileCol = 16 * 48 + 32;    // bytes per column of a shared-memory tile: 16 rows of 24 halves, bank spread
+constexpr uint32_t kTileBytes = 4 * kTileCol;  // four columns
+
+// G: vector pairs (block diagonal) or groups of eight (dense); slots: vectors they make room for.
+constexpr int bat_slots(bool dense, int g) { return (dense ? 8 : 2) * g; }
+// Dense: tiles decoded together.  Four blocks in flight per lane hide the table lookups better than two; with two
+// groups the registers do not allow it.
+constexpr int bat_together(bool dense, int g, int nt) { return dense && g == 1 && nt > 1 ? 2 : 1; }
+// Row stride, in floats, of the partial sums: even, so that pairs stay aligned.
+constexpr int bat_stride(bool dense, int g) { return bat_slots(dense, g) + 2; }
 struct BatSmem {
-    // offsets from the 16 KiB-aligned table copy; total includes the alignment slack
+    // offsets from the 16 KiB-aligned table copy; total includes the alignment slack.  A warp's area: two activation
+    // buffers, then its tiles (dense); the partial sums of all warps take the areas' place at the end.
     uint32_t warps, per_warp, rs, tail, xtail, total;
 };
-__host__ __device__ constexpr BatSmem bat_smem(int ng, int nt) {
+constexpr BatSmem bat_smem(bool dense, int g, int nt) {
     BatSmem S{};
-    S.warps = uint32_t(kFastBytes);  // per warp: tiles, two activation buffers; afterwards the sums of all warps
-    S.per_warp = uint32_t(tiles_at_once(ng, nt)) * kTileBytes + 2u * 8u * uint32_t(ng) * kXVec;
-    S.rs = S.warps + kBatWarps * S.per_warp;
+    S.warps = uint32_t(kFastBytes);
+    S.per_warp = 2u * uint32_t(bat_slots(dense, g)) * kXVec + (dense ? uint32_t(bat_together(dense, g, nt)) * kTileBytes : 0u);
+    const uint32_t sums = uint32_t(nt * 16 * bat_stride(dense, g) * 4);  // per warp
+    S.rs = S.warps + kBatWarps * (S.per_warp > sums ? S.per_warp : sums);
     S.tail = S.rs + uint32_t(nt) * 64u;                 // half [rows][24]
     S.xtail = S.tail + uint32_t(nt) * (16u * 48u);      // float [16][24]
     S.total = S.xtail + 16u * 96u + kSmAlign;
     return S;
 }
-static_assert(kBatWarps * kBatMaxTiles * 16 * part_stride(2) * 4 <= kBatWarps * bat_smem(2, kBatMaxTiles).per_warp, "sums fit");
-static_assert(bat_smem(1, 4).total <= 227 * 1024 && bat_smem(2, 4).total <= 227 * 1024, "shared memory");
+static_assert(bat_smem(false, 2, 4).total <= 227 * 1024 && bat_smem(true, 1, 4).total <= 227 * 1024 &&
+              bat_smem(true, 2, 4).total <= 227 * 1024, "shared memory");
+template <bool DENSE, int G, int NT>
+struct BatShape {
+    static constexpr int slots = bat_slots(DENSE, G), together = bat_together(DENSE, G, NT), stride = bat_stride(DENSE, G);
+    static constexpr BatSmem smem = bat_smem(DENSE, G, NT);
+};
 
 // Half of minus the point, float16 x 2: a[4 s + t] = coordinates 2 t and 2 t + 1 of section s.  Returns the block's scale
 // (minus the gain over sqrt(16 m)).  A nibble z sits in the mantissa of 64 (as z + 8: the exclusive or that sets
@@ -126,14 +144,14 @@ __device__ __forceinline__ uint4 load_eight(const __half* x, int n) {
 }
 
 __device__ __forceinline__ void mma_k16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
-                 : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 __device__ __forceinline__ void mma_k8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
     asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a0), "r"(a1), "r"(b0));
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(b0));
 }
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -147,11 +165,13 @@ __device__ __forceinline__ float cluster_load(uint32_t saddr, uint32_t rank) {
     return v;
 }
 
-// NG: groups of eight vectors; NT: row tiles of a step.
-template <int NG, int NT>
-__global__ void __launch_bounds__(kBatThreads, 1) k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ BatParams P) {
-    constexpr int PS = part_stride(NG), W = kBatWarps, TW = tiles_at_once(NG, NT);
-    constexpr BatSmem S = bat_smem(NG, NT);
+// DENSE, G: see bat_slots; NT: row tiles of a step.
+template <bool DENSE, int G, int NT>
+__global__ void __launch_bounds__(kBatThreads, 1)
+k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ BatParams P) {
+    using Shape = BatShape<DENSE, G, NT>;
+    constexpr int PS = Shape::stride, W = kBatWarps, THREADS = kBatThreads, SLOTS = Shape::slots, TW = Shape::together;
+    constexpr BatSmem S = Shape::smem;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_release();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -168,36 +188,36 @@ __global__ void __launch_bounds__(kBatThreads, 1) k_gemv_batched(const DeviceTab
     float* rs_sm = reinterpret_cast<float*>(smem + S.rs);
     __half* tail_sm = reinterpret_cast<__half*>(smem + S.tail);
     float* xtail = reinterpret_cast<float*>(smem + S.xtail);
-    const uint32_t tile = sm_tab + S.warps + uint32_t(warp) * S.per_warp, xbuf = tile + TW * kTileBytes;
-    constexpr uint32_t kXBuf = 8 * NG * kXVec;
+    constexpr uint32_t kXBuf = SLOTS * kXVec;
+    const uint32_t xbuf = sm_tab + S.warps + uint32_t(warp) * S.per_warp;
+    [[maybe_unused]] const uint32_t tile = xbuf + 2 * kXBuf;
     const int ntail = P.tail ? P.K % 24 : 0, Kx = min(P.K, 24 * P.B);
-    const int row_groups = (P.N + 7) / 8;
 
-    // This lane's words of a step: rows q and q + 8 of NT tiles at column t.  Rows and columns outside the matrix repeat
-    // the last one: such rows are not stored, such columns meet zeros.  words_at moves the lane's two addresses to a
-    // quad; a row group is a uniform offset from there.
-    uint32_t w0[NT][2], w1[NT][2];
-    const unsigned char* lane_words = P.codes + (size_t(q >> 2) * P.B * 16 + size_t(q & 3) * 4);
-    const uint32_t lane_w1 = uint32_t(2 - (q >> 2)) * uint32_t(P.B) * 16u + uint32_t(q) * 2u - uint32_t(q & 3) * 4u;
+    // This lane's words of a step: rows 2 q and 2 q + 1 of NT tiles at column t.  Rows and columns outside the matrix
+    // repeat a row group or column inside: such rows are not stored, such columns meet zeros.  words_at moves the
+    // lane's address to a quad; a tile is a uniform offset from there.
+    uint2 w0[NT];
+    uint32_t w1[NT];
+    const int last_rg = (P.N + 7) / 8 - 1;
     const unsigned char* words = nullptr;
+    const uint32_t lane_w0 = uint32_t((q >> 1) & 1) * uint32_t(P.B) * 16u + uint32_t(q & 1) * 8u;
+    const uint32_t lane_w1 = uint32_t(2 * P.B) * 16u + uint32_t(q & 3) * 4u;
     auto words_at = [&](int t0, int quad) {
-        words = lane_words + (size_t(2 * t0) * 3 * P.B + min(4 * quad + t, P.B - 1)) * 16;
+        words = P.codes + (size_t(min(2 * t0 + (q >> 2), last_rg)) * 3 * P.B + min(4 * quad + t, P.B - 1)) * 16;
     };
     auto load_words = [&](int i, int t0) {
-#pragma unroll
-        for (int rg = 0; rg < 2; ++rg) {
-            const uint32_t off = uint32_t(min(2 * i + rg, row_groups - 1 - 2 * t0)) * 48u * uint32_t(P.B);
-            w0[i][rg] = __ldg(reinterpret_cast<const uint32_t*>(words + off));
-            w1[i][rg] = __ldg(reinterpret_cast<const unsigned short*>(words + (off + lane_w1)));
-        }
+        const int up = min(2 * i, max((last_rg - 2 * t0 - (q >> 2)) & ~1, 0));  // row groups from the first tile's
+        const unsigned char* at = words + uint32_t(up) * 48u * uint32_t(P.B);
+        w0[i] = __ldg(reinterpret_cast<const uint2*>(at + lane_w0));
+        w1[i] = __ldg(reinterpret_cast<const uint32_t*>(at + lane_w1));
     };
     auto stage_rows = [&](int t0, int nt) {
         const int row0 = 16 * t0, rows = min(16 * nt, P.N - row0);
-        for (int i = threadIdx.x; i < rows; i += kBatThreads)
+        for (int i = threadIdx.x; i < rows; i += THREADS)
             asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(smem_u32(rs_sm + i)), "l"(P.row_scales + row0 + i));
         if (ntail) {
             const __half* tl = P.tail + size_t(row0) * ntail;
-            for (int r = threadIdx.x >> 3; r < rows; r += kBatThreads / 8)
+            for (int r = threadIdx.x >> 3; r < rows; r += THREADS / 8)
                 for (int k = threadIdx.x & 7; k < ntail; k += 8) tail_sm[r * 24 + k] = tl[size_t(r) * ntail + k];
         }
     };
@@ -212,7 +232,7 @@ __global__ void __launch_bounds__(kBatThreads, 1) k_gemv_batched(const DeviceTab
         const uint32_t dst = xbuf + slot * kXBuf + uint32_t(x_v) * kXVec + uint32_t(x_u) * 16u;
         if (x_wide) {
 #pragma unroll
-            for (int i = 0; i < 4 * NG; ++i, src += step)
+            for (int i = 0; i < SLOTS / 2; ++i, src += step)
                 if (lane < 24 && 2 * i + x_v < V)
                     asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" :: "r"(dst + uint32_t(i) * 2u * kXVec), "l"(src), "r"(2 * n));
         } else {
@@ -235,24 +255,34 @@ __global__ void __launch_bounds__(kBatThreads, 1) k_gemv_batched(const DeviceTab
     stage_fast_tables_async(tab, smem_raw);
     stage_rows(tile_lo, min(tile_hi - tile_lo, NT));
     pdl_wait();  // x may come from the preceding kernel
-    for (int i = threadIdx.x; i < V * 24; i += kBatThreads) {
+    for (int i = threadIdx.x; i < V * 24; i += THREADS) {
         const int v = i / 24, k = i - 24 * v;
         xtail[i] = k < ntail ? __half2float(P.x[size_t(v) * P.K + 24 * P.B + k]) : 0.f;
     }
 
-    uint32_t x_vec[NG];  // this lane's words of the first column: + column * 48 + section * 16
+    // Block diagonal: lane 4 q + t holds its column of B's coordinates only where q / 2 = t, of vector q % 2 of a pair;
+    // the other lanes (and a vector beyond the last) read a line of zeros.  Dense: word t of a section, of vector q of
+    // a group (results beyond the last vector are never used, whatever they are).
+    const bool mine = (q >> 1) == t;
+    uint32_t x_lane[G];
 #pragma unroll
-    for (int n = 0; n < NG; ++n) x_vec[n] = xbuf + uint32_t(min(8 * n + q, V - 1)) * kXVec + uint32_t(t) * 4u;  // results beyond V are never used
+    for (int g = 0; g < G; ++g) {
+        if (DENSE) x_lane[g] = uint32_t(min(8 * g + q, V - 1)) * kXVec + uint32_t(t) * 4u;
+        else x_lane[g] = mine && 2 * g + (q & 1) < V ? uint32_t(2 * g + (q & 1)) * kXVec + uint32_t(t) * 48u : 192u;
+    }
+    const uint32_t x_step = mine ? 16u : 0u;
 
     for (int t0 = tile_lo; t0 < tile_hi; t0 += NT) {
         const int nt = min(tile_hi - t0, NT);
-        float acc[NT][NG][4];
+        // rows 2 q (k = 0, 1) and 2 q + 1 (k = 2, 3): block diagonal, the lane's own column, vectors 2 g and 2 g + 1;
+        // dense, all columns, vectors 8 g + 2 t and 8 g + 2 t + 1
+        float acc[NT][G][4];
 #pragma unroll
         for (int i = 0; i < NT; ++i)
 #pragma unroll
-            for (int n = 0; n < NG; ++n)
+            for (int g = 0; g < G; ++g)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc[i][n][k] = 0.f;
+                for (int k = 0; k < 4; ++k) acc[i][g][k] = 0.f;
         if (t0 != tile_lo) {
             __syncthreads();  // the sums of the tiles before have been read
             stage_rows(t0, nt);
@@ -264,6 +294,8 @@ __global__ void __launch_bounds__(kBatThreads, 1) k_gemv_batched(const DeviceTab
         }
         uint32_t slot = 0;
         if (quad_lo + warp < quad_hi) stage_x(0, quad_lo + warp);
+        if (!DENSE && lane < 2)  // the line of zeros in both buffers
+            asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" :: "r"(xbuf + uint32_t(lane) * kXBuf + 192u), "r"(0u) : "memory");
         asm volatile("cp.async.commit_group;");
         if (t0 == tile_lo) {
             asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -275,87 +307,121 @@ __global__ void __launch_bounds__(kBatThreads, 1) k_gemv_batched(const DeviceTab
             const int next = min(quad + W, quad_hi - 1);
             if (quad + W < quad_hi) stage_x(slot ^ 1u, next);
             asm volatile("cp.async.commit_group;");
-            const uint32_t x_off = slot * kXBuf;
             words_at(t0, next);
+            const uint32_t x_at = xbuf + slot * kXBuf;
+            if constexpr (!DENSE) {
 #pragma unroll
-            for (int i0 = 0; i0 < NT; i0 += TW) {
-                constexpr int kLeft = NT % TW;  // an odd last tile goes alone
-                const int tw = i0 + TW <= NT ? TW : kLeft;
-                float scale[TW][2];
-#pragma unroll
-                for (int k = 0; k < tw; ++k) {
-                    const int i = i0 + k;
-#pragma unroll
-                    for (int rg = 0; rg < 2; ++rg) {
-                        uint32_t a[12];
-                        scale[k][rg] = decode_halves<false>(sm_tab, w0[i][rg], w1[i][rg], a);
-                        const uint32_t dst = tile + uint32_t(k) * kTileBytes + uint32_t(t) * kTileCol + uint32_t(8 * rg + q) * 48u;
-#pragma unroll
-                        for (int s = 0; s < 3; ++s)
-                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" :: "r"(dst + 16u * s), "r"(a[4 * s]), "r"(a[4 * s + 1]),
-                                         "r"(a[4 * s + 2]), "r"(a[4 * s + 3]) : "memory");
-                    }
+                for (int i = 0; i < NT; ++i) {
+                    uint32_t a[2][12];
+                    const float s0 = decode_halves<false>(sm_tab, w0[i].x, w1[i], a[0]);
+                    const float s1 = decode_halves<true>(sm_tab, w0[i].y, w1[i], a[1]);
                     load_words(i, t0);
-                }
-                __syncwarp();
-                // ldmatrix: lane gives the address of row lane % 8 of matrix lane / 8 = (rows 0-7, section 0),
-                // (8-15, 0), (0-7, 1), (8-15, 1); then the two of section 2
-                uint32_t a[2][TW][4], a2[2][TW][2];
-                auto fragments = [&](int j) {
 #pragma unroll
-                    for (int k = 0; k < tw; ++k) {
-                        const uint32_t at = tile + uint32_t(k) * kTileBytes + uint32_t(j) * kTileCol + uint32_t(lane & 15) * 48u;
-                        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                                     : "=r"(a[j & 1][k][0]), "=r"(a[j & 1][k][1]), "=r"(a[j & 1][k][2]), "=r"(a[j & 1][k][3])
-                                     : "r"(at + uint32_t(lane >> 4) * 16u) : "memory");
-                        asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
-                                     : "=r"(a2[j & 1][k][0]), "=r"(a2[j & 1][k][1]) : "r"(at + 32u) : "memory");
+                    for (int g = 0; g < G; ++g) {
+                        float d[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                        for (int m = 0; m < 3; ++m) {
+                            uint32_t b[4];
+                            q4_lds128(x_at + x_lane[g] + m * x_step, b);
+                            const uint32_t a0[4] = {a[0][4 * m], a[1][4 * m], a[0][4 * m + 1], a[1][4 * m + 1]};
+                            const uint32_t a1[4] = {a[0][4 * m + 2], a[1][4 * m + 2], a[0][4 * m + 3], a[1][4 * m + 3]};
+                            mma_k16(d, a0, b[0], b[1]);
+                            mma_k16(d, a1, b[2], b[3]);
+                        }
+                        fma2(s0, d[0], d[1], acc[i][g][0], acc[i][g][1]);
+                        fma2(s1, d[2], d[3], acc[i][g][2], acc[i][g][3]);
                     }
-                };
-                fragments(0);
+                }
+            } else {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (j < 3) fragments(j + 1);
-                    uint32_t b[NG][3];
-#pragma unroll
-                    for (int n = 0; n < NG; ++n)
-#pragma unroll
-                        for (int s = 0; s < 3; ++s)
-                            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b[n][s]) : "r"(x_vec[n] + x_off + uint32_t(48 * j + 16 * s)));
+                for (int i0 = 0; i0 < NT; i0 += TW) {
+                    constexpr int kLeft = NT % TW;  // an odd last tile goes alone
+                    const int tw = i0 + TW <= NT ? TW : kLeft;
+                    float scale[TW][2];
 #pragma unroll
                     for (int k = 0; k < tw; ++k) {
-                        const float s_lo = __shfl_sync(0xFFFFFFFFu, scale[k][0], (lane & 28) | j);
-                        const float s_hi = __shfl_sync(0xFFFFFFFFu, scale[k][1], (lane & 28) | j);
+                        const int i = i0 + k;
 #pragma unroll
-                        for (int n = 0; n < NG; ++n) {
-                            float d[4];
-                            mma_k16(d, a[j & 1][k], b[n][0], b[n][1]);
-                            mma_k8(d, a2[j & 1][k][0], a2[j & 1][k][1], b[n][2]);
-                            fma2(s_lo, d[0], d[1], acc[i0 + k][n][0], acc[i0 + k][n][1]);
-                            fma2(s_hi, d[2], d[3], acc[i0 + k][n][2], acc[i0 + k][n][3]);
+                        for (int rg = 0; rg < 2; ++rg) {
+                            uint32_t a[12];
+                            scale[k][rg] = rg ? decode_halves<true>(sm_tab, w0[i].y, w1[i], a) : decode_halves<false>(sm_tab, w0[i].x, w1[i], a);
+                            const uint32_t dst = tile + uint32_t(k) * kTileBytes + uint32_t(t) * kTileCol + uint32_t(8 * rg + q) * 48u;
+#pragma unroll
+                            for (int s = 0; s < 3; ++s)
+                                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" :: "r"(dst + 16u * s), "r"(a[4 * s]), "r"(a[4 * s + 1]),
+                                             "r"(a[4 * s + 2]), "r"(a[4 * s + 3]) : "memory");
+                        }
+                        load_words(i, t0);
+                    }
+                    __syncwarp();
+                    // ldmatrix: lane gives the address of row lane % 8 of matrix lane / 8 = (rows 0-7, section 0),
+                    // (8-15, 0), (0-7, 1), (8-15, 1); then the two of section 2
+                    uint32_t a[2][TW][4], a2[2][TW][2];
+                    auto fragments = [&](int j) {
+#pragma unroll
+                        for (int k = 0; k < tw; ++k) {
+                            const uint32_t at = tile + uint32_t(k) * kTileBytes + uint32_t(j) * kTileCol + uint32_t(lane & 15) * 48u;
+                            asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                                         : "=r"(a[j & 1][k][0]), "=r"(a[j & 1][k][1]), "=r"(a[j & 1][k][2]), "=r"(a[j & 1][k][3])
+                                         : "r"(at + uint32_t(lane >> 4) * 16u) : "memory");
+                            asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
+                                         : "=r"(a2[j & 1][k][0]), "=r"(a2[j & 1][k][1]) : "r"(at + 32u) : "memory");
+                        }
+                    };
+                    fragments(0);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if (j < 3) fragments(j + 1);
+                        uint32_t b[G][3];
+#pragma unroll
+                        for (int g = 0; g < G; ++g)
+#pragma unroll
+                            for (int s = 0; s < 3; ++s)
+                                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b[g][s]) : "r"(x_at + x_lane[g] + uint32_t(48 * j + 16 * s)));
+#pragma unroll
+                        for (int k = 0; k < tw; ++k) {
+                            const float s0 = __shfl_sync(0xFFFFFFFFu, scale[k][0], (lane & 28) | j);
+                            const float s1 = __shfl_sync(0xFFFFFFFFu, scale[k][1], (lane & 28) | j);
+#pragma unroll
+                            for (int g = 0; g < G; ++g) {
+                                float d[4] = {0.f, 0.f, 0.f, 0.f};
+                                mma_k16(d, a[j & 1][k], b[g][0], b[g][1]);
+                                mma_k8(d, a2[j & 1][k][0], a2[j & 1][k][1], b[g][2]);
+                                fma2(s0, d[0], d[1], acc[i0 + k][g][0], acc[i0 + k][g][1]);
+                                fma2(s1, d[2], d[3], acc[i0 + k][g][2], acc[i0 + k][g][3]);
+                            }
                         }
                     }
+                    __syncwarp();  // the tile has been read before the next blocks overwrite it
                 }
-                __syncwarp();  // the tile has been read before the next blocks overwrite it
             }
             slot ^= 1u;
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();  // everybody has left the tiles and buffers: the sums take their place
+        __syncthreads();  // everybody has left the buffers and tiles: the sums take their place
 #pragma unroll
         for (int i = 0; i < NT; ++i)
 #pragma unroll
-            for (int n = 0; n < NG; ++n)
+            for (int g = 0; g < G; ++g) {
+                if constexpr (!DENSE) {  // the four columns of a row first; lane t writes the pairs t modulo 4
 #pragma unroll
-                for (int k = 0; k < 4; k += 2)
-                    *reinterpret_cast<float2*>(part + (size_t(i * W + warp) * 16 + q + 4 * k) * PS + 8 * n + 2 * t) =
-                        make_float2(acc[i][n][k], acc[i][n][k + 1]);
+                    for (int k = 0; k < 4; ++k) {
+                        acc[i][g][k] += __shfl_xor_sync(0xFFFFFFFFu, acc[i][g][k], 1);
+                        acc[i][g][k] += __shfl_xor_sync(0xFFFFFFFFu, acc[i][g][k], 2);
+                    }
+                }
+                float* at = part + ((i * W + warp) * 16 + 2 * q) * PS + (DENSE ? 8 * g + 2 * t : 2 * g);
+                if (DENSE || (g & 3) == t) {
+                    *reinterpret_cast<float2*>(at) = make_float2(acc[i][g][0], acc[i][g][1]);
+                    *reinterpret_cast<float2*>(at + PS) = make_float2(acc[i][g][2], acc[i][g][3]);
+                }
+            }
         __syncthreads();
-        // Thread = (tile, vector, row of the tile); the warps' sums in warp order.
-        constexpr int AT_ONCE = kBatThreads / (128 * NG);  // tiles
-        const int r = threadIdx.x & 15, v = (threadIdx.x >> 4) & (8 * NG - 1), rt0 = threadIdx.x / (128 * NG);
-        auto tile_sum = [&](int rt) {
-            const float* at = part + (size_t(rt * W) * 16 + r) * PS + v;
+        // Output `id`: (tile, vector, row of the tile); the warps' sums in warp order.
+        const int ids = nt * (16 * SLOTS);
+        auto warps_sum = [&](int id) {
+            const int r = id & 15, v = (id >> 4) % SLOTS, rt = (id >> 4) / SLOTS;
+            const float* at = part + (rt * W * 16 + r) * PS + v;
             float sum = 0.f;
 #pragma unroll
             for (int w = 0; w < W; ++w) sum += at[w * 16 * PS];
@@ -363,34 +429,33 @@ __global__ void __launch_bounds__(kBatThreads, 1) k_gemv_batched(const DeviceTab
         };
         // Twice the halves' sum (row scale, tail).  A column with a NaN or an infinity has made its products in every row
         // infinite or NaN: 0 x sum makes them all NaN.
-        auto finish = [&](float sum, int rt) {
-            const int i = 16 * rt + r, row = 16 * t0 + i;
-            if (row >= P.N) return;
+        auto finish = [&](float sum, int id) {
+            const int r = id & 15, v = (id >> 4) % SLOTS, rt = (id >> 4) / SLOTS, i = 16 * rt + r, row = 16 * t0 + i;
+            if (row >= P.N || v >= V) return;
             float res = 2.f * rs_sm[i] * fmaf(0.f, sum, sum);
             for (int k = 0; k < ntail; ++k) res = fmaf(__half2float(tail_sm[i * 24 + k]), xtail[24 * v + k], res);
             P.y[size_t(v) * P.N + row] = res;
         };
         if (C == 1) {
-            if (v < V)
-                for (int rt = rt0; rt < nt; rt += AT_ONCE) finish(tile_sum(rt), rt);
+            for (int id = threadIdx.x; id < ids; id += THREADS) finish(warps_sum(id), id);
         } else {
             // The sums over the CTA's columns replace the parts once everybody has read those; then every CTA of the
-            // cluster finishes every C-th turn of tiles.
-            constexpr int PER = (NT + AT_ONCE - 1) / AT_ONCE;
+            // cluster finishes its share of the outputs.
+            constexpr int PER = (NT * 16 * SLOTS + THREADS - 1) / THREADS;
             float sums[PER];
 #pragma unroll
-            for (int j = 0; j < PER; ++j) sums[j] = rt0 + j * AT_ONCE < nt ? tile_sum(rt0 + j * AT_ONCE) : 0.f;
+            for (int j = 0; j < PER; ++j) sums[j] = int(threadIdx.x) + j * THREADS < ids ? warps_sum(int(threadIdx.x) + j * THREADS) : 0.f;
             __syncthreads();
 #pragma unroll
             for (int j = 0; j < PER; ++j)
-                if (rt0 + j * AT_ONCE < nt) part[threadIdx.x + j * kBatThreads] = sums[j];
+                if (int(threadIdx.x) + j * THREADS < ids) part[threadIdx.x + j * THREADS] = sums[j];
             cluster_barrier();
-            if (v < V)
-                for (int j = rank; rt0 + j * AT_ONCE < nt; j += C) {
-                    float sum = 0.f;
-                    for (int c = 0; c < C; ++c) sum += cluster_load(smem_u32(part + threadIdx.x + j * kBatThreads), uint32_t(c));
-                    finish(sum, rt0 + j * AT_ONCE);
-                }
+            const int id_lo = ids * rank / C, id_hi = ids * (rank + 1) / C;
+            for (int id = id_lo + int(threadIdx.x); id < id_hi; id += THREADS) {
+                float sum = 0.f;
+                for (int c = 0; c < C; ++c) sum += cluster_load(smem_u32(part + id), uint32_t(c));
+                finish(sum, id);
+            }
             cluster_barrier();  // the other CTAs have read this one's sums
         }
     }
@@ -408,19 +473,13 @@ namespace {
 struct BatPlan {
     int cluster = 1, groups = 1, nt = 1;
 };
-// Resident clusters of c CTAs when each CTA takes an SM to itself (a GPC holds whole clusters only).
-int resident_clusters(int c, int sms) {
-    if (c == 1) return sms;
-    return c == 2 ? sms / 2 : 0;
-}
-
 // How rows and columns are split: for every cluster size the steps of the busiest warp, in units of one tile x four
 // columns (about 0.5 us on B200), and what else the split costs.
 BatPlan plan_batched(int tiles, int quads, int sms) {
     BatPlan best;
     double best_cost = 1e30;
-    for (int c = 1; c <= 8; c *= 2) {
-        const int room = resident_clusters(c, sms);
+    for (int c = 1; c <= 2; c *= 2) {
+        const int room = sms / c;
         if (c > quads || room == 0) break;
         BatPlan p;
         p.cluster = c;
@@ -437,10 +496,21 @@ BatPlan plan_batched(int tiles, int quads, int sms) {
     return best;
 }
 
-template <int NG>
-auto batched_kernel(int nt) {
-    return nt == 1 ? k_gemv_batched<NG, 1> : (nt == 2 ? k_gemv_batched<NG, 2> : (nt == 3 ? k_gemv_batched<NG, 3> : k_gemv_batched<NG, 4>));
+struct BatKernel {
+    void (*run)(const DeviceTables*, BatParams);
+    uint32_t smem;
+};
+template <bool DENSE, int G, int NT>
+constexpr BatKernel bat_kernel() {
+    return {k_gemv_batched<DENSE, G, NT>, BatShape<DENSE, G, NT>::smem.total};
 }
+// by vectors (up to 2, 4: block diagonal; 8, 16: dense) and tiles of a step
+const BatKernel kBatKernels[4][kBatMaxTiles] = {
+    {bat_kernel<false, 1, 1>(), bat_kernel<false, 1, 2>(), bat_kernel<false, 1, 3>(), bat_kernel<false, 1, 4>()},
+    {bat_kernel<false, 2, 1>(), bat_kernel<false, 2, 2>(), bat_kernel<false, 2, 3>(), bat_kernel<false, 2, 4>()},
+    {bat_kernel<true, 1, 1>(), bat_kernel<true, 1, 2>(), bat_kernel<true, 1, 3>(), bat_kernel<true, 1, 4>()},
+    {bat_kernel<true, 2, 1>(), bat_kernel<true, 2, 2>(), bat_kernel<true, 2, 3>(), bat_kernel<true, 2, 4>()},
+};
 
 }  // namespace
 
@@ -452,10 +522,9 @@ cudaError_t launch_gemv_batched(const void* codes, const float* row_scales, cons
     static PerDeviceOnce once;
     e = once.run([] {
         cudaError_t r = cudaSuccess;
-        for (int nt = 1; nt <= kBatMaxTiles && r == cudaSuccess; ++nt) {
-            r = cudaFuncSetAttribute(batched_kernel<1>(nt), cudaFuncAttributeMaxDynamicSharedMemorySize, int(bat_smem(1, nt).total));
-            if (r == cudaSuccess) r = cudaFuncSetAttribute(batched_kernel<2>(nt), cudaFuncAttributeMaxDynamicSharedMemorySize, int(bat_smem(2, nt).total));
-        }
+        for (const auto& row : kBatKernels)
+            for (const BatKernel& k : row)
+                if (r == cudaSuccess) r = cudaFuncSetAttribute(k.run, cudaFuncAttributeMaxDynamicSharedMemorySize, int(k.smem));
         return r;
     });
     if (e != cudaSuccess) return e;
@@ -474,7 +543,7 @@ cudaError_t launch_gemv_batched(const void* codes, const float* row_scales, cons
     const BatPlan plan = plan_batched(P.tiles, P.quads, sms);
     P.groups = plan.groups;
     P.cluster = plan.cluster;
-    const int ng = batch <= 8 ? 1 : 2;
+    const BatKernel& kernel = kBatKernels[batch <= 2 ? 0 : (batch <= 4 ? 1 : (batch <= 8 ? 2 : 3))][plan.nt - 1];
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -484,11 +553,11 @@ cudaError_t launch_gemv_batched(const void* codes, const float* row_scales, cons
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(unsigned(plan.groups * plan.cluster));
     cfg.blockDim = dim3(kBatThreads);
-    cfg.dynamicSmemBytes = bat_smem(ng, plan.nt).total;
+    cfg.dynamicSmemBytes = kernel.smem;
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = plan.cluster > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, ng == 1 ? batched_kernel<1>(plan.nt) : batched_kernel<2>(plan.nt), static_cast<const DeviceTables*>(table), P);
+    return cudaLaunchKernelEx(&cfg, kernel.run, static_cast<const DeviceTables*>(table), P);
 }
 
 }  // namespace tetra
