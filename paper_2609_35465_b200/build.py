@@ -37,7 +37,7 @@ def _binding_command(out: str):
             "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
             "-isystem", inc, "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"),
             "-isystem", os.path.join(cuda, "include"), "-isystem", sysconfig.get_paths()["include"],
-            os.path.join(CSRC, "binding.cpp"), "-o", out, "-L" + lib, "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10",
+            os.path.join(CSRC, "binding.cpp"), "-o", out, "-L" + lib, "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10",
             "-ldl"]
 
 

@@ -41,6 +41,25 @@ __global__ void __launch_bounds__(256) k_decode_file(const uint8_t* __restrict__
 // in flight.  12288 x 4096: 13.8 us with the map and a row permutation read through L1 and three 2-byte loads,
 // now 10.8 us.
 // ---------------------------------------------------------------------------
+// The (row group, 32 columns) items of a warp, every `warps`-th of them in row-major order, without a division per item.
+struct ItemWalk {
+    int G, cg, step_G, step_cg, col_groups;
+    __device__ __forceinline__ ItemWalk(int warp, int warps, int col_groups_) : col_groups(col_groups_) {
+        G = warp / col_groups;
+        cg = warp - G * col_groups;
+        step_G = warps / col_groups;
+        step_cg = warps - step_G * col_groups;
+    }
+    __device__ __forceinline__ void next() {
+        G += step_G;
+        cg += step_cg;
+        if (cg >= col_groups) {
+            cg -= col_groups;
+            ++G;
+        }
+    }
+};
+
 __global__ void __launch_bounds__(256, 4) k_pack(const uint8_t* __restrict__ codes,
                                                  const DeviceTables* __restrict__ tab,
                                                  uint4* __restrict__ packed, int N, int B) {
@@ -51,27 +70,27 @@ __global__ void __launch_bounds__(256, 4) k_pack(const uint8_t* __restrict__ cod
     __syncthreads();
     pdl_wait();  // the words may come from, the packed matrix be read by, the kernel before
     const int groups = (N + 7) / 8, lane = threadIdx.x & 31;
-    const int col_groups = (B + 31) / 32, items = groups * col_groups;
-    for (int it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += (gridDim.x * blockDim.x) >> 5) {
-        const int G = it / col_groups, c = min((it - G * col_groups) * 32 + lane, B - 1);
+    const uint32_t row_bytes = uint32_t(B) * 6u;
+    for (ItemWalk it((blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5, (B + 31) / 32); it.G < groups; it.next()) {
+        const int G = it.G, c = min(it.cg * 32 + lane, B - 1), rows = min(8, N - 8 * G);
         // a word is 2-byte aligned: its 4-byte aligned part (first or last four bytes) and the other two bytes
-        uint32_t four[8], two[8];
-        bool front[8];
+        const uint8_t* first = codes + (size_t(8 * G) * B + c) * 6;
+        uint32_t four[8], two[8], back[8];
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-            const uint8_t* at = codes + (size_t(min(8 * G + r, N - 1)) * B + c) * 6;
-            front[r] = (reinterpret_cast<uintptr_t>(at) & 2) == 0;
-            four[r] = __ldg(reinterpret_cast<const uint32_t*>(at + (front[r] ? 0 : 2)));
-            two[r] = __ldg(reinterpret_cast<const unsigned short*>(at + (front[r] ? 4 : 0)));
+            const uint8_t* at = first + uint32_t(min(r, rows - 1)) * row_bytes;
+            back[r] = uint32_t(reinterpret_cast<uintptr_t>(at)) & 2u;
+            four[r] = __ldg(reinterpret_cast<const uint32_t*>(at + back[r]));
+            two[r] = __ldg(reinterpret_cast<const unsigned short*>(at + 4 - 2 * back[r]));
         }
         uint32_t w0[8], w1[8];
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-            const uint64_t w = front[r] ? uint64_t(four[r]) | (uint64_t(two[r]) << 32) : uint64_t(two[r]) | (uint64_t(four[r]) << 16);
+            const uint64_t w = back[r] ? uint64_t(two[r]) | (uint64_t(four[r]) << 16) : uint64_t(four[r]) | (uint64_t(two[r]) << 32);
             file_to_device_word(w, abx[trellis_path(w)], &w0[r], &w1[r]);
-            if (8 * G + r >= N) w0[r] = w1[r] = 0u;  // padding rows: the all-zero device word
+            if (r >= rows) w0[r] = w1[r] = 0u;  // padding rows: the all-zero device word
         }
-        if ((it - G * col_groups) * 32 + lane >= B) continue;
+        if (it.cg * 32 + lane >= B) continue;
         uint4* rec = packed + size_t(G) * 3 * B + c;
         rec[0] = make_uint4(w0[0], w0[1], w0[2], w0[3]);
         rec[B] = make_uint4(w0[4], w0[5], w0[6], w0[7]);
@@ -87,23 +106,26 @@ __global__ void __launch_bounds__(256, 4) k_pack(const uint8_t* __restrict__ cod
 // touch every sector six times).  Bound by instruction issue (decoder and byte arithmetic), the stores close behind.
 // 12288 x 4096: 35.8 us with direct stores, now 18.9 us (67 MB).
 // ---------------------------------------------------------------------------
-constexpr int kEmitRows = 2;  // rows decoded and staged at a time (four CTAs then share an SM)
 constexpr int kEmitThreads = 256;
+constexpr int kEmitStage = 2 * 768;  // two rows of 32 blocks at a time
 
-// Coordinates of a block in file order, four int8 per word, from the decoder's -8 y.
-__device__ __forceinline__ void file_order(const FastBlock& fb, uint32_t (&out)[6]) {
+// Coordinates of a block in file order, four int8 per word.  With a nibble's sign bit flipped it is z + 8, so
+// y = -(2 z + p) = (16 - p) - 2 (z + 8), bytewise with 128 added so that no byte borrows.
+__device__ __forceinline__ void file_order(const NibbleBlock& nb, uint32_t (&out)[6]) {
+    const uint32_t top = 0x90909090u - ((nb.p4 >> 2) & 1u) * 0x01010101u;
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
-        uint32_t v[2];  // y of coordinates 2, 6, 3, 7 and 0, 4, 1, 5
-#pragma unroll
-        for (int k = 0; k < 2; ++k)  // 16 - y = the five-bit -y with its sign bit flipped; bytes never borrow
-            v[k] = (0x90909090u - (((fb.y[2 * s + k] >> 3) & 0x1F1F1F1Fu) ^ 0x10101010u)) ^ 0x80808080u;
-        out[2 * s] = prmt(v[1], v[0], 0x6420u);
-        out[2 * s + 1] = prmt(v[1], v[0], 0x7531u);
+        const uint32_t z = nb.z[s];
+        const uint32_t hi = (top - (((z >> 3) & 0x1E1E1E1Eu) ^ 0x10101010u)) ^ 0x80808080u;  // coordinates 2, 6, 3, 7
+        const uint32_t lo = (top - (((z << 1) & 0x1E1E1E1Eu) ^ 0x10101010u)) ^ 0x80808080u;  // coordinates 0, 4, 1, 5
+        static_assert(word_coordinate(0, 1) == 6 && word_coordinate(1, 2) == 1, "order of the nibbles");
+        out[2 * s] = prmt(lo, hi, 0x6420u);
+        out[2 * s + 1] = prmt(lo, hi, 0x7531u);
     }
 }
 
-template <bool WIDE>
+// WIDTH: alignment of a row of y in bytes that the stores may use, 16, 8 or 4 (4: mg goes out bytewise).
+template <int WIDTH>
 __global__ void __launch_bounds__(kEmitThreads, 4)
 k_decode_packed(const uint4* __restrict__ packed, const DeviceTables* __restrict__ tab, int8_t* __restrict__ y_out,
                 uint8_t* __restrict__ mg_out, int N, int B) {
@@ -114,74 +136,73 @@ k_decode_packed(const uint4* __restrict__ packed, const DeviceTables* __restrict
     __syncthreads();
     pdl_wait();  // the packed matrix may come from, the outputs be read by, the kernel before
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned char* stage = base + kFastBytes + warp * (kEmitRows * 768);
-    const int groups = (N + 7) / 8, col_groups = (B + 31) / 32, items = groups * col_groups;
-    const int stride = (gridDim.x * blockDim.x) >> 5;
-    int it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    unsigned char* stage = base + kFastBytes + warp * kEmitStage;
+    const int groups = (N + 7) / 8;
     uint4 lo, hi, w1;
-    auto load = [&](int item) {
-        const int G = item / col_groups, c0 = (item - G * col_groups) * 32;
-        const uint4* rec = packed + size_t(G) * 3 * B + min(c0 + lane, B - 1);
+    auto load = [&](const ItemWalk& at) {
+        const uint4* rec = packed + size_t(at.G) * 3 * B + min(at.cg * 32 + lane, B - 1);
         lo = __ldg(rec);
         hi = __ldg(rec + B);
         w1 = __ldg(rec + 2 * size_t(B));
     };
-    if (it < items) load(it);
-    for (; it < items; it += stride) {
-        const int G = it / col_groups, c0 = (it - G * col_groups) * 32, cols = min(32, B - c0);
+    // a lane's units of the copy out: unit `lane + 32 k` of two rows
+    constexpr int kUnits = 768 / WIDTH, kTurns = 2 * kUnits / 32;
+    uint32_t unit_at[kTurns], unit_off[kTurns];
+    const uint32_t row_bytes = uint32_t(B) * 24u;
+#pragma unroll
+    for (int k = 0; k < kTurns; ++k) {
+        const int u = lane + 32 * k, r = u >= kUnits ? 1 : 0;
+        unit_at[k] = uint32_t(u - r * kUnits) * WIDTH;       // inside its row
+        unit_off[k] = unit_at[k] + (r ? row_bytes : 0u);
+    }
+    ItemWalk it((blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5, (B + 31) / 32);
+    if (it.G < groups) load(it);
+    while (it.G < groups) {
+        const int G = it.G, c0 = it.cg * 32, cols = min(32, B - c0), rows = min(8, N - 8 * G);
         const uint32_t w0[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
         const uint32_t w1p[4] = {w1.x, w1.y, w1.z, w1.w};
-        if (it + stride < items) load(it + stride);
+        it.next();
+        if (it.G < groups) load(it);
+        const size_t block0 = size_t(8 * G) * B + c0;
+        int8_t* y_pair = y_out + block0 * 24;
+        const bool mg_lane = mg_out && lane < cols;
+        uint8_t* mg_at = mg_out + 2 * (block0 + lane);
 #pragma unroll
-        for (int r0 = 0; r0 < 8; r0 += kEmitRows) {
+        for (int r0 = 0; r0 < 8; r0 += 2) {
             __syncwarp();  // the staged rows of the turn before have been read
-            uint32_t mg[kEmitRows];
 #pragma unroll
-            for (int r = 0; r < kEmitRows; ++r) {
-                FastBlock fb;
-                if (r & 1) fast_decode<true>(sm_tab, w0[r0 + r], w1p[(r0 + r) >> 1], fb);
-                else fast_decode<false>(sm_tab, w0[r0 + r], w1p[(r0 + r) >> 1], fb);
+            for (int r = 0; r < 2; ++r) {
+                NibbleBlock nb;
+                if (r) decode_nibbles<true>(sm_tab, w0[r0 + 1], w1p[r0 >> 1], nb);
+                else decode_nibbles<false>(sm_tab, w0[r0], w1p[r0 >> 1], nb);
                 uint32_t y[6];
-                file_order(fb, y);
+                file_order(nb, y);
                 uint2* dst = reinterpret_cast<uint2*>(stage + r * 768 + lane * 24);
 #pragma unroll
                 for (int k = 0; k < 3; ++k) dst[k] = make_uint2(y[2 * k], y[2 * k + 1]);
                 int n2 = 0;  // 16 m
 #pragma unroll
                 for (int k = 0; k < 6; ++k) n2 = dp4a_ss(y[k], y[k], n2);
-                mg[r] = (uint32_t(n2) >> 4) | ((w0[r0 + r] >> 17) & 0x100u);  // g: bit 25 of w0
+                if (mg_lane && r0 + r < rows) {
+                    const uint32_t mg = (uint32_t(n2) >> 4) | ((w0[r0 + r] >> 17) & 0x100u);  // g: bit 25 of w0
+                    if (WIDTH > 4) *reinterpret_cast<uint16_t*>(mg_at) = uint16_t(mg);
+                    else mg_at[0] = uint8_t(mg), mg_at[1] = uint8_t(mg >> 8);
+                }
+                mg_at += 2u * uint32_t(B);
             }
             __syncwarp();
-            const int rows = min(kEmitRows, N - 8 * G - r0);
-            const size_t block0 = size_t(8 * G + r0) * B + c0;
-            if (mg_out && lane < cols) {
 #pragma unroll
-                for (int r = 0; r < kEmitRows; ++r) {
-                    uint8_t* dst = mg_out + 2 * (block0 + size_t(r) * B + lane);
-                    if (r < rows) {
-                        if (WIDE) *reinterpret_cast<uint16_t*>(dst) = uint16_t(mg[r]);
-                        else dst[0] = uint8_t(mg[r]), dst[1] = uint8_t(mg[r] >> 8);
-                    }
+            for (int k = 0; k < kTurns; ++k) {
+                const bool second = lane + 32 * k >= kUnits;
+                if (unit_at[k] < 24u * uint32_t(cols) && r0 + (second ? 1 : 0) < rows) {
+                    int8_t* dst = y_pair + unit_off[k];
+                    const unsigned char* src = stage + (lane + 32 * k) * WIDTH;
+                    if (WIDTH == 16) *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(src);
+                    else if (WIDTH == 8) *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(src);
+                    else *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(src);
                 }
             }
-#pragma unroll
-            for (int r = 0; r < kEmitRows; ++r) {
-                const uint2* src = reinterpret_cast<const uint2*>(stage + r * 768);
-                int8_t* dst = y_out + (block0 + size_t(r) * B) * 24;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const int i = lane + 32 * k;
-                    if (r < rows && i < 3 * cols) {
-                        const uint2 v = src[i];
-                        if (WIDE) {
-                            reinterpret_cast<uint2*>(dst)[i] = v;
-                        } else {
-                            reinterpret_cast<uint32_t*>(dst)[2 * i] = v.x;
-                            reinterpret_cast<uint32_t*>(dst)[2 * i + 1] = v.y;
-                        }
-                    }
-                }
-            }
+            y_pair += 2u * row_bytes;
         }
     }
 }
@@ -220,18 +241,23 @@ cudaError_t launch_decode_packed(const void* packed, const void* table, int8_t* 
     if (e != cudaSuccess) return e;
     const size_t items = size_t((N + 7) / 8) * ((B + 31) / 32);
     if (items > 0x7FFFFFF0u / 32) return cudaErrorInvalidValue;
-    constexpr int smem = int(kTableSmemBytes) + kEmitThreads / 32 * kEmitRows * 768;
+    constexpr int smem = int(kTableSmemBytes) + kEmitThreads / 32 * kEmitStage;
     static PerDeviceOnce once;
     e = once.run([] {
-        cudaError_t r = cudaFuncSetAttribute(k_decode_packed<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (r == cudaSuccess) r = cudaFuncSetAttribute(k_decode_packed<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        auto set = [](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); };
+        cudaError_t r = set(k_decode_packed<16>);
+        if (r == cudaSuccess) r = set(k_decode_packed<8>);
+        if (r == cudaSuccess) r = set(k_decode_packed<4>);
         return r;
     });
     if (e != cudaSuccess) return e;
     const int grid = grid_for(items * 32, kEmitThreads, sms * 4);
-    const bool wide = reinterpret_cast<uintptr_t>(y) % 8 == 0 && reinterpret_cast<uintptr_t>(mg) % 2 == 0;
-    return launch_pdl(wide ? k_decode_packed<true> : k_decode_packed<false>, grid, kEmitThreads, smem, s,
-                      static_cast<const uint4*>(packed), static_cast<const DeviceTables*>(table), y, mg, N, B);
+    // every row and every 32 columns (768 bytes) must keep the alignment; a block count that is odd leaves 8
+    const bool mg_even = reinterpret_cast<uintptr_t>(mg) % 2 == 0;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(y);
+    auto kernel = mg_even && at % 16 == 0 && B % 2 == 0 ? k_decode_packed<16> : (mg_even && at % 8 == 0 ? k_decode_packed<8> : k_decode_packed<4>);
+    return launch_pdl(kernel, grid, kEmitThreads, smem, s, static_cast<const uint4*>(packed), static_cast<const DeviceTables*>(table), y,
+                      mg, N, B);
 }
 
 }  // namespace tetra
