@@ -213,19 +213,18 @@ struct EncShared {
     float hi[3][16 * kHiStride];
     float lo_odd[3][16 * kOddLoStride];
     float hi_odd[3][16 * kOddHiStride];
-    // section tables: [class][pair = alpha + 8 xi][row].  F1 exists twice at even parity: plain and one entry up.
-    alignas(16) float F1[2][2][64 * kRow];
-    alignas(16) float F2[2][64 * kRow];
-    alignas(16) float F3[2][64 * kRow];
+    // section tables, even and odd parity: [section][class][pair = alpha + 8 xi][row]
+    alignas(16) float F[3][2][64 * kRow];
+    alignas(16) float O[3][2][64 * kOddRow];
     float rs[32];             // 1 / sqrt(16 m)
     float w[24];
     uint32_t halves[kHalfVectors];
     uint8_t bytes[64];        // h(alpha) + h'(xi)
-    float red_val[4];
-    uint32_t red_arg[4];
+    float red_val[6];         // per warp: the best of the objective
+    uint32_t red_arg[6];      // and the thread that holds it
     float win_H[20];
     float win_G;
-    int win_arg;
+    int win_arg, win_par;
     // the winner so far, per section: byte pair, class, index and value of its table entry
     int hit_pair[3], hit_cls[3], hit_k[3];
     float hit_target[3];
@@ -600,8 +599,8 @@ __device__ __forceinline__ void section_odd(const float* lo, const float* hi, fl
 // The section tables of one section, thread = byte pair.  EVEN: rows of k; else rows of W / 2.
 template <bool EVEN, bool MID>
 __device__ __forceinline__ void section_rows(EncShared& S, int s, int pair) {
-    float* rows0 = s == 0 ? S.F1[0][0] : (s == 1 ? S.F2[0] : S.F3[0]);
-    float* rows1 = s == 0 ? S.F1[0][1] : (s == 1 ? S.F2[1] : S.F3[1]);
+    float* rows0 = EVEN ? S.F[s][0] : S.O[s][0];
+    float* rows1 = EVEN ? S.F[s][1] : S.O[s][1];
     const uint32_t byte = S.bytes[pair];
     if constexpr (EVEN) {
         float* r0 = rows0 + pair * kRow;
@@ -638,16 +637,6 @@ __device__ __forceinline__ void section_rows(EncShared& S, int s, int pair) {
                 const int k1 = kappa_hs(1, int(b >> 4)) + ones_offset(b);
 #pragma unroll
                 for (int k = 0; k < 5; ++k) r1[k1 + k] = fmaxf(r1[k1 + k], __fadd_rn(h1, lo[kOffRes1 + k]));
-            }
-        }
-        if (s == 0) {  // the second copy, one entry up
-            float* u0 = S.F1[1][0] + pair * kRow;
-            float* u1 = S.F1[1][1] + pair * kRow;
-            u0[0] = u1[0] = kNeg;
-#pragma unroll
-            for (int k = 0; k < kRow - 1; ++k) {
-                u0[k + 1] = r0[k];
-                u1[k + 1] = r1[k];
             }
         }
     } else {
@@ -703,8 +692,8 @@ __device__ __forceinline__ void max_plus(const float (&a)[LA], const float (&b)[
 
 constexpr int kH = 20;  // entries after two sections: norms 16 i (+ 8), i < 20
 
-// Row lengths in use: even parity k <= 9 (one more in the raised copy of F1), the middle list k <= 8 (class 0)
-// and k <= 7.  Odd parity: W / 2 <= 5, the middle list 4 and 3.
+// Row lengths in use: even parity k <= 9, the middle list k <= 8 (class 0) and k <= 7.  Odd parity: W / 2 <= 5, the
+// middle list 4 and 3.
 template <bool EVEN, int PAR>
 __device__ __forceinline__ void join_two(const EncShared& S, int gamma, int xi, bool odd_end, float (&H)[kH]) {
 #pragma unroll
@@ -716,15 +705,18 @@ __device__ __forceinline__ void join_two(const EncShared& S, int gamma, int xi, 
             constexpr int c1 = decltype(ci)::value, c2 = c1 ^ PAR;
             if constexpr (EVEN) {
                 // norms 16 k1 + r1 and 16 k2 + r2: index k1 + k2, plus one when both residues are 8
-                const int raised = !odd_end && odd_overlap(S.bytes[i]) ? 1 : 0;
-                float a[12], b[12];
-                load_row(S.F1[raised][c1] + i * kRow, a);
-                load_row(S.F2[c2] + j * kRow, b);
+                const bool raised = !odd_end && odd_overlap(S.bytes[i]);
+                float r[12], a[12], b[12];
+                load_row(S.F[0][c1] + i * kRow, r);
+                load_row(S.F[1][c2] + j * kRow, b);
+                a[0] = raised ? kNeg : r[0];
+#pragma unroll
+                for (int k = 1; k < 12; ++k) a[k] = raised ? r[k - 1] : r[k];
                 max_plus<11, c2 ? 8 : 9, 0>(a, b, H);
             } else {
                 float a[8], b[8];
-                load_row(S.F1[0][c1] + i * kOddRow, a);
-                load_row(S.F2[c2] + j * kOddRow, b);
+                load_row(S.O[0][c1] + i * kOddRow, a);
+                load_row(S.O[1][c2] + j * kOddRow, b);
                 max_plus<6, c2 ? 4 : 5, c1 & c2>(a, b, H);  // W1 + W2 = 2 (index) + (classes' parity)
             }
         });
@@ -739,7 +731,7 @@ __device__ __forceinline__ void objective(const EncShared& S, int m0, int end_pa
 #pragma unroll
     for (int n = 0; n < NG; ++n) G[n] = kNeg;
     float b[EVEN ? 12 : 8];
-    load_row(S.F3[CLS3] + end_pair * (EVEN ? kRow : kOddRow), b);
+    load_row((EVEN ? S.F[2][CLS3] : S.O[2][CLS3]) + end_pair * (EVEN ? kRow : kOddRow), b);
     max_plus<NA, NB, 0>(H, b, G);
     val = kNeg;
     corr = kNeg;
@@ -906,13 +898,16 @@ __device__ __noinline__ void trace_join(EncShared& S, bool even, int end_pair, i
     const int lane = threadIdx.x & 31;
     const int cls3 = (even ? 0 : 1) ^ par;
     const int row_len = even ? kRow : kOddRow;
+    const float *rows1[2] = {even ? S.F[0][0] : S.O[0][0], even ? S.F[0][1] : S.O[0][1]};
+    const float *rows2[2] = {even ? S.F[1][0] : S.O[1][0], even ? S.F[1][1] : S.O[1][1]};
+    const float* rows3 = even ? S.F[2][cls3] : S.O[2][cls3];
     const int gamma = end_pair & 7, xi = end_pair >> 3;
     // index after two sections and of the third
     int q = 0, k3 = 0;
     {
         const int j = lane, i = n - j;
         const int nb = even ? 10 : 6, na = even ? 19 : 10;
-        const bool hit = j < nb && i >= 0 && i < na && __fadd_rn(S.win_H[i >= 0 && i < na ? i : 0], S.F3[cls3][end_pair * row_len + (j < nb ? j : 0)]) == S.win_G;
+        const bool hit = j < nb && i >= 0 && i < na && __fadd_rn(S.win_H[i >= 0 && i < na ? i : 0], rows3[end_pair * row_len + (j < nb ? j : 0)]) == S.win_G;
         const uint32_t any = __ballot_sync(0xFFFFFFFFu, hit);
         if (any) {
             k3 = __ffs(int(any)) - 1;
@@ -930,7 +925,9 @@ __device__ __noinline__ void trace_join(EncShared& S, bool even, int end_pair, i
     for (int i = lane >> 4; i < (even ? 11 : 6); i += 2) {
         const int j = q - shift - i;
         const int nb = even ? (c2 ? 8 : 9) : (c2 ? 4 : 5);
-        if (hit_i < 0 && j >= 0 && j < nb && __fadd_rn(S.F1[raised][c1][p1 * row_len + i], S.F2[c2][p2 * row_len + j]) == h) hit_i = i;
+        if (hit_i < 0 && i >= raised && j >= 0 && j < nb &&
+            __fadd_rn(rows1[c1][p1 * row_len + i - raised], rows2[c2][p2 * row_len + j]) == h)
+            hit_i = i;
     }
     const uint32_t any = __ballot_sync(0xFFFFFFFFu, hit_i >= 0);
     const int src = any ? __ffs(int(any)) - 1 : 0;
@@ -941,76 +938,32 @@ __device__ __noinline__ void trace_join(EncShared& S, bool even, int end_pair, i
     const int j2 = max(q - w_shift - i1, 0);
     if (lane < 3) {
         const int pair = lane == 0 ? w_p1 : (lane == 1 ? w_p2 : end_pair), cls = lane == 0 ? w_c1 : (lane == 1 ? w_c2 : cls3);
-        const int at = lane == 0 ? i1 : (lane == 1 ? j2 : k3);
-        const float* rows = lane == 0 ? S.F1[w_raised][w_c1] : (lane == 1 ? S.F2[w_c2] : S.F3[cls3]);
+        const int at = lane == 0 ? max(i1 - w_raised, 0) : (lane == 1 ? j2 : k3);
+        const float* rows = lane == 0 ? rows1[w_c1] : (lane == 1 ? rows2[w_c2] : rows3);
         S.hit_pair[lane] = pair;
         S.hit_cls[lane] = cls;
-        S.hit_k[lane] = lane == 0 ? max(i1 - w_raised, 0) : at;
+        S.hit_k[lane] = at;
         S.hit_target[lane] = rows[pair * row_len + at];
     }
 }
 
-template <bool EVEN>
-__device__ __forceinline__ void search_parity(EncShared& S, int tid, bool live, float& best_val, bool& best_even) {
-    const int warp = tid >> 5, lane = tid & 31;
-    if (live) {  // section tables: warps 0, 1 = section 0, warps 2, 3 = section 1, warps 4, 5 = section 2
-        const int s = tid >> 6, pair = tid & 63;
-        if (s == 1) section_rows<EVEN, true>(S, 1, pair);
-        else section_rows<EVEN, false>(S, s, pair);
-    }
-    __syncthreads();
-    float H[kH];
-    float val = kNeg, corr = kNeg;
-    int arg = 0;
-    if (live && tid < 128) {
-        const int end_pair = tid & 63, par = tid >> 6;
-        const int gamma = end_pair & 7, xi = end_pair >> 3;
-        const bool odd_end = odd_overlap(S.bytes[end_pair]) != 0;
-        // squared norm = 16 (index + m0)
-        const int m0 = EVEN ? (odd_end ? 1 : 0) : 2;
-        if (par == 0) {
-            join_two<EVEN, 0>(S, gamma, xi, odd_end, H);
-            objective<EVEN, EVEN ? 0 : 1>(S, m0, end_pair, H, val, corr, arg);
-        } else {
-            join_two<EVEN, 1>(S, gamma, xi, odd_end, H);
-            objective<EVEN, EVEN ? 1 : 0>(S, m0, end_pair, H, val, corr, arg);
-        }
-        // the warp's best; the objective of a non-zero block is positive at its best, so bit patterns compare like values
-        const uint32_t bits = val > 0.f ? __float_as_uint(val) : 0u;
-        const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, bits);
-        const uint32_t who = __ballot_sync(0xFFFFFFFFu, bits == top);
-        if (lane == __ffs(int(who)) - 1) {
-            S.red_val[warp] = top ? val : kNeg;
-            S.red_arg[warp] = uint32_t(tid);
-        }
-    }
-    __syncthreads();
-    bool better = false;
-    uint32_t winner = 0;
-    if (live) {
-        float top = S.red_val[0];
-        winner = S.red_arg[0];
+// Join and objective of one (end pair, class parity); keeps the better of this and what H, val, corr, arg hold.
+template <bool EVEN, int PAR>
+__device__ __forceinline__ void search_end(const EncShared& S, int end_pair, float (&H)[kH], float& val, float& corr, int& arg, int& par) {
+    const bool odd_end = odd_overlap(S.bytes[end_pair]) != 0;
+    const int m0 = EVEN ? (odd_end ? 1 : 0) : 2;  // squared norm = 16 (index + m0)
+    float h[kH], v, c;
+    int n;
+    join_two<EVEN, PAR>(S, end_pair & 7, end_pair >> 3, odd_end, h);
+    objective<EVEN, EVEN ? PAR : PAR ^ 1>(S, m0, end_pair, h, v, c, n);
+    if (v > val) {
+        val = v;
+        corr = c;
+        arg = n;
+        par = PAR;
 #pragma unroll
-        for (int k = 1; k < 4; ++k)
-            if (S.red_val[k] > top) {
-                top = S.red_val[k];
-                winner = S.red_arg[k];
-            }
-        better = top > best_val;  // the same for all threads of the group
-        if (better) {
-            best_val = top;
-            best_even = EVEN;
-            if (uint32_t(tid) == winner) {
-#pragma unroll
-                for (int i = 0; i < kH; ++i) S.win_H[i] = H[i];
-                S.win_G = corr;
-                S.win_arg = arg;
-            }
-        }
+        for (int i = 0; i < kH; ++i) H[i] = h[i];
     }
-    __syncthreads();
-    if (better && warp == 0) trace_join(S, EVEN, int(winner) & 63, int(winner) >> 6, S.win_arg);
-    __syncthreads();
 }
 
 // The file-order word (without the gain bit) of the traced winner; one warp.
@@ -1081,12 +1034,65 @@ k_encode(const float* __restrict__ w, const float* __restrict__ sigma, const Dev
             }
         }
         __syncthreads();
+        const int warp = tid >> 5, lane = tid & 31;
+        if (live) {  // section tables at even parity, two warps per section
+            const int s = tid >> 6, pair = tid & 63;
+            if (s == 1) section_rows<true, true>(S, 1, pair);
+            else section_rows<true, false>(S, s, pair);
+        }
+        __syncthreads();
+        // Join and objective.  Even parity: warps 0..3, thread = (end pair, class parity).  The odd parity has rows of
+        // six entries instead of ten and eleven: warps 4 and 5 do its section tables and both class parities meanwhile.
+        float H[kH];
+        float val = kNeg, corr = kNeg;
+        int arg = 0, par = 0;
+        if (live) {
+            if (warp < 4) {
+                if (warp < 2) search_end<true, 0>(S, tid & 63, H, val, corr, arg, par);
+                else search_end<true, 1>(S, tid & 63, H, val, corr, arg, par);
+            } else {
+                const int pair = tid - 128;
+                section_rows<false, false>(S, 0, pair);
+                section_rows<false, true>(S, 1, pair);
+                section_rows<false, false>(S, 2, pair);
+                asm volatile("bar.sync %0, 64;" ::"r"(1 + group) : "memory");
+                search_end<false, 0>(S, pair, H, val, corr, arg, par);
+                search_end<false, 1>(S, pair, H, val, corr, arg, par);
+            }
+            // the warp's best; the objective of a non-zero block is positive at its best, so bit patterns compare like values
+            const uint32_t bits = val > 0.f ? __float_as_uint(val) : 0u;
+            const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, bits);
+            const uint32_t who = __ballot_sync(0xFFFFFFFFu, bits == top);
+            if (lane == __ffs(int(who)) - 1) {
+                S.red_val[warp] = top ? val : kNeg;
+                S.red_arg[warp] = uint32_t(tid);
+            }
+        }
+        __syncthreads();
         float best_val = kNeg;
-        bool best_even = false;
-        search_parity<false>(S, tid, live, best_val, best_even);
-        search_parity<true>(S, tid, live, best_val, best_even);
+        uint32_t winner = 0;
+        if (live) {  // the odd parity first: it keeps ties
+            best_val = S.red_val[4];
+            winner = S.red_arg[4];
+#pragma unroll
+            for (int k = 5; k < 10; ++k)
+                if (S.red_val[k % 6] > best_val) {
+                    best_val = S.red_val[k % 6];
+                    winner = S.red_arg[k % 6];
+                }
+            if (uint32_t(tid) == winner) {
+#pragma unroll
+                for (int i = 0; i < kH; ++i) S.win_H[i] = H[i];
+                S.win_G = corr;
+                S.win_arg = arg;
+                S.win_par = par;
+            }
+        }
+        const bool best_even = winner < 128u;
+        __syncthreads();
+        if (live && best_val > 0.f && warp == 0) trace_join(S, best_even, int(winner) & 63, S.win_par, S.win_arg);
+        __syncthreads();
         if (live) {  // a warp per section and byte of its pair
-            const int warp = tid >> 5;
             trace_section(S, tab, best_even, warp >> 1, warp & 1);
         }
         __syncthreads();
