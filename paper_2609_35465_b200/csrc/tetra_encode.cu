@@ -203,6 +203,15 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     return d;
 }
 
+// (a0 + b, a1 + b) in one instruction, rounded and flushed like __fadd_rn in this file's build.
+__device__ __forceinline__ void add2(float a0, float a1, float b, float& s0, float& s1) {
+    uint64_t aa, bb, ss;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(aa) : "f"(a0), "f"(a1));
+    asm("mov.b64 %0, {%1, %1};" : "=l"(bb) : "f"(b));
+    asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(ss) : "l"(aa), "l"(bb));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(s0), "=f"(s1) : "l"(ss));
+}
+
 // ---------------------------------------------------------------------------
 // shared memory of a CTA
 // ---------------------------------------------------------------------------
@@ -528,15 +537,20 @@ __device__ __forceinline__ void combine_even(const float* hi, const float (&C)[k
     static_for<0, (kCellCount<CELLS, W> + 1) / 2>([&](auto ti) {
         constexpr int I = 2 * decltype(ti)::value;
         constexpr int KA = kCellNth<CELLS, W, I>, KB = kCellNth<CELLS, W, I + 1>;  // KB = -1: no second cell
-        const float ha = hi[kAtHigh<TABLE, W, KA>];
-        float hb = kNeg;
-        if constexpr (KB >= 0) hb = hi[kAtHigh<TABLE, W, KB>];
+        float sa[LAST + 2], sb[LAST + 2] = {};
+        auto sums = [&](float h, float (&s)[LAST + 2]) {
+#pragma unroll
+            for (int i = 0; i < LAST; i += 2) add2(C[kAtC<V> + i], C[kAtC<V> + i + 1], h, s[i], s[i + 1]);
+            if constexpr (LAST % 2 == 0) s[LAST] = __fadd_rn(h, C[kAtC<V> + LAST]);
+        };
+        sums(hi[kAtHigh<TABLE, W, KA>], sa);
+        if constexpr (KB >= 0) sums(hi[kAtHigh<TABLE, W, KB>], sb);
         static_for<0, KMAX + 1>([&](auto ni) {
             constexpr int N = decltype(ni)::value;
             constexpr bool a = N >= KA && N - KA <= LAST, b = KB >= 0 && N >= KB && N - KB <= LAST;
-            if constexpr (a && b) T[N] = max3(T[N], __fadd_rn(ha, C[kAtC<V> + N - KA]), __fadd_rn(hb, C[kAtC<V> + N - KB]));
-            else if constexpr (a) T[N] = fmaxf(T[N], __fadd_rn(ha, C[kAtC<V> + N - KA]));
-            else if constexpr (b) T[N] = fmaxf(T[N], __fadd_rn(hb, C[kAtC<V> + N - KB]));
+            if constexpr (a && b) T[N] = max3(T[N], sa[N - KA], sb[N - KB]);
+            else if constexpr (a) T[N] = fmaxf(T[N], sa[N - KA]);
+            else if constexpr (b) T[N] = fmaxf(T[N], sb[N - KB]);
         });
     });
 }
@@ -674,19 +688,28 @@ __device__ __forceinline__ void load_row(const float* row, float (&v)[N]) {
     }
 }
 
-// H[i + j + SHIFT] = max(., a[i] + b[j]) for i < NA, j < NB, two candidates per maximum.
+// H[i + j + SHIFT] = max(., a[i] + b[j]) for i < NA, j < NB: two sums per addition, two candidates per maximum.
 template <int NA, int NB, int SHIFT, int LA, int LB, int LH>
 __device__ __forceinline__ void max_plus(const float (&a)[LA], const float (&b)[LB], float (&H)[LH]) {
-    static_for<0, NA + NB - 1>([&](auto ni) {
-        constexpr int n = decltype(ni)::value;
-        constexpr int first = n < NB ? 0 : n - NB + 1, last = n < NA ? n : NA - 1, count = last - first + 1;
-        float v = H[n + SHIFT];
-        static_for<0, count / 2>([&](auto ti) {
-            constexpr int i = first + 2 * decltype(ti)::value;
-            v = max3(v, __fadd_rn(a[i], b[n - i]), __fadd_rn(a[i + 1], b[n - i - 1]));
+    static_for<0, (NB + 1) / 2>([&](auto ji) {
+        constexpr int j = 2 * decltype(ji)::value;
+        constexpr bool two = j + 1 < NB;
+        float s[2][NA + 1];
+#pragma unroll
+        for (int i = 0; i + 1 < NA; i += 2) {
+            add2(a[i], a[i + 1], b[j], s[0][i], s[0][i + 1]);
+            if constexpr (two) add2(a[i], a[i + 1], b[j + 1], s[1][i], s[1][i + 1]);
+        }
+        if constexpr (NA & 1) {
+            s[0][NA - 1] = __fadd_rn(a[NA - 1], b[j]);
+            if constexpr (two) s[1][NA - 1] = __fadd_rn(a[NA - 1], b[j + 1]);
+        }
+        static_for<0, NA + 1>([&](auto ii) {
+            constexpr int i = decltype(ii)::value, n = i + j + SHIFT;
+            if constexpr (two && i > 0 && i < NA) H[n] = max3(H[n], s[0][i], s[1][i - 1]);
+            else if constexpr (i < NA) H[n] = fmaxf(H[n], s[0][i]);
+            else if constexpr (two) H[n] = fmaxf(H[n], s[1][i - 1]);
         });
-        if constexpr (count & 1) v = fmaxf(v, __fadd_rn(a[last], b[n - last]));
-        H[n + SHIFT] = v;
     });
 }
 
