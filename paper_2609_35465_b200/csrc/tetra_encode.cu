@@ -334,37 +334,34 @@ __device__ __forceinline__ void free_step(float (&F)[kMaxW + 1][kMaxK + 1], cons
     });
 }
 
-// Even parity: the tables of (section, half, nibble).  w4: the half's four weights.
-template <bool HIGH, bool MID>
-__device__ __forceinline__ void half_even(const float* w4, int nibble, float* out) {
-    float F[kMaxW + 1][kMaxK + 1], A[kMaxW + 1][kMaxK + 1], B[kMaxW + 1][kMaxK + 1];
+// Even parity: the tables of (section, half, nibble).  w4: the half's four weights; mid: the middle section, whose list
+// has its own limit (M instead of 0 and 1; what the other limits give is not read there).  One copy of this code for
+// all sections: straight-line code is fetched more slowly than it runs.
+template <bool HIGH>
+__device__ __forceinline__ void half_even(const float* w4, int nibble, bool mid, float* out) {
+    float F[kMaxW + 1][kMaxK + 1], A[kMaxW + 1][kMaxK + 1], B[kMaxW + 1][kMaxK + 1], M[kMaxW + 1][kMaxK + 1];
     F[0][0] = 0.f;
     A[0][0] = 0.f;   // only the "up to" tables read it
     B[0][0] = 0.f;
-    float hs0 = 0.f, hs1 = 0.f;  // correlations of the limits' high halves
+    M[0][0] = 0.f;
+    float hs0 = 0.f, hs1 = 0.f, hsm = 0.f;  // correlations of the limits' high halves
     static_for<0, 4>([&](auto ji) {
         constexpr int J = decltype(ji)::value;
-        [[maybe_unused]] constexpr int D0 = kLimit0.hi[J], D1 = kLimit1.hi[J], DM = kLimitM.hi[J];  // digits of the limits' high halves
         const int c = (nibble >> J) & 1;
         float a[5];
         products_even(w4[J], c, a);
         if constexpr (HIGH) {
-            if constexpr (MID) {
-                prefix_step<J, kLimitM.hi[J], kLessM>(F, A, a, c);
-                hs0 = __fadd_rn(hs0, a[DM]);
-            } else {
-                prefix_step<J, kLimit0.hi[J], kLess0>(F, A, a, c);
-                prefix_step<J, kLimit1.hi[J], kLess1>(F, B, a, c);
-                hs0 = __fadd_rn(hs0, a[D0]);
-                hs1 = __fadd_rn(hs1, a[D1]);
-            }
+            constexpr int D0 = kLimit0.hi[J], D1 = kLimit1.hi[J], DM = kLimitM.hi[J];  // digits of the limits' high halves
+            prefix_step<J, kLimit0.hi[J], kLess0>(F, A, a, c);
+            prefix_step<J, kLimit1.hi[J], kLess1>(F, B, a, c);
+            prefix_step<J, kLimitM.hi[J], kLessM>(F, M, a, c);
+            hs0 = __fadd_rn(hs0, a[D0]);
+            hs1 = __fadd_rn(hs1, a[D1]);
+            hsm = __fadd_rn(hsm, a[DM]);
         } else {
-            if constexpr (MID) {
-                prefix_step<J, kLimitM.lo[J], kUpToM>(F, A, a, c);
-            } else {
-                prefix_step<J, kLimit0.lo[J], kUpTo0>(F, A, a, c);
-                prefix_step<J, kLimit1.lo[J], kUpTo1>(F, B, a, c);
-            }
+            prefix_step<J, kLimit0.lo[J], kUpTo0>(F, A, a, c);
+            prefix_step<J, kLimit1.lo[J], kUpTo1>(F, B, a, c);
+            prefix_step<J, kLimitM.lo[J], kUpToM>(F, M, a, c);
         }
         free_step<J>(F, a, c);
     });
@@ -375,15 +372,15 @@ __device__ __forceinline__ void half_even(const float* w4, int nibble, float* ou
                 constexpr int K = decltype(ki)::value;
                 if constexpr (W <= 9 && kFree.v[4][W][K]) out[kAtH<W, K>] = F[W][K];
                 if constexpr (W <= 10 && kLess0orM.v[4][W][K]) {
-                    constexpr bool have = MID ? kLessM.v[4][W][K] : kLess0.v[4][W][K];
-                    float v = kNeg;
-                    if constexpr (have) v = A[W][K];
-                    out[kAtA<W, K>] = v;
+                    float v0 = kNeg, vm = kNeg;
+                    if constexpr (kLess0.v[4][W][K]) v0 = A[W][K];
+                    if constexpr (kLessM.v[4][W][K]) vm = M[W][K];
+                    out[kAtA<W, K>] = mid ? vm : v0;
                 }
-                if constexpr (!MID && kLess1.v[4][W][K]) out[kAtB<W, K>] = B[W][K];
+                if constexpr (kLess1.v[4][W][K]) out[kAtB<W, K>] = B[W][K];
             });
         });
-        out[kOffHs] = hs0;
+        out[kOffHs] = mid ? hsm : hs0;
         out[kOffHs + 1] = hs1;
     } else {
         static_for<0, 2>([&](auto pi) {
@@ -402,15 +399,14 @@ __device__ __forceinline__ void half_even(const float* w4, int nibble, float* ou
         static_for<0, 5>([&](auto ki) {
             constexpr int K = decltype(ki)::value;
             if constexpr (K < 3) {
-                float v = kNeg;
-                if constexpr (MID ? kUpToM.v[4][2][K] : kUpTo0.v[4][2][K]) v = A[2][K];
-                out[kOffRes0 + K] = v;
+                float v0 = kNeg, vm = kNeg;
+                if constexpr (kUpTo0.v[4][2][K]) v0 = A[2][K];
+                if constexpr (kUpToM.v[4][2][K]) vm = M[2][K];
+                out[kOffRes0 + K] = mid ? vm : v0;
             }
-            if constexpr (!MID) {
-                float v = kNeg;
-                if constexpr (kUpTo1.v[4][5][K]) v = B[5][K];
-                out[kOffRes1 + K] = v;
-            }
+            float v1 = kNeg;
+            if constexpr (kUpTo1.v[4][5][K]) v1 = B[5][K];
+            out[kOffRes1 + K] = v1;
         });
     }
 }
@@ -1033,27 +1029,22 @@ k_encode(const float* __restrict__ w, const float* __restrict__ sigma, const Dev
         for (int j = 0; j < 24; ++j) wn2 = fmaf(S.w[j], S.w[j], wn2);
         const bool live = wn2 != 0.f;  // a zero block encodes as the all-zero word
         if (live) {
-            // half tables, lane = section (0 or 2) and nibble, or nibble of the middle section: warps 0 and 1 the high
-            // and low halves of the outer sections at even parity, warps 2 and 3 those of the middle one, warps 4 and
-            // 5 the odd parity
-            const int nibble = tid & 15, outer = (tid & 16) ? 2 : 0;
-            float *lo = S.lo[outer] + nibble * kLoStride, *hi = S.hi[outer] + nibble * kHiStride;
-            float *lo_odd = S.lo_odd[outer] + nibble * kOddLoStride, *hi_odd = S.hi_odd[outer] + nibble * kOddHiStride;
-            const float* wo = S.w + 8 * outer;
-            switch (tid >> 5) {
-                case 0: half_even<true, false>(wo + 4, nibble, hi); break;
-                case 1: half_even<false, false>(wo, nibble, lo); break;
-                case 2: if (outer == 0) half_even<true, true>(S.w + 12, nibble, S.hi[1] + nibble * kHiStride); break;
-                case 3: if (outer == 0) half_even<false, true>(S.w + 8, nibble, S.lo[1] + nibble * kLoStride); break;
-                case 4:
-                    half_odd<true, false>(wo + 4, nibble, hi_odd);
-                    half_odd<false, false>(wo, nibble, lo_odd);
-                    break;
-                default:
-                    if (outer == 0) {
-                        half_odd<true, true>(S.w + 12, nibble, S.hi_odd[1] + nibble * kOddHiStride);
-                        half_odd<false, true>(S.w + 8, nibble, S.lo_odd[1] + nibble * kOddLoStride);
-                    }
+            // half tables, a thread per (section, nibble): warps 0 and 1 the high halves at even parity, 2 and 3 the low
+            // ones, 4 and 5 the odd parity (warp 4 the outer sections, warp 5 the middle one)
+            const int nibble = tid & 15;
+            if (tid < 128) {
+                const int s = (tid & 63) >> 4;
+                if (s < 3) {
+                    if (tid < 64) half_even<true>(S.w + 8 * s + 4, nibble, s == 1, S.hi[s] + nibble * kHiStride);
+                    else half_even<false>(S.w + 8 * s, nibble, s == 1, S.lo[s] + nibble * kLoStride);
+                }
+            } else if (tid < 160) {
+                const int s = (tid & 16) ? 2 : 0;
+                half_odd<true, false>(S.w + 8 * s + 4, nibble, S.hi_odd[s] + nibble * kOddHiStride);
+                half_odd<false, false>(S.w + 8 * s, nibble, S.lo_odd[s] + nibble * kOddLoStride);
+            } else if ((tid & 16) == 0) {
+                half_odd<true, true>(S.w + 12, nibble, S.hi_odd[1] + nibble * kOddHiStride);
+                half_odd<false, true>(S.w + 8, nibble, S.lo_odd[1] + nibble * kOddLoStride);
             }
         }
         __syncthreads();
