@@ -21,14 +21,18 @@
 //     codewords are exactly the triples (alpha, xi), (beta, xi), (alpha + beta, xi) with any complements.  So the
 //     sections' tables hold 64 rows, and joining sections 1 and 2 is, for every xi, an XOR convolution over eight
 //     alphas.  At even parity r = 8 exactly where |h(alpha) & h'(xi)| is odd, a bilinear form.
-// One CTA of 192 threads works on one block at a time: half tables (a thread per section, half and nibble; both
-// parities at once), section tables (a thread per section and byte pair), join and objective (a thread per end
-// state and class parity), and, when a parity improves on the other, the winner traced back through the same
-// tables by one warp per section.  Every sum is formed in the same order wherever it is needed, so the trace
-// matches floats exactly.
+// 192 threads work on one block of weights: half tables (a thread per section, half and nibble; both parities), section
+// tables (a thread per section and byte pair), join and objective (a thread per end state and class parity: four warps
+// the even parity, two the odd one), then the winner is traced back through the same tables, a warp per section and
+// byte of its pair.  Every sum is formed in the same order wherever it is needed, so the trace matches floats exactly.
 //
-// Bound by instruction issue (adds and maxima of the section tables and the join; all tables sit in shared
-// memory).  On 24,576 Gaussian blocks: see the figures at launch_encode.
+// All of it is straight-line code on registers, some 8,000 instructions a block, and what it ran into was the
+// instruction fetch, not the arithmetic: a CTA therefore takes three blocks in step (one SM), and code that differs
+// between sections only by a constant exists once.  24,576 Gaussian blocks: 61.2 ms by scanning the rows of the
+// lists in shared memory; 4.9 ms with these tables and one block per CTA; 2.3 ms three blocks in step; 1.86 ms with
+// two candidates per maximum and the trace once per block; 1.65 ms with the odd parity beside the even one; 1.55 ms
+// with packed additions; 1.45 ms with one copy of the half-table code (37,000 warp-instructions a block, issue slots
+// 53 % busy; what is left is barriers between the phases, 2 of 8 stall cycles per instruction).
 #include <cuda_runtime.h>
 
 #include <cstdint>
