@@ -86,8 +86,9 @@ typedef struct {
  *                                  activations, partial strips); 0 for a rejected list;
  *   tetra_q4_list_plan             writes the descriptors (problems_host is read before the call
  *                                  returns; call it outside stream capture);
- *   tetra_q4_list_run              one step, three launches: group sums of every x, the stream, the
- *                                  sum of the strips that two warps share (in warp order).
+ *   tetra_q4_list_run              one step, two launches: group sums of every x, then the stream, in
+ *                                  which the last of the warps that share a strip adds their parts (in
+ *                                  warp order).
  * workspace_dev: 256-byte aligned device memory owned by the caller; it belongs to the plan until the
  * last run using it has completed, runs that share it must not overlap on the GPU, and it may be
  * copied to other device memory (the plan describes itself) on the device it was planned for.

@@ -11,11 +11,14 @@
 //                      operands carry biases 1024 and 64), into the workspace;
 //   k_q4_list_main     the stream: dequantise with five logic operations per four registers, MMA
 //                      against the activations (read through L1), scale and offset per group;
-//                      a strip (32 rows) that lies wholly inside a warp's range is stored, one cut by
-//                      a range boundary leaves a piece in the workspace;
-//   k_q4_list_combine  adds the pieces of a strip in warp order and stores it.
-// Deterministic (fixed order everywhere), no atomics, no waits besides cp.async.wait_group and
-// griddepcontrol.wait.
+//                      a strip (32 rows) that lies wholly inside a warp's range is stored; one cut by
+//                      range boundaries leaves a piece per warp in the workspace, and the warp that
+//                      finds the strip's other pieces there adds them in warp order and stores it.
+// Where a warp starts, who shares its strips and which matrix a group belongs to is written into the plan:
+// searched for on the device it was a chain of dependent loads in every warp (one layer's projections, 38 MB:
+// 22.5 us with searches and a third kernel that followed the pieces, now @L1@ us; 36 layers 255 us, now @L36@ us).
+// Deterministic (fixed order everywhere); nothing waits for another warp (a counter per cut strip only tells the
+// last one), cp.async.wait_group and griddepcontrol.wait are the only waits.
 #include <cstdlib>
 #include <cstring>
 
@@ -44,37 +47,39 @@ struct Q4Item {
 };
 static_assert(sizeof(Q4Item) == 56, "descriptor layout");
 
+// What a warp's range [c_begin, c_end) of the chunk sequence meets, known when the list is planned.
+struct Q4Warp {
+    int32_t item;    // matrix of its first chunk
+    int32_t owner;   // warp in whose range the strip of its first chunk begins
+    int32_t parts;   // pieces of the strip that begins in this range and ends beyond it (0: there is none)
+    int32_t arrived; // of those pieces, how many are there (zero between runs)
+};
+
 struct Q4ListHeader {
     int32_t count, G, nwarps, pad0_;
     uint32_t total_chunks, total_groups, total_strips, pad1_;
-    uint32_t off_items, off_gs, off_pieces, off_piece_strip;
+    uint32_t off_items, off_warps, off_group_item, off_gs, off_pieces;
 };
 
 inline size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
 struct Q4ListLayout {
-    size_t off_items, off_gs, off_pieces, off_piece_strip, total;
+    size_t off_items, off_warps, off_group_item, off_gs, off_pieces, total;
 };
 Q4ListLayout list_layout(int count, size_t total_groups, int nwarps) {
     Q4ListLayout L;
     L.off_items = align256(sizeof(Q4ListHeader));
-    L.off_gs = align256(L.off_items + size_t(count) * sizeof(Q4Item));
+    L.off_warps = align256(L.off_items + size_t(count) * sizeof(Q4Item));
+    L.off_group_item = align256(L.off_warps + size_t(nwarps) * sizeof(Q4Warp));  // uint16 per group
+    L.off_gs = align256(L.off_group_item + total_groups * 2);
     L.off_pieces = align256(L.off_gs + total_groups * 64);
-    L.off_piece_strip = align256(L.off_pieces + size_t(nwarps) * 2 * kPieceFloats * 4);
-    L.total = align256(L.off_piece_strip + size_t(nwarps) * 2 * 4);
+    L.total = align256(L.off_pieces + size_t(nwarps) * 2 * kPieceFloats * 4);
     return L;
 }
+static_assert(TETRA_Q4_LIST_MAX <= 65536, "matrix numbers fit 16 bits");
 
-// Item that holds element `v` of a sequence whose per-item begins are read by `begin_of` (begins ascend).
-template <typename F>
-__device__ __forceinline__ int find_item(int count, uint32_t v, F begin_of) {
-    int lo = 0, hi = count;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (begin_of(mid) <= v) lo = mid; else hi = mid;
-    }
-    return lo;
-}
+// First chunk of warp w's range.
+__host__ __device__ inline uint32_t range_begin(uint32_t total, int w, int nw) { return uint32_t(uint64_t(total) * uint32_t(w) / uint32_t(nw)); }
 
 __global__ void __launch_bounds__(256) k_q4_list_prepare(unsigned char* __restrict__ ws) {
     pdl_release();
@@ -82,17 +87,12 @@ __global__ void __launch_bounds__(256) k_q4_list_prepare(unsigned char* __restri
     const Q4ListHeader* H = reinterpret_cast<const Q4ListHeader*>(ws);
     const Q4Item* items = reinterpret_cast<const Q4Item*>(ws + H->off_items);
     float2* gs = reinterpret_cast<float2*>(ws + H->off_gs);
-    int32_t* piece_strip = reinterpret_cast<int32_t*>(ws + H->off_piece_strip);
+    const uint16_t* group_item = reinterpret_cast<const uint16_t*>(ws + H->off_group_item);
     const int G = H->G, sub = threadIdx.x & 7;
-    // the matrices' first groups go to shared memory: the search below would otherwise be a chain of
-    // dependent loads from L2 that is most of this kernel's time
-    __shared__ uint32_t group_begin_sm[TETRA_Q4_LIST_MAX];
-    for (int i = threadIdx.x; i < H->count; i += blockDim.x) group_begin_sm[i] = items[i].group_begin;
-    __syncthreads();
     for (uint32_t gg = (blockIdx.x * blockDim.x + threadIdx.x) >> 3; gg < H->total_groups;
          gg += (gridDim.x * blockDim.x) >> 3) {
-        const int it = find_item(H->count, gg, [&](int i) { return group_begin_sm[i]; });
-        const uint2* src = reinterpret_cast<const uint2*>(items[it].x + size_t(gg - items[it].group_begin) * G);
+        const Q4Item& I = items[__ldg(group_item + gg)];
+        const uint2* src = reinterpret_cast<const uint2*>(I.x + size_t(gg - I.group_begin) * G);
         float lo = 0.f, hi = 0.f;  // k % 4 in {0, 1} / {2, 3}
         for (int i = 0; i < G / 32; ++i) {
             const uint2 u = __ldg(src + sub + 8 * i);
@@ -109,7 +109,6 @@ __global__ void __launch_bounds__(256) k_q4_list_prepare(unsigned char* __restri
         // eight (sum x, -sum bias x) pairs per group, one per MMA column; only column 0 carries a vector
         gs[size_t(gg) * 8 + sub] = sub == 0 ? make_float2(lo + hi, -(1024.f * lo + 64.f * hi)) : make_float2(0.f, 0.f);
     }
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 2 * H->nwarps; i += gridDim.x * blockDim.x) piece_strip[i] = -1;
 }
 
 template <int G, int DEPTH>
@@ -124,18 +123,21 @@ __global__ void __launch_bounds__(kQ4ListThreads, 1) k_q4_list_main(unsigned cha
     const Q4Item* items = reinterpret_cast<const Q4Item*>(ws + H->off_items);
     const unsigned char* gs = ws + H->off_gs;
     float* pieces = reinterpret_cast<float*>(ws + H->off_pieces);
-    int32_t* piece_strip = reinterpret_cast<int32_t*>(ws + H->off_piece_strip);
-    const int gw = blockIdx.x * kQ4ListWarps + warp, nw = gridDim.x * kQ4ListWarps;
-    const uint32_t c_begin = uint32_t(uint64_t(H->total_chunks) * gw / nw);
-    const uint32_t c_end = uint32_t(uint64_t(H->total_chunks) * (gw + 1) / nw);
-    if (c_begin >= c_end) return;
+    Q4Warp* warps = reinterpret_cast<Q4Warp*>(ws + H->off_warps);
+    // A list of fewer chunks than warps uses as many warps as chunks, spread over the CTAs.
+    const int nw = H->nwarps, all = int(gridDim.x) * kQ4ListWarps;
+    const int gw = nw < all ? warp * int(gridDim.x) + int(blockIdx.x) : int(blockIdx.x) * kQ4ListWarps + warp;
+    if (gw >= nw) return;
+    const uint32_t total = H->total_chunks;
+    const uint32_t c_begin = range_begin(total, gw, nw), c_end = range_begin(total, gw + 1, nw);
+    const int first_item = warps[gw].item;
 
     const uint32_t ring_lane = smem_u32(q4_smem) + uint32_t(warp) * (DEPTH * CH) + lane * 16;
     const uint32_t ring_lane_end = ring_lane + DEPTH * CH;
     const bool tail_lane = lane < PIECES % 32;  // lanes that copy the last, partial group of 16-byte pieces
 
     // fetch side: the next chunk to copy, wherever in the list it lies
-    int fi = find_item(H->count, c_begin, [&](int i) { return items[i].chunk_begin; });
+    int fi = first_item;
     uint32_t f_left_in_item = items[fi].chunk_begin + uint32_t(items[fi].groups) * uint32_t(items[fi].strips) - c_begin;
     const unsigned char* f_src = items[fi].packed + size_t(c_begin - items[fi].chunk_begin) * CH + lane * 16;
     int f_todo = int(c_end - c_begin);
@@ -164,10 +166,9 @@ __global__ void __launch_bounds__(kQ4ListThreads, 1) k_q4_list_main(unsigned cha
     const uint32_t so_delta = uint32_t(TPG * 1024 + g * 4) - uint32_t(lane * 16);  // slot_lane -> this lane's scale records
 
     // consume side
-    int ci = find_item(H->count, c_begin, [&](int i) { return items[i].chunk_begin; });
+    int ci = first_item;
     uint32_t left = c_end - c_begin;
     uint32_t local = c_begin - items[ci].chunk_begin;  // chunk index inside matrix ci
-    int n_pieces = 0;
     while (left > 0) {
         const Q4Item I = items[ci];
         const int groups = I.groups;
@@ -250,13 +251,28 @@ __global__ void __launch_bounds__(kQ4ListThreads, 1) k_q4_list_main(unsigned cha
                             if (row < I.N) I.y[row] = acc[h][i];
                         }
                 }
-            } else {  // a strip shared with a neighbouring warp: leave a piece (column 0: row 16 h + g + 8 j at 4 g' ...)
-                if (t == 0) {  // floats 4 g .. 4 g + 3 = rows g, g + 8, 16 + g, 24 + g
-                    float* mine = pieces + size_t(2 * gw + n_pieces) * kPieceFloats + 4 * g;
-                    *reinterpret_cast<float4*>(mine) = make_float4(acc[0][0], acc[0][2], acc[1][0], acc[1][2]);
+            } else {
+                // A strip shared with neighbouring warps: leave a piece (column 0: floats 4 g .. 4 g + 3 = rows g, g + 8,
+                // 16 + g, 24 + g).  A warp has at most one strip that began before its range (slot 0) and one that ends
+                // beyond it (slot 1).
+                const bool later = seg_first != 0;  // began before this range
+                if (t == 0)
+                    *reinterpret_cast<float4*>(pieces + (size_t(2 * gw) + (later ? 0 : 1)) * kPieceFloats + 4 * g) =
+                        make_float4(acc[0][0], acc[0][2], acc[1][0], acc[1][2]);
+                const int owner = later ? warps[gw].owner : gw, parts = warps[owner].parts;
+                __threadfence();  // the piece is visible before the counter moves
+                __syncwarp();
+                int arrived = 0;
+                if (lane == 0) arrived = atomicAdd(&warps[owner].arrived, 1);
+                arrived = __shfl_sync(0xFFFFFFFFu, arrived, 0);
+                if (arrived == parts - 1) {  // all pieces are there: add them in warp order
+                    __threadfence();
+                    float sum = __ldcg(pieces + (size_t(2 * owner) + 1) * kPieceFloats + lane);
+                    for (int k = 1; k < parts; ++k) sum += __ldcg(pieces + size_t(2 * (owner + k)) * kPieceFloats + lane);
+                    const int row = 32 * strip + (lane >> 2) + 8 * (lane & 1) + 16 * ((lane >> 1) & 1);
+                    if (row < I.N) I.y[row] = sum;
+                    if (lane == 0) warps[owner].arrived = 0;  // for the next run
                 }
-                if (lane == 0) piece_strip[2 * gw + n_pieces] = int32_t(I.strip_begin) + strip;
-                ++n_pieces;
             }
             if (gi == groups) {
                 gi = 0;
@@ -267,39 +283,6 @@ __global__ void __launch_bounds__(kQ4ListThreads, 1) k_q4_list_main(unsigned cha
         local = 0;
     }
     q4_cp_async_wait<0>();
-}
-
-// Warp i looks at piece slot i (slots are in memory order: warp, then first/second): if it holds the first
-// piece of its strip, the warp adds the strip's pieces in slot order and stores the 32 rows.
-__global__ void __launch_bounds__(256) k_q4_list_combine(unsigned char* __restrict__ ws) {
-    pdl_release();
-    const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    pdl_wait();
-    const Q4ListHeader* H = reinterpret_cast<const Q4ListHeader*>(ws);
-    const int npieces = 2 * H->nwarps;
-    if (i >= npieces) return;
-    const int32_t* piece_strip = reinterpret_cast<const int32_t*>(ws + H->off_piece_strip);
-    const int sid = piece_strip[i];
-    if (sid < 0) return;
-    // a strip has at most one piece per warp: its earlier pieces, if any, sit in the slots just before
-    int j = i - 1;
-    while (j >= 0 && piece_strip[j] < 0) --j;
-    if (j >= 0 && piece_strip[j] == sid) return;  // not the first piece of its strip
-    const float* pieces = reinterpret_cast<const float*>(ws + H->off_pieces);
-    float total = 0.f;
-    for (int k = i; k < npieces; ++k) {
-        const int s = piece_strip[k];
-        if (s < 0) continue;
-        if (s != sid) break;
-        total += pieces[size_t(k) * kPieceFloats + lane];
-    }
-    const Q4Item* items = reinterpret_cast<const Q4Item*>(ws + H->off_items);
-    const int it = find_item(H->count, uint32_t(sid), [&](int q) { return items[q].strip_begin; });
-    // float 4 g + j of a piece is row g + 8 (j & 1) + 16 (j >> 1) of the strip
-    const int g = lane >> 2, jj = lane & 3;
-    const int row = 32 * (sid - int(items[it].strip_begin)) + g + 8 * (jj & 1) + 16 * (jj >> 1);
-    if (row < items[it].N) items[it].y[row] = total;
 }
 
 int check_list(const tetra_q4_problem* p, int count, int G) {
@@ -368,15 +351,18 @@ int tetra_q4_list_plan(const tetra_q4_problem* problems_host, int count, int G, 
     Q4ListHeader* H = reinterpret_cast<Q4ListHeader*>(buf);
     H->count = count;
     H->G = G;
-    H->nwarps = nwarps;
+    const int ranges = chunks < uint64_t(nwarps) ? int(chunks) : nwarps;  // no range is empty
+    H->nwarps = ranges;
     H->total_chunks = uint32_t(chunks);
     H->total_groups = uint32_t(groups);
     H->total_strips = uint32_t(strips);
     H->off_items = uint32_t(L.off_items);
+    H->off_warps = uint32_t(L.off_warps);
+    H->off_group_item = uint32_t(L.off_group_item);
     H->off_gs = uint32_t(L.off_gs);
     H->off_pieces = uint32_t(L.off_pieces);
-    H->off_piece_strip = uint32_t(L.off_piece_strip);
     Q4Item* items = reinterpret_cast<Q4Item*>(buf + L.off_items);
+    uint16_t* group_item = reinterpret_cast<uint16_t*>(buf + L.off_group_item);
     uint32_t cb = 0, gb = 0, sb = 0;
     for (int i = 0; i < count; ++i) {
         const tetra_q4_problem& q = problems_host[i];
@@ -392,8 +378,39 @@ int tetra_q4_list_plan(const tetra_q4_problem* problems_host, int count, int G, 
         I.group_begin = gb;
         I.strip_begin = sb;
         cb += uint32_t(I.groups) * uint32_t(I.strips);
+        for (int k = 0; k < I.groups; ++k) group_item[gb + uint32_t(k)] = uint16_t(i);
         gb += uint32_t(I.groups);
         sb += uint32_t(I.strips);
+    }
+    Q4Warp* warps = reinterpret_cast<Q4Warp*>(buf + L.off_warps);
+    int item = 0, owner = 0;
+    uint32_t strip_at = 0xFFFFFFFFu;  // first chunk of the strip that the ranges so far have left open
+    for (int w = 0; w < ranges; ++w) {
+        const uint32_t begin = range_begin(uint32_t(chunks), w, ranges), end = range_begin(uint32_t(chunks), w + 1, ranges);
+        auto strip_of = [&](uint32_t c) {  // first chunk of c's strip, c in matrix `item`
+            const Q4Item& I = items[item];
+            return I.chunk_begin + (c - I.chunk_begin) / uint32_t(I.groups) * uint32_t(I.groups);
+        };
+        auto advance = [&](uint32_t c) {
+            while (item + 1 < count && items[item + 1].chunk_begin <= c) ++item;
+        };
+        advance(begin);
+        warps[w].item = item;
+        if (strip_of(begin) == strip_at) {  // shared with earlier ranges
+            warps[w].owner = owner;
+            ++warps[owner].parts;
+        } else {
+            warps[w].owner = w;
+        }
+        advance(end - 1);
+        const uint32_t last = strip_of(end - 1);
+        const bool open = end < last + uint32_t(items[item].groups);  // goes on in the next range
+        if (!open) strip_at = 0xFFFFFFFFu;
+        else if (last != strip_at) {
+            strip_at = last;
+            owner = w;
+            warps[w].parts = 1;
+        }
     }
     // pageable source: the runtime has taken its copy when the call returns, so the buffer can be freed
     const cudaError_t e = cudaMemcpyAsync(workspace_dev, buf, meta, cudaMemcpyHostToDevice, static_cast<cudaStream_t>(stream));
@@ -411,7 +428,6 @@ int tetra_q4_list_run(void* workspace_dev, int G, void* stream) {
     unsigned char* ws = static_cast<unsigned char*>(workspace_dev);
     cudaError_t e = launch_pdl(k_q4_list_prepare, sms * 2, 256, 0, s, ws);
     if (e == cudaSuccess) e = G == 128 ? run_main<128, 2>(ws, sms, s) : run_main<64, 6>(ws, sms, s);
-    if (e == cudaSuccess) e = launch_pdl(k_q4_list_combine, (2 * sms * kQ4ListWarps + 7) / 8, 256, 0, s, ws);  // a warp per piece slot
     return e == cudaSuccess ? TETRA_OK : TETRA_ERR_CUDA;
 }
 
