@@ -7,18 +7,19 @@
 // matrices form one sequence in memory order; every warp of a persistent grid owns a contiguous
 // range of it and streams it through its cp.async ring without ever draining it between matrices,
 // and no warp waits for another:
-//   k_q4_list_prepare  per group of every matrix: sum of x and minus the sum of bias_k x_k (the MMA
-//                      operands carry biases 1024 and 64), into the workspace;
-//   k_q4_list_main     the stream: dequantise with five logic operations per four registers, MMA
-//                      against the activations (read through L1), scale and offset per group;
-//                      a strip (32 rows) that lies wholly inside a warp's range is stored; one cut by
-//                      range boundaries leaves a piece per warp in the workspace, and the warp that
-//                      finds the strip's other pieces there adds them in warp order and stores it.
-// Where a warp starts, who shares its strips and which matrix a group belongs to is written into the plan:
-// searched for on the device it was a chain of dependent loads in every warp (one layer's projections, 38 MB:
-// 22.5 us with searches and a third kernel that followed the pieces, now @L1@ us; 36 layers 255 us, now @L36@ us).
+// The rest is one kernel:
+//   * per group of the activations the sum of x and minus the sum of bias_k x_k (the MMA operands carry biases
+//     1024 and 64) are made by each CTA for the few matrices its warps meet, in shared memory, while the first
+//     chunks are on their way; that also brings the activations into L1, where the warps read them;
+//   * the stream: dequantise with five logic operations per four registers, MMA against the activations, scale
+//     and offset per group; a strip (32 rows) that lies wholly inside a warp's range is stored; one cut by range
+//     boundaries leaves a piece per warp in the workspace, and the warp that finds the strip's other pieces there
+//     adds them in warp order and stores it.
+// Where a warp starts and who shares its strips is written into the plan: searched for on the device it was a chain
+// of dependent loads in every warp.  (One layer's projections, 38 MB: 22.5 us with searches, a kernel before this one
+// for the group sums and one after it for the pieces; now @L1@ us.  36 layers: 255 us, now @L36@ us.)
 // Deterministic (fixed order everywhere); nothing waits for another warp (a counter per cut strip only tells the
-// last one), cp.async.wait_group and griddepcontrol.wait are the only waits.
+// last one); CTA barriers, cp.async.wait_group and griddepcontrol.wait are the only waits.
 #include <cstdlib>
 #include <cstring>
 
@@ -58,57 +59,48 @@ struct Q4Warp {
 struct Q4ListHeader {
     int32_t count, G, nwarps, pad0_;
     uint32_t total_chunks, total_groups, total_strips, pad1_;
-    uint32_t off_items, off_warps, off_group_item, off_gs, off_pieces;
+    uint32_t off_items, off_warps, off_pieces;
 };
 
 inline size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
 struct Q4ListLayout {
-    size_t off_items, off_warps, off_group_item, off_gs, off_pieces, total;
+    size_t off_items, off_warps, off_pieces, total;
 };
-Q4ListLayout list_layout(int count, size_t total_groups, int nwarps) {
+Q4ListLayout list_layout(int count, int nwarps) {
     Q4ListLayout L;
     L.off_items = align256(sizeof(Q4ListHeader));
     L.off_warps = align256(L.off_items + size_t(count) * sizeof(Q4Item));
-    L.off_group_item = align256(L.off_warps + size_t(nwarps) * sizeof(Q4Warp));  // uint16 per group
-    L.off_gs = align256(L.off_group_item + total_groups * 2);
-    L.off_pieces = align256(L.off_gs + total_groups * 64);
+    L.off_pieces = align256(L.off_warps + size_t(nwarps) * sizeof(Q4Warp));
     L.total = align256(L.off_pieces + size_t(nwarps) * 2 * kPieceFloats * 4);
     return L;
 }
-static_assert(TETRA_Q4_LIST_MAX <= 65536, "matrix numbers fit 16 bits");
 
 // First chunk of warp w's range.
 __host__ __device__ inline uint32_t range_begin(uint32_t total, int w, int nw) { return uint32_t(uint64_t(total) * uint32_t(w) / uint32_t(nw)); }
 
-__global__ void __launch_bounds__(256) k_q4_list_prepare(unsigned char* __restrict__ ws) {
-    pdl_release();
-    pdl_wait();  // the activations may come from the preceding kernel
-    const Q4ListHeader* H = reinterpret_cast<const Q4ListHeader*>(ws);
-    const Q4Item* items = reinterpret_cast<const Q4Item*>(ws + H->off_items);
-    float2* gs = reinterpret_cast<float2*>(ws + H->off_gs);
-    const uint16_t* group_item = reinterpret_cast<const uint16_t*>(ws + H->off_group_item);
-    const int G = H->G, sub = threadIdx.x & 7;
-    for (uint32_t gg = (blockIdx.x * blockDim.x + threadIdx.x) >> 3; gg < H->total_groups;
-         gg += (gridDim.x * blockDim.x) >> 3) {
-        const Q4Item& I = items[__ldg(group_item + gg)];
-        const uint2* src = reinterpret_cast<const uint2*>(I.x + size_t(gg - I.group_begin) * G);
-        float lo = 0.f, hi = 0.f;  // k % 4 in {0, 1} / {2, 3}
-        for (int i = 0; i < G / 32; ++i) {
-            const uint2 u = __ldg(src + sub + 8 * i);
-            const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
-            const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
-            lo += a.x + a.y;
-            hi += b.x + b.y;
-        }
+constexpr int kQ4ListSums = 4096;  // groups whose sums a CTA holds; a CTA that meets more makes them chunk by chunk
+
+// (sum x, minus the sum of bias_k x_k) of one group, bias 1024 for k % 4 in {0, 1} and 64 for {2, 3}; LANES consecutive
+// lanes each hold every LANES-th four activations, all of them get the result.
+template <int G, int LANES>
+__device__ __forceinline__ float2 group_sums(const __half* x, int sub) {
+    const uint2* src = reinterpret_cast<const uint2*>(x);
+    float lo = 0.f, hi = 0.f;
 #pragma unroll
-        for (int o = 4; o >= 1; o >>= 1) {
-            lo += __shfl_xor_sync(0xFFFFFFFFu, lo, o);
-            hi += __shfl_xor_sync(0xFFFFFFFFu, hi, o);
-        }
-        // eight (sum x, -sum bias x) pairs per group, one per MMA column; only column 0 carries a vector
-        gs[size_t(gg) * 8 + sub] = sub == 0 ? make_float2(lo + hi, -(1024.f * lo + 64.f * hi)) : make_float2(0.f, 0.f);
+    for (int i = 0; i < G / 4; i += LANES) {
+        const uint2 u = G / 4 >= LANES || sub < G / 4 ? __ldg(src + sub + i) : make_uint2(0u, 0u);
+        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
+        const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
+        lo += a.x + a.y;
+        hi += b.x + b.y;
     }
+#pragma unroll
+    for (int o = LANES / 2; o >= 1; o >>= 1) {
+        lo += __shfl_xor_sync(0xFFFFFFFFu, lo, o);
+        hi += __shfl_xor_sync(0xFFFFFFFFu, hi, o);
+    }
+    return make_float2(lo + hi, -(1024.f * lo + 64.f * hi));
 }
 
 template <int G, int DEPTH>
@@ -121,16 +113,16 @@ __global__ void __launch_bounds__(kQ4ListThreads, 1) k_q4_list_main(unsigned cha
     // the plan (written once, long before) and the weights do not depend on the preceding kernel
     const Q4ListHeader* H = reinterpret_cast<const Q4ListHeader*>(ws);
     const Q4Item* items = reinterpret_cast<const Q4Item*>(ws + H->off_items);
-    const unsigned char* gs = ws + H->off_gs;
+    float2* sums = reinterpret_cast<float2*>(q4_smem + size_t(kQ4ListWarps) * DEPTH * CH);
     float* pieces = reinterpret_cast<float*>(ws + H->off_pieces);
     Q4Warp* warps = reinterpret_cast<Q4Warp*>(ws + H->off_warps);
     // A list of fewer chunks than warps uses as many warps as chunks, spread over the CTAs.
     const int nw = H->nwarps, all = int(gridDim.x) * kQ4ListWarps;
     const int gw = nw < all ? warp * int(gridDim.x) + int(blockIdx.x) : int(blockIdx.x) * kQ4ListWarps + warp;
-    if (gw >= nw) return;
+    const bool work = gw < nw;
     const uint32_t total = H->total_chunks;
-    const uint32_t c_begin = range_begin(total, gw, nw), c_end = range_begin(total, gw + 1, nw);
-    const int first_item = warps[gw].item;
+    const uint32_t c_begin = work ? range_begin(total, gw, nw) : 0u, c_end = work ? range_begin(total, gw + 1, nw) : 0u;
+    const int first_item = work ? warps[gw].item : 0;
 
     const uint32_t ring_lane = smem_u32(q4_smem) + uint32_t(warp) * (DEPTH * CH) + lane * 16;
     const uint32_t ring_lane_end = ring_lane + DEPTH * CH;
@@ -159,7 +151,26 @@ __global__ void __launch_bounds__(kQ4ListThreads, 1) k_q4_list_main(unsigned cha
 #pragma unroll
     for (int i = 0; i < DEPTH - 1; ++i) fetch_into(ring_lane + i * CH);
 
-    pdl_wait();  // the group sums come from k_q4_list_prepare, the activations possibly from a kernel before it
+    // the matrices of this CTA's warps follow one another, and so do their groups
+    const int cta_first = int(blockIdx.x) * kQ4ListWarps, cta_next = min(cta_first + kQ4ListWarps, nw - 1);
+    const bool spread = nw < all;
+    const int item_lo = spread ? 0 : warps[cta_first].item, item_hi = spread ? 0 : warps[cta_next].item;
+    const uint32_t group_lo = items[item_lo].group_begin;
+    const bool held = !spread && items[item_hi].group_begin + uint32_t(items[item_hi].groups) - group_lo <= uint32_t(kQ4ListSums);
+    pdl_wait();  // the activations may come from a kernel before
+    if (held) {
+        for (int it = item_lo; it <= item_hi; ++it) {
+            const Q4Item I = items[it];
+            // eight lanes per group; the whole warp goes round, so that all lanes are there for the shuffles
+            for (int k0 = warp * 4; k0 < I.groups; k0 += kQ4ListWarps * 4) {
+                const int k = min(k0 + (lane >> 3), I.groups - 1);
+                const float2 v = group_sums<G, 8>(I.x + size_t(k) * G, lane & 7);
+                if ((lane & 7) == 0) sums[I.group_begin - group_lo + uint32_t(k)] = v;
+            }
+        }
+        __syncthreads();
+    }
+    if (!work) return;
 
     uint32_t slot_lane = ring_lane;                       // slot being consumed
     uint32_t refill_lane = ring_lane + (DEPTH - 1) * CH;  // slot consumed last (empty at the start)
@@ -179,7 +190,7 @@ __global__ void __launch_bounds__(kQ4ListThreads, 1) k_q4_list_main(unsigned cha
         local += in_item;
         // column 0 of the B fragment is the activation vector; the other columns repeat it and are never stored
         const __half* x_lane = I.x + 16 * t;
-        const unsigned char* gs_lane = gs + size_t(I.group_begin) * 64 + t * 16;
+        const float2* item_sums = sums + (I.group_begin - group_lo);
         while (in_item > 0) {
             // one segment: the chunks of this warp that belong to one strip
             const int seg_first = gi;
@@ -190,8 +201,7 @@ __global__ void __launch_bounds__(kQ4ListThreads, 1) k_q4_list_main(unsigned cha
 #pragma unroll
                 for (int i = 0; i < 4; ++i) acc[h][i] = 0.f;
             for (uint32_t c = 0; c < seg_len; ++c, ++gi) {
-                const uint4 csv = __ldg(reinterpret_cast<const uint4*>(gs_lane + size_t(gi) * 64));
-                const uint32_t cs[4] = {csv.x, csv.y, csv.z, csv.w};  // (sum x, -sum bias x) of columns 2 t, 2 t + 1
+                const float2 cs = held ? item_sums[gi] : group_sums<G, 32>(I.x + size_t(gi) * G, lane);
                 fetch_into(refill_lane);
                 q4_cp_async_wait<DEPTH - 1>();  // this chunk has landed
                 __syncwarp();
@@ -215,13 +225,12 @@ __global__ void __launch_bounds__(kQ4ListThreads, 1) k_q4_list_main(unsigned cha
                             a[2] = lop_and_or(ww[m], 0x00F000F0u, 0x54005400u);  // row g,     columns c+2, c+3 (64 + n)
                             a[3] = lop_and_or(w8, 0x00F000F0u, 0x54005400u);     // row g + 8, columns c+2, c+3
                             if (j == 0 && m == 0)
-                                mma_f16_first(d[h], a, xr[0], xr[1], __uint_as_float(cs[1]), __uint_as_float(cs[3]));
+                                mma_f16_first(d[h], a, xr[0], xr[1], cs.y, cs.y);
                             else
                                 mma_f16(d[h], a, xr[2 * m], xr[2 * m + 1]);
                         }
                     }
                 }
-                const float sx_even = __uint_as_float(cs[0]), sx_odd = __uint_as_float(cs[2]);
                 const uint32_t so_lane = slot_lane + so_delta;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -229,9 +238,9 @@ __global__ void __launch_bounds__(kQ4ListThreads, 1) k_q4_list_main(unsigned cha
                     const uint32_t so1 = lds32(so_lane + 64 * h + 32);
                     const float2 r0 = __half22float2(*reinterpret_cast<const __half2*>(&so0));  // (scale, offset)
                     const float2 r1 = __half22float2(*reinterpret_cast<const __half2*>(&so1));
-                    fma2(r0.y, sx_even, sx_odd, acc[h][0], acc[h][1]);
+                    fma2(r0.y, cs.x, cs.x, acc[h][0], acc[h][1]);
                     fma2(r0.x, d[h][0], d[h][1], acc[h][0], acc[h][1]);
-                    fma2(r1.y, sx_even, sx_odd, acc[h][2], acc[h][3]);
+                    fma2(r1.y, cs.x, cs.x, acc[h][2], acc[h][3]);
                     fma2(r1.x, d[h][2], d[h][3], acc[h][2], acc[h][3]);
                 }
                 __syncwarp();  // every lane has read the slot before the next refill targets it
@@ -301,7 +310,7 @@ int check_list(const tetra_q4_problem* p, int count, int G) {
 
 template <int G, int DEPTH>
 cudaError_t run_main(unsigned char* ws, int sms, cudaStream_t s) {
-    const size_t smem = size_t(kQ4ListWarps) * DEPTH * q4_chunk_bytes(G);
+    const size_t smem = size_t(kQ4ListWarps) * DEPTH * q4_chunk_bytes(G) + kQ4ListSums * sizeof(float2);
     static PerDeviceOnce once;
     cudaError_t e = once.run([smem] {
         return cudaFuncSetAttribute(k_q4_list_main<G, DEPTH>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
@@ -321,9 +330,7 @@ size_t tetra_q4_list_workspace_bytes(const tetra_q4_problem* problems_host, int 
     if (check_list(problems_host, count, G) != TETRA_OK) return 0;
     int sms = 0;
     if (device_sms(&sms) != cudaSuccess) return 0;
-    size_t groups = 0;
-    for (int i = 0; i < count; ++i) groups += size_t(problems_host[i].K / G);
-    return list_layout(count, groups, sms * kQ4ListWarps).total;
+    return list_layout(count, sms * kQ4ListWarps).total;
 }
 
 int tetra_q4_list_plan(const tetra_q4_problem* problems_host, int count, int G, void* workspace_dev,
@@ -343,9 +350,9 @@ int tetra_q4_list_plan(const tetra_q4_problem* problems_host, int count, int G, 
         strips += st;
     }
     if (chunks > 0x7FFFFFF0ull || strips > 0x7FFFFFF0ull) return TETRA_ERR_SHAPE;
-    const Q4ListLayout L = list_layout(count, size_t(groups), nwarps);
+    const Q4ListLayout L = list_layout(count, nwarps);
     if (workspace_bytes < L.total) return TETRA_ERR_SIZE;
-    const size_t meta = L.off_gs;
+    const size_t meta = L.off_pieces;
     unsigned char* buf = static_cast<unsigned char*>(std::calloc(1, meta));
     if (!buf) return TETRA_ERR_CUDA;
     Q4ListHeader* H = reinterpret_cast<Q4ListHeader*>(buf);
@@ -358,11 +365,8 @@ int tetra_q4_list_plan(const tetra_q4_problem* problems_host, int count, int G, 
     H->total_strips = uint32_t(strips);
     H->off_items = uint32_t(L.off_items);
     H->off_warps = uint32_t(L.off_warps);
-    H->off_group_item = uint32_t(L.off_group_item);
-    H->off_gs = uint32_t(L.off_gs);
     H->off_pieces = uint32_t(L.off_pieces);
     Q4Item* items = reinterpret_cast<Q4Item*>(buf + L.off_items);
-    uint16_t* group_item = reinterpret_cast<uint16_t*>(buf + L.off_group_item);
     uint32_t cb = 0, gb = 0, sb = 0;
     for (int i = 0; i < count; ++i) {
         const tetra_q4_problem& q = problems_host[i];
@@ -378,7 +382,6 @@ int tetra_q4_list_plan(const tetra_q4_problem* problems_host, int count, int G, 
         I.group_begin = gb;
         I.strip_begin = sb;
         cb += uint32_t(I.groups) * uint32_t(I.strips);
-        for (int k = 0; k < I.groups; ++k) group_item[gb + uint32_t(k)] = uint16_t(i);
         gb += uint32_t(I.groups);
         sb += uint32_t(I.strips);
     }
@@ -426,8 +429,7 @@ int tetra_q4_list_run(void* workspace_dev, int G, void* stream) {
     if (device_sms(&sms) != cudaSuccess) return TETRA_ERR_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     unsigned char* ws = static_cast<unsigned char*>(workspace_dev);
-    cudaError_t e = launch_pdl(k_q4_list_prepare, sms * 2, 256, 0, s, ws);
-    if (e == cudaSuccess) e = G == 128 ? run_main<128, 2>(ws, sms, s) : run_main<64, 6>(ws, sms, s);
+    const cudaError_t e = G == 128 ? run_main<128, 2>(ws, sms, s) : run_main<64, 6>(ws, sms, s);
     return e == cudaSuccess ? TETRA_OK : TETRA_ERR_CUDA;
 }
 
