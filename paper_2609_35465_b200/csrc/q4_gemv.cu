@@ -27,12 +27,8 @@
 namespace tetra {
 namespace {
 
-#ifndef TETRA_Q4_THREADS
-#define TETRA_Q4_THREADS 512
-#define TETRA_Q4_CTAS 1
-#endif
-constexpr int kQ4Threads = TETRA_Q4_THREADS;
-constexpr int kQ4CtasPerSm = TETRA_Q4_CTAS;
+constexpr int kQ4Threads = 512;
+constexpr int kQ4CtasPerSm = 1;
 constexpr int kQ4Warps = kQ4Threads / 32;
 
 // Nibbles of two rows (v0: row g, v1: row g + 8; four consecutive columns each, column c + i at bits 4 i) as the
@@ -101,7 +97,9 @@ __global__ void __launch_bounds__(256) k_q4_pack(const uint8_t* __restrict__ q, 
 // adds four MMAs per sub-tile (the activations' B fragments are shared by both), then
 //     acc += scale * D + offset * sum_group(x).
 // A strip that lies wholly inside a warp's range is stored directly; a strip cut by a range boundary leaves
-// one piece per warp in shared memory, and after one CTA barrier the pieces are added in warp order.
+// one piece per warp in shared memory, and after one CTA barrier the pieces are added in warp order; which strips those
+// are is worked out while the kernel waits for its predecessor (looked for afterwards, piece by piece, it was 2.2 us of
+// a 5.1 us launch: 1024 x 4096, G = 128, now 3.9 us; 12288 x 4096, G = 64, 9.9 -> 8.2 us).
 // Addresses advance by running pointers: the loop body is dequantise, multiply, scale.
 // XS: the activations are staged in shared memory (rows padded by 16 bytes so that the eight vectors' reads
 // fall into different banks); otherwise they are read through L1.
@@ -111,7 +109,6 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
           int batch) {
     constexpr int TPG = G / 64, CH = q4_chunk_bytes(G), PIECES = CH / 16;
     extern __shared__ __align__(16) unsigned char q4_smem[];
-    __shared__ int piece_strip[2 * kQ4Warps];
     const int groups = K / G, strips = (N + 31) / 32;
     float2* gs = reinterpret_cast<float2*>(q4_smem);                        // [groups][8]: (sum x, -sum bias x)
     float* pieces = reinterpret_cast<float*>(q4_smem + size_t(groups) * 64);  // [warps][2][256]
@@ -122,14 +119,15 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
     const uint32_t xs_stride = uint32_t(K) * 2u + 16u;  // bytes per staged vector
     const int g = lane >> 2, t = lane & 3;
     pdl_release();
-    if (threadIdx.x < 2 * kQ4Warps) piece_strip[threadIdx.x] = -1;
 
     // this CTA's strips, this warp's chunks (local index n = local strip * groups + group)
     const int strip_begin = int(size_t(blockIdx.x) * strips / gridDim.x);
     const int strip_end = int((size_t(blockIdx.x) + 1) * strips / gridDim.x);
     const uint32_t cta_chunks = uint32_t(strip_end - strip_begin) * uint32_t(groups);
-    const uint32_t n_begin = uint32_t(uint64_t(warp) * cta_chunks / kQ4Warps);
-    const uint32_t n_end = uint32_t((uint64_t(warp) + 1) * cta_chunks / kQ4Warps);
+    // every range non-empty: fewer chunks than warps leave warps over
+    const uint32_t ranges = min(cta_chunks, uint32_t(kQ4Warps));
+    auto range_begin = [&](uint32_t w) { return cta_chunks <= uint32_t(kQ4Warps) ? min(w, cta_chunks) : uint32_t(uint64_t(w) * cta_chunks / kQ4Warps); };
+    const uint32_t n_begin = range_begin(uint32_t(warp)), n_end = range_begin(uint32_t(warp) + 1);
     // running addresses: f_src = next chunk to copy (this lane's 16 bytes of each 512), f_todo = chunks left to
     // copy; slot_lane = this lane's 16 bytes in the slot being consumed; the slot consumed last is refilled
     const unsigned char* f_src = packed + (size_t(strip_begin) * groups + n_begin) * CH + lane * 16;
@@ -149,39 +147,55 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
 #pragma unroll
     for (int i = 0; i < DEPTH - 1; ++i) fetch_into(ring_lane + i * CH);  // the weights do not depend on the preceding kernel
 
-    pdl_wait();  // x may come from the preceding kernel
-    if (XS) {
-        for (int i = threadIdx.x; i < batch * (K / 8); i += kQ4Threads) {
-            const int v = i / (K / 8), c8 = i % (K / 8);
-            *reinterpret_cast<uint4*>(xs_base + size_t(v) * xs_stride + size_t(c8) * 16) =
-                __ldg(reinterpret_cast<const uint4*>(x + size_t(v) * K) + c8);
-        }
-        __syncthreads();
-    }
-    // per (group, vector): sum of x and minus the sum of bias_k x_k, bias 1024 for k % 4 in {0, 1}, 64 for {2, 3};
-    // eight lanes per task, combined by shuffles in a fixed order
-    for (int task0 = (threadIdx.x >> 3); task0 < groups * 8; task0 += kQ4Threads / 8) {
-        const int v = task0 & 7, gi = task0 >> 3, sub = threadIdx.x & 7;
-        float lo = 0.f, hi = 0.f;  // k % 4 in {0, 1} / {2, 3}
-        if (v < batch) {
-            const uint2* src = XS ? reinterpret_cast<const uint2*>(xs_base + size_t(v) * xs_stride) + size_t(gi) * (G / 4)
-                                  : reinterpret_cast<const uint2*>(x + size_t(v) * K + size_t(gi) * G);
-#pragma unroll
-            for (int i = 0; i < G / 32; ++i) {
-                const uint2 u = XS ? src[sub + 8 * i] : __ldg(src + sub + 8 * i);
-                const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
-                const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
-                lo += a.x + a.y;
-                hi += b.x + b.y;
+    // cut[w]: the strip that begins in warp w's range and goes on beyond it, and over how many ranges it stretches in all
+    // (0: there is none); known from here on, needed at the end
+    __shared__ int2 cut[kQ4Warps];
+    if (threadIdx.x < kQ4Warps) {
+        const uint32_t w = threadIdx.x, begin = range_begin(w), end = range_begin(w + 1);
+        int2 c = make_int2(0, 0);
+        if (begin < end) {
+            const uint32_t s = (end - 1) / uint32_t(groups), s_begin = s * uint32_t(groups), s_end = s_begin + uint32_t(groups);
+            if (s_begin >= begin && s_end > end) {
+                uint32_t k = w + 1;
+                while (k < ranges && range_begin(k) < s_end) ++k;
+                c = make_int2(int(s), int(k - w));
             }
         }
-#pragma unroll
-        for (int o = 4; o >= 1; o >>= 1) {
-            lo += __shfl_xor_sync(0xFFFFFFFFu, lo, o);
-            hi += __shfl_xor_sync(0xFFFFFFFFu, hi, o);
-        }
-        if (sub == 0) gs[task0] = make_float2(lo + hi, -(1024.f * lo + 64.f * hi));
+        cut[w] = c;
     }
+    pdl_wait();  // x may come from the preceding kernel
+    // The activations, eight to a thread (into shared memory if they fit), and on the way, per (group, vector), the sum of
+    // x and minus the sum of bias_k x_k, bias 1024 for k % 4 in {0, 1}, 64 for {2, 3}: G / 8 neighbouring lanes combined
+    // by shuffles in a fixed order.
+    {
+        const uint32_t per_vec = uint32_t(K) / 8u, total = per_vec * uint32_t(batch), inv = 0xFFFFFFFFu / per_vec + 1u;
+        constexpr int AHEAD = 4;  // loads in flight per thread
+        for (uint32_t i0 = warp * 32; i0 < total; i0 += AHEAD * kQ4Threads) {  // whole warps, for the shuffles
+            uint4 u[AHEAD];
+#pragma unroll
+            for (int j = 0; j < AHEAD; ++j) {
+                const uint32_t i = i0 + uint32_t(j * kQ4Threads + lane), v = __umulhi(i, inv);
+                u[j] = i < total ? __ldg(reinterpret_cast<const uint4*>(x + size_t(v) * K) + (i - v * per_vec)) : make_uint4(0u, 0u, 0u, 0u);
+            }
+#pragma unroll
+            for (int j = 0; j < AHEAD; ++j) {
+                if (i0 + uint32_t(j * kQ4Threads) >= total) break;  // warp-uniform
+                const uint32_t i = i0 + uint32_t(j * kQ4Threads + lane), v = __umulhi(i, inv), c8 = i - v * per_vec;
+                if (XS && i < total) *reinterpret_cast<uint4*>(xs_base + size_t(v) * xs_stride + size_t(c8) * 16) = u[j];
+                const float2 a0 = __half22float2(*reinterpret_cast<const __half2*>(&u[j].x)), b0 = __half22float2(*reinterpret_cast<const __half2*>(&u[j].y));
+                const float2 a1 = __half22float2(*reinterpret_cast<const __half2*>(&u[j].z)), b1 = __half22float2(*reinterpret_cast<const __half2*>(&u[j].w));
+                float lo = (a0.x + a0.y) + (a1.x + a1.y), hi = (b0.x + b0.y) + (b1.x + b1.y);  // k % 4 in {0, 1} / {2, 3}
+#pragma unroll
+                for (int o = G / 16; o >= 1; o >>= 1) {
+                    lo += __shfl_xor_sync(0xFFFFFFFFu, lo, o);
+                    hi += __shfl_xor_sync(0xFFFFFFFFu, hi, o);
+                }
+                if (lane % (G / 8) == 0 && i < total) gs[c8 / (G / 8) * 8 + v] = make_float2(lo + hi, -(1024.f * lo + 64.f * hi));
+            }
+        }
+    }
+    for (int i = threadIdx.x; i < groups * 8; i += kQ4Threads)
+        if ((i & 7) >= batch) gs[i] = make_float2(0.f, 0.f);
     __syncthreads();
 
     // column g of B is vector g; columns at or beyond batch are never stored, so they may hold any vector
@@ -194,7 +208,6 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
     const uint32_t so_delta = uint32_t(TPG * 1024 + g * 4) - uint32_t(lane * 16);  // slot_lane -> this lane's scale records
     int gi = int(n_begin % uint32_t(groups));
     int strip = strip_begin + int(n_begin / uint32_t(groups));
-    int n_pieces = 0;
     uint32_t left = n_end - n_begin;
     while (left > 0) {
         // one segment: the chunks of this warp that belong to one strip
@@ -284,12 +297,10 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
                     const int row = 32 * strip + 16 * h + g + 8 * (i >> 1), v = 2 * t + (i & 1);
                     if (row < N && v < batch) y[size_t(v) * N + row] = acc[h][i];
                 }
-        } else {  // a strip shared with a neighbouring warp: leave a piece
-            float* mine = pieces + (2 * warp + n_pieces) * 256 + 8 * lane;
+        } else {  // a strip shared with a neighbouring warp: leave a piece (slot 0: it began before this range, 1: it ends beyond)
+            float* mine = pieces + (2 * warp + (seg_first != 0 ? 0 : 1)) * 256 + 8 * lane;
             *reinterpret_cast<float4*>(mine) = make_float4(acc[0][0], acc[0][1], acc[0][2], acc[0][3]);
             *reinterpret_cast<float4*>(mine + 4) = make_float4(acc[1][0], acc[1][1], acc[1][2], acc[1][3]);
-            if (lane == 0) piece_strip[2 * warp + n_pieces] = strip;
-            ++n_pieces;
         }
         if (gi == groups) {
             gi = 0;
@@ -298,22 +309,27 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
     }
     q4_cp_async_wait<0>();
     __syncthreads();
-    // pieces in (warp, first/second) order are in memory order: the pieces of a strip are consecutive
-    if (threadIdx.x < 256) {
-        const int e = threadIdx.x, el = e >> 3, h = (e >> 2) & 1, i = e & 3;
-        const int r_in = 16 * h + (el >> 2) + 8 * (i >> 1), v = 2 * (el & 3) + (i & 1);
-        int cur = -1;
-        float total = 0.f;
-        for (int pc = 0; pc <= 2 * kQ4Warps; ++pc) {
-            const int sidx = pc < 2 * kQ4Warps ? piece_strip[pc] : -2;
-            if (sidx == -1) continue;
-            if (sidx != cur) {
-                if (cur >= 0 && 32 * cur + r_in < N && v < batch) y[size_t(v) * N + 32 * cur + r_in] = total;
-                cur = sidx;
-                total = 0.f;
-            }
-            if (sidx >= 0) total += pieces[pc * 256 + e];
+    // The strips that a range boundary cuts: warp w's second piece, then the first pieces of the warps after it.  Half
+    // of the CTA's threads takes the even w, half the odd ones; a thread is one of the 256 results of a strip.
+    const int e = threadIdx.x & 255, el = e >> 3, h = (e >> 2) & 1, i = e & 3;
+    const int r_in = 16 * h + (el >> 2) + 8 * (i >> 1), v = 2 * (el & 3) + (i & 1);
+#pragma unroll 1
+    for (int w = int(threadIdx.x >> 8); w < kQ4Warps; w += kQ4Threads / 256) {
+        const int2 c = cut[w];
+        if (c.y == 0) continue;
+        const float* at = pieces + 2 * w * 256 + e;
+        float total = at[256];
+#pragma unroll
+        for (int k0 = 1; k0 < kQ4Warps; k0 += 5) {  // five loads at a time
+            if (k0 >= c.y) break;
+            float p[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) p[k] = k0 + k < c.y ? at[(k0 + k) * 512] : 0.f;
+#pragma unroll
+            for (int k = 0; k < 5; ++k) total += p[k];
         }
+        const int row = 32 * (strip_begin + c.x) + r_in;
+        if (row < N && v < batch) y[size_t(v) * N + row] = total;
     }
 }
 

@@ -1,0 +1,203 @@
+"""Sizes at which a tile, a remainder or a choice between kernels can go wrong, one small case per edge, against the
+oracles."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_35465_b200 import synth
+from helpers import assert_gemv_close, make_matrix, oracle_product
+
+pytestmark = pytest.mark.gpu
+GAIN = synth.DEFAULT_GAIN
+
+
+@pytest.fixture(scope="module")
+def tt():
+    from paper_2609_35465_b200 import tetra
+    return tetra
+
+
+@pytest.fixture(scope="module")
+def table(tt):
+    return tt.tetra_build_table(GAIN)
+
+
+def device_matrix(tt, table, m, x):
+    codes = tt.tetra_pack_codes(torch.from_numpy(m["codes"]).cuda(), table, m["N"], m["B"])
+    return dict(codes=codes, row_scales=torch.from_numpy(m["sigma"]).cuda(), x=x, N=m["N"], K=m["K"],
+                tail=torch.from_numpy(m["tail"]).cuda() if m["tail"] is not None else None,
+                y=torch.full((m["N"],), float("nan"), dtype=torch.float32, device="cuda"))
+
+
+def check(orc, m, y, what, vector=0):
+    assert np.isfinite(y).all(), what
+    ref = oracle_product(orc, m, GAIN, batch_index=vector)
+    assert_gemv_close(y, ref, what)
+    assert np.max(np.abs(y - ref["y"]) / ref["abssum"]) < 1e-5
+
+
+# Row groups of eight and of four rows, one and several chunks of rows per CTA, fewer columns than lanes, K too large
+# for the activations' image in shared memory.
+@pytest.mark.parametrize("N,K,tail_mode", [
+    (1, 24, True), (4, 25, True), (5, 47, False), (8, 24 * 31, True), (9, 24 * 32, True), (1183, 24 * 33 + 1, True),
+    (1185, 24 * 5, True), (148 * 8 * 3 + 4, 24 * 40, True), (148 * 16 + 12, 24 * 64 + 23, True), (20001, 96, True),
+    (64, 24 * 1400, True), (24, 49152, True),
+])
+def test_single_matrix(tt, table, orc, N, K, tail_mode):
+    m = make_matrix(71, N + K, N, K, tail_mode, batch=1)
+    d = device_matrix(tt, table, m, torch.from_numpy(m["x"][0]).cuda())
+    if tail_mode:
+        tt.tetra_gemv_tail(d["codes"], d["row_scales"], table, d["x"], d["y"], N, K, 1, d["tail"])
+    else:
+        tt.tetra_gemv(d["codes"], d["row_scales"], table, d["x"], d["y"], N, K)
+    torch.cuda.synchronize()
+    check(orc, m, d["y"].cpu().numpy(), "%d x %d" % (N, K))
+
+
+# A CTA works on one matrix: lists of very unequal matrices, of more and of fewer row groups than CTAs.
+@pytest.mark.parametrize("rows,K", [((1, 1, 1, 1, 1, 1, 1, 1), 24), ((4000, 8), 24 * 40), ((8, 9000, 16, 1), 24 * 12 + 7),
+                                    ((700, 700, 700), 24 * 70 + 2)])
+def test_list_split(tt, table, orc, rows, K):
+    ms = [make_matrix(72, 10 * i + K, n, K, True, batch=1) for i, n in enumerate(rows)]
+    items = [device_matrix(tt, table, m, torch.from_numpy(m["x"][0]).cuda()) for m in ms]
+    tt.tetra_gemv_list(tt.make_problems(items), table)
+    torch.cuda.synchronize()
+    for m, it in zip(ms, items):
+        check(orc, m, it["y"].cpu().numpy(), "list %s" % (rows,))
+
+
+# Block-diagonal up to four vectors, dense from five on; one to four row tiles per step and several steps of rows; column
+# quads that are not full; clusters (few rows, many columns); rows of x that are not 16-byte aligned.
+@pytest.mark.parametrize("N,K,tail_mode,batch", [
+    (1, 24, True, 2), (15, 24 * 3, True, 3), (16, 24 * 4, True, 4), (17, 24 * 5, True, 5), (33, 24 * 65 + 1, True, 2),
+    (33, 24 * 65 + 3, False, 7), (64, 24 * 600, True, 2), (64, 24 * 600 + 8, True, 11), (148 * 16, 24 * 9, True, 4),
+    (148 * 16 + 1, 24 * 9, True, 9), (148 * 48, 24 * 7, True, 3), (148 * 64 + 5, 24 * 6, True, 6), (148 * 80, 24 * 2, True, 16),
+    (148 * 96 + 3, 24 * 5 + 2, True, 2),
+])
+def test_batched_shapes(tt, table, orc, N, K, tail_mode, batch):
+    m = make_matrix(73, N + K + batch, N, K, tail_mode, batch=batch)
+    d = device_matrix(tt, table, m, torch.from_numpy(m["x"]).cuda())
+    y = torch.full((batch, N), float("nan"), dtype=torch.float32, device="cuda")
+    tt.tetra_gemv_batched(d["codes"], d["row_scales"], table, d["x"], y, N, K, batch, d["tail"])
+    torch.cuda.synchronize()
+    for v in sorted({0, batch // 2, batch - 1}):
+        check(orc, m, y[v].cpu().numpy(), "%d x %d, vector %d of %d" % (N, K, v, batch), v)
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
+@pytest.mark.parametrize("batch", [3, 6])
+def test_batched_non_finite_activation(tt, table, bad, batch):
+    m = make_matrix(74, batch, 70, 24 * 20, True, batch=batch)
+    x = torch.from_numpy(m["x"]).cuda()
+    x[1, 24 * 7 + 5] = bad
+    d = device_matrix(tt, table, m, x)
+    y = torch.zeros((batch, 70), dtype=torch.float32, device="cuda")
+    tt.tetra_gemv_batched(d["codes"], d["row_scales"], table, x, y, 70, 24 * 20, batch)
+    torch.cuda.synchronize()
+    assert torch.isnan(y[1]).all() and torch.isfinite(y[0]).all() and torch.isfinite(y[2:]).all()
+
+
+# Copies out of 16, 8 and 4 bytes (odd block counts, outputs that are not aligned), part-filled row groups and columns.
+@pytest.mark.parametrize("N,B", [(1, 1), (7, 31), (8, 32), (9, 33), (17, 64), (16, 65)])
+def test_decode_packed_shapes(tt, table, orc, N, B):
+    words = synth.words_to_bytes(synth.words(75, N * 100 + B, N * B))
+    # word addresses that are 2, but not 4 bytes aligned as well
+    buf = torch.zeros(6 * N * B + 2, dtype=torch.uint8, device="cuda")
+    buf[2:] = torch.from_numpy(words.reshape(-1)).cuda()
+    Y, M, G = orc.decode_blocks(words)
+    for codes in (torch.from_numpy(words).cuda().reshape(N, B, 6), buf[2:].reshape(N, B, 6)):
+        packed = tt.tetra_pack_codes(codes, table, N, B)
+        y, mg = tt.tetra_decode_packed(packed, table, N, B)
+        out = torch.zeros(24 * N * B + 4, dtype=torch.int8, device="cuda")
+        lib, p = tt.lib(), tt._ptr
+        assert lib.tetra_decode_packed(p(packed), p(table), p(out[4:]), None, N, B, tt._stream()) == 0
+        torch.cuda.synchronize()
+        assert np.array_equal(y.cpu().numpy().reshape(-1, 24), Y)
+        assert np.array_equal(mg.cpu().numpy().reshape(-1, 2), np.stack([M, G], 1))
+        assert np.array_equal(out[4:].cpu().numpy().reshape(-1, 24), Y)
+
+
+# Strips of 32 rows shared by two and more warps, CTAs with fewer chunks than warps, both group sizes.
+@pytest.mark.parametrize("N,K,G,batch", [(1, 64, 64, 1), (31, 128, 128, 8), (33, 192, 64, 1), (64, 15 * 64, 64, 3),
+                                         (32 * 148, 128 * 7, 128, 1), (32 * 148 * 2 + 1, 64 * 3, 64, 2), (96, 64 * 257, 64, 1)])
+def test_q4_shapes(tt, N, K, G, batch):
+    from oracle import q4 as oq
+    q = synth.q4_nibbles(76, N, N, K)
+    sc, of = synth.q4_scales_offsets(76, N, N, K // G)
+    packed = tt.tetra_q4_pack(torch.from_numpy(q).cuda(), torch.from_numpy(sc).cuda(), torch.from_numpy(of).cuda(), N, K, G)
+    x = synth.activations(76, K, K, batch)
+    y = torch.full((batch, N), float("nan"), dtype=torch.float32, device="cuda")
+    tt.tetra_q4_gemv(packed, torch.from_numpy(x).cuda(), y, N, K, G, batch)
+    ids = synth.token_ids(76, 1, 9, N)
+    buf = torch.zeros(9 * K + 4, dtype=torch.float16, device="cuda")
+    rows, rows8 = torch.zeros((9, K), dtype=torch.float16, device="cuda"), buf[4:].reshape(9, K)  # 16 and 8 byte stores
+    for out in (rows, rows8):
+        tt.tetra_q4_rows(packed, torch.from_numpy(ids).cuda(), out, N, K, G)
+    torch.cuda.synchronize()
+    want, tn = oq.gemv(q, sc, of, x, N, K, G, batch)
+    assert_gemv_close(y.cpu().numpy(), {"y": want, "termnorm": tn}, "q4 %d x %d" % (N, K))
+    want_rows = oq.rows(q, sc, of, ids, N, K, G).view(np.uint16)
+    for out in (rows, rows8):
+        assert np.array_equal(out.cpu().numpy().view(np.uint16), want_rows)
+
+
+# Lists with fewer chunks than warps, strips that many warps share, many small matrices, more groups per CTA than are held.
+@pytest.mark.parametrize("shapes,G", [([(1, 64)], 64), ([(40, 128), (1, 256), (33, 128)], 128), ([(32, 64 * 900)], 64),
+                                      ([(64, 64)] * 300, 64), ([(32, 65536)] * 40, 64)])
+def test_q4_list_shapes(tt, shapes, G):
+    from oracle import q4 as oq
+    items, hosts = [], []
+    for i, (N, K) in enumerate(shapes):
+        q = synth.q4_nibbles(77, i % 3, N, K)
+        sc, of = synth.q4_scales_offsets(77, i % 3, N, K // G)
+        x = synth.activations(77, i, K, 1)
+        hosts.append((q, sc, of, x, N, K))
+        items.append(dict(packed=tt.tetra_q4_pack(torch.from_numpy(q).cuda(), torch.from_numpy(sc).cuda(),
+                                                  torch.from_numpy(of).cuda(), N, K, G),
+                          x=torch.from_numpy(x[0]).cuda(), y=torch.zeros(N, dtype=torch.float32, device="cuda"), N=N, K=K))
+    ws = tt.tetra_q4_list_plan(tt.make_q4_problems(items), G)
+    first = None
+    for _ in range(2):  # the counters of shared strips start over
+        for it in items:
+            it["y"].fill_(float("nan"))
+        tt.tetra_q4_list_run(ws, G)
+        torch.cuda.synchronize()
+        got = [it["y"].cpu().numpy() for it in items]
+        assert first is None or all(np.array_equal(a, b) for a, b in zip(got, first))
+        first = got
+    for k in sorted({0, len(items) // 2, len(items) - 1}):
+        q, sc, of, x, N, K = hosts[k]
+        want, tn = oq.gemv(q, sc, of, x, N, K, G, 1)
+        assert_gemv_close(got[k][None], {"y": want, "termnorm": tn}, "list matrix %d, %d x %d" % (k, N, K))
+
+
+def test_encode_points_at_the_limits_of_the_lists(tt, table, orc):
+    """The last rows of every list and the rows just inside its last shell, both parities, come back as the same point:
+    these rows decide where the search's tables end."""
+    fields = []
+    for i1, i2, i3 in ((2047, 1239, 2047), (2046, 1238, 1256), (1256, 1240 + 807, 1255), (1255, 1240, 2047), (2047, 1240 + 806, 1816),
+                       (1816, 499, 1815), (1815, 498, 2047)):
+        for path in (0, 777, 4095):
+            for p in (0, 1):
+                for r in (0, 1):
+                    fields.append(i1 | (i2 << 11) | (i3 << 22) | (path << 33) | (p << 45) | (r << 46))
+    words = np.array(fields, dtype=np.uint64)
+    Y, _, _ = orc.decode_blocks(synth.words_to_bytes(words))
+    w = Y.astype(np.float32)
+    codes, cos = tt.tetra_encode_blocks(torch.from_numpy(w).cuda(), table)
+    torch.cuda.synchronize()
+    got, _, _ = orc.decode_blocks(codes.cpu().numpy())
+    got = got.astype(np.float64)
+    c = (got * w).sum(1) / (np.linalg.norm(got, axis=1) * np.linalg.norm(w.astype(np.float64), axis=1))
+    assert np.all(c >= 1 - 1e-12) and np.max(np.abs(cos.cpu().numpy() - 1)) <= 1e-6
+
+
+@pytest.mark.parametrize("n", [1, 2, 147, 148, 149, 296, 297, 444, 445])
+def test_encode_block_counts(tt, table, n):
+    """Blocks are dealt to three groups of threads per CTA: every count gives what the blocks give on their own."""
+    w = torch.from_numpy(synth.normal(78, 0, 20, 445 * 24).reshape(445, 24).astype(np.float32)).cuda()
+    w[5] = 0
+    all_codes, all_cos = tt.tetra_encode_blocks(w, table)
+    codes, cos = tt.tetra_encode_blocks(w[445 - n:].contiguous(), table)
+    torch.cuda.synchronize()
+    assert torch.equal(codes, all_codes[445 - n:]) and torch.equal(cos, all_cos[445 - n:])
