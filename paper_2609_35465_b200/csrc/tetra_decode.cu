@@ -184,7 +184,7 @@ k_decode_packed(const uint4* __restrict__ packed, const DeviceTables* __restrict
 #pragma unroll
                 for (int k = 0; k < 6; ++k) n2 = dp4a_ss(y[k], y[k], n2);
                 if (mg_lane && r0 + r < rows) {
-                    const uint32_t mg = (uint32_t(n2) >> 4) | ((w0[r0 + r] >> 17) & 0x100u);  // g: bit 25 of w0
+                    const uint32_t mg = (uint32_t(n2) >> 4) | ((w0[r0 + r] >> 21) & 0x100u);  // g: bit 29 of w0
                     if (WIDTH > 4) *reinterpret_cast<uint16_t*>(mg_at) = uint16_t(mg);
                     else mg_at[0] = uint8_t(mg), mg_at[1] = uint8_t(mg >> 8);
                 }

@@ -111,19 +111,20 @@ __device__ __forceinline__ void decode_file_word(const PaperTables* T, uint64_t 
 
 // ---------------------------------------------------------------------------
 // Device word (written by the pack kernel).  48 bits = w0 (32) + w1 (16):
-//   w0: [2..12] i1  [13] r  [14..24] i3  [25] g  [26..29] a  [30, 31, 0, 1] b
+//   w0: [2..12] i1  [13] r  [14..24] i3  [25..28] a  [29] g  [30, 31, 0, 1] b
 //   w1: [0..10] i2  [11] p  [12..15] x
 // (a, b, x) are the Turyn coordinates of the trellis path: the three pattern
 // bytes are h(a)+h'(x), h(b)+h'(x), h(a)+h(b)+h'(x).  i1 with r above it is a
 // byte offset into the row table as it stands; b is one rotation away from its
 // place in a table offset; p sits where i2's byte offset ends and below x, so
-// that (x, p) is one five-bit index.
+// that (x, p) is one five-bit index; g is in the word shifted for i3 where it
+// picks the gain's table (see scale_address).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void file_to_device_word(uint64_t w, uint32_t abx, uint32_t* w0, uint32_t* w1) {
     const uint32_t i1 = uint32_t(w & 0x7FF), i2 = uint32_t((w >> 11) & 0x7FF), i3 = uint32_t((w >> 22) & 0x7FF);
     const uint32_t p = uint32_t((w >> 45) & 1), r = uint32_t((w >> 46) & 1), g = uint32_t((w >> 47) & 1);
     const uint32_t a = abx & 15u, b = (abx >> 4) & 15u, x = abx >> 8;
-    *w0 = (i1 << 2) | (r << 13) | (i3 << 14) | (g << 25) | (a << 26) | (b << 30) | (b >> 2);
+    *w0 = (i1 << 2) | (r << 13) | (i3 << 14) | (a << 25) | (g << 29) | (b << 30) | (b >> 2);
     *w1 = i2 | (p << 11) | (x << 12);
 }
 // The twelve trellis bits of a file-order word: index of DeviceTables::trellis_to_abx.
@@ -135,9 +136,11 @@ constexpr uint32_t kSmMid = 16384;
 constexpr uint32_t kSmScale = 24576;
 constexpr uint32_t kSmMaskH = 25600;
 constexpr uint32_t kSmMaskXp = 25728;
+constexpr uint32_t kScaleGain = 2048;  // from one gain's scale table to the other's
 constexpr uint32_t kSmAlign = 16384;  // the staged copy starts on a 16 KiB boundary of shared memory
 static_assert(kSmMid == offsetof(DeviceTables, mid_fast) - kFastOffset, "staged layout");
 static_assert(kSmScale == offsetof(DeviceTables, scale) - kFastOffset, "staged layout");
+static_assert(kSmScale + kScaleGain == offsetof(DeviceTables, scale1) - kFastOffset && kSmScale % (2 * kScaleGain) == 0, "staged layout");
 static_assert(kSmMaskH == offsetof(DeviceTables, mask_h) - kFastOffset, "staged layout");
 static_assert(kSmMaskXp == offsetof(DeviceTables, mask_xp) - kFastOffset && kSmMaskXp % 128 == 0, "staged layout");
 
@@ -168,7 +171,7 @@ struct FastBlock {
     // MINUS EIGHT TIMES the lattice point, int8 x 4: y[2 s] holds coordinates 8 s + 2, 6, 3, 7 of section s in
     // its bytes 0..3, y[2 s + 1] coordinates 8 s + 0, 4, 1, 5.  The activations' planes use the same order.
     uint32_t y[6];
-    uint32_t goff;  // shared-memory address of the scale table plus 8 g (the gain's column of the table)
+    uint32_t norm0;  // what the squared norm starts from (see scale_address)
 };
 // Coordinate of a block held by byte i of word k.
 __host__ __device__ constexpr int word_coordinate(int k, int i) { return 8 * (k >> 1) + 4 * (i & 1) + (i >> 1) + ((k & 1) ? 0 : 2); }
@@ -184,7 +187,7 @@ static_assert(fast_nibble(word_coordinate(0, 1)) == 3 && fast_nibble(word_coordi
 struct NibbleBlock {
     uint32_t z[3];  // section s: coordinate j's z at bits 4 fast_nibble(j)
     uint32_t p4;    // bit 2: p (the other bits are an address)
-    uint32_t goff;  // shared-memory address of the scale table plus 8 g (the gain's column of the table)
+    uint32_t norm0; // 64 times the shared-memory address of the gain's scale table
 };
 // HI = false: w1 sits in bits 0..15 of `w1pair`; HI = true: in bits 16..31.
 // sm_tab: shared-memory address of the staged tables, a multiple of 16 KiB, so
@@ -195,11 +198,12 @@ __device__ __forceinline__ void decode_nibbles(uint32_t sm_tab, uint32_t w0, uin
     const uint32_t sh = HI ? w1pair >> 14 : w1pair << 2;                 // [2..12] i2, [13] p, [14..17] x
     const uint32_t addr1 = (w0 & 0x3FFCu) | (sm_tab + kSmRows);          // (i1 | r << 11) * 4
     const uint32_t addr2 = (sh & 0x1FFCu) | (sm_tab + kSmMid);
-    const uint32_t addr3i = ((w0 >> 12) & 0x1FFCu) | (sm_tab + kSmRows);
-    const uint32_t a4 = ((w0 >> 24) & 0x3Cu) | (sm_tab + kSmMaskH);
+    const uint32_t w3 = w0 >> 12;
+    const uint32_t addr3i = (w3 & 0x1FFCu) | (sm_tab + kSmRows);
+    const uint32_t a4 = ((w0 >> 23) & 0x3Cu) | (sm_tab + kSmMaskH);
     const uint32_t b4 = (__funnelshift_l(w0, w0, 4) & 0x3Cu) | (sm_tab + kSmMaskH);
     const uint32_t x4 = ((sh >> 11) & 0x7Cu) | (sm_tab + kSmMaskXp);     // (p | x << 1) * 4
-    out.goff = ((w0 >> 22) & 8u) | (sm_tab + kSmScale);
+    out.norm0 = (w3 & (kScaleGain << 6)) | ((sm_tab + kSmScale) << 6);
     const uint32_t row1 = lds32(addr1);
     const uint32_t row2 = lds32(addr2);
     // class of row 3 (Eq. (3)): p ^ r ^ delta, delta = [i2 >= 1240] = bit 11 of i2 + 808; all three at bit 13
@@ -217,7 +221,7 @@ template <bool HI>
 __device__ __forceinline__ void fast_decode(uint32_t sm_tab, uint32_t w0, uint32_t w1pair, FastBlock& out) {
     NibbleBlock nb;
     decode_nibbles<HI>(sm_tab, w0, w1pair, nb);
-    out.goff = nb.goff;
+    out.norm0 = nb.norm0;
     const uint32_t p8 = (nb.p4 & 4u) * 0x02020202u;                      // 8 p in every byte
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
@@ -226,13 +230,14 @@ __device__ __forceinline__ void fast_decode(uint32_t sm_tab, uint32_t w0, uint32
     }
 }
 
-// Shared-memory address of -gain[g] / sqrt(16 m): the squared norm of the packed point is 64 * 16 m, the table has
-// 16 bytes per m (16 m <= 416 for every word, Sec. 3.4, so the address stays inside it).
+// Shared-memory address of -gain[g] / sqrt(16 m).  The squared norm of the packed point is 64 * 16 m and a gain's table
+// has 16 bytes per m (16 m <= 416 for every word, Sec. 3.4), so the sum that starts from 64 times the table's address is
+// 64 times the entry's; the second gain's table lies kScaleGain bytes on, which is g where the word shifted for i3 has it.
 __device__ __forceinline__ uint32_t scale_address(const FastBlock& fb) {
-    int n2 = 0;
+    int n2 = int(fb.norm0);
 #pragma unroll
     for (int k = 0; k < 6; ++k) n2 = dp4a_ss(fb.y[k], fb.y[k], n2);
-    return (uint32_t(n2) >> 6) + fb.goff;
+    return uint32_t(n2) >> 6;
 }
 
 // sum of -y q from the sums of -8 y over the planes of q (high signed, middle, low): every term is a multiple of

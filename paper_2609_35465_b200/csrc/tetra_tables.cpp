@@ -154,6 +154,15 @@ int build_rows(PaperTables* p, int* n0_out) {
 
 }  // namespace
 
+void fill_scales(DeviceTables* t) {
+    std::memset(t->scale, 0, sizeof t->scale);
+    std::memset(t->scale1, 0, sizeof t->scale1);
+    for (int m = 0; m < 32; ++m) {
+        t->scale[m][0] = -(t->gain[0] * t->paper.rsqrt16m[m]);
+        t->scale1[m][0] = -(t->gain[1] * t->paper.rsqrt16m[m]);
+    }
+}
+
 int build_device_tables(DeviceTables* out, const float* gain2) {
     std::memset(out, 0, sizeof *out);
     Turyn turyn;
@@ -203,11 +212,7 @@ int build_device_tables(DeviceTables* out, const float* gain2) {
         out->mask_xp[2 * v] = mhr;
         out->mask_xp[2 * v + 1] = ~mhr;
     }
-    for (int g = 0; g < 2; ++g)
-        for (int m = 0; m < 32; ++m)
-            for (int k = 0; k < 4; ++k) out->scale[g][m][k] = 0.f;
-    for (int g = 0; g < 2; ++g)
-        for (int m = 0; m < 32; ++m) out->scale[0][m][2 * g] = -(out->gain[g] * out->paper.rsqrt16m[m]);
+    fill_scales(out);
     return 0;
 }
 
