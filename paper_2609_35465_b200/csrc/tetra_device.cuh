@@ -136,6 +136,7 @@ constexpr uint32_t kSmMid = 16384;
 constexpr uint32_t kSmScale = 24576;
 constexpr uint32_t kSmMaskH = 25600;
 constexpr uint32_t kSmMaskXp = 25728;
+constexpr uint32_t kSmGap = 25856, kStagedGap = 768;  // nothing to stage there
 constexpr uint32_t kScaleGain = 2048;  // from one gain's scale table to the other's
 constexpr uint32_t kSmAlign = 16384;  // the staged copy starts on a 16 KiB boundary of shared memory
 static_assert(kSmMid == offsetof(DeviceTables, mid_fast) - kFastOffset, "staged layout");
@@ -161,8 +162,10 @@ __device__ __forceinline__ unsigned char* stage_fast_tables_async(const DeviceTa
     const uint32_t s = smem_u32(smem);
     const uint32_t pad = ((s + kSmAlign - 1) & ~(kSmAlign - 1)) - s;
     const char* src = reinterpret_cast<const char*>(tab) + kFastOffset;
-    for (uint32_t i = threadIdx.x; i < kFastBytes / 16; i += blockDim.x)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(s + pad + 16u * i), "l"(src + 16u * i));
+    for (uint32_t i = threadIdx.x; i < (kFastBytes - kStagedGap) / 16; i += blockDim.x) {
+        const uint32_t at = 16u * i + (16u * i >= kSmGap ? kStagedGap : 0u);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(s + pad + at), "l"(src + at));
+    }
     return smem + pad;
 }
 constexpr uint32_t kTableSmemBytes = uint32_t(kFastBytes) + kSmAlign;
