@@ -26,6 +26,22 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], u
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// What the lanes of a B column that carries no vector read as activations: 16 halves of each tile of a group.
+constexpr int kQ4TileZeros = 192;
+__device__ const uint4 q4_zeros[kQ4TileZeros / 16] = {};
+
+// A lane's activations of a group's TILES 64-column tiles, through L1.  Global loads and cp.async are served in order: a
+// load behind a copy waits for the copy's memory, so these go out before the group's copies.
+template <int TILES>
+__device__ __forceinline__ void load_group(const unsigned char* x, uint32_t (&xr)[TILES][8]) {
+#pragma unroll
+    for (int j = 0; j < TILES; ++j) {
+        const uint4 a = __ldg(reinterpret_cast<const uint4*>(x) + 8 * j), b = __ldg(reinterpret_cast<const uint4*>(x) + 8 * j + 1);
+        xr[j][0] = a.x; xr[j][1] = a.y; xr[j][2] = a.z; xr[j][3] = a.w;
+        xr[j][4] = b.x; xr[j][5] = b.y; xr[j][6] = b.z; xr[j][7] = b.w;
+    }
+}
+
 // (a, a) * (b0, b1) + (c0, c1) in one instruction (fma.rn.f32x2).
 __device__ __forceinline__ void fma2(float a, float b0, float b1, float& c0, float& c1) {
     uint64_t aa, bb, cc;

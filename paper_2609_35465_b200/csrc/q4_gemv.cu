@@ -196,12 +196,18 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
     }
     for (int i = threadIdx.x; i < groups * 8; i += kQ4Threads)
         if ((i & 7) >= batch) gs[i] = make_float2(0.f, 0.f);
+    if (XS && threadIdx.x < kQ4TileZeros / 16) reinterpret_cast<uint4*>(xs_base + size_t(batch) * xs_stride)[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
 
-    // column g of B is vector g; columns at or beyond batch are never stored, so they may hold any vector
-    const uint32_t x_vec = uint32_t(g < batch ? g : batch - 1);
-    // this lane's 16 activations of the first tile of group 0: an offset in halves (global) or a shared address
-    const uint32_t x_lane = XS ? smem_u32(xs_base) + x_vec * xs_stride + 32u * t : x_vec * uint32_t(K) + 16u * t;
+    // Column g of B is vector g.  Columns at or beyond batch are never stored and read zeros wherever the walk is
+    // (x_step 0): multiplying zeros takes less power, and large matrices run at the board's limit.
+    const bool fed = g < batch;
+    const uint32_t x_step = fed ? 2u * G : 0u;
+    // this lane's 16 activations of the first tile of group 0: a shared address or a pointer
+    const auto x_lane = [&] {
+        if constexpr (XS) return smem_u32(xs_base) + (fed ? uint32_t(g) * xs_stride + 32u * t : uint32_t(batch) * xs_stride);
+        else return fed ? reinterpret_cast<const unsigned char*>(x + size_t(g) * K + 16 * t) : reinterpret_cast<const unsigned char*>(q4_zeros);
+    }();
     const uint32_t gs_lane = smem_u32(gs) + uint32_t(t) * 16;
     uint32_t slot_lane = ring_lane;                       // slot being consumed
     uint32_t refill_lane = ring_lane + (DEPTH - 1) * CH;  // slot consumed last (empty at the start)
@@ -213,7 +219,7 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
         // one segment: the chunks of this warp that belong to one strip
         const int seg_first = gi;
         const uint32_t seg_len = min(uint32_t(groups - gi), left);
-        uint32_t xo = x_lane + uint32_t(gi) * G * (XS ? 2u : 1u);
+        auto xo = x_lane + uint32_t(gi) * x_step;
         uint32_t gsp = gs_lane + uint32_t(gi) * 64;
         float acc[2][4];
 #pragma unroll
@@ -223,6 +229,8 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
         for (uint32_t c = 0; c < seg_len; ++c) {
             uint32_t cs[4];  // (sum x, -sum bias x) of vectors 2 t, 2 t + 1
             q4_lds128(gsp, cs);
+            [[maybe_unused]] uint32_t xl[TPG][8];
+            if constexpr (!XS) load_group<TPG>(xo, xl);  // ahead of the copies: see there
             fetch_into(refill_lane);
             q4_cp_async_wait<DEPTH - 1>();  // this chunk has landed
             __syncwarp();
@@ -230,7 +238,7 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
 #pragma unroll
             for (int j = 0; j < TPG; ++j) {
                 uint32_t xr[8];
-                if (XS) {
+                if constexpr (XS) {
                     uint32_t lo[4], hi[4];
                     q4_lds128(xo + 128 * j, lo);
                     q4_lds128(xo + 128 * j + 16, hi);
@@ -240,11 +248,8 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
                         xr[4 + i] = hi[i];
                     }
                 } else {
-                    const uint4* xg = reinterpret_cast<const uint4*>(x + xo) + 8 * j;  // L1-resident activations
-                    const uint4 xa = __ldg(xg);
-                    const uint4 xb = __ldg(xg + 1);
-                    xr[0] = xa.x; xr[1] = xa.y; xr[2] = xa.z; xr[3] = xa.w;
-                    xr[4] = xb.x; xr[5] = xb.y; xr[6] = xb.z; xr[7] = xb.w;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) xr[i] = xl[j][i];
                 }
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -283,7 +288,7 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
             refill_lane = slot_lane;
             slot_lane += CH;
             if (slot_lane == ring_lane_end) slot_lane = ring_lane;
-            xo += G * (XS ? 2u : 1u);
+            xo += x_step;
             gsp += 64;
         }
         left -= seg_len;
@@ -401,15 +406,19 @@ int device_sm_count(int* sms) {
 }
 
 constexpr size_t kQ4SmemLimit = 224 * 1024 / kQ4CtasPerSm - 2048;
-constexpr size_t kQ4StageLimit = 40 * 1024;  // activations up to this size are staged in shared memory
+
+template <int G, int DEPTH>
+constexpr size_t q4_smem_bytes(int K, int batch, bool staged) {
+    return size_t(K / G) * 64 + size_t(kQ4Warps) * 2048 + size_t(kQ4Warps) * DEPTH * q4_chunk_bytes(G) +
+           (staged ? size_t(batch) * (size_t(K) * 2 + 16) + kQ4TileZeros : 0);
+}
 
 template <int G, int DEPTH, bool XS>
 cudaError_t launch_q4_variant(const void* packed, const void* x, float* y, int N, int K, int batch, int sms,
                               cudaStream_t s) {
-    const int strips = (N + 31) / 32, groups = K / G;
-    int grid = strips < kQ4CtasPerSm * sms ? strips : kQ4CtasPerSm * sms;
-    const size_t smem = size_t(groups) * 64 + size_t(kQ4Warps) * 2048 + size_t(kQ4Warps) * DEPTH * q4_chunk_bytes(G) +
-                        (XS ? size_t(batch) * (size_t(K) * 2 + 16) : 0);
+    const int strips = (N + 31) / 32;
+    const int grid = strips < kQ4CtasPerSm * sms ? strips : kQ4CtasPerSm * sms;
+    const size_t smem = q4_smem_bytes<G, DEPTH>(K, batch, XS);
     static PerDeviceOnce once;  // per instantiation
     cudaError_t e = once.run([] {
         return cudaFuncSetAttribute(k_q4_gemv<G, DEPTH, XS>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kQ4SmemLimit));
@@ -433,7 +442,9 @@ cudaError_t launch_q4_variant(const void* packed, const void* x, float* y, int N
 template <int G, int DEPTH>
 cudaError_t launch_q4_gemv(const void* packed, const void* x, float* y, int N, int K, int batch, int sms,
                            cudaStream_t s) {
-    if (size_t(batch) * (size_t(K) * 2 + 16) <= kQ4StageLimit)
+    // Staged wherever they fit: read through L1 the activations queue behind the weights' copies, which the same unit
+    // takes in order (see q4_list.cu).
+    if (q4_smem_bytes<G, DEPTH>(K, batch, true) <= kQ4SmemLimit)
         return launch_q4_variant<G, DEPTH, true>(packed, x, y, N, K, batch, sms, s);
     return launch_q4_variant<G, DEPTH, false>(packed, x, y, N, K, batch, sms, s);
 }

@@ -9,18 +9,22 @@
 // and no warp waits for another.  One kernel:
 //   * per group of the activations the sum of x and minus the sum of bias_k x_k (the MMA operands carry biases
 //     1024 and 64) are made by each CTA for the few matrices its warps meet, in shared memory, while the first
-//     chunks are on their way; that also brings the activations into L1, where the warps read them;
+//     chunks are on their way, and the activations stay in shared memory with them.  (Read through L1 they queue behind
+//     the chunks' copies, which the same unit takes in order: a warp then waits for its newest copy before it can
+//     multiply its oldest chunk, and more copies in flight make it worse.  36 layers, 1.37 GB: 269 us from idle and
+//     284 us under the board's power limit, 198 and 222 us with the activations in shared memory);
 //   * the stream: dequantise with five logic operations per four registers, MMA against the activations, scale
 //     and offset per group; a strip (32 rows) that lies wholly inside a warp's range is stored; one cut by range
 //     boundaries leaves a piece per warp in the workspace, and the warp that finds the strip's other pieces there
 //     adds them in warp order and stores it.
 // Where a warp starts and who shares its strips is written into the plan: searched for on the device it was a chain
 // of dependent loads in every warp.  (One layer's projections, 38 MB: 22.5 us with searches, a kernel before this one
-// for the group sums and one after it for the pieces; now 13.0 us.  36 layers: 269 us either way, under the power limit.)
+// for the group sums and one after it for the pieces; now 13.0 us.)
 // Deterministic (fixed order everywhere); nothing waits for another warp (a counter per cut strip only tells the
 // last one); CTA barriers, cp.async.wait_group and griddepcontrol.wait are the only waits.
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 
 #include "../../include/tetra.h"
 #include "../../include/tetra_q4.h"
@@ -78,17 +82,22 @@ Q4ListLayout list_layout(int count, int nwarps) {
 // First chunk of warp w's range.
 __host__ __device__ inline uint32_t range_begin(uint32_t total, int w, int nw) { return uint32_t(uint64_t(total) * uint32_t(w) / uint32_t(nw)); }
 
-constexpr int kQ4ListSums = 4096;  // groups whose sums a CTA holds; a CTA that meets more makes them chunk by chunk
+// Bytes of activations that a CTA holds in shared memory, beside the rings: five vectors of 8192.  A CTA whose warps meet
+// more (short matrices: their activations outweigh their rows) reads them through L1 and makes the sums chunk by chunk.
+constexpr uint32_t kQ4ListX = 80 * 1024;
+template <int G>
+__host__ __device__ constexpr uint32_t list_held_groups() { return kQ4ListX / (2 * G); }
 
 // (sum x, minus the sum of bias_k x_k) of one group, bias 1024 for k % 4 in {0, 1} and 64 for {2, 3}; LANES consecutive
-// lanes each hold every LANES-th four activations, all of them get the result.
-template <int G, int LANES>
-__device__ __forceinline__ float2 group_sums(const __half* x, int sub) {
+// lanes each hold every LANES-th four activations (and copy them to `keep`), all of them get the result.
+template <int G, int LANES, bool KEEP>
+__device__ __forceinline__ float2 group_sums(const __half* x, int sub, uint2* keep) {
     const uint2* src = reinterpret_cast<const uint2*>(x);
     float lo = 0.f, hi = 0.f;
 #pragma unroll
     for (int i = 0; i < G / 4; i += LANES) {
         const uint2 u = G / 4 >= LANES || sub < G / 4 ? __ldg(src + sub + i) : make_uint2(0u, 0u);
+        if (KEEP) keep[sub + i] = u;
         const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
         const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
         lo += a.x + a.y;
@@ -112,7 +121,10 @@ __global__ void __launch_bounds__(kQ4ListThreads, 1) k_q4_list_main(unsigned cha
     // the plan (written once, long before) and the weights do not depend on the preceding kernel
     const Q4ListHeader* H = reinterpret_cast<const Q4ListHeader*>(ws);
     const Q4Item* items = reinterpret_cast<const Q4Item*>(ws + H->off_items);
+    // behind the rings: the held groups' sums, zeros for the B columns without a vector, the held groups' activations
     float2* sums = reinterpret_cast<float2*>(q4_smem + size_t(kQ4ListWarps) * DEPTH * CH);
+    unsigned char* zeros = reinterpret_cast<unsigned char*>(sums + list_held_groups<G>());
+    unsigned char* held_x = zeros + kQ4TileZeros;
     float* pieces = reinterpret_cast<float*>(ws + H->off_pieces);
     Q4Warp* warps = reinterpret_cast<Q4Warp*>(ws + H->off_warps);
     // A list of fewer chunks than warps uses as many warps as chunks, spread over the CTAs.
@@ -155,7 +167,7 @@ __global__ void __launch_bounds__(kQ4ListThreads, 1) k_q4_list_main(unsigned cha
     const bool spread = nw < all;
     const int item_lo = spread ? 0 : warps[cta_first].item, item_hi = spread ? 0 : warps[cta_next].item;
     const uint32_t group_lo = items[item_lo].group_begin;
-    const bool held = !spread && items[item_hi].group_begin + uint32_t(items[item_hi].groups) - group_lo <= uint32_t(kQ4ListSums);
+    const bool held = !spread && items[item_hi].group_begin + uint32_t(items[item_hi].groups) - group_lo <= list_held_groups<G>();
     pdl_wait();  // the activations may come from a kernel before
     if (held) {
         for (int it = item_lo; it <= item_hi; ++it) {
@@ -163,10 +175,12 @@ __global__ void __launch_bounds__(kQ4ListThreads, 1) k_q4_list_main(unsigned cha
             // eight lanes per group; the whole warp goes round, so that all lanes are there for the shuffles
             for (int k0 = warp * 4; k0 < I.groups; k0 += kQ4ListWarps * 4) {
                 const int k = min(k0 + (lane >> 3), I.groups - 1);
-                const float2 v = group_sums<G, 8>(I.x + size_t(k) * G, lane & 7);
-                if ((lane & 7) == 0) sums[I.group_begin - group_lo + uint32_t(k)] = v;
+                const uint32_t at = I.group_begin - group_lo + uint32_t(k);
+                const float2 v = group_sums<G, 8, true>(I.x + size_t(k) * G, lane & 7, reinterpret_cast<uint2*>(held_x + size_t(at) * (2 * G)));
+                if ((lane & 7) == 0) sums[at] = v;
             }
         }
+        if (threadIdx.x < kQ4TileZeros / 16) reinterpret_cast<uint4*>(zeros)[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
     }
     if (!work) return;
@@ -179,117 +193,134 @@ __global__ void __launch_bounds__(kQ4ListThreads, 1) k_q4_list_main(unsigned cha
     int ci = first_item;
     uint32_t left = c_end - c_begin;
     uint32_t local = c_begin - items[ci].chunk_begin;  // chunk index inside matrix ci
-    while (left > 0) {
-        const Q4Item I = items[ci];
-        const int groups = I.groups;
-        int strip = int(local / uint32_t(groups));
-        int gi = int(local - uint32_t(strip) * uint32_t(groups));
-        uint32_t in_item = min(left, uint32_t(groups) * uint32_t(I.strips) - local);
-        left -= in_item;
-        local += in_item;
-        // column 0 of the B fragment is the activation vector; the other columns repeat it and are never stored
-        const __half* x_lane = I.x + 16 * t;
-        const float2* item_sums = sums + (I.group_begin - group_lo);
-        while (in_item > 0) {
-            // one segment: the chunks of this warp that belong to one strip
-            const int seg_first = gi;
-            const uint32_t seg_len = min(uint32_t(groups - gi), in_item);
-            float acc[2][4];
+    auto stream = [&](auto in_shared) {
+        constexpr bool HELD = decltype(in_shared)::value;
+        while (left > 0) {
+            const Q4Item I = items[ci];
+            const int groups = I.groups;
+            int strip = int(local / uint32_t(groups));
+            int gi = int(local - uint32_t(strip) * uint32_t(groups));
+            uint32_t in_item = min(left, uint32_t(groups) * uint32_t(I.strips) - local);
+            left -= in_item;
+            local += in_item;
+            // Column 0 of the B fragment is the activation vector.  The other columns are never stored and read zeros wherever
+            // the walk is: multiplying zeros takes less power, and long lists run at the board's limit.
+            const auto x_lane = [&] {
+                if constexpr (HELD) return g == 0 ? smem_u32(held_x) + (I.group_begin - group_lo) * (2u * G) + 32u * t : smem_u32(zeros);
+                else return reinterpret_cast<const unsigned char*>(g == 0 ? reinterpret_cast<const uint4*>(I.x + 16 * t) : q4_zeros);
+            }();
+            const uint32_t x_step = g == 0 ? 2u * G : 0u;
+            const float2* item_sums = sums + (I.group_begin - group_lo);
+            while (in_item > 0) {
+                // one segment: the chunks of this warp that belong to one strip
+                const int seg_first = gi;
+                const uint32_t seg_len = min(uint32_t(groups - gi), in_item);
+                auto xp = x_lane + uint32_t(gi) * x_step;
+                float acc[2][2] = {};  // column 2 t of rows 16 h + g, 16 h + g + 8
+                for (uint32_t c = 0; c < seg_len; ++c, ++gi) {
+                    const float2 cs = HELD ? item_sums[gi] : group_sums<G, 32, false>(I.x + size_t(gi) * G, lane, nullptr);
+                    [[maybe_unused]] uint32_t xl[TPG][8];
+                    if constexpr (!HELD) load_group<TPG>(xp, xl);  // ahead of the copies: see there
+                    fetch_into(refill_lane);
+                    q4_cp_async_wait<DEPTH - 1>();  // this chunk has landed
+                    __syncwarp();
+                    float d[2][4];
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
+                    for (int j = 0; j < TPG; ++j) {
+                        uint32_t xr[8];
+                        if constexpr (HELD) {
+                            uint32_t lo[4], hi[4];
+                            q4_lds128(xp + 128 * j, lo);
+                            q4_lds128(xp + 128 * j + 16, hi);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[h][i] = 0.f;
-            for (uint32_t c = 0; c < seg_len; ++c, ++gi) {
-                const float2 cs = held ? item_sums[gi] : group_sums<G, 32>(I.x + size_t(gi) * G, lane);
-                fetch_into(refill_lane);
-                q4_cp_async_wait<DEPTH - 1>();  // this chunk has landed
-                __syncwarp();
-                float d[2][4];
+                            for (int i = 0; i < 4; ++i) {
+                                xr[i] = lo[i];
+                                xr[4 + i] = hi[i];
+                            }
+                        } else {
 #pragma unroll
-                for (int j = 0; j < TPG; ++j) {
-                    const uint4* xg = reinterpret_cast<const uint4*>(x_lane + size_t(gi) * G) + 8 * j;  // L1-resident
-                    const uint4 xa = __ldg(xg);
-                    const uint4 xb = __ldg(xg + 1);
-                    const uint32_t xr[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+                            for (int i = 0; i < 8; ++i) xr[i] = xl[j][i];
+                        }
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        uint32_t ww[4];
-                        q4_lds128(slot_lane + j * 1024 + h * 512, ww);
+                        for (int h = 0; h < 2; ++h) {
+                            uint32_t ww[4];
+                            q4_lds128(slot_lane + j * 1024 + h * 512, ww);
 #pragma unroll
-                        for (int m = 0; m < 4; ++m) {
-                            uint32_t a[4];
-                            const uint32_t w8 = ww[m] >> 8;
-                            a[0] = lop_and_or(ww[m], 0x000F000Fu, 0x64006400u);  // row g,     columns c, c+1   (1024 + n)
-                            a[1] = lop_and_or(w8, 0x000F000Fu, 0x64006400u);     // row g + 8, columns c, c+1
-                            a[2] = lop_and_or(ww[m], 0x00F000F0u, 0x54005400u);  // row g,     columns c+2, c+3 (64 + n)
-                            a[3] = lop_and_or(w8, 0x00F000F0u, 0x54005400u);     // row g + 8, columns c+2, c+3
-                            if (j == 0 && m == 0)
-                                mma_f16_first(d[h], a, xr[0], xr[1], cs.y, cs.y);
-                            else
-                                mma_f16(d[h], a, xr[2 * m], xr[2 * m + 1]);
+                            for (int m = 0; m < 4; ++m) {
+                                uint32_t a[4];
+                                const uint32_t w8 = ww[m] >> 8;
+                                a[0] = lop_and_or(ww[m], 0x000F000Fu, 0x64006400u);  // row g,     columns c, c+1   (1024 + n)
+                                a[1] = lop_and_or(w8, 0x000F000Fu, 0x64006400u);     // row g + 8, columns c, c+1
+                                a[2] = lop_and_or(ww[m], 0x00F000F0u, 0x54005400u);  // row g,     columns c+2, c+3 (64 + n)
+                                a[3] = lop_and_or(w8, 0x00F000F0u, 0x54005400u);     // row g + 8, columns c+2, c+3
+                                if (j == 0 && m == 0)
+                                    mma_f16_first(d[h], a, xr[0], xr[1], cs.y, 0.f);
+                                else
+                                    mma_f16(d[h], a, xr[2 * m], xr[2 * m + 1]);
+                            }
                         }
                     }
-                }
-                const uint32_t so_lane = slot_lane + so_delta;
+                    const uint32_t so_lane = slot_lane + so_delta;
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const uint32_t so0 = lds32(so_lane + 64 * h);
-                    const uint32_t so1 = lds32(so_lane + 64 * h + 32);
-                    const float2 r0 = __half22float2(*reinterpret_cast<const __half2*>(&so0));  // (scale, offset)
-                    const float2 r1 = __half22float2(*reinterpret_cast<const __half2*>(&so1));
-                    fma2(r0.y, cs.x, cs.x, acc[h][0], acc[h][1]);
-                    fma2(r0.x, d[h][0], d[h][1], acc[h][0], acc[h][1]);
-                    fma2(r1.y, cs.x, cs.x, acc[h][2], acc[h][3]);
-                    fma2(r1.x, d[h][2], d[h][3], acc[h][2], acc[h][3]);
+                    for (int h = 0; h < 2; ++h) {
+                        const uint32_t so0 = lds32(so_lane + 64 * h);
+                        const uint32_t so1 = lds32(so_lane + 64 * h + 32);
+                        const float2 r0 = __half22float2(*reinterpret_cast<const __half2*>(&so0));  // (scale, offset)
+                        const float2 r1 = __half22float2(*reinterpret_cast<const __half2*>(&so1));
+                        acc[h][0] = fmaf(r0.x, d[h][0], fmaf(r0.y, cs.x, acc[h][0]));
+                        acc[h][1] = fmaf(r1.x, d[h][2], fmaf(r1.y, cs.x, acc[h][1]));
+                    }
+                    xp += x_step;
+                    __syncwarp();  // every lane has read the slot before the next refill targets it
+                    refill_lane = slot_lane;
+                    slot_lane += CH;
+                    if (slot_lane == ring_lane_end) slot_lane = ring_lane;
                 }
-                __syncwarp();  // every lane has read the slot before the next refill targets it
-                refill_lane = slot_lane;
-                slot_lane += CH;
-                if (slot_lane == ring_lane_end) slot_lane = ring_lane;
-            }
-            in_item -= seg_len;
-            // element 8 lane + 4 h + i is (row 16 h + g + 8 (i / 2), column 2 t + (i % 2)) of the strip
-            if (seg_first == 0 && gi == groups) {  // the whole strip was this warp's: store column 0
-                if (t == 0) {
+                in_item -= seg_len;
+                if (seg_first == 0 && gi == groups) {  // the whole strip was this warp's: store column 0
+                    if (t == 0) {
 #pragma unroll
-                    for (int h = 0; h < 2; ++h)
+                        for (int h = 0; h < 2; ++h)
 #pragma unroll
-                        for (int i = 0; i < 4; i += 2) {
-                            const int row = 32 * strip + 16 * h + g + 8 * (i >> 1);
-                            if (row < I.N) I.y[row] = acc[h][i];
-                        }
+                            for (int i = 0; i < 2; ++i) {
+                                const int row = 32 * strip + 16 * h + g + 8 * i;
+                                if (row < I.N) I.y[row] = acc[h][i];
+                            }
+                    }
+                } else {
+                    // A strip shared with neighbouring warps: leave a piece (column 0: floats 4 g .. 4 g + 3 = rows g, g + 8,
+                    // 16 + g, 24 + g).  A warp has at most one strip that began before its range (slot 0) and one that ends
+                    // beyond it (slot 1).
+                    const bool later = seg_first != 0;  // began before this range
+                    if (t == 0)
+                        *reinterpret_cast<float4*>(pieces + (size_t(2 * gw) + (later ? 0 : 1)) * kPieceFloats + 4 * g) =
+                            make_float4(acc[0][0], acc[0][1], acc[1][0], acc[1][1]);
+                    const int owner = later ? warps[gw].owner : gw, parts = warps[owner].parts;
+                    __threadfence();  // the piece is visible before the counter moves
+                    __syncwarp();
+                    int arrived = 0;
+                    if (lane == 0) arrived = atomicAdd(&warps[owner].arrived, 1);
+                    arrived = __shfl_sync(0xFFFFFFFFu, arrived, 0);
+                    if (arrived == parts - 1) {  // all pieces are there: add them in warp order
+                        __threadfence();
+                        float sum = __ldcg(pieces + (size_t(2 * owner) + 1) * kPieceFloats + lane);
+                        for (int k = 1; k < parts; ++k) sum += __ldcg(pieces + size_t(2 * (owner + k)) * kPieceFloats + lane);
+                        const int row = 32 * strip + (lane >> 2) + 8 * (lane & 1) + 16 * ((lane >> 1) & 1);
+                        if (row < I.N) I.y[row] = sum;
+                        if (lane == 0) warps[owner].arrived = 0;  // for the next run
+                    }
                 }
-            } else {
-                // A strip shared with neighbouring warps: leave a piece (column 0: floats 4 g .. 4 g + 3 = rows g, g + 8,
-                // 16 + g, 24 + g).  A warp has at most one strip that began before its range (slot 0) and one that ends
-                // beyond it (slot 1).
-                const bool later = seg_first != 0;  // began before this range
-                if (t == 0)
-                    *reinterpret_cast<float4*>(pieces + (size_t(2 * gw) + (later ? 0 : 1)) * kPieceFloats + 4 * g) =
-                        make_float4(acc[0][0], acc[0][2], acc[1][0], acc[1][2]);
-                const int owner = later ? warps[gw].owner : gw, parts = warps[owner].parts;
-                __threadfence();  // the piece is visible before the counter moves
-                __syncwarp();
-                int arrived = 0;
-                if (lane == 0) arrived = atomicAdd(&warps[owner].arrived, 1);
-                arrived = __shfl_sync(0xFFFFFFFFu, arrived, 0);
-                if (arrived == parts - 1) {  // all pieces are there: add them in warp order
-                    __threadfence();
-                    float sum = __ldcg(pieces + (size_t(2 * owner) + 1) * kPieceFloats + lane);
-                    for (int k = 1; k < parts; ++k) sum += __ldcg(pieces + size_t(2 * (owner + k)) * kPieceFloats + lane);
-                    const int row = 32 * strip + (lane >> 2) + 8 * (lane & 1) + 16 * ((lane >> 1) & 1);
-                    if (row < I.N) I.y[row] = sum;
-                    if (lane == 0) warps[owner].arrived = 0;  // for the next run
+                if (gi == groups) {
+                    gi = 0;
+                    ++strip;
                 }
             }
-            if (gi == groups) {
-                gi = 0;
-                ++strip;
-            }
+            ++ci;
+            local = 0;
         }
-        ++ci;
-        local = 0;
-    }
+    };
+    if (held) stream(std::true_type{});
+    else stream(std::false_type{});
     q4_cp_async_wait<0>();
 }
 
@@ -309,7 +340,7 @@ int check_list(const tetra_q4_problem* p, int count, int G) {
 
 template <int G, int DEPTH>
 cudaError_t run_main(unsigned char* ws, int sms, cudaStream_t s) {
-    const size_t smem = size_t(kQ4ListWarps) * DEPTH * q4_chunk_bytes(G) + kQ4ListSums * sizeof(float2);
+    const size_t smem = size_t(kQ4ListWarps) * DEPTH * q4_chunk_bytes(G) + list_held_groups<G>() * sizeof(float2) + kQ4TileZeros + kQ4ListX;
     static PerDeviceOnce once;
     cudaError_t e = once.run([smem] {
         return cudaFuncSetAttribute(k_q4_list_main<G, DEPTH>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
@@ -428,7 +459,7 @@ int tetra_q4_list_run(void* workspace_dev, int G, void* stream) {
     if (device_sms(&sms) != cudaSuccess) return TETRA_ERR_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     unsigned char* ws = static_cast<unsigned char*>(workspace_dev);
-    const cudaError_t e = G == 128 ? run_main<128, 2>(ws, sms, s) : run_main<64, 6>(ws, sms, s);
+    const cudaError_t e = G == 128 ? run_main<128, 3>(ws, sms, s) : run_main<64, 6>(ws, sms, s);
     return e == cudaSuccess ? TETRA_OK : TETRA_ERR_CUDA;
 }
 

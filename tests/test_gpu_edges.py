@@ -143,7 +143,8 @@ def test_q4_shapes(tt, N, K, G, batch):
 
 # Lists with fewer chunks than warps, strips that many warps share, many small matrices, more groups per CTA than are held.
 @pytest.mark.parametrize("shapes,G", [([(1, 64)], 64), ([(40, 128), (1, 256), (33, 128)], 128), ([(32, 64 * 900)], 64),
-                                      ([(64, 64)] * 300, 64), ([(32, 65536)] * 40, 64)])
+                                      ([(64, 64)] * 300, 64), ([(32, 65536)] * 40, 64),
+                                      ([(64, 1280)] * 200, 128), ([(32, 64 * 320)] * 20, 64)])
 def test_q4_list_shapes(tt, shapes, G):
     from oracle import q4 as oq
     items, hosts = [], []
