@@ -361,6 +361,9 @@ __device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, uns
                 asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "r"(src + 512));
                 asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(h.x), "=r"(h.y), "=r"(h.z), "=r"(h.w) : "r"(src + 1024));
             }
+            LaneX X;
+            load_lane_x(xq_p + (joint ? lane_col : uint32_t(cg * 32 + lane)) * uint32_t(kXqBytesPerCol),
+                        !joint || lane_in, X);
             // prefetch the next pass's record (or the first one of this warp's next unit)
             const uint4* next = nullptr;
             if (pass + 1 < full_passes) {
@@ -379,9 +382,6 @@ __device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, uns
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 1024), "l"(next + 2 * Bu));
             }
             asm volatile("cp.async.commit_group;");
-            LaneX X;
-            load_lane_x(xq_p + (joint ? lane_col : uint32_t(cg * 32 + lane)) * uint32_t(kXqBytesPerCol),
-                        !joint || lane_in, X);
             record_accumulate(sm_tab, a, b, h, X, acc);  // acc is zero when the joint pass begins
             pass_parity ^= 1;
             if (!joint) {
