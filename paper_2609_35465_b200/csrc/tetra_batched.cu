@@ -19,9 +19,9 @@
 //   conflict-free, an MMA pair (k16 + k8) multiplies sixteen blocks of ONE column with eight vectors, and the
 //   block's scale reaches the lanes that hold its results by a shuffle.
 // The line lies where the tensor pipe's time for the zeros overtakes the tile: 4096 x 4096 with 2 / 4 / 8 / 16 vectors
-// takes 6.7 / 7.5 / 9.3 / 13.3 us block diagonal and 8.5 / 8.7 / 9.0 / 11.1 us dense (11.9 us for three vectors and
-// 27.2 us for sixteen at 4096 x 12288 with int8 planes, activations staged by the CTA and a combining kernel;
-// now 7.4 and 24.6 us).
+// takes 6.7 / 7.5 / 9.3 / 13.3 us block diagonal and 8.5 / 8.7 / 8.9 / 10.3 us dense (13.5 us for three vectors and
+// 27.8 us for sixteen at 4096 x 12288 with int8 planes, activations staged by the CTA and a combining kernel;
+// now 7.5 and 22.5 us).
 //
 // A warp's step is NT row tiles x four block columns.  The sixteen warps of a CTA take every sixteenth column quad, so a
 // warp needs nothing from the others until the end: its words come straight from global memory one step ahead, the four

@@ -37,7 +37,9 @@ namespace tetra {
 static_assert(kListMax == TETRA_LIST_MAX, "list length limit must agree with the header");
 
 constexpr int kListWarps = 16, kListThreads = 32 * kListWarps;
-constexpr int kChunkRows = 128;  // rows whose partial sums share the shared-memory buffer
+// A CTA's rows are taken in chunks whose partial sums, scales and tails share shared memory; a chunk has at least this
+// many rows if the CTA has them, and more where there is room: see launch_gemv_list.
+constexpr int kChunkRows = 128;
 
 // Kernel parameters: the list and its split over the grid.  CTAs [cta_begin[i], cta_begin[i + 1]) work on matrix i
 // (entries beyond the list: never reached); the first `extra` of them take base + 1 row groups, the others base.
@@ -58,6 +60,7 @@ struct ListParams {
     int32_t cta_begin[kListMax];
     int32_t image_cols;         // largest number of words per row, if the image fits
     int32_t batch;
+    int32_t chunk;              // row groups of a chunk
     ListMatrix m[kListMax];
 };
 
@@ -65,15 +68,15 @@ struct ListSmem {
     // offsets from the 16 KiB-aligned table copy; total includes the alignment slack
     uint32_t xq, xtail, ring, part, rs, tail, total;
 };
-__host__ __device__ inline ListSmem list_smem(int image_cols) {
+__host__ __device__ inline ListSmem list_smem(int image_cols, int chunk_rows) {  // chunk_rows: a multiple of eight
     ListSmem S;
     S.xq = uint32_t(kFastBytes);
     S.xtail = S.xq + uint32_t(image_cols) * kXqBytesPerCol;               // float [24]: x beyond the last word
     S.ring = S.xtail + 96u;
     S.part = S.ring + kListWarps * 3072u;
-    S.rs = S.part + uint32_t(kChunkRows * kListWarps * 4);                // float [chunk rows]: row scales
-    S.tail = S.rs + uint32_t(kChunkRows * 4);                             // half [chunk rows][24]: tails
-    S.total = S.tail + uint32_t(kChunkRows * 24 * 2) + kSmAlign;
+    S.rs = S.part + uint32_t(chunk_rows * kListWarps * 4);                // float [chunk rows]: row scales
+    S.tail = S.rs + uint32_t(chunk_rows * 4);                             // half [chunk rows][24]: tails
+    S.total = S.tail + uint32_t(chunk_rows * 24 * 2) + kSmAlign;
     return S;
 }
 
@@ -120,11 +123,12 @@ __device__ __forceinline__ float warp_row_sums(float* red, int lane, const float
 template <int R, bool IMAGE>
 __global__ void __launch_bounds__(kListThreads, 1)
 k_gemv_list(const DeviceTables* __restrict__ tab, const __grid_constant__ ListParams L) {
-    constexpr int THREADS = kListThreads, W = kListWarps, CHUNK = kChunkRows / R;
+    constexpr int THREADS = kListThreads, W = kListWarps;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_release();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const ListSmem S = list_smem(IMAGE ? L.image_cols : 0);
+    const int CHUNK = L.chunk;
+    const ListSmem S = list_smem(IMAGE ? L.image_cols : 0, (CHUNK * R + 7) & ~7);
     const uint32_t sm_raw = smem_u32(smem_raw);
     unsigned char* smem = smem_raw + (((sm_raw + kSmAlign - 1) & ~(kSmAlign - 1)) - sm_raw);
     const uint32_t sm_tab = smem_u32(smem);
@@ -355,8 +359,8 @@ struct ListShape {
 };
 
 // Splits the list's row groups of R rows over at most `ctas` CTAs; fills P's shares and returns the CTAs used and
-// the passes of the busiest warp.
-int split_list(const ListShape& Q, int R, int ctas, ListParams& P, int* warp_passes) {
+// the passes of the busiest warp and the row groups of the largest share.
+int split_list(const ListShape& Q, int R, int ctas, ListParams& P, int* warp_passes, int* cta_groups) {
     int n[kListMax] = {}, groups[kListMax] = {}, used = 0;
     long long work = 0, total = 0;
     for (int i = 0; i < Q.count; ++i) {
@@ -387,7 +391,7 @@ int split_list(const ListShape& Q, int R, int ctas, ListParams& P, int* warp_pas
         --n[at];
         --used;
     }
-    *warp_passes = 0;
+    *warp_passes = *cta_groups = 0;
     int begin = 0;
     for (int i = 0; i < kListMax; ++i) {
         P.cta_begin[i] = i < Q.count ? begin : 0x7FFFFFFF;
@@ -401,6 +405,7 @@ int split_list(const ListShape& Q, int R, int ctas, ListParams& P, int* warp_pas
         const long long cells = (long long)(M.base + (M.extra ? 1 : 0)) * bs;
         const int passes = int(((cells + 31) / 32 + kListWarps - 1) / kListWarps);
         if (passes > *warp_passes) *warp_passes = passes;
+        if (M.base + (M.extra ? 1 : 0) > *cta_groups) *cta_groups = M.base + (M.extra ? 1 : 0);
         begin += n[i];
     }
     return begin;
@@ -442,20 +447,31 @@ cudaError_t launch_gemv_list(const ListDesc& list, int batch, const void* table,
     P.batch = batch;
     P.image_cols = Q.max_blocks;
     const DeviceTables* tab = static_cast<const DeviceTables*>(table);
-    int passes = 0;
-    int grid = split_list(Q, 8, sms, P, &passes);
-    const uint32_t smem = list_smem(Q.max_blocks).total;
-    if (smem > 227u * 1024u)  // more columns than the shared-memory image can hold
-        return launch_pdl(k_gemv_list<8, false>, grid, kListThreads, list_smem(0).total, s, tab, P);
+    int passes = 0, groups = 0;
+    int grid = split_list(Q, 8, sms, P, &passes, &groups);
+    constexpr uint32_t kMaxSmem = 227 * 1024;
+    // As few chunks as shared memory allows, of equal size: the rows behind a boundary cost a CTA-wide round of their own
+    // (four launches of a 4B layer, whose gate and up matrices come to 136 rows a CTA: 29.7 us with 128 and 8, 27.4 us).
+    const uint32_t fixed = list_smem(Q.max_blocks, 0).total, row_bytes = (list_smem(Q.max_blocks, 8).total - fixed) / 8;
+    const int room = fixed < kMaxSmem ? int((kMaxSmem - fixed) / row_bytes) & ~7 : 0;
+    if (room < kChunkRows) {  // more columns than the shared-memory image can hold
+        P.chunk = kChunkRows / 8;
+        return launch_pdl(k_gemv_list<8, false>, grid, kListThreads, list_smem(0, kChunkRows).total, s, tab, P);
+    }
+    auto launch = [&](auto kernel, int R) {
+        const int chunks = (groups * R + room - 1) / room;
+        P.chunk = (groups + chunks - 1) / chunks;
+        return launch_pdl(kernel, grid, kListThreads, list_smem(Q.max_blocks, (P.chunk * R + 7) & ~7).total, s, tab, P);
+    };
     // A warp's pass over eight rows is a chain of eight blocks, and every warp runs a whole number of them: half
     // records when their chain is shorter.  A block costs about 82 instructions, a pass about 150 more (record and
     // activations in, row ends): measured on both sides of the line, 12288 x 4096: four passes of eight rows 9.4 us,
     // seven of four 10.2 us; 6144 x 2560: two of eight 6.1 us, three of four 5.6 us.
     const long long chain8 = (long long)passes * (8 * 82 + 150);
-    grid = split_list(Q, 4, sms, P, &passes);
-    if ((long long)passes * (4 * 82 + 150) < chain8) return launch_pdl(k_gemv_list<4, true>, grid, kListThreads, smem, s, tab, P);
-    grid = split_list(Q, 8, sms, P, &passes);
-    return launch_pdl(k_gemv_list<8, true>, grid, kListThreads, smem, s, tab, P);
+    grid = split_list(Q, 4, sms, P, &passes, &groups);
+    if ((long long)passes * (4 * 82 + 150) < chain8) return launch(k_gemv_list<4, true>, 4);
+    grid = split_list(Q, 8, sms, P, &passes, &groups);
+    return launch(k_gemv_list<8, true>, 8);
 }
 
 }  // namespace tetra

@@ -54,11 +54,13 @@ def test_single_matrix(tt, table, orc, N, K, tail_mode):
     check(orc, m, d["y"].cpu().numpy(), "%d x %d" % (N, K))
 
 
-# A CTA works on one matrix: lists of very unequal matrices, of more and of fewer row groups than CTAs.
+# A CTA works on one matrix: lists of very unequal matrices, of more and of fewer row groups than CTAs; long rows that leave
+# the other matrix's rows room for half a CTA's share.
 @pytest.mark.parametrize("rows,K", [((1, 1, 1, 1, 1, 1, 1, 1), 24), ((4000, 8), 24 * 40), ((8, 9000, 16, 1), 24 * 12 + 7),
-                                    ((700, 700, 700), 24 * 70 + 2)])
+                                    ((700, 700, 700), 24 * 70 + 2), ((60001, 64), (24, 24 * 1250))])
 def test_list_split(tt, table, orc, rows, K):
-    ms = [make_matrix(72, 10 * i + K, n, K, True, batch=1) for i, n in enumerate(rows)]
+    Ks = K if isinstance(K, tuple) else (K,) * len(rows)
+    ms = [make_matrix(72, 10 * i + k, n, k, True, batch=1) for i, (n, k) in enumerate(zip(rows, Ks))]
     items = [device_matrix(tt, table, m, torch.from_numpy(m["x"][0]).cuda()) for m in ms]
     tt.tetra_gemv_list(tt.make_problems(items), table)
     torch.cuda.synchronize()
