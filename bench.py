@@ -30,14 +30,14 @@ UNIT = "GB/s"
 NOMINAL_HBM_GBS = 8000.0
 FALLBACK_HBM_GBS = 6650.0
 # DRAM bytes per algorithmic byte of k_gemv_units, from the ncu capture summarised in
-# profiles/k_gemv_units_qwen3_8b.md (dram__bytes_read.sum + dram__bytes_write.sum = 202.5 MB
+# profiles/k_gemv_units_qwen3_8b.md (dram__bytes_read.sum + dram__bytes_write.sum = 203.9 MB
 # for the 198.4 MB of the first 4 layers; every code byte is read once, so traffic grows in
 # proportion to the matrices read and the full pass is scaled by its byte count).
-TRAFFIC_PER_ALGORITHMIC_BYTE = 1.02
+TRAFFIC_PER_ALGORITHMIC_BYTE = 1.03
 # Warp-instructions of k_gemv_units per 32 blocks (one block per lane), by pipe, and wavefronts of the
-# shared-memory/L1 data pipe, from the same capture (smsp__inst_executed.sum and
-# sm__inst_executed_pipe_{alu,fmaheavy,lsu}.sum over the blocks processed / 32).
-KERNEL_COUNTERS = {"instr": 85.9, "alu": 40.1, "fmaheavy": 32.0, "lsu": 9.6, "wavefronts": 21.0}
+# shared-memory/L1 data pipe, from the same capture (smsp__inst_executed.sum; the pipes from their shares of peak
+# over the active cycles, times the blocks processed / 32).
+KERNEL_COUNTERS = {"instr": 80.2, "alu": 34.1, "fmaheavy": 32.8, "lsu": 9.6, "wavefronts": 22.1}
 
 
 def issue_bound_gbs(sm_mhz, sms=148):
@@ -615,7 +615,7 @@ def main():
             del packs, gg, qn, sc, of
             torch.cuda.empty_cache()
         # the same projection shapes as ONE planned list (v, o and down of every layer: 3 x layers matrices,
-        # distinct copies, more than L2 together), three launches per pass (tetra_q4_list_run)
+        # distinct copies, more than L2 together), one launch per pass (tetra_q4_list_run)
         qitems = []
         for layer in range(model.layers):
             for name, qN, qK, qG, _ in q4_shapes[:3]:
@@ -656,7 +656,7 @@ def main():
                                                "below its maximum); the burst figure is 20 passes from idle",
                                        "single_launches_sum_ms": sum(q4[n]["us"] for n in ("v_proj", "o_proj", "down_proj"))
                                                                  * model.layers * 1e-3,
-                                       "launches_per_pass": 3}
+                                       "launches_per_pass": 1}
         del qitems, qws
         torch.cuda.empty_cache()
         out["q4_gemv"] = q4
