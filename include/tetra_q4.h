@@ -53,10 +53,8 @@ int tetra_q4_pack(const void *q_dev, const void *scale_dev, const void *offset_d
  * TETRA_Q4_MAX_BATCH.  x_dev: float16 [batch][K], 16-byte aligned; y_dev:
  * float32 [batch][N].  Products of exact float16 values are accumulated in
  * float32 (tensor-core m16n8k16, one accumulator per group, then scale and
- * offset in float32); one vector with a matrix of many rows is multiplied in
- * whole numbers instead (its group sums are exact), so the last bits of its
- * result may differ from the same vector's in a batch.  One launch, no scratch
- * memory, bit-identical from run to run. */
+ * offset in float32).  One launch, no scratch memory, bit-identical from run
+ * to run. */
 int tetra_q4_gemv(const void *packed_dev, const void *x_dev, float *y_dev, int N, int K, int G, int batch,
                   void *stream);
 

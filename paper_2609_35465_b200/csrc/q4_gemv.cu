@@ -101,12 +101,9 @@ __global__ void __launch_bounds__(256) k_q4_pack(const uint8_t* __restrict__ q, 
 // are is worked out while the kernel waits for its predecessor (looked for afterwards, piece by piece, it was 2.2 us of
 // a 5.1 us launch: 1024 x 4096, G = 128, now 3.9 us; 12288 x 4096, G = 64, 9.9 -> 8.2 us).
 // Addresses advance by running pointers: the loop body is dequantise, multiply, scale.
-// DIGITS: one vector, its activations as six int8 digits in the columns of B (q4_common.cuh), products exact in int32.
-// Half the MMAs, no bias to take off, 24 logic operations per chunk instead of 40: large matrices ran at the board's
-// power limit, and this takes less.
 // XS: the activations are staged in shared memory (rows padded by 16 bytes so that the eight vectors' reads
 // fall into different banks); otherwise they are read through L1.
-template <int G, int DEPTH, bool XS, bool DIGITS>
+template <int G, int DEPTH, bool XS>
 __global__ void __launch_bounds__(kQ4Threads, kQ4CtasPerSm)
 k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x, float* __restrict__ y, int N, int K,
           int batch) {
@@ -184,10 +181,7 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
             for (int j = 0; j < AHEAD; ++j) {
                 if (i0 + uint32_t(j * kQ4Threads) >= total) break;  // warp-uniform
                 const uint32_t i = i0 + uint32_t(j * kQ4Threads + lane), v = __umulhi(i, inv), c8 = i - v * per_vec;
-                if (XS && i < total) {
-                    if constexpr (DIGITS) store_digits(u[j], xs_base + size_t(c8) * 8, q4_digit_stride(K));
-                    else *reinterpret_cast<uint4*>(xs_base + size_t(v) * xs_stride + size_t(c8) * 16) = u[j];
-                }
+                if (XS && i < total) *reinterpret_cast<uint4*>(xs_base + size_t(v) * xs_stride + size_t(c8) * 16) = u[j];
                 const float2 a0 = __half22float2(*reinterpret_cast<const __half2*>(&u[j].x)), b0 = __half22float2(*reinterpret_cast<const __half2*>(&u[j].y));
                 const float2 a1 = __half22float2(*reinterpret_cast<const __half2*>(&u[j].z)), b1 = __half22float2(*reinterpret_cast<const __half2*>(&u[j].w));
                 float lo = (a0.x + a0.y) + (a1.x + a1.y), hi = (b0.x + b0.y) + (b1.x + b1.y);  // k % 4 in {0, 1} / {2, 3}
@@ -196,27 +190,22 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
                     lo += __shfl_xor_sync(0xFFFFFFFFu, lo, o);
                     hi += __shfl_xor_sync(0xFFFFFFFFu, hi, o);
                 }
-                if (lane % (G / 8) == 0 && i < total) {
-                    if constexpr (DIGITS) gs[c8 / (G / 8) * 8 + 7] = make_float2(nan_unless_finite(lo + hi), 0.f);
-                    else gs[c8 / (G / 8) * 8 + v] = make_float2(lo + hi, -(1024.f * lo + 64.f * hi));
-                }
+                if (lane % (G / 8) == 0 && i < total) gs[c8 / (G / 8) * 8 + v] = make_float2(lo + hi, -(1024.f * lo + 64.f * hi));
             }
         }
     }
     for (int i = threadIdx.x; i < groups * 8; i += kQ4Threads)
-        if (DIGITS ? (i & 7) != 7 : (i & 7) >= batch) gs[i] = make_float2(0.f, 0.f);
-    const uint32_t zeros = DIGITS ? uint32_t(kQ4Digits) * q4_digit_stride(K) : uint32_t(batch) * xs_stride;  // behind the activations
-    if (XS && threadIdx.x < kQ4TileZeros / 16) reinterpret_cast<uint4*>(xs_base + zeros)[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
+        if ((i & 7) >= batch) gs[i] = make_float2(0.f, 0.f);
+    if (XS && threadIdx.x < kQ4TileZeros / 16) reinterpret_cast<uint4*>(xs_base + size_t(batch) * xs_stride)[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
 
     // Column g of B is vector g.  Columns at or beyond batch are never stored and read zeros wherever the walk is
     // (x_step 0): multiplying zeros takes less power, and large matrices run at the board's limit.
-    const bool fed = g < (DIGITS ? kQ4Digits : batch);
-    const uint32_t x_step = fed ? (DIGITS ? 1u : 2u) * G : 0u;
+    const bool fed = g < batch;
+    const uint32_t x_step = fed ? 2u * G : 0u;
     // this lane's 16 activations of the first tile of group 0: a shared address or a pointer
     const auto x_lane = [&] {
-        if constexpr (DIGITS) return smem_u32(xs_base) + (fed ? uint32_t(g) * q4_digit_stride(K) + 16u * t : zeros);
-        else if constexpr (XS) return smem_u32(xs_base) + (fed ? uint32_t(g) * xs_stride + 32u * t : zeros);
+        if constexpr (XS) return smem_u32(xs_base) + (fed ? uint32_t(g) * xs_stride + 32u * t : uint32_t(batch) * xs_stride);
         else return fed ? reinterpret_cast<const unsigned char*>(x + size_t(g) * K + 16 * t) : reinterpret_cast<const unsigned char*>(q4_zeros);
     }();
     const uint32_t gs_lane = smem_u32(gs) + uint32_t(t) * 16;
@@ -246,42 +235,38 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
             q4_cp_async_wait<DEPTH - 1>();  // this chunk has landed
             __syncwarp();
             float d[2][4];
-            if constexpr (DIGITS) {
-                digit_sums<TPG>(slot_lane, xo, d);
-            } else {
 #pragma unroll
-                for (int j = 0; j < TPG; ++j) {
-                    uint32_t xr[8];
-                    if constexpr (XS) {
-                        uint32_t lo[4], hi[4];
-                        q4_lds128(xo + 128 * j, lo);
-                        q4_lds128(xo + 128 * j + 16, hi);
+            for (int j = 0; j < TPG; ++j) {
+                uint32_t xr[8];
+                if constexpr (XS) {
+                    uint32_t lo[4], hi[4];
+                    q4_lds128(xo + 128 * j, lo);
+                    q4_lds128(xo + 128 * j + 16, hi);
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            xr[i] = lo[i];
-                            xr[4 + i] = hi[i];
-                        }
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) xr[i] = xl[j][i];
+                    for (int i = 0; i < 4; ++i) {
+                        xr[i] = lo[i];
+                        xr[4 + i] = hi[i];
                     }
+                } else {
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        uint32_t ww[4];
-                        q4_lds128(slot_lane + j * 1024 + h * 512, ww);
+                    for (int i = 0; i < 8; ++i) xr[i] = xl[j][i];
+                }
 #pragma unroll
-                        for (int m = 0; m < 4; ++m) {
-                            uint32_t a[4];
-                            const uint32_t w8 = ww[m] >> 8;
-                            a[0] = lop_and_or(ww[m], 0x000F000Fu, 0x64006400u);  // row g,     columns c, c+1   (1024 + n)
-                            a[1] = lop_and_or(w8, 0x000F000Fu, 0x64006400u);     // row g + 8, columns c, c+1
-                            a[2] = lop_and_or(ww[m], 0x00F000F0u, 0x54005400u);  // row g,     columns c+2, c+3 (64 + n)
-                            a[3] = lop_and_or(w8, 0x00F000F0u, 0x54005400u);     // row g + 8, columns c+2, c+3
-                            if (j == 0 && m == 0)
-                                mma_f16_first(d[h], a, xr[0], xr[1], __uint_as_float(cs[1]), __uint_as_float(cs[3]));
-                            else
-                                mma_f16(d[h], a, xr[2 * m], xr[2 * m + 1]);
-                        }
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t ww[4];
+                    q4_lds128(slot_lane + j * 1024 + h * 512, ww);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {
+                        uint32_t a[4];
+                        const uint32_t w8 = ww[m] >> 8;
+                        a[0] = lop_and_or(ww[m], 0x000F000Fu, 0x64006400u);  // row g,     columns c, c+1   (1024 + n)
+                        a[1] = lop_and_or(w8, 0x000F000Fu, 0x64006400u);     // row g + 8, columns c, c+1
+                        a[2] = lop_and_or(ww[m], 0x00F000F0u, 0x54005400u);  // row g,     columns c+2, c+3 (64 + n)
+                        a[3] = lop_and_or(w8, 0x00F000F0u, 0x54005400u);     // row g + 8, columns c+2, c+3
+                        if (j == 0 && m == 0)
+                            mma_f16_first(d[h], a, xr[0], xr[1], __uint_as_float(cs[1]), __uint_as_float(cs[3]));
+                        else
+                            mma_f16(d[h], a, xr[2 * m], xr[2 * m + 1]);
                     }
                 }
             }
@@ -308,20 +293,8 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
         }
         left -= seg_len;
         gi += int(seg_len);
-        // element e = 8 lane + 4 h + i is (row 16 h + g + 8 (i / 2), vector or digit 2 t + (i % 2)) of the strip
+        // element e = 8 lane + 4 h + i is (row 16 h + g + 8 (i / 2), vector 2 t + (i % 2)) of the strip
         if (seg_first == 0 && gi == groups) {  // the whole strip was this warp's
-            if constexpr (DIGITS) {
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-#pragma unroll
-                    for (int i = 0; i < 4; i += 2) {
-                        float sum = acc[h][i] * digit_weight(2 * t) + acc[h][i + 1] * digit_weight(2 * t + 1);
-                        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
-                        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 2);
-                        const int row = 32 * strip + 16 * h + g + 4 * i;
-                        if (t == 0 && row < N) y[row] = sum;
-                    }
-            } else
 #pragma unroll
             for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -359,12 +332,6 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
             for (int k = 0; k < 5; ++k) p[k] = k0 + k < c.y ? at[(k0 + k) * 512] : 0.f;
 #pragma unroll
             for (int k = 0; k < 5; ++k) total += p[k];
-        }
-        if constexpr (DIGITS) {  // a warp holds the eight columns of four rows
-            total *= digit_weight(v);
-            total += __shfl_xor_sync(0xFFFFFFFFu, total, 1);
-            total += __shfl_xor_sync(0xFFFFFFFFu, total, 8);
-            total += __shfl_xor_sync(0xFFFFFFFFu, total, 16);
         }
         const int row = 32 * (strip_begin + c.x) + r_in;
         if (row < N && v < batch) y[size_t(v) * N + row] = total;
@@ -440,21 +407,21 @@ int device_sm_count(int* sms) {
 
 constexpr size_t kQ4SmemLimit = 224 * 1024 / kQ4CtasPerSm - 2048;
 
-template <int G, int DEPTH, bool XS, bool DIGITS>
-constexpr size_t q4_smem_bytes(int K, int batch) {
+template <int G, int DEPTH>
+constexpr size_t q4_smem_bytes(int K, int batch, bool staged) {
     return size_t(K / G) * 64 + size_t(kQ4Warps) * 2048 + size_t(kQ4Warps) * DEPTH * q4_chunk_bytes(G) +
-           (DIGITS ? size_t(kQ4Digits) * q4_digit_stride(K) + kQ4TileZeros : XS ? size_t(batch) * (size_t(K) * 2 + 16) + kQ4TileZeros : 0);
+           (staged ? size_t(batch) * (size_t(K) * 2 + 16) + kQ4TileZeros : 0);
 }
 
-template <int G, int DEPTH, bool XS, bool DIGITS>
+template <int G, int DEPTH, bool XS>
 cudaError_t launch_q4_variant(const void* packed, const void* x, float* y, int N, int K, int batch, int sms,
                               cudaStream_t s) {
     const int strips = (N + 31) / 32;
     const int grid = strips < kQ4CtasPerSm * sms ? strips : kQ4CtasPerSm * sms;
-    const size_t smem = q4_smem_bytes<G, DEPTH, XS, DIGITS>(K, batch);
+    const size_t smem = q4_smem_bytes<G, DEPTH>(K, batch, XS);
     static PerDeviceOnce once;  // per instantiation
     cudaError_t e = once.run([] {
-        return cudaFuncSetAttribute(k_q4_gemv<G, DEPTH, XS, DIGITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kQ4SmemLimit));
+        return cudaFuncSetAttribute(k_q4_gemv<G, DEPTH, XS>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kQ4SmemLimit));
     });
     if (e != cudaSuccess) return e;
     if (smem > kQ4SmemLimit) return cudaErrorInvalidValue;
@@ -468,24 +435,18 @@ cudaError_t launch_q4_variant(const void* packed, const void* x, float* y, int N
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_q4_gemv<G, DEPTH, XS, DIGITS>, static_cast<const unsigned char*>(packed),
+    return cudaLaunchKernelEx(&cfg, k_q4_gemv<G, DEPTH, XS>, static_cast<const unsigned char*>(packed),
                               static_cast<const __half*>(x), y, N, K, batch);
 }
 
 template <int G, int DEPTH>
 cudaError_t launch_q4_gemv(const void* packed, const void* x, float* y, int N, int K, int batch, int sms,
                            cudaStream_t s) {
-    // One vector in whole numbers: fewer MMAs and logic operations per chunk, three times the work per activation while
-    // they are staged.  That pays from two strips per CTA on: 12288 x 4096, G = 64, 8.6 -> 7.4 us; 20000 x 2048 7.9 -> 7.1;
-    // 151936 x 4096 69.6 -> 58.0 us, no longer at the board's power limit; but 4096 x 12288, G = 128 (one strip)
-    // 8.0 -> 8.8 us and 1024 x 4096 3.8 -> 4.0 us.
-    if (batch == 1 && (N + 31) / 32 >= 2 * kQ4CtasPerSm * sms && q4_smem_bytes<G, DEPTH, true, true>(K, 1) <= kQ4SmemLimit)
-        return launch_q4_variant<G, DEPTH, true, true>(packed, x, y, N, K, batch, sms, s);
     // Staged wherever they fit: read through L1 the activations queue behind the weights' copies, which the same unit
     // takes in order (see q4_list.cu).
-    if (q4_smem_bytes<G, DEPTH, true, false>(K, batch) <= kQ4SmemLimit)
-        return launch_q4_variant<G, DEPTH, true, false>(packed, x, y, N, K, batch, sms, s);
-    return launch_q4_variant<G, DEPTH, false, false>(packed, x, y, N, K, batch, sms, s);
+    if (q4_smem_bytes<G, DEPTH>(K, batch, true) <= kQ4SmemLimit)
+        return launch_q4_variant<G, DEPTH, true>(packed, x, y, N, K, batch, sms, s);
+    return launch_q4_variant<G, DEPTH, false>(packed, x, y, N, K, batch, sms, s);
 }
 
 }  // namespace

@@ -121,8 +121,7 @@ def test_decode_packed_shapes(tt, table, orc, N, B):
 
 # Strips of 32 rows shared by two and more warps, CTAs with fewer chunks than warps, both group sizes.
 @pytest.mark.parametrize("N,K,G,batch", [(1, 64, 64, 1), (31, 128, 128, 8), (33, 192, 64, 1), (64, 15 * 64, 64, 3),
-                                         (32 * 148, 128 * 7, 128, 1), (32 * 148 * 2 + 1, 64 * 3, 64, 2), (96, 64 * 257, 64, 1),
-                                         (32 * 148 * 2 - 32, 64, 64, 1), (32 * 148 * 2 + 1, 64 * 5, 64, 1), (32 * 148 * 3, 128 * 5, 128, 1)])
+                                         (32 * 148, 128 * 7, 128, 1), (32 * 148 * 2 + 1, 64 * 3, 64, 2), (96, 64 * 257, 64, 1)])
 def test_q4_shapes(tt, N, K, G, batch):
     from oracle import q4 as oq
     q = synth.q4_nibbles(76, N, N, K)
@@ -142,31 +141,6 @@ def test_q4_shapes(tt, N, K, G, batch):
     want_rows = oq.rows(q, sc, of, ids, N, K, G).view(np.uint16)
     for out in (rows, rows8):
         assert np.array_equal(out.cpu().numpy().view(np.uint16), want_rows)
-
-
-# One vector as digits: the largest and smallest float16 magnitudes beside each other, zeros; a NaN or an infinity reaches
-# every row.
-@pytest.mark.parametrize("G", [64, 128])
-def test_q4_activation_range(tt, G):
-    from oracle import q4 as oq
-    N, K = 32 * 148 * 2 + 5, 512
-    q = synth.q4_nibbles(78, 0, N, K)
-    sc, of = synth.q4_scales_offsets(78, 0, N, K // G)
-    packed = tt.tetra_q4_pack(torch.from_numpy(q).cuda(), torch.from_numpy(sc).cuda(), torch.from_numpy(of).cuda(), N, K, G)
-    x = np.array([65504, -65504, 2.0 ** -24, -2.0 ** -24, 0, 2.0 ** -14, 1, -2047 * 2.0 ** -24], dtype=np.float16)
-    y = torch.empty((1, N), dtype=torch.float32, device="cuda")
-    for xs in (np.tile(x, K // 8), np.roll(np.tile(x, K // 8), 1), np.tile(x[2:6], K // 4), np.zeros(K, np.float16)):
-        xs = xs.reshape(1, K)
-        tt.tetra_q4_gemv(packed, torch.from_numpy(xs).cuda(), y, N, K, G, 1)
-        torch.cuda.synchronize()
-        want, tn = oq.gemv(q, sc, of, xs, N, K, G, 1)
-        assert_gemv_close(y.cpu().numpy(), {"y": want, "termnorm": tn}, "range")
-    for bad in (float("nan"), float("inf"), float("-inf")):
-        xs = torch.ones((1, K), dtype=torch.float16, device="cuda")
-        xs[0, 201] = bad
-        tt.tetra_q4_gemv(packed, xs, y, N, K, G, 1)
-        torch.cuda.synchronize()
-        assert torch.isnan(y).all()
 
 
 # Lists with fewer chunks than warps, strips that many warps share, many small matrices, more groups per CTA than are held.
