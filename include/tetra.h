@@ -13,6 +13,16 @@
  *   - work is enqueued on `stream` (a cudaStream_t passed as void*, NULL = the
  *     legacy default stream) and the call does not synchronise, except where
  *     stated;
+ *   - calls on one stream take effect in order.  The products read weights
+ *     (codes, row scales, tails, tables, planned workspaces) ahead of the end of
+ *     the kernel before them where that kernel allows it (programmatic dependent
+ *     launch).  tetra_pack_codes, tetra_q4_pack, the plan calls, copies and
+ *     ordinary kernels do not allow it, so a product that follows one of them
+ *     directly, in a captured graph too, multiplies what it wrote.  The products,
+ *     tetra_decode_packed and tetra_q4_rows do allow it: use a result of theirs (y,
+ *     coordinates, rows) as activations as it is, but as row scales, tail or codes
+ *     only behind a copy, an ordinary kernel or a synchronisation; the same goes for
+ *     a kernel of the caller's that executes griddepcontrol.launch_dependents;
  *   - arguments are validated on the host before anything is launched; a
  *     rejected call launches nothing;
  *   - the entry points may be called from several host threads at once (the

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(256) k_q4_pack(const uint8_t* __restrict__ q, 
     constexpr int TPG = G / 64, CH = q4_chunk_bytes(G);
     const int strips = (N + 31) / 32, groups = K / G;
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    pdl_release();
+    // No pdl_release: the products read the packed matrix ahead of their wait (see tetra_device.cuh).
     pdl_wait();  // the matrix may come from, the packed one be read by, the kernel before
     const size_t chunks = size_t(strips) * groups;
     for (size_t chunk = (blockIdx.x * size_t(blockDim.x) + threadIdx.x) >> 5; chunk < chunks;

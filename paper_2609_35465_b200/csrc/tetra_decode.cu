@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(256, 4) k_pack(const uint8_t* __restrict__ cod
                                                  const DeviceTables* __restrict__ tab,
                                                  uint4* __restrict__ packed, int N, int B) {
     __shared__ uint16_t abx[4096];
-    pdl_release();
+    // No pdl_release: the products read codes ahead of their wait (see tetra_device.cuh).
     for (int i = threadIdx.x; i < 512; i += blockDim.x)
         reinterpret_cast<uint4*>(abx)[i] = __ldg(reinterpret_cast<const uint4*>(tab->trellis_to_abx) + i);
     __syncthreads();

@@ -52,11 +52,17 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 }
 
 // ---------------------------------------------------------------------------
-// Programmatic dependent launch.  Every GEMV kernel lets the next kernel of the
-// stream start early (pdl_release) and waits for its own predecessor only when
-// it first touches data a predecessor may have produced (pdl_wait): tables and
-// codes are constants of the model, activations are not.  Both are no-ops for a
-// kernel launched without the attribute.
+// Programmatic dependent launch.  A kernel that calls pdl_release lets the next
+// kernel of the stream start early; pdl_wait waits until every kernel before has
+// completed and its writes are visible.  Both are no-ops for a kernel launched
+// without the attribute.
+//   * The products read weights (codes, row scales, tails, tables, plans) ahead of
+//     pdl_wait, activations and everything else behind it.  Nothing orders a read
+//     ahead of the wait behind the stores of a predecessor that has released, so a
+//     kernel that writes weights (k_pack, k_q4_pack) never calls pdl_release,
+//     wherever its stores are: its dependents start when it has completed.
+//   * A kernel that releases also waits, all of its CTAs, so that the completion of
+//     a kernel implies that of all kernels before it.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
