@@ -47,20 +47,29 @@ def build(force: bool = False, verbose: bool = False) -> str:
     flags = list(FLAGS) + os.environ.get("TETRA_EXTRA_FLAGS", "").split()
     if verbose:
         flags += ["-Xptxas", "-v"]
+    # built beside their place and moved there whole: a program that is running keeps the library it has loaded
+    tmp_lib, tmp_binding = ["%s.tmp.%d" % (path, os.getpid()) for path in (LIB, BINDING)]
     objs = []
     procs = []
-    for src in SOURCES:
-        obj = os.path.join(CSRC, os.path.splitext(src)[0] + ".o")
-        objs.append(obj)
-        procs.append(subprocess.Popen([NVCC] + flags + ["-c", os.path.join(CSRC, src), "-o", obj], cwd=CSRC))
-    tmp_binding = BINDING + ".tmp.%d" % os.getpid()
-    procs.append(subprocess.Popen(_binding_command(tmp_binding)))
-    if any([p.wait() != 0 for p in procs]):
-        raise RuntimeError("the compiler failed")
-    tmp = LIB + ".tmp.%d" % os.getpid()
-    subprocess.run([NVCC, "-shared", "-o", tmp] + objs + ["-lcudart"], check=True, cwd=CSRC)
-    os.replace(tmp, LIB)
-    os.replace(tmp_binding, BINDING)
+    try:
+        for src in SOURCES:
+            obj = os.path.join(CSRC, os.path.splitext(src)[0] + ".o")
+            objs.append(obj)
+            procs.append(subprocess.Popen([NVCC] + flags + ["-c", os.path.join(CSRC, src), "-o", obj], cwd=CSRC))
+        procs.append(subprocess.Popen(_binding_command(tmp_binding)))
+        if any([p.wait() != 0 for p in procs]):
+            raise RuntimeError("the compiler failed")
+        subprocess.run([NVCC, "-shared", "-o", tmp_lib] + objs + ["-lcudart"], check=True, cwd=CSRC)
+        os.replace(tmp_lib, LIB)
+        os.replace(tmp_binding, BINDING)
+    finally:  # a failed or interrupted build leaves nothing beside the sources
+        for p in procs:
+            if p.poll() is None:
+                p.terminate()
+                p.wait()
+        for tmp in (tmp_lib, tmp_binding):
+            if os.path.exists(tmp):
+                os.remove(tmp)
     return LIB
 
 

@@ -1,0 +1,47 @@
+"""The build leaves nothing behind that it does not replace, and no compiled code is part of the source tree."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2609_35465_b200 import build as tbuild
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture
+def away(tmp_path, monkeypatch):
+    """The build's products in a folder of their own, without the compilers."""
+    monkeypatch.setattr(tbuild, "LIB", str(tmp_path / "lib.so"))
+    monkeypatch.setattr(tbuild, "BINDING", str(tmp_path / "binding.so"))
+    monkeypatch.setattr(tbuild, "SOURCES", ["tetra_tables.cpp"])
+    monkeypatch.setattr(tbuild, "_binding_command", lambda out: ["touch", out])
+    return tmp_path
+
+
+def test_a_failed_compiler_leaves_no_files(away, monkeypatch):
+    monkeypatch.setattr(tbuild, "NVCC", "false")
+    with pytest.raises(RuntimeError):
+        tbuild.build(force=True)
+    assert os.listdir(away) == []
+
+
+def test_an_interrupted_build_leaves_no_files(away, monkeypatch):
+    def interrupted(*args, **kwargs):
+        raise KeyboardInterrupt
+    monkeypatch.setattr(tbuild, "NVCC", "true")
+    monkeypatch.setattr(tbuild.subprocess, "run", interrupted)
+    with pytest.raises(KeyboardInterrupt):
+        tbuild.build(force=True)
+    assert os.listdir(away) == []
+
+
+def test_no_compiled_code_is_tracked():
+    if not os.path.exists(os.path.join(ROOT, ".git")):
+        pytest.skip("not a checkout")
+    files = subprocess.run(["git", "ls-files", "-z"], cwd=ROOT, capture_output=True, check=True).stdout.decode().split("\0")
+    for f in filter(None, files):
+        path = os.path.join(ROOT, f)
+        if os.path.isfile(path):
+            with open(path, "rb") as fh:
+                assert fh.read(4) != b"\x7fELF", f
