@@ -24,6 +24,7 @@ namespace {
 // The C ABI, looked up in the library tetra.py names.
 struct Api {
     decltype(&tetra_status_string) status_string;
+    decltype(&tetra_table_bytes) table_bytes;
     decltype(&tetra_gemv) gemv;
     decltype(&tetra_gemv_tail) gemv_tail;
     decltype(&tetra_gemv_list) gemv_list;
@@ -74,6 +75,9 @@ void* need(PyObject* o, size_t nbytes, const char* what, const char* name) {
         fail(tetra_error, "%s%s: tensor is neither on the device nor in pinned host memory", what, name);
     return t.data_ptr();
 }
+
+// The blob of tetra_build_table.
+void* table_of(PyObject* o, const char* what) { return need(o, api.table_bytes(), what, " table"); }
 
 int integer(PyObject* o) {
     const long v = PyLong_AsLong(o);
@@ -135,7 +139,7 @@ struct GemvArgs {
 // library rejects is passed on unchecked.
 GemvArgs gemv_args(PyObject* codes, PyObject* row_scales, PyObject* table, PyObject* x, PyObject* y, int N, int K, int batch,
                    PyObject* tail, bool tail_rule, const char* what) {
-    GemvArgs g{nullptr, nullptr, pointer(table), nullptr, nullptr, nullptr, N, K, batch};
+    GemvArgs g{nullptr, nullptr, table_of(table, what), nullptr, nullptr, nullptr, N, K, batch};
     if (N <= 0 || K <= 0 || batch <= 0) {
         g.codes = pointer(codes);
         g.row_scales = pointer(row_scales);
@@ -189,7 +193,7 @@ FASTCALL(py_gemv_batched) {
         const GemvArgs g = gemv_args(a[0], a[1], a[2], a[3], a[4], integer(a[5]), integer(a[6]), integer(a[7]), a[8], a[8] != Py_None, "tetra_gemv_batched");
         const at::Tensor& ws = tensor(a[9]);
         void* wp = ws.data_ptr();
-        const size_t wn = size_t(ws.numel());
+        const size_t wn = size_t(ws.numel()) * ws.element_size();
         void* s = stream_of(a[10]);
         check(unlocked([&] {
                   return api.gemv_batched(g.codes, static_cast<float*>(g.row_scales), g.table, g.x, static_cast<float*>(g.y), g.N, g.K, g.batch, g.tail, wp, wn, s);
@@ -201,7 +205,7 @@ FASTCALL(py_gemv_batched) {
 // problems (array of tetra_problem with the buffer interface), table, stream
 FASTCALL(py_gemv_list) {
     return guarded(n, 3, [&] {
-        void* table = pointer(a[1]);
+        void* table = table_of(a[1], "tetra_gemv_list");
         void* s = stream_of(a[2]);
         Py_buffer b;
         if (PyObject_GetBuffer(a[0], &b, PyBUF_SIMPLE) != 0) throw Failed();
@@ -216,7 +220,7 @@ FASTCALL(py_gemv_list) {
 // workspace, table, stream
 FASTCALL(py_grouped_run) {
     return guarded(n, 3, [&] {
-        void *ws = pointer(a[0]), *table = pointer(a[1]), *s = stream_of(a[2]);
+        void *ws = pointer(a[0]), *table = table_of(a[1], "tetra_gemv_grouped_run"), *s = stream_of(a[2]);
         check(unlocked([&] { return api.grouped_run(ws, table, s); }), "tetra_gemv_grouped_run");
         return same(Py_None);
     });
@@ -230,7 +234,7 @@ void need_bytes_type(const at::Tensor& t, size_t nbytes, const char* what) {
 FASTCALL(py_pack_codes) {
     return guarded(n, 6, [&] {
         const at::Tensor& codes = tensor(a[0]);
-        void* table = pointer(a[1]);
+        void* table = table_of(a[1], "tetra_pack_codes");
         const int N = integer(a[2]), B = integer(a[3]);
         need_bytes_type(codes, 0, "tetra_pack_codes");
         if (long(codes.numel()) != long(N) * B * 6)
@@ -239,7 +243,7 @@ FASTCALL(py_pack_codes) {
         void* s = stream_of(a[5]);
         const at::Tensor out = a[4] == Py_None ? device_empty({int64_t(nbytes)}, at::kByte, codes) : tensor(a[4]);
         if (size_t(out.numel()) < nbytes) fail(PyExc_AssertionError, "tetra_pack_codes: out holds fewer than %zu bytes", nbytes);
-        void *src = codes.data_ptr(), *dst = out.data_ptr();
+        void *src = codes.data_ptr(), *dst = a[4] == Py_None ? out.data_ptr() : need(a[4], nbytes, "tetra_pack_codes", " out");
         check(unlocked([&] { return api.pack_codes(src, table, dst, N, B, s); }), "tetra_pack_codes");
         return a[4] == Py_None ? THPVariable_Wrap(out) : same(a[4]);
     });
@@ -248,14 +252,15 @@ FASTCALL(py_pack_codes) {
 FASTCALL(py_decode_packed) {
     return guarded(n, 6, [&] {
         const at::Tensor& packed = tensor(a[0]);
-        void* table = pointer(a[1]);
         const int N = integer(a[2]), B = integer(a[3]);
+        void* src = need(a[0], api.codes_bytes(N, B), "tetra_decode_packed", " packed");
+        void* table = table_of(a[1], "tetra_decode_packed");
         const int want = PyObject_IsTrue(a[4]);
         void* s = stream_of(a[5]);
         const at::Tensor y = device_empty({N, B, 24}, at::kChar, packed);
         at::Tensor mg;
         if (want) mg = device_empty({N, B, 2}, at::kByte, packed);
-        void *src = packed.data_ptr(), *dy = y.data_ptr(), *dm = want ? mg.data_ptr() : nullptr;
+        void *dy = y.data_ptr(), *dm = want ? mg.data_ptr() : nullptr;
         check(unlocked([&] { return api.decode_packed(src, table, static_cast<int8_t*>(dy), static_cast<uint8_t*>(dm), N, B, s); }), "tetra_decode_packed");
         return Py_BuildValue("(NN)", THPVariable_Wrap(y), want ? THPVariable_Wrap(mg) : same(Py_None));
     });
@@ -265,8 +270,8 @@ FASTCALL(py_encode_blocks) {
     return guarded(n, 5, [&] {
         const at::Tensor& w = tensor(a[0]);
         const int64_t count = w.numel() / 24;
+        void* table = table_of(a[1], "tetra_encode_blocks");
         void* wp = need(a[0], size_t(4) * 24 * size_t(count), "tetra_encode_blocks", " w");
-        void* table = pointer(a[1]);
         void* sigma = need(a[2], size_t(4) * size_t(count), "tetra_encode_blocks", " sigma");
         const int want = PyObject_IsTrue(a[3]);
         void* s = stream_of(a[4]);
@@ -349,6 +354,7 @@ FASTCALL(py_setup) {
             if (!f) fail(PyExc_OSError, "%s: no symbol %s", path, name);
         };
         get(api.status_string, "tetra_status_string");
+        get(api.table_bytes, "tetra_table_bytes");
         get(api.gemv, "tetra_gemv");
         get(api.gemv_tail, "tetra_gemv_tail");
         get(api.gemv_list, "tetra_gemv_list");
