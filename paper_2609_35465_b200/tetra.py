@@ -121,12 +121,16 @@ def _ptr(t):
     return C.c_void_p(t.data_ptr()) if t is not None else C.c_void_p(0)
 
 
+def _nbytes(t) -> int:
+    return t.numel() * t.element_size()
+
+
 def _need(t, nbytes: int, what: str, cuda: bool = True):
     """The tensor handed over as `what` holds at least nbytes, contiguously, where the call reads or writes it.
     The C ABI sees plain pointers; a tensor that is too small would be read or written past its end."""
     if t is None:
         return
-    have = t.numel() * t.element_size()
+    have = _nbytes(t)
     if have < nbytes:
         raise TetraError("%s: tensor of %d bytes, the call needs %d" % (what, have, nbytes))
     if not t.is_contiguous():
@@ -177,6 +181,7 @@ def tetra_build_table(gain=None, device="cuda", stream=None) -> torch.Tensor:
 
 def tetra_decode_blocks(codes: torch.Tensor, table: torch.Tensor, want_mg: bool = True, stream=None):
     """codes: uint8 [..., 6] file-order words on the device -> (y int8 [n, 24], mg uint8 [n, 2] or None)."""
+    _need(table, tetra_table_bytes(), "tetra_decode_blocks table")
     assert codes.dtype == torch.uint8 and codes.is_cuda and codes.is_contiguous()
     n = codes.numel() // WORD_BYTES
     y = torch.empty((n, BLOCK), dtype=torch.int8, device=codes.device)
@@ -233,7 +238,8 @@ def tetra_grouped_workspace_bytes(problems) -> int:
 
 def tetra_gemv_grouped_plan(problems, workspace: torch.Tensor, stream=None):
     """Writes the plan of a list of products (ctypes array from make_problems) into the workspace."""
-    _check(lib().tetra_gemv_grouped_plan(problems, len(problems), _ptr(workspace), workspace.numel(),
+    _need(workspace, 0, "tetra_gemv_grouped_plan workspace")
+    _check(lib().tetra_gemv_grouped_plan(problems, len(problems), _ptr(workspace), _nbytes(workspace),
                                          _stream(stream)), "tetra_gemv_grouped_plan")
 
 
@@ -244,12 +250,19 @@ def tetra_gemv_grouped_run(workspace: torch.Tensor, table, stream=None):
 
 def tetra_gemv_grouped(problems, table, workspace: torch.Tensor, stream=None):
     """plan + run."""
-    _check(lib().tetra_gemv_grouped(problems, len(problems), _ptr(table), _ptr(workspace), workspace.numel(),
+    _need(table, tetra_table_bytes(), "tetra_gemv_grouped table")
+    _need(workspace, 0, "tetra_gemv_grouped workspace")
+    _check(lib().tetra_gemv_grouped(problems, len(problems), _ptr(table), _ptr(workspace), _nbytes(workspace),
                                     _stream(stream)), "tetra_gemv_grouped")
 
 
 def tetra_gemv_paper_design(codes, row_stride: int, row_scales, table, x, y, N: int, K: int, batch: int = 1,
                             tail=None, stream=None):
+    what = "tetra_gemv_paper_design"
+    _need(table, tetra_table_bytes(), what + " table")
+    if N > 0 and row_stride > 0:
+        _need(codes, (N - 1) * row_stride + WORD_BYTES * _blocks(K, tail is not None), what + " codes")
+    _need_gemv(what, None, row_scales, x, y, N, K, batch, tail, tail is not None)
     _check(lib().tetra_gemv_paper_design(_ptr(codes), row_stride, _ptr(row_scales), _ptr(table), _ptr(x), _ptr(y),
                                          N, K, batch, _ptr(tail), _stream(stream)), "tetra_gemv_paper_design")
     return y
@@ -258,6 +271,12 @@ def tetra_gemv_paper_design(codes, row_stride: int, row_scales, table, x, y, N: 
 def tetra_gemv_hostio(codes, row_scales, table, x_host, y_host, x_stage, y_stage, N: int, K: int, batch: int = 1,
                       tail=None, stream=None):
     """x_host / y_host: pinned CPU tensors; the copies and the product are enqueued on the stream."""
+    what = "tetra_gemv_hostio"
+    _need(table, tetra_table_bytes(), what + " table")
+    _need_gemv(what, codes, row_scales, x_stage, y_stage, N, K, batch, tail, tail is not None)
+    if N > 0 and K > 0 and batch > 0:
+        _need(x_host, 2 * batch * K, what + " x_host", cuda=False)
+        _need(y_host, 4 * batch * N, what + " y_host", cuda=False)
     _check(lib().tetra_gemv_hostio(_ptr(codes), _ptr(row_scales), _ptr(table), _ptr(x_host), _ptr(y_host),
                                    _ptr(x_stage), _ptr(y_stage), N, K, batch, _ptr(tail), _stream(stream)),
            "tetra_gemv_hostio")
@@ -266,11 +285,15 @@ def tetra_gemv_hostio(codes, row_scales, table, x_host, y_host, x_stage, y_stage
 def tetra_gemv_grouped_hostio(workspace, table, x_host, x_dev, y_host=None, y_dev=None, stream=None):
     """A planned run with pinned host activations / results (one copy in, the kernels, one copy out); with
     y_host = y_dev = None the plan's y pointers are taken to aim at mapped pinned host memory (no copy out)."""
-    y_bytes = 0 if y_dev is None else y_dev.numel() * y_dev.element_size()
-    _check(lib().tetra_gemv_grouped_hostio(_ptr(workspace), _ptr(table), _ptr(x_host), _ptr(x_dev),
-                                           x_dev.numel() * x_dev.element_size(), _ptr(y_host), _ptr(y_dev),
-                                           y_bytes, _stream(stream)),
-           "tetra_gemv_grouped_hostio")
+    what = "tetra_gemv_grouped_hostio"
+    x_bytes, y_bytes = _nbytes(x_dev), 0 if y_dev is None else _nbytes(y_dev)
+    _need(table, tetra_table_bytes(), what + " table")
+    _need(x_host, x_bytes, what + " x_host", cuda=False)
+    _need(y_host, y_bytes, what + " y_host", cuda=False)
+    for t, name in ((x_dev, " x_dev"), (y_dev, " y_dev")):
+        _need(t, 0, what + name)
+    _check(lib().tetra_gemv_grouped_hostio(_ptr(workspace), _ptr(table), _ptr(x_host), _ptr(x_dev), x_bytes,
+                                           _ptr(y_host), _ptr(y_dev), y_bytes, _stream(stream)), what)
 
 
 NOALLOC_MAX_K = 24576
@@ -324,10 +347,18 @@ def tetra_encode_blocks(w, table, sigma=None, want_cosine=True, stream=None):
 
 
 def make_q4_problems(items):
-    """items: iterable of dicts(packed, x, y, N, K) of device tensors -> ctypes array of tetra_q4_problem."""
+    """items: iterable of dicts(packed, x, y, N, K) of device tensors -> ctypes array of tetra_q4_problem.
+
+    The list's group size comes with the plan: here `packed` has to hold the matrix at the larger size that K allows,
+    the one that takes fewer bytes."""
     items = list(items)
     arr = (Q4Problem * len(items))()
     for i, it in enumerate(items):
+        N, K, what = it["N"], it["K"], "problem %d" % i
+        if N > 0 and K > 0:
+            _need(it["packed"], lib().tetra_q4_packed_bytes(N, K, 64 if K % 128 else 128), what + " packed")
+            _need(it["x"], 2 * K, what + " x")
+            _need(it["y"], 4 * N, what + " y")
         arr[i] = Q4Problem(it["packed"].data_ptr(), it["x"].data_ptr(), it["y"].data_ptr(), it["N"], it["K"])
     return arr
 

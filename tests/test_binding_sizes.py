@@ -80,3 +80,56 @@ def test_batched_workspace_is_counted_in_bytes(tt):
                 tt.tetra_gemv_batched(u8(48, "cuda"), rs, table, x, y, 8, 24, 2, None, ws)
     torch.cuda.synchronize()
     assert not y.any()
+
+
+def short(t):
+    """All of a tensor but its last element."""
+    return t.reshape(-1)[:-1]
+
+
+# The calls that go through ctypes: comparison arms, host activations, plans, 4-bit lists.  Sources are cut by one element in
+# turn; nothing here reaches the library.
+@pytest.mark.parametrize("name", ["table", "codes", "row_scales", "x", "y", "tail"])
+def test_paper_design_sizes(tt, name, monkeypatch):
+    monkeypatch.setattr(torch.Tensor, "is_pinned", lambda self: True)
+    t = dict(table=u8(tt.tetra_table_bytes()), codes=u8(3 * 14 + 12), row_scales=torch.zeros(4), tail=torch.zeros((4, 2), dtype=torch.float16),
+             x=torch.zeros(50, dtype=torch.float16), y=torch.zeros(4))
+    t[name] = short(t[name])
+    with pytest.raises(tt.TetraError, match="%s: .*needs" % name):
+        tt.tetra_gemv_paper_design(t["codes"], 14, t["row_scales"], t["table"], t["x"], t["y"], 4, 50, 1, t["tail"])
+
+
+@pytest.mark.parametrize("name", ["table", "codes", "row_scales", "x", "y", "x_host", "y_host"])
+def test_hostio_sizes(tt, name, monkeypatch):
+    monkeypatch.setattr(torch.Tensor, "is_pinned", lambda self: True)
+    h, f = torch.zeros((2, 48), dtype=torch.float16), torch.zeros((2, 8))
+    t = dict(table=u8(tt.tetra_table_bytes()), codes=u8(96), row_scales=torch.zeros(8), x=h, y=f, x_host=h, y_host=f)
+    t[name] = short(t[name])
+    with pytest.raises(tt.TetraError, match="%s: .*needs" % name):
+        tt.tetra_gemv_hostio(t["codes"], t["row_scales"], t["table"], t["x_host"], t["y_host"], t["x"], t["y"], 8, 48, 2)
+
+
+@pytest.mark.parametrize("name", ["table", "x_host", "y_host"])
+def test_grouped_hostio_sizes(tt, name, monkeypatch):
+    monkeypatch.setattr(torch.Tensor, "is_pinned", lambda self: True)
+    t = dict(table=u8(tt.tetra_table_bytes()), x_host=torch.zeros(24, dtype=torch.float16), y_host=torch.zeros(8))
+    x_dev, y_dev = t["x_host"].clone(), t["y_host"].clone()
+    t[name] = short(t[name])
+    with pytest.raises(tt.TetraError, match="%s: .*needs" % name):
+        tt.tetra_gemv_grouped_hostio(u8(4096), t["table"], t["x_host"], x_dev, t["y_host"], y_dev)
+
+
+@pytest.mark.parametrize("name", ["packed", "x", "y"])
+def test_q4_problem_sizes(tt, name, monkeypatch):
+    monkeypatch.setattr(torch.Tensor, "is_pinned", lambda self: True)
+    for K, G in ((192, 64), (256, 128)):
+        it = dict(packed=u8(tt.tetra_q4_packed_bytes(40, K, G)), x=torch.zeros(K, dtype=torch.float16), y=torch.zeros(40), N=40, K=K)
+        tt.make_q4_problems([it])
+        it[name] = short(it[name])
+        with pytest.raises(tt.TetraError, match="%s: .*needs" % name):
+            tt.make_q4_problems([it])
+
+
+def test_a_plan_wants_a_workspace_on_the_device(tt):
+    with pytest.raises(tt.TetraError, match="workspace.*neither"):
+        tt.tetra_gemv_grouped_plan((tt.Problem * 1)(), u8(4096))
