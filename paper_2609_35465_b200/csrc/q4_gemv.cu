@@ -398,13 +398,6 @@ int check_shape(int N, int K, int G) {
     return TETRA_OK;
 }
 
-int device_sm_count(int* sms) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
-    return cuda_status(e);
-}
-
 constexpr size_t kQ4SmemLimit = 224 * 1024 / kQ4CtasPerSm - 2048;
 
 template <int G, int DEPTH>
@@ -470,9 +463,11 @@ int tetra_q4_pack(const void* q_dev, const void* scale_dev, const void* offset_d
         return TETRA_ERR_ALIGN;
     const size_t need = tetra_q4_packed_bytes(N, K, G);
     if (packed_bytes < need) return TETRA_ERR_SIZE;
+    int sms = 0;
+    if (device_sms(&sms) != cudaSuccess) return TETRA_ERR_CUDA;
     const size_t chunks = size_t((N + 31) / 32) * (K / G);
-    const size_t ctas = (chunks + 7) / 8;  // a warp per chunk
-    const unsigned grid = unsigned(ctas < 148 * 64 ? ctas : 148 * 64);
+    const size_t ctas = (chunks + 7) / 8, most = size_t(sms) * 64;  // a warp per chunk
+    const unsigned grid = unsigned(ctas < most ? ctas : most);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const auto* q = static_cast<const uint8_t*>(q_dev);
     const auto *scale = static_cast<const __half*>(scale_dev), *offset = static_cast<const __half*>(offset_dev);
@@ -488,8 +483,7 @@ int tetra_q4_gemv(const void* packed_dev, const void* x_dev, float* y_dev, int N
     if (batch < 1 || batch > TETRA_Q4_MAX_BATCH) return TETRA_ERR_BATCH;
     if (!aligned(packed_dev, 16) || !aligned(x_dev, 16) || !aligned(y_dev, 4)) return TETRA_ERR_ALIGN;
     int sms = 0;
-    const int drc = device_sm_count(&sms);
-    if (drc != TETRA_OK) return drc;
+    if (device_sms(&sms) != cudaSuccess) return TETRA_ERR_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     return cuda_status(G == 128 ? launch_q4_gemv<128, 3>(packed_dev, x_dev, y_dev, N, K, batch, sms, s)
                                 : launch_q4_gemv<64, 6>(packed_dev, x_dev, y_dev, N, K, batch, sms, s));

@@ -219,7 +219,10 @@ static int grid_for(size_t items, int threads, int cap) {
 
 cudaError_t launch_decode_file(const void* codes, const void* table, int8_t* y, uint8_t* mg, size_t nblocks,
                                cudaStream_t s) {
-    k_decode_file<<<grid_for(nblocks, 256, 148 * 32), 256, 0, s>>>(
+    int sms = 0;
+    const cudaError_t e = device_sms(&sms);
+    if (e != cudaSuccess) return e;
+    k_decode_file<<<grid_for(nblocks, 256, sms * 32), 256, 0, s>>>(
         static_cast<const uint8_t*>(codes), static_cast<const DeviceTables*>(table), y, mg, nblocks);
     return cudaGetLastError();
 }

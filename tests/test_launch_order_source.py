@@ -1,5 +1,5 @@
-"""What the kernels' sources must keep to so that calls on one stream take effect in order (tetra_device.cuh, programmatic
-dependent launch): read from the source, because a launch that starts too early is not an error that a run shows."""
+"""What the kernels' sources must keep to, read from the source because a run does not show it: calls on one stream take
+effect in order (tetra_device.cuh, programmatic dependent launch), and launches ask the device for its size."""
 import os
 import re
 
@@ -8,14 +8,18 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_35465_b200", "csrc")
 
 
-def kernels():
-    """name -> (parameters, body) of every __global__ function, comments taken out."""
-    found = {}
+def sources():
+    """(file name, text without comments) of the CUDA sources."""
     for f in sorted(os.listdir(CSRC)):
-        if not f.endswith((".cu", ".cuh")):
-            continue
-        text = open(os.path.join(CSRC, f)).read()
-        text = re.sub(r"//[^\n]*|/\*.*?\*/", "", text, flags=re.S)
+        if f.endswith((".cu", ".cuh")):
+            text = open(os.path.join(CSRC, f)).read()
+            yield f, re.sub(r"//[^\n]*|/\*.*?\*/", "", text, flags=re.S)
+
+
+def kernels():
+    """name -> (parameters, body) of every __global__ function."""
+    found = {}
+    for _, text in sources():
         for m in re.finditer(r"__global__\s+void\s+(?:__launch_bounds__\([^)]*\)\s*)?(\w+)\s*\(([^)]*)\)\s*\{", text):
             depth, at = 1, m.end()
             while depth:
@@ -45,3 +49,8 @@ def test_a_kernel_that_writes_packed_codes_does_not_release_its_dependents():
 def test_a_kernel_that_releases_its_dependents_waits_for_its_predecessors(name):
     body = KERNELS[name][1]
     assert "pdl_release" not in body or "pdl_wait" in body
+
+
+def test_no_launch_is_written_for_one_number_of_multiprocessors():
+    for f, text in sources():
+        assert not re.search(r"\b148\b", text), f
