@@ -22,7 +22,7 @@ def _stale() -> bool:
     if not os.path.exists(LIB) or not os.path.exists(BINDING):
         return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".o")]  # the objects are the build's own
     deps += [os.path.join(os.path.dirname(HERE), "include", h) for h in ("tetra.h", "tetra_q4.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 

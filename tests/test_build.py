@@ -36,6 +36,27 @@ def test_an_interrupted_build_leaves_no_files(away, monkeypatch):
     assert os.listdir(away) == []
 
 
+def test_a_finished_build_is_not_stale(away, monkeypatch):
+    """Its objects lie beside the sources and may be younger than the first of its two products."""
+    csrc, old = away / "csrc", 1_000_000_000
+    csrc.mkdir()
+    monkeypatch.setattr(tbuild, "CSRC", str(csrc))
+    monkeypatch.setattr(tbuild, "HERE", str(away / "include"))
+    for name, at in (("a.cu", old), ("binding.cpp", old), ("a.o", old + 20)):
+        (csrc / name).write_text("")
+        os.utime(csrc / name, (at, at))
+    (away / "include").mkdir()
+    for h in ("tetra.h", "tetra_q4.h"):
+        (away / "include" / h).write_text("")
+        os.utime(away / "include" / h, (old, old))
+    for path, at in ((tbuild.BINDING, old + 10), (tbuild.LIB, old + 30)):
+        open(path, "w").close()
+        os.utime(path, (at, at))
+    assert not tbuild._stale()
+    os.utime(csrc / "a.cu", (old + 15, old + 15))
+    assert tbuild._stale()
+
+
 def test_no_compiled_code_is_tracked():
     if not os.path.exists(os.path.join(ROOT, ".git")):
         pytest.skip("not a checkout")
