@@ -18,9 +18,18 @@ FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-li
          "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall", "--use_fast_math"]
 
 
+def built_for() -> str:
+    """What the binding is tied to; the file holds this text, and tetra.py asks for it before the first call."""
+    import torch
+    return "torch %s, Python %d.%d" % (torch.__version__, sys.version_info[0], sys.version_info[1])
+
+
 def _stale() -> bool:
     if not os.path.exists(LIB) or not os.path.exists(BINDING):
         return True
+    with open(BINDING, "rb") as f:
+        if built_for().encode() not in f.read():
+            return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".o")]  # the objects are the build's own
     deps += [os.path.join(os.path.dirname(HERE), "include", h) for h in ("tetra.h", "tetra_q4.h")]
@@ -34,7 +43,7 @@ def _binding_command(out: str):
     inc, lib = os.path.join(root, "include"), os.path.join(root, "lib")
     cuda = os.path.dirname(os.path.dirname(NVCC))
     return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-            "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+            "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), '-DTETRA_BUILT_FOR="%s"' % built_for(),
             "-isystem", inc, "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"),
             "-isystem", os.path.join(cuda, "include"), "-isystem", sysconfig.get_paths()["include"],
             os.path.join(CSRC, "binding.cpp"), "-o", out, "-L" + lib, "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10",

@@ -385,4 +385,11 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_binding", "Argument marshalling o
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__binding() { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__binding() {
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_for", TETRA_BUILT_FOR) != 0) {  // see build.py
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
+}

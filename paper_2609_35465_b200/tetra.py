@@ -53,6 +53,10 @@ def _native():
             from . import _binding
         except ImportError as e:
             raise TetraError("binding not built (run python -m paper_2609_35465_b200.build): %s" % e)
+        from .build import built_for
+        if _binding.built_for != built_for():  # it uses torch's C++ classes, whose layout goes with the version
+            raise TetraError("binding built for %s, this is %s (run python -m paper_2609_35465_b200.build)"
+                             % (_binding.built_for, built_for()))
         _binding.setup(LIB_PATH, TetraError)
         _nat = _binding
     return _nat

@@ -1,4 +1,5 @@
-"""The build leaves nothing behind that it does not replace, and no compiled code is part of the source tree."""
+"""The build leaves nothing behind that it does not replace and knows what its products are good for; no compiled code is
+part of the source tree."""
 import os
 import subprocess
 
@@ -50,11 +51,25 @@ def test_a_finished_build_is_not_stale(away, monkeypatch):
         (away / "include" / h).write_text("")
         os.utime(away / "include" / h, (old, old))
     for path, at in ((tbuild.BINDING, old + 10), (tbuild.LIB, old + 30)):
-        open(path, "w").close()
+        with open(path, "w") as f:
+            f.write(tbuild.built_for())
         os.utime(path, (at, at))
     assert not tbuild._stale()
     os.utime(csrc / "a.cu", (old + 15, old + 15))
     assert tbuild._stale()
+
+
+def test_a_binding_for_another_torch_is_stale_and_refused(monkeypatch):
+    tbuild.build()
+    assert not tbuild._stale()
+    from paper_2609_35465_b200 import tetra
+    monkeypatch.setattr(tetra, "_nat", None)
+    tetra._native()
+    monkeypatch.setattr(tetra, "_nat", None)
+    monkeypatch.setattr(tbuild.sys, "version_info", (3, 99))
+    assert tbuild._stale()
+    with pytest.raises(tetra.TetraError, match="built for"):
+        tetra._native()
 
 
 def test_no_compiled_code_is_tracked():
