@@ -85,8 +85,8 @@ typedef struct {
  *   tetra_q4_list_workspace_bytes  size of the scratch buffer (descriptors, partial strips); 0 for a rejected list;
  *   tetra_q4_list_plan             writes the descriptors (problems_host is read before the call
  *                                  returns; call it outside stream capture);
- *   tetra_q4_list_run              one step, one launch; of the warps that share a strip the last adds
- *                                  their parts, in warp order.
+ *   tetra_q4_list_run              one step, one launch, G as planned; of the warps that share a strip the
+ *                                  last adds their parts, in warp order.
  * workspace_dev: 256-byte aligned device memory owned by the caller; it belongs to the plan until the
  * last run using it has completed, runs that share it must not overlap on the GPU, and it may be
  * copied to other device memory (the plan describes itself) on the device it was planned for.

@@ -42,14 +42,13 @@ struct Q4Item {
     const unsigned char* packed;
     const __half* x;
     float* y;
-    int32_t N, K;
+    int32_t N;
     int32_t groups, strips;
     uint32_t chunk_begin;  // chunks of the matrices before this one
     uint32_t group_begin;  // groups of the matrices before this one (index into the group sums)
-    uint32_t strip_begin;  // strips of the matrices before this one
     uint32_t pad_;
 };
-static_assert(sizeof(Q4Item) == 56, "descriptor layout");
+static_assert(sizeof(Q4Item) == 48, "descriptor layout");
 
 // What a warp's range [c_begin, c_end) of the chunk sequence meets, known when the list is planned.
 struct Q4Warp {
@@ -60,8 +59,8 @@ struct Q4Warp {
 };
 
 struct Q4ListHeader {
-    int32_t count, G, nwarps, pad0_;
-    uint32_t total_chunks, total_groups, total_strips, pad1_;
+    int32_t nwarps;
+    uint32_t total_chunks;
     uint32_t off_items, off_warps, off_pieces;
 };
 
@@ -372,32 +371,26 @@ int tetra_q4_list_plan(const tetra_q4_problem* problems_host, int count, int G, 
     int sms = 0;
     if (device_sms(&sms) != cudaSuccess) return TETRA_ERR_CUDA;
     const int nwarps = sms * kQ4ListWarps;
-    uint64_t chunks = 0, groups = 0, strips = 0;
+    uint64_t chunks = 0;
     for (int i = 0; i < count; ++i) {
         const uint64_t gr = uint64_t(problems_host[i].K / G), st = uint64_t((problems_host[i].N + 31) / 32);
         chunks += gr * st;
-        groups += gr;
-        strips += st;
     }
-    if (chunks > 0x7FFFFFF0ull || strips > 0x7FFFFFF0ull) return TETRA_ERR_SHAPE;
+    if (chunks > 0x7FFFFFF0ull) return TETRA_ERR_SHAPE;  // strips and groups are no more than chunks
     const Q4ListLayout L = list_layout(count, nwarps);
     if (workspace_bytes < L.total) return TETRA_ERR_SIZE;
     const size_t meta = L.off_pieces;
     unsigned char* buf = static_cast<unsigned char*>(std::calloc(1, meta));
     if (!buf) return TETRA_ERR_CUDA;
     Q4ListHeader* H = reinterpret_cast<Q4ListHeader*>(buf);
-    H->count = count;
-    H->G = G;
     const int ranges = chunks < uint64_t(nwarps) ? int(chunks) : nwarps;  // no range is empty
     H->nwarps = ranges;
     H->total_chunks = uint32_t(chunks);
-    H->total_groups = uint32_t(groups);
-    H->total_strips = uint32_t(strips);
     H->off_items = uint32_t(L.off_items);
     H->off_warps = uint32_t(L.off_warps);
     H->off_pieces = uint32_t(L.off_pieces);
     Q4Item* items = reinterpret_cast<Q4Item*>(buf + L.off_items);
-    uint32_t cb = 0, gb = 0, sb = 0;
+    uint32_t cb = 0, gb = 0;
     for (int i = 0; i < count; ++i) {
         const tetra_q4_problem& q = problems_host[i];
         Q4Item& I = items[i];
@@ -405,15 +398,12 @@ int tetra_q4_list_plan(const tetra_q4_problem* problems_host, int count, int G, 
         I.x = static_cast<const __half*>(q.x);
         I.y = q.y;
         I.N = q.N;
-        I.K = q.K;
         I.groups = q.K / G;
         I.strips = (q.N + 31) / 32;
         I.chunk_begin = cb;
         I.group_begin = gb;
-        I.strip_begin = sb;
         cb += uint32_t(I.groups) * uint32_t(I.strips);
         gb += uint32_t(I.groups);
-        sb += uint32_t(I.strips);
     }
     Q4Warp* warps = reinterpret_cast<Q4Warp*>(buf + L.off_warps);
     int item = 0, owner = 0;
