@@ -85,6 +85,12 @@ int integer(PyObject* o) {
     return int(v);
 }
 
+bool truth(PyObject* o) {
+    const int v = PyObject_IsTrue(o);
+    if (v < 0) throw Failed();
+    return v != 0;
+}
+
 void* stream_of(PyObject* o) {
     if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
     PyObject* handle = PyObject_GetAttrString(o, "cuda_stream");
@@ -253,9 +259,9 @@ FASTCALL(py_decode_packed) {
     return guarded(n, 6, [&] {
         const at::Tensor& packed = tensor(a[0]);
         const int N = integer(a[2]), B = integer(a[3]);
+        const bool want = truth(a[4]);
         void* src = need(a[0], api.codes_bytes(N, B), "tetra_decode_packed", " packed");
         void* table = table_of(a[1], "tetra_decode_packed");
-        const int want = PyObject_IsTrue(a[4]);
         void* s = stream_of(a[5]);
         const at::Tensor y = device_empty({N, B, 24}, at::kChar, packed);
         at::Tensor mg;
@@ -270,10 +276,10 @@ FASTCALL(py_encode_blocks) {
     return guarded(n, 5, [&] {
         const at::Tensor& w = tensor(a[0]);
         const int64_t count = w.numel() / 24;
+        const bool want = truth(a[3]);
         void* table = table_of(a[1], "tetra_encode_blocks");
         void* wp = need(a[0], size_t(4) * 24 * size_t(count), "tetra_encode_blocks", " w");
         void* sigma = need(a[2], size_t(4) * size_t(count), "tetra_encode_blocks", " sigma");
-        const int want = PyObject_IsTrue(a[3]);
         void* s = stream_of(a[4]);
         const at::Tensor codes = device_empty({count, 6}, at::kByte, w);
         at::Tensor cos;

@@ -1,5 +1,5 @@
 """The binding refuses tensors that hold less than a call reads or writes, before anything is launched: the C ABI takes
-plain pointers.  The sizes are looked at first, so most of this needs no GPU."""
+plain pointers.  Flags and sizes are looked at first, so most of this needs no GPU."""
 import pytest
 import torch
 
@@ -80,6 +80,18 @@ def test_batched_workspace_is_counted_in_bytes(tt):
                 tt.tetra_gemv_batched(u8(48, "cuda"), rs, table, x, y, 8, 24, 2, None, ws)
     torch.cuda.synchronize()
     assert not y.any()
+
+
+class Undecided:
+    def __bool__(self):
+        raise ValueError("neither")
+
+
+def test_a_flag_without_a_truth_value_is_an_error(tt):
+    with pytest.raises(ValueError, match="neither"):
+        tt.tetra_decode_packed(u8(48), None, 8, 1, Undecided())
+    with pytest.raises(ValueError, match="neither"):
+        tt.tetra_encode_blocks(torch.zeros((0, 24)), None, None, Undecided())
 
 
 def short(t):
