@@ -1,10 +1,12 @@
 // Native half of the Python binding: size checks of the tensors, their pointers, the current stream and the call
 // of the C ABI, in one C++ function per entry point.
 //
-// A decode step is a chain of calls whose kernels take a few microseconds; marshalling the arguments in Python and
-// through ctypes took 5.5 us (three arguments) to 11.5 us (ten) a call besides the 2 us of the launch itself, more
-// than most of those kernels.  Here it takes well under a microsecond.  tetra.py keeps the public functions
-// (names, defaults, documentation) and passes their arguments on by position.
+// A decode step is a chain of calls whose kernels take a few microseconds.  Marshalling the arguments in Python and
+// through ctypes took 5.5 us (three arguments) to 11.5 us (ten) a call besides the launch itself, more than most of
+// those kernels.  Host time of a call here, its launch included (medians on two hosts): one product 2.5-2.9 us, a planned
+// list's two launches 4.1-4.9, packing 2.1-2.5 and 0.9 more where it allocates its output, decode_packed with two outputs
+// 4.2-4.5; a call that launches nothing takes 0.2 us.  tetra.py keeps the public functions (names, defaults,
+// documentation) and passes their arguments on by position.
 #include <Python.h>
 #include <dlfcn.h>
 
@@ -129,7 +131,7 @@ PyObject* same(PyObject* o) {
 #define FASTCALL(name) PyObject* name(PyObject*, PyObject* const* a, Py_ssize_t n)
 
 // Device memory from torch's caching allocator, without the dispatcher's detour (0.5 us a tensor; loading a layer
-// makes 22 of them).
+// makes 22 of them).  Not a function that torch promises to keep: a binding serves the version it was built for only.
 at::Tensor device_empty(at::IntArrayRef shape, at::ScalarType type, const at::Tensor& like) {
     if (!like.is_cuda()) fail(tetra_error, "expected a tensor on the device");
     return at::detail::empty_cuda(shape, type, like.device(), c10::nullopt);

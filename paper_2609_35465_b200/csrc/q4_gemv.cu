@@ -44,8 +44,8 @@ __device__ __forceinline__ uint32_t q4_pack_word(uint32_t v0, uint32_t v1) {
 // One warp per chunk (strip, group): lane 4 g + t reads, for every sub-tile, the 16 columns 16 t .. of rows g and
 // g + 8 (eight bytes each; the four lanes of a row read one sector) and writes the lane's 16 bytes, then the row's
 // scale and offset.  Bound by HBM (the matrix once in, once out); neighbouring warps take neighbouring groups, so
-// the sectors of the scale tables are shared through L1.  4096 x 12288, G = 128: 36.9 us with a thread per packed
-// word and byte loads, now 10.9 us (56 MB, 5.2 TB/s).
+// the sectors of the scale tables are shared through L1.  4096 x 12288, G = 128: 10.9 us (56 MB, 5.2 TB/s);
+// with a thread per packed word and byte loads 36.9 us.
 template <int G>
 __global__ void __launch_bounds__(256) k_q4_pack(const uint8_t* __restrict__ q, const __half* __restrict__ scale,
                                                  const __half* __restrict__ offset, unsigned char* __restrict__ packed,
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(256) k_q4_pack(const uint8_t* __restrict__ q, 
 // A strip that lies wholly inside a warp's range is stored directly; a strip cut by a range boundary leaves
 // one piece per warp in shared memory, and after one CTA barrier the pieces are added in warp order; which strips those
 // are is worked out while the kernel waits for its predecessor (looked for afterwards, piece by piece, it was 2.2 us of
-// a 5.1 us launch: 1024 x 4096, G = 128, now 3.9 us; 12288 x 4096, G = 64, 9.9 -> 8.2 us).
+// a 5.1 us launch: 1024 x 4096, G = 128, now 3.7 us).
 // Addresses advance by running pointers: the loop body is dequantise, multiply, scale.
 // XS: the activations are staged in shared memory (rows padded by 16 bytes so that the eight vectors' reads
 // fall into different banks); otherwise they are read through L1.
@@ -342,8 +342,8 @@ k_q4_gemv(const unsigned char* __restrict__ packed, const __half* __restrict__ x
 // tile: one 16-byte load (a quarter of the 64 bytes in which the tile holds the row and its neighbour eight rows
 // away), the row's scale record, 32 bytes out.  WIDE: `out` allows 16-byte stores.  A short call is the chain token
 // number -> weights -> store, and only resident warps hide it: one token per CTA row (two or four tokens a thread,
-// their loads together, take 5.8 and 8.4 us where one takes 4.6).
-// 1024 tokens x 4096: 7.9 us with a thread per four columns, now 4.6 us.
+// their loads together, take 5.8 and 8.4 us where one takes 4.8).
+// 1024 tokens x 4096: 4.8 us; with a thread per four columns 7.9 us.
 template <int G, bool WIDE>
 __global__ void __launch_bounds__(256) k_q4_rows(const unsigned char* __restrict__ packed, const int32_t* __restrict__ ids,
                                                  int count, __half* __restrict__ out, int N, int K) {

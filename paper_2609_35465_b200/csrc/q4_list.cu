@@ -12,14 +12,15 @@
 //     chunks are on their way, and the activations stay in shared memory with them.  (Read through L1 they queue behind
 //     the chunks' copies, which the same unit takes in order: a warp then waits for its newest copy before it can
 //     multiply its oldest chunk, and more copies in flight make it worse.  36 layers, 1.37 GB: 269 us from idle and
-//     284 us under the board's power limit, 198 and 222 us with the activations in shared memory);
+//     284 us under the board's power limit; with the activations in shared memory 201 us from idle and, by the board,
+//     227 to 244 us under the limit);
 //   * the stream: dequantise with five logic operations per four registers, MMA against the activations, scale
 //     and offset per group; a strip (32 rows) that lies wholly inside a warp's range is stored; one cut by range
 //     boundaries leaves a piece per warp in the workspace, and the warp that finds the strip's other pieces there
 //     adds them in warp order and stores it.
 // Where a warp starts and who shares its strips is written into the plan: searched for on the device it was a chain
 // of dependent loads in every warp.  (One layer's projections, 38 MB: 22.5 us with searches, a kernel before this one
-// for the group sums and one after it for the pieces; now 13.0 us.)
+// for the group sums and one after it for the pieces; now 12.5 us.)
 // Deterministic (fixed order everywhere); nothing waits for another warp (a counter per cut strip only tells the
 // last one); CTA barriers, cp.async.wait_group and griddepcontrol.wait are the only waits.
 #include <cstdlib>

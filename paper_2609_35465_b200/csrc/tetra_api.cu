@@ -219,7 +219,7 @@ int tetra_gemv_batched(const void* codes, const float* row_scales, const void* t
     if (B <= 0 || B > kMaxBlocksPerRow) return TETRA_ERR_SHAPE;
     if (workspace_bytes < batched_workspace_bytes(N, B)) return TETRA_ERR_SIZE;
     // One vector: the integer products of the single-matrix kernel need fewer instructions per block than the
-    // conversion to float16 that several vectors share (4096 x 4096: 5.4 us against 6.8 us for two vectors).
+    // conversion to float16 that several vectors share (4096 x 4096: 5.6 us against 6.5 us for two vectors).
     if (batch <= kBatchedMinVectors - 1)
         return tetra_gemv_tail(codes, row_scales, table, x, y, N, K, batch, tail, stream);
     return cuda_status(launch_gemv_batched(codes, row_scales, table, x, y, N, K, batch, (K % 24) ? tail : nullptr,

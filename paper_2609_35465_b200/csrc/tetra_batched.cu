@@ -18,10 +18,11 @@
 //   five and more: dense B.  A block's 24 halves go through a shared-memory tile whose rows keep stores and ldmatrix
 //   conflict-free, an MMA pair (k16 + k8) multiplies sixteen blocks of ONE column with eight vectors, and the
 //   block's scale reaches the lanes that hold its results by a shuffle.
-// The line lies where the tensor pipe's time for the zeros overtakes the tile: 4096 x 4096 with 2 / 4 / 8 / 16 vectors
-// takes 6.7 / 7.5 / 9.3 / 13.3 us block diagonal and 8.5 / 8.7 / 8.9 / 10.3 us dense (13.5 us for three vectors and
-// 27.8 us for sixteen at 4096 x 12288 with int8 planes, activations staged by the CTA and a combining kernel;
-// now 7.5 and 22.5 us).
+// The line lies where the tensor pipe's time for the zeros overtakes the tile.  Block diagonal / dense, 2, 3, 4 vectors:
+// 4096 x 4096 6.5 / 8.2, 7.6 / 8.2, 7.8 / 8.4 us; 4096 x 12288 13.8 / 18.7, 16.3 / 19.1, 16.1 / 18.9; 1024 x 4096
+// 3.9 / 4.7, 4.4 / 4.7, 4.4 / 4.7.  Eight and sixteen on 4096 x 4096: 9.3 and 13.3 us in a build that had them block
+// diagonal, 8.7 and 10.1 dense.  (Int8 planes, activations staged by the CTA and a combining kernel: 13.5 us for three
+// vectors on 4096 x 4096, 27.8 us for sixteen on 4096 x 12288, against 7.6 and 22.8.)
 //
 // A warp's step is NT row tiles x four block columns.  The sixteen warps of a CTA take every sixteenth column quad, so a
 // warp needs nothing from the others until the end: its words come straight from global memory one step ahead, the four
@@ -67,7 +68,7 @@ constexpr int bat_slots(bool dense, int g) { return (dense ? 8 : 2) * g; }
 constexpr int bat_together(bool dense, int g, int nt) { return dense && g == 1 && nt > 1 ? 2 : 1; }
 // Activation buffers of a warp.  Dense: the fragments of a step's columns go to registers at its start, once for all its
 // tiles, so one buffer serves (read per tile they were a sixth of the shared-memory traffic, which keeps its pipe 78 %
-// busy: 4096 x 12288, 16 vectors 24.6 -> 22.5 us).
+// busy: 4096 x 12288, 16 vectors 2 us more).
 constexpr bool bat_hold(bool dense) { return dense; }
 // Row stride, in floats, of the partial sums: even, so that pairs stay aligned.
 constexpr int bat_stride(bool dense, int g) { return bat_slots(dense, g) + 2; }
@@ -472,7 +473,8 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
     }
 }
 
-// Scratch that a caller brings: the call keeps its partial sums in shared memory and leaves it untouched.
+// Scratch that a caller brings: the call keeps its partial sums in shared memory and leaves it untouched.  The size is
+// the one that the entry point has always asked for, so what it refused it still refuses.
 size_t batched_workspace_bytes(int N, int blocks_per_row) {
     const long long row_tiles = (N + 511) / 512, cells = row_tiles * ((blocks_per_row + 3) / 4);
     const long long pieces = (cells < 1024 ? (cells < 1 ? 1 : cells) : 1024) + row_tiles;
@@ -485,7 +487,16 @@ struct BatPlan {
     int cluster = 1, groups = 1, nt = 1;
 };
 // How rows and columns are split: for every cluster size the steps of the busiest warp, in units of one tile x four
-// columns (about 0.5 us on B200), and what else the split costs.
+// columns (0.8-0.9 us with up to four vectors, 0.9-1.3 with eight, 1.2-1.7 with sixteen), and what else the split
+// costs: a chunk of tiles its words, barriers and sums, a cluster its barriers and the other CTA's sums.  One CTA / two, us:
+//   vectors   1184 x 12288   2368 x 12288   3000 x 12288   4096 x 12288   1024 x 4080   2368 x 4080   512 x 4080
+//         3     9.1 /  8.0    10.0 / 11.4    15.8 / 14.0    16.0 / 17.4     4.6 / 5.5     5.4 / 7.0    4.3 / 4.3
+//         8    11.8 /  9.3    12.5 / 13.2    20.3 / 16.8    20.4 / 20.3     5.2 / 5.8     6.2 / 7.7    5.0 / 4.7
+//        16    14.9 / 10.8    15.7 / 14.8    22.8 / 19.3    23.0 / 24.3     6.5 / 6.7     7.4 / 8.7    6.3 / 5.7
+//   chosen           two            one            two            one           one           one          one
+// Short of the best by up to 10 % where rows are few and columns are 4080 or so (a constant of 3 that does not go with the
+// vectors), elsewhere within 6 %.  As many tiles to a step as registers allow: 12288 x 4080 with at most 1, 2, 3, 4 tiles
+// 22.7 / 19.6 / 18.0 / 18.0 us for three vectors, 34.7 / 26.9 / 24.9 / 24.9 for sixteen.
 BatPlan plan_batched(int tiles, int quads, int sms) {
     BatPlan best;
     double best_cost = 1e30;

@@ -38,8 +38,9 @@ __global__ void __launch_bounds__(256) k_decode_file(const uint8_t* __restrict__
 //
 // A lane per record (row group, column).  Bound by HBM (six bytes in, six out per word) once the trellis map, one
 // random lookup per word, is in shared memory and a word is one 4-byte and one 2-byte load, all 16 loads of a record
-// in flight.  12288 x 4096: 13.8 us with the map and a row permutation read through L1 and three 2-byte loads,
-// now 10.8 us.
+// in flight.  12288 x 4096 (25 MB), one packing behind another: 8.1 us, 3.1 TB/s (7.6 us if each one released the next
+// while it runs, which packing may not: see tetra_device.cuh).  With the map and a row permutation read through L1 and
+// three 2-byte loads a packing took 3 us more.
 // ---------------------------------------------------------------------------
 // The (row group, 32 columns) items of a warp, every `warps`-th of them in row-major order, without a division per item.
 struct ItemWalk {
@@ -102,9 +103,12 @@ __global__ void __launch_bounds__(256, 4) k_pack(const uint8_t* __restrict__ cod
 // ---------------------------------------------------------------------------
 // tetra_decode_packed: the GEMV's own decoder, emitting coordinates instead of
 // multiplying.  A warp per (row group, 32 columns), the next item's record on its way meanwhile; a row's 768 bytes go
-// through shared memory, so that they leave as contiguous 8-byte stores (a lane's 24 bytes, stored word by word,
-// touch every sector six times).  Bound by instruction issue (decoder and byte arithmetic), the stores close behind.
-// 12288 x 4096: 35.8 us with direct stores, now 18.9 us (67 MB).
+// through shared memory, so that they leave as contiguous 16-byte stores (a lane's 24 bytes, stored word by word,
+// touch every sector six times).  12288 x 4096 (67 MB, 10.2 us at the copy bandwidth): 14.5 us a call one behind another.
+// Captured alone (19.0 us): 136 warp-instructions per 32 blocks; while warps are active, 76 % of the launch, the L1 and
+// shared-memory pipe is 75 % busy (table lookups, rows staged and read back) and issue slots 56 %; warps wait for
+// their first records (long scoreboard 3.0 of 12 stall cycles per instruction: two items a warp) and for the logic
+// pipe (1.8).  Direct stores made it 17 us longer.
 // ---------------------------------------------------------------------------
 constexpr int kEmitThreads = 256;
 constexpr int kEmitStage = 2 * 768;  // two rows of 32 blocks at a time

@@ -178,8 +178,14 @@ static inline long long problem_tasks(const Problem& q) {
 }
 // Space for the fine mode is reserved for every list of at most kFineMaxTasks (row group, column group)
 // pairs; the plan then takes the fine mode when the list has at most five such pairs per warp of the
-// grid (measured on B200: below that the coarse units leave most warps idle, above it the fine mode's
-// partial sums and counters cost more than they gain).
+// grid: below that the coarse units leave most warps idle, above it the fine mode's partial sums and
+// counters cost more than they gain.  What the coarse units lose goes with their length and how they
+// happen to divide, so five is a middle.  Fine / coarse, us, on 2368 warps:
+//   pairs per warp 0.3 (2048 x 2304) 7.2 / 6.8; 0.8 (2560 x 4096) 9.2 / 16.4; 1.1 (20000 x 768) 10.9 / 7.6; 1.3 (4096 x
+//   4096) 11.7 / 16.6; 2.0 (q, k, v of an 8B layer) 13.7 / 17.6; 2.9 (nine 2048 x 2304) 18.1 / 13.1; 3.5 (4096 x 12288)
+//   19.5 / 22.3; 3.9 (12288 x 4096) 19.6 / 21.3; 4.1 (gate and up of a 4B layer) 22.0 / 16.4; 4.8 (three 3000 x 7000)
+//   24.9 / 33.7; 5.4 (q, k, v, gate and up of a 4B layer) 26.5 / 20.4; 5.8 (q, k, v and gate of an 8B layer) 27.7 / 22.5;
+//   6.2 (5120 x 17408) 29.4 / 44.7; 7.8 (gate and up of an 8B layer) 32.9 / 21.8; 14.5 (an 8B layer) 44.3 / 35.2.
 static bool list_may_be_fine(const Problem* problems, int count) {
     long long tasks = 0;
     for (int i = 0; i < count; ++i) tasks += problem_tasks(problems[i]);
@@ -634,9 +640,12 @@ cudaError_t grouped_plan(const Problem* problems_host, int count, void* ws_dev, 
         long long total = 0;
         for (int i = 0; i < count; ++i) total += unit_work(i) * problem_units(problems_host[i]);
         // The last tenth of the work is not assigned: warps that finish early claim it unit by unit, which
-        // evens out what the cost model and the SMs' unequal speeds leave (measured on the Qwen3-8B pass:
-        // the average scheduler idled 4.2 % of the kernel's time behind the slowest one).  Only when a warp
-        // has at least a few units.
+        // evens out what the cost model and the SMs' unequal speeds leave.  Nothing / 5 % / a tenth / a fifth
+        // claimed: Qwen3-8B pass 836 / 827 / 802 / 804 us, 16 layers of it 387 / 374 / 368 / 369, Qwen3-14B pass
+        // 1522 / 1477 / 1425 / 1439.  Only when a warp has at least eight units: with fewer, a unit claimed last
+        // is too large a share of a warp's work (two layers of the 4B model 45.5 us without, 50.2 with a tenth;
+        // one of the 14B 68.0 / 78.1; but eight of the 8B 204 / 199).  Beyond the line it can still cost: 14B,
+        // whose units are single row groups, four layers 178 without, 191 with; sixteen 647 / 648.
         H->dyn_start = int32_t(units);
         if (units >= 8LL * nwarps) {
             const long long planned = total - total * kDynamicTailPermille / 1000;

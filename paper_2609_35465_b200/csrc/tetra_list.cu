@@ -5,14 +5,13 @@
 // Sec. 5.2 of the paper times one launch per matrix; on B200 such a launch holds
 // a few microseconds of work, so what is left of it is a chain of latencies:
 // dependency wait, activations, their fixed-point image, the passes, the sums.
-// The kernel is arranged to shorten that chain (%globaltimer stamps on q, k, v of
-// an 8B layer, 8.5 us a launch before: 1.3 us of prologue instructions ahead of
-// the wait, 1.3 us of image, 3.1 us of passes, 0.7 us of epilogue, and CTAs that
-// straddled two matrices and finished 2.5 us after the others):
+// The kernel is arranged to shorten that chain (q, k, v of an 8B layer: 6.8 us a
+// launch.  %globaltimer stamps in an arrangement that took 8.5: 1.3 us of prologue
+// instructions ahead of the wait, 1.3 us of image, 3.1 us of passes, 0.7 us of
+// epilogue, and CTAs that straddled two matrices and finished 2.5 us after the others):
 //   * one CTA of sixteen warps per SM: the image and the tables are built and
 //     fetched once per SM (two CTAs of eight warps, which let the next launch start
-//     in the gaps of this one, spend more on doing both twice: q, k, v 7.8 against
-//     6.3 us);
+//     in the gaps of this one, spend more on doing both twice: q, k, v 1.5 us more);
 //   * a CTA works on ONE matrix; the host cuts every matrix's row groups into the
 //     CTAs' shares, and the kernel finds its share with a few comparisons of
 //     parameters: no division, no chain of loads;

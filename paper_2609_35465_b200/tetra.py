@@ -6,8 +6,8 @@ streams.  There is no CPU fallback: if the library is missing or a call fails,
 an exception is raised.
 
 The calls of a decode step, of the encoder and of loading go through _binding.so
-(csrc/binding.cpp), which checks the tensors and calls the library in well under
-a microsecond; plans, tables and the comparison arms go through ctypes.
+(csrc/binding.cpp), which checks the tensors and calls the library in C++; plans,
+tables and the comparison arms go through ctypes.
 """
 import ctypes as C
 import os
