@@ -61,8 +61,8 @@ def test_batched_agrees_with_the_batch1_path(tt, table):
 
 
 def test_batched_vectors_with_very_different_magnitudes(tt, table, orc):
-    """Every vector has its own fixed-point step per block column: a vector 4096 times smaller than its
-    neighbour keeps full precision."""
+    """Activations are used as the float16 values they are, every vector in a column of its own: a vector 4096 times
+    smaller than its neighbour keeps full precision."""
     m = make_matrix(53, 2, 128, 1200, True, batch=4)
     m["x"][1] = (m["x"][1].astype(np.float32) / 4096).astype(np.float16)
     m["x"][2] = (m["x"][2].astype(np.float32) * 512).astype(np.float16)

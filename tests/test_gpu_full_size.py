@@ -106,9 +106,8 @@ def test_down_proj_batch_sweep_sampled_rows(orc, batch):
 @pytest.mark.parametrize("batch", shapes.CONFIG4_BATCHES)
 def test_down_proj_batched_sampled_rows(orc, batch):
     """Config 4 through tetra_gemv_batched (decode once, tensor-core contraction): the shape and the batch
-    sizes the benchmark's sweep times.  Rows: first and last, the rows around the 16- and 32-row tile edges,
-    around the boundaries of the 16-warp tile groups (512 rows) and around the CTA ranges' cuts, and random
-    ones; every vector of the batch."""
+    sizes the benchmark's sweep times.  Rows: first and last, the rows around the edges of 16-row tiles and of
+    larger powers of two, and random ones; every vector of the batch."""
     from paper_2609_35465_b200 import tetra as tt
     m = shapes.CONFIG4
     table = tt.tetra_build_table(synth.DEFAULT_GAIN)
@@ -133,12 +132,10 @@ def test_down_proj_batched_sampled_rows(orc, batch):
 
 @pytest.mark.parametrize("batch,words", [(5, 384), (16, 384), (2, 640), (4, 640)])
 def test_batched_long_cta_ranges_sampled_rows(orc, batch, words):
-    """8192 x 9232 through tetra_gemv_batched: 16 tile groups x 96 column groups are more than ten cells per
-    CTA, so every CTA rebuilds its activation image in the middle of its range (after eight passes with five
-    to eight vectors, after four with more) and most CTAs cross a tile-group boundary; K leaves a float16
-    tail of 16.  With two to four vectors (another kernel, whose image holds sixteen passes) 8192 x 15376:
-    160 column groups, seventeen cells per CTA.  Rows around the tile-group boundaries and random ones, every
-    vector."""
+    """8192 x 9232 through tetra_gemv_batched, dense: three and four 16-row tiles to a CTA, six column quads to a
+    warp, so activation buffers and words are refilled many times over; K leaves a float16 tail of 16.  With two
+    and four vectors (block diagonal) 8192 x 15376: ten quads to a warp.  Rows around the edges of tiles and of
+    larger powers of two and random ones, every vector."""
     from paper_2609_35465_b200 import tetra as tt
     N, K = 8192, 24 * words + 16
     m = make_matrix(23, 7 + batch, N, K, True, batch=batch)
@@ -160,7 +157,7 @@ def test_batched_long_cta_ranges_sampled_rows(orc, batch, words):
 def test_tall_matrix_sampled_rows(orc):
     """151,936 x 4096 (the row count of the model's vocabulary; 155 MB of codes, 18,992 row groups): the index
     arithmetic of every path far beyond the projection shapes.  One launch, the planned list, three vectors
-    through the tensor-core kernel; rows at both ends, around the tile-group edges and random ones."""
+    through the tensor-core kernel; rows at both ends, around edges of tiles and random ones."""
     from paper_2609_35465_b200 import tetra as tt
     N, K, batch = 151936, 4096, 3
     B, ntail = K // 24, K % 24
