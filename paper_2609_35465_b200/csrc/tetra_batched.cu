@@ -123,7 +123,7 @@ __device__ __forceinline__ float decode_halves(uint32_t sm_tab, uint32_t w0, uin
     }
     const __half2 n = __hadd2(n0, n1);
     const __half m4 = __hadd(__hadd(__low2half(n), __high2half(n)), __ushort_as_half(0x6400));  // 1024 + 4 m
-    return lds32f(uint32_t(__half_as_ushort(m4)) * 4u + (nb.norm0 >> 6) - 0x6400u * 4u);
+    return lds32f(uint32_t(__half_as_ushort(m4)) * 2u + (nb.norm0 >> kNormShift) - 0x6400u * 2u);
 }
 
 // Eight consecutive activations starting at x[0], of which `n` exist; x is 2-byte aligned.

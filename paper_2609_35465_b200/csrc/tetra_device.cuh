@@ -140,15 +140,17 @@ __device__ __forceinline__ uint32_t trellis_path(uint64_t w) { return uint32_t((
 constexpr uint32_t kSmRows = 0;
 constexpr uint32_t kSmMid = 16384;
 constexpr uint32_t kSmScale = 24576;
-constexpr uint32_t kSmMaskH = 25600;
-constexpr uint32_t kSmMaskXp = 25728;
-constexpr uint32_t kSmGap = 25856, kStagedGap = 768;  // nothing to stage there
-constexpr uint32_t kScaleGain = 2048;  // from one gain's scale table to the other's
+constexpr uint32_t kSmMaskH = 24832;
+constexpr uint32_t kSmMaskXp = 24960;
+constexpr uint32_t kSmGap = 25088, kStagedGap = 512;  // nothing to stage there
+constexpr uint32_t kScaleGain = 1024;  // from one gain's scale table to the other's
+constexpr int kNormShift = 7;          // from the squared norm of eight times the point (1024 m) to bytes of a scale table
 constexpr uint32_t kSmAlign = 16384;  // the staged copy starts on a 16 KiB boundary of shared memory
 static_assert(kSmMid == offsetof(DeviceTables, mid_fast) - kFastOffset, "staged layout");
 static_assert(kSmScale == offsetof(DeviceTables, scale) - kFastOffset, "staged layout");
 static_assert(kSmScale + kScaleGain == offsetof(DeviceTables, scale1) - kFastOffset && kSmScale % (2 * kScaleGain) == 0, "staged layout");
-static_assert(kSmMaskH == offsetof(DeviceTables, mask_h) - kFastOffset, "staged layout");
+static_assert(sizeof(DeviceTables::scale) / 32 << kNormShift == 1024, "bytes per norm");
+static_assert(kSmMaskH == offsetof(DeviceTables, mask_h) - kFastOffset && kSmMaskH % 64 == 0, "staged layout");
 static_assert(kSmMaskXp == offsetof(DeviceTables, mask_xp) - kFastOffset && kSmMaskXp % 128 == 0, "staged layout");
 
 // Copies the staged part of the tables to the first 16 KiB boundary of the
@@ -196,7 +198,7 @@ static_assert(fast_nibble(word_coordinate(0, 1)) == 3 && fast_nibble(word_coordi
 struct NibbleBlock {
     uint32_t z[3];  // section s: coordinate j's z at bits 4 fast_nibble(j)
     uint32_t p4;    // bit 2: p (the other bits are an address)
-    uint32_t norm0; // 64 times the shared-memory address of the gain's scale table
+    uint32_t norm0; // 128 times the shared-memory address of the gain's scale table
 };
 // HI = false: w1 sits in bits 0..15 of `w1pair`; HI = true: in bits 16..31.
 // sm_tab: shared-memory address of the staged tables, a multiple of 16 KiB, so
@@ -212,7 +214,7 @@ __device__ __forceinline__ void decode_nibbles(uint32_t sm_tab, uint32_t w0, uin
     const uint32_t a4 = ((w0 >> 23) & 0x3Cu) | (sm_tab + kSmMaskH);
     const uint32_t b4 = (__funnelshift_l(w0, w0, 4) & 0x3Cu) | (sm_tab + kSmMaskH);
     const uint32_t x4 = ((sh >> 11) & 0x7Cu) | (sm_tab + kSmMaskXp);     // (p | x << 1) * 4
-    out.norm0 = (w3 & (kScaleGain << 6)) | ((sm_tab + kSmScale) << 6);
+    out.norm0 = (w3 & (kScaleGain << kNormShift)) | ((sm_tab + kSmScale) << kNormShift);
     const uint32_t row1 = lds32(addr1);
     const uint32_t row2 = lds32(addr2);
     // class of row 3 (Eq. (3)): p ^ r ^ delta, delta = [i2 >= 1240] = bit 11 of i2 + 808; all three at bit 13
@@ -240,13 +242,13 @@ __device__ __forceinline__ void fast_decode(uint32_t sm_tab, uint32_t w0, uint32
 }
 
 // Shared-memory address of -gain[g] / sqrt(16 m).  The squared norm of the packed point is 64 * 16 m and a gain's table
-// has 16 bytes per m (16 m <= 416 for every word, Sec. 3.4), so the sum that starts from 64 times the table's address is
-// 64 times the entry's; the second gain's table lies kScaleGain bytes on, which is g where the word shifted for i3 has it.
+// has 8 bytes per m (16 m <= 416 for every word, Sec. 3.4), so the sum that starts from 128 times the table's address is
+// 128 times the entry's; the second gain's table lies kScaleGain bytes on, which is g where the word shifted for i3 has it.
 __device__ __forceinline__ uint32_t scale_address(const FastBlock& fb) {
     int n2 = int(fb.norm0);
 #pragma unroll
     for (int k = 0; k < 6; ++k) n2 = dp4a_ss(fb.y[k], fb.y[k], n2);
-    return uint32_t(n2) >> 6;
+    return uint32_t(n2) >> kNormShift;
 }
 
 // sum of -y q from the sums of -8 y over the planes of q (high signed, middle, low): every term is a multiple of
@@ -260,7 +262,7 @@ __device__ __forceinline__ int combine_planes(int dh, int dm, int dl) { return d
 // step = 2^(E-22) with 2^E <= max|x| < 2^(E+1); q_j = rint(x_j / step), |q_j| < 2^23,
 // stored as three byte planes (bits 23..16 signed, 15..8 and 7..0 unsigned), four
 // coordinates per 32-bit word in the decoder's order (word_coordinate): words 0..5 high, 6..11 middle, 12..17 low plane;
-// word 18 = step (float), word 19 is spare.  A float16 x_j is held exactly when
+// words 18 and 19 = step (float), twice.  A float16 x_j is held exactly when
 // |x_j| >= 2^(E-12); smaller ones are rounded to a multiple of the step.  If a value
 // is NaN or infinite the step is NaN (and the planes zero).
 // The 24 activations of block column c, as twelve pairs of float16 (zeros beyond K).
@@ -345,7 +347,7 @@ __device__ __forceinline__ void quantise_column(const __half* __restrict__ x, in
         }
     }
     out[18] = __float_as_uint(step);
-    out[19] = 0u;
+    out[19] = out[18];
 }
 
 }  // namespace tetra

@@ -17,7 +17,7 @@ struct PaperTables {
 static_assert(sizeof(PaperTables) == 18816, "paper table blob is 18,816 bytes");
 
 constexpr uint32_t kTableMagic = 0x54455442u;  // "TETB"
-constexpr uint32_t kTableVersion = 10;
+constexpr uint32_t kTableVersion = 11;
 // Nibble of a fast table word that belongs to coordinate j of a section: neighbours are sixteen bits apart, so that one
 // mask picks the pair (j, j + 1) as the two halves of a register.
 constexpr int fast_nibble(int j) { return (j >> 1) + 4 * (j & 1); }
@@ -39,20 +39,20 @@ struct DeviceTables {
     //  sub-table's offset can be OR-ed into an index instead of added)
     uint32_t rows_fast[4096];   // +0
     uint32_t mid_fast[2048];    // +16384: rows_fast[mix(i2)], indexed by i2 directly
-    float scale[32][4];         // +24576: -gain[0] / sqrt(16 m) in entry [m][0], 16 bytes per m.  Minus: the fast decoder
-                                //         emits minus (eight times) the point.
-    uint32_t spare0_[128];      // +25088
+    float scale[32][2];         // +24576: -gain[0] / sqrt(16 m) in entry [m][0], 8 bytes per m: sixteen neighbouring norms in
+                                //         different banks.  Minus: the fast decoder emits minus (eight times) the point.
     // Pattern-byte masks of the Turyn coordinates: nibble fast_nibble(j) all ones where the Hamming word has coordinate j
     // set; H for a and b, H' for x.  mask_xp has x and the parity in one index, x << 1 | p, and is complemented
     // where p = 1.
-    uint32_t mask_h[16];        // +25600
-    uint32_t spare2_[16];       // +25664
-    uint32_t mask_xp[32];       // +25728
-    uint32_t spare1_[192];      // +25856
-    float scale1[32][4];        // +26624: the same for gain[1], at a power of two from the first
+    uint32_t mask_h[16];        // +24832
+    uint32_t spare0_[16];       // +24896
+    uint32_t mask_xp[32];       // +24960
+    uint32_t spare1_[128];      // +25088
+    float scale1[32][2];        // +25600: the same for gain[1], at a power of two from the first
     // ---- pack-time only (global memory) ------------------------------------
     // 12 trellis bits (s8 | b1<<6 | b2<<7 | b3<<11) -> Turyn coordinates a | b<<4 | x<<8.
     uint16_t trellis_to_abx[4096];
+    uint32_t spare2_[320];      // the blob keeps its size
 };
 
 constexpr size_t kFastOffset = offsetof(DeviceTables, rows_fast);
