@@ -186,6 +186,17 @@ constexpr HalfList kHalfListHost = half_list();
 constexpr int kHalfVectors = kHalfListHost.n;
 __device__ const HalfList kHalfList = half_list();
 
+// Where the low tables keep the best over weights W, W - 2, ...: offset | largest kappa << 16.
+struct LowIndex {
+    uint32_t v[kMaxW + 1];
+};
+constexpr LowIndex low_index() {
+    LowIndex L{};
+    for (int w = 0; w <= kMaxW; ++w) L.v[w] = uint32_t(c_offset(w)) | (uint32_t(c_last(w)) << 16);
+    return L;
+}
+__device__ const LowIndex kLowIndex = low_index();
+
 template <int I, int N, typename F>
 __device__ __forceinline__ void static_for(F&& f) {
     if constexpr (I < N) {
@@ -232,6 +243,7 @@ struct EncShared {
     float rs[32];             // 1 / sqrt(16 m)
     float w[24];
     uint32_t halves[kHalfVectors];
+    uint32_t low_index[kMaxW + 1];
     uint8_t bytes[64];        // h(alpha) + h'(xi)
     float red_val[6];         // per warp: the best of the objective
     uint32_t red_arg[6];      // and the thread that holds it
@@ -777,24 +789,28 @@ __device__ __forceinline__ bool row_in_list(int section, int cls, int w, uint32_
     if (section == 1) return cls ? w <= 7 : (w <= 6 || (w == 8 && row <= kLastRowMiddle0));
     return cls ? (w <= 9 || (w == 11 && row <= kLastRowClass1)) : (w <= 8 || (w == 10 && row <= kLastRowClass0));
 }
-// correlation and kappa of a half vector, the sums in the tables' order
-__device__ __forceinline__ float half_corr(bool even, const float* w4, int nibble, uint32_t value, int& kap) {
-    float sum = 0.f;
-    kap = 0;
+// The products of a half with the values of every rank, a lane each: lane 5 j + r holds w_j y(pattern bit j, rank r).
+__device__ __forceinline__ float half_products(bool even, const float* w4, int nibble) {
+    const int lane = threadIdx.x & 31, j = min(lane / 5, 3), r = lane - 5 * (lane / 5), c = (nibble >> j) & 1, t = (r + 1) >> 1;
+    const int v0 = (r & 1) ? 4 * t : -4 * t;
+    return __fmul_rn(w4[j], float(even ? (c ? 2 - v0 : v0) : (c ? v0 - 1 : 1 - v0)));
+}
+// Correlation of a half vector from those, the sum in the tables' order; all lanes.
+__device__ __forceinline__ float half_corr(float products, uint32_t value) {
+    float sum = __shfl_sync(0xFFFFFFFFu, products, int(value & 7u));
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int c = (nibble >> j) & 1, r = int((value >> (4 * j)) & 7u), t = (r + 1) >> 1;
-        const int v0 = (r & 1) ? 4 * t : -4 * t;
-        int y;
-        if (even) {
-            y = c ? 2 - v0 : v0;
-            kap += c ? ((r & 1) ? t * t - t : t * t + t) : t * t;
-        } else {
-            y = c ? v0 - 1 : 1 - v0;
-        }
-        sum = __fadd_rn(sum, __fmul_rn(w4[j], float(y)));
-    }
+    for (int j = 1; j < 4; ++j) sum = __fadd_rn(sum, __shfl_sync(0xFFFFFFFFu, products, 5 * j + int((value >> (4 * j)) & 7u)));
     return sum;
+}
+// kappa of a half vector at even parity: four bits per rank, by pattern bit.
+__device__ __forceinline__ int half_kappa(int nibble, uint32_t value) {
+    constexpr uint32_t k0 = 0x44110u, k1 = 0x62200u;
+    static_assert(kappa(0, 1) == 1 && kappa(0, 2) == 1 && kappa(0, 3) == 4 && kappa(0, 4) == 4 && kappa(0, 0) == 0, "kappa");
+    static_assert(kappa(1, 1) == 0 && kappa(1, 2) == 2 && kappa(1, 3) == 2 && kappa(1, 4) == 6 && kappa(1, 0) == 0, "kappa");
+    uint32_t kap = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) kap += (((nibble >> j) & 1 ? k1 : k0) >> ((value >> (4 * j) & 7u) * 4u)) & 15u;
+    return int(kap);
 }
 
 // Looks for the row of section s whose correlation with the pair's byte (e = 0) or its complement (e = 1) is the
@@ -817,48 +833,41 @@ __device__ __noinline__ void trace_section(EncShared& S, const DeviceTables* __r
         float high_corr = 0.f;
         int high_kap = 0;
         bool have = false;
+        const float high_products = half_products(even, w + 4, nhi), low_products = half_products(even, w, nlo);
+        const uint32_t lim = s == 1 ? kLastRowMiddle0 >> 16 : (cls ? kLastRowClass1 >> 16 : kLastRowClass0 >> 16);
+        const bool limited = !(s == 1 && cls);            // the list has a partial shell
+        const int full = s == 1 ? (cls ? 7 : 6) : (cls ? 9 : 8);
+#pragma unroll 1
         for (int i0 = 0; i0 < kHalfVectors && !have; i0 += 32) {
-            const int i = i0 + lane;
+            const bool there = i0 + lane < kHalfVectors;
+            const uint32_t hv = S.halves[there ? i0 + lane : 0];
+            const int wh = int(hv >> 16);
+            const uint32_t v = hv & 0xFFFFu;
+            const float hc = half_corr(high_products, v);
             bool hit = false;
-            uint32_t hv = 0;
-            float hc = 0.f;
             int hk = 0;
-            if (i < kHalfVectors) {
-                hv = S.halves[i];
-                const int wh = int(hv >> 16);
-                const uint32_t v = hv & 0xFFFFu;
-                hc = half_corr(even, w + 4, nhi, v, hk);
-                const uint32_t lim = s == 1 ? kLastRowMiddle0 >> 16 : (cls ? kLastRowClass1 >> 16 : kLastRowClass0 >> 16);
-                const bool limited = !(s == 1 && cls);            // the list has a partial shell
-                const int full = s == 1 ? (cls ? 7 : 6) : (cls ? 9 : 8);
-                if (even) {
-                    auto partner = [&](int W) {  // best low half of weights W, W - 2, ...
-                        if (W < 0) return;
-                        int off = 0, last = 0;
-                        static_for<0, kMaxW + 1>([&](auto ai) {
-                            constexpr int a = decltype(ai)::value;
-                            if (W == a) { off = kAtC<a>; last = kLastC<a>; }
-                        });
-                        const int kl = kap - hk;
-                        if (kl >= 0 && kl <= last) hit = hit || __fadd_rn(hc, lo[off + kl]) == target;
-                    };
-                    partner(full - wh);
-                    if (limited && v < lim) partner(full + 2 - wh);
-                    if (limited && v == lim) {
-                        const int kl = kap - hk;
-                        const int n = cls ? 5 : 3, off = cls ? kOffRes1 : kOffRes0;
-                        if (kl >= 0 && kl < n) hit = hit || __fadd_rn(hc, lo[off + kl]) == target;
-                    }
-                } else {
-                    const int wl = w_total - wh;
-                    if (wl >= 0) {
-                        const bool whole = w_total <= full || (limited && v < lim);
-                        if (whole) hit = __fadd_rn(hc, lo[wl]) == target;
-                        else if (limited && v == lim) hit = __fadd_rn(hc, lo[cls ? 13 : 12]) == target;
-                    }
+            if (even) {
+                hk = half_kappa(nhi, v);
+                const int kl = kap - hk;
+                auto partner = [&](int W) {  // best low half of weights W, W - 2, ...
+                    const uint32_t at = S.low_index[max(W, 0)];
+                    if (W >= 0 && kl >= 0 && kl <= int(at >> 16)) hit = hit || __fadd_rn(hc, lo[int(at & 0xFFFFu) + kl]) == target;
+                };
+                partner(full - wh);
+                if (limited && v < lim) partner(full + 2 - wh);
+                if (limited && v == lim) {
+                    const int n = cls ? 5 : 3, off = cls ? kOffRes1 : kOffRes0;
+                    if (kl >= 0 && kl < n) hit = hit || __fadd_rn(hc, lo[off + kl]) == target;
+                }
+            } else {
+                const int wl = w_total - wh;
+                if (wl >= 0) {
+                    const bool whole = w_total <= full || (limited && v < lim);
+                    if (whole) hit = __fadd_rn(hc, lo[wl]) == target;
+                    else if (limited && v == lim) hit = __fadd_rn(hc, lo[cls ? 13 : 12]) == target;
                 }
             }
-            const uint32_t any = __ballot_sync(0xFFFFFFFFu, hit);
+            const uint32_t any = __ballot_sync(0xFFFFFFFFu, hit && there);
             if (any) {
                 const int src = __ffs(int(any)) - 1;
                 high = __shfl_sync(0xFFFFFFFFu, hv, src);
@@ -868,19 +877,15 @@ __device__ __noinline__ void trace_section(EncShared& S, const DeviceTables* __r
             }
         }
         // 2. the low half: sum, norm and membership decide
+#pragma unroll 1
         for (int i0 = 0; i0 < kHalfVectors && have && !found; i0 += 32) {
-            const int i = i0 + lane;
-            bool hit = false;
-            uint32_t cand = 0;
-            if (i < kHalfVectors) {
-                const uint32_t lv = S.halves[i];
-                int lk;
-                const float lc = half_corr(even, w, nlo, lv & 0xFFFFu, lk);
-                const int wt = int(high >> 16) + int(lv >> 16);
-                cand = ((high & 0xFFFFu) << 16) | (lv & 0xFFFFu);
-                hit = __fadd_rn(high_corr, lc) == target && (wt & 1) == cls && (even ? high_kap + lk == kap : wt == w_total) &&
-                      row_in_list(s, cls, wt, cand);
-            }
+            const bool there = i0 + lane < kHalfVectors;
+            const uint32_t lv = S.halves[there ? i0 + lane : 0];
+            const float lc = half_corr(low_products, lv & 0xFFFFu);
+            const int wt = int(high >> 16) + int(lv >> 16);
+            const uint32_t cand = ((high & 0xFFFFu) << 16) | (lv & 0xFFFFu);
+            const bool hit = there && __fadd_rn(high_corr, lc) == target && (wt & 1) == cls &&
+                             (even ? high_kap + half_kappa(nlo, lv) == kap : wt == w_total) && row_in_list(s, cls, wt, cand);
             const uint32_t any = __ballot_sync(0xFFFFFFFFu, hit);
             if (any) {
                 row = __shfl_sync(0xFFFFFFFFu, cand, __ffs(int(any)) - 1);
@@ -1017,15 +1022,21 @@ k_encode(const float* __restrict__ w, const float* __restrict__ sigma, const Dev
     if (tid < 64) S.bytes[tid] = uint8_t(pair_byte(tid));
     if (tid < 32) S.rs[tid] = tab->paper.rsqrt16m[tid];
     for (int i = tid; i < kHalfVectors; i += kEncThreads) S.halves[i] = kHalfList.v[i];
+    if (tid <= kMaxW) S.low_index[tid] = kLowIndex.v[tid];
     const float gain0 = tab->gain[0], gain1 = tab->gain[1];
 
     // every group of every CTA takes the same number of turns; the first groups of all CTAs come first, so that few
     // blocks spread over all SMs
     const size_t per_turn = size_t(gridDim.x) * kEncGroups;
+    const size_t place = size_t(group) * gridDim.x + blockIdx.x;
+    float next_w = tid < 24 && place < nblocks ? w[place * 24 + tid] : 0.f;  // a turn ahead
     for (size_t first = 0; first < nblocks; first += per_turn) {
-        const size_t block = first + size_t(group) * gridDim.x + blockIdx.x;
+        const size_t block = first + place;
         const bool mine = block < nblocks;
-        if (tid < 24) S.w[tid] = mine ? w[block * 24 + tid] : 0.f;
+        if (tid < 24) {
+            S.w[tid] = next_w;
+            next_w = block + per_turn < nblocks ? w[(block + per_turn) * 24 + tid] : 0.f;
+        }
         if (tid < 3) S.hit_pair[tid] = S.hit_cls[tid] = S.hit_k[tid] = 0;  // what a block without a best point (NaN) is traced to
         __syncthreads();
         float wn2 = 0.f;
