@@ -1065,9 +1065,9 @@ k_encode(const float* __restrict__ w, const float* __restrict__ sigma, const Dev
         __syncthreads();
         const int warp = tid >> 5, lane = tid & 31;
         if (live) {  // section tables at even parity, two warps per section
-            const int s = tid >> 6, pair = tid & 63;
-            if (s == 1) section_rows<true, true>(S, 1, pair);
-            else section_rows<true, false>(S, s, pair);
+            const int pair = tid & 63;
+            if (tid < 64) section_rows<true, true>(S, 1, pair);
+            else section_rows<true, false>(S, tid < 128 ? 0 : 2, pair);
         }
         __syncthreads();
         // Join and objective.  Even parity: warps 0..3, thread = (end pair, class parity).  The odd parity has rows of
