@@ -241,7 +241,7 @@ struct EncShared {
     alignas(16) float F[3][2][64 * kRow];
     alignas(16) float O[3][2][64 * kOddRow];
     float rs[32];             // 1 / sqrt(16 m)
-    float w[24];
+    float w[2][24];           // this turn's and the next one's
     uint32_t halves[kHalfVectors];
     uint32_t low_index[kMaxW + 1];
     uint8_t bytes[64];        // h(alpha) + h'(xi)
@@ -253,6 +253,8 @@ struct EncShared {
     // the winner so far, per section: byte pair, class, index and value of its table entry
     int hit_pair[3], hit_cls[3], hit_k[3];
     float hit_target[3];
+    float out_val, out_wn2;   // of the traced block: the best of the objective, the squared norm of its weights
+    int out_live, out_even;
     // its row, looked for with the pair's byte and with its complement: index inside the section's list, or none
     uint32_t found_row[3][2];
     bool found[3][2];
@@ -815,12 +817,12 @@ __device__ __forceinline__ int half_kappa(int nibble, uint32_t value) {
 
 // Looks for the row of section s whose correlation with the pair's byte (e = 0) or its complement (e = 1) is the
 // winner's at its index of the section's table.
-__device__ __noinline__ void trace_section(EncShared& S, const DeviceTables* __restrict__ tab, bool even, int s, int e) {
+__device__ __noinline__ void trace_section(EncShared& S, const DeviceTables* __restrict__ tab, const float* w24, bool even, int s, int e) {
     const int lane = threadIdx.x & 31;
     const int cls = S.hit_cls[s], k = S.hit_k[s];
     const float target = S.hit_target[s];
     const int w_total = 2 * k + cls;  // odd parity: the row's weight
-    const float* w = S.w + 8 * s;
+    const float* w = w24 + 8 * s;
     uint32_t row = 0;
     const uint32_t byte = S.bytes[S.hit_pair[s]] ^ (e ? 0xFFu : 0u);
     bool found = false;
@@ -1029,19 +1031,41 @@ k_encode(const float* __restrict__ w, const float* __restrict__ sigma, const Dev
     // blocks spread over all SMs
     const size_t per_turn = size_t(gridDim.x) * kEncGroups;
     const size_t place = size_t(group) * gridDim.x + blockIdx.x;
-    float next_w = tid < 24 && place < nblocks ? w[place * 24 + tid] : 0.f;  // a turn ahead
-    for (size_t first = 0; first < nblocks; first += per_turn) {
-        const size_t block = first + place;
-        const bool mine = block < nblocks;
-        if (tid < 24) {
-            S.w[tid] = next_w;
-            next_w = block + per_turn < nblocks ? w[(block + per_turn) * 24 + tid] : 0.f;
+    const int warp = tid >> 5, lane = tid & 31;
+    float next_w = 0.f;  // a turn ahead of its place in shared memory
+    if (tid < 24) {
+        S.w[0][tid] = place < nblocks ? w[place * 24 + tid] : 0.f;
+        next_w = place + per_turn < nblocks ? w[(place + per_turn) * 24 + tid] : 0.f;
+    }
+    // The word of a traced block, its gain bit, its cosine; one warp.
+    auto emit = [&](size_t block) {
+        const bool live = S.out_live != 0;
+        const float best_val = S.out_val;
+        const uint64_t best_word = live && best_val > 0.f ? winner_word(S, tab, S.out_even != 0) : 0ull;
+        if (block < nblocks && lane == 0) {
+            const float sg_ = sigma ? sigma[block] : 1.f;
+            // gain bit: argmin_g (gain sigma)^2 - 2 gain sigma <w, y> / |y|
+            const float c = best_val;
+            const float e0 = gain0 * sg_ * (gain0 * sg_ - 2.f * c), e1 = gain1 * sg_ * (gain1 * sg_ - 2.f * c);
+            const uint64_t word = live ? best_word | (uint64_t(e1 < e0 ? 1u : 0u) << 47) : 0u;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) codes[block * 6 + k] = uint8_t(word >> (8 * k));
+            if (cosine) cosine[block] = live ? best_val / sqrtf(S.out_wn2) : 0.f;
         }
-        if (tid < 3) S.hit_pair[tid] = S.hit_cls[tid] = S.hit_k[tid] = 0;  // what a block without a best point (NaN) is traced to
-        __syncthreads();
+    };
+    __syncthreads();
+    int buf = 0;
+    size_t first = 0;
+    for (; first < nblocks; first += per_turn, buf ^= 1) {
+        const size_t block = first + place;
+        const float* w24 = S.w[buf];
+        if (tid < 24) {
+            S.w[buf ^ 1][tid] = next_w;
+            next_w = block + 2 * per_turn < nblocks ? w[(block + 2 * per_turn) * 24 + tid] : 0.f;
+        }
         float wn2 = 0.f;
 #pragma unroll
-        for (int j = 0; j < 24; ++j) wn2 = fmaf(S.w[j], S.w[j], wn2);
+        for (int j = 0; j < 24; ++j) wn2 = fmaf(w24[j], w24[j], wn2);
         const bool live = wn2 != 0.f;  // a zero block encodes as the all-zero word
         if (live) {
             // half tables, a thread per (section, nibble): warps 0 and 1 the high halves at even parity, 2 and 3 the low
@@ -1050,21 +1074,22 @@ k_encode(const float* __restrict__ w, const float* __restrict__ sigma, const Dev
             if (tid < 128) {
                 const int s = (tid & 63) >> 4;
                 if (s < 3) {
-                    if (tid < 64) half_even<true>(S.w + 8 * s + 4, nibble, s == 1, S.hi[s] + nibble * kHiStride);
-                    else half_even<false>(S.w + 8 * s, nibble, s == 1, S.lo[s] + nibble * kLoStride);
+                    if (tid < 64) half_even<true>(w24 + 8 * s + 4, nibble, s == 1, S.hi[s] + nibble * kHiStride);
+                    else half_even<false>(w24 + 8 * s, nibble, s == 1, S.lo[s] + nibble * kLoStride);
                 }
             } else if (tid < 160) {
                 const int s = (tid & 16) ? 2 : 0;
-                half_odd<true, false>(S.w + 8 * s + 4, nibble, S.hi_odd[s] + nibble * kOddHiStride);
-                half_odd<false, false>(S.w + 8 * s, nibble, S.lo_odd[s] + nibble * kOddLoStride);
+                half_odd<true, false>(w24 + 8 * s + 4, nibble, S.hi_odd[s] + nibble * kOddHiStride);
+                half_odd<false, false>(w24 + 8 * s, nibble, S.lo_odd[s] + nibble * kOddLoStride);
             } else if ((tid & 16) == 0) {
-                half_odd<true, true>(S.w + 12, nibble, S.hi_odd[1] + nibble * kOddHiStride);
-                half_odd<false, true>(S.w + 8, nibble, S.lo_odd[1] + nibble * kOddLoStride);
+                half_odd<true, true>(w24 + 12, nibble, S.hi_odd[1] + nibble * kOddHiStride);
+                half_odd<false, true>(w24 + 8, nibble, S.lo_odd[1] + nibble * kOddLoStride);
             }
         }
+        if (warp == 5 && first) emit(block - per_turn);  // the block of the turn before; this warp's half tables are the shortest
         __syncthreads();
-        const int warp = tid >> 5, lane = tid & 31;
-        if (live) {  // section tables at even parity, two warps per section
+        if (live) {  // section tables at even parity, two warps per section; the schedulers of warps 0 and 1 have a warp more
+                     // than the others and get the middle section's, the shorter ones
             const int pair = tid & 63;
             if (tid < 64) section_rows<true, true>(S, 1, pair);
             else section_rows<true, false>(S, tid < 128 ? 0 : 2, pair);
@@ -1109,36 +1134,36 @@ k_encode(const float* __restrict__ w, const float* __restrict__ sigma, const Dev
                     best_val = S.red_val[k % 6];
                     winner = S.red_arg[k % 6];
                 }
-            if (uint32_t(tid) == winner) {
-#pragma unroll
-                for (int i = 0; i < kH; ++i) S.win_H[i] = H[i];
-                S.win_G = corr;
-                S.win_arg = arg;
-                S.win_par = par;
-            }
         }
         const bool best_even = winner < 128u;
-        __syncthreads();
-        if (live && best_val > 0.f && warp == 0) trace_join(S, best_even, int(winner) & 63, S.win_par, S.win_arg);
-        __syncthreads();
-        if (live) {  // a warp per section and byte of its pair
-            trace_section(S, tab, best_even, warp >> 1, warp & 1);
+        if (uint32_t(warp) == winner >> 5) {  // the winner's warp traces it through the join
+            if (live && best_val > 0.f) {
+                if (uint32_t(tid) == winner) {
+#pragma unroll
+                    for (int i = 0; i < kH; ++i) S.win_H[i] = H[i];
+                    S.win_G = corr;
+                    S.win_arg = arg;
+                    S.win_par = par;
+                }
+                __syncwarp();
+                trace_join(S, best_even, int(winner) & 63, S.win_par, S.win_arg);
+            } else if (lane < 3) {
+                S.hit_pair[lane] = S.hit_cls[lane] = S.hit_k[lane] = 0;  // what a block without a best point (NaN) is traced to
+            }
         }
         __syncthreads();
-        const uint64_t best_word = live && tid < 32 && best_val > 0.f ? winner_word(S, tab, best_even) : 0ull;
-
-        if (mine && tid == 0) {
-            const float sg_ = sigma ? sigma[block] : 1.f;
-            // gain bit: argmin_g (gain sigma)^2 - 2 gain sigma <w, y> / |y|
-            const float c = best_val;
-            const float e0 = gain0 * sg_ * (gain0 * sg_ - 2.f * c), e1 = gain1 * sg_ * (gain1 * sg_ - 2.f * c);
-            const uint64_t word = live ? best_word | (uint64_t(e1 < e0 ? 1u : 0u) << 47) : 0u;
-#pragma unroll
-            for (int k = 0; k < 6; ++k) codes[block * 6 + k] = uint8_t(word >> (8 * k));
-            if (cosine) cosine[block] = live ? best_val / sqrtf(wn2) : 0.f;
+        if (live) {  // a warp per section and byte of its pair
+            trace_section(S, tab, w24, best_even, warp >> 1, warp & 1);
+        }
+        if (tid == 160) {
+            S.out_val = best_val;
+            S.out_wn2 = wn2;
+            S.out_live = live;
+            S.out_even = best_even;
         }
         __syncthreads();
     }
+    if (warp == 5) emit(first - per_turn + place);
 }
 
 }  // namespace
