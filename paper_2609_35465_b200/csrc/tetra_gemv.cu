@@ -298,7 +298,8 @@ __device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, uns
     // bytes (one 16-byte part per lane), filled with cp.async one pass ahead, so the prefetch holds
     // no registers while eight blocks are being decoded.  Each lane reads back only what it copied.
     const uint32_t ring = sm_tab + uint32_t(kFastBytes) + uint32_t(kUnitWarps * kRedFloats * 4) + uint32_t(warp) * 3072u + uint32_t(lane) * 16u;
-    int pass_parity = 0;
+    uint32_t slot = ring;                  // of the pass at hand
+    const uint32_t slots = 2 * ring + 1536;  // the two slots' sum
 
     for (;; u += u_step) {
         if (u >= u_end) {
@@ -341,67 +342,59 @@ __device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, uns
 
         if (!have_record) {
             const uint4* first = CGf > 0 ? codes0 + lane : rem_rec;
-            const uint32_t dst = ring + uint32_t(pass_parity * 1536);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst), "l"(first));
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 512), "l"(first + Bu));
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 1024), "l"(first + 2 * Bu));
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(slot), "l"(first));
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(slot + 512), "l"(first + Bu));
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(slot + 1024), "l"(first + 2 * Bu));
             asm volatile("cp.async.commit_group;");
         }
-        have_record = false;
         float s0 = 0.f, s1 = 0.f, s2 = 0.f;  // per row group: this lane's partial row sum (row lane / 4)
         float acc[8];
 #pragma unroll
         for (int r = 0; r < 8; ++r) acc[r] = 0.f;
 
-        // One pass = one 48-byte record per lane: the full column groups of each row group in turn,
-        // then the joint pass over the partial column group (a single call site of the decoder).
-        const int full_passes = ng * CGf, passes = full_passes + (rem ? 1 : 0);
-        int gi = 0, cg = 0;
-        for (int pass = 0; pass < passes; ++pass) {
-            const bool joint = pass >= full_passes;
+        // One pass = one 48-byte record per lane: the full column groups of each row group in turn, then the joint pass over
+        // the partial column group (a single call site of the decoder).  A segment is a row group's full column groups, or
+        // the joint pass: inside one, records and activations follow at fixed distances.
+        int gi = 0;
+        bool joint = CGf == 0, lane_on = !joint || lane_in;
+        int seg = joint ? 1 : CGf;                                         // passes left in the segment
+        // places are kept as 16-byte units from the matrix's first record, in 32 bits
+        const uint32_t unit0 = uint32_t(g0) * 3u * Bu + uint32_t(lane), unit_rem = uint32_t(rem_rec - codes_p);
+        uint32_t record = joint ? unit_rem : unit0;                        // of the pass at hand
+        uint32_t x_at = (joint ? lane_col : uint32_t(lane)) * uint32_t(kXqBytesPerCol);
+        // the first record behind the segment: the next row group's, the joint pass's, the next unit's
+        constexpr uint32_t kNone = 0xFFFFFFFFu;
+        auto behind = [&]() -> uint32_t {
+            if (!joint && gi + 1 < ng) return unit0 + uint32_t(gi + 1) * 3u * Bu;
+            if (!joint && rem) return unit_rem;
+            return next_unit_here ? unit0 + uint32_t(u_step * R) * 3u * Bu : kNone;
+        };
+        uint32_t after = behind();
+        for (;;) {
             uint4 a, b, h;
             {
                 asm volatile("cp.async.wait_group 0;" ::: "memory");
-                const uint32_t src = ring + uint32_t(pass_parity * 1536);
-                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w) : "r"(src));
-                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "r"(src + 512));
-                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(h.x), "=r"(h.y), "=r"(h.z), "=r"(h.w) : "r"(src + 1024));
+                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w) : "r"(slot));
+                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "r"(slot + 512));
+                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(h.x), "=r"(h.y), "=r"(h.z), "=r"(h.w) : "r"(slot + 1024));
             }
+            slot = slots - slot;
             // ahead of the next record's copies: the same unit serves both in order, and a load behind a copy waits for
             // memory (Qwen3-8B pass 810 -> 803 us)
             LaneX X;
-            load_lane_x(xq_p + (joint ? lane_col : uint32_t(cg * 32 + lane)) * uint32_t(kXqBytesPerCol),
-                        !joint || lane_in, X);
+            load_lane_x(xq_p + x_at, lane_on, X);
+            x_at += 32 * kXqBytesPerCol;
             // prefetch the next pass's record (or the first one of this warp's next unit)
-            const uint4* next = nullptr;
-            if (pass + 1 < full_passes) {
-                const bool wrap = cg + 1 == CGf;
-                next = codes0 + size_t(wrap ? gi + 1 : gi) * 3 * Bu + (wrap ? 0 : cg + 1) * 32 + lane;
-            } else if (pass + 1 < passes) {
-                next = rem_rec;
-            } else if (next_unit_here) {
-                next = codes0 + size_t(u_step) * R * 3 * Bu + lane;
-                have_record = true;
-            }
-            if (next) {
-                const uint32_t dst = ring + uint32_t((pass_parity ^ 1) * 1536);
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst), "l"(next));
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 512), "l"(next + Bu));
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 1024), "l"(next + 2 * Bu));
+            record = seg == 1 ? after : record + 32u;
+            if (record != kNone) {
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(slot), "l"(codes_p + record));
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(slot + 512), "l"(codes_p + (record + Bu)));
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(slot + 1024), "l"(codes_p + (record + 2 * Bu)));
             }
             asm volatile("cp.async.commit_group;");
-            record_accumulate(sm_tab, a, b, h, X, acc);  // acc is zero when the joint pass begins
-            pass_parity ^= 1;
-            if (!joint) {
-                if (++cg == CGf) {  // row group done: fold its eight accumulators into this lane's row
-                    const float t = transpose_partial(red, lane, acc);
-                    if (gi == 0) s0 = t; else if (gi == 1) s1 = t; else s2 = t;
-#pragma unroll
-                    for (int r = 0; r < 8; ++r) acc[r] = 0.f;
-                    cg = 0;
-                    ++gi;
-                }
-            } else {
+            record_accumulate(sm_tab, a, b, h, X, acc);  // acc is zero when a segment begins
+            if (--seg) continue;
+            if (joint) {
                 // lane -> (row group, column); lane l then sums, for row l / 4, the columns
                 // k = l % 4, l % 4 + 4, ... of every row group's segment of the buffer
                 __syncwarp();
@@ -414,8 +407,26 @@ __device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, uns
                     if (R > 1) s1 += rr[rem + k];
                     if (R > 2) s2 += rr[2 * rem + k];
                 }
+                break;
             }
+            // row group done: fold its eight accumulators into this lane's row
+            const float t = transpose_partial(red, lane, acc);
+            if (gi == 0) s0 = t; else if (gi == 1) s1 = t; else s2 = t;
+#pragma unroll
+            for (int r = 0; r < 8; ++r) acc[r] = 0.f;
+            ++gi;
+            x_at = uint32_t(lane) * uint32_t(kXqBytesPerCol);
+            seg = CGf;
+            if (gi == ng) {
+                if (!rem) break;
+                joint = true;
+                lane_on = lane_in;
+                seg = 1;
+                x_at = lane_col * uint32_t(kXqBytesPerCol);
+            }
+            after = behind();
         }
+        have_record = next_unit_here;
         // row scale, tail (Sec. 5.1; four lanes per row share the tail), store
         {
             const Problem P = problems[p];
