@@ -35,6 +35,14 @@ __device__ __forceinline__ int dp4a_su(uint32_t a, uint32_t b, int c) {  // sign
     asm("dp4a.s32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
     return d;
 }
+// c + the low (HIGH: high) two bytes of b . the half words of a, all signed
+template <bool HIGH>
+__device__ __forceinline__ int dp2a(uint32_t a, uint32_t b, int c) {
+    int d;
+    if (HIGH) asm("dp2a.hi.s32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    else asm("dp2a.lo.s32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
 // Loads from the staged tables: they never change after staging, so the loads
 // are not volatile and the compiler may schedule them freely.
 __device__ __forceinline__ uint32_t lds32(uint32_t saddr) {
@@ -254,6 +262,8 @@ __device__ __forceinline__ uint32_t scale_address(const FastBlock& fb) {
 // sum of -y q from the sums of -8 y over the planes of q (high signed, middle, low): every term is a multiple of
 // 8 and |sum y q| <= sqrt(24 * 416) * 2^23 < 2^30, so the int32 is exact.
 __device__ __forceinline__ int combine_planes(int dh, int dm, int dl) { return dh * 8192 + ((dm * 256 + dl) >> 3); }
+// the same from two planes, high signed sixteen bits and low eight
+__device__ __forceinline__ int combine_planes(int dh, int dl) { return dh * 32 + (dl >> 3); }
 
 // ---------------------------------------------------------------------------
 // Activations
@@ -262,7 +272,7 @@ __device__ __forceinline__ int combine_planes(int dh, int dm, int dl) { return d
 // step = 2^(E-22) with 2^E <= max|x| < 2^(E+1); q_j = rint(x_j / step), |q_j| < 2^23,
 // stored as three byte planes (bits 23..16 signed, 15..8 and 7..0 unsigned), four
 // coordinates per 32-bit word in the decoder's order (word_coordinate): words 0..5 high, 6..11 middle, 12..17 low plane;
-// words 18 and 19 = step (float), twice.  A float16 x_j is held exactly when
+// word 18 = step (float), word 19 is spare.  A float16 x_j is held exactly when
 // |x_j| >= 2^(E-12); smaller ones are rounded to a multiple of the step.  If a value
 // is NaN or infinite the step is NaN (and the planes zero).
 // The 24 activations of block column c, as twelve pairs of float16 (zeros beyond K).
@@ -347,7 +357,19 @@ __device__ __forceinline__ void quantise_column(const __half* __restrict__ x, in
         }
     }
     out[18] = __float_as_uint(step);
-    out[19] = out[18];
+    out[19] = 0u;
+}
+// The planned list's record of a column, from that: the upper two planes as sixteen bits, two values to a word (words 2 k
+// and 2 k + 1: the four values of word k), then the low plane, step and spare word as they were.
+__device__ __forceinline__ void pair_planes(uint32_t (&q)[20]) {
+    uint32_t hi[12];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        hi[2 * k] = prmt(q[k], q[6 + k], 0x1504u);
+        hi[2 * k + 1] = prmt(q[k], q[6 + k], 0x3726u);
+    }
+#pragma unroll
+    for (int k = 0; k < 12; ++k) q[k] = hi[k];
 }
 
 }  // namespace tetra

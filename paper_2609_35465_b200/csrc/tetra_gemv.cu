@@ -235,6 +235,7 @@ __global__ void __launch_bounds__(256) k_prepare_x(unsigned char* __restrict__ w
         const Problem P = problems[p];
         uint32_t q[20];
         quantise_column(static_cast<const __half*>(P.x), P.K, gc - col_prefix[p], q);
+        pair_planes(q);
 #pragma unroll
         for (int k = 0; k < 5; ++k) xq[size_t(gc) * 5 + k] = make_uint4(q[4 * k], q[4 * k + 1], q[4 * k + 2], q[4 * k + 3]);
     }
@@ -248,11 +249,11 @@ __global__ void __launch_bounds__(256) k_prepare_x(unsigned char* __restrict__ w
 }
 
 // This lane's activation record (global memory, L1/L2 resident) into registers.
-__device__ __forceinline__ void load_lane_x(const unsigned char* xq_rec, bool active, LaneX& X) {
+__device__ __forceinline__ void load_lane_x(const unsigned char* xq_rec, bool active, LanePairs& X) {
     const uint4* src = reinterpret_cast<const uint4*>(xq_rec);
     const uint4 t0 = __ldg(src), t1 = __ldg(src + 1), t2 = __ldg(src + 2), t3 = __ldg(src + 3), t4 = __ldg(src + 4);
     X.hi[0] = t0.x; X.hi[1] = t0.y; X.hi[2] = t0.z; X.hi[3] = t0.w; X.hi[4] = t1.x; X.hi[5] = t1.y;
-    X.mid[0] = t1.z; X.mid[1] = t1.w; X.mid[2] = t2.x; X.mid[3] = t2.y; X.mid[4] = t2.z; X.mid[5] = t2.w;
+    X.hi[6] = t1.z; X.hi[7] = t1.w; X.hi[8] = t2.x; X.hi[9] = t2.y; X.hi[10] = t2.z; X.hi[11] = t2.w;
     X.lo[0] = t3.x; X.lo[1] = t3.y; X.lo[2] = t3.z; X.lo[3] = t3.w; X.lo[4] = t4.x; X.lo[5] = t4.y;
     X.step = active ? __uint_as_float(t4.z) : 0.f;  // an inactive lane contributes exact zeros
 }
@@ -381,7 +382,7 @@ __device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, uns
             slot = slots - slot;
             // ahead of the next record's copies: the same unit serves both in order, and a load behind a copy waits for
             // memory (Qwen3-8B pass 810 -> 803 us)
-            LaneX X;
+            LanePairs X;
             load_lane_x(xq_p + x_at, lane_on, X);
             x_at += 32 * kXqBytesPerCol;
             // prefetch the next pass's record (or the first one of this warp's next unit)
@@ -392,7 +393,7 @@ __device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, uns
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(slot + 1024), "l"(codes_p + (record + 2 * Bu)));
             }
             asm volatile("cp.async.commit_group;");
-            record_accumulate(sm_tab, a, b, h, X, acc);  // acc is zero when a segment begins
+            record_accumulate<8>(sm_tab, a, b, h, X, acc);  // acc is zero when a segment begins
             if (--seg) continue;
             if (joint) {
                 // lane -> (row group, column); lane l then sums, for row l / 4, the columns
@@ -516,7 +517,7 @@ __device__ __noinline__ void units_fine(unsigned char* __restrict__ ws, unsigned
                 asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(h.x), "=r"(h.y), "=r"(h.z), "=r"(h.w) : "r"(src + 1024));
             }
             const uint32_t col = uint32_t(cg * 32 + lane);
-            LaneX X;
+            LanePairs X;
             load_lane_x(xq_p + min(col, Bu - 1) * uint32_t(kXqBytesPerCol), col < Bu, X);
             if (cg + 1 < c1) {
                 const uint4* next = codes + min(uint32_t((cg + 1) * 32 + lane), Bu - 1);
@@ -527,7 +528,7 @@ __device__ __noinline__ void units_fine(unsigned char* __restrict__ ws, unsigned
             }
             asm volatile("cp.async.commit_group;");
             float v[8];
-            record_values(sm_tab, a, b, h, X, v);
+            record_values<8>(sm_tab, a, b, h, X, v);
 #pragma unroll
             for (int r = 0; r < 8; ++r) acc[r] += v[r];
             parity ^= 1;
