@@ -17,10 +17,11 @@
 //                 k_gemv_units serves a planned list of matrices from one
 //                 persistent grid: k_prepare_x first writes the fixed-point
 //                 activations of every matrix to the plan's scratch area, then
-//                 every warp walks independent units (eight rows of one matrix,
-//                 all columns), so no warp ever waits for another.
+//                 every warp walks its own range of units (up to 24 rows of one
+//                 matrix, all columns), and no warp ever waits for another.
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
@@ -116,47 +117,49 @@ cudaError_t launch_gemv_paper(const void* codes, size_t row_stride, const float*
 // ===========================================================================
 // Workspace written by grouped_plan (host) and read by both kernels:
 //   PlanHeader | Problem[count] | unit_prefix[count + 1] | col_prefix[count + 1]
-//              | warp_start[nwarps + 1] (optional) | pad | xq records
-// A unit is groups_per_unit(B) consecutive row groups of one matrix, all columns.
+//              | WarpCut[ranges + 1] (optional) | col_start[] | pad | counters | partial sums | xq records
+// A unit is groups_per_unit(B) consecutive row groups of one matrix, all columns; a pass is 32 of its columns (or the joint
+// pass over its row groups' last, partial column groups).
 struct PlanHeader {
     int32_t count;
     int32_t total_units;  // sum over matrices of their units
     int32_t total_cols;   // sum over matrices of words per row
-    int32_t nwarps;       // warps the unit ranges were cut for (0: no ranges, units are dealt round-robin)
+    int32_t nwarps;       // warps of the grid that the ranges were cut for (0: no ranges, units are dealt round-robin)
+    int32_t warps_per_cta;  // warps of a CTA that have a range
     uint32_t off_problems, off_unit_prefix, off_col_prefix, off_xq;
-    uint32_t off_warp_start;
-    // fine mode (small lists): a unit is one row group x a slice of the column groups
-    uint32_t off_fine;      // FineInfo[count], 0 in coarse mode
-    uint32_t off_counters;  // int32 per row group: slices of the group that have finished
-    uint32_t off_partials;  // float [row group][slice][8]
-    int32_t total_groups;
-    // coarse mode with unit ranges: units [0, dyn_start) are cut into the warps' ranges; the units from
+    uint32_t off_cuts, off_col_start;
+    uint32_t off_counters;  // int32 per range: pieces that have arrived of the unit cut behind it
+    uint32_t off_partials;  // float [range][2][kPieceFloats]
+    // units [0, dyn_start) are cut into the warps' ranges; the units from
     // dyn_start on are claimed one at a time through dyn_next by warps that have finished their range
     // (k_prepare_x sets dyn_next = dyn_start before every run)
     int32_t dyn_start;
+    int32_t dyn_matrix;  // matrix of unit dyn_start
     int32_t dyn_next;
-    int32_t pad_[1];
 };
-#ifndef TETRA_DYN_PERMILLE
-#define TETRA_DYN_PERMILLE 100
-#endif
-constexpr int kDynamicTailPermille = TETRA_DYN_PERMILLE;  // share of the list's work left for the claimed units
+constexpr int kDynamicTailPermille = 100;  // share of the list's work left for the claimed units
+constexpr int kClaimPasses = 128;          // passes per warp from which on there are claimed units (see grouped_plan)
+// What the ranges are cut by: a pass, and a row group's fold, row scales and tail.  (With two per unit instead of four per row
+// group the warps that have units of one row group, 16 passes each, finished 8 % before those with units of three.)
+constexpr int kPassCost = 8, kFoldCost = 4;
 
-struct FineInfo {
-    int32_t slices;          // column slices per row group
-    int32_t cgs_per_slice;   // column groups per slice (the last slice may hold fewer)
-    int32_t group_prefix;    // row groups of the matrices before this one
-    int32_t partial_prefix;  // floats of partial sums before this matrix
+// Where a warp's range begins; the next entry is where it ends.  A range that begins inside a unit (pass > 0) shares that
+// unit with the ranges before it: `first` is the one in which the unit begins, `pieces` the number of ranges it touches.
+struct WarpCut {
+    int32_t unit, pass, first, pieces;
+    int32_t matrix;  // of the unit
+    int32_t pad_[3];
 };
+constexpr int kColsPerStart = 64;  // col_start names the matrix of every 64th column of the list
+constexpr size_t kSingleCols = 1024;  // columns of a plan that single_plan_fill writes, at most
+constexpr int kPieceFloats = 24;  // row sums of a unit's row groups
 
-constexpr int kMaxPlanWarps = 8192;    // room reserved for warp_start in a planned list's workspace
-constexpr long long kFineMaxTasks = 65536;  // upper bound of the (row group, column group) pairs of a fine-mode list
+constexpr int kMaxPlanWarps = 8192;    // room reserved for the ranges in a planned list's workspace
+constexpr size_t kPiecesBytes = size_t(kMaxPlanWarps) * (4 + 2 * kPieceFloats * 4);  // their counters and partial sums
 
-static inline long long problem_tasks(const Problem& q);
-
-static size_t plan_meta_bytes(int count, int nwarps) {
+static size_t plan_meta_bytes(int count, int nwarps, size_t cols) {
     size_t b = sizeof(PlanHeader) + size_t(count) * sizeof(Problem) + 2 * size_t(count + 1) * 4 +
-               (nwarps ? size_t(nwarps + 1) * 4 : 0) + size_t(count) * sizeof(FineInfo);
+               16 + (nwarps ? size_t(nwarps + 1) * sizeof(WarpCut) : 0) + size_t(cols / kColsPerStart + 1) * 4;
     return (b + 255) & ~size_t(255);
 }
 
@@ -173,29 +176,6 @@ __host__ __device__ inline int groups_per_unit(int B) {
     const int r = 32 / rem;
     return r < 3 ? r : 3;
 }
-static inline long long problem_tasks(const Problem& q) {
-    return (long long)((q.N + 7) / 8) * ((problem_blocks(q) + 31) / 32);
-}
-// Space for the fine mode is reserved for every list of at most kFineMaxTasks (row group, column group)
-// pairs; the plan then takes the fine mode when the list has at most five such pairs per warp of the
-// grid: below that the coarse units leave most warps idle, above it the fine mode's partial sums and
-// counters cost more than they gain.  What the coarse units lose goes with their length and how they
-// happen to divide, so five is a middle.  Fine / coarse, us, on 2368 warps:
-//   pairs per warp 0.3 (2048 x 2304) 7.2 / 6.8; 0.8 (2560 x 4096) 9.2 / 16.4; 1.1 (20000 x 768) 10.9 / 7.6; 1.3 (4096 x
-//   4096) 11.7 / 16.6; 2.0 (q, k, v of an 8B layer) 13.7 / 17.6; 2.9 (nine 2048 x 2304) 18.1 / 13.1; 3.5 (4096 x 12288)
-//   19.5 / 22.3; 3.9 (12288 x 4096) 19.6 / 21.3; 4.1 (gate and up of a 4B layer) 22.0 / 16.4; 4.8 (three 3000 x 7000)
-//   24.9 / 33.7; 5.4 (q, k, v, gate and up of a 4B layer) 26.5 / 20.4; 5.8 (q, k, v and gate of an 8B layer) 27.7 / 22.5;
-//   6.2 (5120 x 17408) 29.4 / 44.7; 7.8 (gate and up of an 8B layer) 32.9 / 21.8; 14.5 (an 8B layer) 44.3 / 35.2.
-static bool list_may_be_fine(const Problem* problems, int count) {
-    long long tasks = 0;
-    for (int i = 0; i < count; ++i) tasks += problem_tasks(problems[i]);
-    return tasks <= kFineMaxTasks;
-}
-static bool list_is_fine(const Problem* problems, int count, int nwarps) {
-    long long tasks = 0;
-    for (int i = 0; i < count; ++i) tasks += problem_tasks(problems[i]);
-    return tasks <= kFineMaxTasks && tasks <= 5LL * (nwarps ? nwarps : 2048);
-}
 static inline int problem_units(const Problem& q) {
     const int R = groups_per_unit(problem_blocks(q));
     return ((q.N + 7) / 8 + R - 1) / R;
@@ -204,53 +184,47 @@ static inline int problem_units(const Problem& q) {
 size_t grouped_workspace_bytes(const Problem* problems, int count) {
     size_t cols = 0;
     for (int i = 0; i < count; ++i) cols += size_t(problem_blocks(problems[i]));
-    size_t bytes = plan_meta_bytes(count, kMaxPlanWarps) + cols * kXqBytesPerCol;
-    if (list_may_be_fine(problems, count)) {  // counters and partial sums of the fine mode
-        long long groups = 0, tasks = 0;
-        for (int i = 0; i < count; ++i) { groups += (problems[i].N + 7) / 8; tasks += problem_tasks(problems[i]); }
-        bytes = ((bytes + 255) & ~size_t(255)) + size_t(groups) * 4 + 256 + size_t(tasks) * 8 * 4;
-    }
-    return bytes;
+    return plan_meta_bytes(count, kMaxPlanWarps, cols) + kPiecesBytes + cols * kXqBytesPerCol;
 }
 
-// Largest p with prefix[p] <= v (prefix[0] = 0, prefix[count] > v).
-__device__ __forceinline__ int find_problem(const int32_t* __restrict__ prefix, int count, int v) {
-    int lo = 0, hi = count;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(prefix + mid) <= v) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
-__global__ void __launch_bounds__(256) k_prepare_x(unsigned char* __restrict__ ws) {
+// One thread per column of the list.  What bounds it is a chain of dependent loads, so all that the plan says about a thread's
+// column is read ahead of the wait, and its matrix is named by the plan instead of searched for (one 8B layer 6 -> 3 us).
+__global__ void __launch_bounds__(128) k_prepare_x(unsigned char* __restrict__ ws) {
     pdl_release();
-    pdl_wait();  // the activations (and the plan) may come from the previous kernel of the stream
     const PlanHeader* H = reinterpret_cast<const PlanHeader*>(ws);
     const Problem* problems = reinterpret_cast<const Problem*>(ws + H->off_problems);
     const int32_t* col_prefix = reinterpret_cast<const int32_t*>(ws + H->off_col_prefix);
+    const int32_t* col_start = reinterpret_cast<const int32_t*>(ws + H->off_col_start);
     uint4* xq = reinterpret_cast<uint4*>(ws + H->off_xq);
-    for (int gc = blockIdx.x * blockDim.x + threadIdx.x; gc < H->total_cols; gc += gridDim.x * blockDim.x) {
-        const int p = find_problem(col_prefix, H->count, gc);
-        const Problem P = problems[p];
+    const int total = H->total_cols, threads = int(gridDim.x * blockDim.x);
+    int gc = blockIdx.x * blockDim.x + threadIdx.x;
+    const __half* x = nullptr;
+    int K = 0, c = 0;
+    auto find = [&] {
+        if (gc >= total) return;
+        int p = __ldg(col_start + gc / kColsPerStart);
+        while (__ldg(col_prefix + p + 1) <= gc) ++p;
+        c = gc - __ldg(col_prefix + p);
+        x = static_cast<const __half*>(problems[p].x);
+        K = problems[p].K;
+    };
+    find();
+    pdl_wait();  // the activations may come from the previous kernel of the stream
+    for (; gc < total; gc += threads, find()) {
         uint32_t q[20];
-        quantise_column(static_cast<const __half*>(P.x), P.K, gc - col_prefix[p], q);
+        quantise_column(x, K, c, q);
         pair_planes(q);
 #pragma unroll
         for (int k = 0; k < 5; ++k) xq[size_t(gc) * 5 + k] = make_uint4(q[4 * k], q[4 * k + 1], q[4 * k + 2], q[4 * k + 3]);
     }
-    if (!H->off_fine && blockIdx.x == 0 && threadIdx.x == 0)
+    if (blockIdx.x == 0 && threadIdx.x == 0)
         reinterpret_cast<PlanHeader*>(ws)->dyn_next = H->dyn_start;  // the claimed units start over
-    if (H->off_fine) {  // fine mode: the per-row-group arrival counters start every run at zero
-        int32_t* counters = reinterpret_cast<int32_t*>(ws + H->off_counters);
-        for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < H->total_groups; g += gridDim.x * blockDim.x)
-            counters[g] = 0;
-    }
+    int32_t* counters = reinterpret_cast<int32_t*>(ws + H->off_counters);  // and so do the arrivals at cut units
+    for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < H->nwarps; w += threads) counters[w] = 0;
 }
 
 // This lane's activation record (global memory, L1/L2 resident) into registers.
-__device__ __forceinline__ void load_lane_x(const unsigned char* xq_rec, bool active, LanePairs& X) {
-    const uint4* src = reinterpret_cast<const uint4*>(xq_rec);
+__device__ __forceinline__ void load_lane_x(const uint4* src, bool active, LanePairs& X) {
     const uint4 t0 = __ldg(src), t1 = __ldg(src + 1), t2 = __ldg(src + 2), t3 = __ldg(src + 3), t4 = __ldg(src + 4);
     X.hi[0] = t0.x; X.hi[1] = t0.y; X.hi[2] = t0.z; X.hi[3] = t0.w; X.hi[4] = t1.x; X.hi[5] = t1.y;
     X.hi[6] = t1.z; X.hi[7] = t1.w; X.hi[8] = t2.x; X.hi[9] = t2.y; X.hi[10] = t2.z; X.hi[11] = t2.w;
@@ -263,44 +237,91 @@ __device__ __forceinline__ void load_lane_x(const unsigned char* xq_rec, bool ac
 #endif
 constexpr int kUnitThreads = TETRA_UNIT_THREADS;
 constexpr int kUnitWarps = kUnitThreads / 32;
+constexpr int kUnitFloats = kRedFloats + 96;  // per warp: the transpose buffer, and a sum per row group and lane
 
-// Coarse mode: every warp walks its range of units (up to three row groups of one matrix, all columns).
-__device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, unsigned char* smem, uint32_t sm_tab) {
+// The persistent kernel of a planned list: every warp walks its range of units (up to three row groups of one matrix, all
+// columns).  All that it needs to know is in the workspace, so a workspace can be copied or moved and still runs correctly:
+// the host needs no record of it.
+__global__ void __launch_bounds__(kUnitThreads, 1)
+k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ ws) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_release();
+    unsigned char* smem = stage_fast_tables(tab, smem_raw);
+    const uint32_t sm_tab = smem_u32(smem);
+    __syncthreads();  // the only CTA-wide barrier: the tables are staged (by cp.async, the plan read meanwhile: 783 instead of
+                      // 773 us for the 8B pass)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float* red = reinterpret_cast<float*>(smem + kFastBytes) + warp * kRedFloats;
+    float* red = reinterpret_cast<float*>(smem + kFastBytes) + warp * kUnitFloats;
+    float* sums = red + kRedFloats + lane;  // of row group gi, row lane / 4: this lane's part at 32 gi
     const PlanHeader* H = reinterpret_cast<const PlanHeader*>(ws);
     const Problem* problems = reinterpret_cast<const Problem*>(ws + H->off_problems);
     const int32_t* unit_prefix = reinterpret_cast<const int32_t*>(ws + H->off_unit_prefix);
     const int32_t* col_prefix = reinterpret_cast<const int32_t*>(ws + H->off_col_prefix);
-    const unsigned char* xq_all = ws + H->off_xq;
     const int total_units = H->total_units;
 
-    // Units of this warp: a contiguous range cut for equal work when the plan holds ranges for this
+    // This warp's share: a contiguous range cut for equal work when the plan holds ranges for this
     // grid (neighbouring warps then walk neighbouring row groups of the same matrices), else every
     // (warps in grid)-th unit.
     const int gw = blockIdx.x * kUnitWarps + warp, nw = gridDim.x * kUnitWarps;
     int u = gw, u_end = total_units, u_step = nw;
     bool claim = false;  // after the range: claim the units from dyn_start on, one at a time
-    if (H->nwarps == nw) {
-        const int32_t* warp_start = reinterpret_cast<const int32_t*>(ws + H->off_warp_start);
-        u = __ldg(warp_start + gw);
-        u_end = __ldg(warp_start + gw + 1);
-        u_step = 1;
-        claim = H->dyn_start < total_units;
-    }
+    int pass0 = 0;       // where in its first unit the range begins
+    const WarpCut* cut = nullptr;
     int p = -1, p_begin = 0, p_end = 0;  // matrix of the current unit and its range of units
     // per matrix, kept in registers across its units (everything else is re-read where it is needed)
     const uint4* codes_p = nullptr;
-    const unsigned char* xq_p = xq_all;
+    uint32_t x_p = 0;                    // its activation records, in 16-byte units from the workspace's first byte
     int G = 1;
     uint32_t Bu = 1;
     bool have_record = false;            // the ring already holds the first record of the unit about to start
+    auto enter_matrix = [&] {
+        p_end = __ldg(unit_prefix + p + 1);
+        p_begin = __ldg(unit_prefix + p);
+        const Problem& Q = problems[p];
+        const int K = Q.K;
+        Bu = uint32_t(Q.tail ? K / 24 : (K + 23) / 24);
+        G = (Q.N + 7) / 8;
+        codes_p = static_cast<const uint4*>(Q.codes);
+        x_p = (H->off_xq >> 4) + uint32_t(__ldg(col_prefix + p)) * uint32_t(kXqBytesPerCol / 16);
+        have_record = false;
+    };
     // Code records reach the decoder through a per-warp ring in shared memory: two slots of 3 x 512
     // bytes (one 16-byte part per lane), filled with cp.async one pass ahead, so the prefetch holds
     // no registers while eight blocks are being decoded.  Each lane reads back only what it copied.
-    const uint32_t ring = sm_tab + uint32_t(kFastBytes) + uint32_t(kUnitWarps * kRedFloats * 4) + uint32_t(warp) * 3072u + uint32_t(lane) * 16u;
+    const uint32_t ring = sm_tab + uint32_t(kFastBytes) + uint32_t(kUnitWarps * kUnitFloats * 4) + uint32_t(warp) * 3072u + uint32_t(lane) * 16u;
     uint32_t slot = ring;                  // of the pass at hand
     const uint32_t slots = 2 * ring + 1536;  // the two slots' sum
+
+    auto request = [&](uint32_t dst, uint32_t at) {  // the three parts of the record at `at`
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst), "l"(codes_p + at));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 512), "l"(codes_p + (at + Bu)));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 1024), "l"(codes_p + (at + 2 * Bu)));
+    };
+    // ahead of the wait: the plan, and the first record of a range that begins in a full column group
+    if (H->nwarps == nw) {
+        const bool has_range = warp < H->warps_per_cta;
+        u = u_end = total_units;
+        u_step = 1;
+        if (has_range) {
+            cut = reinterpret_cast<const WarpCut*>(ws + H->off_cuts) + (blockIdx.x * H->warps_per_cta + warp);
+            u = __ldg(&cut[0].unit);
+            pass0 = __ldg(&cut[0].pass);
+            u_end = __ldg(&cut[1].unit) + (__ldg(&cut[1].pass) > 0);
+            claim = H->dyn_start < total_units;
+            if (u < u_end) {
+                p = __ldg(&cut[0].matrix);
+                enter_matrix();
+                const int R = groups_per_unit(int(Bu)), CGf = int(Bu >> 5), g0 = (u - p_begin) * R;
+                const int gi = CGf ? pass0 / CGf : 0;
+                if (CGf && gi < min(R, G - g0)) {
+                    request(slot, uint32_t(g0 + gi) * 3u * Bu + uint32_t(lane + 32 * (pass0 - gi * CGf)));
+                    have_record = true;
+                }
+            }
+        }
+    }
+    asm volatile("cp.async.commit_group;");
+    pdl_wait();  // the activation records (and zeroed counters) come from k_prepare_x
 
     for (;; u += u_step) {
         if (u >= u_end) {
@@ -315,18 +336,13 @@ __device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, uns
             if (c >= total_units) break;
             u = c;
             u_end = c + 1;
+            if (p < H->dyn_matrix) p_end = 0, p = H->dyn_matrix - 1;
+            cut = nullptr;  // (the last range ends where the first of these units begins)
             have_record = false;
         }
         if (u >= p_end) {  // first unit, or the walk has left the matrix: units only go up
-            do { ++p; p_end = __ldg(unit_prefix + p + 1); } while (u >= p_end);
-            p_begin = __ldg(unit_prefix + p);
-            const Problem& Q = problems[p];
-            const int K = Q.K;
-            Bu = uint32_t(Q.tail ? K / 24 : (K + 23) / 24);
-            G = (Q.N + 7) / 8;
-            codes_p = static_cast<const uint4*>(Q.codes);
-            xq_p = xq_all + size_t(__ldg(col_prefix + p)) * kXqBytesPerCol;
-            have_record = false;
+            do ++p; while (u >= __ldg(unit_prefix + p + 1));
+            enter_matrix();
         }
         const int CGf = int(Bu >> 5);   // full column groups
         const int rem = int(Bu & 31);   // columns of the last, partial one
@@ -341,14 +357,32 @@ __device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, uns
         const uint4* rem_rec = codes0 + size_t(lane_in ? lane_grp : 0) * 3 * Bu + lane_col;
         const bool next_unit_here = CGf > 0 && u + u_step < min(u_end, p_end);
 
+        // the passes of this unit that the range holds: all of them, unless the range begins or ends inside it
+        int left = ng * CGf + (rem > 0);
+        const bool ends_inside = cut && u == __ldg(&cut[1].unit);  // (a range that ends between two units does not reach the second)
+        if (ends_inside) left = __ldg(&cut[1].pass);
+        left -= pass0;
+        bool joint = pass0 >= ng * CGf;
+        int gi = joint ? 0 : pass0 / CGf;
+        const int cg0 = pass0 - gi * CGf;
+        const uint32_t unit0 = uint32_t(g0) * 3u * Bu + uint32_t(lane), unit_rem = uint32_t(rem_rec - codes_p);
+        // places are kept as 16-byte units from the matrix's first record, in 32 bits
+        uint32_t record = joint ? unit_rem : unit0 + uint32_t(gi) * 3u * Bu + 32u * uint32_t(cg0);  // of the pass at hand
+
         if (!have_record) {
-            const uint4* first = CGf > 0 ? codes0 + lane : rem_rec;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(slot), "l"(first));
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(slot + 512), "l"(first + Bu));
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(slot + 1024), "l"(first + 2 * Bu));
+            request(slot, record);
             asm volatile("cp.async.commit_group;");
         }
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f;  // per row group: this lane's partial row sum (row lane / 4)
+        sums[0] = sums[32] = sums[64] = 0.f;
+        {   // row scales and tails of the unit, which its end would wait for (8B pass 781 -> 773 us)
+            const Problem& Q = problems[p];
+            const int row0 = 8 * g0, rows = min(8 * ng, Q.N - row0), ntail = Q.tail ? Q.K % 24 : 0;
+            if (ntail && 128 * lane < 2 * rows * ntail + 127) {
+                const char* at = static_cast<const char*>(Q.tail) + 2 * size_t(row0) * ntail;
+                asm volatile("prefetch.global.L1 [%0];" :: "l"(at + min(128 * lane, 2 * rows * ntail - 1)));
+            }
+            if (lane == 31) asm volatile("prefetch.global.L1 [%0];" :: "l"(Q.row_scales + row0));
+        }
         float acc[8];
 #pragma unroll
         for (int r = 0; r < 8; ++r) acc[r] = 0.f;
@@ -356,18 +390,14 @@ __device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, uns
         // One pass = one 48-byte record per lane: the full column groups of each row group in turn, then the joint pass over
         // the partial column group (a single call site of the decoder).  A segment is a row group's full column groups, or
         // the joint pass: inside one, records and activations follow at fixed distances.
-        int gi = 0;
-        bool joint = CGf == 0, lane_on = !joint || lane_in;
-        int seg = joint ? 1 : CGf;                                         // passes left in the segment
-        // places are kept as 16-byte units from the matrix's first record, in 32 bits
-        const uint32_t unit0 = uint32_t(g0) * 3u * Bu + uint32_t(lane), unit_rem = uint32_t(rem_rec - codes_p);
-        uint32_t record = joint ? unit_rem : unit0;                        // of the pass at hand
-        uint32_t x_at = (joint ? lane_col : uint32_t(lane)) * uint32_t(kXqBytesPerCol);
+        bool lane_on = !joint || lane_in;
+        int seg = joint ? 1 : min(CGf - cg0, left);                        // passes left in the segment
+        left -= seg;                                                       // and behind it
+        uint32_t x_at = x_p + (joint ? lane_col : uint32_t(lane + 32 * cg0)) * uint32_t(kXqBytesPerCol / 16);
         // the first record behind the segment: the next row group's, the joint pass's, the next unit's
         constexpr uint32_t kNone = 0xFFFFFFFFu;
         auto behind = [&]() -> uint32_t {
-            if (!joint && gi + 1 < ng) return unit0 + uint32_t(gi + 1) * 3u * Bu;
-            if (!joint && rem) return unit_rem;
+            if (left) return gi + 1 < ng ? unit0 + uint32_t(gi + 1) * 3u * Bu : unit_rem;
             return next_unit_here ? unit0 + uint32_t(u_step * R) * 3u * Bu : kNone;
         };
         uint32_t after = behind();
@@ -383,15 +413,11 @@ __device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, uns
             // ahead of the next record's copies: the same unit serves both in order, and a load behind a copy waits for
             // memory (Qwen3-8B pass 810 -> 803 us)
             LanePairs X;
-            load_lane_x(xq_p + x_at, lane_on, X);
-            x_at += 32 * kXqBytesPerCol;
+            load_lane_x(reinterpret_cast<const uint4*>(ws) + x_at, lane_on, X);
+            x_at += 32 * kXqBytesPerCol / 16;
             // prefetch the next pass's record (or the first one of this warp's next unit)
             record = seg == 1 ? after : record + 32u;
-            if (record != kNone) {
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(slot), "l"(codes_p + record));
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(slot + 512), "l"(codes_p + (record + Bu)));
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(slot + 1024), "l"(codes_p + (record + 2 * Bu)));
-            }
+            if (record != kNone) request(slot, record);
             asm volatile("cp.async.commit_group;");
             record_accumulate<8>(sm_tab, a, b, h, X, acc);  // acc is zero when a segment begins
             if (--seg) continue;
@@ -403,31 +429,69 @@ __device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, uns
                 for (int r = 0; r < 8; ++r) red[r * kRedStride + lane] = acc[r];
                 __syncwarp();
                 const float* rr = red + (lane >> 2) * kRedStride;
+                float s0 = sums[0], s1 = sums[32], s2 = sums[64];
                 for (int k = lane & 3; k < rem; k += 4) {
                     s0 += rr[k];
                     if (R > 1) s1 += rr[rem + k];
                     if (R > 2) s2 += rr[2 * rem + k];
                 }
+                sums[0] = s0;
+                sums[32] = s1;
+                sums[64] = s2;
                 break;
             }
             // row group done: fold its eight accumulators into this lane's row
-            const float t = transpose_partial(red, lane, acc);
-            if (gi == 0) s0 = t; else if (gi == 1) s1 = t; else s2 = t;
+            sums[32 * gi] = transpose_partial(red, lane, acc);
 #pragma unroll
             for (int r = 0; r < 8; ++r) acc[r] = 0.f;
+            if (!left) break;
             ++gi;
-            x_at = uint32_t(lane) * uint32_t(kXqBytesPerCol);
-            seg = CGf;
+            x_at = x_p + uint32_t(lane) * uint32_t(kXqBytesPerCol / 16);
+            seg = min(CGf, left);
             if (gi == ng) {
-                if (!rem) break;
                 joint = true;
                 lane_on = lane_in;
                 seg = 1;
-                x_at = lane_col * uint32_t(kXqBytesPerCol);
+                x_at = x_p + lane_col * uint32_t(kXqBytesPerCol / 16);
             }
+            left -= seg;
             after = behind();
         }
         have_record = next_unit_here;
+        // A unit that other ranges share: this range's piece goes to the workspace, and the last piece to arrive finds the
+        // others there (a counter, nothing waits on it) and adds them in the ranges' order.
+        const WarpCut* shared = pass0 ? cut : (ends_inside ? cut + 1 : nullptr);
+        pass0 = 0;
+        if (shared) {
+            const int first = __ldg(&shared->first), pieces = __ldg(&shared->pieces);
+            const int range = blockIdx.x * H->warps_per_cta + warp;
+            float* partials = reinterpret_cast<float*>(ws + H->off_partials);
+            // a range's piece of the unit that it ends in lies behind its piece of the unit that it begins in
+            float* mine = partials + size_t(2 * range + (range == first)) * kPieceFloats + (lane >> 2);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                float v = sums[32 * k];
+                v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
+                v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
+                if ((lane & 3) == 0) __stcg(mine + 8 * k, v);
+            }
+            __threadfence();
+            __syncwarp();
+            int arrived = 0;
+            if (lane == 0) arrived = atomicAdd(reinterpret_cast<int32_t*>(ws + H->off_counters) + first, 1);
+            if (__shfl_sync(0xFFFFFFFFu, arrived, 0) != pieces - 1) continue;
+            __threadfence();
+            float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+            for (int k = lane & 3; k < pieces; k += 4) {
+                const float* theirs = partials + size_t(2 * (first + k) + (k == 0)) * kPieceFloats + (lane >> 2);
+                s0 += __ldcg(theirs);
+                s1 += __ldcg(theirs + 8);
+                s2 += __ldcg(theirs + 16);
+            }
+            sums[0] = s0;
+            sums[32] = s1;
+            sums[64] = s2;
+        }
         // row scale, tail (Sec. 5.1; four lanes per row share the tail), store
         {
             const Problem P = problems[p];
@@ -435,7 +499,7 @@ __device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, uns
             const __half* xh = static_cast<const __half*>(P.x) + 24 * Bu;
             for (int gk = 0; gk < ng; ++gk) {
                 const int row = (g0 + gk) * 8 + (lane >> 2);
-                float sum = gk == 0 ? s0 : (gk == 1 ? s1 : s2);
+                float sum = sums[32 * gk];
                 if (row < P.N) {
                     sum *= __ldg(P.row_scales + row);
                     const __half* tl = static_cast<const __half*>(P.tail) + size_t(row) * ntail;
@@ -450,187 +514,41 @@ __device__ __forceinline__ void units_coarse(unsigned char* __restrict__ ws, uns
     }
 }
 
-// Fine mode of the planned list, for lists too small to fill the GPU with coarse units (single
-// matrices, the matrices of one layer): a unit is one row group x a slice of the column groups.
-// Each unit leaves eight partial row sums in the scratch area and bumps its row group's counter; the
-// unit that finds all the other slices done adds them up in slice order (fixed order, no waiting,
-// no floating-point atomics), applies the row scale and the tail, and stores.
-__device__ __noinline__ void units_fine(unsigned char* __restrict__ ws, unsigned char* smem, uint32_t sm_tab) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float* red = reinterpret_cast<float*>(smem + kFastBytes) + warp * kRedFloats;
-    const PlanHeader* H = reinterpret_cast<const PlanHeader*>(ws);
-    const Problem* problems = reinterpret_cast<const Problem*>(ws + H->off_problems);
-    const int32_t* unit_prefix = reinterpret_cast<const int32_t*>(ws + H->off_unit_prefix);
-    const int32_t* col_prefix = reinterpret_cast<const int32_t*>(ws + H->off_col_prefix);
-    const FineInfo* fine = reinterpret_cast<const FineInfo*>(ws + H->off_fine);
-    int32_t* counters = reinterpret_cast<int32_t*>(ws + H->off_counters);
-    float* partials = reinterpret_cast<float*>(ws + H->off_partials);
-    const unsigned char* xq_all = ws + H->off_xq;
-    const int total_units = H->total_units;
-    const uint32_t ring = sm_tab + uint32_t(kFastBytes) + uint32_t(kUnitWarps * kRedFloats * 4) +
-                          uint32_t(warp) * 3072u + uint32_t(lane) * 16u;
-
-    // equal shares of consecutive units per warp (units of a list in fine mode are of similar size)
-    const int gw = blockIdx.x * kUnitWarps + warp, nw = gridDim.x * kUnitWarps;
-    int u = int((long long)total_units * gw / nw);
-    const int u_end = int((long long)total_units * (gw + 1) / nw);
-    int p = -1, p_begin = 0, p_end = 0;
-    Problem P{};
-    FineInfo F{};
-    int CG = 1;
-    uint32_t Bu = 1;
-    const unsigned char* xq_p = xq_all;
-
-    for (; u < u_end; ++u) {
-        if (u >= p_end) {
-            do { ++p; p_end = __ldg(unit_prefix + p + 1); } while (u >= p_end);
-            p_begin = __ldg(unit_prefix + p);
-            P = problems[p];
-            F = fine[p];
-            Bu = uint32_t(P.tail ? P.K / 24 : (P.K + 23) / 24);
-            CG = int((Bu + 31) >> 5);
-            xq_p = xq_all + size_t(__ldg(col_prefix + p)) * kXqBytesPerCol;
-        }
-        const int local = u - p_begin;
-        const int g = local / F.slices, slice = local - g * F.slices;
-        const int c0 = slice * F.cgs_per_slice, c1 = min(CG, c0 + F.cgs_per_slice);
-        const uint4* codes = static_cast<const uint4*>(P.codes) + size_t(g) * 3 * Bu;
-
-        float acc[8];
-#pragma unroll
-        for (int r = 0; r < 8; ++r) acc[r] = 0.f;
-        {   // first record of the unit into ring slot 0
-            const uint4* first = codes + min(uint32_t(c0 * 32 + lane), Bu - 1);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(ring), "l"(first));
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(ring + 512), "l"(first + Bu));
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(ring + 1024), "l"(first + 2 * Bu));
-            asm volatile("cp.async.commit_group;");
-        }
-        int parity = 0;
-        for (int cg = c0; cg < c1; ++cg) {
-            uint4 a, b, h;
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-            {
-                const uint32_t src = ring + uint32_t(parity * 1536);
-                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w) : "r"(src));
-                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "r"(src + 512));
-                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(h.x), "=r"(h.y), "=r"(h.z), "=r"(h.w) : "r"(src + 1024));
-            }
-            const uint32_t col = uint32_t(cg * 32 + lane);
-            LanePairs X;
-            load_lane_x(xq_p + min(col, Bu - 1) * uint32_t(kXqBytesPerCol), col < Bu, X);
-            if (cg + 1 < c1) {
-                const uint4* next = codes + min(uint32_t((cg + 1) * 32 + lane), Bu - 1);
-                const uint32_t dst = ring + uint32_t((parity ^ 1) * 1536);
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst), "l"(next));
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 512), "l"(next + Bu));
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 1024), "l"(next + 2 * Bu));
-            }
-            asm volatile("cp.async.commit_group;");
-            float v[8];
-            record_values<8>(sm_tab, a, b, h, X, v);
-#pragma unroll
-            for (int r = 0; r < 8; ++r) acc[r] += v[r];
-            parity ^= 1;
-        }
-        float sum = transpose_partial(red, lane, acc);
-        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
-        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 2);
-        float* mine = partials + F.partial_prefix + (size_t(g) * F.slices + slice) * 8;
-        if ((lane & 3) == 0) mine[lane >> 2] = sum;
-        __threadfence();   // the partial sums are visible before the counter moves
-        __syncwarp();
-        int arrived = 0;
-        if (lane == 0) arrived = atomicAdd(counters + F.group_prefix + g, 1);
-        arrived = __shfl_sync(0xFFFFFFFFu, arrived, 0);
-        if (arrived == F.slices - 1) {  // every slice of this row group is in: finish the rows
-            __threadfence();
-            const int row = g * 8 + lane;
-            if (lane < 8 && row < P.N) {
-                const float* all = partials + F.partial_prefix + size_t(g) * F.slices * 8 + lane;
-                float total = 0.f;
-                for (int k = 0; k < F.slices; ++k) total += __ldcg(all + 8 * k);
-                float res = __ldg(P.row_scales + row) * total;
-                const int ntail = P.tail ? P.K % 24 : 0;
-                const __half* xh = static_cast<const __half*>(P.x) + 24 * Bu;
-                const __half* tl = static_cast<const __half*>(P.tail) + size_t(row) * ntail;
-                for (int k = 0; k < ntail; ++k) res = fmaf(__half2float(tl[k]), __half2float(xh[k]), res);
-                P.y[row] = res;
-            }
-        }
-    }
-}
-
-// The persistent kernel of a planned list.  The plan in the workspace says which of the two modes it
-// was cut for (PlanHeader::off_fine), so a workspace can be copied or moved and still runs correctly:
-// the host needs no record of it.
-__global__ void __launch_bounds__(kUnitThreads, 1)
-k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ ws) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    pdl_release();
-    unsigned char* smem = stage_fast_tables(tab, smem_raw);
-    const uint32_t sm_tab = smem_u32(smem);
-    __syncthreads();  // the only CTA-wide barrier: tables are staged
-    pdl_wait();       // the plan's activation records (and zeroed counters) come from k_prepare_x
-    if (reinterpret_cast<const PlanHeader*>(ws)->off_fine) units_fine(ws, smem, sm_tab);
-    else units_coarse(ws, smem, sm_tab);
-}
-
-
-cudaError_t grouped_plan(const Problem* problems_host, int count, void* ws_dev, size_t ws_bytes, cudaStream_t s) {
-    if (ws_bytes < grouped_workspace_bytes(problems_host, count)) return cudaErrorInvalidValue;
+cudaError_t grouped_plan(const Problem* problems, int count, void* ws_dev, size_t ws_bytes, cudaStream_t s) {
+    if (ws_bytes < grouped_workspace_bytes(problems, count)) return cudaErrorInvalidValue;
     int sms = 0;
     cudaError_t e = device_sms(&sms);
     if (e != cudaSuccess) return e;
     int nwarps = sms * kUnitWarps;  // the grid grouped_run launches on this device
     if (nwarps > kMaxPlanWarps) nwarps = 0;
-    const size_t meta = plan_meta_bytes(count, nwarps);
+    size_t all_cols = 0;
+    for (int i = 0; i < count; ++i) all_cols += size_t(problem_blocks(problems[i]));
+    const size_t meta = plan_meta_bytes(count, nwarps, all_cols);
     unsigned char* buf = static_cast<unsigned char*>(calloc(1, meta));
     if (!buf) return cudaErrorMemoryAllocation;
     PlanHeader* H = reinterpret_cast<PlanHeader*>(buf);
     H->count = count;
     H->nwarps = nwarps;
+    // Matrices whose units are longest come first, so that the units claimed at the end are short (14B, 6 / 16 / 36 layers
+    // 260 / 637 / 1394 -> 242 / 620 / 1375 us; results do not depend on the order).
+    Problem* problems_host = reinterpret_cast<Problem*>(buf + sizeof(PlanHeader));
+    auto longest = [](const Problem& q) {
+        const int Bi = problem_blocks(q);
+        return groups_per_unit(Bi) * (Bi / 32) + (Bi % 32 ? 1 : 0);
+    };
+    memcpy(problems_host, problems, size_t(count) * sizeof(Problem));
+    std::stable_sort(problems_host, problems_host + count, [&](const Problem& a, const Problem& b) { return longest(a) > longest(b); });
     H->off_problems = uint32_t(sizeof(PlanHeader));
     H->off_unit_prefix = H->off_problems + uint32_t(count) * uint32_t(sizeof(Problem));
     H->off_col_prefix = H->off_unit_prefix + uint32_t(count + 1) * 4u;
-    H->off_warp_start = H->off_col_prefix + uint32_t(count + 1) * 4u;
-    H->off_xq = uint32_t(plan_meta_bytes(count, kMaxPlanWarps));
-    memcpy(buf + H->off_problems, problems_host, size_t(count) * sizeof(Problem));
+    H->off_cuts = (H->off_col_prefix + uint32_t(count + 1) * 4u + 15u) & ~15u;
+    H->off_col_start = H->off_cuts + uint32_t(nwarps ? (nwarps + 1) * sizeof(WarpCut) : 0);
+    H->off_counters = uint32_t(plan_meta_bytes(count, kMaxPlanWarps, all_cols));
+    H->off_partials = H->off_counters + uint32_t(kMaxPlanWarps) * 4u;
+    H->off_xq = H->off_counters + uint32_t(kPiecesBytes);
     int32_t* up = reinterpret_cast<int32_t*>(buf + H->off_unit_prefix);
     int32_t* cp = reinterpret_cast<int32_t*>(buf + H->off_col_prefix);
-    const bool fine_mode = list_is_fine(problems_host, count, nwarps);
     long long units = 0, cols = 0;
-    if (fine_mode) {
-        // column groups per unit: aim at about four units per warp of the grid
-        long long tasks = 0, groups = 0;
-        for (int i = 0; i < count; ++i) { tasks += problem_tasks(problems_host[i]); groups += (problems_host[i].N + 7) / 8; }
-        const long long want = 4LL * (nwarps ? nwarps : 2048);
-        long long per = tasks / want;
-        if (per < 1) per = 1;
-        H->off_fine = H->off_col_prefix + uint32_t(count + 1) * 4u + (nwarps ? uint32_t(nwarps + 1) * 4u : 0u);
-        FineInfo* fi = reinterpret_cast<FineInfo*>(buf + H->off_fine);
-        size_t xq_end = size_t(H->off_xq);
-        for (int i = 0; i < count; ++i) xq_end += size_t(problem_blocks(problems_host[i])) * kXqBytesPerCol;
-        xq_end = (xq_end + 255) & ~size_t(255);
-        H->off_counters = uint32_t(xq_end);
-        H->off_partials = uint32_t((xq_end + size_t(groups) * 4 + 255) & ~size_t(255));
-        H->total_groups = int32_t(groups);
-        long long gp = 0, pp = 0;
-        for (int i = 0; i < count; ++i) {
-            const int CGi = (problem_blocks(problems_host[i]) + 31) / 32, Gi = (problems_host[i].N + 7) / 8;
-            const int cps = int(per < CGi ? per : CGi);
-            const int slices = (CGi + cps - 1) / cps;
-            fi[i] = FineInfo{slices, cps, int32_t(gp), int32_t(pp)};
-            up[i] = int32_t(units);
-            cp[i] = int32_t(cols);
-            units += (long long)Gi * slices;
-            cols += problem_blocks(problems_host[i]);
-            gp += Gi;
-            pp += (long long)Gi * slices * 8;
-        }
-        nwarps = 0;  // the fine kernel cuts equal shares itself
-        H->nwarps = 0;
-    } else
     for (int i = 0; i < count; ++i) {
         up[i] = int32_t(units);
         cp[i] = int32_t(cols);
@@ -642,50 +560,97 @@ cudaError_t grouped_plan(const Problem* problems_host, int count, void* ws_dev, 
     if (units > 0x7FFFFFF0LL || cols > 0x7FFFFFF0LL) e = cudaErrorInvalidValue;
     H->total_units = int32_t(units);
     H->total_cols = int32_t(cols);
+    if (e == cudaSuccess) {
+        int32_t* start = reinterpret_cast<int32_t*>(buf + H->off_col_start);
+        int i = 0;
+        for (long long c = 0; c < cols; c += kColsPerStart) {
+            while (cp[i + 1] <= c) ++i;
+            start[c / kColsPerStart] = i;
+        }
+    }
+    H->dyn_start = int32_t(units);
     if (e == cudaSuccess && nwarps) {
-        // Cut the unit sequence into nwarps contiguous ranges of equal work; a unit costs its number of
-        // column groups plus a little for its prologue and epilogue.
-        auto unit_work = [&](int i) {
-            const int Bi = problem_blocks(problems_host[i]);
-            return (long long)(groups_per_unit(Bi) * (Bi / 32) + (Bi % 32 ? 1 : 0)) * 8 + 2;
+        // Cut the sequence of passes into contiguous ranges of equal work.  A cut inside a unit costs its two sides a store of
+        // sums and an atomic, two of each per warp and run; cut between units only, a list of a few layers leaves most warps
+        // waiting for those with one unit more (4B, one / two / six layers 28.9 / 40.9 / 92.6 us, cut inside units
+        // 24.8 / 39.0 / 87.3; 14B, one layer 59.2 and 51.4).
+        auto unit_passes = [&](int i, long long k) {
+            const int Bi = problem_blocks(problems_host[i]), G = (problems_host[i].N + 7) / 8, R = groups_per_unit(Bi);
+            const int ng = int(G - k * R < R ? G - k * R : R);
+            return ng * (Bi / 32) + (Bi % 32 ? 1 : 0);
         };
-        long long total = 0;
-        for (int i = 0; i < count; ++i) total += unit_work(i) * problem_units(problems_host[i]);
-        // The last tenth of the work is not assigned: warps that finish early claim it unit by unit, which
-        // evens out what the cost model and the SMs' unequal speeds leave.  Nothing / 5 % / a tenth / a fifth
-        // claimed: Qwen3-8B pass 836 / 827 / 802 / 804 us, 16 layers of it 387 / 374 / 368 / 369, Qwen3-14B pass
-        // 1522 / 1477 / 1425 / 1439.  Only when a warp has at least eight units: with fewer, a unit claimed last
-        // is too large a share of a warp's work (two layers of the 4B model 45.5 us without, 50.2 with a tenth;
-        // one of the 14B 68.0 / 78.1; but eight of the 8B 204 / 199).  Beyond the line it can still cost: 14B,
-        // whose units are single row groups, four layers 178 without, 191 with; sixteen 647 / 648.
-        H->dyn_start = int32_t(units);
-        if (units >= 8LL * nwarps) {
+        auto unit_cost = [&](int i, long long k) {
+            const int G = (problems_host[i].N + 7) / 8, R = groups_per_unit(problem_blocks(problems_host[i]));
+            return (long long)unit_passes(i, k) * kPassCost + kFoldCost * int(G - k * R < R ? G - k * R : R);
+        };
+        auto full_work = [&](int i) { return unit_cost(i, 0); };      // of all units but the last
+        auto matrix_work = [&](int i) {
+            const long long U = problem_units(problems_host[i]);
+            return (U - 1) * full_work(i) + unit_cost(i, U - 1);
+        };
+        long long total = 0, passes = 0;
+        for (int i = 0; i < count; ++i) {
+            const long long U = problem_units(problems_host[i]);
+            total += matrix_work(i);
+            passes += (U - 1) * unit_passes(i, 0) + unit_passes(i, U - 1);
+        }
+        // Of a long list the last tenth of the work is not assigned: warps that finish early claim it unit by unit, which
+        // evens out what the cost model and the warps' unequal speeds leave.  A unit claimed last still makes the others wait
+        // for it, which shorter lists do not make up for.  All assigned / a tenth claimed, us: 8B, 8 / 12 / 16 / 36 layers
+        // 187 / 274 / 360 / 791 and 191 / 269 / 355 / 772; 4B, 10 / 16 / 36 135 / 208 / 451 and 136 / 205 / 434; 14B, 4 /
+        // 36 layers 167 / 1436 and 168 / 1375 (7 passes per warp are a layer of the 4B model, 13 of the 8B, 24 of the 14B).
+        // 6 % claimed: 8B, 36 layers 785; 15 % 777.  Units claimed while the one before is at work, so that its first record
+        // is not waited for: 779 (a warp then holds one more unit at the end); two or three short units at a time: 14B 1410.
+        const bool claimed = passes >= (long long)kClaimPasses * nwarps;
+        if (claimed) {
             const long long planned = total - total * kDynamicTailPermille / 1000;
             long long acc = 0;
             int i = 0;
-            while (i < count - 1 && acc + unit_work(i) * problem_units(problems_host[i]) <= planned) {
-                acc += unit_work(i) * problem_units(problems_host[i]);
-                ++i;
-            }
-            long long ds = up[i] + (planned - acc) / unit_work(i);
+            while (i < count - 1 && acc + matrix_work(i) <= planned) acc += matrix_work(i++);
+            long long ds = up[i] + (planned - acc) / full_work(i);
             if (ds > units) ds = units;
             H->dyn_start = int32_t(ds);
-            total = acc + (ds - up[i]) * unit_work(i);
+            total = acc + (ds - up[i]) * full_work(i);
         }
-        int32_t* wsx = reinterpret_cast<int32_t*>(buf + H->off_warp_start);
+        long long per = (passes + sms - 1) / sms;  // warps of a CTA that have a range: no more than passes
+        if (per > kUnitWarps) per = kUnitWarps;
+        H->warps_per_cta = int32_t(per);
+        const int ranges = int(per) * sms;
+        WarpCut* cuts = reinterpret_cast<WarpCut*>(buf + H->off_cuts);
         int pi = 0;
         long long before = 0;  // work of matrices 0..pi-1
-        for (int w = 0; w < nwarps; ++w) {
-            const long long target = total * w / nwarps;
-            while (pi < count - 1 && before + unit_work(pi) * problem_units(problems_host[pi]) <= target) {
-                before += unit_work(pi) * problem_units(problems_host[pi]);
-                ++pi;
+        for (int w = 0; w < ranges; ++w) {
+            const long long target = total * w / ranges;
+            while (pi < count - 1 && before + matrix_work(pi) <= target) before += matrix_work(pi++);
+            const long long k = (target - before) / full_work(pi);
+            long long uu = up[pi] + k, pass = (target - before - k * full_work(pi)) / kPassCost;
+            if (pass >= unit_passes(pi, k)) { pass = 0; ++uu; }
+            if (w && (uu < cuts[w - 1].unit || (uu == cuts[w - 1].unit && pass <= cuts[w - 1].pass && cuts[w - 1].pass))) {
+                // fewer passes than ranges: one pass behind the range before
+                uu = cuts[w - 1].unit;
+                pass = cuts[w - 1].pass + 1;
+                int pj = 0;
+                while (pj < count - 1 && up[pj + 1] <= uu) ++pj;
+                if (uu >= units || pass >= unit_passes(pj, uu - up[pj])) { ++uu; pass = 0; }
             }
-            long long uu = up[pi] + (target - before) / unit_work(pi);
-            if (uu > H->dyn_start) uu = H->dyn_start;
-            wsx[w] = int32_t(uu);
+            if (uu >= H->dyn_start) { uu = H->dyn_start; pass = 0; }
+            int pj = pi;  // (a cut may have moved on from the matrix that its target lies in, or back from it)
+            while (pj > 0 && up[pj] > uu) --pj;
+            while (pj < count - 1 && up[pj + 1] <= uu) ++pj;
+            cuts[w] = WarpCut{int32_t(uu), int32_t(pass), w, 1, pj, {0, 0, 0}};
         }
-        wsx[nwarps] = H->dyn_start;
+        int pj = 0;
+        while (pj < count - 1 && up[pj + 1] <= H->dyn_start) ++pj;
+        H->dyn_matrix = pj;
+        cuts[ranges] = WarpCut{H->dyn_start, 0, ranges, 1, pj, {0, 0, 0}};
+        // who shares a cut unit: the range before the first that begins inside it, and all that begin inside it
+        for (int w = 1; w < ranges; ++w) {
+            if (!cuts[w].pass) continue;
+            int last = w;
+            while (last + 1 < ranges && cuts[last + 1].unit == cuts[w].unit) ++last;
+            for (int v = w; v <= last; ++v) { cuts[v].first = w - 1; cuts[v].pieces = last - w + 2; }
+            w = last;
+        }
     }
     // pageable source: the runtime stages it before returning, so the buffer can be freed
     if (e == cudaSuccess) e = cudaMemcpyAsync(ws_dev, buf, meta, cudaMemcpyHostToDevice, s);
@@ -693,14 +658,14 @@ cudaError_t grouped_plan(const Problem* problems_host, int count, void* ws_dev, 
     return e;
 }
 
-size_t single_plan_meta_bytes() { return plan_meta_bytes(1, 0); }
+size_t single_plan_meta_bytes() { return plan_meta_bytes(1, 0, kSingleCols); }
 
 size_t single_plan_scratch_bytes(int blocks_per_row) {
-    return plan_meta_bytes(1, 0) + size_t(blocks_per_row) * kXqBytesPerCol;
+    return plan_meta_bytes(1, 0, kSingleCols) + size_t(blocks_per_row) * kXqBytesPerCol;
 }
 
 void single_plan_fill(const Problem& problem, unsigned char* meta_host) {
-    memset(meta_host, 0, plan_meta_bytes(1, 0));
+    memset(meta_host, 0, plan_meta_bytes(1, 0, kSingleCols));
     PlanHeader* H = reinterpret_cast<PlanHeader*>(meta_host);
     H->count = 1;
     H->total_units = problem_units(problem);
@@ -709,23 +674,25 @@ void single_plan_fill(const Problem& problem, unsigned char* meta_host) {
     H->nwarps = 0;  // no unit ranges: the kernel deals units round-robin
     H->off_unit_prefix = H->off_problems + uint32_t(sizeof(Problem));
     H->off_col_prefix = H->off_unit_prefix + 8u;
-    H->off_xq = uint32_t(plan_meta_bytes(1, 0));
+    H->off_xq = uint32_t(plan_meta_bytes(1, 0, kSingleCols));
     memcpy(meta_host + H->off_problems, &problem, sizeof(Problem));
     int32_t* up = reinterpret_cast<int32_t*>(meta_host + H->off_unit_prefix);
     int32_t* cp = reinterpret_cast<int32_t*>(meta_host + H->off_col_prefix);
     up[0] = 0; up[1] = H->total_units;
     cp[0] = 0; cp[1] = H->total_cols;
+    H->off_col_start = H->off_col_prefix + 8u;  // all zeros: one matrix
+    H->dyn_start = H->total_units;
 }
 
 cudaError_t grouped_run(void* ws_dev, const void* table, cudaStream_t s) {
     int sms = 0;
     cudaError_t e = device_sms(&sms);
     if (e != cudaSuccess) return e;
-    const uint32_t smem = kTableSmemBytes + kUnitWarps * kRedFloats * 4 + kUnitWarps * 3072;
+    const uint32_t smem = kTableSmemBytes + kUnitWarps * kUnitFloats * 4 + kUnitWarps * 3072;
     static PerDeviceOnce once;
     e = once.run([smem] { return cudaFuncSetAttribute(k_gemv_units, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)); });
     if (e != cudaSuccess) return e;
-    e = launch_pdl(k_prepare_x, sms * 2, 256, 0, s, static_cast<unsigned char*>(ws_dev));
+    e = launch_pdl(k_prepare_x, sms * 4, 128, 0, s, static_cast<unsigned char*>(ws_dev));
     if (e != cudaSuccess) return e;
     return launch_pdl(k_gemv_units, sms, kUnitThreads, smem, s, static_cast<const DeviceTables*>(table),
                       static_cast<unsigned char*>(ws_dev));

@@ -204,3 +204,28 @@ def test_encode_block_counts(tt, table, n):
     codes, cos = tt.tetra_encode_blocks(w[445 - n:].contiguous(), table)
     torch.cuda.synchronize()
     assert torch.equal(codes, all_codes[445 - n:]) and torch.equal(cos, all_cos[445 - n:])
+
+
+# Planned lists are cut into the warps' ranges by passes (32 columns of a row group): one unit shared by many ranges, fewer
+# passes than CTAs and than warps, joint passes over three row groups' last columns on either side of a cut, a last unit with
+# fewer row groups, units of one pass, several matrices in a range, the plan's order against the caller's.
+@pytest.mark.parametrize("mats", [
+    [(8, 24 * 32 * 63, True)], [(8, 24 * 32 * 40, True), (1, 24, True)], [(24, 24 * 42, True)], [(200, 24 * (32 * 5 + 10), True)],
+    [(17, 24 * 37, True), (1, 24 * 33, False), (8 * 148, 24 * 32, True)], [(8 * 2368 + 9, 24 * 5, True)],
+    [(3000, 24 * 42, True), (40, 24 * 700 + 7, True), (3001, 24 * 32, True)], [(1, 24 * 3, True)] * 40,
+    [(8 * 300, 24 * 32 * 9, True), (16 * 75 + 3, 24 * (32 * 9 + 11) + 5, True)],
+])
+def test_planned_list_ranges(tt, table, orc, mats):
+    ms = [make_matrix(83, 1000 * i + N, N, K, tail, batch=1) for i, (N, K, tail) in enumerate(mats)]
+    items = [device_matrix(tt, table, m, torch.from_numpy(m["x"][0]).cuda()) for m in ms]
+    problems = tt.make_problems(items)
+    ws = torch.full((tt.tetra_grouped_workspace_bytes(problems),), 0xA5, dtype=torch.uint8, device="cuda")
+    tt.tetra_gemv_grouped(problems, table, ws)
+    first = [it["y"].clone() for it in items]
+    for it in items:
+        it["y"].fill_(float("nan"))
+    tt.tetra_gemv_grouped_run(ws, table)
+    torch.cuda.synchronize()
+    for m, it, y in zip(ms, items, first):
+        assert torch.equal(it["y"], y)
+        check(orc, m, y.cpu().numpy(), "%d x %d of %d" % (m["N"], m["K"], len(ms)))
