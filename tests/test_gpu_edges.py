@@ -54,6 +54,13 @@ def test_single_matrix(tt, table, orc, N, K, tail_mode):
     check(orc, m, d["y"].cpu().numpy(), "%d x %d" % (N, K))
 
 
+# The activations' image by sections or by columns: on both sides of a section per thread and of a column per thread.
+@pytest.mark.parametrize("N,K,tail_mode", [(9, 24 * 170 + 7, True), (9, 24 * 170 + 7, False), (9, 24 * 171, True), (33, 24 * 512 + 3, True),
+                                           (33, 24 * 512 + 3, False), (8, 24 * 1024 + 1, True)])
+def test_image_by_columns(tt, table, orc, N, K, tail_mode):
+    test_single_matrix(tt, table, orc, N, K, tail_mode)
+
+
 # A CTA works on one matrix: lists of very unequal matrices, of more and of fewer row groups than CTAs; long rows that leave
 # the other matrix's rows room for half a CTA's share.
 @pytest.mark.parametrize("rows,K", [((1, 1, 1, 1, 1, 1, 1, 1), 24), ((4000, 8), 24 * 40), ((8, 9000, 16, 1), 24 * 12 + 7),
