@@ -30,14 +30,14 @@ UNIT = "GB/s"
 NOMINAL_HBM_GBS = 8000.0
 FALLBACK_HBM_GBS = 6650.0
 # DRAM bytes per algorithmic byte of k_gemv_units, from the ncu capture summarised in
-# profiles/k_gemv_units_qwen3_8b.md (dram__bytes_read.sum + dram__bytes_write.sum = 203.9 MB
+# profiles/k_gemv_units_qwen3_8b.md (dram__bytes_read.sum + dram__bytes_write.sum = 206.1 MB
 # for the 198.4 MB of the first 4 layers; every code byte is read once, so traffic grows in
 # proportion to the matrices read and the full pass is scaled by its byte count).
-TRAFFIC_PER_ALGORITHMIC_BYTE = 1.03
+TRAFFIC_PER_ALGORITHMIC_BYTE = 1.04
 # Warp-instructions of k_gemv_units per 32 blocks (one block per lane), by pipe, and wavefronts of the
 # shared-memory/L1 data pipe, from the same capture (smsp__inst_executed.sum; the pipes from their shares of peak
 # over the active cycles, times the blocks processed / 32).
-KERNEL_COUNTERS = {"instr": 80.2, "alu": 34.1, "fmaheavy": 32.8, "lsu": 9.6, "wavefronts": 22.1}
+KERNEL_COUNTERS = {"instr": 77.6, "alu": 32.0, "fmaheavy": 32.5, "lsu": 9.8, "wavefronts": 21.5}
 
 
 def issue_bound_gbs(sm_mhz, sms=148):

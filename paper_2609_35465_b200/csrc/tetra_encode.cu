@@ -31,8 +31,9 @@
 // between sections only by a constant exists once.  24,576 Gaussian blocks: 61.2 ms by scanning the rows of the
 // lists in shared memory; 4.9 ms with these tables and one block per CTA; 2.3 ms three blocks in step; 1.86 ms with
 // two candidates per maximum and the trace once per block; 1.65 ms with the odd parity beside the even one; 1.55 ms
-// with packed additions; 1.45 ms with one copy of the half-table code (37,000 warp-instructions a block, issue slots
-// 53 % busy; what is left is barriers between the phases, 2 of 8 stall cycles per instruction).
+// with packed additions; 1.45 ms with one copy of the half-table code; 1.30 ms with five barriers a turn instead of eight, the
+// winner's warp tracing it and everything a turn ahead that can be (35,500 warp-instructions a block, issue slots
+// 58 % busy; what is left is instruction fetch and the barriers between the phases).
 #include <cuda_runtime.h>
 
 #include <cstdint>

@@ -124,9 +124,8 @@ def test_grouped_launch_one_layer(tt, table, orc):
     [(40, 49152, True), (3000, 24 * 64, True), (16, 49152 - 24, True)],               # the largest K, coarse mode
 ])
 def test_grouped_small_lists(tt, table, orc, shapes_list):
-    """Small lists run in the planned path's fine mode (one row group x a slice of the column
-    groups per unit, slices summed in fixed order by the last one to finish): every row checked,
-    and a second run of the same plan gives the same bits."""
+    """Small lists, whose units are cut into the warps' ranges (the pieces' sums added in fixed order by the
+    last to arrive): every row checked, and a second run of the same plan gives the same bits."""
     mats = [make_matrix(38, 100 * i + N, N, K, tm) for i, (N, K, tm) in enumerate(shapes_list)]
     devs = [upload(tt, table, m) for m in mats]
     problems = tt.make_problems(devs)
@@ -264,7 +263,7 @@ def test_gemv_list_rejects_long_lists(tt, table):
 # a plan describes itself: the workspace can be moved
 # ---------------------------------------------------------------------------
 @pytest.mark.parametrize("shapes_list", [
-    [(1024, 4096, True), (33, 749, False)],                                            # fine mode
+    [(1024, 4096, True), (33, 749, False)],                                            # fewer passes than warps
     [(40, 49152, True), (3000, 24 * 64, True), (16, 49152 - 24, True)],                # coarse mode
 ])
 def test_planned_workspace_can_be_copied_to_another_address(tt, table, orc, shapes_list):
