@@ -193,9 +193,12 @@ size_t grouped_workspace_bytes(const Problem* problems, int count) {
     return plan_meta_bytes(count, kMaxPlanWarps, cols) + kPiecesBytes + cols * kXqBytesPerCol;
 }
 
-// One thread per column of the list.  What bounds it is a chain of dependent loads, so all that the plan says about a thread's
-// column is read ahead of the wait, and its matrix is named by the plan instead of searched for (one 8B layer 6 -> 3 us).
+// One thread per column of the list.  What bounds it is a chain of dependent loads; a column's matrix is named by the plan
+// instead of searched for.  The plan may come from the kernel before (tetra_gemv_noalloc writes one, a caller may have copied
+// it), so nothing of it is read ahead of the wait; and k_gemv_units, which does read it ahead of its own, is released only
+// when the grids before this one are complete.
 __global__ void __launch_bounds__(128) k_prepare_x(unsigned char* __restrict__ ws) {
+    pdl_wait();  // the activations and the plan may come from the previous kernel of the stream
     pdl_release();
     const PlanHeader* H = reinterpret_cast<const PlanHeader*>(ws);
     const Problem* problems = reinterpret_cast<const Problem*>(ws + H->off_problems);
@@ -216,7 +219,6 @@ __global__ void __launch_bounds__(128) k_prepare_x(unsigned char* __restrict__ w
         cols = (K + 23) / 24;  // (one more than the words of a row where there is a tail)
     };
     find();
-    pdl_wait();  // the activations may come from the previous kernel of the stream
     for (; gc < total; gc += threads, find()) {
         if (c >= cols) continue;
         uint32_t q[20];
@@ -305,7 +307,8 @@ k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ w
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 512), "l"(codes_p + (at + Bu)));
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 1024), "l"(codes_p + (at + 2 * Bu)));
     };
-    // ahead of the wait: the plan, and the first record of a range that begins in a full column group
+    // ahead of the wait: the plan, and the first record of a range that begins in a full column group (both are older than
+    // k_prepare_x, which releases this kernel behind its own wait)
     if (H->nwarps == nw) {
         const bool has_range = warp < H->warps_per_cta;
         u = u_end = total_units;

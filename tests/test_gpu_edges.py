@@ -236,3 +236,27 @@ def test_planned_list_ranges(tt, table, orc, mats):
     for m, it, y in zip(ms, items, first):
         assert torch.equal(it["y"], y)
         check(orc, m, y.cpu().numpy(), "%d x %d of %d" % (m["N"], m["K"], len(ms)))
+
+
+# A plan that the kernel just before the run wrote, over the plan of a run still in flight: nothing of it may be read early.
+def test_plan_written_by_the_kernel_before(tt, table, orc):
+    sizes = [[(2048, 24 * 85, True), (17, 24 * 33 + 5, True)], [(40, 24 * 700 + 7, True), (3001, 24 * 32, True), (9, 24 * 5, True)]]
+    plans, items, mats = [], [], []
+    for i, shapes in enumerate(sizes):
+        ms = [make_matrix(84, 1000 * i + N, N, K, tail, batch=1) for N, K, tail in shapes]
+        its = [device_matrix(tt, table, m, torch.from_numpy(m["x"][0]).cuda()) for m in ms]
+        problems = tt.make_problems(its)
+        ws = torch.zeros(tt.tetra_grouped_workspace_bytes(problems), dtype=torch.uint8, device="cuda")
+        tt.tetra_gemv_grouped_plan(problems, ws)
+        plans.append(ws)
+        items.append(its)
+        mats.append(ms)
+    shared = torch.zeros(max(p.numel() for p in plans), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    for turn in range(40):
+        torch.bitwise_or(plans[turn % 2], 0, out=shared[:plans[turn % 2].numel()])
+        tt.tetra_gemv_grouped_run(shared, table)
+    torch.cuda.synchronize()
+    for ms, its in zip(mats, items):
+        for m, it in zip(ms, its):
+            check(orc, m, it["y"].cpu().numpy(), "%d x %d" % (m["N"], m["K"]))
