@@ -196,7 +196,7 @@ size_t grouped_workspace_bytes(const Problem* problems, int count) {
 // One thread per column of the list.  What bounds it is a chain of dependent loads; a column's matrix is named by the plan
 // instead of searched for.  The plan may come from the kernel before (tetra_gemv_noalloc writes one, a caller may have copied
 // it), so nothing of it is read ahead of the wait; and k_gemv_units, which does read it ahead of its own, is released only
-// when the grids before this one are complete.
+// when the grids before this one are complete (8B pass 764.5 us instead of 762.4, one layer of it 34.1 instead of 32.7).
 __global__ void __launch_bounds__(128) k_prepare_x(unsigned char* __restrict__ ws) {
     pdl_wait();  // the activations and the plan may come from the previous kernel of the stream
     pdl_release();
