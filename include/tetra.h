@@ -278,7 +278,8 @@ int tetra_gemv_grouped_hostio(void *workspace_dev, const void *table, const void
  *     tetra_gemv_tail.
  *   - Enqueues three kernels on `stream` (the first writes the product's
  *     description into the array from its own parameters, so no host memory is
- *     referenced after the call returns); does not synchronise. */
+ *     referenced after the call returns), and three more for every further 64 GB
+ *     of codes; does not synchronise. */
 int tetra_gemv_noalloc(const void *codes, const float *row_scales, const void *table,
                        const void *x, float *y, int N, int K, const void *tail, void *stream);
 

@@ -181,6 +181,27 @@ static inline int problem_units(const Problem& q) {
     return ((q.N + 7) / 8 + R - 1) / R;
 }
 
+// k_gemv_units keeps the places of a matrix's records as 16-byte units in 32 bits (in 64 bits a pass of the 8B model takes 770
+// to 775 us instead of 765).  A matrix that is larger is planned as slices of this many rows: problems of their own, one behind
+// the other, that share their activation records.
+static inline long long slice_rows(const Problem& q) { return 8 * (0xFFFFFFFELL / (3 * problem_blocks(q)) / 6 * 6); }
+int problem_slices(const Problem& q) { return int((q.N + slice_rows(q) - 1) / slice_rows(q)); }
+Problem problem_slice(const Problem& q, int i) {
+    const long long rows = slice_rows(q), row0 = i * rows;
+    Problem p = q;
+    p.codes = static_cast<const char*>(q.codes) + row0 / 8 * 48 * problem_blocks(q);
+    p.row_scales = q.row_scales + row0;
+    if (q.tail) p.tail = static_cast<const char*>(q.tail) + 2 * row0 * (q.K % 24);
+    p.y = q.y + row0;
+    p.N = int32_t(q.N - row0 < rows ? q.N - row0 : rows);
+    return p;
+}
+// b is the slice behind a: its columns are a's
+static inline bool same_columns(const Problem& a, const Problem& b) {
+    return a.N == slice_rows(a) && b.x == a.x && b.K == a.K && !b.tail == !a.tail &&
+           b.codes == static_cast<const char*>(a.codes) + (long long)(a.N / 8) * 48 * problem_blocks(a);
+}
+
 // The activation records of 32 columns lie together, part by part: 16 bytes of every column, then the next 16.  A warp's load
 // is then 512 contiguous bytes, four wavefronts, and not 32 pieces 80 bytes apart (8B pass 773 -> 763 us, one layer of it
 // 34.7 -> 32.7).
@@ -189,8 +210,12 @@ __device__ __forceinline__ uint32_t record_at(uint32_t col) { return (col >> 5) 
 
 size_t grouped_workspace_bytes(const Problem* problems, int count) {
     size_t cols = 0;
-    for (int i = 0; i < count; ++i) cols += size_t(problem_cols(problems[i]));
-    return plan_meta_bytes(count, kMaxPlanWarps, cols) + kPiecesBytes + cols * kXqBytesPerCol;
+    int slices = 0;
+    for (int i = 0; i < count; ++i) {
+        cols += size_t(problem_cols(problems[i]));
+        slices += problem_slices(problems[i]);
+    }
+    return plan_meta_bytes(slices, kMaxPlanWarps, cols) + kPiecesBytes + cols * kXqBytesPerCol;
 }
 
 // One thread per column of the list.  What bounds it is a chain of dependent loads; a column's matrix is named by the plan
@@ -525,15 +550,19 @@ k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ w
     }
 }
 
-cudaError_t grouped_plan(const Problem* problems, int count, void* ws_dev, size_t ws_bytes, cudaStream_t s) {
-    if (ws_bytes < grouped_workspace_bytes(problems, count)) return cudaErrorInvalidValue;
+cudaError_t grouped_plan(const Problem* problems, int matrices, void* ws_dev, size_t ws_bytes, cudaStream_t s) {
+    if (ws_bytes < grouped_workspace_bytes(problems, matrices)) return cudaErrorInvalidValue;
     int sms = 0;
     cudaError_t e = device_sms(&sms);
     if (e != cudaSuccess) return e;
     int nwarps = sms * kUnitWarps;  // the grid grouped_run launches on this device
     if (nwarps > kMaxPlanWarps) nwarps = 0;
     size_t all_cols = 0;
-    for (int i = 0; i < count; ++i) all_cols += size_t(problem_cols(problems[i]));
+    int count = 0;  // of slices
+    for (int i = 0; i < matrices; ++i) {
+        all_cols += size_t(problem_cols(problems[i]));
+        count += problem_slices(problems[i]);
+    }
     const size_t meta = plan_meta_bytes(count, nwarps, all_cols);
     unsigned char* buf = static_cast<unsigned char*>(calloc(1, meta));
     if (!buf) return cudaErrorMemoryAllocation;
@@ -547,7 +576,8 @@ cudaError_t grouped_plan(const Problem* problems, int count, void* ws_dev, size_
         const int Bi = problem_blocks(q);
         return groups_per_unit(Bi) * (Bi / 32) + (Bi % 32 ? 1 : 0);
     };
-    memcpy(problems_host, problems, size_t(count) * sizeof(Problem));
+    for (int i = 0, at = 0; i < matrices; ++i)
+        for (int k = 0; k < problem_slices(problems[i]); ++k) problems_host[at++] = problem_slice(problems[i], k);
     std::stable_sort(problems_host, problems_host + count, [&](const Problem& a, const Problem& b) { return longest(a) > longest(b); });
     H->off_problems = uint32_t(sizeof(PlanHeader));
     H->off_unit_prefix = H->off_problems + uint32_t(count) * uint32_t(sizeof(Problem));
@@ -564,7 +594,7 @@ cudaError_t grouped_plan(const Problem* problems, int count, void* ws_dev, size_
         up[i] = int32_t(units);
         cp[i] = int32_t(cols);
         units += problem_units(problems_host[i]);
-        cols += problem_cols(problems_host[i]);
+        if (i + 1 == count || !same_columns(problems_host[i], problems_host[i + 1])) cols += problem_cols(problems_host[i]);
     }
     up[count] = int32_t(units);
     cp[count] = int32_t(cols);

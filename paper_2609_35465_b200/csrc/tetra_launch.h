@@ -92,6 +92,9 @@ cudaError_t launch_encode(const float* w, const float* sigma, const void* table,
 // buffer; copied to the start of a scratch area of single_plan_scratch_bytes(blocks)
 // bytes, it makes that area a valid argument of grouped_run.
 size_t single_plan_meta_bytes();
+// A matrix too large for one plan is run as slices of its rows.
+int problem_slices(const Problem& problem);
+Problem problem_slice(const Problem& problem, int i);
 size_t single_plan_scratch_bytes(int blocks_per_row);
 void single_plan_fill(const Problem& problem, unsigned char* meta_host);
 

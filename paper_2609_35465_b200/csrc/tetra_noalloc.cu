@@ -82,9 +82,11 @@ extern "C" int tetra_gemv_noalloc(const void* codes, const float* row_scales, co
     PlanBlob blob;
     static_assert(sizeof blob.bytes >= 256, "plan blob");
     if (single_plan_meta_bytes() > sizeof blob.bytes) return TETRA_ERR_SIZE;
-    single_plan_fill(problem, blob.bytes);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    k_write_plan<<<1, 64, 0, s>>>(static_cast<unsigned char*>(scratch), blob);
-    if (cudaGetLastError() != cudaSuccess) return TETRA_ERR_CUDA;
-    return grouped_run(scratch, table, s) == cudaSuccess ? TETRA_OK : TETRA_ERR_CUDA;
+    for (int i = 0; i < problem_slices(problem); ++i) {  // one, up to 64 GB
+        single_plan_fill(problem_slice(problem, i), blob.bytes);
+        k_write_plan<<<1, 64, 0, s>>>(static_cast<unsigned char*>(scratch), blob);
+        if (cudaGetLastError() != cudaSuccess || grouped_run(scratch, table, s) != cudaSuccess) return TETRA_ERR_CUDA;
+    }
+    return TETRA_OK;
 }

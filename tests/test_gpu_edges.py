@@ -260,3 +260,38 @@ def test_plan_written_by_the_kernel_before(tt, table, orc):
     for ms, its in zip(mats, items):
         for m, it in zip(ms, its):
             check(orc, m, it["y"].cpu().numpy(), "%d x %d" % (m["N"], m["K"]))
+
+
+# One matrix of more than 64 GB: places of records beyond 2^32 sixteen-byte units.  All rows are the origin but the first row
+# group's and the last two's, which lie where a place in 32 bits would wrap around to rows of the beginning.
+@pytest.mark.parametrize("entry,B", [("grouped", 2048), ("noalloc", 1024), ("list", 2048)])
+def test_matrix_beyond_64_gigabytes(tt, table, orc, entry, B):
+    G = (1 << 32) // (3 * B) + 3
+    N, K = 8 * G, 24 * B
+    torch.cuda.empty_cache()
+    if torch.cuda.mem_get_info()[0] < (72 << 30):
+        pytest.skip("less than 72 GB free")
+    m = make_matrix(85, B, 24, K, True, batch=1)
+    codes = torch.zeros(G * 3 * B * 16, dtype=torch.uint8, device="cuda")
+    packed = tt.tetra_pack_codes(torch.from_numpy(m["codes"]).cuda(), table, 24, B)
+    part = 3 * B * 16
+    codes[:part] = packed[:part]
+    codes[-2 * part:] = packed[part:]
+    rows = torch.cat([torch.arange(8), torch.arange(N - 16, N)]).cuda()
+    scales = torch.ones(N, device="cuda")
+    scales[rows] = torch.from_numpy(m["sigma"]).cuda()
+    x, y = torch.from_numpy(m["x"][0]).cuda(), torch.full((N,), float("nan"), device="cuda")
+    problems = tt.make_problems([dict(codes=codes, row_scales=scales, x=x, tail=None, y=y, N=N, K=K)])
+    if entry == "grouped":
+        ws = torch.empty(tt.tetra_grouped_workspace_bytes(problems), dtype=torch.uint8, device="cuda")
+        tt.tetra_gemv_grouped(problems, table, ws)
+    elif entry == "noalloc":
+        tt.tetra_gemv_noalloc(codes, scales, table, x, y, N, K)
+    else:
+        tt.tetra_gemv_list(problems, table)
+    torch.cuda.synchronize()
+    check(orc, m, y[rows].cpu().numpy(), "%s, %d x %d" % (entry, N, K))
+    y[rows] = 0
+    assert torch.count_nonzero(y) == 0
+    del codes
+    torch.cuda.empty_cache()
