@@ -183,7 +183,7 @@ int tetra_gemv_grouped_plan(const tetra_problem* problems_host, int count, void*
     if (rc) return rc;
     if (!workspace_dev) return TETRA_ERR_NULL;
     if (!aligned(workspace_dev, 16)) return TETRA_ERR_ALIGN;
-    if (workspace_bytes < grouped_workspace_bytes(reinterpret_cast<const Problem*>(problems_host), count))
+    if (workspace_bytes < grouped_workspace_least(reinterpret_cast<const Problem*>(problems_host), count))
         return TETRA_ERR_SIZE;
     return cuda_status(grouped_plan(reinterpret_cast<const Problem*>(problems_host), count, workspace_dev,
                                     workspace_bytes, as_stream(stream)));

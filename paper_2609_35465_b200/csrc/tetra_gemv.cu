@@ -116,20 +116,24 @@ cudaError_t launch_gemv_paper(const void* codes, size_t row_stride, const float*
 // Planned list of matrices: k_prepare_x + k_gemv_units
 // ===========================================================================
 // Workspace written by grouped_plan (host) and read by both kernels:
-//   PlanHeader | Problem[count] | unit_prefix[count + 1] | col_prefix[count + 1]
-//              | WarpCut[ranges + 1] (optional) | col_start[] | pad | counters | partial sums | xq records
+//   PlanHeader | Problem[count] | unit_prefix[count + 1] | col_prefix[count + 1] | WarpCut[ranges + 1] (optional) | col_start[]
+//              | pad | counters | partial sums | pad | xq records
 // A unit is groups_per_unit(B) consecutive row groups of one matrix, all columns; a pass is 32 of its columns (or the joint
 // pass over its row groups' last, partial column groups).
 struct PlanHeader {
     int32_t count;
     int32_t total_units;  // sum over matrices of their units
-    int32_t total_cols;   // sum over matrices of words per row, each rounded up to 32 (so is col_prefix)
+    int32_t total_cols;   // sum over matrices of words per row, each rounded up to 32 if `aligned`
+    int32_t aligned;      // (where the workspace has room for that)
+    int32_t row_groups;   // of a unit, at most
     int32_t nwarps;       // warps of the grid that the ranges were cut for (0: no ranges, units are dealt round-robin)
     int32_t warps_per_cta;  // warps of a CTA that have a range
     uint32_t off_problems, off_unit_prefix, off_col_prefix, off_xq;
     uint32_t off_cuts, off_col_start;
-    uint32_t off_counters;  // int32 per range: pieces that have arrived of the unit cut behind it
-    uint32_t off_partials;  // float [range][2][kPieceFloats]
+    int32_t col_shift;      // col_start names the matrix of every 2^col_shift-th column of the list
+    uint32_t off_counters;  // int32 per unit or per range, whichever are fewer: pieces of the cut unit that have arrived
+    int32_t counters;
+    uint32_t off_partials;  // float [slot][8]: a cut unit's row sums, a slot per piece and row group
     // units [0, dyn_start) are cut into the warps' ranges; the units from
     // dyn_start on are claimed one at a time through dyn_next by warps that have finished their range
     // (k_prepare_x sets dyn_next = dyn_start before every run)
@@ -144,24 +148,18 @@ constexpr int kClaimPasses = 128;          // passes per warp from which on ther
 constexpr int kPassCost = 8, kFoldCost = 4;
 
 // Where a warp's range begins; the next entry is where it ends.  A range that begins inside a unit (pass > 0) shares that
-// unit with the ranges before it: `first` is the one in which the unit begins, `pieces` the number of ranges it touches.
+// unit with the ranges before it: `pieces` ranges in all, of which the first, the one in which the unit begins, is `back` ranges
+// before this one; `slot` is the unit's first.  (Twelve bytes: the cuts for 160 multiprocessors have to lie in the 32 KB that
+// the workspace has always had for them.)
 struct WarpCut {
-    int32_t unit, pass, first, pieces;
-    int32_t matrix;  // of the unit
-    int32_t pad_[3];
+    int32_t unit;
+    uint32_t at;     // matrix of the unit << 8 | pass
+    uint32_t piece;  // slot << 16 | pieces << 8 | back
+    __device__ __host__ static int pass(uint32_t at) { return int(at & 255u); }
+    __device__ __host__ static int matrix(uint32_t at) { return int(at >> 8); }
 };
-constexpr int kColsPerStart = 64;  // col_start names the matrix of every 64th column of the list
-constexpr size_t kSingleCols = 1024;  // columns of a plan that single_plan_fill writes, at most
-constexpr int kPieceFloats = 24;  // row sums of a unit's row groups
-
-constexpr int kMaxPlanWarps = 8192;    // room reserved for the ranges in a planned list's workspace
-constexpr size_t kPiecesBytes = size_t(kMaxPlanWarps) * (4 + 2 * kPieceFloats * 4);  // their counters and partial sums
-
-static size_t plan_meta_bytes(int count, int nwarps, size_t cols) {
-    size_t b = sizeof(PlanHeader) + size_t(count) * sizeof(Problem) + 2 * size_t(count + 1) * 4 +
-               16 + (nwarps ? size_t(nwarps + 1) * sizeof(WarpCut) : 0) + size_t(cols / kColsPerStart + 1) * 4;
-    return (b + 255) & ~size_t(255);
-}
+constexpr int kMaxUnitPasses = 3 * 63 + 1;  // (more than one row group: at most ten columns beside full groups, 2048 columns)
+static_assert(kMaxUnitPasses < 256, "a pass, and the pieces of a unit, in eight bits");
 
 static inline int problem_blocks(const Problem& q) {
     return (q.tail || q.K % 24 == 0) ? q.K / 24 : (q.K + 23) / 24;
@@ -170,14 +168,14 @@ static inline int problem_blocks(const Problem& q) {
 // Row groups (of eight rows) one unit covers.  When the last column group of a matrix is at most
 // half full (B mod 32 in 1..16), up to three consecutive row groups share one pass over it, so that
 // pass runs with most lanes busy instead of B mod 32 of them.
-__host__ __device__ inline int groups_per_unit(int B) {
-    const int rem = B & 31;
-    if (rem == 0 || rem > 16) return 1;
-    const int r = 32 / rem;
-    return r < 3 ? r : 3;
+constexpr int kMaxRowGroups = 3;
+__host__ __device__ inline int groups_per_unit(int B, int most) {
+    const uint32_t rem = uint32_t(B) & 31u;
+    const int r = rem - 1u < 10u ? 3 : (rem - 1u < 16u ? 2 : 1);
+    return r < most ? r : most;
 }
-static inline int problem_units(const Problem& q) {
-    const int R = groups_per_unit(problem_blocks(q));
+static inline int problem_units(const Problem& q, int row_groups) {
+    const int R = groups_per_unit(problem_blocks(q), row_groups);
     return ((q.N + 7) / 8 + R - 1) / R;
 }
 
@@ -204,19 +202,57 @@ static inline bool same_columns(const Problem& a, const Problem& b) {
 
 // The activation records of 32 columns lie together, part by part: 16 bytes of every column, then the next 16.  A warp's load
 // is then 512 contiguous bytes, four wavefronts, and not 32 pieces 80 bytes apart (8B pass 773 -> 763 us, one layer of it
-// 34.7 -> 32.7).
-static inline long long problem_cols(const Problem& q) { return (problem_blocks(q) + 31LL) & ~31LL; }
-__device__ __forceinline__ uint32_t record_at(uint32_t col) { return (col >> 5) * uint32_t(2 * kXqBytesPerCol) + (col & 31u); }
-
-size_t grouped_workspace_bytes(const Problem* problems, int count) {
-    size_t cols = 0;
-    int slices = 0;
-    for (int i = 0; i < count; ++i) {
-        cols += size_t(problem_cols(problems[i]));
-        slices += problem_slices(problems[i]);
-    }
-    return plan_meta_bytes(slices, kMaxPlanWarps, cols) + kPiecesBytes + cols * kXqBytesPerCol;
+// 34.7 -> 32.7).  In a plan whose columns are not aligned a column's 80 bytes lie together and a matrix takes no more than
+// those (the same times and 769.6 us, 35.9 us with them).
+static inline long long problem_cols(const Problem& q, bool aligned) {
+    const int B = problem_blocks(q);
+    return aligned ? (B + 31) & ~31 : B;
 }
+template <bool ALIGNED>
+__device__ __forceinline__ uint32_t record_at(uint32_t col) {
+    constexpr uint32_t U = kXqBytesPerCol / 16;
+    return ALIGNED ? (col >> 5) * (32 * U) + (col & 31u) : col * U;
+}
+
+// Bytes of a plan: what the kernels read, and what they keep beside it.
+static size_t plan_meta_bytes(int count, int ranges, int starts) {
+    const size_t b = sizeof(PlanHeader) + size_t(count) * sizeof(Problem) + 2 * size_t(count + 1) * 4 +
+                     (ranges ? size_t(ranges + 1) * sizeof(WarpCut) : 0) + size_t(starts) * 4;
+    return (b + 255) & ~size_t(255);
+}
+static size_t plan_bytes(size_t meta, int counters, size_t slots, size_t cols) {
+    return ((meta + size_t(counters) * 4 + slots * 32 + 127) & ~size_t(127)) + cols * kXqBytesPerCol;
+}
+// Entries of col_start: a column in 64, but no more than four a matrix.
+static int col_shift_for(size_t cols, int count) {
+    int shift = 6;
+    while ((cols >> shift) + 1 > 4 * size_t(count)) ++shift;
+    return shift;
+}
+
+// What a caller is asked for.  A list of at most kRoomTasks (row group, column group) pairs is given 32 bytes a pair, which hold
+// the pieces of any cut of units of one row group.  A longer one is given six slots a range and room for aligned columns, but
+// planned without them too: callers may have a workspace of a fixed size, and these were not always asked for (8B, 4 / 8 / 12 /
+// 36 layers 99.8 / 184 / 266 / 764 us, in the smaller workspace 117 / 195 / 273 / 779).
+constexpr long long kRoomTasks = 65536;
+constexpr size_t kCutsRoom = 8193 * 4, kMatrixRoom = 16, kRangesRoom = 2560;  // (2560 ranges: 160 multiprocessors)
+static_assert((kRangesRoom + 1) * sizeof(WarpCut) + sizeof(PlanHeader) - 56 < kCutsRoom, "the cuts have room");
+static size_t workspace_bytes(const Problem* problems, int count, bool slots_of_long_lists) {
+    size_t cols = 0, groups = 0, tasks = 0;
+    for (int i = 0; i < count; ++i) {
+        const size_t B = size_t(problem_blocks(problems[i])), G = (size_t(problems[i].N) + 7) / 8;
+        cols += B;
+        groups += G;
+        tasks += G * ((B + 31) / 32);
+    }
+    size_t b = (56 + size_t(count) * (sizeof(Problem) + kMatrixRoom) + 2 * size_t(count + 1) * 4 + kCutsRoom + 255) & ~size_t(255);
+    b += cols * kXqBytesPerCol;
+    if (tasks <= size_t(kRoomTasks)) b = ((b + 255) & ~size_t(255)) + groups * 4 + 256 + tasks * 32;
+    else if (slots_of_long_lists) b += kRangesRoom * (4 + 6 * 32) + size_t(count) * 31 * kXqBytesPerCol;
+    return b;
+}
+size_t grouped_workspace_bytes(const Problem* problems, int count) { return workspace_bytes(problems, count, true); }
+size_t grouped_workspace_least(const Problem* problems, int count) { return workspace_bytes(problems, count, false); }
 
 // One thread per column of the list.  What bounds it is a chain of dependent loads; a column's matrix is named by the plan
 // instead of searched for.  The plan may come from the kernel before (tetra_gemv_noalloc writes one, a caller may have copied
@@ -233,15 +269,18 @@ __global__ void __launch_bounds__(128) k_prepare_x(unsigned char* __restrict__ w
     const int total = H->total_cols, threads = int(gridDim.x * blockDim.x);
     int gc = blockIdx.x * blockDim.x + threadIdx.x;
     const __half* x = nullptr;
-    int K = 0, c = 0, cols = 0;
+    int K = 0, c = 0, cols = 0, begin = 0;
+    const int col_shift = H->col_shift;
+    const bool aligned = H->aligned;
     auto find = [&] {
         if (gc >= total) return;
-        int p = __ldg(col_start + gc / kColsPerStart);
+        int p = __ldg(col_start + (gc >> col_shift));
         while (__ldg(col_prefix + p + 1) <= gc) ++p;
-        c = gc - __ldg(col_prefix + p);
+        begin = __ldg(col_prefix + p);
+        c = gc - begin;
         x = static_cast<const __half*>(problems[p].x);
         K = problems[p].K;
-        cols = (K + 23) / 24;  // (one more than the words of a row where there is a tail)
+        cols = problems[p].tail ? K / 24 : (K + 23) / 24;
     };
     find();
     for (; gc < total; gc += threads, find()) {
@@ -249,18 +288,22 @@ __global__ void __launch_bounds__(128) k_prepare_x(unsigned char* __restrict__ w
         uint32_t q[20];
         quantise_column(x, K, c, q);
         pair_planes(q);
+        uint4* rec = xq + size_t(begin) * (kXqBytesPerCol / 16) + (aligned ? record_at<true>(uint32_t(c)) : record_at<false>(uint32_t(c)));
+        const int part = aligned ? 32 : 1;
 #pragma unroll
-        for (int k = 0; k < 5; ++k) xq[record_at(uint32_t(gc)) + 32 * k] = make_uint4(q[4 * k], q[4 * k + 1], q[4 * k + 2], q[4 * k + 3]);
+        for (int k = 0; k < 5; ++k) rec[part * k] = make_uint4(q[4 * k], q[4 * k + 1], q[4 * k + 2], q[4 * k + 3]);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0)
         reinterpret_cast<PlanHeader*>(ws)->dyn_next = H->dyn_start;  // the claimed units start over
     int32_t* counters = reinterpret_cast<int32_t*>(ws + H->off_counters);  // and so do the arrivals at cut units
-    for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < H->nwarps; w += threads) counters[w] = 0;
+    for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < H->counters; w += threads) counters[w] = 0;
 }
 
 // This lane's activation record (global memory, L1/L2 resident) into registers.
+template <bool ALIGNED>
 __device__ __forceinline__ void load_lane_x(const uint4* src, bool active, LanePairs& X) {
-    const uint4 t0 = __ldg(src), t1 = __ldg(src + 32), t2 = __ldg(src + 64), t3 = __ldg(src + 96), t4 = __ldg(src + 128);
+    constexpr int part = ALIGNED ? 32 : 1;
+    const uint4 t0 = __ldg(src), t1 = __ldg(src + part), t2 = __ldg(src + 2 * part), t3 = __ldg(src + 3 * part), t4 = __ldg(src + 4 * part);
     X.hi[0] = t0.x; X.hi[1] = t0.y; X.hi[2] = t0.z; X.hi[3] = t0.w; X.hi[4] = t1.x; X.hi[5] = t1.y;
     X.hi[6] = t1.z; X.hi[7] = t1.w; X.hi[8] = t2.x; X.hi[9] = t2.y; X.hi[10] = t2.z; X.hi[11] = t2.w;
     X.lo[0] = t3.x; X.lo[1] = t3.y; X.lo[2] = t3.z; X.lo[3] = t3.w; X.lo[4] = t4.x; X.lo[5] = t4.y;
@@ -274,17 +317,9 @@ constexpr int kUnitThreads = TETRA_UNIT_THREADS;
 constexpr int kUnitWarps = kUnitThreads / 32;
 constexpr int kUnitFloats = kRedFloats + 96;  // per warp: the transpose buffer, and a sum per row group and lane
 
-// The persistent kernel of a planned list: every warp walks its range of units (up to three row groups of one matrix, all
-// columns).  All that it needs to know is in the workspace, so a workspace can be copied or moved and still runs correctly:
-// the host needs no record of it.
-__global__ void __launch_bounds__(kUnitThreads, 1)
-k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ ws) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    pdl_release();
-    unsigned char* smem = stage_fast_tables(tab, smem_raw);
-    const uint32_t sm_tab = smem_u32(smem);
-    __syncthreads();  // the only CTA-wide barrier: the tables are staged (by cp.async, the plan read meanwhile: 783 instead of
-                      // 773 us for the 8B pass)
+// Every warp walks its range of passes.
+template <bool ALIGNED>
+__device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsigned char* smem, uint32_t sm_tab) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float* red = reinterpret_cast<float*>(smem + kFastBytes) + warp * kUnitFloats;
     float* sums = red + kRedFloats + lane;  // of row group gi, row lane / 4: this lane's part at 32 gi
@@ -340,14 +375,15 @@ k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ w
         u_step = 1;
         if (has_range) {
             cut = reinterpret_cast<const WarpCut*>(ws + H->off_cuts) + (blockIdx.x * H->warps_per_cta + warp);
+            const uint32_t at = __ldg(&cut[0].at);
             u = __ldg(&cut[0].unit);
-            pass0 = __ldg(&cut[0].pass);
-            u_end = __ldg(&cut[1].unit) + (__ldg(&cut[1].pass) > 0);
+            pass0 = WarpCut::pass(at);
+            u_end = __ldg(&cut[1].unit) + (WarpCut::pass(__ldg(&cut[1].at)) > 0);
             claim = H->dyn_start < total_units;
             if (u < u_end) {
-                p = __ldg(&cut[0].matrix);
+                p = WarpCut::matrix(at);
                 enter_matrix();
-                const int R = groups_per_unit(int(Bu)), CGf = int(Bu >> 5), g0 = (u - p_begin) * R;
+                const int R = groups_per_unit(int(Bu), H->row_groups), CGf = int(Bu >> 5), g0 = (u - p_begin) * R;
                 const int gi = CGf ? pass0 / CGf : 0;
                 if (CGf && gi < min(R, G - g0)) {
                     request(slot, uint32_t(g0 + gi) * 3u * Bu + uint32_t(lane + 32 * (pass0 - gi * CGf)));
@@ -357,7 +393,7 @@ k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ w
         }
     }
     asm volatile("cp.async.commit_group;");
-    pdl_wait();  // the activation records (and zeroed counters) come from k_prepare_x
+    if (ALIGNED) pdl_wait();  // the activation records (and zeroed counters) come from k_prepare_x
 
     for (;; u += u_step) {
         if (u >= u_end) {
@@ -382,7 +418,7 @@ k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ w
         }
         const int CGf = int(Bu >> 5);   // full column groups
         const int rem = int(Bu & 31);   // columns of the last, partial one
-        const int R = groups_per_unit(int(Bu));
+        const int R = groups_per_unit(int(Bu), H->row_groups);
         const int g0 = (u - p_begin) * R;
         const int ng = min(R, G - g0);
         const uint4* codes0 = codes_p + size_t(g0) * 3 * Bu;
@@ -396,7 +432,7 @@ k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ w
         // the passes of this unit that the range holds: all of them, unless the range begins or ends inside it
         int left = ng * CGf + (rem > 0);
         const bool ends_inside = cut && u == __ldg(&cut[1].unit);  // (a range that ends between two units does not reach the second)
-        if (ends_inside) left = __ldg(&cut[1].pass);
+        if (ends_inside) left = WarpCut::pass(__ldg(&cut[1].at));
         left -= pass0;
         bool joint = pass0 >= ng * CGf;
         int gi = joint ? 0 : pass0 / CGf;
@@ -429,7 +465,7 @@ k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ w
         bool lane_on = !joint || lane_in;
         int seg = joint ? 1 : min(CGf - cg0, left);                        // passes left in the segment
         left -= seg;                                                       // and behind it
-        uint32_t x_at = x_p + record_at(joint ? lane_col : uint32_t(lane + 32 * cg0));
+        uint32_t x_at = x_p + record_at<ALIGNED>(joint ? lane_col : uint32_t(lane + 32 * cg0));
         // the first record behind the segment: the next row group's, the joint pass's, the next unit's
         constexpr uint32_t kNone = 0xFFFFFFFFu;
         auto behind = [&]() -> uint32_t {
@@ -449,7 +485,7 @@ k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ w
             // ahead of the next record's copies: the same unit serves both in order, and a load behind a copy waits for
             // memory (Qwen3-8B pass 810 -> 803 us)
             LanePairs X;
-            load_lane_x(reinterpret_cast<const uint4*>(ws) + x_at, lane_on, X);
+            load_lane_x<ALIGNED>(reinterpret_cast<const uint4*>(ws) + x_at, lane_on, X);
             x_at += 32 * kXqBytesPerCol / 16;
             // prefetch the next pass's record (or the first one of this warp's next unit)
             record = seg == 1 ? after : record + 32u;
@@ -482,13 +518,13 @@ k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ w
             for (int r = 0; r < 8; ++r) acc[r] = 0.f;
             if (!left) break;
             ++gi;
-            x_at = x_p + uint32_t(lane);
+            x_at = x_p + record_at<ALIGNED>(uint32_t(lane));
             seg = min(CGf, left);
             if (gi == ng) {
                 joint = true;
                 lane_on = lane_in;
                 seg = 1;
-                x_at = x_p + record_at(lane_col);
+                x_at = x_p + record_at<ALIGNED>(lane_col);
             }
             left -= seg;
             after = behind();
@@ -499,30 +535,35 @@ k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ w
         const WarpCut* shared = pass0 ? cut : (ends_inside ? cut + 1 : nullptr);
         pass0 = 0;
         if (shared) {
-            const int first = __ldg(&shared->first), pieces = __ldg(&shared->pieces);
+            const uint32_t info = __ldg(&shared->piece);
             const int range = blockIdx.x * H->warps_per_cta + warp;
-            float* partials = reinterpret_cast<float*>(ws + H->off_partials);
-            // a range's piece of the unit that it ends in lies behind its piece of the unit that it begins in
-            float* mine = partials + size_t(2 * range + (range == first)) * kPieceFloats + (lane >> 2);
+            const int pieces = int(info >> 8 & 255u), first = range + int(shared - cut) - int(info & 255u);
+            float* all = reinterpret_cast<float*>(ws + H->off_partials) + size_t(info >> 16) * 8 + (lane >> 2);
+            float* mine = all + (range - first) * ng * 8;
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
+            for (int k = 0; k < kMaxRowGroups; ++k) {
                 float v = sums[32 * k];
                 v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
                 v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
-                if ((lane & 3) == 0) __stcg(mine + 8 * k, v);
+                if ((lane & 3) == 0 && k < ng) __stcg(mine + 8 * k, v);
             }
             __threadfence();
             __syncwarp();
             int arrived = 0;
-            if (lane == 0) arrived = atomicAdd(reinterpret_cast<int32_t*>(ws + H->off_counters) + first, 1);
+            if (lane == 0) arrived = atomicAdd(reinterpret_cast<int32_t*>(ws + H->off_counters) + (H->counters == total_units ? u : first), 1);
             if (__shfl_sync(0xFFFFFFFFu, arrived, 0) != pieces - 1) continue;
             __threadfence();
             float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-            for (int k = lane & 3; k < pieces; k += 4) {
-                const float* theirs = partials + size_t(2 * (first + k) + (k == 0)) * kPieceFloats + (lane >> 2);
-                s0 += __ldcg(theirs);
-                s1 += __ldcg(theirs + 8);
-                s2 += __ldcg(theirs + 16);
+            if (ng == 1) {
+#pragma unroll 4
+                for (int k = lane & 3; k < pieces; k += 4) s0 += __ldcg(all + 8 * k);
+            } else {  // (of two row groups the third sum is not read)
+                for (int k = lane & 3; k < pieces; k += 4) {
+                    const float* theirs = all + k * ng * 8;
+                    s0 += __ldcg(theirs);
+                    s1 += __ldcg(theirs + 8);
+                    if (ng > 2) s2 += __ldcg(theirs + 16);
+                }
             }
             sums[0] = s0;
             sums[32] = s1;
@@ -550,31 +591,148 @@ k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ w
     }
 }
 
-cudaError_t grouped_plan(const Problem* problems, int matrices, void* ws_dev, size_t ws_bytes, cudaStream_t s) {
-    if (ws_bytes < grouped_workspace_bytes(problems, matrices)) return cudaErrorInvalidValue;
-    int sms = 0;
-    cudaError_t e = device_sms(&sms);
-    if (e != cudaSuccess) return e;
-    int nwarps = sms * kUnitWarps;  // the grid grouped_run launches on this device
-    if (nwarps > kMaxPlanWarps) nwarps = 0;
-    size_t all_cols = 0;
+// (Out of line: with both copies in the kernel a pass of the 8B model takes 769 us instead of 764.)
+__device__ __noinline__ void walk_unaligned(unsigned char* ws, unsigned char* smem, uint32_t sm_tab) { walk_units<false>(ws, smem, sm_tab); }
+
+// The persistent kernel of a planned list.  All that it needs to know is in the workspace, so a workspace can be copied or moved
+// and still runs correctly: the host needs no record of it.
+__global__ void __launch_bounds__(kUnitThreads, 1)
+k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ ws) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_release();
+    unsigned char* smem = stage_fast_tables(tab, smem_raw);
+    const uint32_t sm_tab = smem_u32(smem);
+    __syncthreads();  // the only CTA-wide barrier: the tables are staged (by cp.async, the plan read meanwhile: 783 instead of
+                      // 773 us for the 8B pass)
+    if (reinterpret_cast<const PlanHeader*>(ws)->aligned) {
+        walk_units<true>(ws, smem, sm_tab);
+    } else {
+        pdl_wait();
+        walk_unaligned(ws, smem, sm_tab);
+    }
+}
+
+// Cuts the list's passes into the ranges of the grid's warps; `inside`: also inside units.  Returns the slots that the pieces of
+// cut units take.
+static size_t cut_ranges(PlanHeader* H, const Problem* problems, const int32_t* up, WarpCut* cuts, int sms, bool inside) {
+    const int count = H->count;
+    const long long units = H->total_units;
+    // Cut the sequence of passes into contiguous ranges of equal work.  A cut inside a unit costs its two sides a store of
+    // sums and an atomic, two of each per warp and run; cut between units only, a list of a few layers leaves most warps
+    // waiting for those with one unit more (4B, one / two / six layers 28.9 / 40.9 / 92.6 us, cut inside units
+    // 24.8 / 39.0 / 87.3; 14B, one layer 59.2 and 51.4).
+    auto unit_groups = [&](int i, long long k) {
+        const int G = (problems[i].N + 7) / 8, R = groups_per_unit(problem_blocks(problems[i]), H->row_groups);
+        return int(G - k * R < R ? G - k * R : R);
+    };
+    auto unit_passes = [&](int i, long long k) {
+        const int Bi = problem_blocks(problems[i]);
+        return unit_groups(i, k) * (Bi / 32) + (Bi % 32 ? 1 : 0);
+    };
+    auto unit_cost = [&](int i, long long k) { return (long long)unit_passes(i, k) * kPassCost + kFoldCost * unit_groups(i, k); };
+    auto full_work = [&](int i) { return unit_cost(i, 0); };      // of all units but the last
+    auto matrix_work = [&](int i) {
+        const long long U = problem_units(problems[i], H->row_groups);
+        return (U - 1) * full_work(i) + unit_cost(i, U - 1);
+    };
+    long long total = 0, passes = 0;
+    for (int i = 0; i < count; ++i) {
+        const long long U = problem_units(problems[i], H->row_groups);
+        total += matrix_work(i);
+        passes += (U - 1) * unit_passes(i, 0) + unit_passes(i, U - 1);
+    }
+    // Of a long list the last tenth of the work is not assigned: warps that finish early claim it unit by unit, which
+    // evens out what the cost model and the warps' unequal speeds leave.  A unit claimed last still makes the others wait
+    // for it, which shorter lists do not make up for.  All assigned / a tenth claimed, us: 8B, 8 / 12 / 16 / 36 layers
+    // 187 / 274 / 360 / 791 and 191 / 269 / 355 / 772; 4B, 10 / 16 / 36 135 / 208 / 451 and 136 / 205 / 434; 14B, 4 /
+    // 36 layers 167 / 1436 and 168 / 1375 (7 passes per warp are a layer of the 4B model, 13 of the 8B, 24 of the 14B).
+    // 6 % claimed: 8B, 36 layers 785; 15 % 777.  Units claimed while the one before is at work, so that its first record
+    // is not waited for: 779 (a warp then holds one more unit at the end); two or three short units at a time: 14B 1410.
+    // Cut between units, claimed units also make up for unequal ranges, from eight units per warp on (8B, eight layers 204
+    // without and 199 with them; 4B, two layers, 45.5 and 50.2).
+    H->dyn_start = int32_t(units);
+    const bool claimed = inside ? passes >= (long long)kClaimPasses * H->nwarps : units >= 8LL * H->nwarps;
+    if (claimed) {
+        const long long planned = total - total * kDynamicTailPermille / 1000;
+        long long acc = 0;
+        int i = 0;
+        while (i < count - 1 && acc + matrix_work(i) <= planned) acc += matrix_work(i++);
+        long long ds = up[i] + (planned - acc) / full_work(i);
+        if (ds > units) ds = units;
+        H->dyn_start = int32_t(ds);
+        total = acc + (ds - up[i]) * full_work(i);
+    }
+    long long per = (passes + sms - 1) / sms;  // warps of a CTA that have a range: no more than passes
+    if (per > kUnitWarps) per = kUnitWarps;
+    H->warps_per_cta = int32_t(per);
+    const int ranges = int(per) * sms;
+    auto matrix_of = [&](int from, long long uu) {
+        while (from > 0 && up[from] > uu) --from;
+        while (from < count - 1 && up[from + 1] <= uu) ++from;
+        return from;
+    };
+    int pi = 0;
+    long long before = 0;  // work of matrices 0..pi-1
+    for (int w = 0; w < ranges; ++w) {
+        const long long target = total * w / ranges;
+        while (pi < count - 1 && before + matrix_work(pi) <= target) before += matrix_work(pi++);
+        const long long k = (target - before) / full_work(pi);
+        long long uu = up[pi] + k, pass = inside ? (target - before - k * full_work(pi)) / kPassCost : 0;
+        if (pass >= unit_passes(pi, k)) { pass = 0; ++uu; }
+        if (w && inside) {
+            const WarpCut& last = cuts[w - 1];
+            const int last_pass = WarpCut::pass(last.at);
+            if (uu < last.unit || (uu == last.unit && pass <= last_pass && last_pass)) {
+                // fewer passes than ranges: one pass behind the range before
+                uu = last.unit;
+                pass = last_pass + 1;
+                const int pj = matrix_of(WarpCut::matrix(last.at), uu);
+                if (uu >= units || pass >= unit_passes(pj, uu - up[pj])) { ++uu; pass = 0; }
+            }
+        }
+        if (uu >= H->dyn_start) { uu = H->dyn_start; pass = 0; }
+        // (a cut may have moved on from the matrix that its target lies in, or back from it)
+        cuts[w] = WarpCut{int32_t(uu), uint32_t(matrix_of(pi, uu)) << 8 | uint32_t(pass), 0};
+    }
+    H->dyn_matrix = matrix_of(0, H->dyn_start);
+    cuts[ranges] = WarpCut{H->dyn_start, uint32_t(H->dyn_matrix) << 8, 0};
+    // who shares a cut unit: the range before the first that begins inside it, and all that begin inside it
+    size_t slots = 0;
+    for (int w = 1; w < ranges; ++w) {
+        if (!WarpCut::pass(cuts[w].at)) continue;
+        int last = w;
+        while (last + 1 < ranges && cuts[last + 1].unit == cuts[w].unit) ++last;
+        const int i = WarpCut::matrix(cuts[w].at), pieces = last - w + 2;
+        for (int v = w; v <= last; ++v) cuts[v].piece = uint32_t(slots) << 16 | uint32_t(pieces) << 8 | uint32_t(v - w + 1);
+        slots += size_t(pieces) * unit_groups(i, cuts[w].unit - up[i]);
+        w = last;
+    }
+    H->counters = slots ? int32_t(units < ranges ? units : ranges) : 0;
+    return slots;
+}
+
+// The plan of a list for a grid of `sms` CTAs in ws_bytes of workspace: its first `meta` bytes, allocated.  Of these the first
+// that has room: ranges cut inside units of up to three row groups, inside units of one, between units, which takes no slots; no
+// ranges; and of each with aligned columns or without.
+static cudaError_t make_plan(const Problem* problems, int matrices, int sms, size_t ws_bytes, unsigned char** plan, size_t* meta_bytes) {
+    long long exact_cols = 0;
     int count = 0;  // of slices
     for (int i = 0; i < matrices; ++i) {
-        all_cols += size_t(problem_cols(problems[i]));
+        exact_cols += problem_blocks(problems[i]);
         count += problem_slices(problems[i]);
     }
-    const size_t meta = plan_meta_bytes(count, nwarps, all_cols);
-    unsigned char* buf = static_cast<unsigned char*>(calloc(1, meta));
+    const int max_ranges = sms * kUnitWarps;
+    const size_t all = plan_meta_bytes(count, max_ranges, 4 * count);
+    unsigned char* buf = static_cast<unsigned char*>(calloc(1, all));
     if (!buf) return cudaErrorMemoryAllocation;
     PlanHeader* H = reinterpret_cast<PlanHeader*>(buf);
     H->count = count;
-    H->nwarps = nwarps;
     // Matrices whose units are longest come first, so that the units claimed at the end are short (14B, 6 / 16 / 36 layers
-    // 260 / 637 / 1394 -> 242 / 620 / 1375 us; results do not depend on the order).
+    // 260 / 637 / 1394 -> 242 / 620 / 1375 us).
     Problem* problems_host = reinterpret_cast<Problem*>(buf + sizeof(PlanHeader));
     auto longest = [](const Problem& q) {
         const int Bi = problem_blocks(q);
-        return groups_per_unit(Bi) * (Bi / 32) + (Bi % 32 ? 1 : 0);
+        return groups_per_unit(Bi, kMaxRowGroups) * (Bi / 32) + (Bi % 32 ? 1 : 0);
     };
     for (int i = 0, at = 0; i < matrices; ++i)
         for (int k = 0; k < problem_slices(problems[i]); ++k) problems_host[at++] = problem_slice(problems[i], k);
@@ -582,146 +740,108 @@ cudaError_t grouped_plan(const Problem* problems, int matrices, void* ws_dev, si
     H->off_problems = uint32_t(sizeof(PlanHeader));
     H->off_unit_prefix = H->off_problems + uint32_t(count) * uint32_t(sizeof(Problem));
     H->off_col_prefix = H->off_unit_prefix + uint32_t(count + 1) * 4u;
-    H->off_cuts = (H->off_col_prefix + uint32_t(count + 1) * 4u + 15u) & ~15u;
-    H->off_col_start = H->off_cuts + uint32_t(nwarps ? (nwarps + 1) * sizeof(WarpCut) : 0);
-    H->off_counters = uint32_t(plan_meta_bytes(count, kMaxPlanWarps, all_cols));
-    H->off_partials = H->off_counters + uint32_t(kMaxPlanWarps) * 4u;
-    H->off_xq = H->off_counters + uint32_t(kPiecesBytes);
+    H->off_cuts = H->off_col_prefix + uint32_t(count + 1) * 4u;
     int32_t* up = reinterpret_cast<int32_t*>(buf + H->off_unit_prefix);
     int32_t* cp = reinterpret_cast<int32_t*>(buf + H->off_col_prefix);
-    long long units = 0, cols = 0;
-    for (int i = 0; i < count; ++i) {
-        up[i] = int32_t(units);
-        cp[i] = int32_t(cols);
-        units += problem_units(problems_host[i]);
-        if (i + 1 == count || !same_columns(problems_host[i], problems_host[i + 1])) cols += problem_cols(problems_host[i]);
-    }
-    up[count] = int32_t(units);
-    cp[count] = int32_t(cols);
-    if (units > 0x7FFFFFF0LL || cols > 0x7FFFFFF0LL) e = cudaErrorInvalidValue;
-    H->total_units = int32_t(units);
-    H->total_cols = int32_t(cols);
-    if (e == cudaSuccess) {
-        int32_t* start = reinterpret_cast<int32_t*>(buf + H->off_col_start);
-        int i = 0;
-        for (long long c = 0; c < cols; c += kColsPerStart) {
-            while (cp[i + 1] <= c) ++i;
-            start[c / kColsPerStart] = i;
-        }
-    }
-    H->dyn_start = int32_t(units);
-    if (e == cudaSuccess && nwarps) {
-        // Cut the sequence of passes into contiguous ranges of equal work.  A cut inside a unit costs its two sides a store of
-        // sums and an atomic, two of each per warp and run; cut between units only, a list of a few layers leaves most warps
-        // waiting for those with one unit more (4B, one / two / six layers 28.9 / 40.9 / 92.6 us, cut inside units
-        // 24.8 / 39.0 / 87.3; 14B, one layer 59.2 and 51.4).
-        auto unit_passes = [&](int i, long long k) {
-            const int Bi = problem_blocks(problems_host[i]), G = (problems_host[i].N + 7) / 8, R = groups_per_unit(Bi);
-            const int ng = int(G - k * R < R ? G - k * R : R);
-            return ng * (Bi / 32) + (Bi % 32 ? 1 : 0);
-        };
-        auto unit_cost = [&](int i, long long k) {
-            const int G = (problems_host[i].N + 7) / 8, R = groups_per_unit(problem_blocks(problems_host[i]));
-            return (long long)unit_passes(i, k) * kPassCost + kFoldCost * int(G - k * R < R ? G - k * R : R);
-        };
-        auto full_work = [&](int i) { return unit_cost(i, 0); };      // of all units but the last
-        auto matrix_work = [&](int i) {
-            const long long U = problem_units(problems_host[i]);
-            return (U - 1) * full_work(i) + unit_cost(i, U - 1);
-        };
-        long long total = 0, passes = 0;
+    if (exact_cols + 31LL * count > 0x7FFFFFF0LL) { free(buf); return cudaErrorInvalidValue; }
+    auto place_units = [&](int row_groups) {
+        long long units = 0;
         for (int i = 0; i < count; ++i) {
-            const long long U = problem_units(problems_host[i]);
-            total += matrix_work(i);
-            passes += (U - 1) * unit_passes(i, 0) + unit_passes(i, U - 1);
+            up[i] = int32_t(units);
+            units += problem_units(problems_host[i], row_groups);
         }
-        // Of a long list the last tenth of the work is not assigned: warps that finish early claim it unit by unit, which
-        // evens out what the cost model and the warps' unequal speeds leave.  A unit claimed last still makes the others wait
-        // for it, which shorter lists do not make up for.  All assigned / a tenth claimed, us: 8B, 8 / 12 / 16 / 36 layers
-        // 187 / 274 / 360 / 791 and 191 / 269 / 355 / 772; 4B, 10 / 16 / 36 135 / 208 / 451 and 136 / 205 / 434; 14B, 4 /
-        // 36 layers 167 / 1436 and 168 / 1375 (7 passes per warp are a layer of the 4B model, 13 of the 8B, 24 of the 14B).
-        // 6 % claimed: 8B, 36 layers 785; 15 % 777.  Units claimed while the one before is at work, so that its first record
-        // is not waited for: 779 (a warp then holds one more unit at the end); two or three short units at a time: 14B 1410.
-        const bool claimed = passes >= (long long)kClaimPasses * nwarps;
-        if (claimed) {
-            const long long planned = total - total * kDynamicTailPermille / 1000;
-            long long acc = 0;
-            int i = 0;
-            while (i < count - 1 && acc + matrix_work(i) <= planned) acc += matrix_work(i++);
-            long long ds = up[i] + (planned - acc) / full_work(i);
-            if (ds > units) ds = units;
-            H->dyn_start = int32_t(ds);
-            total = acc + (ds - up[i]) * full_work(i);
+        up[count] = H->total_units = int32_t(units);
+        H->row_groups = row_groups;
+        return units <= 0x7FFFFFF0LL;
+    };
+    auto place_columns = [&](bool aligned) {
+        long long cols = 0;
+        for (int i = 0; i < count; ++i) {
+            cp[i] = int32_t(cols);
+            if (i + 1 == count || !same_columns(problems_host[i], problems_host[i + 1])) cols += problem_cols(problems_host[i], aligned);
         }
-        long long per = (passes + sms - 1) / sms;  // warps of a CTA that have a range: no more than passes
-        if (per > kUnitWarps) per = kUnitWarps;
-        H->warps_per_cta = int32_t(per);
-        const int ranges = int(per) * sms;
-        WarpCut* cuts = reinterpret_cast<WarpCut*>(buf + H->off_cuts);
-        int pi = 0;
-        long long before = 0;  // work of matrices 0..pi-1
-        for (int w = 0; w < ranges; ++w) {
-            const long long target = total * w / ranges;
-            while (pi < count - 1 && before + matrix_work(pi) <= target) before += matrix_work(pi++);
-            const long long k = (target - before) / full_work(pi);
-            long long uu = up[pi] + k, pass = (target - before - k * full_work(pi)) / kPassCost;
-            if (pass >= unit_passes(pi, k)) { pass = 0; ++uu; }
-            if (w && (uu < cuts[w - 1].unit || (uu == cuts[w - 1].unit && pass <= cuts[w - 1].pass && cuts[w - 1].pass))) {
-                // fewer passes than ranges: one pass behind the range before
-                uu = cuts[w - 1].unit;
-                pass = cuts[w - 1].pass + 1;
-                int pj = 0;
-                while (pj < count - 1 && up[pj + 1] <= uu) ++pj;
-                if (uu >= units || pass >= unit_passes(pj, uu - up[pj])) { ++uu; pass = 0; }
-            }
-            if (uu >= H->dyn_start) { uu = H->dyn_start; pass = 0; }
-            int pj = pi;  // (a cut may have moved on from the matrix that its target lies in, or back from it)
-            while (pj > 0 && up[pj] > uu) --pj;
-            while (pj < count - 1 && up[pj + 1] <= uu) ++pj;
-            cuts[w] = WarpCut{int32_t(uu), int32_t(pass), w, 1, pj, {0, 0, 0}};
+        cp[count] = H->total_cols = int32_t(cols);
+        H->aligned = aligned;
+    };
+    size_t meta = 0, slots = 0;
+    auto fits = [&](bool aligned) {  // and where everything lies
+        place_columns(aligned);
+        const int ranges = H->warps_per_cta * sms;
+        H->off_col_start = H->off_cuts + uint32_t(ranges ? (ranges + 1) * sizeof(WarpCut) : 0);
+        H->col_shift = col_shift_for(size_t(H->total_cols), count);
+        meta = plan_meta_bytes(count, ranges, (H->total_cols >> H->col_shift) + 1);
+        const size_t bytes = plan_bytes(meta, H->counters, slots, size_t(H->total_cols));
+        H->off_counters = uint32_t(meta);
+        H->off_partials = H->off_counters + uint32_t(H->counters) * 4u;
+        H->off_xq = uint32_t(bytes - size_t(H->total_cols) * kXqBytesPerCol);
+        return bytes <= ws_bytes;
+    };
+    WarpCut* cuts = reinterpret_cast<WarpCut*>(buf + H->off_cuts);
+    bool room = false;
+    for (int way = 0; way < 4 && !room; ++way) {
+        const bool inside = way < 2;
+        if (!place_units(way == 1 ? 1 : kMaxRowGroups)) break;
+        H->nwarps = way < 3 ? max_ranges : 0;
+        if (way < 3) {
+            slots = cut_ranges(H, problems_host, up, cuts, sms, inside);
+        } else {
+            H->warps_per_cta = H->counters = 0;
+            slots = 0;
+            H->dyn_start = H->total_units;
         }
-        int pj = 0;
-        while (pj < count - 1 && up[pj + 1] <= H->dyn_start) ++pj;
-        H->dyn_matrix = pj;
-        cuts[ranges] = WarpCut{H->dyn_start, 0, ranges, 1, pj, {0, 0, 0}};
-        // who shares a cut unit: the range before the first that begins inside it, and all that begin inside it
-        for (int w = 1; w < ranges; ++w) {
-            if (!cuts[w].pass) continue;
-            int last = w;
-            while (last + 1 < ranges && cuts[last + 1].unit == cuts[w].unit) ++last;
-            for (int v = w; v <= last; ++v) { cuts[v].first = w - 1; cuts[v].pieces = last - w + 2; }
-            w = last;
-        }
+        room = slots <= 65536 && (fits(true) || fits(false));
     }
+    if (!room) { free(buf); return cudaErrorInvalidValue; }
+    int32_t* start = reinterpret_cast<int32_t*>(buf + H->off_col_start);
+    for (int c = 0, i = 0; c <= H->total_cols >> H->col_shift; ++c) {
+        while (i < count - 1 && cp[i + 1] <= (long long)c << H->col_shift) ++i;
+        start[c] = i;
+    }
+    *plan = buf;
+    *meta_bytes = meta;
+    return cudaSuccess;
+}
+
+cudaError_t grouped_plan(const Problem* problems, int matrices, void* ws_dev, size_t ws_bytes, cudaStream_t s) {
+    int sms = 0;
+    cudaError_t e = device_sms(&sms);
+    if (e != cudaSuccess) return e;
+    unsigned char* plan = nullptr;
+    size_t meta = 0;
+    e = make_plan(problems, matrices, sms, ws_bytes, &plan, &meta);
+    if (e != cudaSuccess) return e;
     // pageable source: the runtime stages it before returning, so the buffer can be freed
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ws_dev, buf, meta, cudaMemcpyHostToDevice, s);
-    free(buf);
+    e = cudaMemcpyAsync(ws_dev, plan, meta, cudaMemcpyHostToDevice, s);
+    free(plan);
     return e;
 }
 
-size_t single_plan_meta_bytes() { return plan_meta_bytes(1, 0, kSingleCols); }
+size_t single_plan_meta_bytes() { return plan_meta_bytes(1, 0, 1); }
 
 size_t single_plan_scratch_bytes(int blocks_per_row) {
-    return plan_meta_bytes(1, 0, kSingleCols) + size_t((blocks_per_row + 31) & ~31) * kXqBytesPerCol;
+    return single_plan_meta_bytes() + size_t((blocks_per_row + 31) & ~31) * kXqBytesPerCol;
 }
 
 void single_plan_fill(const Problem& problem, unsigned char* meta_host) {
-    memset(meta_host, 0, plan_meta_bytes(1, 0, kSingleCols));
+    memset(meta_host, 0, single_plan_meta_bytes());
     PlanHeader* H = reinterpret_cast<PlanHeader*>(meta_host);
     H->count = 1;
-    H->total_units = problem_units(problem);
-    H->total_cols = int32_t(problem_cols(problem));
+    H->row_groups = kMaxRowGroups;
+    H->aligned = 1;
+    H->total_units = problem_units(problem, kMaxRowGroups);
+    H->total_cols = int32_t(problem_cols(problem, true));
     H->off_problems = uint32_t(sizeof(PlanHeader));
     H->nwarps = 0;  // no unit ranges: the kernel deals units round-robin
     H->off_unit_prefix = H->off_problems + uint32_t(sizeof(Problem));
     H->off_col_prefix = H->off_unit_prefix + 8u;
-    H->off_xq = uint32_t(plan_meta_bytes(1, 0, kSingleCols));
+    H->off_xq = uint32_t(single_plan_meta_bytes());
     memcpy(meta_host + H->off_problems, &problem, sizeof(Problem));
     int32_t* up = reinterpret_cast<int32_t*>(meta_host + H->off_unit_prefix);
     int32_t* cp = reinterpret_cast<int32_t*>(meta_host + H->off_col_prefix);
     up[0] = 0; up[1] = H->total_units;
     cp[0] = 0; cp[1] = H->total_cols;
-    H->off_col_start = H->off_col_prefix + 8u;  // all zeros: one matrix
+    H->off_col_start = H->off_col_prefix + 8u;  // one entry, zero: one matrix
+    H->col_shift = 31;
     H->dyn_start = H->total_units;
 }
 

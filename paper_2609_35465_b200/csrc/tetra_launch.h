@@ -71,8 +71,9 @@ cudaError_t launch_gemv_list(const ListDesc& list, int batch, const void* table,
 
 // Planned list of batch-1 products.  grouped_plan writes descriptors and prefix
 // arrays to the workspace (once per list); grouped_run enqueues the activation
-// pre-pass and the persistent GEMV kernel (every step).
+// pre-pass and the persistent GEMV kernel (every step).  grouped_workspace_least is what grouped_plan takes at least.
 size_t grouped_workspace_bytes(const Problem* problems_host, int count);
+size_t grouped_workspace_least(const Problem* problems_host, int count);
 cudaError_t grouped_plan(const Problem* problems_host, int count, void* ws_dev, size_t ws_bytes, cudaStream_t s);
 cudaError_t grouped_run(void* ws_dev, const void* table, cudaStream_t s);
 

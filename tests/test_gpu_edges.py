@@ -295,3 +295,47 @@ def test_matrix_beyond_64_gigabytes(tt, table, orc, entry, B):
     assert torch.count_nonzero(y) == 0
     del codes
     torch.cuda.empty_cache()
+
+
+def least_workspace(mats):
+    """What a plan has always been given at least: 80 bytes a column, room for the plan, and for a list of at most 65,536 pairs of
+    eight rows and 32 columns what their sums take."""
+    cols = groups = pairs = 0
+    for N, K, tail in mats:
+        B = K // 24 if tail or K % 24 == 0 else -(-K // 24)
+        cols += B
+        groups += -(-N // 8)
+        pairs += -(-N // 8) * -(-B // 32)
+    up = lambda v: -(-v // 256) * 256  # noqa: E731
+    size = up(56 + 72 * len(mats) + 8 + 4 * 8193) + 80 * cols
+    return size if pairs > 65536 else up(size) + 4 * groups + 256 + 32 * pairs
+
+
+# A workspace of that size and not a byte more: ranges cut inside units, between units where the list is too long for the
+# pieces' sums, more matrices than there is room to align.
+@pytest.mark.parametrize("mats", [
+    [(1024, 4096, True)], [(8, 24, True)], [(1, 24 * 3, True)] * 40, [(8, 24 * 5, True)] * 700,
+    [(40, 24 * 700 + 7, True), (3001, 24 * 32, True), (33, 749, False)], [(3000, 24 * 42, True)], [(8 * 32769, 24 * 33, True)],
+    [(8 * 22000 + 3, 24 * 75 + 1, True), (16, 24 * 2047, True)],
+])
+def test_planned_list_in_the_smallest_workspace(tt, table, orc, mats):
+    ms = [make_matrix(86, 1000 * i + N, N, K, tail, batch=1) for i, (N, K, tail) in enumerate(mats)]
+    items = [device_matrix(tt, table, m, torch.from_numpy(m["x"][0]).cuda()) for m in ms]
+    problems = tt.make_problems(items)
+    n = least_workspace(mats)
+    assert n <= tt.tetra_grouped_workspace_bytes(problems)
+    buf = torch.full((n + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+    with pytest.raises(tt.TetraError, match="-6"):
+        tt.tetra_gemv_grouped_plan(problems, buf[:n - 1])
+    tt.tetra_gemv_grouped_plan(problems, buf[:n])
+    for _ in range(2):
+        for it in items:
+            it["y"].fill_(float("nan"))
+        tt.tetra_gemv_grouped_run(buf[:n], table)
+    torch.cuda.synchronize()
+    assert bool((buf[n:] == 0xA5).all())
+    for m, it in list(zip(ms, items))[:12] + list(zip(ms, items))[-1:]:
+        rows = np.unique(np.concatenate([np.arange(0, m["N"], max(1, m["N"] // 4000)), np.arange(max(0, m["N"] - 50), m["N"])]))
+        y = it["y"].cpu().numpy()
+        assert np.isfinite(y).all()
+        assert_gemv_close(y[rows], oracle_product(orc, m, GAIN, rows=rows), "%d x %d" % (m["N"], m["K"]))
