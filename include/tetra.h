@@ -179,7 +179,7 @@ int tetra_gemv_list(const tetra_problem *problems_host, int count, const void *t
  *   tetra_grouped_workspace_bytes  size of the scratch buffer for this list; of a list
  *                                  of more than 65,536 pieces (eight rows x 32 words of
  *                                  a row) 501,760 + 2,480 * count bytes may be left out,
- *                                  which costs such a list up to a sixth of its speed;
+ *                                  which costs some such lists a seventh of their speed;
  *   tetra_gemv_grouped_plan        copies descriptors and index arrays into it
  *                                  (problems_host is read before the call returns);
  *   tetra_gemv_grouped_run         one step: a small pre-pass kernel rewrites the

@@ -233,7 +233,7 @@ static int col_shift_for(size_t cols, int count) {
 // What a caller is asked for.  A list of at most kRoomTasks (row group, column group) pairs is given 32 bytes a pair, which hold
 // the pieces of any cut of units of one row group.  A longer one is given six slots a range and room for aligned columns, but
 // planned without them too: callers may have a workspace of a fixed size, and these were not always asked for (8B, 4 / 8 / 12 /
-// 36 layers 99.8 / 184 / 266 / 764 us, in the smaller workspace 117 / 195 / 273 / 779).
+// 36 layers 98 / 182 / 266 / 764 us, in the smaller workspace 113 / 189 / 265 / 753).
 constexpr long long kRoomTasks = 65536;
 constexpr size_t kCutsRoom = 8193 * 4, kMatrixRoom = 16, kRangesRoom = 2560;  // (2560 ranges: 160 multiprocessors)
 static_assert((kRangesRoom + 1) * sizeof(WarpCut) + sizeof(PlanHeader) - 56 < kCutsRoom, "the cuts have room");
@@ -324,16 +324,14 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
     float* red = reinterpret_cast<float*>(smem + kFastBytes) + warp * kUnitFloats;
     float* sums = red + kRedFloats + lane;  // of row group gi, row lane / 4: this lane's part at 32 gi
     const PlanHeader* H = reinterpret_cast<const PlanHeader*>(ws);
-    const Problem* problems = reinterpret_cast<const Problem*>(ws + H->off_problems);
-    const int32_t* unit_prefix = reinterpret_cast<const int32_t*>(ws + H->off_unit_prefix);
-    const int32_t* col_prefix = reinterpret_cast<const int32_t*>(ws + H->off_col_prefix);
-    const int total_units = H->total_units;
+    const Problem* problems = reinterpret_cast<const Problem*>(ws + sizeof(PlanHeader));
+    auto unit_prefix = [&](int i) { return __ldg(reinterpret_cast<const int32_t*>(ws + H->off_unit_prefix) + i); };
 
     // This warp's share: a contiguous range cut for equal work when the plan holds ranges for this
     // grid (neighbouring warps then walk neighbouring row groups of the same matrices), else every
     // (warps in grid)-th unit.
     const int gw = blockIdx.x * kUnitWarps + warp, nw = gridDim.x * kUnitWarps;
-    int u = gw, u_end = total_units, u_step = nw;
+    int u = gw, u_end = H->total_units, u_step = nw;
     bool claim = false;  // after the range: claim the units from dyn_start on, one at a time
     int pass0 = 0;       // where in its first unit the range begins
     const WarpCut* cut = nullptr;
@@ -345,14 +343,14 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
     uint32_t Bu = 1;
     bool have_record = false;            // the ring already holds the first record of the unit about to start
     auto enter_matrix = [&] {
-        p_end = __ldg(unit_prefix + p + 1);
-        p_begin = __ldg(unit_prefix + p);
+        p_end = unit_prefix(p + 1);
+        p_begin = unit_prefix(p);
         const Problem& Q = problems[p];
         const int K = Q.K;
         Bu = uint32_t(Q.tail ? K / 24 : (K + 23) / 24);
         G = (Q.N + 7) / 8;
         codes_p = static_cast<const uint4*>(Q.codes);
-        x_p = (H->off_xq >> 4) + uint32_t(__ldg(col_prefix + p)) * uint32_t(kXqBytesPerCol / 16);
+        x_p = (H->off_xq >> 4) + uint32_t(__ldg(reinterpret_cast<const int32_t*>(ws + H->off_col_prefix) + p)) * uint32_t(kXqBytesPerCol / 16);
         have_record = false;
     };
     // Code records reach the decoder through a per-warp ring in shared memory: two slots of 3 x 512
@@ -367,11 +365,20 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 512), "l"(codes_p + (at + Bu)));
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 1024), "l"(codes_p + (at + 2 * Bu)));
     };
-    // ahead of the wait: the plan, and the first record of a range that begins in a full column group (both are older than
-    // k_prepare_x, which releases this kernel behind its own wait)
+    // This lane's place in the joint pass over the partial column group of a unit's ng row groups: whether it has one, its
+    // column, and its record from the unit's first.
+    struct Place { bool in; uint32_t col, record; };
+    auto joint_place = [&](int ng) {
+        const int rem = int(Bu & 31u), group = rem ? min(lane / max(rem, 1), 3) : 0;
+        const bool in = rem && group < ng;
+        const uint32_t col = (Bu & ~31u) + (in ? uint32_t(lane - group * rem) : 0u);
+        return Place{in, col, uint32_t(in ? group : 0) * 3u * Bu + col};
+    };
+    // ahead of the wait: the plan, and the range's first record (both are older than k_prepare_x, which releases this kernel
+    // behind its own wait); with a joint pass's too q, k, v of an 8B layer 13.1 -> 12.9 us
     if (H->nwarps == nw) {
         const bool has_range = warp < H->warps_per_cta;
-        u = u_end = total_units;
+        u = u_end = H->total_units;
         u_step = 1;
         if (has_range) {
             cut = reinterpret_cast<const WarpCut*>(ws + H->off_cuts) + (blockIdx.x * H->warps_per_cta + warp);
@@ -379,16 +386,15 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
             u = __ldg(&cut[0].unit);
             pass0 = WarpCut::pass(at);
             u_end = __ldg(&cut[1].unit) + (WarpCut::pass(__ldg(&cut[1].at)) > 0);
-            claim = H->dyn_start < total_units;
+            claim = H->dyn_start < H->total_units;
             if (u < u_end) {
                 p = WarpCut::matrix(at);
                 enter_matrix();
                 const int R = groups_per_unit(int(Bu), H->row_groups), CGf = int(Bu >> 5), g0 = (u - p_begin) * R;
-                const int gi = CGf ? pass0 / CGf : 0;
-                if (CGf && gi < min(R, G - g0)) {
-                    request(slot, uint32_t(g0 + gi) * 3u * Bu + uint32_t(lane + 32 * (pass0 - gi * CGf)));
-                    have_record = true;
-                }
+                const int gi = CGf ? pass0 / CGf : 0, ng = min(R, G - g0);
+                const bool full = CGf && gi < ng;
+                request(slot, uint32_t(g0) * 3u * Bu + (full ? uint32_t(gi) * 3u * Bu + uint32_t(lane + 32 * (pass0 - gi * CGf)) : joint_place(ng).record));
+                have_record = true;
             }
         }
     }
@@ -405,7 +411,7 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
             int c = 0;
             if (lane == 0) c = atomicAdd(&reinterpret_cast<PlanHeader*>(ws)->dyn_next, 1);
             c = __shfl_sync(0xFFFFFFFFu, c, 0);
-            if (c >= total_units) break;
+            if (c >= H->total_units) break;
             u = c;
             u_end = c + 1;
             if (p < H->dyn_matrix) p_end = 0, p = H->dyn_matrix - 1;
@@ -413,7 +419,7 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
             have_record = false;
         }
         if (u >= p_end) {  // first unit, or the walk has left the matrix: units only go up
-            do ++p; while (u >= __ldg(unit_prefix + p + 1));
+            do ++p; while (u >= unit_prefix(p + 1));
             enter_matrix();
         }
         const int CGf = int(Bu >> 5);   // full column groups
@@ -421,12 +427,9 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
         const int R = groups_per_unit(int(Bu), H->row_groups);
         const int g0 = (u - p_begin) * R;
         const int ng = min(R, G - g0);
-        const uint4* codes0 = codes_p + size_t(g0) * 3 * Bu;
-        // this lane's place in the joint pass over the partial column group: row group, column
-        const int lane_grp = rem ? min(lane / max(rem, 1), 3) : 0;
-        const bool lane_in = rem && lane_grp < ng;
-        const uint32_t lane_col = uint32_t(CGf * 32) + (lane_in ? uint32_t(lane - lane_grp * rem) : 0u);
-        const uint4* rem_rec = codes0 + size_t(lane_in ? lane_grp : 0) * 3 * Bu + lane_col;
+        const Place place = joint_place(ng);
+        const bool lane_in = place.in;
+        const uint32_t lane_col = place.col;
         const bool next_unit_here = CGf > 0 && u + u_step < min(u_end, p_end);
 
         // the passes of this unit that the range holds: all of them, unless the range begins or ends inside it
@@ -437,7 +440,7 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
         bool joint = pass0 >= ng * CGf;
         int gi = joint ? 0 : pass0 / CGf;
         const int cg0 = pass0 - gi * CGf;
-        const uint32_t unit0 = uint32_t(g0) * 3u * Bu + uint32_t(lane), unit_rem = uint32_t(rem_rec - codes_p);
+        const uint32_t unit0 = uint32_t(g0) * 3u * Bu + uint32_t(lane), unit_rem = uint32_t(g0) * 3u * Bu + place.record;
         // places are kept as 16-byte units from the matrix's first record, in 32 bits
         uint32_t record = joint ? unit_rem : unit0 + uint32_t(gi) * 3u * Bu + 32u * uint32_t(cg0);  // of the pass at hand
 
@@ -532,6 +535,15 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
         have_record = next_unit_here;
         // A unit that other ranges share: this range's piece goes to the workspace, and the last piece to arrive finds the
         // others there (a counter, nothing waits on it) and adds them in the ranges' order.
+        // What the end of the unit needs is loaded here: the fence behind a piece empties L1, and what is read behind it waits for
+        // L2 one load after the other (1024 x 4096 8.5 -> 8.3 us, 8B pass 766 -> 760).
+        const Problem& Q = problems[p];
+        const int N = Q.N, ntail = Q.tail ? Q.K % 24 : 0, row0 = 8 * g0 + (lane >> 2);
+        const __half *tails = static_cast<const __half*>(Q.tail), *xh = static_cast<const __half*>(Q.x) + 24 * Bu;
+        float* y = Q.y;
+        float scale[kMaxRowGroups];
+#pragma unroll
+        for (int k = 0; k < kMaxRowGroups; ++k) scale[k] = k < ng && row0 + 8 * k < N ? __ldg(Q.row_scales + row0 + 8 * k) : 0.f;
         const WarpCut* shared = pass0 ? cut : (ends_inside ? cut + 1 : nullptr);
         pass0 = 0;
         if (shared) {
@@ -540,6 +552,7 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
             const int pieces = int(info >> 8 & 255u), first = range + int(shared - cut) - int(info & 255u);
             float* all = reinterpret_cast<float*>(ws + H->off_partials) + size_t(info >> 16) * 8 + (lane >> 2);
             float* mine = all + (range - first) * ng * 8;
+            const uint32_t counter = H->off_counters + 4u * uint32_t(H->counters == H->total_units ? u : first);
 #pragma unroll
             for (int k = 0; k < kMaxRowGroups; ++k) {
                 float v = sums[32 * k];
@@ -550,7 +563,7 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
             __threadfence();
             __syncwarp();
             int arrived = 0;
-            if (lane == 0) arrived = atomicAdd(reinterpret_cast<int32_t*>(ws + H->off_counters) + (H->counters == total_units ? u : first), 1);
+            if (lane == 0) arrived = atomicAdd(reinterpret_cast<int32_t*>(ws + counter), 1);
             if (__shfl_sync(0xFFFFFFFFu, arrived, 0) != pieces - 1) continue;
             __threadfence();
             float s0 = 0.f, s1 = 0.f, s2 = 0.f;
@@ -570,23 +583,18 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
             sums[64] = s2;
         }
         // row scale, tail (Sec. 5.1; four lanes per row share the tail), store
-        {
-            const Problem P = problems[p];
-            const int ntail = P.tail ? P.K % 24 : 0;
-            const __half* xh = static_cast<const __half*>(P.x) + 24 * Bu;
-            for (int gk = 0; gk < ng; ++gk) {
-                const int row = (g0 + gk) * 8 + (lane >> 2);
-                float sum = sums[32 * gk];
-                if (row < P.N) {
-                    sum *= __ldg(P.row_scales + row);
-                    const __half* tl = static_cast<const __half*>(P.tail) + size_t(row) * ntail;
-                    for (int k = lane & 3; k < ntail; k += 4)
-                        sum = fmaf(__half2float(tl[k]), __half2float(xh[k]), sum);
-                }
-                sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
-                sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 2);
-                if (row < P.N && (lane & 3) == 0) P.y[row] = sum;
+#pragma unroll
+        for (int gk = 0; gk < kMaxRowGroups; ++gk) {
+            if (gk >= ng) break;
+            const int row = row0 + 8 * gk;
+            float sum = sums[32 * gk] * scale[gk];
+            if (row < N) {
+                const __half* tl = tails + size_t(row) * ntail;
+                for (int k = lane & 3; k < ntail; k += 4) sum = fmaf(__half2float(tl[k]), __half2float(xh[k]), sum);
             }
+            sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
+            sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 2);
+            if (row < N && (lane & 3) == 0) y[row] = sum;
         }
     }
 }
@@ -629,18 +637,27 @@ static size_t cut_ranges(PlanHeader* H, const Problem* problems, const int32_t* 
         const int Bi = problem_blocks(problems[i]);
         return unit_groups(i, k) * (Bi / 32) + (Bi % 32 ? 1 : 0);
     };
-    auto unit_cost = [&](int i, long long k) { return (long long)unit_passes(i, k) * kPassCost + kFoldCost * unit_groups(i, k); };
+    long long passes = 0;
+    for (int i = 0; i < count; ++i) {
+        const long long U = problem_units(problems[i], H->row_groups);
+        passes += (U - 1) * unit_passes(i, 0) + unit_passes(i, U - 1);
+    }
+    long long per = (passes + sms - 1) / sms;  // warps of a CTA that have a range: no more than passes
+    if (per > kUnitWarps) per = kUnitWarps;
+    H->warps_per_cta = int32_t(per);
+    const int ranges = int(per) * sms;
+    // With no more passes than ranges each has its own: cut by cost some warps get two (3072 x 4096 10.1 us instead of 9.6), and a
+    // list of few passes begins in a later CTA (64 x 768 5.3 instead of 5.1).
+    const bool one_each = inside && passes <= ranges;
+    const int fold_cost = one_each ? 0 : kFoldCost;
+    auto unit_cost = [&](int i, long long k) { return (long long)unit_passes(i, k) * kPassCost + fold_cost * unit_groups(i, k); };
     auto full_work = [&](int i) { return unit_cost(i, 0); };      // of all units but the last
     auto matrix_work = [&](int i) {
         const long long U = problem_units(problems[i], H->row_groups);
         return (U - 1) * full_work(i) + unit_cost(i, U - 1);
     };
-    long long total = 0, passes = 0;
-    for (int i = 0; i < count; ++i) {
-        const long long U = problem_units(problems[i], H->row_groups);
-        total += matrix_work(i);
-        passes += (U - 1) * unit_passes(i, 0) + unit_passes(i, U - 1);
-    }
+    long long total = 0;
+    for (int i = 0; i < count; ++i) total += matrix_work(i);
     // Of a long list the last tenth of the work is not assigned: warps that finish early claim it unit by unit, which
     // evens out what the cost model and the warps' unequal speeds leave.  A unit claimed last still makes the others wait
     // for it, which shorter lists do not make up for.  All assigned / a tenth claimed, us: 8B, 8 / 12 / 16 / 36 layers
@@ -662,10 +679,6 @@ static size_t cut_ranges(PlanHeader* H, const Problem* problems, const int32_t* 
         H->dyn_start = int32_t(ds);
         total = acc + (ds - up[i]) * full_work(i);
     }
-    long long per = (passes + sms - 1) / sms;  // warps of a CTA that have a range: no more than passes
-    if (per > kUnitWarps) per = kUnitWarps;
-    H->warps_per_cta = int32_t(per);
-    const int ranges = int(per) * sms;
     auto matrix_of = [&](int from, long long uu) {
         while (from > 0 && up[from] > uu) --from;
         while (from < count - 1 && up[from + 1] <= uu) ++from;
@@ -674,12 +687,12 @@ static size_t cut_ranges(PlanHeader* H, const Problem* problems, const int32_t* 
     int pi = 0;
     long long before = 0;  // work of matrices 0..pi-1
     for (int w = 0; w < ranges; ++w) {
-        const long long target = total * w / ranges;
+        const long long target = one_each ? (w < passes ? w * (long long)kPassCost : total) : total * w / ranges;
         while (pi < count - 1 && before + matrix_work(pi) <= target) before += matrix_work(pi++);
         const long long k = (target - before) / full_work(pi);
         long long uu = up[pi] + k, pass = inside ? (target - before - k * full_work(pi)) / kPassCost : 0;
         if (pass >= unit_passes(pi, k)) { pass = 0; ++uu; }
-        if (w && inside) {
+        if (w && inside && !one_each) {
             const WarpCut& last = cuts[w - 1];
             const int last_pass = WarpCut::pass(last.at);
             if (uu < last.unit || (uu == last.unit && pass <= last_pass && last_pass)) {
@@ -713,12 +726,15 @@ static size_t cut_ranges(PlanHeader* H, const Problem* problems, const int32_t* 
 
 // The plan of a list for a grid of `sms` CTAs in ws_bytes of workspace: its first `meta` bytes, allocated.  Of these the first
 // that has room: ranges cut inside units of up to three row groups, inside units of one, between units, which takes no slots; no
-// ranges; and of each with aligned columns or without.
+// ranges; and of each with aligned columns or without.  A list with no more (row group, column group) pairs than warps begins with
+// the second: a piece for each pair, 6 of a row group of 4096 columns instead of 16 of a unit (units of three: 1024 x 2560 8.6 us,
+// 512 x 4096 8.3; of one 7.5 and 7.6.  Above the line: one layer of the 8B model 33.4 and 36.1, q, k, v of it 12.9 and 13.0).
 static cudaError_t make_plan(const Problem* problems, int matrices, int sms, size_t ws_bytes, unsigned char** plan, size_t* meta_bytes) {
-    long long exact_cols = 0;
+    long long exact_cols = 0, tasks = 0;
     int count = 0;  // of slices
     for (int i = 0; i < matrices; ++i) {
         exact_cols += problem_blocks(problems[i]);
+        tasks += (long long)((problems[i].N + 7) / 8) * ((problem_blocks(problems[i]) + 31) / 32);
         count += problem_slices(problems[i]);
     }
     const int max_ranges = sms * kUnitWarps;
@@ -778,7 +794,7 @@ static cudaError_t make_plan(const Problem* problems, int matrices, int sms, siz
     };
     WarpCut* cuts = reinterpret_cast<WarpCut*>(buf + H->off_cuts);
     bool room = false;
-    for (int way = 0; way < 4 && !room; ++way) {
+    for (int way = tasks <= max_ranges ? 1 : 0; way < 4 && !room; ++way) {
         const bool inside = way < 2;
         if (!place_units(way == 1 ? 1 : kMaxRowGroups)) break;
         H->nwarps = way < 3 ? max_ranges : 0;

@@ -238,6 +238,16 @@ def test_planned_list_ranges(tt, table, orc, mats):
         check(orc, m, y.cpu().numpy(), "%d x %d of %d" % (m["N"], m["K"], len(ms)))
 
 
+# No more pairs of eight rows and 32 columns than warps: units of one row group, and a pass for each range; one pair more; far fewer;
+# ranges that begin in a joint pass.
+@pytest.mark.parametrize("mats", [
+    [(8 * 1184, 24 * 42, True)], [(8 * 1184 + 1, 24 * 42, True)], [(64, 768, True)], [(1024, 2560, True), (8, 24 * 3, True)],
+    [(8 * 147, 24 * 45 + 11, True)], [(512, 24 * 170 + 16, True), (24, 24 * 170 + 16, True), (9, 24 * 700, True)],
+])
+def test_planned_list_of_few_passes(tt, table, orc, mats):
+    test_planned_list_ranges(tt, table, orc, mats)
+
+
 # A plan that the kernel just before the run wrote, over the plan of a run still in flight: nothing of it may be read early.
 def test_plan_written_by_the_kernel_before(tt, table, orc):
     sizes = [[(2048, 24 * 85, True), (17, 24 * 33 + 5, True)], [(40, 24 * 700 + 7, True), (3001, 24 * 32, True), (9, 24 * 5, True)]]
