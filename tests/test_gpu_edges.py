@@ -248,7 +248,7 @@ def test_planned_list_of_few_passes(tt, table, orc, mats):
     test_planned_list_ranges(tt, table, orc, mats)
 
 
-# A plan that the kernel just before the run wrote, over the plan of a run still in flight: nothing of it may be read early.
+# A plan in place of another one between runs, copied by an ordinary kernel (test_gpu_order.py has one that lets the run start early).
 def test_plan_written_by_the_kernel_before(tt, table, orc):
     sizes = [[(2048, 24 * 85, True), (17, 24 * 33 + 5, True)], [(40, 24 * 700 + 7, True), (3001, 24 * 32, True), (9, 24 * 5, True)]]
     plans, items, mats = [], [], []

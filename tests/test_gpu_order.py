@@ -134,3 +134,56 @@ def test_q4_product_behind_packing(tt, N, K, G):
     check(pack, [lambda: tt.tetra_q4_gemv(packed, x, y, N, K, G, 3), lambda: tt.tetra_q4_gemv(packed, x, y, N, K, G, 1),
                  lambda: tt.tetra_q4_list_run(plan, G), lambda: tt.tetra_q4_rows(packed, ids, rows, N, K, G), behind_rows],
           [y, rows])
+
+
+# Writes n 16-byte pieces to `to`, but lets the next kernel of the stream start first and waits for about 50 us (a bounded number of
+# turns) before it does.
+LATE_COPY = """
+extern "C" __global__ void late_copy(const uint4* from, uint4* to, int n) {
+    asm volatile("griddepcontrol.launch_dependents;");
+    const long long begin = clock64();
+    for (int turn = 0; turn < 1000000 && clock64() - begin < 100000; ++turn) {}
+    for (int i = threadIdx.x; i < n; i += blockDim.x) to[i] = from[i];
+}
+"""
+
+
+@pytest.mark.parametrize("shapes", [[(64, 24 * 40)], [(4096, 24 * 42 + 5), (17, 24 * 33 + 5), (3001, 24 * 32)]])
+def test_run_behind_a_kernel_that_writes_the_plan_late(tt, shapes):
+    """Nothing of a plan is read before the kernel that writes it is complete.  The plan that lies there before is of the same shapes,
+    with other matrices, inputs and outputs, all of them valid: a word read too early is only a wrong number.  (That the run's second
+    kernel, which reads the plan ahead of its own wait, is let go only behind the first one's does not show in a run: it finds no
+    registers beside the first.  test_launch_order_source.py reads it from the source.)"""
+    table = tt.tetra_build_table(synth.DEFAULT_GAIN)
+    late_copy = torch.cuda._compile_kernel(LATE_COPY, "late_copy")
+    held, plans, outputs, want = [], [], [], []
+    for which in range(2):
+        items = []
+        for i, (N, K) in enumerate(shapes):
+            seed = 1000 * which + 10 * i
+            packed = tt.tetra_pack_codes(random_bytes(seed, N, K // 24, 6), table, N, K // 24)
+            items.append(dict(codes=packed, row_scales=torch.rand(N, device="cuda"), x=halves(seed + 1, K), N=N, K=K,
+                              tail=halves(seed + 2, N, K % 24) if K % 24 else None, y=torch.zeros(N, device="cuda")))
+        problems = tt.make_problems(items)
+        ws = torch.zeros(-(-tt.tetra_grouped_workspace_bytes(problems) // 16) * 16, dtype=torch.uint8, device="cuda")
+        tt.tetra_gemv_grouped_plan(problems, ws)
+        held.append(items)
+        plans.append(ws)
+        outputs.append([it["y"] for it in items])
+    for ws, ys in zip(plans, outputs):
+        other = ws.clone()
+        tt.tetra_gemv_grouped_run(other, table)
+        torch.cuda.synchronize()
+        want.append([y.clone() for y in ys])
+    shared = plans[0].clone()
+    for turn in range(1, 9):
+        which = turn % 2
+        for ys in outputs:
+            for y in ys:
+                y.fill_(-1.0)
+        torch.cuda.synchronize()
+        late_copy(grid=(1, 1, 1), block=(1024, 1, 1), args=[plans[which], shared, plans[which].numel() // 16])
+        tt.tetra_gemv_grouped_run(shared, table)
+        torch.cuda.synchronize()
+        assert all(torch.equal(y, w) for y, w in zip(outputs[which], want[which])), turn
+        assert all(bool((y == -1.0).all()) for y in outputs[1 - which]), turn

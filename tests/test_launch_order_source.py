@@ -51,6 +51,18 @@ def test_a_kernel_that_releases_its_dependents_waits_for_its_predecessors(name):
     assert "pdl_release" not in body or "pdl_wait" in body
 
 
+def waits_before_it_reads_and_releases(body, workspace):
+    """A kernel whose dependents read the workspace ahead of their own wait: it waits for what wrote it first of all."""
+    return body.index("pdl_wait") < body.index("pdl_release") and workspace not in body[:body.index("pdl_wait")]
+
+
+def test_the_kernel_ahead_of_the_planned_list_waits_before_it_reads_the_plan_or_releases():
+    body = KERNELS["k_prepare_x"][1]
+    assert waits_before_it_reads_and_releases(body, "ws")
+    assert not waits_before_it_reads_and_releases(body.replace("pdl_wait", "X").replace("pdl_release", "pdl_wait").replace("X", "pdl_release"), "ws")
+    assert not waits_before_it_reads_and_releases(body.replace("pdl_wait", "p = ws; pdl_wait"), "ws")
+
+
 def test_no_launch_is_written_for_one_number_of_multiprocessors():
     for f, text in sources():
         assert not re.search(r"\b148\b", text), f
