@@ -18,6 +18,7 @@ using namespace tetra;
 namespace {
 
 constexpr int kNoAllocMaxBlocks = TETRA_NOALLOC_MAX_K / 24;         // words per row
+static_assert(kNoAllocMaxBlocks % 32 == 0, "a plan's columns are rounded up to 32: the largest K has room too");
 constexpr size_t kNoAllocScratchBytes = 256 + size_t(kNoAllocMaxBlocks) * 80;
 
 // Every GPU that loads the library holds this array until the process exits.

@@ -272,6 +272,36 @@ def test_plan_written_by_the_kernel_before(tt, table, orc):
             check(orc, m, it["y"].cpu().numpy(), "%d x %d" % (m["N"], m["K"]))
 
 
+# The largest K of the call that brings its own scratch, both rules; one weight more is refused.
+@pytest.mark.parametrize("K,tail_mode", [(24576, True), (24575, False), (24575, True)])
+def test_noalloc_largest_rows(tt, table, orc, K, tail_mode):
+    m = make_matrix(87, K, 41, K, tail_mode, batch=1)
+    d = device_matrix(tt, table, m, torch.from_numpy(m["x"][0]).cuda())
+    tt.tetra_gemv_noalloc(d["codes"], d["row_scales"], table, d["x"], d["y"], 41, K, d["tail"])
+    torch.cuda.synchronize()
+    check(orc, m, d["y"].cpu().numpy(), "noalloc 41 x %d" % K)
+    p = tt._ptr
+    assert tt.lib().tetra_gemv_noalloc(p(d["codes"]), p(d["row_scales"]), p(table), p(d["x"]), p(d["y"]), 41, tt.NOALLOC_MAX_K + 1,
+                                       None, tt._stream()) == -6
+
+
+# A plan made for a grid of another size deals its units round-robin: here because the number of warps in the plan is overwritten.
+def test_planned_list_dealt_round_robin(tt, table, orc):
+    ms = [make_matrix(88, 1000 * i + N, N, K, tail, batch=1)
+          for i, (N, K, tail) in enumerate([(8 * 2600 + 1, 24 * 32, True), (3001, 24 * 42 + 3, True), (40, 24 * 700 + 7, True), (33, 749, False)])]
+    items = [device_matrix(tt, table, m, torch.from_numpy(m["x"][0]).cuda()) for m in ms]
+    problems = tt.make_problems(items)
+    ws = torch.zeros(-(-tt.tetra_grouped_workspace_bytes(problems) // 4), dtype=torch.int32, device="cuda")
+    tt.tetra_gemv_grouped_plan(problems, ws)
+    warps = torch.cuda.get_device_properties(0).multi_processor_count * 16
+    assert int(ws[5]) == warps and int(ws[1]) > warps  # its warps; its units
+    ws[5] = 0
+    tt.tetra_gemv_grouped_run(ws, table)
+    torch.cuda.synchronize()
+    for m, it in zip(ms, items):
+        check(orc, m, it["y"].cpu().numpy(), "%d x %d" % (m["N"], m["K"]))
+
+
 # One matrix of more than 64 GB: places of records beyond 2^32 sixteen-byte units.  All rows are the origin but the first row
 # group's and the last two's, which lie where a place in 32 bits would wrap around to rows of the beginning.
 @pytest.mark.parametrize("entry,B", [("grouped", 2048), ("noalloc", 1024), ("list", 2048)])
