@@ -176,10 +176,11 @@ int tetra_gemv_list(const tetra_problem *problems_host, int count, const void *t
  * (the tables staged in shared memory once, every warp walking independent
  * eight-row units of the whole list).  The list is planned once and run many
  * times:
- *   tetra_grouped_workspace_bytes  size of the scratch buffer for this list; of a list
- *                                  of more than 65,536 pieces (eight rows x 32 words of
- *                                  a row) 501,760 + 2,480 * count bytes may be left out,
- *                                  which costs some such lists a seventh of their speed;
+ *   tetra_grouped_workspace_bytes  size of the scratch buffer for this list.  A list of
+ *                                  more than 65,536 pieces (eight rows x 32 words of a
+ *                                  row) is planned in less too, down to 80 bytes for
+ *                                  every word of a row of each matrix, 72 a matrix and
+ *                                  33,092; some such lists run a seventh slower then;
  *   tetra_gemv_grouped_plan        copies descriptors and index arrays into it
  *                                  (problems_host is read before the call returns);
  *   tetra_gemv_grouped_run         one step: a small pre-pass kernel rewrites the

@@ -183,7 +183,10 @@ static inline int problem_units(const Problem& q, int row_groups) {
 // to 775 us instead of 765).  A matrix that is larger is planned as slices of this many rows: problems of their own, one behind
 // the other, that share their activation records.
 static inline long long slice_rows(const Problem& q) { return 8 * (0xFFFFFFFELL / (3 * problem_blocks(q)) / 6 * 6); }
-int problem_slices(const Problem& q) { return int((q.N + slice_rows(q) - 1) / slice_rows(q)); }
+int problem_slices(const Problem& q) {
+    if ((q.N + 7LL) / 8 * 3 * problem_blocks(q) < 0x80000000LL) return 1;
+    return int((q.N + slice_rows(q) - 1) / slice_rows(q));
+}
 Problem problem_slice(const Problem& q, int i) {
     const long long rows = slice_rows(q), row0 = i * rows;
     Problem p = q;
@@ -196,7 +199,7 @@ Problem problem_slice(const Problem& q, int i) {
 }
 // b is the slice behind a: its columns are a's
 static inline bool same_columns(const Problem& a, const Problem& b) {
-    return a.N == slice_rows(a) && b.x == a.x && b.K == a.K && !b.tail == !a.tail &&
+    return b.x == a.x && b.K == a.K && !b.tail == !a.tail && a.N == slice_rows(a) &&
            b.codes == static_cast<const char*>(a.codes) + (long long)(a.N / 8) * 48 * problem_blocks(a);
 }
 
@@ -231,24 +234,27 @@ static int col_shift_for(size_t cols, int count) {
 }
 
 // What a caller is asked for.  A list of at most kRoomTasks (row group, column group) pairs is given 32 bytes a pair, which hold
-// the pieces of any cut of units of one row group.  A longer one is given six slots a range and room for aligned columns, but
+// the pieces of any cut of units of one row group.  A longer one is given six slots a range and room for aligned columns (where
+// that is less than a sixteenth of its codes), but
 // planned without them too: callers may have a workspace of a fixed size, and these were not always asked for (8B, 4 / 8 / 12 /
 // 36 layers 98 / 182 / 266 / 764 us, in the smaller workspace 113 / 189 / 265 / 753).
 constexpr long long kRoomTasks = 65536;
 constexpr size_t kCutsRoom = 8193 * 4, kMatrixRoom = 16, kRangesRoom = 2560;  // (2560 ranges: 160 multiprocessors)
 static_assert((kRangesRoom + 1) * sizeof(WarpCut) + sizeof(PlanHeader) - 56 < kCutsRoom, "the cuts have room");
-static size_t workspace_bytes(const Problem* problems, int count, bool slots_of_long_lists) {
-    size_t cols = 0, groups = 0, tasks = 0;
+static size_t workspace_bytes(const Problem* problems, int count, bool room_of_long_lists) {
+    size_t cols = 0, groups = 0, tasks = 0, blocks = 0, padding = 0;
     for (int i = 0; i < count; ++i) {
         const size_t B = size_t(problem_blocks(problems[i])), G = (size_t(problems[i].N) + 7) / 8;
         cols += B;
+        padding += (32 - B % 32) % 32 * kXqBytesPerCol;
+        blocks += G * B;
         groups += G;
         tasks += G * ((B + 31) / 32);
     }
     size_t b = (56 + size_t(count) * (sizeof(Problem) + kMatrixRoom) + 2 * size_t(count + 1) * 4 + kCutsRoom + 255) & ~size_t(255);
     b += cols * kXqBytesPerCol;
     if (tasks <= size_t(kRoomTasks)) b = ((b + 255) & ~size_t(255)) + groups * 4 + 256 + tasks * 32;
-    else if (slots_of_long_lists) b += kRangesRoom * (4 + 6 * 32) + size_t(count) * 31 * kXqBytesPerCol;
+    else if (room_of_long_lists) b += kRangesRoom * (4 + 6 * 32) + (padding <= 3 * blocks ? padding + 256 : 0);
     return b;
 }
 size_t grouped_workspace_bytes(const Problem* problems, int count) { return workspace_bytes(problems, count, true); }
@@ -620,28 +626,25 @@ k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ w
     }
 }
 
+// A matrix as the ranges are cut: units of up to R of its G row groups, each of CG full column groups and perhaps a partial one.
+struct MatrixUnits {
+    int R, G, CG, partial;
+    long long units;
+    int groups(long long k) const { return int(G - k * R < R ? G - k * R : R); }  // of unit k
+    int passes(long long k) const { return groups(k) * CG + partial; }
+};
+
 // Cuts the list's passes into the ranges of the grid's warps; `inside`: also inside units.  Returns the slots that the pieces of
 // cut units take.
-static size_t cut_ranges(PlanHeader* H, const Problem* problems, const int32_t* up, WarpCut* cuts, int sms, bool inside) {
+static size_t cut_ranges(PlanHeader* H, const MatrixUnits* M, const int32_t* up, WarpCut* cuts, int sms, bool inside) {
     const int count = H->count;
     const long long units = H->total_units;
     // Cut the sequence of passes into contiguous ranges of equal work.  A cut inside a unit costs its two sides a store of
     // sums and an atomic, two of each per warp and run; cut between units only, a list of a few layers leaves most warps
     // waiting for those with one unit more (4B, one / two / six layers 28.9 / 40.9 / 92.6 us, cut inside units
     // 24.8 / 39.0 / 87.3; 14B, one layer 59.2 and 51.4).
-    auto unit_groups = [&](int i, long long k) {
-        const int G = (problems[i].N + 7) / 8, R = groups_per_unit(problem_blocks(problems[i]), H->row_groups);
-        return int(G - k * R < R ? G - k * R : R);
-    };
-    auto unit_passes = [&](int i, long long k) {
-        const int Bi = problem_blocks(problems[i]);
-        return unit_groups(i, k) * (Bi / 32) + (Bi % 32 ? 1 : 0);
-    };
     long long passes = 0;
-    for (int i = 0; i < count; ++i) {
-        const long long U = problem_units(problems[i], H->row_groups);
-        passes += (U - 1) * unit_passes(i, 0) + unit_passes(i, U - 1);
-    }
+    for (int i = 0; i < count; ++i) passes += (M[i].units - 1) * M[i].passes(0) + M[i].passes(M[i].units - 1);
     long long per = (passes + sms - 1) / sms;  // warps of a CTA that have a range: no more than passes
     if (per > kUnitWarps) per = kUnitWarps;
     H->warps_per_cta = int32_t(per);
@@ -650,11 +653,10 @@ static size_t cut_ranges(PlanHeader* H, const Problem* problems, const int32_t* 
     // list of few passes begins in a later CTA (64 x 768 5.3 instead of 5.1).
     const bool one_each = inside && passes <= ranges;
     const int fold_cost = one_each ? 0 : kFoldCost;
-    auto unit_cost = [&](int i, long long k) { return (long long)unit_passes(i, k) * kPassCost + fold_cost * unit_groups(i, k); };
-    auto full_work = [&](int i) { return unit_cost(i, 0); };      // of all units but the last
+    auto full_work = [&](int i) { return (long long)M[i].passes(0) * kPassCost + fold_cost * M[i].groups(0); };  // of all units but the last
     auto matrix_work = [&](int i) {
-        const long long U = problem_units(problems[i], H->row_groups);
-        return (U - 1) * full_work(i) + unit_cost(i, U - 1);
+        const long long U = M[i].units;
+        return (U - 1) * full_work(i) + M[i].passes(U - 1) * kPassCost + fold_cost * M[i].groups(U - 1);
     };
     long long total = 0;
     for (int i = 0; i < count; ++i) total += matrix_work(i);
@@ -685,13 +687,24 @@ static size_t cut_ranges(PlanHeader* H, const Problem* problems, const int32_t* 
         return from;
     };
     int pi = 0;
-    long long before = 0;  // work of matrices 0..pi-1
+    long long before = 0, work = matrix_work(0), unit_work = full_work(0);  // work of matrices 0..pi-1, of matrix pi, of its units
+    const long long step = total / ranges, step_rest = total % ranges;
+    long long target = 0, rest = 0;
     for (int w = 0; w < ranges; ++w) {
-        const long long target = one_each ? (w < passes ? w * (long long)kPassCost : total) : total * w / ranges;
-        while (pi < count - 1 && before + matrix_work(pi) <= target) before += matrix_work(pi++);
-        const long long k = (target - before) / full_work(pi);
-        long long uu = up[pi] + k, pass = inside ? (target - before - k * full_work(pi)) / kPassCost : 0;
-        if (pass >= unit_passes(pi, k)) { pass = 0; ++uu; }
+        if (w) {  // total * w / ranges, in steps
+            target += step;
+            if ((rest += step_rest) >= ranges) rest -= ranges, ++target;
+        }
+        if (one_each) target = w < passes ? w * (long long)kPassCost : total;
+        while (pi < count - 1 && before + work <= target) {
+            before += work;
+            work = matrix_work(++pi);
+            unit_work = full_work(pi);
+        }
+        const long long at = target - before;
+        const long long k = at >> 32 ? at / unit_work : uint32_t(at) / uint32_t(unit_work);
+        long long uu = up[pi] + k, pass = inside ? (at - k * unit_work) / kPassCost : 0;
+        if (pass >= M[pi].passes(k)) { pass = 0; ++uu; }
         if (w && inside && !one_each) {
             const WarpCut& last = cuts[w - 1];
             const int last_pass = WarpCut::pass(last.at);
@@ -700,7 +713,7 @@ static size_t cut_ranges(PlanHeader* H, const Problem* problems, const int32_t* 
                 uu = last.unit;
                 pass = last_pass + 1;
                 const int pj = matrix_of(WarpCut::matrix(last.at), uu);
-                if (uu >= units || pass >= unit_passes(pj, uu - up[pj])) { ++uu; pass = 0; }
+                if (uu >= units || pass >= M[pj].passes(uu - up[pj])) { ++uu; pass = 0; }
             }
         }
         if (uu >= H->dyn_start) { uu = H->dyn_start; pass = 0; }
@@ -717,7 +730,7 @@ static size_t cut_ranges(PlanHeader* H, const Problem* problems, const int32_t* 
         while (last + 1 < ranges && cuts[last + 1].unit == cuts[w].unit) ++last;
         const int i = WarpCut::matrix(cuts[w].at), pieces = last - w + 2;
         for (int v = w; v <= last; ++v) cuts[v].piece = uint32_t(slots) << 16 | uint32_t(pieces) << 8 | uint32_t(v - w + 1);
-        slots += size_t(pieces) * unit_groups(i, cuts[w].unit - up[i]);
+        slots += size_t(pieces) * M[i].groups(cuts[w].unit - up[i]);
         w = last;
     }
     H->counters = slots ? int32_t(units < ranges ? units : ranges) : 0;
@@ -726,9 +739,10 @@ static size_t cut_ranges(PlanHeader* H, const Problem* problems, const int32_t* 
 
 // The plan of a list for a grid of `sms` CTAs in ws_bytes of workspace: its first `meta` bytes, allocated.  Of these the first
 // that has room: ranges cut inside units of up to three row groups, inside units of one, between units, which takes no slots; no
-// ranges; and of each with aligned columns or without.  A list with no more (row group, column group) pairs than warps begins with
-// the second: a piece for each pair, 6 of a row group of 4096 columns instead of 16 of a unit (units of three: 1024 x 2560 8.6 us,
-// 512 x 4096 8.3; of one 7.5 and 7.6.  Above the line: one layer of the 8B model 33.4 and 36.1, q, k, v of it 12.9 and 13.0).
+// ranges; and of each with aligned columns or without.  A list with at most two (row group, column group) pairs per warp
+// begins with the second: a piece for each pair, 6 of a row group of 4096 columns instead of 16 of a unit (units of three and of
+// one: 1024 x 2560 8.6 and 7.5 us, 512 x 4096 8.3 and 7.6, 4096 x 4096 12.1 and 10.8, q, k, v of an 8B layer 12.9 and 12.8; above
+// the line one layer of the 8B model 33.4 and 36.1).
 static cudaError_t make_plan(const Problem* problems, int matrices, int sms, size_t ws_bytes, unsigned char** plan, size_t* meta_bytes) {
     long long exact_cols = 0, tasks = 0;
     int count = 0;  // of slices
@@ -739,7 +753,7 @@ static cudaError_t make_plan(const Problem* problems, int matrices, int sms, siz
     }
     const int max_ranges = sms * kUnitWarps;
     const size_t all = plan_meta_bytes(count, max_ranges, 4 * count);
-    unsigned char* buf = static_cast<unsigned char*>(calloc(1, all));
+    unsigned char* buf = static_cast<unsigned char*>(calloc(1, all + size_t(count) * sizeof(MatrixUnits)));
     if (!buf) return cudaErrorMemoryAllocation;
     PlanHeader* H = reinterpret_cast<PlanHeader*>(buf);
     H->count = count;
@@ -751,8 +765,9 @@ static cudaError_t make_plan(const Problem* problems, int matrices, int sms, siz
         return groups_per_unit(Bi, kMaxRowGroups) * (Bi / 32) + (Bi % 32 ? 1 : 0);
     };
     for (int i = 0, at = 0; i < matrices; ++i)
-        for (int k = 0; k < problem_slices(problems[i]); ++k) problems_host[at++] = problem_slice(problems[i], k);
-    std::stable_sort(problems_host, problems_host + count, [&](const Problem& a, const Problem& b) { return longest(a) > longest(b); });
+        for (int k = 0, n = problem_slices(problems[i]); k < n; ++k) problems_host[at++] = n == 1 ? problems[i] : problem_slice(problems[i], k);
+    auto before = [&](const Problem& a, const Problem& b) { return longest(a) > longest(b); };
+    if (!std::is_sorted(problems_host, problems_host + count, before)) std::stable_sort(problems_host, problems_host + count, before);
     H->off_problems = uint32_t(sizeof(PlanHeader));
     H->off_unit_prefix = H->off_problems + uint32_t(count) * uint32_t(sizeof(Problem));
     H->off_col_prefix = H->off_unit_prefix + uint32_t(count + 1) * 4u;
@@ -760,11 +775,14 @@ static cudaError_t make_plan(const Problem* problems, int matrices, int sms, siz
     int32_t* up = reinterpret_cast<int32_t*>(buf + H->off_unit_prefix);
     int32_t* cp = reinterpret_cast<int32_t*>(buf + H->off_col_prefix);
     if (exact_cols + 31LL * count > 0x7FFFFFF0LL) { free(buf); return cudaErrorInvalidValue; }
+    MatrixUnits* M = reinterpret_cast<MatrixUnits*>(buf + all);
     auto place_units = [&](int row_groups) {
         long long units = 0;
         for (int i = 0; i < count; ++i) {
+            const int B = problem_blocks(problems_host[i]), R = groups_per_unit(B, row_groups), G = (problems_host[i].N + 7) / 8;
+            M[i] = MatrixUnits{R, G, B / 32, B % 32 > 0, (G + R - 1) / R};
             up[i] = int32_t(units);
-            units += problem_units(problems_host[i], row_groups);
+            units += M[i].units;
         }
         up[count] = H->total_units = int32_t(units);
         H->row_groups = row_groups;
@@ -794,12 +812,12 @@ static cudaError_t make_plan(const Problem* problems, int matrices, int sms, siz
     };
     WarpCut* cuts = reinterpret_cast<WarpCut*>(buf + H->off_cuts);
     bool room = false;
-    for (int way = tasks <= max_ranges ? 1 : 0; way < 4 && !room; ++way) {
+    for (int way = tasks <= 2LL * max_ranges ? 1 : 0; way < 4 && !room; ++way) {
         const bool inside = way < 2;
         if (!place_units(way == 1 ? 1 : kMaxRowGroups)) break;
         H->nwarps = way < 3 ? max_ranges : 0;
         if (way < 3) {
-            slots = cut_ranges(H, problems_host, up, cuts, sms, inside);
+            slots = cut_ranges(H, M, up, cuts, sms, inside);
         } else {
             H->warps_per_cta = H->counters = 0;
             slots = 0;
