@@ -237,7 +237,7 @@ static int col_shift_for(size_t cols, int count) {
 // the pieces of any cut of units of one row group.  A longer one is given six slots a range and room for aligned columns (where
 // that is less than a sixteenth of its codes), but
 // planned without them too: callers may have a workspace of a fixed size, and these were not always asked for (8B, 4 / 8 / 12 /
-// 36 layers 98 / 182 / 266 / 764 us, in the smaller workspace 113 / 189 / 265 / 753).
+// 36 layers 97 / 181 / 263 / 754 us, in the smaller workspace 117 / 195 / 274 / 781).
 constexpr long long kRoomTasks = 65536;
 constexpr size_t kCutsRoom = 8193 * 4, kMatrixRoom = 16, kRangesRoom = 2560;  // (2560 ranges: 160 multiprocessors)
 static_assert((kRangesRoom + 1) * sizeof(WarpCut) + sizeof(PlanHeader) - 56 < kCutsRoom, "the cuts have room");
@@ -323,9 +323,9 @@ constexpr int kUnitThreads = TETRA_UNIT_THREADS;
 constexpr int kUnitWarps = kUnitThreads / 32;
 constexpr int kUnitFloats = kRedFloats + 96;  // per warp: the transpose buffer, and a sum per row group and lane
 
-// Every warp walks its range of passes.
-template <bool ALIGNED>
-__device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsigned char* smem, uint32_t sm_tab) {
+// Every warp walks its range of passes.  wait: for k_prepare_x.
+template <bool ALIGNED, typename Wait>
+__device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsigned char* smem, uint32_t sm_tab, Wait wait) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float* red = reinterpret_cast<float*>(smem + kFastBytes) + warp * kUnitFloats;
     float* sums = red + kRedFloats + lane;  // of row group gi, row lane / 4: this lane's part at 32 gi
@@ -342,10 +342,10 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
     int pass0 = 0;       // where in its first unit the range begins
     const WarpCut* cut = nullptr;
     int p = -1, p_begin = 0, p_end = 0;  // matrix of the current unit and its range of units
-    // per matrix, kept in registers across its units (everything else is re-read where it is needed)
+    // per matrix, kept in registers across its units (everything else is re-read where it is needed: with the row groups in a
+    // register too the 8B pass takes 764 us instead of 755, with more of these re-read 774)
     const uint4* codes_p = nullptr;
     uint32_t x_p = 0;                    // its activation records, in 16-byte units from the workspace's first byte
-    int G = 1;
     uint32_t Bu = 1;
     bool have_record = false;            // the ring already holds the first record of the unit about to start
     auto enter_matrix = [&] {
@@ -354,7 +354,6 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
         const Problem& Q = problems[p];
         const int K = Q.K;
         Bu = uint32_t(Q.tail ? K / 24 : (K + 23) / 24);
-        G = (Q.N + 7) / 8;
         codes_p = static_cast<const uint4*>(Q.codes);
         x_p = (H->off_xq >> 4) + uint32_t(__ldg(reinterpret_cast<const int32_t*>(ws + H->off_col_prefix) + p)) * uint32_t(kXqBytesPerCol / 16);
         have_record = false;
@@ -397,7 +396,7 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
                 p = WarpCut::matrix(at);
                 enter_matrix();
                 const int R = groups_per_unit(int(Bu), H->row_groups), CGf = int(Bu >> 5), g0 = (u - p_begin) * R;
-                const int gi = CGf ? pass0 / CGf : 0, ng = min(R, G - g0);
+                const int gi = CGf ? pass0 / CGf : 0, ng = min(R, (problems[p].N + 7) / 8 - g0);
                 const bool full = CGf && gi < ng;
                 request(slot, uint32_t(g0) * 3u * Bu + (full ? uint32_t(gi) * 3u * Bu + uint32_t(lane + 32 * (pass0 - gi * CGf)) : joint_place(ng).record));
                 have_record = true;
@@ -405,7 +404,7 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
         }
     }
     asm volatile("cp.async.commit_group;");
-    if (ALIGNED) pdl_wait();  // the activation records (and zeroed counters) come from k_prepare_x
+    wait();  // the activation records (and zeroed counters) come from k_prepare_x
 
     for (;; u += u_step) {
         if (u >= u_end) {
@@ -432,7 +431,7 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
         const int rem = int(Bu & 31);   // columns of the last, partial one
         const int R = groups_per_unit(int(Bu), H->row_groups);
         const int g0 = (u - p_begin) * R;
-        const int ng = min(R, G - g0);
+        const int ng = min(R, (problems[p].N + 7) / 8 - g0);
         const Place place = joint_place(ng);
         const bool lane_in = place.in;
         const uint32_t lane_col = place.col;
@@ -606,7 +605,10 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
 }
 
 // (Out of line: with both copies in the kernel a pass of the 8B model takes 769 us instead of 764.)
-__device__ __noinline__ void walk_unaligned(unsigned char* ws, unsigned char* smem, uint32_t sm_tab) { walk_units<false>(ws, smem, sm_tab); }
+template <typename Wait>
+__device__ __noinline__ void walk_unaligned(unsigned char* ws, unsigned char* smem, uint32_t sm_tab, Wait wait) {
+    walk_units<false>(ws, smem, sm_tab, wait);
+}
 
 // The persistent kernel of a planned list.  All that it needs to know is in the workspace, so a workspace can be copied or moved
 // and still runs correctly: the host needs no record of it.
@@ -618,12 +620,9 @@ k_gemv_units(const DeviceTables* __restrict__ tab, unsigned char* __restrict__ w
     const uint32_t sm_tab = smem_u32(smem);
     __syncthreads();  // the only CTA-wide barrier: the tables are staged (by cp.async, the plan read meanwhile: 783 instead of
                       // 773 us for the 8B pass)
-    if (reinterpret_cast<const PlanHeader*>(ws)->aligned) {
-        walk_units<true>(ws, smem, sm_tab);
-    } else {
-        pdl_wait();
-        walk_unaligned(ws, smem, sm_tab);
-    }
+    const auto wait = [] { pdl_wait(); };
+    if (reinterpret_cast<const PlanHeader*>(ws)->aligned) walk_units<true>(ws, smem, sm_tab, wait);
+    else walk_unaligned(ws, smem, sm_tab, wait);
 }
 
 // A matrix as the ranges are cut: units of up to R of its G row groups, each of CG full column groups and perhaps a partial one.
