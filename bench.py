@@ -30,14 +30,14 @@ UNIT = "GB/s"
 NOMINAL_HBM_GBS = 8000.0
 FALLBACK_HBM_GBS = 6650.0
 # DRAM bytes per algorithmic byte of k_gemv_units, from the ncu capture summarised in
-# profiles/k_gemv_units_qwen3_8b.md (dram__bytes_read.sum + dram__bytes_write.sum = 206.1 MB
+# profiles/k_gemv_units_qwen3_8b.md (dram__bytes_read.sum + dram__bytes_write.sum = 206.9 MB
 # for the 198.4 MB of the first 4 layers; every code byte is read once, so traffic grows in
 # proportion to the matrices read and the full pass is scaled by its byte count).
 TRAFFIC_PER_ALGORITHMIC_BYTE = 1.04
 # Warp-instructions of k_gemv_units per 32 blocks (one block per lane), by pipe, and wavefronts of the
 # shared-memory/L1 data pipe, from the same capture (smsp__inst_executed.sum; the pipes from their shares of peak
 # over the active cycles, times the blocks processed / 32).
-KERNEL_COUNTERS = {"instr": 77.6, "alu": 32.0, "fmaheavy": 32.5, "lsu": 9.8, "wavefronts": 21.5}
+KERNEL_COUNTERS = {"instr": 77.6, "alu": 31.9, "fmaheavy": 33.0, "lsu": 10.0, "wavefronts": 21.7}
 
 
 def issue_bound_gbs(sm_mhz, sms=148):
@@ -384,12 +384,12 @@ def main():
                      "frac": gbs / peak, "peak_kind": peak_kind + " copy bandwidth",
                      "traffic": (None if TRAFFIC_PER_ALGORITHMIC_BYTE is None
                                  else TRAFFIC_PER_ALGORITHMIC_BYTE * dp.algorithmic_bytes),
-                     "limiter": "instruction issue, not HBM: %.1f warp-instructions per 32 blocks (logic/permute "
-                                "pipe %.1f, integer multiply-add pipe %.1f, load/store %.1f; both arithmetic pipes "
-                                "take one warp-instruction every two cycles per SM sub-partition); shared-memory "
-                                "data pipe %.0f wavefronts per 32 blocks" % (
-                                    KERNEL_COUNTERS["instr"], KERNEL_COUNTERS["alu"], KERNEL_COUNTERS["fmaheavy"],
-                                    KERNEL_COUNTERS["lsu"], KERNEL_COUNTERS["wavefronts"]),
+                     "limiter": "shared-memory data pipe, then instruction issue, not HBM: per 32 blocks %.1f wavefronts "
+                                "(one per cycle and SM, shared by four sub-partitions), %.1f warp-instructions (logic/"
+                                "permute pipe %.1f, integer multiply-add pipe %.1f, load/store %.1f; both arithmetic "
+                                "pipes take one every two cycles per sub-partition)" % (
+                                    KERNEL_COUNTERS["wavefronts"], KERNEL_COUNTERS["instr"], KERNEL_COUNTERS["alu"],
+                                    KERNEL_COUNTERS["fmaheavy"], KERNEL_COUNTERS["lsu"]),
                      "issue_bound_gbs": issue_bound_gbs(clocks.get("sm_max_mhz") or 1965),
                      "counters_per_32_blocks": KERNEL_COUNTERS},
         "paper_context": {"L40S_tokens_per_s": [113.8, 95.0, 57.2], "L40S_bits_per_weight": 2.148,

@@ -173,8 +173,8 @@ int tetra_gemv_list(const tetra_problem *problems_host, int count, const void *t
                     void *stream);
 
 /* Batch-1 products of a list of independent matrices from one persistent grid
- * (the tables staged in shared memory once, every warp walking independent
- * eight-row units of the whole list).  The list is planned once and run many
+ * (the tables staged in shared memory once, every warp walking its share of the
+ * whole list).  The list is planned once and run many
  * times:
  *   tetra_grouped_workspace_bytes  size of the scratch buffer for this list.  A list of
  *                                  more than 65,536 pieces (eight rows x 32 words of a
@@ -189,8 +189,11 @@ int tetra_gemv_list(const tetra_problem *problems_host, int count, const void *t
  * workspace_dev: 16-byte aligned device memory owned by the caller; it belongs to
  * the plan until the last run using it has completed, and runs that share a
  * workspace must not overlap on the GPU.  The plan in the workspace describes
- * itself (list, mode, index arrays): a planned workspace may be copied to other
+ * itself (list, shares, index arrays): a planned workspace may be copied to other
  * device memory and run from there, on the device it was planned for.
+ * Runs of one plan give the same bits.  A row's sum over its blocks may be taken in
+ * another order, which shows in the last bits of the float32, where the list, its
+ * order, the size of the workspace or the device's number of multiprocessors differs.
  * tetra_gemv_grouped_plan copies from host memory it frees before returning:
  * call it outside stream capture (tetra_gemv_grouped_run may be captured).
  * tetra_gemv_grouped = plan + run.  Lists of at most TETRA_LIST_MAX matrices are

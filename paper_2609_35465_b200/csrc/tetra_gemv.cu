@@ -5,11 +5,12 @@
 //                 Fig. "decode", FP32 multiply-accumulate, shuffle reduction.
 //                 Kept as a comparison arm and cross-check.
 //   k_gemv_units  the B200 design (also in k_gemv_list, tetra_list.cu): a lane owns one block column and keeps its
-//                 24 activations in registers as 24-bit fixed point (three int8
-//                 planes, power-of-two step per block column, so float16 inputs
+//                 24 activations in registers as 24-bit fixed point (here an int16 and
+//                 an int8 plane, in k_gemv_list three int8 planes; power-of-two step per
+//                 block column, so float16 inputs
 //                 within 2^12 of the column's largest are held exactly); it
 //                 walks the rows, decodes each word into packed int8 with table
-//                 lookups and exclusive ors and multiplies with DP4A: products and the sum over
+//                 lookups and exclusive ors and multiplies with DP2A and DP4A: products and the sum over
 //                 a block are exact integers, one rounding when the block's sum
 //                 becomes a float, FP32 accumulation across blocks.  The ALU
 //                 pipe only unpacks fields; the integer-MAD pipe does the
@@ -17,8 +18,10 @@
 //                 k_gemv_units serves a planned list of matrices from one
 //                 persistent grid: k_prepare_x first writes the fixed-point
 //                 activations of every matrix to the plan's scratch area, then
-//                 every warp walks its own range of units (up to 24 rows of one
-//                 matrix, all columns), and no warp ever waits for another.
+//                 every warp walks its own range of passes (32 columns of eight
+//                 rows), which may begin and end inside a unit (up to 24 rows of
+//                 one matrix, all columns); the last of the warps that share a
+//                 unit adds their sums, and no warp ever waits for another.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -757,7 +760,8 @@ static cudaError_t make_plan(const Problem* problems, int matrices, int sms, siz
     PlanHeader* H = reinterpret_cast<PlanHeader*>(buf);
     H->count = count;
     // Matrices whose units are longest come first, so that the units claimed at the end are short (14B, 6 / 16 / 36 layers
-    // 260 / 637 / 1394 -> 242 / 620 / 1375 us).
+    // 260 / 637 / 1394 -> 242 / 620 / 1375 us).  What a row's sum is made of does not depend on the order, but where a unit is
+    // cut does, and with it the order of its sums: the same plan gives the same bits, another list or order may differ in the last.
     Problem* problems_host = reinterpret_cast<Problem*>(buf + sizeof(PlanHeader));
     auto longest = [](const Problem& q) {
         const int Bi = problem_blocks(q);

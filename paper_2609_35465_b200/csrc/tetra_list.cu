@@ -19,7 +19,8 @@
 //     wait for the predecessor in the stream (programmatic dependent launch) and
 //     waited for only after the image has been built: the decode tables, every
 //     warp's first code record, row scales, tails;
-//   * the image takes a thread per (column, section), eight activations each;
+//   * the image takes a thread per (column, section), eight activations each, as
+//     long as there is a thread for each, and beyond a thread per column;
 //   * the warps split the CTA's passes evenly in memory order, a pass being 32
 //     consecutive (row group, column) cells: where a row ends inside a pass the
 //     next row group's first columns fill the lanes.  A row group is a record's
@@ -217,8 +218,8 @@ k_gemv_list(const DeviceTables* __restrict__ tab, const __grid_constant__ ListPa
         if (s == 0) *reinterpret_cast<float*>(rec + 72) = step;
     };
     // The three sections of column c.  With more sections than threads a thread takes a column and the activations are read
-    // in one round instead of two or three, each of which waits for memory (4096 x 12288 10.1 -> 9.6 us, 5003 x 7001 9.0 ->
-    // 8.7).  Up to a section per thread the shorter chain is the better one (4096 x 4096, 170 columns: image 0.5 us).
+    // in one round instead of two or three, each of which waits for memory (4096 x 12288 9.95 -> 9.49 us, 1024 x 6000
+    // 4.41 -> 4.03, 5003 x 7001 9.07 -> 8.89).  Up to a section per thread the shorter chain is the better one (4096 x 4096, 170 columns: image 0.5 us).
     const bool by_column = 3 * Bu > uint32_t(THREADS);
     auto image_sections = [&](uint32_t c, const uint32_t (&w)[12]) {
         float inv;

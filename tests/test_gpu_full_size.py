@@ -41,7 +41,7 @@ def test_qwen3_8b_full_pass_sampled_rows(orc):
     assert dp.algorithmic_bytes == 1785397248
     picks = list(range(7)) + [7 * 17 + k for k in range(7)] + list(range(245, 252))
     _check_sampled(dp, orc, picks)
-    # rerun: bit-identical (fixed summation order, no atomics)
+    # rerun: bit-identical (fixed summation order: atomics only count arrivals and hand out units)
     dp.run_grouped()
     torch.cuda.synchronize()
     assert np.array_equal(dp.y_all.cpu().numpy()[used], y[used])

@@ -121,7 +121,7 @@ def test_grouped_launch_one_layer(tt, table, orc):
     [(512, 2560, True), (264, 12288, True), (72, 17408, True), (9, 24 * 33, True)],   # a few matrices
     [(1024, 4096, True)],                                                             # a single one
     [(33, 24 * 31 + 5, False), (7, 48, True), (1, 24, True)],                         # tiny and ragged
-    [(40, 49152, True), (3000, 24 * 64, True), (16, 49152 - 24, True)],               # the largest K, coarse mode
+    [(40, 49152, True), (3000, 24 * 64, True), (16, 49152 - 24, True)],               # the largest K, rows of 64 passes
 ])
 def test_grouped_small_lists(tt, table, orc, shapes_list):
     """Small lists, whose units are cut into the warps' ranges (the pieces' sums added in fixed order by the
@@ -264,7 +264,7 @@ def test_gemv_list_rejects_long_lists(tt, table):
 # ---------------------------------------------------------------------------
 @pytest.mark.parametrize("shapes_list", [
     [(1024, 4096, True), (33, 749, False)],                                            # fewer passes than warps
-    [(40, 49152, True), (3000, 24 * 64, True), (16, 49152 - 24, True)],                # coarse mode
+    [(40, 49152, True), (3000, 24 * 64, True), (16, 49152 - 24, True)],                # rows of 64 passes
 ])
 def test_planned_workspace_can_be_copied_to_another_address(tt, table, orc, shapes_list):
     mats = [make_matrix(40, 100 * i + N, N, K, tm) for i, (N, K, tm) in enumerate(shapes_list)]
