@@ -118,7 +118,7 @@ cudaError_t launch_gemv_paper(const void* codes, size_t row_stride, const float*
 // ===========================================================================
 // Planned list of matrices: k_prepare_x + k_gemv_units
 // ===========================================================================
-// Workspace written by grouped_plan (host) and read by both kernels:
+// Workspace, written by grouped_plan (the plan, up to the first pad) and by the kernels:
 //   PlanHeader | Problem[count] | unit_prefix[count + 1] | col_prefix[count + 1] | WarpCut[ranges + 1] (optional) | col_start[]
 //              | pad | counters | partial sums | pad | xq records
 // A unit is groups_per_unit(B) consecutive row groups of one matrix, all columns; a pass is 32 of its columns (or the joint
@@ -145,7 +145,7 @@ struct PlanHeader {
     int32_t dyn_next;
 };
 constexpr int kDynamicTailPermille = 100;  // share of the list's work left for the claimed units
-constexpr int kClaimPasses = 128;          // passes per warp from which on there are claimed units (see grouped_plan)
+constexpr int kClaimPasses = 128;          // passes per warp from which on there are claimed units (see cut_ranges)
 // What the ranges are cut by: a pass, and a row group's fold, row scales and tail.  (With two per unit instead of four per row
 // group the warps that have units of one row group, 16 passes each, finished 8 % before those with units of three.)
 constexpr int kPassCost = 8, kFoldCost = 4;
@@ -238,9 +238,9 @@ static int col_shift_for(size_t cols, int count) {
 
 // What a caller is asked for.  A list of at most kRoomTasks (row group, column group) pairs is given 32 bytes a pair, which hold
 // the pieces of any cut of units of one row group.  A longer one is given six slots a range and room for aligned columns (where
-// that is less than a sixteenth of its codes), but
-// planned without them too: callers may have a workspace of a fixed size, and these were not always asked for (8B, 4 / 8 / 12 /
-// 36 layers 97 / 181 / 263 / 754 us, in the smaller workspace 117 / 195 / 274 / 781).
+// that is less than a sixteenth of its codes), but planned without them too: callers may have a workspace of a fixed size, and
+// these were not always asked for (8B, 4 / 8 / 12 / 36 layers 97 / 181 / 263 / 754 us, in the smaller workspace 117 / 195 /
+// 274 / 781).
 constexpr long long kRoomTasks = 65536;
 constexpr size_t kCutsRoom = 8193 * 4, kMatrixRoom = 16, kRangesRoom = 2560;  // (2560 ranges: 160 multiprocessors)
 static_assert((kRangesRoom + 1) * sizeof(WarpCut) + sizeof(PlanHeader) - 56 < kCutsRoom, "the cuts have room");
@@ -541,8 +541,6 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
             after = behind();
         }
         have_record = next_unit_here;
-        // A unit that other ranges share: this range's piece goes to the workspace, and the last piece to arrive finds the
-        // others there (a counter, nothing waits on it) and adds them in the ranges' order.
         // What the end of the unit needs is loaded here: the fence behind a piece empties L1, and what is read behind it waits for
         // L2 one load after the other (1024 x 4096 8.5 -> 8.3 us, 8B pass 766 -> 760).
         const Problem& Q = problems[p];
@@ -552,6 +550,8 @@ __device__ __forceinline__ void walk_units(unsigned char* __restrict__ ws, unsig
         float scale[kMaxRowGroups];
 #pragma unroll
         for (int k = 0; k < kMaxRowGroups; ++k) scale[k] = k < ng && row0 + 8 * k < N ? __ldg(Q.row_scales + row0 + 8 * k) : 0.f;
+        // A unit that other ranges share: this range's piece goes to the workspace, and the last piece to arrive finds the
+        // others there (a counter, nothing waits on it) and adds them in the ranges' order.
         const WarpCut* shared = pass0 ? cut : (ends_inside ? cut + 1 : nullptr);
         pass0 = 0;
         if (shared) {
