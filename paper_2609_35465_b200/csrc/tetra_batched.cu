@@ -42,7 +42,8 @@
 
 namespace tetra {
 
-constexpr uint32_t kXVec = 4 * 48 + 16;        // bytes per vector of an activation buffer: four columns, a line of zeros
+constexpr uint32_t kXVec = 4 * 48 + 16;        // bytes per vector of an activation buffer: four columns, and a line of zeros
+                                               // or what a row that is not aligned needs more
 constexpr int kBatMaxTiles = 4;                // row tiles of a step
 
 struct BatParams {
@@ -70,6 +71,8 @@ constexpr int bat_together(bool dense, int g, int nt) { return dense && g == 1 &
 // tiles, so one buffer serves (read per tile they were a sixth of the shared-memory traffic, which keeps its pipe 78 %
 // busy: 4096 x 12288, 16 vectors 2 us more).
 constexpr bool bat_hold(bool dense) { return dense; }
+// Block diagonal: two buffers, and one for rows of x as they lie in memory if those are not aligned.
+constexpr uint32_t bat_buffers(bool dense, bool wide) { return bat_hold(dense) ? 1 : (wide ? 2 : 3); }
 // Row stride, in floats, of the partial sums: even, so that pairs stay aligned.
 constexpr int bat_stride(bool dense, int g) { return bat_slots(dense, g) + 2; }
 struct BatSmem {
@@ -77,10 +80,10 @@ struct BatSmem {
     // buffers, then its tiles (dense); the partial sums of all warps take the areas' place at the end.
     uint32_t warps, per_warp, rs, tail, xtail, total;
 };
-constexpr BatSmem bat_smem(bool dense, int g, int nt) {
+constexpr BatSmem bat_smem(bool dense, int g, int nt, bool wide) {
     BatSmem S{};
     S.warps = uint32_t(kFastBytes);
-    S.per_warp = (bat_hold(dense) ? 1u : 2u) * uint32_t(bat_slots(dense, g)) * kXVec + (dense ? uint32_t(bat_together(dense, g, nt)) * kTileBytes : 0u);
+    S.per_warp = bat_buffers(dense, wide) * uint32_t(bat_slots(dense, g)) * kXVec + (dense ? uint32_t(bat_together(dense, g, nt)) * kTileBytes : 0u);
     const uint32_t sums = uint32_t(nt * 16 * bat_stride(dense, g) * 4);  // per warp
     S.rs = S.warps + kBatWarps * (S.per_warp > sums ? S.per_warp : sums);
     S.tail = S.rs + uint32_t(nt) * 64u;                 // half [rows][24]
@@ -88,13 +91,14 @@ constexpr BatSmem bat_smem(bool dense, int g, int nt) {
     S.total = S.xtail + 16u * 96u + kSmAlign;
     return S;
 }
-static_assert(bat_smem(false, 2, 4).total <= 227 * 1024 && bat_smem(true, 1, 4).total <= 227 * 1024 &&
-              bat_smem(true, 2, 4).total <= 227 * 1024, "shared memory");
-template <bool DENSE, int G, int NT>
+static_assert(bat_smem(false, 2, 4, false).total <= 227 * 1024 && bat_smem(true, 1, 4, false).total <= 227 * 1024 &&
+              bat_smem(true, 2, 4, false).total <= 227 * 1024, "shared memory");
+template <bool DENSE, int G, int NT, bool WIDE>
 struct BatShape {
     static constexpr int slots = bat_slots(DENSE, G), together = bat_together(DENSE, G, NT), stride = bat_stride(DENSE, G);
     static constexpr bool hold = bat_hold(DENSE);
-    static constexpr BatSmem smem = bat_smem(DENSE, G, NT);
+    static constexpr uint32_t buffers = bat_buffers(DENSE, WIDE);
+    static constexpr BatSmem smem = bat_smem(DENSE, G, NT, WIDE);
 };
 
 // Half of minus the point, float16 x 2: a[4 s + t] = coordinates 2 t and 2 t + 1 of section s.  Returns the block's scale
@@ -126,29 +130,6 @@ __device__ __forceinline__ float decode_halves(uint32_t sm_tab, uint32_t w0, uin
     return lds32f(uint32_t(__half_as_ushort(m4)) * 2u + (nb.norm0 >> kNormShift) - 0x6400u * 2u);
 }
 
-// Eight consecutive activations starting at x[0], of which `n` exist; x is 2-byte aligned.
-__device__ __forceinline__ uint4 load_eight(const __half* x, int n) {
-    uint32_t w[4] = {0u, 0u, 0u, 0u};
-    const unsigned short* h = reinterpret_cast<const unsigned short*>(x);
-    if (n < 8) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-            if (i < n) w[i >> 1] |= uint32_t(__ldg(h + i)) << (16 * (i & 1));
-    } else if ((reinterpret_cast<uintptr_t>(x) & 3) == 0) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) w[i] = __ldg(reinterpret_cast<const uint32_t*>(x) + i);
-    } else {
-        const uint32_t first = __ldg(h), last = __ldg(h + 7);
-        const uint32_t* mid = reinterpret_cast<const uint32_t*>(h + 1);
-        const uint32_t m0 = __ldg(mid), m1 = __ldg(mid + 1), m2 = __ldg(mid + 2);
-        w[0] = first | (m0 << 16);
-        w[1] = __funnelshift_l(m0, m1, 16);
-        w[2] = __funnelshift_l(m1, m2, 16);
-        w[3] = (m2 >> 16) | (last << 16);
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
 __device__ __forceinline__ void mma_k16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
@@ -171,11 +152,11 @@ __device__ __forceinline__ float cluster_load(uint32_t saddr, uint32_t rank) {
     return v;
 }
 
-// DENSE, G: see bat_slots; NT: row tiles of a step.
-template <bool DENSE, int G, int NT>
+// DENSE, G: see bat_slots; NT: row tiles of a step; WIDE: every row of x is 16-byte aligned.
+template <bool DENSE, int G, int NT, bool WIDE>
 __global__ void __launch_bounds__(kBatThreads, 1)
 k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ BatParams P) {
-    using Shape = BatShape<DENSE, G, NT>;
+    using Shape = BatShape<DENSE, G, NT, WIDE>;
     constexpr int PS = Shape::stride, W = kBatWarps, THREADS = kBatThreads, SLOTS = Shape::slots, TW = Shape::together;
     constexpr BatSmem S = Shape::smem;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -196,7 +177,7 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
     float* xtail = reinterpret_cast<float*>(smem + S.xtail);
     constexpr uint32_t kXBuf = SLOTS * kXVec;
     const uint32_t xbuf = sm_tab + S.warps + uint32_t(warp) * S.per_warp;
-    [[maybe_unused]] const uint32_t tile = xbuf + (Shape::hold ? 1 : 2) * kXBuf;
+    [[maybe_unused]] const uint32_t tile = xbuf + Shape::buffers * kXBuf;
     const int ntail = P.tail ? P.K % 24 : 0, Kx = min(P.K, 24 * P.B);
 
     // This lane's words of a step: rows 2 q and 2 q + 1 of NT tiles at column t.  Rows and columns outside the matrix
@@ -229,27 +210,47 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
     };
     // The activations of a quad's four columns, twelve units of eight per vector, into buffer `slot`; zeros beyond the
     // last column.  Lanes 0..23: unit lane % 12 of every second vector.
-    const bool x_wide = ((reinterpret_cast<uintptr_t>(P.x) | (uintptr_t(P.K) * 2)) & 15) == 0;
     const int x_v = lane >= 12 ? 1 : 0, x_u = lane - 12 * x_v;
-    auto stage_x = [&](uint32_t slot, int quad) {
+    [[maybe_unused]] auto stage_aligned = [&](uint32_t slot, int quad) {
         const int k = 96 * quad + 8 * x_u, n = min(max(Kx - k, 0), 8);
         const __half* src = P.x + (n ? size_t(x_v) * P.K + k : 0);
         const size_t step = n ? 2 * size_t(P.K) : 0;
         const uint32_t dst = xbuf + slot * kXBuf + uint32_t(x_v) * kXVec + uint32_t(x_u) * 16u;
-        if (x_wide) {
 #pragma unroll
-            for (int i = 0; i < SLOTS / 2; ++i, src += step)
-                if (lane < 24 && 2 * i + x_v < V)
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" :: "r"(dst + uint32_t(i) * 2u * kXVec), "l"(src), "r"(2 * n));
-        } else {
-#pragma unroll 1
-            for (int i = 0; 2 * i < V; ++i, src += step)
-                if (lane < 24 && 2 * i + x_v < V) {
-                    const uint4 e = load_eight(src, n);
-                    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" :: "r"(dst + uint32_t(i) * 2u * kXVec), "r"(e.x), "r"(e.y), "r"(e.z), "r"(e.w)
-                                 : "memory");
-                }
+        for (int i = 0; i < SLOTS / 2; ++i, src += step)
+            if (lane < 24 && 2 * i + x_v < V)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" :: "r"(dst + uint32_t(i) * 2u * kXVec), "l"(src), "r"(2 * n));
+    };
+    // Rows of x that are not 16-byte aligned come as they lie in memory, thirteen aligned units: a vector's quad starts
+    // x_skip halves into its part of the buffer, the same for all quads (192 bytes).  The first unit may begin up to seven
+    // halves ahead of the row, within the same 16 bytes; they are not used.  (Loaded, shifted and stored by the lanes, a
+    // pair of vectors after the other, a step waited for memory up to eight times: 5003 x 7001 with 3 / 8 / 16 vectors
+    // 17.8 / 25.3 / 37.7 us, 16.8 / 20.4 / 26.2 this way.)
+    const uint32_t x_half = uint32_t(reinterpret_cast<uintptr_t>(P.x) >> 1);
+    [[maybe_unused]] auto x_skip = [&](int v) { return (x_half + uint32_t(v) * uint32_t(P.K)) & 7u; };
+    [[maybe_unused]] auto stage_raw = [&](uint32_t slot, int quad) {
+        const int v0 = lane >= 13 ? 1 : 0, u = lane - 13 * v0;
+        if (lane < 26) {
+#pragma unroll 2
+            for (int v = v0; v < V; v += 2) {
+                const int skip = int(x_skip(v)), k = 96 * quad + 8 * u - skip, n = min(max(Kx - k, 0), 8);
+                const __half* src = P.x + (ptrdiff_t(v) * P.K + 96 * quad - skip) + 8 * u;
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" :: "r"(xbuf + slot * kXBuf + uint32_t(v) * kXVec + uint32_t(u) * 16u),
+                             "l"(n ? src : P.x - x_skip(0)), "r"(2 * n));
+            }
         }
+    };
+    [[maybe_unused]] constexpr uint32_t kRaw = Shape::hold ? 0u : 2u;  // dense: the fragments are read from where the rows arrive
+    auto stage_x = [&](uint32_t slot, int quad) {
+        if constexpr (WIDE) stage_aligned(slot, quad);
+        else stage_raw(kRaw, quad);
+    };
+    // 32 bits that start `skip` halves on from a word of shared memory
+    [[maybe_unused]] auto lds_from = [&](uint32_t at, uint32_t skip) {
+        uint32_t lo, hi;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(lo) : "r"(at + 4u * (skip >> 1)));
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(hi) : "r"(at + 4u * (skip >> 1) + 4u));
+        return __funnelshift_r(lo, hi, 16u * (skip & 1u));
     };
 
     // ---- before the wait: what does not depend on the activations ------------------------------------------
@@ -270,10 +271,11 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
     // the other lanes (and a vector beyond the last) read a line of zeros.  Dense: word t of a section, of vector q of
     // a group (results beyond the last vector are never used, whatever they are).
     const bool mine = (q >> 1) == t;
+    [[maybe_unused]] const bool x_words = WIDE || ((reinterpret_cast<uintptr_t>(P.x) | (uintptr_t(P.K) * 2)) & 3) == 0;  // fragments are words of the buffer
     uint32_t x_lane[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-        if (DENSE) x_lane[g] = uint32_t(min(8 * g + q, V - 1)) * kXVec + uint32_t(t) * 4u;
+        if (DENSE) x_lane[g] = uint32_t(min(8 * g + q, V - 1)) * kXVec + uint32_t(t) * 4u + (!WIDE && x_words ? 2u * x_skip(min(8 * g + q, V - 1)) : 0u);
         else x_lane[g] = mine && 2 * g + (q & 1) < V ? uint32_t(2 * g + (q & 1)) * kXVec + uint32_t(t) * 48u : 192u;
     }
     const uint32_t x_step = mine ? 16u : 0u;
@@ -319,8 +321,20 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
 #pragma unroll
                     for (int g = 0; g < G; ++g)
 #pragma unroll
-                        for (int s = 0; s < 3; ++s)
-                            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b_held[j][g][s]) : "r"(x_at + x_lane[g] + uint32_t(48 * j + 16 * s)));
+                        for (int s = 0; s < 3; ++s) {
+                            const uint32_t from = x_at + x_lane[g] + uint32_t(48 * j + 16 * s);
+                            if (x_words) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b_held[j][g][s]) : "r"(from));
+                            else b_held[j][g][s] = lds_from(from, x_skip(min(8 * g + q, V - 1)));
+                        }
+                __syncwarp();
+            } else if constexpr (!WIDE) {  // into their places, a lane a word; the next rows then take the ones in memory order
+#pragma unroll
+                for (int i = 0; i < SLOTS * 48 / 32; ++i) {
+                    const int id = lane + 32 * i, v = id / 48, word = id - 48 * v;
+                    if (v < V)
+                        asm volatile("st.shared.u32 [%0], %1;" :: "r"(x_at + uint32_t(v) * kXVec + 4u * uint32_t(word)),
+                                     "r"(lds_from(xbuf + kRaw * kXBuf + uint32_t(v) * kXVec + 4u * uint32_t(word), x_skip(v))) : "memory");
+                }
                 __syncwarp();
             }
             if (quad + W < quad_hi) stage_x(Shape::hold ? 0u : slot ^ 1u, next);
@@ -522,17 +536,18 @@ struct BatKernel {
     void (*run)(const DeviceTables*, BatParams);
     uint32_t smem;
 };
-template <bool DENSE, int G, int NT>
+template <bool DENSE, int G, int NT, bool WIDE>
 constexpr BatKernel bat_kernel() {
-    return {k_gemv_batched<DENSE, G, NT>, BatShape<DENSE, G, NT>::smem.total};
+    return {k_gemv_batched<DENSE, G, NT, WIDE>, BatShape<DENSE, G, NT, WIDE>::smem.total};
 }
-// by vectors (up to 2, 4: block diagonal; 8, 16: dense) and tiles of a step
-const BatKernel kBatKernels[4][kBatMaxTiles] = {
-    {bat_kernel<false, 1, 1>(), bat_kernel<false, 1, 2>(), bat_kernel<false, 1, 3>(), bat_kernel<false, 1, 4>()},
-    {bat_kernel<false, 2, 1>(), bat_kernel<false, 2, 2>(), bat_kernel<false, 2, 3>(), bat_kernel<false, 2, 4>()},
-    {bat_kernel<true, 1, 1>(), bat_kernel<true, 1, 2>(), bat_kernel<true, 1, 3>(), bat_kernel<true, 1, 4>()},
-    {bat_kernel<true, 2, 1>(), bat_kernel<true, 2, 2>(), bat_kernel<true, 2, 3>(), bat_kernel<true, 2, 4>()},
+#define BAT_TILES(dense, g, wide) {bat_kernel<dense, g, 1, wide>(), bat_kernel<dense, g, 2, wide>(), bat_kernel<dense, g, 3, wide>(), bat_kernel<dense, g, 4, wide>()}
+// By alignment of the rows of x, vectors (up to 2, 4: block diagonal; 8, 16: dense) and tiles of a step.  One kernel for
+// aligned and other rows costs the aligned ones registers: 4096 x 12288, 16 vectors, 26.0 us instead of 22.8.
+const BatKernel kBatKernels[2][4][kBatMaxTiles] = {
+    {BAT_TILES(false, 1, false), BAT_TILES(false, 2, false), BAT_TILES(true, 1, false), BAT_TILES(true, 2, false)},
+    {BAT_TILES(false, 1, true), BAT_TILES(false, 2, true), BAT_TILES(true, 1, true), BAT_TILES(true, 2, true)},
 };
+#undef BAT_TILES
 
 }  // namespace
 
@@ -544,9 +559,10 @@ cudaError_t launch_gemv_batched(const void* codes, const float* row_scales, cons
     static PerDeviceOnce once;
     e = once.run([] {
         cudaError_t r = cudaSuccess;
-        for (const auto& row : kBatKernels)
-            for (const BatKernel& k : row)
-                if (r == cudaSuccess) r = cudaFuncSetAttribute(k.run, cudaFuncAttributeMaxDynamicSharedMemorySize, int(k.smem));
+        for (const auto& rows : kBatKernels)
+            for (const auto& row : rows)
+                for (const BatKernel& k : row)
+                    if (r == cudaSuccess) r = cudaFuncSetAttribute(k.run, cudaFuncAttributeMaxDynamicSharedMemorySize, int(k.smem));
         return r;
     });
     if (e != cudaSuccess) return e;
@@ -565,7 +581,8 @@ cudaError_t launch_gemv_batched(const void* codes, const float* row_scales, cons
     const BatPlan plan = plan_batched(P.tiles, P.quads, sms);
     P.groups = plan.groups;
     P.cluster = plan.cluster;
-    const BatKernel& kernel = kBatKernels[batch <= 2 ? 0 : (batch <= 4 ? 1 : (batch <= 8 ? 2 : 3))][plan.nt - 1];
+    const bool wide = ((reinterpret_cast<uintptr_t>(x) | (uintptr_t(K) * 2)) & 15) == 0;
+    const BatKernel& kernel = kBatKernels[wide][batch <= 2 ? 0 : (batch <= 4 ? 1 : (batch <= 8 ? 2 : 3))][plan.nt - 1];
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;

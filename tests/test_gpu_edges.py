@@ -93,6 +93,25 @@ def test_batched_shapes(tt, table, orc, N, K, tail_mode, batch):
         check(orc, m, y[v].cpu().numpy(), "%d x %d, vector %d of %d" % (N, K, v, batch), v)
 
 
+# Rows of x at every 2-byte place of 16 bytes: copied as they lie and shifted on the chip.  Neighbouring values, which the
+# copies bring along, are NaN: none of them may reach a result.
+@pytest.mark.parametrize("batch", [2, 3, 8, 16])
+@pytest.mark.parametrize("K,tail_mode,offset", [(24 * 9, True, 0), (24 * 9, True, 1), (24 * 70 + 4, True, 2), (24 * 70 + 5, True, 3),
+                                                (24 * 70 + 2, False, 6), (24 * 71 + 7, False, 7), (24 * 4, True, 5)])
+def test_batched_unaligned_activations(tt, table, orc, K, tail_mode, offset, batch):
+    N = 41
+    m = make_matrix(77, K + batch, N, K, tail_mode, batch=batch)
+    buf = torch.full((batch * K + 32,), float("nan"), dtype=torch.float16, device="cuda")
+    x = buf[8 + offset:8 + offset + batch * K].view(batch, K)
+    x.copy_(torch.from_numpy(m["x"]))
+    d = device_matrix(tt, table, m, x)
+    y = torch.full((batch, N), float("nan"), dtype=torch.float32, device="cuda")
+    tt.tetra_gemv_batched(d["codes"], d["row_scales"], table, x, y, N, K, batch, d["tail"])
+    torch.cuda.synchronize()
+    for v in range(batch):
+        check(orc, m, y[v].cpu().numpy(), "K %d, offset %d, vector %d of %d" % (K, offset, v, batch), v)
+
+
 @pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
 @pytest.mark.parametrize("batch", [3, 6])
 def test_batched_non_finite_activation(tt, table, bad, batch):
