@@ -39,6 +39,7 @@
 
 #include "q4_common.cuh"
 #include "tetra_gemv_common.cuh"
+#include "tetra_rows.h"
 
 namespace tetra {
 
@@ -222,28 +223,46 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
                 asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" :: "r"(dst + uint32_t(i) * 2u * kXVec), "l"(src), "r"(2 * n));
     };
     // Rows of x that are not 16-byte aligned come as they lie in memory, thirteen aligned units: a vector's quad starts
-    // x_skip halves into its part of the buffer, the same for all quads (192 bytes).  The first unit may begin up to seven
-    // halves ahead of the row, within the same 16 bytes; they are not used.  (Loaded, shifted and stored by the lanes, a
-    // pair of vectors after the other, a step waited for memory up to eight times: 5003 x 7001 with 3 / 8 / 16 vectors
-    // 17.8 / 25.3 / 37.7 us, 16.8 / 20.4 / 26.2 this way.)
+    // x_skip halves into its part of the buffer, the same for all quads.  What the first unit brings along from ahead of
+    // the row is not used.  (Loaded, shifted and stored by the lanes, a pair of vectors after the other, a step waited for
+    // memory up to eight times: 5003 x 7001 with 3 / 8 / 16 vectors 17.8 / 25.3 / 37.7 us, 16.8 / 20.4 / 26.2 this way.)
+    [[maybe_unused]] constexpr uint32_t kRaw = Shape::hold ? 0u : 2u;  // dense: the fragments are read from where the rows arrive
     const uint32_t x_half = uint32_t(reinterpret_cast<uintptr_t>(P.x) >> 1);
-    [[maybe_unused]] auto x_skip = [&](int v) { return (x_half + uint32_t(v) * uint32_t(P.K)) & 7u; };
-    [[maybe_unused]] auto stage_raw = [&](uint32_t slot, int quad) {
-        const int v0 = lane >= 13 ? 1 : 0, u = lane - 13 * v0;
-        if (lane < 26) {
+    [[maybe_unused]] auto x_skip = [&](int v) { return row_skip(x_half, v, P.K); };
+    [[maybe_unused]] const __half* x_unit = P.x + (8u - x_skip(0));  // an aligned address, for copies of nothing
+    [[maybe_unused]] auto stage_raw = [&](int quad, int first_unit) {
+        const int v0 = lane >= kRowUnits ? 1 : 0, u = lane - kRowUnits * v0;
+        if (u >= first_unit && u < kRowUnits) {
 #pragma unroll 2
             for (int v = v0; v < V; v += 2) {
-                const int skip = int(x_skip(v)), k = 96 * quad + 8 * u - skip, n = min(max(Kx - k, 0), 8);
-                const __half* src = P.x + (ptrdiff_t(v) * P.K + 96 * quad - skip) + 8 * u;
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" :: "r"(xbuf + slot * kXBuf + uint32_t(v) * kXVec + uint32_t(u) * 16u),
-                             "l"(n ? src : P.x - x_skip(0)), "r"(2 * n));
+                const RowUnit unit = row_unit(x_skip(v), quad, u, Kx);
+                const __half* src = P.x + (ptrdiff_t(v) * P.K + unit.from);
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" :: "r"(xbuf + kRaw * kXBuf + uint32_t(v) * kXVec + uint32_t(u) * 16u),
+                             "l"(unit.halves ? src : x_unit), "r"(2 * unit.halves));
             }
         }
     };
-    [[maybe_unused]] constexpr uint32_t kRaw = Shape::hold ? 0u : 2u;  // dense: the fragments are read from where the rows arrive
+    // Quad 0 of rows that begin within a unit: the first units half by half, for nothing is read ahead of x.
+    [[maybe_unused]] auto stage_raw_begin = [&] {
+        constexpr int PER = (SLOTS * 8 + 31) / 32;
+        unsigned short begin[PER];
+        const int h = lane & 7;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int v = 4 * i + (lane >> 3), k = h - int(x_skip(v));
+            begin[i] = v < V && k >= 0 && k < Kx ? __half_as_ushort(P.x[size_t(v) * P.K + k]) : (unsigned short)0;
+        }
+        stage_raw(0, 1);
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int v = 4 * i + (lane >> 3);
+            if (v < V)  // zeros ahead of the row: not used
+                asm volatile("st.shared.u16 [%0], %1;" :: "r"(xbuf + kRaw * kXBuf + uint32_t(v) * kXVec + 2u * uint32_t(h)), "h"(begin[i]) : "memory");
+        }
+    };
     auto stage_x = [&](uint32_t slot, int quad) {
         if constexpr (WIDE) stage_aligned(slot, quad);
-        else stage_raw(kRaw, quad);
+        else stage_raw(quad, 0);
     };
     // 32 bits that start `skip` halves on from a word of shared memory
     [[maybe_unused]] auto lds_from = [&](uint32_t at, uint32_t skip) {
@@ -301,7 +320,8 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
             }
         }
         uint32_t slot = 0;
-        if (quad_lo + warp < quad_hi) stage_x(0, quad_lo + warp);
+        if (!WIDE && quad_lo + warp == 0 && rows_begin_within_a_unit(x_half)) stage_raw_begin();
+        else if (quad_lo + warp < quad_hi) stage_x(0, quad_lo + warp);
         if (!DENSE && lane < 2)  // the line of zeros in both buffers
             asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" :: "r"(xbuf + uint32_t(lane) * kXBuf + 192u), "r"(0u) : "memory");
         asm volatile("cp.async.commit_group;");

@@ -112,6 +112,25 @@ def test_batched_unaligned_activations(tt, table, orc, K, tail_mode, offset, bat
         check(orc, m, y[v].cpu().numpy(), "K %d, offset %d, vector %d of %d" % (K, offset, v, batch), v)
 
 
+# Rows shorter than 16 bytes: several begin in the 16 bytes that x begins in.
+@pytest.mark.parametrize("batch", [2, 4, 7, 16])
+@pytest.mark.parametrize("K,offset", [(1, 3), (3, 5), (6, 7)])
+def test_batched_rows_shorter_than_a_unit(tt, table, orc, K, offset, batch):
+    N = 17
+    m = make_matrix(78, K + batch, N, K, False, batch=batch)
+    buf = torch.full((batch * K + 32,), float("nan"), dtype=torch.float16, device="cuda")
+    x = buf[8 + offset:8 + offset + batch * K].view(batch, K)
+    x.copy_(torch.from_numpy(m["x"]))
+    d = device_matrix(tt, table, m, x)
+    y = torch.full((batch, N), float("nan"), dtype=torch.float32, device="cuda")
+    tt.tetra_gemv_batched(d["codes"], d["row_scales"], table, x, y, N, K, batch)
+    torch.cuda.synchronize()
+    for v in range(batch):
+        ref = oracle_product(orc, m, GAIN, batch_index=v)
+        # a row's few coordinates may all be zero: the bound is then zero, and so is the result
+        assert (np.abs(y[v].cpu().numpy() - ref["y"]) <= 1e-5 * ref["abssum"]).all(), "K %d, vector %d of %d" % (K, v, batch)
+
+
 @pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
 @pytest.mark.parametrize("batch", [3, 6])
 def test_batched_non_finite_activation(tt, table, bad, batch):
