@@ -74,6 +74,11 @@ constexpr int bat_together(bool dense, int g, int nt) { return dense && g == 1 &
 constexpr bool bat_hold(bool dense) { return dense; }
 // Block diagonal: two buffers, and one for rows of x as they lie in memory if those are not aligned.
 constexpr uint32_t bat_buffers(bool dense, bool wide) { return bat_hold(dense) ? 1 : (wide ? 2 : 3); }
+// Whether a step asks for the next quad's activations behind its first tile's lookups instead of ahead of them.  Ahead /
+// behind, two vectors, us: one tile 2048 x 2304 3.54 / 3.59, two tiles 4096 x 12288 13.4 / 12.8, 4096 x 4096 7.3 / 7.1, three
+// 5003 x 7008 12.3 / 11.9, four 9000 x 1104 4.77 / 4.72.  With four vectors it is a matter of the tiles and of how the copies
+// are written (4096 x 12288 15.6 / 15.1 in the best form of each, 9728 x 2560 13.6 / 13.8, 2048 x 2304 3.82 / 3.87).
+constexpr bool bat_late(bool dense, int g, int nt, bool wide) { return !dense && wide && g == 1 && nt > 1; }
 // Row stride, in floats, of the partial sums: even, so that pairs stay aligned.
 constexpr int bat_stride(bool dense, int g) { return bat_slots(dense, g) + 2; }
 struct BatSmem {
@@ -99,6 +104,7 @@ struct BatShape {
     static constexpr int slots = bat_slots(DENSE, G), together = bat_together(DENSE, G, NT), stride = bat_stride(DENSE, G);
     static constexpr bool hold = bat_hold(DENSE);
     static constexpr uint32_t buffers = bat_buffers(DENSE, WIDE);
+    static constexpr bool late = bat_late(DENSE, G, NT, WIDE);
     static constexpr BatSmem smem = bat_smem(DENSE, G, NT, WIDE);
 };
 
@@ -164,7 +170,7 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
     pdl_release();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int q = lane >> 2, t = lane & 3;
-    const int V = P.batch, C = P.cluster;
+    const int V = SLOTS == 2 ? 2 : P.batch, C = P.cluster;  // one vector takes another kernel
     const int group = int(blockIdx.x) / C, rank = int(blockIdx.x) - group * C;
     // this CTA's row tiles (shared with its cluster) and column quads
     const int tile_lo = int((long long)group * P.tiles / P.groups), tile_hi = int((long long)(group + 1) * P.tiles / P.groups);
@@ -212,15 +218,32 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
     // The activations of a quad's four columns, twelve units of eight per vector, into buffer `slot`; zeros beyond the
     // last column.  Lanes 0..23: unit lane % 12 of every second vector.
     const int x_v = lane >= 12 ? 1 : 0, x_u = lane - 12 * x_v;
+    // How addresses and tests are written moves the registers of the loops behind, and the time by 1 to 3 %.  Best of those
+    // tried: offsets from x for four vectors (pointers: 5003 x 7008 with three 13.85 us, offsets 13.46), pointers elsewhere;
+    // one test for lane and vector with eight copies (5003 x 7008 with 11 vectors: two tests 18.85, one 18.65).
+    [[maybe_unused]] const __half* x_src = P.x + size_t(x_v) * P.K + 8 * x_u;
+    [[maybe_unused]] const uint32_t x_off = uint32_t(x_v) * uint32_t(P.K) + 8u * uint32_t(x_u);
+    [[maybe_unused]] const int x_left = Kx - 8 * x_u;
+    [[maybe_unused]] const int x_first = SLOTS == 16 && lane >= 24 ? SLOTS : x_v;
     [[maybe_unused]] auto stage_aligned = [&](uint32_t slot, int quad) {
-        const int k = 96 * quad + 8 * x_u, n = min(max(Kx - k, 0), 8);
-        const __half* src = P.x + (n ? size_t(x_v) * P.K + k : 0);
-        const size_t step = n ? 2 * size_t(P.K) : 0;
+        const int k = 96 * quad;
         const uint32_t dst = xbuf + slot * kXBuf + uint32_t(x_v) * kXVec + uint32_t(x_u) * 16u;
+        auto copy = [&](int i, const __half* src, int n) {
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" :: "r"(dst + uint32_t(i) * 2u * kXVec), "l"(src), "r"(2 * n));
+        };
+        if constexpr (SLOTS == 4) {
+            const int n = min(max(x_left - k, 0), 8);
 #pragma unroll
-        for (int i = 0; i < SLOTS / 2; ++i, src += step)
-            if (lane < 24 && 2 * i + x_v < V)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" :: "r"(dst + uint32_t(i) * 2u * kXVec), "l"(src), "r"(2 * n));
+            for (int i = 0; i < SLOTS / 2; ++i)
+                if (lane < 24 && 2 * i + x_v < V) copy(i, P.x + (n ? x_off + uint32_t(k) + uint32_t(2 * i) * uint32_t(P.K) : 0u), n);
+        } else {
+            const int n = min(max(Kx - 8 * x_u - k, 0), 8);
+            const __half* src = n ? x_src + k : P.x;
+            const size_t step = n ? 2 * size_t(P.K) : 0;
+#pragma unroll
+            for (int i = 0; i < SLOTS / 2; ++i, src += step)
+                if ((SLOTS == 16 || lane < 24) && 2 * i + x_first < V) copy(i, src, n);
+        }
     };
     // Rows of x that are not 16-byte aligned come as they lie in memory, thirteen aligned units: a vector's quad starts
     // x_skip halves into its part of the buffer, the same for all quads.  What the first unit brings along from ahead of
@@ -357,8 +380,11 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
                 }
                 __syncwarp();
             }
-            if (quad + W < quad_hi) stage_x(Shape::hold ? 0u : slot ^ 1u, next);
-            asm volatile("cp.async.commit_group;");
+            auto stage_next = [&] {
+                if (quad + W < quad_hi) stage_x(Shape::hold ? 0u : slot ^ 1u, next);
+                asm volatile("cp.async.commit_group;");
+            };
+            if constexpr (!Shape::late) stage_next();
             words_at(t0, next);
             if constexpr (!DENSE) {
 #pragma unroll
@@ -367,6 +393,7 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
                     const float s0 = decode_halves<false>(sm_tab, w0[i].x, w1[i], a[0]);
                     const float s1 = decode_halves<true>(sm_tab, w0[i].y, w1[i], a[1]);
                     load_words(i, t0);
+                    if (Shape::late && i == 0) stage_next();
 #pragma unroll
                     for (int g = 0; g < G; ++g) {
                         float d[4] = {0.f, 0.f, 0.f, 0.f};
