@@ -72,13 +72,16 @@ constexpr int bat_together(bool dense, int g, int nt) { return dense && g == 1 &
 // tiles, so one buffer serves (read per tile they were a sixth of the shared-memory traffic, which keeps its pipe 78 %
 // busy: 4096 x 12288, 16 vectors 2 us more).
 constexpr bool bat_hold(bool dense) { return dense; }
-// Block diagonal: two buffers, and one for rows of x as they lie in memory if those are not aligned.
-constexpr uint32_t bat_buffers(bool dense, bool wide) { return bat_hold(dense) ? 1 : (wide ? 2 : 3); }
+// Block diagonal: two by turns, or, for rows of x that are not aligned, one for them as they lie in memory and one for
+// them in their places: it is filled at the start of a step, when the step before has been read.
+constexpr uint32_t bat_buffers(bool dense) { return bat_hold(dense) ? 1 : 2; }
 // Whether a step asks for the next quad's activations behind its first tile's lookups instead of ahead of them.  Ahead /
 // behind, two vectors, us: one tile 2048 x 2304 3.54 / 3.59, two tiles 4096 x 12288 13.4 / 12.8, 4096 x 4096 7.3 / 7.1, three
 // 5003 x 7008 12.3 / 11.9, four 9000 x 1104 4.77 / 4.72.  With four vectors it is a matter of the tiles and of how the copies
-// are written (4096 x 12288 15.6 / 15.1 in the best form of each, 9728 x 2560 13.6 / 13.8, 2048 x 2304 3.82 / 3.87).
-constexpr bool bat_late(bool dense, int g, int nt, bool wide) { return !dense && wide && g == 1 && nt > 1; }
+// are written (4096 x 12288 15.6 / 15.1 in the best form of each, 9728 x 2560 13.6 / 13.8, 2048 x 2304 3.82 / 3.87).  Rows that
+// are not aligned are put into their places there too: 4096 x 4097 with 2 / 3 vectors 7.8 / 9.2 ahead, 7.4 / 9.1 behind; 700 x 804
+// with three 2.84 and 2.90, 9000 x 1100 6.68 and 6.83.
+constexpr bool bat_late(bool dense, int g, int nt, bool wide) { return !dense && (wide ? g == 1 && nt > 1 : nt == 2); }
 // Row stride, in floats, of the partial sums: even, so that pairs stay aligned.
 constexpr int bat_stride(bool dense, int g) { return bat_slots(dense, g) + 2; }
 struct BatSmem {
@@ -86,10 +89,10 @@ struct BatSmem {
     // buffers, then its tiles (dense); the partial sums of all warps take the areas' place at the end.
     uint32_t warps, per_warp, rs, tail, xtail, total;
 };
-constexpr BatSmem bat_smem(bool dense, int g, int nt, bool wide) {
+constexpr BatSmem bat_smem(bool dense, int g, int nt) {
     BatSmem S{};
     S.warps = uint32_t(kFastBytes);
-    S.per_warp = bat_buffers(dense, wide) * uint32_t(bat_slots(dense, g)) * kXVec + (dense ? uint32_t(bat_together(dense, g, nt)) * kTileBytes : 0u);
+    S.per_warp = bat_buffers(dense) * uint32_t(bat_slots(dense, g)) * kXVec + (dense ? uint32_t(bat_together(dense, g, nt)) * kTileBytes : 0u);
     const uint32_t sums = uint32_t(nt * 16 * bat_stride(dense, g) * 4);  // per warp
     S.rs = S.warps + kBatWarps * (S.per_warp > sums ? S.per_warp : sums);
     S.tail = S.rs + uint32_t(nt) * 64u;                 // half [rows][24]
@@ -97,15 +100,15 @@ constexpr BatSmem bat_smem(bool dense, int g, int nt, bool wide) {
     S.total = S.xtail + 16u * 96u + kSmAlign;
     return S;
 }
-static_assert(bat_smem(false, 2, 4, false).total <= 227 * 1024 && bat_smem(true, 1, 4, false).total <= 227 * 1024 &&
-              bat_smem(true, 2, 4, false).total <= 227 * 1024, "shared memory");
+static_assert(bat_smem(false, 2, 4).total <= 227 * 1024 && bat_smem(true, 1, 4).total <= 227 * 1024 &&
+              bat_smem(true, 2, 4).total <= 227 * 1024, "shared memory");
 template <bool DENSE, int G, int NT, bool WIDE>
 struct BatShape {
     static constexpr int slots = bat_slots(DENSE, G), together = bat_together(DENSE, G, NT), stride = bat_stride(DENSE, G);
     static constexpr bool hold = bat_hold(DENSE);
-    static constexpr uint32_t buffers = bat_buffers(DENSE, WIDE);
+    static constexpr uint32_t buffers = bat_buffers(DENSE);
     static constexpr bool late = bat_late(DENSE, G, NT, WIDE);
-    static constexpr BatSmem smem = bat_smem(DENSE, G, NT, WIDE);
+    static constexpr BatSmem smem = bat_smem(DENSE, G, NT);
 };
 
 // Half of minus the point, float16 x 2: a[4 s + t] = coordinates 2 t and 2 t + 1 of section s.  Returns the block's scale
@@ -249,20 +252,26 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
     // x_skip halves into its part of the buffer, the same for all quads.  What the first unit brings along from ahead of
     // the row is not used.  (Loaded, shifted and stored by the lanes, a pair of vectors after the other, a step waited for
     // memory up to eight times: 5003 x 7001 with 3 / 8 / 16 vectors 17.8 / 25.3 / 37.7 us, 16.8 / 20.4 / 26.2 this way.)
-    [[maybe_unused]] constexpr uint32_t kRaw = Shape::hold ? 0u : 2u;  // dense: the fragments are read from where the rows arrive
+    [[maybe_unused]] constexpr uint32_t kRaw = Shape::hold ? 0u : 1u;  // dense: the fragments are read from where the rows arrive
     const uint32_t x_half = uint32_t(reinterpret_cast<uintptr_t>(P.x) >> 1);
     [[maybe_unused]] auto x_skip = [&](int v) { return row_skip(x_half, v, P.K); };
     [[maybe_unused]] const __half* x_unit = P.x + (8u - x_skip(0));  // an aligned address, for copies of nothing
     [[maybe_unused]] auto stage_raw = [&](int quad, int first_unit) {
         const int v0 = lane >= kRowUnits ? 1 : 0, u = lane - kRowUnits * v0;
-        if (u >= first_unit && u < kRowUnits) {
+        auto copy = [&](int v) {
+            const RowUnit unit = row_unit(x_skip(v), quad, u, Kx);
+            const __half* src = P.x + (ptrdiff_t(v) * P.K + unit.from);
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" :: "r"(xbuf + kRaw * kXBuf + uint32_t(v) * kXVec + uint32_t(u) * 16u),
+                         "l"(unit.halves ? src : x_unit), "r"(2 * unit.halves));
+        };
+        if constexpr (DENSE || NT == 1) {  // a loop is less code ahead of a short launch's only step: 700 x 804 with four vectors 2.80 us, unrolled 2.95
+            if (u >= first_unit && u < kRowUnits)
 #pragma unroll 2
-            for (int v = v0; v < V; v += 2) {
-                const RowUnit unit = row_unit(x_skip(v), quad, u, Kx);
-                const __half* src = P.x + (ptrdiff_t(v) * P.K + unit.from);
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" :: "r"(xbuf + kRaw * kXBuf + uint32_t(v) * kXVec + uint32_t(u) * 16u),
-                             "l"(unit.halves ? src : x_unit), "r"(2 * unit.halves));
-            }
+                for (int v = v0; v < V; v += 2) copy(v);
+        } else {
+#pragma unroll
+            for (int i = 0; i < SLOTS / 2; ++i)
+                if (u >= first_unit && u < kRowUnits && 2 * i + v0 < V) copy(2 * i + v0);
         }
     };
     // Quad 0 of rows that begin within a unit: the first units half by half, for nothing is read ahead of x.
@@ -345,7 +354,7 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
         uint32_t slot = 0;
         if (!WIDE && quad_lo + warp == 0 && rows_begin_within_a_unit(x_half)) stage_raw_begin();
         else if (quad_lo + warp < quad_hi) stage_x(0, quad_lo + warp);
-        if (!DENSE && lane < 2)  // the line of zeros in both buffers
+        if (!DENSE && lane < (WIDE ? 2 : 1))  // the line of zeros in the buffers that fragments are read from
             asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" :: "r"(xbuf + uint32_t(lane) * kXBuf + 192u), "r"(0u) : "memory");
         asm volatile("cp.async.commit_group;");
         if (t0 == tile_lo) {
@@ -370,17 +379,18 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
                             else b_held[j][g][s] = lds_from(from, x_skip(min(8 * g + q, V - 1)));
                         }
                 __syncwarp();
-            } else if constexpr (!WIDE) {  // into their places, a lane a word; the next rows then take the ones in memory order
-#pragma unroll
-                for (int i = 0; i < SLOTS * 48 / 32; ++i) {
-                    const int id = lane + 32 * i, v = id / 48, word = id - 48 * v;
-                    if (v < V)
-                        asm volatile("st.shared.u32 [%0], %1;" :: "r"(x_at + uint32_t(v) * kXVec + 4u * uint32_t(word)),
-                                     "r"(lds_from(xbuf + kRaw * kXBuf + uint32_t(v) * kXVec + 4u * uint32_t(word), x_skip(v))) : "memory");
-                }
-                __syncwarp();
             }
             auto stage_next = [&] {
+                if constexpr (!Shape::hold && !WIDE) {  // into their places, a lane a word; the next rows then take the ones in memory order
+#pragma unroll
+                    for (int i = 0; i < SLOTS * 48 / 32; ++i) {
+                        const int id = lane + 32 * i, v = id / 48, word = id - 48 * v;
+                        if (v < V)
+                            asm volatile("st.shared.u32 [%0], %1;" :: "r"(x_at + uint32_t(v) * kXVec + 4u * uint32_t(word)),
+                                         "r"(lds_from(xbuf + kRaw * kXBuf + uint32_t(v) * kXVec + 4u * uint32_t(word), x_skip(v))) : "memory");
+                    }
+                    __syncwarp();
+                }
                 if (quad + W < quad_hi) stage_x(Shape::hold ? 0u : slot ^ 1u, next);
                 asm volatile("cp.async.commit_group;");
             };
@@ -468,7 +478,7 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
                     __syncwarp();  // the tile has been read before the next blocks overwrite it
                 }
             }
-            if (!Shape::hold) slot ^= 1u;
+            if (!Shape::hold && WIDE) slot ^= 1u;
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();  // everybody has left the buffers and tiles: the sums take their place
