@@ -613,13 +613,14 @@ cudaError_t launch_gemv_batched(const void* codes, const float* row_scales, cons
     int sms = 0;
     cudaError_t e = device_sms(&sms);
     if (e != cudaSuccess) return e;
-    static PerDeviceOnce once;
-    e = once.run([] {
+    // The first call for aligned rows, or for others, loads the sixteen kernels of its kind and not the other sixteen.
+    const bool wide = ((reinterpret_cast<uintptr_t>(x) | (uintptr_t(K) * 2)) & 15) == 0;
+    static PerDeviceOnce once[2];
+    e = once[wide].run([wide] {
         cudaError_t r = cudaSuccess;
-        for (const auto& rows : kBatKernels)
-            for (const auto& row : rows)
-                for (const BatKernel& k : row)
-                    if (r == cudaSuccess) r = cudaFuncSetAttribute(k.run, cudaFuncAttributeMaxDynamicSharedMemorySize, int(k.smem));
+        for (const auto& row : kBatKernels[wide])
+            for (const BatKernel& k : row)
+                if (r == cudaSuccess) r = cudaFuncSetAttribute(k.run, cudaFuncAttributeMaxDynamicSharedMemorySize, int(k.smem));
         return r;
     });
     if (e != cudaSuccess) return e;
@@ -638,7 +639,6 @@ cudaError_t launch_gemv_batched(const void* codes, const float* row_scales, cons
     const BatPlan plan = plan_batched(P.tiles, P.quads, sms);
     P.groups = plan.groups;
     P.cluster = plan.cluster;
-    const bool wide = ((reinterpret_cast<uintptr_t>(x) | (uintptr_t(K) * 2)) & 15) == 0;
     const BatKernel& kernel = kBatKernels[wide][batch <= 2 ? 0 : (batch <= 4 ? 1 : (batch <= 8 ? 2 : 3))][plan.nt - 1];
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

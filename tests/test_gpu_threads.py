@@ -85,3 +85,32 @@ def test_first_calls_from_several_threads_at_once():
     res = subprocess.run([sys.executable, "-c", CHILD], capture_output=True, text=True, timeout=600)
     assert res.returncode == 0, res.stdout[-2000:] + res.stderr[-4000:]
     assert "THREADS-OK" in res.stdout
+
+FIRST_IN_CAPTURE = textwrap.dedent('''
+    import torch
+    from paper_2609_35465_b200 import synth, tetra as tt
+    table = tt.tetra_build_table(synth.DEFAULT_GAIN)
+    N, K, V = 40, 24 * 9 + 1, 3
+    codes = tt.tetra_pack_codes(torch.from_numpy(synth.codes(82, 0, N, 9)).cuda(), table, N, 9)
+    scales = torch.ones(N, device="cuda")
+    tail = torch.ones((N, 1), dtype=torch.float16, device="cuda")
+    x = torch.randn((V, K), device="cuda").half()
+    y, z, ws = torch.zeros((V, N), device="cuda"), torch.zeros((V, N), device="cuda"), torch.empty(tt.tetra_batched_workspace_bytes(N, K), dtype=torch.uint8, device="cuda")
+    xa = torch.randn((V, K - 1), device="cuda").half()
+    tt.tetra_gemv_batched(codes, scales, table, xa, y, N, K - 1, V, None, ws)   # rows that are 16-byte aligned
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        tt.tetra_gemv_batched(codes, scales, table, x, y, N, K, V, tail, ws)    # and others
+    graph.replay()
+    tt.tetra_gemv_batched(codes, scales, table, x, z, N, K, V, tail, ws)
+    torch.cuda.synchronize()
+    assert torch.equal(y, z) and bool(y.any())
+    print("captured")
+''')
+
+
+def test_the_first_call_for_rows_that_are_not_aligned_may_be_captured():
+    """Its set-up is its own, apart from that of the calls for aligned rows before it."""
+    res = subprocess.run([sys.executable, "-c", FIRST_IN_CAPTURE], capture_output=True, text=True, timeout=600)
+    assert res.returncode == 0 and "captured" in res.stdout, res.stdout + res.stderr
