@@ -93,8 +93,9 @@ def test_batched_shapes(tt, table, orc, N, K, tail_mode, batch):
         check(orc, m, y[v].cpu().numpy(), "%d x %d, vector %d of %d" % (N, K, v, batch), v)
 
 
-# Rows of x at every 2-byte place of 16 bytes: copied as they lie and shifted on the chip.  Neighbouring values, which the
-# copies bring along, are NaN: none of them may reach a result.
+# Rows of x at every 2-byte place of 16 bytes: copied as they lie and shifted on the chip.  What lies around x is NaN and may
+# not reach a result.  (What the copies bring along ahead of a vector is the end of the one before: see the non-finite
+# activations below.)
 @pytest.mark.parametrize("batch", [2, 3, 8, 16])
 @pytest.mark.parametrize("K,tail_mode,offset", [(24 * 9, True, 0), (24 * 9, True, 1), (24 * 70 + 4, True, 2), (24 * 70 + 5, True, 3),
                                                 (24 * 70 + 2, False, 6), (24 * 71 + 7, False, 7), (24 * 4, True, 5)])
@@ -142,6 +143,67 @@ def test_batched_non_finite_activation(tt, table, bad, batch):
     tt.tetra_gemv_batched(d["codes"], d["row_scales"], table, x, y, 70, 24 * 20, batch)
     torch.cuda.synchronize()
     assert torch.isnan(y[1]).all() and torch.isfinite(y[0]).all() and torch.isfinite(y[2:]).all()
+
+
+# The same in rows that are not 16-byte aligned, where a copy brings the end of a vector along ahead of the next: first and
+# last activation of a vector in the middle, and one that two quads of columns share a copy of.
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("place", [0, 96, 24 * 20 + 4])
+@pytest.mark.parametrize("batch", [3, 4, 6, 16])
+def test_batched_non_finite_activation_in_unaligned_rows(tt, table, bad, place, batch):
+    N, K = 70, 24 * 20 + 5
+    m = make_matrix(79, batch, N, K, False, batch=batch)
+    for offset in (0, 3):
+        buf = torch.zeros(batch * K + 16, dtype=torch.float16, device="cuda")
+        x = buf[offset:offset + batch * K].view(batch, K)
+        x.copy_(torch.from_numpy(m["x"]))
+        x[1, place] = bad
+        d = device_matrix(tt, table, m, x)
+        y = torch.zeros((batch, N), dtype=torch.float32, device="cuda")
+        tt.tetra_gemv_batched(d["codes"], d["row_scales"], table, x, y, N, K, batch)
+        torch.cuda.synchronize()
+        assert torch.isnan(y[1]).all() and torch.isfinite(y[0]).all() and torch.isfinite(y[2:]).all()
+
+
+# Rows of x that are not 16-byte aligned have kernels of their own: two, three and four row tiles a step for each class of
+# vectors, three steps to a warp, and a second round of rows (six tiles to a CTA are two rounds of three).  The tiles follow
+# from the rows; with 41 quads of columns a CTA has them to itself.  x at a 2-byte and at a 4-byte place: dense fragments are
+# shifted or read as words.  Then a cluster of two CTAs (few rows, many columns).  Sampled rows, every vector.
+_MATRICES = {}
+
+
+def sampled_batched(tt, table, orc, N, K, offset, batch):
+    if (N, K) not in _MATRICES:
+        m = make_matrix(80, N + K, N, K, True, batch=16)
+        _MATRICES[N, K] = m, device_matrix(tt, table, m, None)
+    m, d = _MATRICES[N, K]
+    buf = torch.full((batch * K + 16,), float("nan"), dtype=torch.float16, device="cuda")
+    x = buf[offset:offset + batch * K].view(batch, K)
+    x.copy_(torch.from_numpy(m["x"][:batch]))
+    y = torch.full((batch, N), float("nan"), dtype=torch.float32, device="cuda")
+    tt.tetra_gemv_batched(d["codes"], d["row_scales"], table, x, y, N, K, batch, d["tail"])
+    torch.cuda.synchronize()
+    yh = y.cpu().numpy()
+    assert np.isfinite(yh).all()
+    rows = np.unique([r for r in (0, 15, 16, 31, 32, 47, 48, 63, N // 2, N - 17, N - 16, N - 1) if 0 <= r < N])
+    for v in range(batch):
+        ref = oracle_product(orc, m, GAIN, rows=rows, batch_index=v, threads=4)
+        assert_gemv_close(yh[v][rows], ref, "%d x %d, offset %d, vector %d of %d" % (N, K, offset, v, batch))
+        assert np.max(np.abs(yh[v][rows] - ref["y"]) / ref["abssum"]) < 1e-5
+
+
+@pytest.mark.parametrize("K,offset", [(24 * 162 + 5, 3), (24 * 162 + 4, 2)])
+@pytest.mark.parametrize("tiles", [2, 3, 4, 6])
+@pytest.mark.parametrize("batch", [2, 4, 7, 16])
+def test_batched_unaligned_tiles(tt, table, orc, tiles, K, offset, batch):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    sampled_batched(tt, table, orc, 16 * sms * (tiles - 1) + 17, K, offset, batch)
+
+
+@pytest.mark.parametrize("K,offset", [(24 * 600 + 1, 0), (24 * 600 + 4, 0), (24 * 600, 5)])
+@pytest.mark.parametrize("batch", [2, 4, 7, 16])
+def test_batched_unaligned_cluster(tt, table, orc, K, offset, batch):
+    sampled_batched(tt, table, orc, 64, K, offset, batch)
 
 
 # Copies out of 16, 8 and 4 bytes (odd block counts, outputs that are not aligned), part-filled row groups and columns.
