@@ -554,6 +554,8 @@ size_t batched_workspace_bytes(int N, int blocks_per_row) {
 
 namespace {
 
+constexpr int kBatMaxCluster = 2;
+static_assert(kBatMaxCluster <= kNormClusterMax, "the scale tables' addresses");
 struct BatPlan {
     int cluster = 1, groups = 1, nt = 1;
 };
@@ -571,7 +573,7 @@ struct BatPlan {
 BatPlan plan_batched(int tiles, int quads, int sms) {
     BatPlan best;
     double best_cost = 1e30;
-    for (int c = 1; c <= 2; c *= 2) {
+    for (int c = 1; c <= kBatMaxCluster; c *= 2) {
         const int room = sms / c;
         if (c > quads || room == 0) break;
         BatPlan p;

@@ -153,6 +153,10 @@ constexpr uint32_t kSmMaskXp = 24960;
 constexpr uint32_t kSmGap = 25088, kStagedGap = 512;  // nothing to stage there
 constexpr uint32_t kScaleGain = 1024;  // from one gain's scale table to the other's
 constexpr int kNormShift = 7;          // from the squared norm of eight times the point (1024 m) to bytes of a scale table
+// In a cluster a shared-memory address holds the CTA's rank from bit 24 on.  NibbleBlock::norm0 keeps an address shifted left,
+// so only the rank's lowest bits are left in it: with more CTAs the lookups would go to another CTA's copy of the table (the
+// same entries, through the cluster's network).
+constexpr int kNormClusterMax = 1 << (32 - 24 - kNormShift);
 constexpr uint32_t kSmAlign = 16384;  // the staged copy starts on a 16 KiB boundary of shared memory
 static_assert(kSmMid == offsetof(DeviceTables, mid_fast) - kFastOffset, "staged layout");
 static_assert(kSmScale == offsetof(DeviceTables, scale) - kFastOffset, "staged layout");
@@ -206,7 +210,7 @@ static_assert(fast_nibble(word_coordinate(0, 1)) == 3 && fast_nibble(word_coordi
 struct NibbleBlock {
     uint32_t z[3];  // section s: coordinate j's z at bits 4 fast_nibble(j)
     uint32_t p4;    // bit 2: p (the other bits are an address)
-    uint32_t norm0; // 128 times the shared-memory address of the gain's scale table
+    uint32_t norm0; // 128 times the shared-memory address of the gain's scale table; clusters: kNormClusterMax
 };
 // HI = false: w1 sits in bits 0..15 of `w1pair`; HI = true: in bits 16..31.
 // sm_tab: shared-memory address of the staged tables, a multiple of 16 KiB, so

@@ -66,3 +66,13 @@ def test_the_kernel_ahead_of_the_planned_list_waits_before_it_reads_the_plan_or_
 def test_no_launch_is_written_for_one_number_of_multiprocessors():
     for f, text in sources():
         assert not re.search(r"\b148\b", text), f
+
+
+def test_clusters_stay_within_what_the_scale_tables_addresses_hold():
+    """A shared-memory address of a cluster's CTA holds its rank from bit 24 on; the decoder keeps one shifted left."""
+    text = "".join(t for _, t in sources())
+    shift = int(re.search(r"kNormShift = (\d+);", text).group(1))
+    assert re.search(r"kNormClusterMax = 1 << \(32 - 24 - kNormShift\);", text)
+    assert int(re.search(r"kBatMaxCluster = (\d+);", text).group(1)) <= 1 << (32 - 24 - shift)
+    users = [f for f, t in sources() if "cudaLaunchAttributeClusterDimension" in t]
+    assert users == ["tetra_batched.cu"] and "static_assert(kBatMaxCluster <= kNormClusterMax" in text
