@@ -14,15 +14,15 @@
 //   (rows q and q + 8), and B is block diagonal -- column 2 t + v of B is zero outside the k range that lane t feeds --
 //   so D[q][2 t + v] is the product of lane (q, t)'s own block with vector v of its own column and arrives in that same
 //   lane, next to the block's scale: six MMAs for two blocks per lane and two vectors, no shuffle, no shared-memory
-//   tile, and B is the activations as they lie in memory;
+//   tile, and B is the activations as they lie in memory (rows that are not 16-byte aligned: shifted to where aligned ones are);
 //   five and more: dense B.  A block's 24 halves go through a shared-memory tile whose rows keep stores and ldmatrix
 //   conflict-free, an MMA pair (k16 + k8) multiplies sixteen blocks of ONE column with eight vectors, and the
 //   block's scale reaches the lanes that hold its results by a shuffle.
 // The line lies where the tensor pipe's time for the zeros overtakes the tile.  Block diagonal / dense, 2, 3, 4 vectors:
-// 4096 x 4096 6.5 / 8.2, 7.6 / 8.2, 7.8 / 8.4 us; 4096 x 12288 13.8 / 18.7, 16.3 / 19.1, 16.1 / 18.9; 1024 x 4096
-// 3.9 / 4.7, 4.4 / 4.7, 4.4 / 4.7.  Eight and sixteen on 4096 x 4096: 9.3 and 13.3 us in a build that had them block
-// diagonal, 8.7 and 10.1 dense.  (Int8 planes, activations staged by the CTA and a combining kernel: 13.5 us for three
-// vectors on 4096 x 4096, 27.8 us for sixteen on 4096 x 12288, against 7.6 and 22.8.)
+// 4096 x 4096 7.1 / 9.0, 8.2 / 9.1, 8.2 / 9.2 us; 4096 x 12288 12.8 / 18.6, 15.5 / 18.7, 15.7 / 18.9; 1024 x 4096
+// 4.0 / 4.9, 4.5 / 4.9, 4.5 / 4.9.  Eight and sixteen on 4096 x 4096, in an earlier series: 9.3 and 13.3 us in a build that
+// had them block diagonal, 8.7 and 10.1 dense.  (Int8 planes, activations staged by the CTA and a combining kernel: 13.5 us
+// for three vectors on 4096 x 4096, 27.8 us for sixteen on 4096 x 12288, against 7.7 and 22.1.)
 //
 // A warp's step is NT row tiles x four block columns.  The sixteen warps of a CTA take every sixteenth column quad, so a
 // warp needs nothing from the others until the end: its words come straight from global memory one step ahead, the four
@@ -76,11 +76,11 @@ constexpr bool bat_hold(bool dense) { return dense; }
 // them in their places: it is filled at the start of a step, when the step before has been read.
 constexpr uint32_t bat_buffers(bool dense) { return bat_hold(dense) ? 1 : 2; }
 // Whether a step asks for the next quad's activations behind its first tile's lookups instead of ahead of them.  Ahead /
-// behind, two vectors, us: one tile 2048 x 2304 3.54 / 3.59, two tiles 4096 x 12288 13.4 / 12.8, 4096 x 4096 7.3 / 7.1, three
-// 5003 x 7008 12.3 / 11.9, four 9000 x 1104 4.77 / 4.72.  With four vectors it is a matter of the tiles and of how the copies
-// are written (4096 x 12288 15.6 / 15.1 in the best form of each, 9728 x 2560 13.6 / 13.8, 2048 x 2304 3.82 / 3.87).  Rows that
-// are not aligned are put into their places there too: 4096 x 4097 with 2 / 3 vectors 7.8 / 9.2 ahead, 7.4 / 9.1 behind; 700 x 804
-// with three 2.84 and 2.90, 9000 x 1100 6.68 and 6.83.
+// behind, us, two vectors: one tile 2048 x 2304 3.47 / 3.54 (700 x 800 2.23 / 2.19), two tiles 4096 x 12288 13.5 / 12.7, three
+// 5003 x 7008 12.3 / 11.8, four 9000 x 1104 4.79 / 4.73.  Four vectors gain with two tiles only (4096 x 12288 15.6 / 15.1, but
+// 9728 x 2560 13.6 / 13.8 and 2048 x 2304 3.83 / 3.87) and stay ahead.  Rows that are not aligned are put into their places
+// there too: two tiles, 4096 x 4097 with 2 / 3 vectors, 7.8 / 9.2 ahead and 7.5 / 9.1 behind; one, 700 x 804 with three, 2.95
+// and 3.00; four, 9000 x 1100 with three, 6.6 and 7.1.
 constexpr bool bat_late(bool dense, int g, int nt, bool wide) { return !dense && (wide ? g == 1 && nt > 1 : nt == 2); }
 // Row stride, in floats, of the partial sums: even, so that pairs stay aligned.
 constexpr int bat_stride(bool dense, int g) { return bat_slots(dense, g) + 2; }
@@ -251,7 +251,9 @@ k_gemv_batched(const DeviceTables* __restrict__ tab, const __grid_constant__ Bat
     // Rows of x that are not 16-byte aligned come as they lie in memory, thirteen aligned units: a vector's quad starts
     // x_skip halves into its part of the buffer, the same for all quads.  What the first unit brings along from ahead of
     // the row is not used.  (Loaded, shifted and stored by the lanes, a pair of vectors after the other, a step waited for
-    // memory up to eight times: 5003 x 7001 with 3 / 8 / 16 vectors 17.8 / 25.3 / 37.7 us, 16.8 / 20.4 / 26.2 this way.)
+    // memory up to eight times.  5003 x 7001 with 2 / 3 / 8 / 16 vectors 13.7 / 17.6 / 24.9 / 37.3 us, 13.4 / 16.4 / 20.1 / 25.5
+    // this way.  Two vectors are up to 3 % slower where a warp has a step or two, 2048 x 2305 4.03 and 4.09: a step more of
+    // shared memory in a short chain.)
     [[maybe_unused]] constexpr uint32_t kRaw = Shape::hold ? 0u : 1u;  // dense: the fragments are read from where the rows arrive
     const uint32_t x_half = uint32_t(reinterpret_cast<uintptr_t>(P.x) >> 1);
     [[maybe_unused]] auto x_skip = [&](int v) { return row_skip(x_half, v, P.K); };
@@ -563,13 +565,15 @@ struct BatPlan {
 // columns (0.8-0.9 us with up to four vectors, 0.9-1.3 with eight, 1.2-1.7 with sixteen), and what else the split
 // costs: a chunk of tiles its words, barriers and sums, a cluster its barriers and the other CTA's sums.  One CTA / two, us:
 //   vectors   1184 x 12288   2368 x 12288   3000 x 12288   4096 x 12288   1024 x 4080   2368 x 4080   512 x 4080
-//         3     9.1 /  8.0    10.0 / 11.4    15.8 / 14.0    16.0 / 17.4     4.6 / 5.5     5.4 / 7.0    4.3 / 4.3
-//         8    11.8 /  9.3    12.5 / 13.2    20.3 / 16.8    20.4 / 20.3     5.2 / 5.8     6.2 / 7.7    5.0 / 4.7
-//        16    14.9 / 10.8    15.7 / 14.8    22.8 / 19.3    23.0 / 24.3     6.5 / 6.7     7.4 / 8.7    6.3 / 5.7
+//         3     9.0 /  7.9     9.6 / 10.9    15.3 / 13.5    15.5 / 16.9     4.2 / 5.4     5.1 / 6.7    4.2 / 4.3
+//         8    12.0 /  9.3    12.8 / 13.1    19.9 / 16.5    20.0 / 20.0     5.1 / 5.6     5.9 / 7.4    5.0 / 4.7
+//        16    15.1 / 10.9    16.0 / 14.6    22.2 / 18.9    22.3 / 23.5     6.3 / 6.4     7.0 / 8.3    6.2 / 5.5
 //   chosen           two            one            two            one           one           one          one
 // Short of the best by up to 10 % where rows are few and columns are 4080 or so (a constant of 3 that does not go with the
-// vectors), elsewhere within 6 %.  As many tiles to a step as registers allow: 12288 x 4080 with at most 1, 2, 3, 4 tiles
-// 22.7 / 19.6 / 18.0 / 18.0 us for three vectors, 34.7 / 26.9 / 24.9 / 24.9 for sixteen.
+// vectors) and 9 % for sixteen vectors on 2368 x 12288, elsewhere within 6 %.  As many tiles to a step as registers allow:
+// 12288 x 4080 with at most 1, 2, 3, 4 tiles 22.3 / 19.4 / 17.2 / 17.2 us for three vectors, 34.2 / 26.6 / 24.4 / 24.4 for
+// sixteen.  Larger clusters than two: with the whole rank kept in the scale tables' address (kNormClusterMax) four CTAs took
+// 7.4 us instead of 9.6 for sixteen vectors on 512 x 12288, and everything above 600 rows 1.5 to 3 times as long.
 BatPlan plan_batched(int tiles, int quads, int sms) {
     BatPlan best;
     double best_cost = 1e30;
@@ -600,8 +604,9 @@ constexpr BatKernel bat_kernel() {
     return {k_gemv_batched<DENSE, G, NT, WIDE>, BatShape<DENSE, G, NT, WIDE>::smem.total};
 }
 #define BAT_TILES(dense, g, wide) {bat_kernel<dense, g, 1, wide>(), bat_kernel<dense, g, 2, wide>(), bat_kernel<dense, g, 3, wide>(), bat_kernel<dense, g, 4, wide>()}
-// By alignment of the rows of x, vectors (up to 2, 4: block diagonal; 8, 16: dense) and tiles of a step.  One kernel for
-// aligned and other rows costs the aligned ones registers: 4096 x 12288, 16 vectors, 26.0 us instead of 22.8.
+// By alignment of the rows of x, vectors (up to 2, 4: block diagonal; 8, 16: dense) and tiles of a step.  With both ways of
+// copying in each kernel, chosen as it runs, the aligned rows paid in registers: 4096 x 12288 with 16 vectors 26.0 us; 22.1 now.
+// (The lanes' loads of before beside the aligned copies: 22.8.)
 const BatKernel kBatKernels[2][4][kBatMaxTiles] = {
     {BAT_TILES(false, 1, false), BAT_TILES(false, 2, false), BAT_TILES(true, 1, false), BAT_TILES(true, 2, false)},
     {BAT_TILES(false, 1, true), BAT_TILES(false, 2, true), BAT_TILES(true, 1, true), BAT_TILES(true, 2, true)},
